@@ -98,6 +98,18 @@ def _workload(c, seed):
                           c["recipe"], seed)
 
 
+def _new_tokens(c, p, seed, dev):
+    """q, k, v and gate of the decoded tokens, [steps, B, heads, d] each."""
+    g = torch.Generator(device=dev)
+    g.manual_seed(seed + 5000)
+    kw = dict(generator=g, device=dev, dtype=torch.float32)
+    n, B, H, Hkv, d = c["steps"], c["B"], c["H"], c["Hkv"], c["d"]
+    q = torch.randn(n, B, H, d, **kw).to(p.dtype)
+    k = torch.randn(n, B, Hkv, d, **kw).to(p.dtype)
+    v = torch.randn(n, B, Hkv, d, **kw).to(p.dtype)
+    return q, k, v, torch.rand(n, B, H, d, **kw).to(p.dtype) if c["gate"] else None
+
+
 def prepare(case, seed):
     dev = "cuda"
     c, p, w = case, _params(case), _workload(case, seed)
@@ -125,14 +137,9 @@ def prepare(case, seed):
     # header words and (S, z) of the prefix: what a pass puts back
     s["kept_header"] = s["state"][:256].clone()
     s["kept_sz"] = s["state"][lay["S"]: lay["scratch"]].clone()
-    g = torch.Generator(device=dev)
-    g.manual_seed(seed + 5000)
-    kw = dict(generator=g, device=dev, dtype=torch.float32)
-    n, B, H, Hkv, d = c["steps"], c["B"], c["H"], c["Hkv"], c["d"]
-    s["q"] = torch.randn(n, B, H, d, **kw).to(p.dtype).unbind(0)
-    s["k"] = torch.randn(n, B, Hkv, d, **kw).to(p.dtype).unbind(0)
-    s["v"] = torch.randn(n, B, Hkv, d, **kw).to(p.dtype).unbind(0)
-    s["g"] = torch.rand(n, B, H, d, **kw).to(p.dtype).unbind(0) if c["gate"] else None
+    new = _new_tokens(c, p, seed, dev)
+    s["q"], s["k"], s["v"], s["g"] = (None if x is None else x.unbind(0) for x in new)
+    n, B, H, d = c["steps"], c["B"], c["H"], c["d"]
     s["y"] = torch.empty(n, B, H, d, dtype=p.dtype, device=dev)
     s["y_step"] = s["y"].unbind(0)
     cap, buf = lay["capacity"], s["state"]
@@ -216,3 +223,102 @@ def tolerance(case):
     if case["dtype"] == "fp32":
         return {"rel": 5e-6, "max": 5e-5, "differ": 1e-3}
     return {"rel": 8e-3, "max": 0.5, "differ": 1e-3}
+
+
+def _phi(x, W):
+    """Norm-preserved feature map of x [..., n, d] with W [..., d, d_f], in float64."""
+    f = x @ W
+    u = f * (x.norm(dim=-1, keepdim=True) / f.norm(dim=-1, keepdim=True).clamp_min(1e-12))
+    return torch.cat([u.softmax(-1), (-u).softmax(-1)], -1)
+
+
+def _exact_head_group(c, p, Q, K, V, G, Wq, Wk, row0):
+    """One (batch, KV head): Q [rep, N, d], K, V [N, d], G [rep, N - row0, d], Wq [rep, d, d], Wk [d, d] in float64.
+    Outputs of the rows from row0 on, scores and selection of all tokens, and the linear state after the last token."""
+    C, lam, d, N, dev = c["chunk"], c["topk"], c["d"], K.shape[0], K.device
+    rep, T, window = Q.shape[0], -(-N // C), c["max_salient"] // lam
+    pad = lambda x: torch.nn.functional.pad(x, (0, 0, 0, T * C - x.shape[-2]))
+    Qc, Kc, Vc = pad(Q).view(rep, T, C, d), pad(K).view(T, C, d), pad(V).view(T, C, d)
+    # scores: row r of a chunk has the window of columns r+1 .. r+C of (previous chunk, this chunk)
+    two = torch.cat([torch.cat([torch.zeros_like(Kc[:1]), Kc[:-1]]), Kc], 1)                 # [T, 2C, d]
+    r, j = torch.arange(C, device=dev)[:, None], torch.arange(2 * C, device=dev)[None]
+    own = j == r + C
+    seen = ((j > r) & (j <= r + C))[None].expand(T, C, 2 * C).clone()
+    seen[0] &= j >= C
+    scores = torch.empty(rep, T * C, dtype=torch.float64, device=dev)
+    for h in range(rep):
+        l = (Qc[h] @ two.transpose(1, 2) * p.c().sm_scale).masked_fill(~seen, -math.inf)
+        a = l.softmax(-1)
+        b = l.masked_fill(own, -math.inf).softmax(-1).nan_to_num(0.0)
+        scores[h] = (a * ((a + p.eps) / (b + p.eps)).log()).sum(-1).reshape(-1)
+    live = (torch.arange(T * C, device=dev) < N).view(T, C)
+    sc = scores.view(rep, T, C).masked_fill(~live, -math.inf)
+    order = sc.sort(dim=-1, descending=True, stable=True).indices[..., :lam]
+    chosen = torch.zeros(rep, T, C, dtype=torch.bool, device=dev).scatter_(2, order, True) & live
+    pos = torch.arange(T * C, device=dev).view(T, C).expand(rep, T, C)
+    sel = pos.masked_fill(~chosen, T * C).sort(-1).values[..., :lam]
+    sel = sel.masked_fill(sel == T * C, -1).int()
+    # linear state chunk by chunk; S, z before chunk t is answered hold the chunks up to t-2
+    la = lam < C or window > 0
+    S = torch.zeros(rep, 2 * d, d, dtype=torch.float64, device=dev)
+    z = torch.zeros(rep, 2 * d, dtype=torch.float64, device=dev)
+    Y = torch.empty(rep, N - row0, d, dtype=torch.float64, device=dev)
+    for t in range(T):
+        if la and t >= 2:
+            fold = [(t - 2, ~chosen[:, t - 2])] if lam < C else []
+            if window and t - 2 - window >= 0:
+                fold.append((t - 2 - window, chosen[:, t - 2 - window]))
+            for a, w in fold:
+                f = _phi(Kc[a], Wk) * w[..., None]
+                S += f.transpose(1, 2) @ Vc[a]
+                z += f.sum(1)
+        lo, hi = max(t * C, row0), min((t + 1) * C, N)
+        if lo >= hi:
+            continue
+        q = Q[:, lo:hi]
+        first = max(t - 1 - window, 0) if window else 0      # routed chunks before it have left the cache
+        loc = max(t - 1, 0) * C
+        n_c = max(t - 1 - first, 0)
+        mask = torch.cat([chosen[:, first: first + n_c].reshape(rep, 1, n_c * C).expand(rep, hi - lo, n_c * C),
+                          (torch.arange(loc, hi, device=dev) <= torch.arange(lo, hi, device=dev)[:, None]).expand(rep, -1, -1)], 2)
+        k0 = first * C if n_c else loc
+        l = (q @ K[k0: hi].T * p.c().sm_scale).masked_fill_(~mask, -math.inf)
+        m = l.amax(-1, keepdim=True).clamp_min(0.0 if la else -math.inf)
+        e = (l - m).exp()
+        num, den = e @ V[k0: hi], e.sum(-1, keepdim=True)
+        if la:
+            f = _phi(q, Wq)
+            n_la = f @ S
+            num += (n_la if G is None else n_la * G[:, lo - row0: hi - row0]) * (-m).exp()
+            den = den + (f @ z[..., None]) * (-m).exp()
+        Y[:, lo - row0: hi - row0] = num / den
+    return Y, scores[:, :N], sel, S, z
+
+
+def exact(case, seed):
+    """The outputs of run() in float64 with plain torch.  None where it would take too long."""
+    c, p = case, _params(case)
+    total = c["N"] + c["steps"]
+    visible = min(total, (c["max_salient"] // c["topk"] + 3) * c["chunk"]) if c["max_salient"] else total
+    rows = c["steps"] if c["steps"] else c["N"]
+    if c["B"] * c["H"] * (rows * visible / 2 + total * c["chunk"] * 4) > 1e11:
+        return None
+    dev, w = "cuda", _workload(c, seed)
+    Q, K, V = synth.make_qkv(w, dev)
+    Wq, Wk = synth.make_npmap_weights(w, dev)
+    if c["kind"] == "decode":
+        *new, G = (None if x is None else x.permute(1, 2, 0, 3) for x in _new_tokens(c, p, seed, dev))
+        Q, K, V = (torch.cat([x, n], 2) for x, n in zip((Q, K, V), new))
+    else:
+        G = synth.make_gate(w, dev) if c["gate"] else None
+    rep, out = c["H"] // c["Hkv"], []
+    for b in range(c["B"]):
+        for kv in range(c["Hkv"]):
+            hs = slice(kv * rep, (kv + 1) * rep)
+            out.append(_exact_head_group(c, p, Q[b, hs].double(), K[b, kv].double(), V[b, kv].double(),
+                                         None if G is None else G[b, hs].double(), Wq[hs].double(), Wk[kv].double(),
+                                         c["N"] if c["kind"] == "decode" else 0))
+    Y, scores, sel, S, z = (torch.cat(x).unflatten(0, (c["B"], c["H"])) for x in zip(*out))
+    if c["kind"] == "decode":
+        return (Y.permute(2, 0, 1, 3), scores[:, :, c["N"]:], sel[:, :, -(-c["N"] // c["chunk"]) - 2], S.flatten(), z.flatten())
+    return (Y, scores, sel) + ((S.flatten(), z.flatten()) if c["state"] else ())
