@@ -1,18 +1,20 @@
 // Decode: one step of the Recurrent Form (Sec. 3.3) on the decode state.
 //
-//   step_append_score : appends (k_t, v_t) to the K/V history and computes the
-//                       Self-Saliency Score of the new token (Sec. 3.1).
-//   step_route        : when the new token opens a chunk, the chunk that has just
-//                       left the two-chunk local region is routed (Eq.
-//                       delayed_selection, Eq. cache_routing_sum): top-k positions
-//                       into sel_idx, every other token into (S, z) through the
-//                       NP-Map.
-//   step_attend       : split-KV pass over the salient cache h_t (selected rows of
-//                       the routed chunks + the local region), one partial
-//                       (max, sum, numerator) per split; HBM-bound.
-//   step_merge        : combines the partials, reads out the linear branch and
-//                       applies y = (N_SA + N_LA) / (D_SA + D_LA).
+//   step_route  : (one step in chunk) when the new token opens a chunk, the chunk that has just left the two-chunk
+//                 local region is routed (Eq. delayed_selection, Eq. cache_routing_sum): top-k positions into
+//                 sel_idx, every other token into (S, z) through the NP-Map.
+//   step_main   : everything that reads much: the split-KV pass over the salient cache h_t (selected rows of the
+//                 routed chunks + the local region; one partial (max, sum, numerator) per block and KV group) and the
+//                 linear branch's read-out phi(q) (S, z).  The pass leaves the new token's logits against its window.
+//   step_merge  : combines the partials under one denominator, y = (N_SA + N_LA) / (D_SA + D_LA), appends (k_t, v_t) to
+//                 the history, scores the new token (Sec. 3.1) and counts it.
+//
+// A step of a small batch is bound by latency, not by bytes, so the three are launched with programmatic stream
+// serialization: a kernel's blocks are resident before its predecessor has ended and wait for it in
+// griddepcontrol.wait.  Every block of every kernel executes that wait, so the end of a kernel still implies the end
+// of all before it; and nothing is read before the wait.
 #include "still_common.cuh"
+#include "still_step_f32.cuh"
 #include "still_step_mma.cuh"
 #include "still_tc.h"
 
@@ -20,7 +22,10 @@
 
 namespace still {
 
-constexpr int kMaxSplits = 32;  // history splits; one more partial holds the local region
+// Records of a head in the scratch of the state, d + 2 floats each: partials of the history, the linear branch, and in
+// the last two the new token's logits against its window (at most 128).
+constexpr int kRecords = 33, kMaxSplits = 30, kLinRecord = 30, kLogitRecord = 31;
+constexpr int kStepThreads = kStepWarps * 32;
 
 long long state_kv_rows(const still_params_t *p, long long capacity) {
     if (p->max_salient <= 0 || p->topk <= 0) return capacity;
@@ -29,33 +34,12 @@ long long state_kv_rows(const still_params_t *p, long long capacity) {
 }
 
 size_t step_scratch_bytes(const still_params_t *p, long long) {
-    return (size_t)p->B * p->H * (kMaxSplits + 1) * (p->d + 2) * sizeof(float);
+    return (size_t)p->B * p->H * kRecords * (p->d + 2) * sizeof(float);
 }
 
-template <int n, typename T>
-__device__ __forceinline__ void load_vec(const T *p, float (&out)[n]);
-template <>
-__device__ __forceinline__ void load_vec<2, float>(const float *p, float (&out)[2]) {
-    float2 v = *reinterpret_cast<const float2 *>(p);
-    out[0] = v.x; out[1] = v.y;
-}
-template <>
-__device__ __forceinline__ void load_vec<4, float>(const float *p, float (&out)[4]) {
-    float4 v = *reinterpret_cast<const float4 *>(p);
-    out[0] = v.x; out[1] = v.y; out[2] = v.z; out[3] = v.w;
-}
-template <>
-__device__ __forceinline__ void load_vec<2, __nv_bfloat16>(const __nv_bfloat16 *p, float (&out)[2]) {
-    float2 v = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(p));
-    out[0] = v.x; out[1] = v.y;
-}
-template <>
-__device__ __forceinline__ void load_vec<4, __nv_bfloat16>(const __nv_bfloat16 *p, float (&out)[4]) {
-    uint2 raw = *reinterpret_cast<const uint2 *>(p);
-    float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&raw.x));
-    float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162 *>(&raw.y));
-    out[0] = a.x; out[1] = a.y; out[2] = b.x; out[3] = b.y;
-}
+// The kernel's predecessor in the stream has ended and its writes are visible; the successor may be made resident.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // What a step expects to find in the header of the decode state.
 struct StateKey {
@@ -78,70 +62,27 @@ __device__ __forceinline__ int state_mismatch(const int32_t *hdr, const StateKey
     return have != k.t ? 1 : 0;
 }
 
-// grid (H, B), 32 threads: one warp scores the new token of one query head.  This is the first kernel of a
-// step: every block compares the header with the call and leaves the state untouched on a mismatch (block
-// (0, 0) records it); the later kernels of the step only look at the status word.
-template <typename T>
-__global__ void step_append_score_kernel(T *__restrict__ kc, T *__restrict__ vc,
-                                         float *__restrict__ score, int32_t *__restrict__ hdr,
-                                         const T *__restrict__ q, const T *__restrict__ k,
-                                         const T *__restrict__ v, StateKey key, int H, int Hkv, long long cap,
-                                         long long kvr, int d, int C, long long t, float scale, float eps) {
-    __shared__ float qs[128];
-    const int h = blockIdx.x, b = blockIdx.y, rep = H / Hkv, kv = h / rep, lane = threadIdx.x;
-    {
-        const int bad = state_mismatch(hdr, key);
-        if (bad != 0) {
-            if (h == 0 && b == 0 && lane == 0 && bad != 4) report_status(hdr + 14, STILL_ERR_STATE_MISMATCH, bad);
-            return;
-        }
-    }
-    const T *kn = k + ((long long)b * Hkv + kv) * d;
-    // K / V rows live in a ring of kvr rows per KV head (kvr = capacity unless the salient cache has a budget)
-    T *krow = kc + (((long long)b * Hkv + kv) * kvr + t % kvr) * d;
-    if (h % rep == 0) {
-        const T *vn = v + ((long long)b * Hkv + kv) * d;
-        T *vrow = vc + (((long long)b * Hkv + kv) * kvr + t % kvr) * d;
-        for (int i = lane; i < d; i += 32) {
-            krow[i] = kn[i];
-            vrow[i] = vn[i];
-        }
-    }
-    for (int i = lane; i < d; i += 32) qs[i] = ld_f(q + ((long long)b * H + h) * d + i);
-    __syncwarp();
-    const int spl = C >> 5;
-    float l[4];
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        l[i] = -INFINITY;
-        if (i < spl) {
-            int j = lane + 32 * i;
-            long long pos = t - (C - 1) + j;
-            if (pos >= 0) {
-                // the new key is read from the input, not from the cache row another block writes
-                const T *kr = (pos == t) ? kn : kc + (((long long)b * Hkv + kv) * kvr + pos % kvr) * d;
-                float acc = 0.f;
-                for (int x = 0; x < d; ++x) acc = fmaf(qs[x], ld_f(kr + x), acc);
-                l[i] = acc * scale;
-            }
-        }
-    }
-    float s = window_score(l, lane, spl, C, eps);
-    if (lane == 0) score[((long long)b * H + h) * cap + t] = s;
-}
-
-// grid (H, B), 256 threads.  Routes chunk cr (complete, C tokens): top-k into sel_idx / sel_mask, the other tokens
+// fp32 states; grid (H, B), 256 threads.  Routes chunk cr (complete, C tokens): top-k into sel_idx / sel_mask, the other tokens
 // into (S, z).  With a salient-cache budget of `window` chunks the selected tokens of chunk cr - window leave the
 // cache at the same moment and are folded into (S, z) as well.
 template <typename T>
 __global__ void __launch_bounds__(256)
-step_route_kernel(const T *__restrict__ kc, const T *__restrict__ vc, const float *__restrict__ score,
-                  int32_t *__restrict__ sel_idx, uint32_t *__restrict__ sel_mask, float *__restrict__ S,
-                  float *__restrict__ z, const T *__restrict__ Wk, const T *__restrict__ bk, const int32_t *__restrict__ hdr,
+step_route_kernel(T *kc, T *vc, float *score,
+                  int32_t *sel_idx, uint32_t *sel_mask, float *S,
+                  float *z, T *Wk, T *bk, int32_t *hdr, StateKey key,
                   int H, int Hkv, long long cap, long long kvr, int d, int df, int C, int lam, long long cr, int window,
                   int w_in_smem) {
     extern __shared__ float smem[];
-    if (hdr[14] != 0) return;   // the step's first kernel found the state not to match the call
+    grid_dep_wait();
+    grid_dep_launch();
+    {   // the step's first kernel when there is a chunk to route: the header against the call
+        const int bad = state_mismatch(hdr, key);
+        if (bad != 0) {
+            if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && bad != 4)
+                report_status(hdr + 14, STILL_ERR_STATE_MISMATCH, bad);
+            return;
+        }
+    }
     const int dp = 2 * df;
     float *ph = smem;                 // [C][dp]
     float *vs = ph + C * dp;          // [C][d]
@@ -241,158 +182,564 @@ step_route_kernel(const T *__restrict__ kc, const T *__restrict__ vc, const floa
     }
 }
 
-// grid (n_splits + 1, Hkv, B), 128 threads: warp w serves query heads w, w+4, ... of the group.
-// Split s < n_splits covers routed chunks [s*cps, (s+1)*cps); split n_splits is the local region.
-template <typename T, int DPL>
-__global__ void __launch_bounds__(128)
-step_attend_kernel(const T *__restrict__ kc, const T *__restrict__ vc,
-                   const int32_t *__restrict__ sel_idx, const T *__restrict__ q,
-                   float *__restrict__ part, const int32_t *__restrict__ hdr, int H, int Hkv, long long cap, int C,
-                   int lam, long long t, int n_splits, long long cps, long long n_routed, float scale) {
-    constexpr int d = DPL * 32;
-    __shared__ float qs[4][d];
-    if (hdr[14] != 0) return;
-    const int split = blockIdx.x, kv = blockIdx.y, b = blockIdx.z, rep = H / Hkv;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const T *kh = kc + ((long long)b * Hkv + kv) * cap * d;
-    const T *vh = vc + ((long long)b * Hkv + kv) * cap * d;
-    const bool local = split == n_splits;
-    const long long c_cur = t / C;
-    for (int hh = warp; hh < rep; hh += 4) {
-        const int h = kv * rep + hh;
-        const long long bh = (long long)b * H + h;
-        for (int i = lane; i < d; i += 32) qs[warp][i] = ld_f(q + bh * d + i);
-        __syncwarp();
-        long long n_e, loc0 = 0;
-        const int32_t *si = nullptr;
-        if (local) {
-            loc0 = c_cur >= 1 ? (c_cur - 1) * C : 0;
-            n_e = t + 1 - loc0;
-        } else {
-            long long c_lo = split * cps, c_hi = (c_lo + cps < n_routed) ? c_lo + cps : n_routed;
-            n_e = c_hi > c_lo ? (c_hi - c_lo) * lam : 0;
-            si = sel_idx + (bh * (cap / C) + c_lo) * lam;
-        }
-        float m = -INFINITY, l = 0.f, o[DPL];
-#pragma unroll
-        for (int e = 0; e < DPL; ++e) o[e] = 0.f;
-        for (long long e0 = 0; e0 < n_e; e0 += 32) {
-            long long e = e0 + lane;
-            long long pos = -1;
-            if (e < n_e) pos = local ? loc0 + e : (long long)si[e];
-            float s = -INFINITY;
-            if (pos >= 0) {
-                const T *kr = kh + pos * d;
-                float acc = 0.f;
-#pragma unroll 4
-                for (int x = 0; x < d; x += 4) {
-                    float kk[4];
-                    load_vec<4>(kr + x, kk);
-                    float4 qq = *reinterpret_cast<const float4 *>(&qs[warp][x]);
-                    acc = fmaf(qq.x, kk[0], acc);
-                    acc = fmaf(qq.y, kk[1], acc);
-                    acc = fmaf(qq.z, kk[2], acc);
-                    acc = fmaf(qq.w, kk[3], acc);
-                }
-                s = acc * scale;
-            }
-            float mn = fmaxf(m, warp_max(s));
-            if (mn == -INFINITY) continue;
-            float alpha = expf(m - mn);
-            float pj = (pos >= 0) ? expf(s - mn) : 0.f;
-            l = l * alpha + warp_sum(pj);
-            m = mn;
-#pragma unroll
-            for (int x = 0; x < DPL; ++x) o[x] *= alpha;
-            const int cnt = (n_e - e0 < 32) ? (int)(n_e - e0) : 32;
-            for (int j = 0; j < cnt; ++j) {
-                float pb = __shfl_sync(0xffffffffu, pj, j);
-                long long pp = __shfl_sync(0xffffffffu, pos, j);
-                if (pp < 0) continue;
-                float vv[DPL];
-                load_vec<DPL>(vh + pp * d + lane * DPL, vv);
-#pragma unroll
-                for (int x = 0; x < DPL; ++x) o[x] = fmaf(pb, vv[x], o[x]);
-            }
-        }
-        float *pr = part + (bh * (kMaxSplits + 1) + split) * (d + 2);
-        if (lane == 0) {
-            pr[0] = m;
-            pr[1] = l;
-        }
-#pragma unroll
-        for (int x = 0; x < DPL; ++x) pr[2 + lane * DPL + x] = o[x];
-        __syncwarp();
+// The same for bf16 states on the tensor cores; grid (H, B), 256 threads.  f = K W_k and S += phi(K)^T V are bf16
+// products with fp32 accumulation (the features are bf16 in the prefill as well); f is kept in fp32 and a row of f is
+// replaced in place by the row's features, zero for a token that stays out.  The state is read straight into the
+// accumulators and written back from them.  What bounds it is the read and write of S (128 KB a head each way) and, for
+// few heads, the chain of loads, two products and the row-wise softmax.
+template <int D>
+struct RoutePlan {
+    int k, v, w, f, sc, flag, total;   // byte offsets
+    __host__ __device__ RoutePlan(int C, int df) {
+        k = 0;
+        v = k + C * D * 2;
+        w = v + C * D * 2;
+        f = w + D * df * 2;              // f [C][df] fp32, then phi [C][2 df] bf16
+        sc = f + C * df * 4;
+        flag = sc + C * 4;
+        total = flag + C * 4;
     }
-}
+};
+template <int D>
+__global__ void __launch_bounds__(256)
+step_route_mma_kernel(__nv_bfloat16 *kc, __nv_bfloat16 *vc, float *score, int32_t *sel_idx, uint32_t *sel_mask, float *S,
+                      float *z, __nv_bfloat16 *Wk, __nv_bfloat16 *bk, int32_t *hdr, StateKey key, int H, int Hkv, long long cap,
+                      long long kvr, int df, int C, int lam, long long cr, int window) {
+    extern __shared__ __align__(128) uint8_t route_smem[];
+    grid_dep_wait();
+    grid_dep_launch();
+    {   // the step's first kernel when there is a chunk to route: the header against the call
+        const int bad = state_mismatch(hdr, key);
+        if (bad != 0) {
+            if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0 && bad != 4)
+                report_status(hdr + 14, STILL_ERR_STATE_MISMATCH, bad);
+            return;
+        }
+    }
+    const RoutePlan<D> plan(C, df);
+    uint8_t *ks = route_smem + plan.k, *vs = route_smem + plan.v, *ws = route_smem + plan.w, *fs = route_smem + plan.f;
+    float *sc = reinterpret_cast<float *>(route_smem + plan.sc);
+    int *flag = reinterpret_cast<int *>(route_smem + plan.flag);
+    const int h = blockIdx.x, b = blockIdx.y, kv = h / (H / Hkv), dp = 2 * df;
+    const long long bh = (long long)b * H + h, row0 = (long long)b * Hkv + kv;
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, g = lane >> 2, tig = lane & 3;
+    // 16-byte pieces of a row are swizzled by the row: ldmatrix reads eight rows of one piece without conflicts
+    constexpr int kRowB = D * 2, kPieces = D / 8;
+    const int w_pieces = df / 8, f_row = df * 4;
+    auto w_off = [&](int row, int piece) { return row * df * 2 + ((w_pieces >= 8 ? piece ^ (row & 7) : piece ^ ((row >> 1) & 3)) << 4); };
 
-// grid (H, B), 128 threads.
-template <typename T>
-__global__ void __launch_bounds__(128)
-step_merge_kernel(const float *__restrict__ part, const float *__restrict__ S,
-                  const float *__restrict__ z, const T *__restrict__ q, const T *__restrict__ g,
-                  const T *__restrict__ Wq, const T *__restrict__ bq, T *__restrict__ y,
-                  int32_t *__restrict__ hdr, int H, int d, int df, int n_splits, int la,
-                  long long t) {
-    __shared__ float qs[128], phi[256], red[4];
-    if (hdr[14] != 0) return;   // mismatch recorded by the step's first kernel: no output, token count unchanged
-    const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
-    const long long bh = (long long)b * H + h;
-    const int dp = 2 * df;
-    const float *pr = part + bh * (kMaxSplits + 1) * (d + 2);
-    float M = -INFINITY;
-    for (int s = 0; s <= n_splits; ++s) M = fmaxf(M, pr[s * (d + 2)]);
-    float Lsum = 0.f, O = 0.f;
-    for (int s = 0; s <= n_splits; ++s) {
-        float ms = pr[s * (d + 2)];
-        if (ms == -INFINITY) continue;
-        float w = expf(ms - M);
-        Lsum += w * pr[s * (d + 2) + 1];
-        if (tid < d) O += w * pr[s * (d + 2) + 2 + tid];
+    const bool fold0 = lam < C, fold1 = window > 0 && cr >= window;
+    auto load_chunk = [&](long long chunk) {   // (a chunk never straddles the ring's end)
+        const long long r = chunk * C % kvr;
+        const __nv_bfloat16 *kh = kc + (row0 * kvr + r) * D, *vh = vc + (row0 * kvr + r) * D;
+        for (int i = tid; i < C * kPieces; i += 256) {
+            const int row = i / kPieces, piece = i % kPieces, dst = row * kRowB + ((piece ^ (row & 7)) << 4);
+            cp_async16(ks + dst, kh + (long long)row * D + piece * 8, true);
+            cp_async16(vs + dst, vh + (long long)row * D + piece * 8, true);
+        }
+    };
+    if (fold0 || fold1) {
+        for (int i = tid; i < D * w_pieces; i += 256) {
+            const int row = i / w_pieces, piece = i % w_pieces;
+            cp_async16(ws + w_off(row, piece), Wk + ((long long)kv * D + row) * df + piece * 8, true);
+        }
+        load_chunk(fold0 ? cr : cr - window);
     }
-    float nla = 0.f, dla = 0.f;
-    if (la) {
-        for (int i = tid; i < d; i += blockDim.x) qs[i] = ld_f(q + bh * d + i);
+    cp_async_commit();
+    for (int i = tid; i < C; i += 256) {
+        sc[i] = score[bh * cap + cr * C + i];
+        flag[i] = 0;
+    }
+    __syncthreads();
+    if (lam > 0) select_chunk(sc, flag, C, C, lam, cr * C, sel_idx + (bh * (cap / C) + cr) * lam);
+    __syncthreads();
+    if (tid < C / 32) {  // the same selection as bit masks (read by the split-KV pass)
+        uint32_t bits = 0u;
+        for (int j = 0; j < 32; ++j) bits |= (flag[tid * 32 + j] ? 1u : 0u) << j;
+        sel_mask[(bh * (cap / C) + cr) * (C / 32) + tid] = bits;
+    }
+    for (int pass = 0; pass < 2; ++pass) {   // the unselected tokens of chunk cr; the selected ones of the chunk that leaves
+        if (!(pass == 0 ? fold0 : fold1)) continue;
         __syncthreads();
-        if (warp == 0) {
-            float ep[4], en[4];
-            npmap_row(qs, Wq + (long long)h * d * df, bq ? bq + (long long)h * df : (const T *)nullptr, d,
-                      df, lane, ep, en);
+        if (pass == 1) {
+            const long long chunk = cr - window;
+            if (fold0) {
+                load_chunk(chunk);
+                cp_async_commit();
+            }
+            for (int i = tid; i < C; i += 256)
+                flag[i] = !((sel_mask[(bh * (cap / C) + chunk) * (C / 32) + i / 32] >> (i & 31)) & 1u);
+        }
+        cp_async_wait<0>();
+        __syncthreads();
+        // f = K W_k: 16 tokens x 32 features at a time
+        for (int u = warp; u < (C / 16) * (df / 32); u += 8) {
+            const int mt = u / (df / 32), n0 = u % (df / 32) * 32;
+            float acc[4][4] = {};
+#pragma unroll
+            for (int k16 = 0; k16 < D / 16; ++k16) {
+                uint32_t af[4], bf[4];
+                const int arow = mt * 16 + ((lane >> 3) & 1) * 8 + (lane & 7), apiece = k16 * 2 + (lane >> 4);
+                ldmatrix_x4(af, ks + arow * kRowB + ((apiece ^ (arow & 7)) << 4));
+#pragma unroll
+                for (int np = 0; np < 2; ++np) {
+                    ldmatrix_x4_trans(bf, ws + w_off(k16 * 16 + ((lane >> 3) & 1) * 8 + (lane & 7), n0 / 8 + np * 2 + (lane >> 4)));
+                    mma_16816(acc[np * 2], af, bf[0], bf[1]);
+                    mma_16816(acc[np * 2 + 1], af, bf[2], bf[3]);
+                }
+            }
+#pragma unroll
+            for (int nt = 0; nt < 4; ++nt)
+#pragma unroll
+                for (int hr = 0; hr < 2; ++hr) {
+                    const int row = mt * 16 + g + hr * 8, col = n0 + nt * 8 + tig * 2;
+                    *reinterpret_cast<float2 *>(fs + row * f_row + (((col >> 2) ^ (row & 7)) << 4) + (col & 3) * 4) =
+                        make_float2(acc[nt][hr * 2], acc[nt][hr * 2 + 1]);
+                }
+        }
+        __syncthreads();
+        // a warp per row: u = f ||x|| / ||f||, phi = [softmax(u), softmax(-u)], rounded as the prefill stores it
+        for (int r = warp; r < C; r += 8) {
+            const bool out = flag[r] != 0;   // the token stays out of this pass
+            float f[4], ep[4], en[4];
+            float nx2 = 0.f, nf2 = 0.f, umax = -INFINITY, umin = INFINITY;
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj) {
+                f[jj] = 0.f;
+                if (jj * 32 < df) {
+                    const int j = lane + 32 * jj;
+                    f[jj] = *reinterpret_cast<const float *>(fs + r * f_row + (((j >> 2) ^ (r & 7)) << 4) + (j & 3) * 4);
+                    if (bk) f[jj] += ld_f(bk + (long long)kv * df + j);
+                    nf2 = fmaf(f[jj], f[jj], nf2);
+                }
+                if (jj * 32 < D) {
+                    const int j = lane + 32 * jj;
+                    const float x = ld_f(reinterpret_cast<const __nv_bfloat16 *>(ks + r * kRowB + (((j >> 3) ^ (r & 7)) << 4)) + (j & 7));
+                    nx2 = fmaf(x, x, nx2);
+                }
+            }
+            nx2 = warp_sum(nx2);
+            nf2 = warp_sum(nf2);
+            const float ratio = sqrtf(nx2) / fmaxf(sqrtf(nf2), 1e-12f);
 #pragma unroll
             for (int jj = 0; jj < 4; ++jj)
-                if (jj < (df >> 5)) {
-                    T a, c2;
-                    st_f(&a, ep[jj]);
-                    st_f(&c2, en[jj]);
-                    phi[lane + 32 * jj] = ld_f(&a);
-                    phi[df + lane + 32 * jj] = ld_f(&c2);
+                if (jj * 32 < df) {
+                    f[jj] *= ratio;
+                    umax = fmaxf(umax, f[jj]);
+                    umin = fminf(umin, f[jj]);
+                }
+            umax = warp_max(umax);
+            umin = warp_min(umin);
+            float zp = 0.f, zn = 0.f;
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj) {
+                ep[jj] = en[jj] = 0.f;
+                if (jj * 32 < df) {
+                    ep[jj] = expf(f[jj] - umax);
+                    en[jj] = expf(umin - f[jj]);
+                    zp += ep[jj];
+                    zn += en[jj];
+                }
+            }
+            zp = warp_sum(zp);   // (also: every lane has read its f before any lane overwrites the row)
+            zn = warp_sum(zn);
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj)
+                if (jj * 32 < df) {
+                    const int j = lane + 32 * jj, jn = df + j;
+                    st_f(reinterpret_cast<__nv_bfloat16 *>(fs + r * f_row + (((j >> 3) ^ (r & 7)) << 4)) + (j & 7), out ? 0.f : ep[jj] / zp);
+                    st_f(reinterpret_cast<__nv_bfloat16 *>(fs + r * f_row + (((jn >> 3) ^ (r & 7)) << 4)) + (jn & 7), out ? 0.f : en[jj] / zn);
                 }
         }
         __syncthreads();
-        const float *Sh = S + bh * dp * d;
-        if (tid < d)
-            for (int f = 0; f < dp; ++f) nla = fmaf(phi[f], Sh[(long long)f * d + tid], nla);
-        float part_d = 0.f;
-        for (int f = tid; f < dp; f += blockDim.x) part_d = fmaf(phi[f], z[bh * dp + f], part_d);
-        part_d = warp_sum(part_d);
-        if (lane == 0) red[warp] = part_d;
-        __syncthreads();
-        dla = red[0] + red[1] + red[2] + red[3];
-        if (g && tid < d) nla *= ld_f(g + bh * d + tid);
-    }
-    if (tid < d) {
-        float fs = 1.f, fl = 0.f;
-        if (dla > 0.f) {
-            float ms = fmaxf(M, 0.f);
-            fs = expf(M - ms);
-            fl = expf(-ms);
+        // S += phi^T V: 16 features x 64 value columns at a time
+        for (int u = warp; u < (dp / 16) * (D / 64); u += 8) {
+            const int mt = u / (D / 64), e0 = u % (D / 64) * 64;
+            float acc[8][4];
+            float *Sr = S + (bh * dp + mt * 16 + g) * D + e0 + tig * 2;
+#pragma unroll
+            for (int nt = 0; nt < 8; ++nt) {
+                const float2 lo = *reinterpret_cast<const float2 *>(Sr + nt * 8), hi = *reinterpret_cast<const float2 *>(Sr + 8 * D + nt * 8);
+                acc[nt][0] = lo.x; acc[nt][1] = lo.y; acc[nt][2] = hi.x; acc[nt][3] = hi.y;
+            }
+            for (int k16 = 0; k16 < C / 16; ++k16) {
+                uint32_t af[4], bf[4];
+                const int arow = k16 * 16 + (lane >> 4) * 8 + (lane & 7), apiece = mt * 2 + ((lane >> 3) & 1);
+                ldmatrix_x4_trans(af, fs + arow * f_row + ((apiece ^ (arow & 7)) << 4));
+                const int brow = k16 * 16 + ((lane >> 3) & 1) * 8 + (lane & 7);
+#pragma unroll
+                for (int np = 0; np < 4; ++np) {
+                    const int bpiece = e0 / 8 + np * 2 + (lane >> 4);
+                    ldmatrix_x4_trans(bf, vs + brow * kRowB + ((bpiece ^ (brow & 7)) << 4));
+                    mma_16816(acc[np * 2], af, bf[0], bf[1]);
+                    mma_16816(acc[np * 2 + 1], af, bf[2], bf[3]);
+                }
+            }
+#pragma unroll
+            for (int nt = 0; nt < 8; ++nt) {
+                *reinterpret_cast<float2 *>(Sr + nt * 8) = make_float2(acc[nt][0], acc[nt][1]);
+                *reinterpret_cast<float2 *>(Sr + 8 * D + nt * 8) = make_float2(acc[nt][2], acc[nt][3]);
+            }
         }
-        st_f(y + bh * d + tid, (O * fs + fl * nla) / (Lsum * fs + fl * dla));
+        for (int f = tid; f < dp; f += 256) {
+            float acc = 0.f;
+            for (int r = 0; r < C; ++r)
+                acc += ld_f(reinterpret_cast<const __nv_bfloat16 *>(fs + r * f_row + (((f >> 3) ^ (r & 7)) << 4)) + (f & 7));
+            z[bh * dp + f] += acc;
+        }
+    }
+    cp_async_wait<0>();
+}
+
+// Arguments of step_main_kernel / step_merge_kernel.  (Pointers are neither const nor restrict: their contents come
+// from kernels that may still run when a block becomes resident, and must not be loaded ahead of the wait.)
+template <typename T>
+struct StepArgs {
+    T *kc, *vc;
+    float *score;
+    uint32_t *sel_mask;
+    float *S, *z, *part;
+    int32_t *hdr;
+    T *q, *k, *v, *g, *Wq, *bq, *y;
+    StateKey key;
+    AttendView view;             // view.rep: query heads of a KV group
+    long long cap, kvr, t;
+    int B, H, Hkv, df, la;
+    float eps;
+    // Plan.  A unit is what shares its K / V rows: the query heads of one (batch, KV head) (fp32: up to four of them).
+    // The units' tiles form one line of units * tiles, of which block i takes [i * per, (i + 1) * per): blocks that
+    // divide the line evenly, whatever the number of groups.  Items: the linear read-outs, one per (batch, query head).
+    int heads_per_unit, units_per_group, tiles;
+    long long per, total;
+    int first_item_block, n_items;   // blocks from first_item_block on share the items evenly
+    int item_warps;                  // warps that work on an item together
+};
+
+// First block that works on unit u, and how many do.
+__device__ __forceinline__ long long unit_first_block(long long per, int tiles, long long u) { return u * tiles / per; }
+__device__ __forceinline__ int unit_blocks(long long per, int tiles, long long u) {
+    return (int)(((u + 1) * tiles - 1) / per - u * tiles / per) + 1;
+}
+
+// Eight (bf16) or four (fp32) consecutive values as fp32.
+__device__ __forceinline__ void load16(const __nv_bfloat16 *p, float (&o)[8]) {
+    const uint4 r = *reinterpret_cast<const uint4 *>(p);
+    const uint32_t w[4] = {r.x, r.y, r.z, r.w};
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        o[2 * i] = __uint_as_float(w[i] << 16);
+        o[2 * i + 1] = __uint_as_float(w[i] & 0xffff0000u);
+    }
+}
+__device__ __forceinline__ void load16(const float *p, float (&o)[4]) {
+    const float4 r = *reinterpret_cast<const float4 *>(p);
+    o[0] = r.x; o[1] = r.y; o[2] = r.z; o[3] = r.w;
+}
+
+// Read-outs are worked on by groups of NW warps (1, 2 or all 8 of a block).
+template <int NW>
+__device__ __forceinline__ void group_sync() {
+    if constexpr (NW == 1) __syncwarp();
+    else if constexpr (NW == kStepWarps) __syncthreads();
+    else asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)(threadIdx.x >> 5) / NW), "n"(NW * 32) : "memory");
+}
+// Shared memory of a group beside the rings, in floats: q [D], phi [2 d_f], sums of z [8], partial sums [NW][D].
+constexpr int kItemFloats = 128 + 256 + 8;
+constexpr int kItemSmem = kStepWarps * (kItemFloats + 128) * 4;
+
+// Linear read-out of one (batch, query head): N_LA = phi(q) S, D_LA = phi(q) z into the head's last record.  S [2 d_f, D]
+// fp32 (128 KB at d = d_f = 128) and W_q are what it costs.  A warp takes a contiguous slice of either through its
+// cp.async ring, first W_q, then S, so that the whole ring is in flight also while phi(q) is formed.  (With the rows
+// requested into registers instead, a warp had too little in flight: 512 read-outs took 60 us, 1.1 TB/s.)
+template <typename T, int D, int NW, class Ring>
+__device__ __forceinline__ void linear_item(const StepArgs<T> &a, long long bh, uint8_t *ring, float *smem) {
+    constexpr int V = 16 / (int)sizeof(T);
+    constexpr int LPR = D / 4, RPW = 32 / LPR;        // lanes per row of S (16 bytes each), rows per warp and load
+    constexpr int kStage = Ring::kStage, kStages = Ring::kStages;
+    const int warp = (threadIdx.x >> 5) % NW, lane = threadIdx.x & 31, tid = warp * 32 + lane;
+    const int df = a.df, dp = 2 * df, h = (int)(bh % a.H), jpl = df >> 5;
+    float *qs = smem, *ph = qs + D, *redz = ph + 256, *red = redz + 8;
+    const int w_bytes = D * df * (int)sizeof(T) / NW, s_bytes = dp * D * 4 / NW;   // this warp's slices
+    const int n_w = (w_bytes + kStage - 1) / kStage, n_s = (s_bytes + kStage - 1) / kStage;
+    const char *w_src = reinterpret_cast<const char *>(a.Wq + (long long)h * D * df) + (long long)warp * w_bytes;
+    const char *s_src = reinterpret_cast<const char *>(a.S + bh * dp * D) + (long long)warp * s_bytes;
+    auto issue = [&](int c) {
+        if (c < n_w + n_s) {
+            const bool is_w = c < n_w;
+            const int off = (is_w ? c : c - n_w) * kStage, bytes = min(kStage, (is_w ? w_bytes : s_bytes) - off);
+            const char *src = (is_w ? w_src : s_src) + off;
+            uint8_t *dst = ring + c % kStages * kStage;
+#pragma unroll 4
+            for (int i = lane * 16; i < bytes; i += 512) cp_async16(dst + i, src + i, true);
+        }
+        cp_async_commit();
+    };
+#pragma unroll
+    for (int c = 0; c < kStages; ++c) issue(c);
+    for (int i = tid; i < D; i += NW * 32) qs[i] = ld_f(a.q + bh * D + i);
+    float dz = 0.f, zv[8];
+#pragma unroll
+    for (int i = 0; i < 8 / NW + (8 % NW ? 1 : 0); ++i) zv[i] = tid + i * NW * 32 < dp ? a.z[bh * dp + tid + i * NW * 32] : 0.f;
+    group_sync<NW>();
+    {   // f = q W_q: 16 bytes of a row per lane
+        const int lpr = df / V, rpl = 32 / lpr, cg = lane % lpr;
+        float acc[V];
+#pragma unroll
+        for (int e = 0; e < V; ++e) acc[e] = 0.f;
+        for (int c = 0; c < n_w; ++c) {
+            cp_async_wait<kStages - 1>();
+            __syncwarp();
+            const T *wr = reinterpret_cast<const T *>(ring + c % kStages * kStage) + cg * V;
+            const int r0 = (warp * w_bytes + c * kStage) / (df * (int)sizeof(T));
+            const int rows = min(kStage, w_bytes - c * kStage) / (df * (int)sizeof(T));
+#pragma unroll 4
+            for (int r = lane / lpr; r < rows; r += rpl) {
+                float w[V];
+                load16(wr + r * df, w);
+                const float x = qs[r0 + r];
+#pragma unroll
+                for (int e = 0; e < V; ++e) acc[e] = fmaf(x, w[e], acc[e]);
+            }
+            __syncwarp();
+            issue(c + kStages);
+        }
+        for (int o = lpr; o < 32; o <<= 1) {
+#pragma unroll
+            for (int e = 0; e < V; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
+        }
+        if (lane < lpr) {
+#pragma unroll
+            for (int e = 0; e < V; ++e) red[warp * df + cg * V + e] = acc[e];
+        }
+        group_sync<NW>();
+    }
+    {   // every warp forms the norms and sums; features are rounded to the storage type, as the prefill stores them
+        float nx2 = 0.f, nf2 = 0.f, f[4], umax = -INFINITY, umin = INFINITY;
+        for (int i = lane; i < D; i += 32) nx2 += qs[i] * qs[i];
+        nx2 = warp_sum(nx2);
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+            f[jj] = 0.f;
+            if (jj < jpl) {
+                if (a.bq) f[jj] = ld_f(a.bq + (long long)h * df + lane + 32 * jj);
+#pragma unroll
+                for (int w = 0; w < NW; ++w) f[jj] += red[w * df + lane + 32 * jj];
+            }
+            nf2 += f[jj] * f[jj];
+        }
+        nf2 = warp_sum(nf2);
+        const float ratio = sqrtf(nx2) / fmaxf(sqrtf(nf2), 1e-12f);
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj)
+            if (jj < jpl) {
+                f[jj] *= ratio;
+                umax = fmaxf(umax, f[jj]);
+                umin = fminf(umin, f[jj]);
+            }
+        umax = warp_max(umax);
+        umin = warp_min(umin);
+        float zp = 0.f, zn = 0.f, ep[4], en[4];
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) {
+            ep[jj] = en[jj] = 0.f;
+            if (jj < jpl) {
+                ep[jj] = expf(f[jj] - umax);
+                en[jj] = expf(umin - f[jj]);
+                zp += ep[jj];
+                zn += en[jj];
+            }
+        }
+        zp = warp_sum(zp);
+        zn = warp_sum(zn);
+        if (warp == 0) {
+#pragma unroll
+            for (int jj = 0; jj < 4; ++jj)
+                if (jj < jpl) {
+                    T p0, p1;
+                    st_f(&p0, ep[jj] / zp);
+                    st_f(&p1, en[jj] / zn);
+                    ph[lane + 32 * jj] = ld_f(&p0);
+                    ph[df + lane + 32 * jj] = ld_f(&p1);
+                }
+        }
+        group_sync<NW>();
+    }
+    float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int c = n_w; c < n_w + n_s; ++c) {
+        cp_async_wait<kStages - 1>();
+        __syncwarp();
+        const int off = (c - n_w) * kStage, rows = min(kStage, s_bytes - off) / (D * 4);
+        const float *sr = reinterpret_cast<const float *>(ring + c % kStages * kStage) + lane * 4;
+        const float *pr = ph + (warp * s_bytes + off) / (D * 4) + lane / LPR;
+#pragma unroll 4
+        for (int r = 0; r < rows; r += RPW) {
+            const float4 x = *reinterpret_cast<const float4 *>(sr + r * D);
+            const float p = pr[r];
+            acc.x = fmaf(p, x.x, acc.x);
+            acc.y = fmaf(p, x.y, acc.y);
+            acc.z = fmaf(p, x.z, acc.z);
+            acc.w = fmaf(p, x.w, acc.w);
+        }
+        __syncwarp();
+        issue(c + kStages);
+    }
+    cp_async_wait<0>();
+    if constexpr (RPW == 2) {
+        acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 16);
+        acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 16);
+        acc.z += __shfl_xor_sync(0xffffffffu, acc.z, 16);
+        acc.w += __shfl_xor_sync(0xffffffffu, acc.w, 16);
+    }
+    if (lane < LPR) *reinterpret_cast<float4 *>(red + warp * D + lane * 4) = acc;
+#pragma unroll
+    for (int i = 0; i < 8 / NW + (8 % NW ? 1 : 0); ++i)
+        if (tid + i * NW * 32 < dp) dz = fmaf(ph[tid + i * NW * 32], zv[i], dz);
+    dz = warp_sum(dz);
+    if (lane == 0) redz[warp] = dz;
+    group_sync<NW>();
+    float *rec = a.part + (bh * kRecords + kLinRecord) * (D + 2);
+    for (int i = tid; i < D; i += NW * 32) {
+        float n = 0.f;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) n += red[w * D + i];
+        rec[2 + i] = n;
+    }
+    if (tid == 0) {
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < NW; ++w) s += redz[w];
+        rec[1] = s;
+    }
+    group_sync<NW>();
+}
+
+// This block's share of the read-outs, by groups of NW warps.
+template <typename T, int D, int NW, class Ring>
+__device__ __forceinline__ void work_on_items(const StepArgs<T> &a, uint8_t *smem) {
+    constexpr int kGroups = kStepWarps / NW;
+    const int warp = threadIdx.x >> 5, group = warp / NW, blocks = (int)gridDim.x - a.first_item_block;
+    const long long worker = (int)blockIdx.x - a.first_item_block + (long long)group * blocks, workers = (long long)blocks * kGroups;
+    float *mine = reinterpret_cast<float *>(smem + Ring::kTotal) + group * (kItemFloats + NW * 128);
+    for (long long i = worker; i < a.n_items; i += workers) linear_item<T, D, NW, Ring>(a, i, smem + warp * Ring::kWarp, mine);
+}
+
+// Rings of the cache pass.
+template <typename T, int D>
+struct StepRing : AttendPlan<D> {};
+template <int D>
+struct StepRing<float, D> : AttendPlanF32<D> {};
+// Shared memory of step_main_kernel: the rings, and the read-outs' staging beside them.
+template <typename T, int D>
+constexpr int step_main_smem() {
+    return StepRing<T, D>::kTotal + kItemSmem;
+}
+static_assert(step_main_smem<__nv_bfloat16, 128>() <= 232448 && step_main_smem<float, 128>() <= 232448, "shared memory of a step");
+
+// One block per SM.  At large batches the bytes of K, V and S bound it (B = 64, 32K prefix, every token: 6.6 TB/s a step,
+// 1.27 ms; with one launch each for the append and score, the cache pass in equal splits per group and the merge with
+// its read-out it was 1.65 ms; B = 16, 16K, a quarter kept: 143 us, before 305 us), at one sequence the latency of a
+// block's chain (one user, 2K prefix: below the 14 us in which the host issues a step, before 68 us).
+template <typename T, int D, int NT>
+__global__ void __launch_bounds__(kStepThreads, 1)
+step_main_kernel(const __grid_constant__ StepArgs<T> a) {
+    extern __shared__ __align__(128) uint8_t step_smem[];
+    grid_dep_wait();
+    grid_dep_launch();
+    {   // the header against the call; on a mismatch nothing is written but the status word
+        const int bad = state_mismatch(a.hdr, a.key);
+        if (bad != 0) {
+            if (blockIdx.x == 0 && threadIdx.x == 0 && bad != 4) report_status(a.hdr + 14, STILL_ERR_STATE_MISMATCH, bad);
+            return;
+        }
+    }
+    const long long lo = blockIdx.x * a.per, hi = min(lo + a.per, a.total);
+    const int rep = a.H / a.Hkv;
+    for (long long x = lo; x < hi;) {
+        const long long u = x / a.tiles;
+        const int tile_lo = (int)(x - u * a.tiles), tile_hi = (int)min((long long)a.tiles, hi - u * a.tiles);
+        const long long row = u / a.units_per_group;               // batch * Hkv + KV head
+        const int h0 = (int)(u % a.units_per_group) * a.heads_per_unit;
+        const long long bh = row / a.Hkv * a.H + row % a.Hkv * rep + h0;
+        const long long slot = blockIdx.x - unit_first_block(a.per, a.tiles, u);
+        AttendView v = a.view;
+        v.rep = min(a.heads_per_unit, rep - h0);
+        const T *kh = a.kc + row * a.kvr * D, *vh = a.vc + row * a.kvr * D;
+        const uint32_t *mask = a.sel_mask + bh * v.n_chunk_cap * (v.C / 32);
+        float *part = a.part + (bh * kRecords + slot) * (D + 2), *logits = a.part + (bh * kRecords + kLogitRecord) * (D + 2);
+        if constexpr (sizeof(T) == 2)
+            attend_segment<D, NT>(v, kh, vh, a.k + row * D, a.v + row * D, a.q + bh * D, mask, tile_lo, tile_hi, step_smem, part,
+                                  logits, kRecords * (D + 2));
+        else
+            attend_segment_f32<D>(v, kh, vh, a.k + row * D, a.v + row * D, a.q + bh * D, mask, tile_lo, tile_hi,
+                                  step_smem, part, logits, kRecords * (D + 2));
+        x = u * a.tiles + tile_hi;
+    }
+    if ((int)blockIdx.x < a.first_item_block) return;
+    using Ring = StepRing<T, D>;
+    if (a.item_warps == 1) work_on_items<T, D, 1, Ring>(a, step_smem);
+    else if (a.item_warps == 2) work_on_items<T, D, 2, Ring>(a, step_smem);
+    else work_on_items<T, D, kStepWarps, Ring>(a, step_smem);
+}
+
+// grid (H, B), D threads: one output column each.
+template <typename T, int D>
+__global__ void __launch_bounds__(D)
+step_merge_kernel(const __grid_constant__ StepArgs<T> a) {
+    __shared__ float wts[32];
+    grid_dep_wait();
+    grid_dep_launch();
+    if (a.hdr[14] != 0) return;   // mismatch recorded by the step's first kernel: no output, token count unchanged
+    const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, rep = a.H / a.Hkv;
+    const long long bh = (long long)b * a.H + h;
+    const long long u = ((long long)b * a.Hkv + h / rep) * a.units_per_group + h % rep / a.heads_per_unit;
+    const int n = unit_blocks(a.per, a.tiles, u);    // at most kMaxSplits
+    const float *pr = a.part + bh * kRecords * (D + 2);
+    if (h % rep == 0) {   // the new row of the K / V history (position p lives in ring row p % kvr)
+        const long long row = (long long)b * a.Hkv + h / rep, dst = (row * a.kvr + (uint32_t)a.t % (uint32_t)a.kvr) * D + tid;
+        a.kc[dst] = a.k[row * D + tid];
+        a.vc[dst] = a.v[row * D + tid];
+    }
+    float nla = 0.f, dla = 0.f;
+    if (a.la) {
+        nla = pr[kLinRecord * (D + 2) + 2 + tid];
+        dla = pr[kLinRecord * (D + 2) + 1];
+        if (a.g) nla *= ld_f(a.g + bh * D + tid);
+    }
+    // every warp forms the weights of the partials (at most 30)
+    const float ms = lane < n ? pr[lane * (D + 2)] : -INFINITY, ls = lane < n ? pr[lane * (D + 2) + 1] : 0.f;
+    const float M = warp_max(ms);
+    const float w = ms == -INFINITY ? 0.f : expf(ms - M);
+    const float L = warp_sum(ms == -INFINITY ? 0.f : w * ls);
+    if (tid < 32) wts[lane] = w;
+    __syncthreads();
+    float O = 0.f;
+#pragma unroll 4
+    for (int s = 0; s < n; ++s) {
+        const float ws = wts[s], x = pr[s * (D + 2) + 2 + tid];
+        if (ws != 0.f) O = fmaf(ws, x, O);
+    }
+    float fs = 1.f, fl = 0.f;
+    if (dla > 0.f) {
+        const float mm = fmaxf(M, 0.f);
+        fs = expf(M - mm);
+        fl = expf(-mm);
+    }
+    st_f(a.y + bh * D + tid, (O * fs + fl * nla) / (L * fs + fl * dla));
+    if (tid >= D - 32) {   // Self-Saliency Score of the new token: its window's logits lie in the head's last records
+        const int C = a.view.C;
+        float l[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int j = lane + 32 * i;
+            l[i] = j < C && a.view.t - (C - 1) + j >= 0 ? pr[kLogitRecord * (D + 2) + j] : -INFINITY;
+        }
+        const float sc = window_score(l, lane, C >> 5, C, a.eps);
+        if (lane == 0) a.score[bh * a.cap + a.t] = sc;
     }
     if (h == 0 && b == 0 && tid == 0) {
-        long long nt = t + 1;
-        hdr[12] = (int32_t)(nt & 0xffffffffll);
-        hdr[13] = (int32_t)(nt >> 32);
+        const long long nt = a.t + 1;
+        a.hdr[12] = (int32_t)(nt & 0xffffffffll);
+        a.hdr[13] = (int32_t)(nt >> 32);
     }
 }
 
@@ -402,95 +749,136 @@ step_merge_kernel(const float *__restrict__ part, const float *__restrict__ S,
         if (e__ != cudaSuccess) return STILL_ERR_CUDA; \
     } while (0)
 
+template <typename... Params, typename... Args>
+static cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+template <typename T>
+static int launch_route(const still_params_t *p, const StepArgs<T> &a, int32_t *sel, const T *Wk, const T *bk, long long cr,
+                        int window, cudaStream_t st, int *launches) {
+    const int C = p->chunk, d = p->d, df = p->d_f;
+    T *wk = const_cast<T *>(Wk), *bkp = const_cast<T *>(bk);
+    if constexpr (sizeof(T) == 2) {
+        auto launch = [&](auto kernel, int smem, int max_smem) -> int {
+            STILL_CUDA(ensure_dynamic_smem((const void *)kernel, max_smem));
+            STILL_CUDA(launch_dependent(kernel, dim3(p->H, p->B), dim3(256), smem, st, a.kc, a.vc, a.score, sel, a.sel_mask, a.S, a.z,
+                                        wk, bkp, a.hdr, a.key, p->H, p->Hkv, a.cap, a.kvr, df, C, p->topk, cr, window));
+            return STILL_OK;
+        };
+        const int rc = d == 64 ? launch(step_route_mma_kernel<64>, RoutePlan<64>(C, df).total, RoutePlan<64>(128, 64).total)
+                               : launch(step_route_mma_kernel<128>, RoutePlan<128>(C, df).total, RoutePlan<128>(128, 128).total);
+        if (rc != STILL_OK) return rc;
+    } else {
+        size_t smem = ((size_t)C * 2 * df + (size_t)C * d + 8 * (size_t)d + C) * 4 + (size_t)C * 4;
+        const int w_in_smem = smem + (size_t)d * df * sizeof(T) <= 200 * 1024 ? 1 : 0;
+        if (w_in_smem) smem += (size_t)d * df * sizeof(T);
+        STILL_CUDA(cudaFuncSetAttribute(step_route_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        STILL_CUDA(launch_dependent(step_route_kernel<T>, dim3(p->H, p->B), dim3(256), smem, st, a.kc, a.vc, a.score, sel, a.sel_mask,
+                                    a.S, a.z, wk, bkp, a.hdr, a.key, p->H, p->Hkv, a.cap, a.kvr, d, df, C, p->topk, cr, window,
+                                    w_in_smem));
+    }
+    ++*launches;
+    return STILL_OK;
+}
+
+template <typename T, int D, int NT>
+static int launch_main(const StepArgs<T> &a, unsigned grid, cudaStream_t st, int *launches) {
+    constexpr int kSmem = step_main_smem<T, D>();
+    STILL_CUDA(ensure_dynamic_smem((const void *)step_main_kernel<T, D, NT>, kSmem));
+    profile_mark_begin(st);
+    STILL_CUDA(launch_dependent(step_main_kernel<T, D, NT>, dim3(grid), dim3(kStepThreads), kSmem, st, a));
+    profile_mark_end(st);
+    STILL_CUDA(launch_dependent(step_merge_kernel<T, D>, dim3(a.H, a.B), dim3(D), 0, st, a));
+    *launches += 2;
+    return STILL_OK;
+}
+
 template <typename T>
 static int step_typed(const still_params_t *p, char *state, const still_state_layout_t *L, long long t,
                       const T *q, const T *k, const T *v, const T *g, const T *Wq, const T *bq,
                       const T *Wk, const T *bk, T *y, cudaStream_t st, int *launches) {
-    const int C = p->chunk, d = p->d, df = p->d_f, lam = p->topk;
-    const long long cap = L->capacity, kvr = state_kv_rows(p, cap);
-    T *kc = reinterpret_cast<T *>(state + L->k_cache), *vc = reinterpret_cast<T *>(state + L->v_cache);
-    float *score = reinterpret_cast<float *>(state + L->score);
-    int32_t *sel = reinterpret_cast<int32_t *>(state + L->sel_idx);
-    uint32_t *smask = reinterpret_cast<uint32_t *>(state + L->sel_mask);
-    float *S = reinterpret_cast<float *>(state + L->S), *z = reinterpret_cast<float *>(state + L->z);
-    float *part = reinterpret_cast<float *>(state + L->scratch);
-    int32_t *hdr = reinterpret_cast<int32_t *>(state + L->header);
+    const int C = p->chunk, d = p->d, df = p->d_f, lam = p->topk, rep = p->H / p->Hkv;
+    const long long cap = L->capacity;
     const int window = lam > 0 ? (int)(p->max_salient / lam) : 0;   // chunks whose selections the salient cache holds
-    const bool la = lam < C || window > 0;
-
-    const StateKey key{p->B, p->H, p->Hkv, p->d, p->d_f, p->chunk, p->topk, p->dtype, cap, t};
-    step_append_score_kernel<T><<<dim3(p->H, p->B), 32, 0, st>>>(kc, vc, score, hdr, q, k, v, key, p->H, p->Hkv,
-                                                                  cap, kvr, d, C, t, p->sm_scale, p->eps);
-    ++*launches;
-    STILL_CUDA(cudaGetLastError());
-
+    constexpr bool kBf16 = sizeof(T) == 2;
+    if (kBf16 && rep > 16) return STILL_ERR_UNSUPPORTED;            // the group's heads are two tiles of eight
     const long long c_cur = t / C;
+
+    StepArgs<T> a{};
+    a.kc = reinterpret_cast<T *>(state + L->k_cache);
+    a.vc = reinterpret_cast<T *>(state + L->v_cache);
+    a.score = reinterpret_cast<float *>(state + L->score);
+    a.sel_mask = reinterpret_cast<uint32_t *>(state + L->sel_mask);
+    a.S = reinterpret_cast<float *>(state + L->S);
+    a.z = reinterpret_cast<float *>(state + L->z);
+    a.part = reinterpret_cast<float *>(state + L->scratch);
+    a.hdr = reinterpret_cast<int32_t *>(state + L->header);
+    a.q = const_cast<T *>(q); a.k = const_cast<T *>(k); a.v = const_cast<T *>(v); a.g = const_cast<T *>(g);
+    a.Wq = const_cast<T *>(Wq); a.bq = const_cast<T *>(bq); a.y = y;
+    a.key = StateKey{p->B, p->H, p->Hkv, p->d, p->d_f, p->chunk, p->topk, p->dtype, cap, t};
+    a.cap = cap;
+    a.kvr = state_kv_rows(p, cap);
+    a.t = t;
+    a.B = p->B; a.H = p->H; a.Hkv = p->Hkv; a.df = df;
+    a.la = lam < C || window > 0;
+    a.eps = p->eps;
+    AttendView &w = a.view;
+    w.kvr = a.kvr;
+    w.t = (int)t;
+    w.loc0 = (int)(c_cur >= 1 ? (c_cur - 1) * C : 0);
+    // routed chunks still cached: all, with a budget the last `window` before the local region, none when topk = 0
+    w.first_pos = lam <= 0 ? w.loc0 : window > 0 ? (int)(std::max<long long>(0, c_cur - 1 - window) * C) : 0;
+    w.C = C; w.lam = lam; w.rep = rep; w.n_chunk_cap = (int)(cap / C);
+    w.scale = p->sm_scale;
+    w.scale_log2 = p->sm_scale * 1.4426950408889634f;
+
     if (t % C == 0 && c_cur >= 2) {
-        size_t smem = ((size_t)C * 2 * df + (size_t)C * d + 8 * (size_t)d + C) * 4 + (size_t)C * 4;
-        const int w_in_smem = smem + (size_t)d * df * sizeof(T) <= 200 * 1024 ? 1 : 0;
-        if (w_in_smem) smem += (size_t)d * df * sizeof(T);
-        STILL_CUDA(cudaFuncSetAttribute(step_route_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                        (int)smem));
-        step_route_kernel<T><<<dim3(p->H, p->B), 256, smem, st>>>(kc, vc, score, sel, smask, S, z, Wk, bk, hdr, p->H,
-                                                                  p->Hkv, cap, kvr, d, df, C, lam, c_cur - 2, window, w_in_smem);
-        ++*launches;
-        STILL_CUDA(cudaGetLastError());
+        const int rc = launch_route<T>(p, a, reinterpret_cast<int32_t *>(state + L->sel_idx), Wk, bk, c_cur - 2, window, st, launches);
+        if (rc != STILL_OK) return rc;
     }
 
-    const long long n_routed = (lam > 0 && c_cur >= 2) ? c_cur - 1 : 0;  // chunks 0..c_cur-2
-    int n_splits = 1;
-    if constexpr (sizeof(T) == 2) {
-        // bf16: tensor-core split-KV pass, the query heads of a KV group share every K / V row read
-        if (p->H / p->Hkv > 16) return STILL_ERR_UNSUPPORTED;  // the group's heads are the 16 rows of one MMA tile
-        // with a budget, the routed chunks still cached are the last `window` ones before the local region
-        const long long first_pos = window > 0 ? std::max<long long>(0, c_cur - 1 - window) * C : 0;
-        const long long nb = (t + 32) / 32 - first_pos / 32;  // 32-position key blocks
-        const long long groups = (long long)p->B * p->Hkv;
-        const long long want = (6 * 148 + groups - 1) / groups;  // about six waves of CTAs
-        n_splits = (int)std::max<long long>(1, std::min<long long>({want, (long long)kMaxSplits + 1, (nb + 3) / 4}));
-        dim3 grid(n_splits, p->Hkv, p->B);
-        const float scale_log2 = p->sm_scale * 1.4426950408889634f;
-        // a topk of 0 keeps nothing of the routed chunks: the kernel then sees only the local region
-        profile_mark_begin(st);
-        if (d == 64) {
-            STILL_CUDA(ensure_dynamic_smem((const void *)step_attend_mma_kernel<64>, AttendPlan<64>::kTotal));
-            step_attend_mma_kernel<64><<<grid, 128, AttendPlan<64>::kTotal, st>>>(
-                (const __nv_bfloat16 *)kc, (const __nv_bfloat16 *)vc, smask, (const __nv_bfloat16 *)q, part, hdr, p->H, p->Hkv,
-                cap, kvr, C, lam, t, first_pos, n_splits, kMaxSplits + 1, scale_log2);
+    int n_sm = 0, dev = 0;
+    STILL_CUDA(cudaGetDevice(&dev));
+    STILL_CUDA(cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev));
+    constexpr int kKeys = kBf16 ? kTileKeys : kTileKeysF32;
+    a.heads_per_unit = kBf16 ? rep : kUnitHeadsF32;
+    a.units_per_group = (rep + a.heads_per_unit - 1) / a.heads_per_unit;
+    a.tiles = (int)((t - w.first_pos) / kKeys) + 1;
+    a.total = (long long)p->B * p->Hkv * a.units_per_group * a.tiles;
+    a.n_items = a.la ? p->B * p->H : 0;
+    // Few read-outs (a sequence or two): a block each, beside the blocks of the cache pass.  More: every block takes its
+    // share of the tiles and then of the read-outs.
+    const bool apart = a.n_items <= n_sm / 2;
+    const long long blocks = apart ? n_sm - a.n_items : n_sm;
+    a.per = std::max<long long>({(a.total + blocks - 1) / blocks, (a.tiles + kMaxSplits - 2) / (kMaxSplits - 1), 1});
+    const long long used = (a.total + a.per - 1) / a.per;           // blocks with tiles
+    a.first_item_block = apart ? (int)used : 0;
+    // The fewer warps share a read-out, the more run side by side and the longer one takes.
+    a.item_warps = a.n_items <= n_sm ? kStepWarps : a.n_items <= n_sm * (kStepWarps / 2) ? 2 : 1;
+    const unsigned grid = (unsigned)(apart ? used + a.n_items : n_sm);
+    if (d == 64) {
+        if constexpr (kBf16) {
+            return rep <= 8 ? launch_main<T, 64, 1>(a, grid, st, launches) : launch_main<T, 64, 2>(a, grid, st, launches);
         } else {
-            STILL_CUDA(ensure_dynamic_smem((const void *)step_attend_mma_kernel<128>, AttendPlan<128>::kTotal));
-            step_attend_mma_kernel<128><<<grid, 128, AttendPlan<128>::kTotal, st>>>(
-                (const __nv_bfloat16 *)kc, (const __nv_bfloat16 *)vc, smask, (const __nv_bfloat16 *)q, part, hdr, p->H, p->Hkv,
-                cap, kvr, C, lam, t, first_pos, n_splits, kMaxSplits + 1, scale_log2);
+            return launch_main<T, 64, 1>(a, grid, st, launches);
         }
-        profile_mark_end(st);
-        ++*launches;
-        STILL_CUDA(cudaGetLastError());
-        n_splits -= 1;  // the merge kernel reads partials 0 .. n_splits inclusive
-    } else {
-        if (n_routed > 0) {
-            long long want = (2048 + (long long)p->B * p->Hkv - 1) / ((long long)p->B * p->Hkv);
-            n_splits = (int)std::max<long long>(1, std::min<long long>({want, (long long)kMaxSplits, n_routed}));
-        }
-        const long long cps = n_routed > 0 ? (n_routed + n_splits - 1) / n_splits : 1;
-        dim3 grid(n_splits + 1, p->Hkv, p->B);
-        profile_mark_begin(st);
-        if (d == 64)
-            step_attend_kernel<T, 2><<<grid, 128, 0, st>>>(kc, vc, sel, q, part, hdr, p->H, p->Hkv, cap, C, lam, t,
-                                                           n_splits, cps, n_routed, p->sm_scale);
-        else
-            step_attend_kernel<T, 4><<<grid, 128, 0, st>>>(kc, vc, sel, q, part, hdr, p->H, p->Hkv, cap, C, lam, t,
-                                                           n_splits, cps, n_routed, p->sm_scale);
-        profile_mark_end(st);
-        ++*launches;
-        STILL_CUDA(cudaGetLastError());
     }
-
-    step_merge_kernel<T><<<dim3(p->H, p->B), 128, 0, st>>>(part, S, z, q, g, Wq, bq, y, hdr, p->H, d, df,
-                                                           n_splits, la ? 1 : 0, t);
-    ++*launches;
-    STILL_CUDA(cudaGetLastError());
-    return STILL_OK;
+    if constexpr (kBf16) {
+        return rep <= 8 ? launch_main<T, 128, 1>(a, grid, st, launches) : launch_main<T, 128, 2>(a, grid, st, launches);
+    } else {
+        return launch_main<T, 128, 1>(a, grid, st, launches);
+    }
 }
 
 int step_launch(const still_params_t *p, char *state, const still_state_layout_t *L, long long t_pos,

@@ -1,16 +1,20 @@
 // Split-KV pass of the decode step for bf16 (Sec. 3.3: N_SA, D_SA over the salient cache h_t).
 //
-// HBM-bound: every step reads the K and V history once.  One CTA serves one (batch, KV head) and a
-// range of 32-position key blocks; the query heads of the group (at most 16) are the rows of one
-// m16n8k16 tensor-core tile, so the K / V rows are read once for the whole group.  Which rows a
-// query head sees is a per-head membership mask: for a position in a routed chunk, whether the
-// head's selection (the sel_mask words of the decode state) contains it; for the two-chunk local region, every position up to the
-// new token.  Key blocks are streamed by 16-byte cp.async into padded shared-memory rows, two stages per
-// warp; a row is read from memory only if some head of the group selected it (the union of the group's
-// salient caches, read once for the group rather than once per head) and gets weight zero for the heads
-// that did not; with topk = chunk that is every row.
-// Each warp runs its own online softmax over its blocks; the four warps are merged through shared
-// memory and the CTA writes one partial (max, sum, numerator) per head and split.
+// HBM-bound: every step reads the K and V history once, for all query heads of a KV group together.  The history of
+// a group is cut into tiles of 16 positions; a warp takes every eighth tile of its block's range through a ring of
+// 16-byte cp.async stages (no padding: the 16-byte pieces of a row are XOR-swizzled by the row, so that the copies and
+// the ldmatrix reads are free of bank conflicts).  Keys are the rows of the tensor-core tiles and the group's query
+// heads their columns -- S^T = K Q^T, then O^T += V^T P^T -- because a group has at most 16 heads and usually four:
+// as rows of an m16n8k16 they would fill a quarter of the tile, as columns they fill half.  P^T changes from an
+// accumulator to an operand fragment by one movmatrix per eight keys, without shared memory.
+//
+// Which rows a query head sees is a per-head membership mask: for a position in a routed chunk, whether the head's
+// selection (the sel_mask words of the decode state) contains it; for the two-chunk local region, every position up
+// to the new token.  A row is read from memory only if some head of the group selected it; with topk = chunk that is
+// every row.  A tile without a new maximum (most of them, past the first few) costs one vote instead of a reduction and
+// a rescaling of O.  (Raising the maximum only when it is exceeded by 2^8, as the prefill does, gained nothing here and
+// cost precision: the largest weight is then no longer exactly one when it is rounded to bf16, and the output's error
+// against 64 bits grew from 2.0e-3 to 2.3e-3.)
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -30,12 +34,12 @@ __device__ __forceinline__ void cp_async_wait() { asm volatile("cp.async.wait_gr
 __device__ __forceinline__ void ldmatrix_x4(uint32_t (&r)[4], const void *p) {
     const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p));
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
 }
 __device__ __forceinline__ void ldmatrix_x4_trans(uint32_t (&r)[4], const void *p) {
     const uint32_t a = static_cast<uint32_t>(__cvta_generic_to_shared(p));
     asm volatile("ldmatrix.sync.aligned.m8n8.x4.trans.shared.b16 {%0, %1, %2, %3}, [%4];"
-                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a));
+                 : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]) : "r"(a) : "memory");
 }
 // D (16x8, fp32) += A (16x16, bf16, row) * B (16x8, bf16, col)
 __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4], uint32_t b0, uint32_t b1) {
@@ -43,6 +47,12 @@ __device__ __forceinline__ void mma_16816(float (&c)[4], const uint32_t (&a)[4],
                  "{%0, %1, %2, %3};"
                  : "+f"(c[0]), "+f"(c[1]), "+f"(c[2]), "+f"(c[3])
                  : "r"(a[0]), "r"(a[1]), "r"(a[2]), "r"(a[3]), "r"(b0), "r"(b1));
+}
+// Transpose of an 8x8 matrix of 16-bit elements held one row per four lanes.
+__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
+    uint32_t r;
+    asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(r) : "r"(a));
+    return r;
 }
 __device__ __forceinline__ float ex2_approx(float x) {
     float y;
@@ -55,237 +65,265 @@ __device__ __forceinline__ uint32_t pack2_bf16(float lo, float hi) {
     return r;
 }
 
-template <int D>
-struct AttendPlan {
-    static constexpr int kRow = D * 2 + 16;          // padded row: ldmatrix without bank conflicts
-    static constexpr int kTile = 32 * kRow;          // 32 keys
-    static constexpr int kStage = 2 * kTile;         // K and V
-    static constexpr int kWarp = 2 * kStage;         // two stages
-    static constexpr int kTotal = 4 * kWarp;
+// Geometry of a decode step's cache pass (see step_main_kernel).
+struct AttendView {
+    long long kvr;       // ring rows per KV head
+    int first_pos, t;    // first position read, position of the new token
+    int loc0;            // first position of the local region
+    int C, lam, rep, n_chunk_cap;
+    float scale, scale_log2;
 };
 
-// grid (n_splits, Hkv, B), 128 threads.  first_pos: a multiple of the chunk size.  part: [B*H][max_splits][D + 2] = running max (natural
-// log units), sum, numerator.
+constexpr int kStepWarps = 8;
+constexpr int kTileKeys = 16;
+
 template <int D>
-__global__ void __launch_bounds__(128)
-step_attend_mma_kernel(const __nv_bfloat16 *__restrict__ kc, const __nv_bfloat16 *__restrict__ vc,
-                       const uint32_t *__restrict__ sel_mask, const __nv_bfloat16 *__restrict__ q,
-                       float *__restrict__ part, const int32_t *__restrict__ hdr, int H, int Hkv, long long cap, long long kvr, int C,
-                       int lam, long long t, long long first_pos, int n_splits, int max_splits, float scale_log2) {
+struct AttendPlan {
+    static constexpr int kRow = D * 2;                     // bytes of a row
+    static constexpr int kPieces = D / 8;                  // 16-byte pieces of a row
+    static constexpr int kTile = kTileKeys * kRow;         // K or V rows of a tile
+    static constexpr int kStage = 2 * kTile;
+    static constexpr int kStages = D == 128 ? 3 : 4;       // per warp: 24 KB / 16 KB, 196 KB / 131 KB a block
+    static constexpr int kWarp = kStages * kStage;
+    static constexpr int kTotal = kStepWarps * kWarp;
+};
+
+// Tiles [tile_lo, tile_hi) of one KV head by one block of 8 warps.  kh, vh: the head's rows; k_new, v_new: the new
+// token's (position t is read from the call's inputs, not from the row that another block is writing); qh: the
+// group's queries; mask: sel_mask of the group's first head.  Leaves one record per head (maximum in natural-log
+// units, sum, numerator [D]) at part + head * part_stride, and the new token's logits against the last C positions,
+// oldest first, at logits + head * part_stride.  NT: tiles of 8 heads.
+template <int D, int NT>
+__device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_bfloat16 *kh, const __nv_bfloat16 *vh,
+                                               const __nv_bfloat16 *k_new, const __nv_bfloat16 *v_new,
+                                               const __nv_bfloat16 *qh, const uint32_t *mask, int tile_lo, int tile_hi,
+                                               uint8_t *smem, float *part, float *logits, long long part_stride) {
     using P = AttendPlan<D>;
-    extern __shared__ __align__(16) uint8_t attend_smem[];
-    if (hdr[14] != 0) return;   // the step's first kernel found the state not to match the call
-    uint8_t *smem = attend_smem;
-    const int split = blockIdx.x, kv = blockIdx.y, b = blockIdx.z, rep = H / Hkv;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int g = lane >> 2, tig = lane & 3;          // fragment row (and row + 8), column pair
-    // K / V rows live in a ring of kvr rows per KV head (position p in row p % kvr; kvr is a multiple of the chunk
-    // size, so a 32-position block never straddles the end)
-    const __nv_bfloat16 *kh = kc + ((long long)b * Hkv + kv) * kvr * D;
-    const __nv_bfloat16 *vh = vc + ((long long)b * Hkv + kv) * kvr * D;
+    const int g = lane >> 2, tig = lane & 3;
     uint8_t *my = smem + warp * P::kWarp;
 
-    const long long c_cur = t / C;
-    const long long loc0 = c_cur >= 1 ? (c_cur - 1) * C : 0;   // first position of the local region
-    const int n_chunk_cap = (int)(cap / C);
-    // key blocks covering positions first_pos..t (first_pos > 0 with a salient-cache budget: older chunks have
-    // left the cache for the linear state)
-    const int kb0 = (int)(first_pos / 32), nb = (int)((t + 32) / 32);
-    const int per = (nb - kb0 + n_splits - 1) / n_splits;
-    const int kb_lo = kb0 + split * per, kb_hi = min(nb, kb_lo + per);
-
-    // Q fragments of the group's heads (rows >= rep are zero)
-    uint32_t qa[D / 16][4];
-    {
-        const long long hq = (long long)b * H + (long long)kv * rep;
+    // Q^T as B fragments: columns are heads (head >= rep: zero)
+    uint32_t qb[NT][D / 16][2];
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks) {
-            const int col = ks * 16 + tig * 2;
-            qa[ks][0] = g < rep ? *reinterpret_cast<const uint32_t *>(q + (hq + g) * D + col) : 0u;
-            qa[ks][1] = g + 8 < rep ? *reinterpret_cast<const uint32_t *>(q + (hq + g + 8) * D + col) : 0u;
-            qa[ks][2] = g < rep ? *reinterpret_cast<const uint32_t *>(q + (hq + g) * D + col + 8) : 0u;
-            qa[ks][3] = g + 8 < rep ? *reinterpret_cast<const uint32_t *>(q + (hq + g + 8) * D + col + 8) : 0u;
+            const int h = nt * 8 + g, col = ks * 16 + tig * 2;
+            qb[nt][ks][0] = h < v.rep ? *reinterpret_cast<const uint32_t *>(qh + h * D + col) : 0u;
+            qb[nt][ks][1] = h < v.rep ? *reinterpret_cast<const uint32_t *>(qh + h * D + col + 8) : 0u;
         }
+    float o[NT][D / 16][4];
+    float m_run[NT][2], l_run[NT][2];   // of heads 8 nt + 2 tig and + 1, log2 domain; l: this thread's keys only
+#pragma unroll
+    for (int nt = 0; nt < NT; ++nt) {
+#pragma unroll
+        for (int i = 0; i < D / 16; ++i) o[nt][i][0] = o[nt][i][1] = o[nt][i][2] = o[nt][i][3] = 0.f;
+        m_run[nt][0] = m_run[nt][1] = -INFINITY;
+        l_run[nt][0] = l_run[nt][1] = 0.f;
     }
-    float o[D / 8][4];
-#pragma unroll
-    for (int i = 0; i < D / 8; ++i) o[i][0] = o[i][1] = o[i][2] = o[i][3] = 0.f;
-    float m_run[2] = {-INFINITY, -INFINITY}, l_run[2] = {0.f, 0.f};   // rows g and g + 8, log2 domain
 
-    // Rows of a block that no query head of the group sees are not read from memory (a zero-filling copy with
-    // no source bytes): with topk < chunk only the union of the group's selections crosses HBM.
-    auto load_block = [&](int kb, int stage, uint32_t rows_needed) {
+    // Membership of tile j's 16 positions (bits 0-15) for the head in this lane (lanes >= group size: 0).
+    auto member_word = [&](int j) -> uint32_t {
+        if (j >= tile_hi || lane >= v.rep) return 0u;
+        const int p0 = v.first_pos + j * kTileKeys;
+        if (p0 >= v.loc0) {
+            const int last = v.t - p0;   // positions up to the new token
+            return last >= 15 ? 0xffffu : ((1u << (last + 1)) - 1u);
+        }
+        if (v.lam >= v.C) return 0xffffu;
+        // (chunk sizes are multiples of 32: words run on from chunk to chunk)
+        return mask[(long long)lane * v.n_chunk_cap * (v.C / 32) + (p0 >> 5)] >> (p0 & 16) & 0xffffu;
+    };
+    const int c_piece = lane % P::kPieces, c_row = lane / P::kPieces;   // this lane's piece and first row of a copy
+    constexpr int kRowsPerIt = 32 / P::kPieces;
+    auto load_tile = [&](int j, int stage, uint32_t rows) {
         uint8_t *ks = my + stage * P::kStage, *vs = ks + P::kTile;
-        constexpr int kChunksPerRow = D / 8;
-        const long long p0 = (long long)kb * 32;
-        const long long r0 = p0 % kvr;   // ring row of the block's first position (one division per block)
+        const int p0 = v.first_pos + j * kTileKeys;
+        // position p lives in ring row p % kvr; kvr is a multiple of the chunk size, so a tile never straddles the end
+        const long long r0 = (uint32_t)p0 % (uint32_t)v.kvr;
+        const __nv_bfloat16 *kp = kh + (r0 + c_row) * D + c_piece * 8, *vp = vh + (r0 + c_row) * D + c_piece * 8;
+        const int t_row = v.t - p0;   // row of the new token if it lies in this tile
 #pragma unroll
-        for (int i = lane; i < 32 * kChunksPerRow; i += 32) {
-            const int row = i / kChunksPerRow, ch = i % kChunksPerRow;
-            const bool valid = (rows_needed >> row) & 1u;
-            const long long src = (valid ? r0 + row : 0) * D + ch * 8;
-            cp_async16(ks + row * P::kRow + ch * 16, kh + src, valid);
-            cp_async16(vs + row * P::kRow + ch * 16, vh + src, valid);
+        for (int it = 0; it < kTileKeys / kRowsPerIt; ++it) {
+            const int row = it * kRowsPerIt + c_row;
+            const int dst = row * P::kRow + ((c_piece ^ (row & 7)) << 4);
+            const bool valid = (rows >> row) & 1u;
+            const bool is_new = row == t_row;
+            cp_async16(ks + dst, is_new ? k_new + c_piece * 8 : kp + it * kRowsPerIt * D, valid);
+            cp_async16(vs + dst, is_new ? v_new + c_piece * 8 : vp + it * kRowsPerIt * D, valid);
         }
-    };
-    // Membership word of block kb for the head in this lane (lanes >= group size: 0): bit j = position 32 kb + j is
-    // visible to the head.  Local region: every position up to the new token; routed chunks: the head's selection
-    // (bit masks written when the chunk was routed), all of it when topk = chunk.
-    auto member_word = [&](int kb) -> uint32_t {
-        if (kb >= kb_hi || lane >= rep) return 0u;
-        const long long p0 = (long long)kb * 32;
-        if (p0 >= loc0) {
-            const long long last = t - p0;   // positions up to the new token
-            return last >= 31 ? 0xffffffffu : ((1u << (int)(last + 1)) - 1u);
-        }
-        if (lam >= C) return 0xffffffffu;
-        if (lam <= 0) return 0u;
-        const int chunk = (int)(p0 / C), word = (int)((p0 % C) / 32);
-        return sel_mask[(((long long)b * H + (long long)kv * rep + lane) * n_chunk_cap + chunk) * (C / 32) + word];
     };
 
-    // The membership words run two blocks ahead of the compute and one ahead of the copies they steer.
-    const int first = kb_lo + warp;
-    uint32_t m_cur = member_word(first), m_next = member_word(first + 4);
-    if (first < kb_hi) load_block(first, 0, __reduce_or_sync(0xffffffffu, m_cur));
-    cp_async_commit();
-    int it = 0;
-    for (int kb = first; kb < kb_hi; kb += 4, ++it) {
-        const int stage = it & 1;
-        const uint32_t m_after = member_word(kb + 8);
-        if (kb + 4 < kb_hi) load_block(kb + 4, stage ^ 1, __reduce_or_sync(0xffffffffu, m_next));
+    // ring: kStages - 1 tiles in flight; membership words run one tile ahead of the copies they steer
+    constexpr int kAhead = P::kStages - 1;
+    uint32_t words[kAhead + 1];   // words[i]: tile (current + i) of this warp
+    const int first = tile_lo + warp;
+#pragma unroll
+    for (int i = 0; i <= kAhead; ++i) words[i] = member_word(first + kStepWarps * i);
+#pragma unroll
+    for (int i = 0; i < kAhead; ++i) {
+        if (first + kStepWarps * i < tile_hi) load_tile(first + kStepWarps * i, i, __reduce_or_sync(0xffffffffu, words[i]));
         cp_async_commit();
-
-        // membership of the block's 32 positions for rows g and g + 8 (bit j: position 32 kb + j)
-        uint32_t vis[2];
-        vis[0] = __shfl_sync(0xffffffffu, m_cur, g);
-        vis[1] = __shfl_sync(0xffffffffu, m_cur, g + 8);
-        m_cur = m_next;
-        m_next = m_after;
-        cp_async_wait<1>();
+    }
+    int stage = 0;
+    for (int j = first; j < tile_hi; j += kStepWarps) {
+        const uint32_t after = member_word(j + kStepWarps * (kAhead + 1));
+        {
+            int ps = stage + kAhead;
+            if (ps >= P::kStages) ps -= P::kStages;
+            const int jn = j + kStepWarps * kAhead;
+            if (jn < tile_hi) load_tile(jn, ps, __reduce_or_sync(0xffffffffu, words[kAhead]));
+            cp_async_commit();
+        }
+        const uint32_t word = words[0];
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) words[i] = words[i + 1];
+        words[kAhead] = after;
+        cp_async_wait<kAhead>();
         __syncwarp();
         const uint8_t *ks = my + stage * P::kStage, *vs = ks + P::kTile;
 
-        // S = Q K^T for 32 keys: 4 n-tiles of 8 keys
-        float s[4][4];
+        // S^T = K Q^T: rows are keys g and g + 8, columns heads 2 tig and 2 tig + 1.  Two chains of products, of even and
+        // odd k-steps: half the latency, and fewer roundings in a row.
+        float s[NT][4], s_odd[NT][4];
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt) s[nt][0] = s[nt][1] = s[nt][2] = s[nt][3] = 0.f;
+        for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
-        for (int ks16 = 0; ks16 < D / 16; ++ks16) {
+            for (int e = 0; e < 4; ++e) s[nt][e] = s_odd[nt][e] = 0.f;
 #pragma unroll
-            for (int np = 0; np < 2; ++np) {
-                // matrices: (keys 16 np .. +8, d lo), (same keys, d hi), (keys 16 np + 8 .., d lo), (.., d hi)
-                uint32_t bfr[4];
-                const int key = np * 16 + ((lane >> 4) << 3) + (lane & 7);
-                const int dcol = ks16 * 16 + (((lane >> 3) & 1) << 3);
-                ldmatrix_x4(bfr, ks + key * P::kRow + dcol * 2);
-                mma_16816(s[np * 2], qa[ks16], bfr[0], bfr[1]);
-                mma_16816(s[np * 2 + 1], qa[ks16], bfr[2], bfr[3]);
+        for (int k16 = 0; k16 < D / 16; ++k16) {
+            uint32_t a[4];
+            const int row = ((lane >> 3) & 1) * 8 + (lane & 7), piece = k16 * 2 + (lane >> 4);
+            ldmatrix_x4(a, ks + row * P::kRow + ((piece ^ (row & 7)) << 4));
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) mma_16816(k16 & 1 ? s_odd[nt] : s[nt], a, qb[nt][k16][0], qb[nt][k16][1]);
+        }
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) s[nt][e] += s_odd[nt][e];
+        const int slot0 = v.first_pos + j * kTileKeys - (v.t - (v.C - 1));   // slot of the tile's first key in the window
+        if (slot0 > -kTileKeys) {
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt)
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    const int h = nt * 8 + tig * 2 + (e & 1), sl = slot0 + g + (e >> 1) * 8;
+                    if (h < v.rep && sl >= 0 && sl < v.C) logits[h * part_stride + sl] = s[nt][e] * v.scale;
+                }
+        }
+        bool grow = false;
+#pragma unroll
+        for (int nt = 0; nt < NT; ++nt) {
+#pragma unroll
+            for (int hh = 0; hh < 2; ++hh) {
+                const uint32_t vis = __shfl_sync(0xffffffffu, word, nt * 8 + tig * 2 + hh);
+                s[nt][hh] = (vis >> g) & 1u ? s[nt][hh] * v.scale_log2 : -INFINITY;
+                s[nt][2 + hh] = (vis >> (g + 8)) & 1u ? s[nt][2 + hh] * v.scale_log2 : -INFINITY;
+                grow |= fmaxf(s[nt][hh], s[nt][2 + hh]) > m_run[nt][hh];
             }
         }
-        // mask, scale, online softmax (rows g and g + 8; a thread holds columns 8 nt + 2 tig + {0, 1})
-        float mx[2] = {-INFINITY, -INFINITY};
+        if (__any_sync(0xffffffffu, grow)) {
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt)
+            for (int nt = 0; nt < NT; ++nt) {
+                float alpha[2];
 #pragma unroll
-            for (int e = 0; e < 4; ++e) {
-                const int col = nt * 8 + tig * 2 + (e & 1), hr = e >> 1;
-                const bool on = (vis[hr] >> col) & 1u;
-                s[nt][e] = on ? s[nt][e] * scale_log2 : -INFINITY;
-                mx[hr] = fmaxf(mx[hr], s[nt][e]);
+                for (int hh = 0; hh < 2; ++hh) {
+                    float mx = fmaxf(s[nt][hh], s[nt][2 + hh]);
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+                    const float mn = fmaxf(m_run[nt][hh], mx);
+                    alpha[hh] = (mn == -INFINITY) ? 1.f : ex2_approx(m_run[nt][hh] - mn);
+                    m_run[nt][hh] = mn;
+                    l_run[nt][hh] *= alpha[hh];
+                }
+#pragma unroll
+                for (int i = 0; i < D / 16; ++i) {
+                    o[nt][i][0] *= alpha[0];
+                    o[nt][i][1] *= alpha[1];
+                    o[nt][i][2] *= alpha[0];
+                    o[nt][i][3] *= alpha[1];
+                }
             }
-        float alpha[2];
-#pragma unroll
-        for (int hr = 0; hr < 2; ++hr) {
-            mx[hr] = fmaxf(mx[hr], __shfl_xor_sync(0xffffffffu, mx[hr], 1));
-            mx[hr] = fmaxf(mx[hr], __shfl_xor_sync(0xffffffffu, mx[hr], 2));
-            const float mn = fmaxf(m_run[hr], mx[hr]);
-            alpha[hr] = (mn == -INFINITY) ? 1.f : ex2_approx(m_run[hr] - mn);
-            m_run[hr] = mn;
         }
-        float ls[2] = {0.f, 0.f};
-        uint32_t pa[2][4];   // P as A fragments of the two 16-key k-steps
+        uint32_t pb[NT][2];   // P^T as B fragments
 #pragma unroll
-        for (int nt = 0; nt < 4; ++nt) {
+        for (int nt = 0; nt < NT; ++nt) {
             float pv[4];
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
-                const int hr = e >> 1;
-                pv[e] = (m_run[hr] == -INFINITY) ? 0.f : ex2_approx(s[nt][e] - m_run[hr]);
-                ls[hr] += pv[e];
+                const float m = m_run[nt][e & 1];
+                pv[e] = (m == -INFINITY) ? 0.f : ex2_approx(s[nt][e] - m);
             }
-            pa[nt >> 1][(nt & 1) * 2 + 0] = pack2_bf16(pv[0], pv[1]);   // row g
-            pa[nt >> 1][(nt & 1) * 2 + 1] = pack2_bf16(pv[2], pv[3]);   // row g + 8
+            l_run[nt][0] += pv[0] + pv[2];
+            l_run[nt][1] += pv[1] + pv[3];
+            pb[nt][0] = movmatrix_trans(pack2_bf16(pv[0], pv[1]));
+            pb[nt][1] = movmatrix_trans(pack2_bf16(pv[2], pv[3]));
         }
+        // O^T += V^T P^T: rows are value columns
 #pragma unroll
-        for (int hr = 0; hr < 2; ++hr) {
-            ls[hr] += __shfl_xor_sync(0xffffffffu, ls[hr], 1);
-            ls[hr] += __shfl_xor_sync(0xffffffffu, ls[hr], 2);
-            l_run[hr] = l_run[hr] * alpha[hr] + ls[hr];
+        for (int dt = 0; dt < D / 16; ++dt) {
+            uint32_t a[4];
+            const int row = (lane >> 4) * 8 + (lane & 7), piece = dt * 2 + ((lane >> 3) & 1);
+            ldmatrix_x4_trans(a, vs + row * P::kRow + ((piece ^ (row & 7)) << 4));
+#pragma unroll
+            for (int nt = 0; nt < NT; ++nt) mma_16816(o[nt][dt], a, pb[nt][0], pb[nt][1]);
         }
-#pragma unroll
-        for (int dt = 0; dt < D / 8; ++dt) {
-            o[dt][0] *= alpha[0];
-            o[dt][1] *= alpha[0];
-            o[dt][2] *= alpha[1];
-            o[dt][3] *= alpha[1];
-        }
-        // O += P V: k-steps of 16 keys, n-tiles of 8 value columns
-#pragma unroll
-        for (int kk = 0; kk < 2; ++kk) {
-#pragma unroll
-            for (int dp = 0; dp < D / 16; ++dp) {
-                // matrices (transposed on load): (keys 16 kk .. +8, d 16 dp ..), (keys + 8, same d),
-                // (keys, d + 8), (keys + 8, d + 8)
-                uint32_t bfr[4];
-                const int key = kk * 16 + (((lane >> 3) & 1) << 3) + (lane & 7);
-                const int dcol = dp * 16 + ((lane >> 4) << 3);
-                ldmatrix_x4_trans(bfr, vs + key * P::kRow + dcol * 2);
-                mma_16816(o[dp * 2], pa[kk], bfr[0], bfr[1]);
-                mma_16816(o[dp * 2 + 1], pa[kk], bfr[2], bfr[3]);
-            }
-        }
-        __syncwarp();
+        __syncwarp();   // the stage may be overwritten
+        if (++stage == P::kStages) stage = 0;
     }
     cp_async_wait<0>();
     __syncthreads();
 
-    // merge the four warps: smem [4 warps][16 rows][D + 2]
+    // merge the eight warps: [8 warps][rep][D + 2] in shared memory
     float *mg = reinterpret_cast<float *>(smem);
     constexpr int kStride = D + 2;
+    const int rep = v.rep;
 #pragma unroll
-    for (int hr = 0; hr < 2; ++hr) {
-        const int row = g + hr * 8;
-        float *dst = mg + (warp * 16 + row) * kStride;
-        if (tig == 0) {
-            dst[0] = m_run[hr];
-            dst[1] = l_run[hr];
-        }
+    for (int nt = 0; nt < NT; ++nt) {
 #pragma unroll
-        for (int dt = 0; dt < D / 8; ++dt) {
-            dst[2 + dt * 8 + tig * 2] = o[dt][hr * 2];
-            dst[2 + dt * 8 + tig * 2 + 1] = o[dt][hr * 2 + 1];
+        for (int hh = 0; hh < 2; ++hh) {
+            const int h = nt * 8 + tig * 2 + hh;
+            float l = l_run[nt][hh];
+            l += __shfl_xor_sync(0xffffffffu, l, 4);
+            l += __shfl_xor_sync(0xffffffffu, l, 8);
+            l += __shfl_xor_sync(0xffffffffu, l, 16);
+            if (h < rep) {
+                float *dst = mg + (warp * rep + h) * kStride;
+                if (g == 0) {
+                    dst[0] = m_run[nt][hh];
+                    dst[1] = l;
+                }
+#pragma unroll
+                for (int dt = 0; dt < D / 16; ++dt) {
+                    dst[2 + dt * 16 + g] = o[nt][dt][hh];
+                    dst[2 + dt * 16 + g + 8] = o[nt][dt][2 + hh];
+                }
+            }
         }
     }
     __syncthreads();
-    for (int idx = threadIdx.x; idx < rep * kStride; idx += blockDim.x) {
-        const int row = idx / kStride, col = idx % kStride;
-        float M = -INFINITY;
+    for (int idx = threadIdx.x; idx < rep * kStride; idx += kStepWarps * 32) {
+        const int h = idx / kStride, col = idx % kStride;
+        float mw[kStepWarps], M = -INFINITY;
 #pragma unroll
-        for (int w = 0; w < 4; ++w) M = fmaxf(M, mg[(w * 16 + row) * kStride]);
+        for (int w = 0; w < kStepWarps; ++w) {
+            mw[w] = mg[(w * rep + h) * kStride];
+            M = fmaxf(M, mw[w]);
+        }
         float acc = 0.f;
         if (col == 0) {
             acc = M * 0.6931471805599453f;   // the merge kernel works in natural-log units
         } else {
 #pragma unroll
-            for (int w = 0; w < 4; ++w) {
-                const float mw = mg[(w * 16 + row) * kStride];
-                if (mw != -INFINITY) acc += ex2_approx(mw - M) * mg[(w * 16 + row) * kStride + col];
-            }
+            for (int w = 0; w < kStepWarps; ++w)
+                if (mw[w] != -INFINITY) acc += ex2_approx(mw[w] - M) * mg[(w * rep + h) * kStride + col];
         }
-        const long long bh = (long long)b * H + (long long)kv * rep + row;
-        part[(bh * max_splits + split) * kStride + col] = acc;
+        part[h * part_stride + col] = acc;
     }
+    __syncthreads();   // the staging space is the next segment's ring
 }
 
 }  // namespace still

@@ -179,6 +179,45 @@ def test_c5_full_size_sampled(k, steps):
     _decode_case(w, w.N, steps, n_heads=4 if k == 64 else 3, want_y=False)
 
 
+@pytest.mark.parametrize("dtype,B,H,Hkv,d,C,k,n0,steps", [
+    ("bf16", 40, 16, 4, 64, 32, 8, 70, 40),     # 640 read-outs: a warp each
+    ("bf16", 12, 16, 2, 128, 64, 16, 130, 70),  # 192 read-outs: two warps each; blocks span several groups
+    ("bf16", 1, 1, 1, 64, 32, 8, 2100, 40),     # one group, cut into as many partials as the scratch holds
+    ("fp32", 2, 20, 2, 64, 32, 8, 70, 40),      # ten heads per group: units of four, four and two
+    ("fp32", 1, 1, 1, 128, 64, 16, 1500, 70),
+])
+def test_decode_splits(dtype, B, H, Hkv, d, C, k, n0, steps):
+    _decode_case(synth.Workload("t", B, H, Hkv, d, n0, C, k, dtype, "iid", 1234), n0, steps, gate=True)
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("d,df,C,k,budget", [(64, 32, 32, 8, 0), (128, 32, 128, 16, 0), (128, 64, 64, 16, 32), (128, 128, 32, 4, 0)])
+def test_decode_feature_sizes_and_bias(dtype, d, df, C, k, budget):
+    # narrower maps than the head and a bias, through routing and read-out
+    if dtype == "fp32":
+        budget = 0
+    B, H, Hkv, n0, steps = 1, 4, 2, 2 * C + 5, 2 * C
+    w = synth.Workload("t", B, H, Hkv, d, n0 + steps, C, k, dtype, "iid", 8)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    g = torch.Generator(device="cuda").manual_seed(9)
+    mk = lambda *s: (torch.randn(*s, generator=g, device="cuda") * 0.05).to(w.torch_dtype)  # noqa: E731
+    Wq, Wk, bq, bk = mk(H, d, df), mk(Hkv, d, df), mk(H, df), mk(Hkv, df)
+    p = still.StillParams(B, H, Hkv, d, C, k, w.torch_dtype, d_f=df, sm_scale=w.sm_scale, max_salient=budget)
+    cap, lay = w.N, still.state_layout(p, w.N)
+    state = torch.zeros(lay["total"], dtype=torch.uint8, device="cuda")
+    cut = lambda x: x[:, :, :n0].contiguous()  # noqa: E731
+    still.hybrid_attn_fwd(p, cut(Q), cut(K), cut(V), Wq, Wk, bq=bq, bk=bk, state=state, state_max_tokens=cap)
+    Y = torch.stack([still.hybrid_attn_step(p, state, cap, t, *(x[:, :, t].contiguous() for x in (Q, K, V)), Wq, Wk, bq=bq, bk=bk)
+                     for t in range(n0, w.N)], 2)
+    scores = state[lay["score"]: lay["score"] + B * H * lay["capacity"] * 4].view(torch.float32).view(B, H, -1)[:, :, : w.N]
+    hp = oracle.HeadParams(C, k, w.sm_scale, max_salient=budget)
+    for h in range(H):
+        forced = oracle.select(scores[0, h].cpu().numpy().astype(np.float64), C, k)
+        out = oracle.chunkwise(U.f64(Q[0, h]), U.f64(K[0, h // 2]), U.f64(V[0, h // 2]), U.f64(Wq[h]), U.f64(Wk[h // 2]), hp,
+                               bq=U.f64(bq[h]), bk=U.f64(bk[h // 2]), forced_idx=forced, rows=list(range(n0, w.N)))
+        assert np.abs(U.f64(Y[0, h]) - out["y"]).max() <= U.TOL[w.torch_dtype]
+
+
 def test_state_full_and_mismatch():
     w = synth.Workload("t", 1, 2, 2, 64, 64, 32, 8, "bf16", "iid", 5)
     p = U.params_of(w)
