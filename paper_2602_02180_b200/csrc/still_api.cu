@@ -60,6 +60,7 @@ static inline bool la_active(const still_params_t *p) { return p->topk < p->chun
 struct FwdPlan {
     size_t status, scores, sel_idx, phiQ, phiK, csum, zpre, segs, nla, dla, ypart, dpart, ksel, vsel, phiKsel, total;
     long long T, sel_rows;  // chunks; rows of the compacted salient K/V per head
+    int n_seg;              // segments of the fp32 scan
     bool la, tc, tc_la;
 };
 
@@ -109,6 +110,16 @@ static FwdPlan plan_fwd(const still_params_t *p, long long N) {
             // (with a budget: phi(K) of the selected rows, from which the leaving tokens enter the state)
             if (w.tc_la && p->max_salient > 0) w.phiKsel = take(BH * (size_t)w.sel_rows * dp * 2);
         }
+    }
+    if (w.la && !w.tc_la) {
+        // Segments of the fp32 scan, enough for two waves of two blocks per SM.  Their sums are extra workspace: a call
+        // that fits the library's static workspace with fewer segments takes fewer.
+        const long long units = (long long)BH * (p->d / 64);
+        w.n_seg = (int)std::max<long long>(1, std::min<long long>((592 + units - 1) / units, T - 2));
+        const size_t per_seg = BH * dp * (size_t)(p->d + 1) * 4;
+        if (off <= STILL_STATIC_WORKSPACE_BYTES)
+            while (w.n_seg > 1 && off + align_up(w.n_seg * per_seg, 1024) > STILL_STATIC_WORKSPACE_BYTES) --w.n_seg;
+        if (w.n_seg > 1) w.segs = take(w.n_seg * per_seg);
     }
     w.total = off;
     return w;
@@ -186,89 +197,103 @@ __global__ void sel_mask_kernel(const int32_t *__restrict__ sel_idx, uint32_t *_
 
 // ------------------------------------------------------------------ FMA path launches
 
-template <typename T>
-static int launch_score_select(const still_params_t *p, long long N, long long Tn, const T *Q,
-                               const T *K, float *scores, int32_t *sel, cudaStream_t st) {
-    const int C = p->chunk, d = p->d;
-    size_t smem = ((size_t)2 * C * (d + 1) + (size_t)C * d + C) * 4 + (size_t)C * 4;
-    STILL_CUDA(set_smem(score_select_kernel<T>, smem));
-    dim3 grid((unsigned)Tn, p->H, p->B);
-    score_select_kernel<T><<<grid, 256, smem, st>>>(Q, K, scores, sel, p->H, p->Hkv, N, d, C,
-                                                    p->topk, p->sm_scale, p->eps);
+template <typename T, int NJ>
+static int launch_score_select_t(const still_params_t *p, long long N, long long Tn, const T *Q, const T *K, float *scores,
+                                 int32_t *sel, cudaStream_t st) {
+    const size_t smem = score_select_smem(p->chunk, p->d);
+    STILL_CUDA(set_smem(score_select_kernel<T, NJ>, smem));
+    score_select_kernel<T, NJ><<<dim3((unsigned)Tn, p->H, p->B), 256, smem, st>>>(Q, K, scores, sel, p->H, p->Hkv, N, p->d,
+                                                                                  p->topk, p->sm_scale, p->eps);
     ++g_launches;
     STILL_CUDA(cudaGetLastError());
     return STILL_OK;
+}
+
+template <typename T>
+static int launch_score_select(const still_params_t *p, long long N, long long Tn, const T *Q, const T *K, float *scores,
+                               int32_t *sel, cudaStream_t st) {
+    switch (p->chunk) {
+        case 32: return launch_score_select_t<T, 2>(p, N, Tn, Q, K, scores, sel, st);
+        case 64: return launch_score_select_t<T, 3>(p, N, Tn, Q, K, scores, sel, st);
+        default: return launch_score_select_t<T, 5>(p, N, Tn, Q, K, scores, sel, st);
+    }
 }
 
 template <typename T>
 static int launch_npmap(const still_params_t *p, long long N, int heads, const T *X, const T *W,
                         const T *bias, T *phi, cudaStream_t st) {
-    size_t smem = ((size_t)p->d * p->d_f + p->d_f + 8 * (size_t)p->d) * 4;
-    STILL_CUDA(set_smem(npmap_kernel<T, T>, smem));
-    dim3 grid((unsigned)((N + 63) / 64), heads, p->B);
-    npmap_kernel<T, T><<<grid, 256, smem, st>>>(X, W, bias, phi, heads, N, p->d, p->d_f);
-    ++g_launches;
-    STILL_CUDA(cudaGetLastError());
-    return STILL_OK;
+    const size_t smem = npmap_smem(p->d, p->d_f);
+    const dim3 grid((unsigned)((N + 63) / 64), heads, p->B);
+    auto launch = [&](auto kernel) -> int {
+        STILL_CUDA(set_smem(kernel, smem));
+        kernel<<<grid, 256, smem, st>>>(X, W, bias, phi, heads, N, p->d);
+        ++g_launches;
+        STILL_CUDA(cudaGetLastError());
+        return STILL_OK;
+    };
+    switch (p->d_f) {
+        case 32: return launch(npmap_kernel<T, 32>);
+        case 64: return launch(npmap_kernel<T, 64>);
+        default: return launch(npmap_kernel<T, 128>);
+    }
 }
 
-template <typename T, int FPT>
-static int launch_la_scan_t(const still_params_t *p, long long N, long long Tn, const T *phiQ,
-                            const T *phiK, const T *V, const T *G, const int32_t *sel, float *nla,
-                            float *dla, float *S_out, float *z_out, cudaStream_t st) {
-    constexpr int DP = FPT * 8;
-    size_t smem = ((size_t)32 * DP + 32 * 32 + 8 * 32 * 33 + DP) * 4 + (size_t)p->chunk * 4;
-    STILL_CUDA(set_smem(la_scan_kernel<T, T, FPT>, smem));
-    dim3 grid(p->B * p->H, p->d / 32);
-    int n_route = (int)std::max<long long>(0, Tn - 2);
-    la_scan_kernel<T, T, FPT><<<grid, 256, smem, st>>>(phiQ, phiK, V, G, sel, nla, dla, S_out, z_out,
-                                                       p->H, p->Hkv, N, p->d, p->chunk, p->topk,
-                                                       n_route);
-    ++g_launches;
-    STILL_CUDA(cudaGetLastError());
-    return STILL_OK;
+template <typename T, int DP>
+static int launch_la_scan_t(const still_params_t *p, long long N, long long Tn, const T *phiQ, const T *phiK, const T *V,
+                            const T *G, const int32_t *sel, float *nla, float *dla, float *sums, int n_seg, float *S_out,
+                            float *z_out, cudaStream_t st) {
+    const size_t smem = la_seg_smem(DP);
+    STILL_CUDA(set_smem(la_seg_kernel<T, DP>, smem));
+    const int seg_chunks = (int)((Tn + n_seg - 1) / n_seg);
+    n_seg = (int)((Tn + seg_chunks - 1) / seg_chunks);
+    auto pass = [&](int segments, int sum_only) -> int {
+        la_seg_kernel<T, DP><<<dim3(p->B * p->H, segments, p->d / 64), 256, smem, st>>>(
+            phiQ, phiK, V, G, sel, nla, dla, sums, S_out, z_out, p->H, p->Hkv, N, p->d, p->chunk, p->topk, seg_chunks, n_seg, sum_only);
+        ++g_launches;
+        STILL_CUDA(cudaGetLastError());
+        return STILL_OK;
+    };
+    if (n_seg > 1) {
+        int rc = pass(n_seg - 1, 1);
+        if (rc != STILL_OK) return rc;
+        const long long n4 = (long long)p->B * p->H * DP * (p->d + 1) / 4;
+        la_prefix_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>(sums, n4, n_seg);
+        ++g_launches;
+        STILL_CUDA(cudaGetLastError());
+    }
+    return pass(n_seg, 0);
 }
 
 template <typename T>
 static int launch_la_scan(const still_params_t *p, long long N, long long Tn, const T *phiQ,
                           const T *phiK, const T *V, const T *G, const int32_t *sel, float *nla,
-                          float *dla, float *S_out, float *z_out, cudaStream_t st) {
+                          float *dla, float *sums, int n_seg, float *S_out, float *z_out, cudaStream_t st) {
     switch (p->d_f) {
-        case 32: return launch_la_scan_t<T, 8>(p, N, Tn, phiQ, phiK, V, G, sel, nla, dla, S_out, z_out, st);
-        case 64: return launch_la_scan_t<T, 16>(p, N, Tn, phiQ, phiK, V, G, sel, nla, dla, S_out, z_out, st);
-        default: return launch_la_scan_t<T, 32>(p, N, Tn, phiQ, phiK, V, G, sel, nla, dla, S_out, z_out, st);
+        case 32: return launch_la_scan_t<T, 64>(p, N, Tn, phiQ, phiK, V, G, sel, nla, dla, sums, n_seg, S_out, z_out, st);
+        case 64: return launch_la_scan_t<T, 128>(p, N, Tn, phiQ, phiK, V, G, sel, nla, dla, sums, n_seg, S_out, z_out, st);
+        default: return launch_la_scan_t<T, 256>(p, N, Tn, phiQ, phiK, V, G, sel, nla, dla, sums, n_seg, S_out, z_out, st);
     }
 }
 
-template <typename T, int RPW, int DPL>
-static int launch_sa_merge_t(const still_params_t *p, long long N, long long Tn, const T *Q,
-                             const T *K, const T *V, const int32_t *sel, const float *nla,
-                             const float *dla, T *Y, cudaStream_t st) {
-    constexpr int C = RPW * 8, d = DPL * 32;
-    size_t smem = ((size_t)C * d + 32 * (d + 1) + 32 * d) * 4 + 32 * 8;
-    STILL_CUDA(set_smem(sa_merge_kernel<T, RPW, DPL>, smem));
-    dim3 grid((unsigned)Tn, p->H, p->B);
-    sa_merge_kernel<T, RPW, DPL><<<grid, 256, smem, st>>>(Q, K, V, sel, nla, dla, Y, p->H, p->Hkv, N,
-                                                          p->topk, p->sm_scale);
-    ++g_launches;
-    STILL_CUDA(cudaGetLastError());
-    return STILL_OK;
-}
-
 template <typename T>
-static int launch_sa_merge(const still_params_t *p, long long N, long long Tn, const T *Q, const T *K,
+static int launch_sa_merge(const still_params_t *p, long long N, const T *Q, const T *K,
                            const T *V, const int32_t *sel, const float *nla, const float *dla, T *Y,
                            cudaStream_t st) {
-#define STILL_SA_CASE(CC, DD, RPW, DPL) \
-    if (p->chunk == CC && p->d == DD) return launch_sa_merge_t<T, RPW, DPL>(p, N, Tn, Q, K, V, sel, nla, dla, Y, st);
-    STILL_SA_CASE(32, 64, 4, 2)
-    STILL_SA_CASE(32, 128, 4, 4)
-    STILL_SA_CASE(64, 64, 8, 2)
-    STILL_SA_CASE(64, 128, 8, 4)
-    STILL_SA_CASE(128, 64, 16, 2)
-    STILL_SA_CASE(128, 128, 16, 4)
-#undef STILL_SA_CASE
-    return STILL_ERR_UNSUPPORTED;
+    auto launch = [&](auto kernel, int rows, int threads, int smem) -> int {
+        STILL_CUDA(set_smem(kernel, smem));
+        const dim3 grid((unsigned)((N + rows - 1) / rows), p->H, p->B);
+        kernel<<<grid, threads, smem, st>>>(Q, K, V, sel, nla, dla, Y, p->H, p->Hkv, N, p->chunk, p->topk, p->sm_scale);
+        ++g_launches;
+        STILL_CUDA(cudaGetLastError());
+        return STILL_OK;
+    };
+    // 64 rows a block halve the shared-memory reads per product; 32 where the chunk is that short or 64 would leave SMs idle
+    const bool small = p->chunk == 32 || (N + 63) / 64 * p->H * p->B <= 148;
+#define STILL_SA(DD, ROWS, RT) \
+    launch(sa_merge_kernel<T, DD, ROWS, RT>, ROWS, SaPlan<DD, ROWS, RT>::kThreads, SaPlan<DD, ROWS, RT>::kBytes)
+    if (p->d == 64) return small ? STILL_SA(64, 32, 2) : STILL_SA(64, 64, 4);
+    return small ? STILL_SA(128, 32, 2) : STILL_SA(128, 64, 4);
+#undef STILL_SA
 }
 
 template <typename T>
@@ -317,7 +342,8 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
             dla = reinterpret_cast<float *>(ws + w.dla);
             if ((rc = launch_npmap<T>(p, N, p->H, Q, Wq, bq, phiQ, st)) != STILL_OK) return rc;
             if ((rc = launch_npmap<T>(p, N, p->Hkv, K, Wk, bk, phiK, st)) != STILL_OK) return rc;
-            if ((rc = launch_la_scan<T>(p, N, w.T, phiQ, phiK, V, G, sel, nla, dla, S_out, z_out, st)) != STILL_OK)
+            if ((rc = launch_la_scan<T>(p, N, w.T, phiQ, phiK, V, G, sel, nla, dla, reinterpret_cast<float *>(ws + w.segs), w.n_seg, S_out,
+                                        z_out, st)) != STILL_OK)
                 return rc;
             if (w.tc && Y) {   // the tensor-core attention kernel takes the linear branch as bf16 parts
                 ypart = ws + w.ypart;
@@ -338,7 +364,7 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
                              reinterpret_cast<int *>(ws + w.status), st, &g_launches);
         } else {
             profile_mark_begin(st);
-            rc = launch_sa_merge<T>(p, N, w.T, Q, K, V, sel, nla, dla, Y, st);
+            rc = launch_sa_merge<T>(p, N, Q, K, V, sel, nla, dla, Y, st);
             profile_mark_end(st);
         }
         if (rc != STILL_OK) return rc;

@@ -1,79 +1,143 @@
 // fp32 FMA kernels of the STILL layer: the path for fp32 inputs and for bf16
 // shapes the tensor-core kernels do not cover.  Arithmetic is fp32 throughout;
-// T is the storage type of Q/K/V/G/W/Y, TP the storage type of the NP-Map
-// features kept in the workspace.
+// T is the storage type of Q/K/V/G/W/Y and of the NP-Map features kept in the
+// workspace.
+//
+// All of them are register-tiled products over shared memory: a thread owns a tile
+// of outputs and takes 16-byte pieces of its rows, so that one shared-memory access
+// serves 8 or more multiply-adds, and the multiply-adds are the packed form (two per
+// instruction), which leaves issue slots for the loads.  At B = 1, H = 32, d = 64 and
+// 2000 tokens a quarter of which stays selected (4.5 G multiply-adds, 120 us at the
+// FMA pipes' rate) the layer took 1930 us with one shared-memory access per operand
+// and a scan over the chunks in one block per 32 value columns; see each kernel.
 #pragma once
 #include "still_common.cuh"
 
 namespace still {
 
+__device__ __forceinline__ float4 ld4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
+__device__ __forceinline__ float4 ld4(const __nv_bfloat16 *p) {
+    const uint2 r = *reinterpret_cast<const uint2 *>(p);
+    return make_float4(__uint_as_float(r.x << 16), __uint_as_float(r.x & 0xffff0000u), __uint_as_float(r.y << 16),
+                       __uint_as_float(r.y & 0xffff0000u));
+}
+__device__ __forceinline__ void st4(float *p, float4 v) { *reinterpret_cast<float4 *>(p) = v; }
+__device__ __forceinline__ void st4(__nv_bfloat16 *p, float4 v) {
+    st_f(p, v.x); st_f(p + 1, v.y); st_f(p + 2, v.z); st_f(p + 3, v.w);
+}
+__device__ __forceinline__ float2 lo2(const float4 &v) { return make_float2(v.x, v.y); }
+__device__ __forceinline__ float2 hi2(const float4 &v) { return make_float2(v.z, v.w); }
+__device__ __forceinline__ float2 dup2(float x) { return make_float2(x, x); }
+// Four values of a row into shared memory: fp32 rows as an asynchronous copy, bf16 rows converted on the way.
+__device__ __forceinline__ void stage4(float *dst, const float *src, bool valid) {
+    const uint32_t d = static_cast<uint32_t>(__cvta_generic_to_shared(dst));
+    const int bytes = valid ? 16 : 0;
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(d), "l"(src), "r"(bytes) : "memory");
+}
+__device__ __forceinline__ void stage4(float *dst, const __nv_bfloat16 *src, bool valid) {
+    *reinterpret_cast<float4 *>(dst) = valid ? ld4(src) : make_float4(0.f, 0.f, 0.f, 0.f);
+}
+__device__ __forceinline__ void stage_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+__device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_group 0;" ::: "memory"); }
+
 // ---------------------------------------------------------------------------
 // Self-Saliency Score (Sec. 3.1) + per-chunk top-k (Sec. 3.3, delayed selection).
-// One block per (chunk, head, batch).  A warp scores one token at a time: lane j
-// holds the logits of window slots j, j+32, ...; slot C-1 is the token itself.
-// a_diag is the softmax over the window, a_nodiag the softmax over the window
-// without the token (own max, so it cannot underflow to 0/0), and
-// Score = sum_j a_diag_j log((a_diag_j + eps) / (a_nodiag_j + eps)).
+// One block of 256 threads per (chunk, head, batch).  The logits of 32 rows at a time
+// against the C + 32 keys their windows cover: a warp owns four rows, a lane NJ =
+// C / 32 + 1 keys of each.  Then a warp scores one token at a time: lane j holds the
+// logits of window slots j, j+32, ...; slot C-1 is the token itself (window_score).
+// (2000 tokens x 32 heads: 62 us, with one read per operand and multiply 117 us.)
 // Selection: rank under (score descending, position ascending), NaN as -inf;
 // the k best are written in ascending position order, -1 padded.
 // ---------------------------------------------------------------------------
-template <typename T>
+inline size_t score_select_smem(int C, int d) {
+    return ((size_t)(2 * C + 32) * (d + 4) + (size_t)32 * (C + 33) + C) * 4 + (size_t)C * 4;
+}
+template <typename T, int NJ>
 __global__ void __launch_bounds__(256)
 score_select_kernel(const T *__restrict__ Q, const T *__restrict__ K, float *__restrict__ scores,
-                    int32_t *__restrict__ sel_idx, int H, int Hkv, long long N, int d, int C,
-                    int lam, float scale, float eps) {
-    extern __shared__ float smem[];
+                    int32_t *__restrict__ sel_idx, int H, int Hkv, long long N, int d, int lam, float scale, float eps) {
+    constexpr int C = 32 * (NJ - 1);
+    extern __shared__ __align__(16) float smem[];
     const int c = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
-    const int kv = h / (H / Hkv);
+    const int kv = h / (H / Hkv), ds = d + 4;
     const long long base = (long long)c * C;
     const int Tn = gridDim.x;
-    float *kbuf = smem;                       // [2C][d+1]: previous chunk, then this chunk
-    float *qbuf = kbuf + 2 * C * (d + 1);     // [C][d]
-    float *sc = qbuf + C * d;                 // [C]
+    float *kbuf = smem;                       // [2C][d + 4]: previous chunk, then this chunk
+    float *qbuf = kbuf + 2 * C * ds;          // [32][d + 4]
+    float *lg = qbuf + 32 * ds;               // [32][C + 33]
+    float *sc = lg + 32 * (C + 33);           // [C]
     int *flag = reinterpret_cast<int *>(sc + C);  // [C]
     const T *Qh = Q + ((long long)b * H + h) * N * d;
     const T *Kh = K + ((long long)b * Hkv + kv) * N * d;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, d4 = d >> 2;
 
-    for (int i = threadIdx.x; i < 2 * C * d; i += blockDim.x) {
-        int row = i / d, col = i - row * d;
-        long long pos = base - C + row;
-        kbuf[row * (d + 1) + col] = (pos >= 0 && pos < N) ? ld_f(Kh + pos * d + col) : 0.f;
+    for (int i = threadIdx.x; i < 2 * C * d4; i += 256) {
+        const int row = i / d4, col = (i - row * d4) * 4;
+        const long long pos = base - C + row;
+        const bool in = pos >= 0 && pos < N;
+        stage4(kbuf + row * ds + col, Kh + (in ? pos * d : 0) + col, in);
     }
-    for (int i = threadIdx.x; i < C * d; i += blockDim.x) {
-        int row = i / d;
-        long long pos = base + row;
-        qbuf[i] = (pos < N) ? ld_f(Qh + pos * d + (i - row * d)) : 0.f;
-    }
-    __syncthreads();
-
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nwarp = blockDim.x >> 5;
-    const int spl = C >> 5;  // window slots per lane (C is a multiple of 32, at most 128)
-    for (int r = warp; r < C; r += nwarp) {
-        if (base + r >= N) {
-            if (lane == 0) sc[r] = 0.f;
+    for (int r0 = 0; r0 < C; r0 += 32) {
+        if (base + r0 >= N) {   // (rows past the end of a ragged chunk)
+            if (threadIdx.x < 32) sc[r0 + threadIdx.x] = 0.f;
             continue;
         }
-        float l[4];
+        for (int i = threadIdx.x; i < 32 * d4; i += 256) {
+            const int row = i / d4, col = (i - row * d4) * 4;
+            const long long pos = base + r0 + row;
+            stage4(qbuf + row * ds + col, Qh + (pos < N ? pos * d : 0) + col, pos < N);
+        }
+        stage_commit();
+        stage_wait();
+        __syncthreads();
+        // rows r0 + 4 warp + i, keys (rows of kbuf) r0 + lane + 32 j
+        float2 acc[4][NJ];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            l[i] = -INFINITY;
-            if (i < spl) {
-                int j = lane + 32 * i;            // window slot; token position base + r - (C-1) + j
-                long long pos = base + r - (C - 1) + j;
-                if (pos >= 0) {
-                    const float *kr = kbuf + (r + 1 + j) * (d + 1);
-                    const float *qr = qbuf + r * d;
-                    float acc = 0.f;
-                    for (int x = 0; x < d; ++x) acc = fmaf(qr[x], kr[x], acc);
-                    l[i] = acc * scale;
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) acc[i][j] = make_float2(0.f, 0.f);
+        const float *qr = qbuf + 4 * warp * ds, *kr = kbuf + (r0 + lane) * ds;
+#pragma unroll 4
+        for (int x = 0; x < d; x += 4) {
+            float4 q[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) q[i] = *reinterpret_cast<const float4 *>(qr + i * ds + x);
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) {
+                const float4 k = *reinterpret_cast<const float4 *>(kr + 32 * j * ds + x);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    acc[i][j] = __ffma2_rn(lo2(q[i]), lo2(k), acc[i][j]);
+                    acc[i][j] = __ffma2_rn(hi2(q[i]), hi2(k), acc[i][j]);
                 }
             }
         }
-        float s = window_score(l, lane, spl, C, eps);
-        if (lane == 0) {
-            sc[r] = s;
-            if (scores) scores[((long long)b * H + h) * N + base + r] = s;
+#pragma unroll
+        for (int i = 0; i < 4; ++i)
+#pragma unroll
+            for (int j = 0; j < NJ; ++j) lg[(4 * warp + i) * (C + 33) + lane + 32 * j] = (acc[i][j].x + acc[i][j].y) * scale;
+        __syncwarp();   // a warp scores the rows it has the logits of
+#pragma unroll 1
+        for (int i = 0; i < 4; ++i) {
+            const int r = r0 + 4 * warp + i;
+            if (base + r >= N) {
+                if (lane == 0) sc[r] = 0.f;
+                continue;
+            }
+            float l[4];
+#pragma unroll
+            for (int s = 0; s < 4; ++s) {   // slot lane + 32 s is row r + 1 + slot of kbuf
+                const int slot = lane + 32 * s;
+                l[s] = s < NJ - 1 && base + r - (C - 1) + slot >= 0 ? lg[(4 * warp + i) * (C + 33) + 4 * warp + i + 1 + slot] : -INFINITY;
+            }
+            const float s = window_score(l, lane, NJ - 1, C, eps);
+            if (lane == 0) {
+                sc[r] = s;
+                if (scores) scores[((long long)b * H + h) * N + base + r] = s;
+            }
         }
+        __syncthreads();
     }
     __syncthreads();
     if (lam <= 0) return;
@@ -85,275 +149,519 @@ score_select_kernel(const T *__restrict__ Q, const T *__restrict__ K, float *__r
 // ---------------------------------------------------------------------------
 // Norm-Preserved Feature Map (Sec. 3.2, Eq. feature_map) of every row of X.
 // u = f(x) ||x|| / ||f(x)||, f(x) = xW + b; phi = [softmax(u), softmax(-u)].
-// grid (ceil(N/64), heads, B); a warp maps one row at a time.
+// grid (ceil(N/64), heads, B), 256 threads: 64 rows as a product with W; thread
+// (tr, tc) owns four rows and DF / 16 features, the sixteen threads of a row form
+// its norms, extrema and sums.  (2000 tokens x 40 heads: 38 us; a warp per row: 159 us.)
 // ---------------------------------------------------------------------------
-template <typename T, typename TP>
+inline size_t npmap_smem(int d, int df) { return ((size_t)d * df + (size_t)64 * (d + 4)) * 4; }
+template <typename T, int DF>
 __global__ void __launch_bounds__(256)
 npmap_kernel(const T *__restrict__ X, const T *__restrict__ W, const T *__restrict__ bias,
-             TP *__restrict__ phi, int heads, long long N, int d, int df) {
-    extern __shared__ float smem[];
-    float *Ws = smem;             // [d][df]
-    float *bs = Ws + d * df;      // [df]
-    float *xs = bs + df;          // [8][d]
-    const int hd = blockIdx.y, b = blockIdx.z;
-    const T *Wh = W + (long long)hd * d * df;
-    for (int i = threadIdx.x; i < d * df; i += blockDim.x) Ws[i] = ld_f(Wh + i);
-    for (int i = threadIdx.x; i < df; i += blockDim.x) bs[i] = bias ? ld_f(bias + (long long)hd * df + i) : 0.f;
+             T *__restrict__ phi, int heads, long long N, int d) {
+    constexpr int VC = DF >= 64 ? 4 : 2, NV = DF / (16 * VC);   // columns VC (tc + 16 j) .. + VC
+    extern __shared__ __align__(16) float smem[];
+    const int ds = d + 4, d4 = d >> 2;
+    float *Ws = smem;             // [d][DF]
+    float *xs = Ws + d * DF;      // [64][d + 4]
+    const int hd = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, tr = tid >> 4, tc = tid & 15;
+    const T *Wh = W + (long long)hd * d * DF;
+    const long long row0 = (long long)blockIdx.x * 64, head0 = ((long long)b * heads + hd) * N;
+    for (int i = tid; i < d * DF / 4; i += 256) stage4(Ws + 4 * i, Wh + 4 * i, true);
+    for (int i = tid; i < 64 * d4; i += 256) {
+        const int r = i / d4, col = (i - r * d4) * 4;
+        const bool in = row0 + r < N;
+        stage4(xs + r * ds + col, X + (head0 + (in ? row0 + r : 0)) * d + col, in);
+    }
+    stage_commit();
+    stage_wait();
     __syncthreads();
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const int jpl = df >> 5;  // features per lane (df in {32, 64, 128})
-    float *xw = xs + warp * d;
-    for (int rr = warp; rr < 64; rr += 8) {
-        long long row = (long long)blockIdx.x * 64 + rr;
-        if (row >= N) break;
-        const T *xr = X + (((long long)b * heads + hd) * N + row) * d;
-        for (int i = lane; i < d; i += 32) xw[i] = ld_f(xr + i);
-        __syncwarp();
-        float ep[4], en[4];
-        npmap_row(xw, Ws, bias ? bs : (const float *)nullptr, d, df, lane, ep, en);
-        TP *pr = phi + (((long long)b * heads + hd) * N + row) * 2 * df;
+    float f[4][NV * VC];
 #pragma unroll
-        for (int jj = 0; jj < 4; ++jj)
-            if (jj < jpl) {
-                int j = lane + 32 * jj;
-                st_f(pr + j, ep[jj]);
-                st_f(pr + df + j, en[jj]);
+    for (int j = 0; j < NV; ++j)
+#pragma unroll
+        for (int e = 0; e < VC; ++e) {
+            const float bv = bias ? ld_f(bias + (long long)hd * DF + VC * (tc + 16 * j) + e) : 0.f;
+#pragma unroll
+            for (int i = 0; i < 4; ++i) f[i][j * VC + e] = bv;
+        }
+#pragma unroll 2
+    for (int x = 0; x < d; x += 4) {
+        float4 q[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) q[i] = *reinterpret_cast<const float4 *>(xs + (4 * tr + i) * ds + x);
+#pragma unroll
+        for (int xx = 0; xx < 4; ++xx) {
+            float2 w[NV * VC / 2];
+#pragma unroll
+            for (int j = 0; j < NV; ++j) {
+                const float *wr = Ws + (x + xx) * DF + VC * (tc + 16 * j);
+                if constexpr (VC == 4) {
+                    const float4 v = *reinterpret_cast<const float4 *>(wr);
+                    w[2 * j] = lo2(v);
+                    w[2 * j + 1] = hi2(v);
+                } else {
+                    w[j] = *reinterpret_cast<const float2 *>(wr);
+                }
             }
-        __syncwarp();
+#pragma unroll
+            for (int i = 0; i < 4; ++i) {
+                const float2 qq = dup2(xx == 0 ? q[i].x : xx == 1 ? q[i].y : xx == 2 ? q[i].z : q[i].w);
+#pragma unroll
+                for (int j = 0; j < NV * VC / 2; ++j) {
+                    const float2 r = __ffma2_rn(qq, w[j], make_float2(f[i][2 * j], f[i][2 * j + 1]));
+                    f[i][2 * j] = r.x;
+                    f[i][2 * j + 1] = r.y;
+                }
+            }
+        }
+    }
+    auto over_row = [](float v, auto op) {   // over the sixteen threads of a row
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1) v = op(v, __shfl_xor_sync(0xffffffffu, v, o));
+        return v;
+    };
+    auto add = [](float a, float c) { return a + c; };
+    auto mx = [](float a, float c) { return fmaxf(a, c); };
+    auto mn = [](float a, float c) { return fminf(a, c); };
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+        const long long row = row0 + 4 * tr + i;
+        float nx2 = 0.f, nf2 = 0.f, umax = -INFINITY, umin = INFINITY;
+        for (int x = tc; x < d; x += 16) {
+            const float v = xs[(4 * tr + i) * ds + x];
+            nx2 = fmaf(v, v, nx2);
+        }
+#pragma unroll
+        for (int j = 0; j < NV * VC; ++j) nf2 = fmaf(f[i][j], f[i][j], nf2);
+        nx2 = over_row(nx2, add);
+        nf2 = over_row(nf2, add);
+        const float ratio = sqrtf(nx2) / fmaxf(sqrtf(nf2), 1e-12f);
+#pragma unroll
+        for (int j = 0; j < NV * VC; ++j) {
+            f[i][j] *= ratio;
+            umax = fmaxf(umax, f[i][j]);
+            umin = fminf(umin, f[i][j]);
+        }
+        umax = over_row(umax, mx);
+        umin = over_row(umin, mn);
+        float p[NV * VC], n[NV * VC], zp = 0.f, zn = 0.f;
+#pragma unroll
+        for (int j = 0; j < NV * VC; ++j) {
+            p[j] = expf(f[i][j] - umax);
+            n[j] = expf(umin - f[i][j]);
+            zp += p[j];
+            zn += n[j];
+        }
+        zp = over_row(zp, add);
+        zn = over_row(zn, add);
+        if (row < N) {
+            T *pr = phi + (head0 + row) * 2 * DF;
+#pragma unroll
+            for (int j = 0; j < NV; ++j) {
+                T *dst = pr + VC * (tc + 16 * j);
+                if constexpr (VC == 4) {
+                    st4(dst, make_float4(p[4 * j] / zp, p[4 * j + 1] / zp, p[4 * j + 2] / zp, p[4 * j + 3] / zp));
+                    st4(dst + DF, make_float4(n[4 * j] / zn, n[4 * j + 1] / zn, n[4 * j + 2] / zn, n[4 * j + 3] / zn));
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 2; ++e) {
+                        st_f(dst + e, p[2 * j + e] / zp);
+                        st_f(dst + DF + e, n[2 * j + e] / zn);
+                    }
+                }
+            }
+        }
     }
 }
 
 // ---------------------------------------------------------------------------
 // Linear-attention branch (Algorithm 1 "Linear Attention Branch"; Eq.
-// cache_routing_sum): sequential scan over chunks of one (batch, head) for a
-// slice of 32 value columns.  At chunk c the state holds the LA tokens of chunks
-// <= c-2:  S += sum_{i in M^LA_{c-2}} phi_k(k_i)^T v_i,  z += sum phi_k(k_i)^T;
-// then N_LA = (phi_q(q) S) . g and D_LA = phi_q(q) z for the rows of chunk c.
-// Thread (fg, e): fg = warp = group of FPT features, e = lane = value column.
-// grid (B*H, d/32).  Final S, z go to the decode state when asked.
+// cache_routing_sum) as a two-level scan over the chunks of one (batch, head).  The
+// chunks are cut into n_seg segments that run side by side.  Before chunk c is
+// answered, chunk c-2 is folded:  S += sum_{i in M^LA_{c-2}} phi_k(k_i)^T v_i,
+// z += sum phi_k(k_i)^T;  then N_LA = (phi_q(q) S) . g and D_LA = phi_q(q) z for the
+// rows of chunk c.
+//   sum_only = 1: what segment blockIdx.y folds, into sums (blockIdx.y < n_seg - 1)
+//   sum_only = 0: the scan of a segment, from sums made exclusive prefixes by
+//                 la_prefix_kernel
+// grid (B*H, segments, d / 64), 256 threads: thread (tf, te) owns DP / 16 features x
+// four of the block's 64 value columns of S in registers; for the read-out S passes
+// through shared memory and a thread owns four rows x four columns of N_LA.  The same
+// 2000 tokens: 32 + 71 us and 5 us for the prefix, against 833 us for the scan of all
+// chunks by one block per 32 value columns.
+// Final S, z go to the decode state when asked.
 // ---------------------------------------------------------------------------
-template <typename T, typename TP, int FPT>
+inline size_t la_seg_smem(int dp) { return ((size_t)64 * dp + 64 * 64 + (size_t)dp * 64 + dp) * 4 + 64 * 4 + 16; }
+template <typename T, int DP>
 __global__ void __launch_bounds__(256)
-la_scan_kernel(const TP *__restrict__ phiQ, const TP *__restrict__ phiK, const T *__restrict__ V,
-               const T *__restrict__ G, const int32_t *__restrict__ sel_idx,
-               float *__restrict__ N_LA, float *__restrict__ D_LA, float *__restrict__ S_out,
-               float *__restrict__ z_out, int H, int Hkv, long long N, int d, int C, int lam,
-               int n_route /* chunks folded into the returned state */) {
-    constexpr int DP = FPT * 8;
-    extern __shared__ float smem[];
-    float *ph = smem;                 // [32][DP] feature rows of the current sub-tile
-    float *vt = ph + 32 * DP;         // [32][32]
-    float *red = vt + 32 * 32;        // [8][32][33]
-    float *zs = red + 8 * 32 * 33;    // [DP]
-    int *keep = reinterpret_cast<int *>(zs + DP);  // [C] 1 = LA token
-    const int bh = blockIdx.x, b = bh / H, h = bh % H, kv = h / (H / Hkv);
-    const int e0 = blockIdx.y * 32;
-    const int lane = threadIdx.x & 31, fg = threadIdx.x >> 5;
+la_seg_kernel(const T *__restrict__ phiQ, const T *__restrict__ phiK, const T *__restrict__ V,
+              const T *__restrict__ G, const int32_t *__restrict__ sel_idx, float *__restrict__ N_LA,
+              float *__restrict__ D_LA, float *__restrict__ sums, float *__restrict__ S_out,
+              float *__restrict__ z_out, int H, int Hkv, long long N, int d, int C, int lam, int seg_chunks,
+              int n_seg, int sum_only) {
+    constexpr int FPT = DP / 16;
+    extern __shared__ __align__(16) float smem[];
+    float *ph = smem;                 // [64][DP] feature rows of the current sub-tile
+    float *vs = ph + 64 * DP;         // [64][64]
+    float *Ss = vs + 64 * 64;         // [DP][64]
+    float *zs = Ss + DP * 64;         // [DP]
+    int *list = reinterpret_cast<int *>(zs + DP);   // [64] tokens of the sub-tile to fold; their number
+    int *n_list = list + 64;
+    const int bh = blockIdx.x, seg = blockIdx.y, b = bh / H, h = bh % H, kv = h / (H / Hkv);
+    const int e0 = blockIdx.z * 64, tid = threadIdx.x, te = tid & 15, tf = tid >> 4, warp = tid >> 5, lane = tid & 31;
     const long long Tn = (N + C - 1) / C;
-    const TP *pq = phiQ + (long long)bh * N * DP;
-    const TP *pk = phiK + ((long long)b * Hkv + kv) * N * DP;
+    const T *pq = phiQ + (long long)bh * N * DP;
+    const T *pk = phiK + ((long long)b * Hkv + kv) * N * DP;
     const T *vh = V + ((long long)b * Hkv + kv) * N * d;
-    float S[FPT];
+    float *mine = sums + ((long long)seg * gridDim.x + bh) * DP * (d + 1);   // [DP][d], then z [DP]
+    float2 S[FPT / 2][4];   // features tf * FPT + 2 i, + 1; columns e0 + 4 te + e
 #pragma unroll
-    for (int i = 0; i < FPT; ++i) S[i] = 0.f;
-    for (int i = threadIdx.x; i < DP; i += blockDim.x) zs[i] = 0.f;
-    __syncthreads();
-
-    const long long n_iter = (Tn > (long long)n_route + 2) ? Tn : (long long)n_route + 2;
-    for (long long c = 0; c < n_iter; ++c) {
-        if (c >= 2 && c - 2 < n_route) {
+    for (int i = 0; i < FPT / 2; ++i)
+#pragma unroll
+        for (int e = 0; e < 4; ++e) S[i][e] = make_float2(0.f, 0.f);
+    for (int i = tid; i < DP; i += 256) zs[i] = 0.f;
+    if (!sum_only && seg > 0) {
+#pragma unroll
+        for (int i = 0; i < FPT / 2; ++i) {
+            const float4 a = ld4(mine + (long long)(tf * FPT + 2 * i) * d + e0 + 4 * te);
+            const float4 c = ld4(mine + (long long)(tf * FPT + 2 * i + 1) * d + e0 + 4 * te);
+            S[i][0] = make_float2(a.x, c.x);
+            S[i][1] = make_float2(a.y, c.y);
+            S[i][2] = make_float2(a.z, c.z);
+            S[i][3] = make_float2(a.w, c.w);
+        }
+        for (int i = tid; i < DP; i += 256) zs[i] = mine[(long long)DP * d + i];
+    }
+    const int W = C < 64 ? C : 64;    // tokens of a sub-tile
+    const long long c1 = min((long long)(seg + 1) * seg_chunks, Tn);
+    for (long long c = (long long)seg * seg_chunks; c < c1; ++c) {
+        if (c >= 2) {
             const long long ub = (c - 2) * C;  // chunk c-2 is complete
-            for (int i = threadIdx.x; i < C; i += blockDim.x) keep[i] = 1;
-            __syncthreads();
             const int32_t *si = sel_idx + ((long long)bh * Tn + (c - 2)) * lam;
-            for (int i = threadIdx.x; i < lam; i += blockDim.x) {
-                int32_t p = si[i];
-                if (p >= 0) keep[p - ub] = 0;
-            }
-            __syncthreads();
-            for (int sub = 0; sub < C; sub += 32) {
-                for (int i = threadIdx.x; i < 32 * DP; i += blockDim.x) {
-                    int row = i / DP;
-                    ph[i] = keep[sub + row] ? ld_f(pk + (ub + sub + row) * DP + (i - row * DP)) : 0.f;
-                }
-                for (int i = threadIdx.x; i < 32 * 32; i += blockDim.x) {
-                    int row = i >> 5, col = i & 31;
-                    vt[i] = ld_f(vh + (ub + sub + row) * d + e0 + col);
+            for (int sub = 0; sub < C; sub += W) {
+                __syncthreads();
+                if (warp == 0) {   // the sub-tile's tokens that were not selected, in order
+                    int n = 0;
+                    uint64_t out = 0;   // bit r: token sub + r was selected
+                    for (int i = lane; i < lam; i += 32) {
+                        const long long r = si[i] - ub - sub;
+                        if (r >= 0 && r < W) out |= 1ull << r;
+                    }
+                    const uint32_t lo = __reduce_or_sync(0xffffffffu, (uint32_t)out), hi = __reduce_or_sync(0xffffffffu, (uint32_t)(out >> 32));
+                    for (int r0 = 0; r0 < W; r0 += 32) {
+                        const uint32_t keep = ~(r0 == 0 ? lo : hi);
+                        if ((keep >> lane) & 1u) list[n + __popc(keep & ((1u << lane) - 1u))] = sub + r0 + lane;
+                        n += __popc(keep);
+                    }
+                    if (lane == 0) *n_list = n;
                 }
                 __syncthreads();
-                for (int i = 0; i < 32; ++i) {
-                    float vv = vt[i * 32 + lane];
+                const int n = *n_list;
+                for (int i = tid; i < n * (DP / 4); i += 256) {
+                    const int row = i / (DP / 4), col = (i % (DP / 4)) * 4;
+                    stage4(ph + row * DP + col, pk + (ub + list[row]) * DP + col, true);
+                }
+                for (int i = tid; i < n * 16; i += 256) {
+                    const int row = i >> 4, col = (i & 15) * 4;
+                    stage4(vs + row * 64 + col, vh + (ub + list[row]) * d + e0 + col, true);
+                }
+                stage_commit();
+                stage_wait();
+                __syncthreads();
+#pragma unroll 2
+                for (int i = 0; i < n; ++i) {
+                    const float4 v = *reinterpret_cast<const float4 *>(vs + i * 64 + 4 * te);
+                    const float2 v2[4] = {dup2(v.x), dup2(v.y), dup2(v.z), dup2(v.w)};
 #pragma unroll
-                    for (int ii = 0; ii < FPT; ++ii) S[ii] = fmaf(ph[i * DP + fg * FPT + ii], vv, S[ii]);
+                    for (int q = 0; q < FPT / 4; ++q) {
+                        const float4 p = *reinterpret_cast<const float4 *>(ph + i * DP + tf * FPT + 4 * q);
+#pragma unroll
+                        for (int e = 0; e < 4; ++e) {
+                            S[2 * q][e] = __ffma2_rn(lo2(p), v2[e], S[2 * q][e]);
+                            S[2 * q + 1][e] = __ffma2_rn(hi2(p), v2[e], S[2 * q + 1][e]);
+                        }
+                    }
                 }
-                if (threadIdx.x < DP) {
-                    float a = zs[threadIdx.x];
-                    for (int i = 0; i < 32; ++i) a += ph[i * DP + threadIdx.x];
-                    zs[threadIdx.x] = a;
+                if (tid < DP) {
+                    float a = zs[tid];
+                    for (int i = 0; i < n; ++i) a += ph[i * DP + tid];
+                    zs[tid] = a;
                 }
-                __syncthreads();
             }
         }
-        if (c >= Tn) continue;
-        const long long base = c * C;
-        for (int sub = 0; sub < C; sub += 32) {
-            if (base + sub >= N) break;
-            for (int i = threadIdx.x; i < 32 * DP; i += blockDim.x) {
-                int row = i / DP;
-                long long pos = base + sub + row;
-                ph[i] = (pos < N) ? ld_f(pq + pos * DP + (i - row * DP)) : 0.f;
+        if (sum_only) continue;
+        if (c < 2) {   // nothing has left the local region yet: the branch is zero
+            for (long long i = tid; i < (long long)C * 16; i += 256) {
+                const long long pos = c * C + i / 16;
+                if (pos < N) st4(N_LA + ((long long)bh * N + pos) * d + e0 + (i % 16) * 4, make_float4(0.f, 0.f, 0.f, 0.f));
             }
-            __syncthreads();
-            for (int r = 0; r < 32; ++r) {
-                float acc = 0.f;
+            if (blockIdx.z == 0)
+                for (int r = tid; r < C; r += 256)
+                    if (c * C + r < N) D_LA[(long long)bh * N + c * C + r] = 0.f;
+            continue;
+        }
+        __syncthreads();
 #pragma unroll
-                for (int ii = 0; ii < FPT; ++ii) acc = fmaf(ph[r * DP + fg * FPT + ii], S[ii], acc);
-                red[(fg * 32 + r) * 33 + lane] = acc;
+        for (int i = 0; i < FPT / 2; ++i) {
+            *reinterpret_cast<float4 *>(Ss + (tf * FPT + 2 * i) * 64 + 4 * te) = make_float4(S[i][0].x, S[i][1].x, S[i][2].x, S[i][3].x);
+            *reinterpret_cast<float4 *>(Ss + (tf * FPT + 2 * i + 1) * 64 + 4 * te) = make_float4(S[i][0].y, S[i][1].y, S[i][2].y, S[i][3].y);
+        }
+        for (int sub = 0; sub < C; sub += W) {
+            const long long base = c * C + sub;
+            if (base >= N) break;
+            const int rows = (int)min((long long)W, N - base);
+            if (sub > 0) __syncthreads();
+            for (int i = tid; i < rows * (DP / 4); i += 256) {
+                const int row = i / (DP / 4), col = (i % (DP / 4)) * 4;
+                stage4(ph + row * DP + col, pq + (base + row) * DP + col, true);
             }
+            stage_commit();
+            stage_wait();
             __syncthreads();
-            for (int i = threadIdx.x; i < 32 * 32; i += blockDim.x) {
-                int r = i >> 5, e = i & 31;
-                long long pos = base + sub + r;
-                if (pos < N) {
-                    float acc = 0.f;
+            if (4 * tf < rows) {   // rows 4 tf .. + 3 (rows past the end hold stale features and are not stored)
+                float2 acc[4][2];
 #pragma unroll
-                    for (int w = 0; w < 8; ++w) acc += red[(w * 32 + r) * 33 + e];
-                    long long o = ((long long)bh * N + pos) * d + e0 + e;
-                    if (G) acc *= ld_f(G + o);
-                    N_LA[o] = acc;
+                for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
+#pragma unroll 2
+                for (int f = 0; f < DP; f += 4) {
+                    float4 p[4];
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) p[i] = *reinterpret_cast<const float4 *>(ph + (4 * tf + i) * DP + f);
+#pragma unroll
+                    for (int ff = 0; ff < 4; ++ff) {
+                        const float4 s = *reinterpret_cast<const float4 *>(Ss + (f + ff) * 64 + 4 * te);
+#pragma unroll
+                        for (int i = 0; i < 4; ++i) {
+                            const float2 pp = dup2(ff == 0 ? p[i].x : ff == 1 ? p[i].y : ff == 2 ? p[i].z : p[i].w);
+                            acc[i][0] = __ffma2_rn(pp, lo2(s), acc[i][0]);
+                            acc[i][1] = __ffma2_rn(pp, hi2(s), acc[i][1]);
+                        }
+                    }
                 }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (4 * tf + i < rows) {
+                        const long long o = ((long long)bh * N + base + 4 * tf + i) * d + e0 + 4 * te;
+                        float4 v = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
+                        if (G) {
+                            const float4 gg = ld4(G + o);
+                            v = make_float4(v.x * gg.x, v.y * gg.y, v.z * gg.z, v.w * gg.w);
+                        }
+                        st4(N_LA + o, v);
+                    }
             }
-            if (blockIdx.y == 0) {
-                for (int r = fg; r < 32; r += 8) {
-                    long long pos = base + sub + r;
+            if (blockIdx.z == 0) {
+                for (int r = warp; r < rows; r += 8) {
                     float acc = 0.f;
                     for (int f = lane; f < DP; f += 32) acc = fmaf(ph[r * DP + f], zs[f], acc);
                     acc = warp_sum(acc);
-                    if (lane == 0 && pos < N) D_LA[(long long)bh * N + pos] = acc;
+                    if (lane == 0) D_LA[(long long)bh * N + base + r] = acc;
                 }
             }
-            __syncthreads();
         }
     }
-    if (S_out) {
+    const bool last = !sum_only && seg == n_seg - 1;
+    if (sum_only || (last && S_out)) {
+        __syncthreads();
+        float *So = sum_only ? mine : S_out + (long long)bh * DP * d, *zo = sum_only ? mine + (long long)DP * d : z_out + (long long)bh * DP;
 #pragma unroll
-        for (int ii = 0; ii < FPT; ++ii)
-            S_out[((long long)bh * DP + fg * FPT + ii) * d + e0 + lane] = S[ii];
-        if (blockIdx.y == 0)
-            for (int i = threadIdx.x; i < DP; i += blockDim.x) z_out[(long long)bh * DP + i] = zs[i];
+        for (int i = 0; i < FPT / 2; ++i) {
+            st4(So + (long long)(tf * FPT + 2 * i) * d + e0 + 4 * te, make_float4(S[i][0].x, S[i][1].x, S[i][2].x, S[i][3].x));
+            st4(So + (long long)(tf * FPT + 2 * i + 1) * d + e0 + 4 * te, make_float4(S[i][0].y, S[i][1].y, S[i][2].y, S[i][3].y));
+        }
+        if (blockIdx.z == 0)
+            for (int i = tid; i < DP; i += 256) zo[i] = zs[i];
+    }
+}
+// sums [n_seg][n]: segment s receives the sum of the segments before it (the last segment's own sum is not needed).
+__global__ void __launch_bounds__(256)
+la_prefix_kernel(float *__restrict__ sums, long long n4, int n_seg) {
+    const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
+    if (i >= n4) return;
+    float4 *p = reinterpret_cast<float4 *>(sums) + i;
+    float4 run = make_float4(0.f, 0.f, 0.f, 0.f);
+    for (int s0 = 0; s0 < n_seg; s0 += 8) {   // eight independent loads in flight, then the running sum
+        float4 v[8];
+#pragma unroll
+        for (int s = 0; s < 8; ++s) v[s] = s0 + s < n_seg - 1 ? p[(long long)(s0 + s) * n4] : make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+            if (s0 + s < n_seg) p[(long long)(s0 + s) * n4] = run;
+            run = make_float4(run.x + v[s].x, run.y + v[s].y, run.z + v[s].z, run.w + v[s].w);
+        }
     }
 }
 
 // ---------------------------------------------------------------------------
 // Softmax-attention branch + merge (Algorithm 1 "Softmax Attention Branch" and
-// the output line; Sec. 3.3 merge equation).  One block per (chunk, head,
-// batch).  The keys of chunk c are the selected tokens of chunks 0..c-2 (through
-// sel_idx), all of chunk c-1 and the causal part of chunk c; they are streamed
-// through shared memory 32 at a time.  A warp owns RPW query rows; per key tile a
-// lane computes one logit per row, the row's running max / sum are updated
-// online, and each lane accumulates DPL output columns.
+// the output line; Sec. 3.3 merge equation).  One block of 16 ROWS / RT threads per
+// ROWS queries of a chunk, head and batch.  The keys of chunk c are the selected tokens of
+// chunks 0..c-2 (through sel_idx), all of chunk c-1 and the causal part of chunk c;
+// they pass through two buffers of KT keys.  Thread (ty, tx) owns RT rows: of the
+// logits the keys tx, tx + 16, ..., of the output the columns 4 tx .. + 3 (and + 64).
+// The rows' probabilities go from one product to the other through shared memory that
+// only the half warp of the row reads.  Bound by shared-memory reads (69 % of the rate):
+// 32 heads x 2000 tokens, d = 64, a quarter selected take 250 us with RT = 4 (16 warps an
+// SM), 264 us with RT = 8 (8 warps); with one read per operand and multiply 756 us.
 // Merge: with m the running max, ms = max(m, 0):
 //   y = (o e^{m-ms} + e^{-ms} N_LA) / (l e^{m-ms} + e^{-ms} D_LA).
 // ---------------------------------------------------------------------------
-template <typename T, int RPW, int DPL>
-__global__ void __launch_bounds__(256)
+template <int D, int ROWS, int RT>
+struct SaPlan {
+    static constexpr int kThreads = ROWS / RT * 16;
+    static constexpr int KT = D == 64 ? 64 : 32;
+    static constexpr int kQ = 0, kK = ROWS * (D + 4), kV = kK + 2 * KT * (D + 4), kP = kV + 2 * KT * D;   // in floats
+    static constexpr int kPos = kP + ROWS * (KT + 4);
+    static constexpr int kBytes = (kPos + 2 * KT) * 4;
+};
+template <typename T, int D, int ROWS, int RT>
+__global__ void __launch_bounds__(SaPlan<D, ROWS, RT>::kThreads)
 sa_merge_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V,
                 const int32_t *__restrict__ sel_idx, const float *__restrict__ N_LA,
-                const float *__restrict__ D_LA, T *__restrict__ Y, int H, int Hkv, long long N,
+                const float *__restrict__ D_LA, T *__restrict__ Y, int H, int Hkv, long long N, int C,
                 int lam, float scale) {
-    constexpr int C = RPW * 8, d = DPL * 32;
-    extern __shared__ float smem[];
-    float *qs = smem;                 // [C][d]
-    float *ks = qs + C * d;           // [32][d+1]
-    float *vs = ks + 32 * (d + 1);    // [32][d]
-    long long *kpos = reinterpret_cast<long long *>(vs + 32 * d);  // [32]
-    const int c = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
+    using P = SaPlan<D, ROWS, RT>;
+    constexpr int KT = P::KT, kThreads = P::kThreads, NK = KT / 16, NV = D / 64, DS = D + 4, PS = KT + 4;
+    extern __shared__ __align__(16) float smem[];
+    float *qs = smem + P::kQ, *ps = smem + P::kP;
+    int *kpos = reinterpret_cast<int *>(smem + P::kPos);   // [2][KT]
+    const int h = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, tx = tid & 15, ty = tid >> 4;
     const int kv = h / (H / Hkv);
-    const long long Tn = gridDim.x, base = (long long)c * C, bh = (long long)b * H + h;
-    const T *Qh = Q + bh * N * d;
-    const T *Kh = K + ((long long)b * Hkv + kv) * N * d;
-    const T *Vh = V + ((long long)b * Hkv + kv) * N * d;
+    const long long row0 = (long long)(gridDim.x - 1 - blockIdx.x) * ROWS;   // the longest key streams first
+    const long long c = row0 / C, Tn = (N + C - 1) / C, bh = (long long)b * H + h;
+    const T *Qh = Q + bh * N * D;
+    const T *Kh = K + ((long long)b * Hkv + kv) * N * D;
+    const T *Vh = V + ((long long)b * Hkv + kv) * N * D;
     const int32_t *si = sel_idx + bh * Tn * lam;
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long n_sel = c >= 2 ? (c - 1) * lam : 0, loc0 = c >= 1 ? (c - 1) * C : 0;
+    const long long loc1 = min(row0 + ROWS, N), L = n_sel + (loc1 - loc0);
 
-    for (int i = threadIdx.x; i < C * d; i += blockDim.x) {
-        int row = i / d;
-        long long pos = base + row;
-        qs[i] = (pos < N) ? ld_f(Qh + pos * d + (i - row * d)) : 0.f;
+    auto load_tile = [&](long long t0, int buf) {
+        float *ks = smem + P::kK + buf * KT * DS, *vs = smem + P::kV + buf * KT * D;
+        for (int i = tid; i < KT * (D / 4); i += kThreads) {
+            const int row = i / (D / 4), col = (i % (D / 4)) * 4;
+            const long long e = t0 + row;
+            const long long p = e < n_sel ? (long long)si[e] : e < L ? loc0 + (e - n_sel) : -1;
+            stage4(ks + row * DS + col, Kh + (p >= 0 ? p * D : 0) + col, p >= 0);
+            stage4(vs + row * D + col, Vh + (p >= 0 ? p * D : 0) + col, p >= 0);
+            if (col == 0) kpos[buf * KT + row] = (int)p;
+        }
+        stage_commit();
+    };
+    for (int i = tid; i < ROWS * (D / 4); i += kThreads) {
+        const int row = i / (D / 4), col = (i % (D / 4)) * 4;
+        const bool in = row0 + row < N;
+        stage4(qs + row * DS + col, Qh + (in ? row0 + row : 0) * D + col, in);
     }
-    const long long n_sel = (c >= 2) ? (long long)(c - 1) * lam : 0;
-    const long long loc0 = (c >= 1) ? base - C : 0;
-    const long long loc1 = (base + C < N) ? base + C : N;
-    const long long L = n_sel + (loc1 - loc0);
-
-    float m[RPW], l[RPW], o[RPW][DPL];
+    load_tile(0, 0);
+    float m[RT], l[RT];
+    float2 o[RT][2 * NV];
 #pragma unroll
-    for (int r = 0; r < RPW; ++r) {
+    for (int r = 0; r < RT; ++r) {
         m[r] = -INFINITY;
         l[r] = 0.f;
 #pragma unroll
-        for (int e = 0; e < DPL; ++e) o[r][e] = 0.f;
+        for (int e = 0; e < 2 * NV; ++e) o[r][e] = make_float2(0.f, 0.f);
     }
-    for (long long t0 = 0; t0 < L; t0 += 32) {
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            long long e = t0 + threadIdx.x, p = -1;
-            if (e < n_sel) p = si[e];
-            else if (e < L) p = loc0 + (e - n_sel);
-            kpos[threadIdx.x] = p;
-        }
-        __syncthreads();
-        for (int i = threadIdx.x; i < 32 * d; i += blockDim.x) {
-            int row = i / d, col = i - row * d;
-            long long p = kpos[row];
-            ks[row * (d + 1) + col] = (p >= 0) ? ld_f(Kh + p * d + col) : 0.f;
-            vs[i] = (p >= 0) ? ld_f(Vh + p * d + col) : 0.f;
-        }
-        __syncthreads();
-        const long long p = kpos[lane];
+    int buf = 0;
+    for (long long t0 = 0; t0 < L; t0 += KT, buf ^= 1) {
+        stage_wait();
+        __syncthreads();   // the tile is there, and everybody has left the other buffer
+        if (t0 + KT < L) load_tile(t0 + KT, buf ^ 1);
+        const float *ks = smem + P::kK + buf * KT * DS, *vs = smem + P::kV + buf * KT * D;
+        float2 acc[RT][NK];
 #pragma unroll
-        for (int r = 0; r < RPW; ++r) {
-            const long long t = base + warp * RPW + r;
-            const float *qr = qs + (warp * RPW + r) * d;
-            const float *kr = ks + lane * (d + 1);
-            float s = 0.f;
-#pragma unroll 8
-            for (int x = 0; x < d; ++x) s = fmaf(qr[x], kr[x], s);
-            const bool ok = (p >= 0) && (p <= t) && (t < N);
-            s = ok ? s * scale : -INFINITY;
-            float mn = fmaxf(m[r], warp_max(s));
-            if (mn == -INFINITY) continue;  // nothing visible yet (uniform across the warp)
-            float alpha = expf(m[r] - mn);
-            float pj = ok ? expf(s - mn) : 0.f;
-            l[r] = l[r] * alpha + warp_sum(pj);
-            m[r] = mn;
+        for (int r = 0; r < RT; ++r)
 #pragma unroll
-            for (int e = 0; e < DPL; ++e) o[r][e] *= alpha;
-            for (int j = 0; j < 32; ++j) {
-                float pb = __shfl_sync(0xffffffffu, pj, j);
+            for (int j = 0; j < NK; ++j) acc[r][j] = make_float2(0.f, 0.f);
+#pragma unroll 2
+        for (int x = 0; x < D; x += 4) {
+            float4 k[NK];
 #pragma unroll
-                for (int e = 0; e < DPL; ++e) o[r][e] = fmaf(pb, vs[j * d + lane + 32 * e], o[r][e]);
+            for (int j = 0; j < NK; ++j) k[j] = *reinterpret_cast<const float4 *>(ks + (tx + 16 * j) * DS + x);
+#pragma unroll
+            for (int r = 0; r < RT; ++r) {
+                const float4 q = *reinterpret_cast<const float4 *>(qs + (ty * RT + r) * DS + x);
+#pragma unroll
+                for (int j = 0; j < NK; ++j) {
+                    acc[r][j] = __ffma2_rn(lo2(q), lo2(k[j]), acc[r][j]);
+                    acc[r][j] = __ffma2_rn(hi2(q), hi2(k[j]), acc[r][j]);
+                }
             }
         }
+        int kp[NK];
+#pragma unroll
+        for (int j = 0; j < NK; ++j) kp[j] = kpos[buf * KT + tx + 16 * j];
+#pragma unroll
+        for (int r = 0; r < RT; ++r) {
+            const long long t = row0 + ty * RT + r;
+            float s[NK], mx = -INFINITY;
+#pragma unroll
+            for (int j = 0; j < NK; ++j) {
+                s[j] = kp[j] >= 0 && kp[j] <= t ? (acc[r][j].x + acc[r][j].y) * scale : -INFINITY;
+                mx = fmaxf(mx, s[j]);
+            }
+#pragma unroll
+            for (int w = 8; w > 0; w >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
+            const float mnew = fmaxf(m[r], mx);
+            const float alpha = mnew == -INFINITY ? 1.f : expf(m[r] - mnew);
+            m[r] = mnew;
+            float sum = 0.f;
+#pragma unroll
+            for (int j = 0; j < NK; ++j) {
+                const float p = kp[j] >= 0 && kp[j] <= t && mnew != -INFINITY ? expf(s[j] - mnew) : 0.f;
+                sum += p;
+                ps[(ty * RT + r) * PS + tx + 16 * j] = p;
+            }
+            l[r] = l[r] * alpha + sum;   // (this thread's keys only)
+#pragma unroll
+            for (int e = 0; e < 2 * NV; ++e) o[r][e] = __fmul2_rn(o[r][e], dup2(alpha));
+        }
+        __syncwarp();
+#pragma unroll 1
+        for (int k = 0; k < KT; k += 4) {
+            float4 p[RT];
+#pragma unroll
+            for (int r = 0; r < RT; ++r) p[r] = *reinterpret_cast<const float4 *>(ps + (ty * RT + r) * PS + k);
+#pragma unroll
+            for (int kk = 0; kk < 4; ++kk) {
+#pragma unroll
+                for (int e = 0; e < NV; ++e) {
+                    const float4 v = *reinterpret_cast<const float4 *>(vs + (k + kk) * D + 64 * e + 4 * tx);
+#pragma unroll
+                    for (int r = 0; r < RT; ++r) {
+                        const float2 pp = dup2(kk == 0 ? p[r].x : kk == 1 ? p[r].y : kk == 2 ? p[r].z : p[r].w);
+                        o[r][2 * e] = __ffma2_rn(pp, lo2(v), o[r][2 * e]);
+                        o[r][2 * e + 1] = __ffma2_rn(pp, hi2(v), o[r][2 * e + 1]);
+                    }
+                }
+            }
+        }
+        __syncwarp();
     }
 #pragma unroll
-    for (int r = 0; r < RPW; ++r) {
-        const long long t = base + warp * RPW + r;
+    for (int r = 0; r < RT; ++r) {
+        const long long t = row0 + ty * RT + r;
+#pragma unroll
+        for (int w = 8; w > 0; w >>= 1) l[r] += __shfl_xor_sync(0xffffffffu, l[r], w);
         if (t >= N) continue;
-        float dla = D_LA ? D_LA[bh * N + t] : 0.f;
+        const float dla = D_LA ? D_LA[bh * N + t] : 0.f;
         float fs = 1.f, fl = 0.f;
         if (dla > 0.f) {
-            float ms = fmaxf(m[r], 0.f);
+            const float ms = fmaxf(m[r], 0.f);
             fs = expf(m[r] - ms);
             fl = expf(-ms);
         }
-        float den = l[r] * fs + fl * dla;
+        const float den = l[r] * fs + fl * dla;
 #pragma unroll
-        for (int e = 0; e < DPL; ++e) {
-            long long oidx = (bh * N + t) * d + lane + 32 * e;
-            float num = o[r][e] * fs;
-            if (dla > 0.f) num += fl * N_LA[oidx];
-            st_f(Y + oidx, num / den);
+        for (int e = 0; e < NV; ++e) {
+            const long long oidx = (bh * N + t) * D + 64 * e + 4 * tx;
+            float4 num = make_float4(o[r][2 * e].x * fs, o[r][2 * e].y * fs, o[r][2 * e + 1].x * fs, o[r][2 * e + 1].y * fs);
+            if (dla > 0.f) {
+                const float4 n = ld4(N_LA + oidx);
+                num = make_float4(num.x + fl * n.x, num.y + fl * n.y, num.z + fl * n.z, num.w + fl * n.w);
+            }
+            st4(Y + oidx, make_float4(num.x / den, num.y / den, num.z / den, num.w / den));
         }
     }
 }

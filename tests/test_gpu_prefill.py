@@ -165,6 +165,26 @@ def test_paper_literal_scale_one():
         assert np.abs(U.f64(Y[b, h]) - out["y"]).max() < 1e-4
 
 
+@pytest.mark.parametrize("dtype,d,df,C,k,N", [
+    ("fp32", 64, 32, 32, 8, 32 * 11 + 5), ("fp32", 128, 64, 64, 64 - 1, 64 * 9 + 1), ("fp32", 128, 32, 128, 32, 128 * 6 + 127),
+    ("bf16", 128, 128, 32, 8, 32 * 9 + 31), ("bf16", 64, 32, 64, 16, 64 * 7),   # bf16 shapes of the FMA kernels
+])
+def test_fma_kernels_feature_sizes_and_bias(dtype, d, df, C, k, N):
+    # maps narrower than the head and a bias, scan segments of one and two chunks, ragged ends
+    B, H, Hkv = 1, 4, 2
+    w = _small("t", dtype, B, H, Hkv, d, N, C, k)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    G = synth.make_gate(w, "cuda")
+    g = torch.Generator(device="cuda").manual_seed(10)
+    mk = lambda *s: (torch.randn(*s, generator=g, device="cuda") * 0.05).to(w.torch_dtype)  # noqa: E731
+    Wq, Wk, bq, bk = mk(H, d, df), mk(Hkv, d, df), mk(H, df), mk(Hkv, df)
+    p = still.StillParams(B, H, Hkv, d, C, k, w.torch_dtype, d_f=df, sm_scale=w.sm_scale)
+    Y, scores, sel = still.hybrid_attn_fwd(p, Q, K, V, Wq, Wk, G=G, bq=bq, bk=bk)
+    heads = [(0, h) for h in range(H)]
+    U.check_selection(scores, sel, C, k, heads)
+    U.check_outputs(w, Q, K, V, Wq, Wk, Y, scores, sel, heads, G=G, bq=bq, bk=bk)
+
+
 @pytest.mark.parametrize("k", [64, 16])
 def test_growing_logits_rescale_the_accumulator(k):
     # The tensor-core kernel keeps a row's softmax reference until a tile's maximum exceeds it by 2^8 and then
