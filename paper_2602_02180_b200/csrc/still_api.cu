@@ -333,7 +333,8 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
             n_parts = 2;
             rc = tc_la_branch(p, N, Q, K, V, G, Wq, bq, Wk, bk, sel, phiK, reinterpret_cast<float *>(ws + w.csum),
                               reinterpret_cast<float *>(ws + w.zpre), ypart, dpart, reinterpret_cast<float *>(ws + w.segs), S_out,
-                              z_out, w.phiKsel ? ws + w.phiKsel : nullptr, w.phiKsel ? ws + w.vsel : nullptr, w.sel_rows,
+                              z_out, w.phiKsel ? ws + w.phiKsel : nullptr, Y && w.ksel ? ws + w.ksel : nullptr,
+                              (Y || w.phiKsel) && w.vsel ? ws + w.vsel : nullptr, w.sel_rows,
                               reinterpret_cast<int *>(ws + w.status), st, &g_launches);
             if (rc != STILL_OK) return rc;
         } else {
@@ -360,7 +361,7 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
     // (4) softmax-attention branch + merge.
     if (Y) {
         if (w.tc) {
-            rc = tc_sa_merge(p, N, Q, K, V, sel, ypart, dpart, n_parts, Y, ws + w.ksel, ws + w.vsel, w.sel_rows,
+            rc = tc_sa_merge(p, N, Q, K, V, sel, ypart, dpart, n_parts, Y, ws + w.ksel, ws + w.vsel, w.sel_rows, !w.tc_la,
                              reinterpret_cast<int *>(ws + w.status), st, &g_launches);
         } else {
             profile_mark_begin(st);

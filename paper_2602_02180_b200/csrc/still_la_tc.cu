@@ -6,8 +6,9 @@
 //   phi = [softmax(u), softmax(-u)], stored as bf16 (the B operand of the bf16 state-update GEMM) once
 //   per KV head, together with the column sums of every chunk.
 //
-// z_delta_kernel / z_scan_kernel -- the normaliser z of Eq. cache_routing_sum after every routed chunk:
-//   column sums of the chunk minus the rows of its selected tokens, then a running sum over chunks.
+// gather_kernel / z_scan_kernel -- the rows of the selected tokens in selection order, with the sums of their features,
+//   and the normaliser z of Eq. cache_routing_sum after every routed chunk: column sums of the chunk minus the rows of
+//   its selected tokens, as a running sum over chunks.
 //
 // la_fused_kernel -- Algorithm 1 "Linear Attention Branch" with the state of Eq. cache_routing_sum kept
 //   in tensor memory and the query-side NP-Map computed on the fly (phi(Q) never reaches HBM).  One CTA
@@ -35,6 +36,7 @@
 #include "still_tc.h"
 
 #include <algorithm>
+#include <type_traits>
 
 #include "still_tc_ptx.cuh"
 
@@ -282,50 +284,122 @@ npmap_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
 }
 
 // ------------------------------------------------------------------------------------------
-// Normaliser prefix z (Eq. cache_routing_sum): z after chunk c = sum over the chunks 0..c of the features
-// of their unselected tokens = (column sums of phi(K) over the chunk) - (rows of its selected tokens).
+// Selected rows, and the normaliser z (Eq. cache_routing_sum): z after chunk c = sum over the chunks 0..c of the
+// features of their unselected tokens = (column sums of phi(K) over the chunk) - (rows of its selected tokens).
 // ------------------------------------------------------------------------------------------
-// grid (routed chunks, B*H), 2 d_f threads: zpre[bh][c][f] = csum[kv][c][f] - sum_i phi(K)[sel[bh][c][i]][f], plus,
-// with a salient-cache budget of `window` chunks, the selected rows of chunk c - window, which leave the cache
-// for the state when chunk c is routed.
-__global__ void z_delta_kernel(const float *__restrict__ csum, const __nv_bfloat16 *__restrict__ phiK,
-                               const int32_t *__restrict__ sel_idx, float *__restrict__ zpre, int H, int Hkv, long long N,
-                               int Tn, int n_routed, int lam, int C, int window, int NF) {
-    const int c = blockIdx.x, bh = blockIdx.y, b = bh / H, h = bh % H, kv = b * Hkv + h / (H / Hkv), f = threadIdx.x;
-    float d = 0.f;
-    if (lam < C) {   // (with lam = C every token of the chunk is selected: nothing is left over)
-        d = csum[((long long)kv * Tn + c) * NF + f];
-        const int32_t *si = sel_idx + ((long long)bh * Tn + c) * lam;
-        for (int i = 0; i < lam; ++i) {
-            const int p = si[i];
-            if (p >= 0) d -= __bfloat162float(phiK[((long long)kv * N + p) * NF + f]);
+// grid (T + 1, B*H), 256 threads: the lam selected tokens of chunk blockIdx.x of a query head, read once for everything
+// that is made of them: their K and V rows in selection order (row j of a head is token sel_idx[j]; K_sel / V_sel, what
+// the attention kernel tiles), with a salient-cache budget also their phi(K) rows (phi_sel, from which the tokens that
+// leave the cache enter the state), and the sum of the phi(K) rows (selsum [B*H, n_routed, 2 DF], of the routed chunks).
+// -1 entries and the rows of the padding (block T) are zero.  NULL outputs are not made.  Bound by the bytes written
+// and the rows read: 32 heads x 131072 tokens, d = 128, 32 of 128 selected, with phi_sel: three kernels that each
+// gathered for themselves (and one that summed a row after the other) took 1023 us.
+template <int D, int DF>
+__global__ void __launch_bounds__(256)
+gather_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restrict__ V, const __nv_bfloat16 *__restrict__ phiK,
+              const int32_t *__restrict__ sel_idx, __nv_bfloat16 *__restrict__ Ksel, __nv_bfloat16 *__restrict__ Vsel,
+              __nv_bfloat16 *__restrict__ phi_sel, float *__restrict__ selsum, int H, int Hkv, long long N, int lam,
+              long long sel_rows, int n_routed) {
+    constexpr int kVec = D / 8, kPhiVec = 2 * DF / 8;       // 16-byte pieces of a row
+    constexpr int kPer = 32 / kVec, kPhiPer = 32 / kPhiVec;  // rows that a warp moves at a time
+    __shared__ int pos[128];
+    __shared__ float sums[8 * kPhiPer][2 * DF];
+    const int bh = blockIdx.y, b = bh / H, h = bh % H, c = blockIdx.x, Tn = gridDim.x - 1;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const long long src0 = ((long long)b * Hkv + h / (H / Hkv)) * N, dst0 = (long long)bh * sel_rows + (long long)c * lam;
+    if (c == Tn) {   // padding up to sel_rows
+        const long long n = (sel_rows - (long long)Tn * lam) * kVec, n_phi = n / kVec * kPhiVec;
+        const uint4 zero = make_uint4(0, 0, 0, 0);
+        for (long long i = threadIdx.x; i < n; i += 256) {
+            if (Ksel) reinterpret_cast<uint4 *>(Ksel + dst0 * D)[i] = zero;
+            if (Vsel) reinterpret_cast<uint4 *>(Vsel + dst0 * D)[i] = zero;
+        }
+        if (phi_sel)
+            for (long long i = threadIdx.x; i < n_phi; i += 256) reinterpret_cast<uint4 *>(phi_sel + dst0 * (2 * DF))[i] = zero;
+        return;
+    }
+    for (int i = threadIdx.x; i < lam; i += 256) pos[i] = sel_idx[((long long)bh * Tn + c) * lam + i];
+    __syncthreads();
+    // K and V rows: K in even, V in odd groups of lanes
+    {
+        const int piece = lane % kVec, which = (lane / kVec) & 1;
+        const __nv_bfloat16 *src = which ? V : K;
+        __nv_bfloat16 *dst = which ? Vsel : Ksel;
+        if (dst != nullptr) {
+#pragma unroll 4
+            for (int r = warp * (kPer / 2) + lane / (2 * kVec); r < lam; r += 8 * (kPer / 2)) {
+                const int p = pos[r];
+                uint4 v = make_uint4(0, 0, 0, 0);
+                if (p >= 0) v = reinterpret_cast<const uint4 *>(src + (src0 + p) * D)[piece];
+                reinterpret_cast<uint4 *>(dst + (dst0 + r) * D)[piece] = v;
+            }
         }
     }
-    if (window > 0 && c >= window) {
-        const int32_t *si = sel_idx + ((long long)bh * Tn + (c - window)) * lam;
-        for (int i = 0; i < lam; ++i) {
-            const int p = si[i];
-            if (p >= 0) d += __bfloat162float(phiK[((long long)kv * N + p) * NF + f]);
+    // phi(K) rows and their sum
+    if (phi_sel == nullptr && c >= n_routed) return;
+    const int piece = lane % kPhiVec;
+    float acc[8];
+#pragma unroll
+    for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+#pragma unroll 4
+    for (int r = warp * kPhiPer + lane / kPhiVec; r < lam; r += 8 * kPhiPer) {
+        const int p = pos[r];
+        uint4 v = make_uint4(0, 0, 0, 0);
+        if (p >= 0) v = reinterpret_cast<const uint4 *>(phiK + (src0 + p) * (2 * DF))[piece];
+        if (phi_sel) reinterpret_cast<uint4 *>(phi_sel + (dst0 + r) * (2 * DF))[piece] = v;
+        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            acc[2 * e] += __uint_as_float(w[e] << 16);
+            acc[2 * e + 1] += __uint_as_float(w[e] & 0xffff0000u);
         }
     }
-    zpre[((long long)bh * n_routed + c) * NF + f] = d;
+    if (c >= n_routed) return;
+    float *mine = &sums[warp * kPhiPer + lane / kPhiVec][piece * 8];
+    *reinterpret_cast<float4 *>(mine) = make_float4(acc[0], acc[1], acc[2], acc[3]);
+    *reinterpret_cast<float4 *>(mine + 4) = make_float4(acc[4], acc[5], acc[6], acc[7]);
+    __syncthreads();
+    for (int f = threadIdx.x; f < 2 * DF; f += 256) {   // in a fixed order: the sums are reproducible
+        float s = 0.f;
+#pragma unroll
+        for (int w = 0; w < 8 * kPhiPer; ++w) s += sums[w][f];
+        selsum[((long long)bh * n_routed + c) * (2 * DF) + f] = s;
+    }
 }
-// grid (B*H), 2 d_f threads: in-place running sum over the routed chunks; the last value is the state's z.
-__global__ void z_scan_kernel(float *__restrict__ zpre, float *__restrict__ z_out, int n_routed, int NF) {
-    const int bh = blockIdx.x, f = threadIdx.x;
+// grid (B*H, 2 d_f / 32), up to 1024 threads: z [B*H, n_routed, 2 d_f] after every routed chunk.  What chunk c adds: its column
+// sums less its selected rows (nothing when lam = C), plus, with a salient-cache budget of `window` chunks, the selected
+// rows of chunk c - window, which leave the cache for the state when chunk c is routed.  Two levels: each of the block's
+// warps sums a part of the chunks, and adds them up again from the sum of the parts before.  (One thread per feature
+// over all chunks took 132 us for 1022 chunks of 32 heads, a chain of loads; this takes 53 us.)
+__global__ void __launch_bounds__(1024)
+z_scan_kernel(const float *__restrict__ csum, const float *__restrict__ selsum, float *__restrict__ zpre, float *__restrict__ z_out,
+              int H, int Hkv, int Tn, int n_routed, int all_selected, int window, int NF) {
+    __shared__ float part[32][33];
+    const int bh = blockIdx.x, b = bh / H, h = bh % H, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int f = blockIdx.y * 32 + lane;
+    const float *cs = csum + ((long long)b * Hkv + h / (H / Hkv)) * Tn * NF + f;
+    const float *ss = selsum + (long long)bh * n_routed * NF + f;
     float *z = zpre + (long long)bh * n_routed * NF + f;
+    auto delta = [&](int c) -> float {
+        float d = 0.f;
+        if (!all_selected) d = cs[(long long)c * NF] - ss[(long long)c * NF];
+        if (window > 0 && c >= window) d += all_selected ? cs[(long long)(c - window) * NF] : ss[(long long)(c - window) * NF];
+        return d;
+    };
+    const int warps = blockDim.x >> 5, per = (n_routed + warps - 1) / warps, c0 = warp * per, c1 = min(c0 + per, n_routed);
     float acc = 0.f;
-    for (int c0 = 0; c0 < n_routed; c0 += 8) {   // eight independent loads in flight, then the running sum
-        float v[8];
-#pragma unroll
-        for (int i = 0; i < 8; ++i) v[i] = c0 + i < n_routed ? z[(long long)(c0 + i) * NF] : 0.f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
-            acc += v[i];
-            if (c0 + i < n_routed) z[(long long)(c0 + i) * NF] = acc;
-        }
+#pragma unroll 8
+    for (int c = c0; c < c1; ++c) acc += delta(c);
+    part[warp][lane] = acc;
+    __syncthreads();
+    acc = 0.f;
+    for (int w = 0; w < warp; ++w) acc += part[w][lane];
+#pragma unroll 8
+    for (int c = c0; c < c1; ++c) {
+        acc += delta(c);
+        z[(long long)c * NF] = acc;
     }
-    if (z_out != nullptr) z_out[(long long)bh * NF + f] = acc;
+    if (z_out != nullptr && warp == warps - 1) z_out[(long long)bh * NF + f] = acc;
 }
 
 // ------------------------------------------------------------------------------------------
@@ -693,14 +767,21 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             const int n_sums = seg * sum_parts;
 #pragma unroll 1
             for (int q = 0; q < DF / 32; ++q) {
+                // (a sum's 32 columns are requested together, two sums at a time: requested one value at a time, the
+                // start of a segment took 90 us)
                 uint32_t sreg[32];
+                float acc[32];
 #pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    float acc = 0.f;
-                    if (e < D)
-                        for (int g2 = 0; g2 < n_sums; ++g2) acc += P0[(long long)g2 * (DF * D) + (q * 32 + j) * D + e];
-                    sreg[j] = __float_as_uint(acc);
+                for (int j = 0; j < 32; ++j) acc[j] = 0.f;
+                if (e < D) {
+                    const float *Pq = P0 + (q * 32) * D + e;
+#pragma unroll 2
+                    for (int g2 = 0; g2 < n_sums; ++g2)
+#pragma unroll
+                        for (int j = 0; j < 32; ++j) acc[j] += Pq[(long long)g2 * (DF * D) + j * D];
                 }
+#pragma unroll
+                for (int j = 0; j < 32; ++j) sreg[j] = __float_as_uint(acc[j]);
                 tmem_st32(taddr + col_state + q * 32, sreg);
             }
             tmem_wait_st();
@@ -708,7 +789,18 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             __syncwarp();
             if (lane == 0) mbar_arrive(init_done);
         }
+        constexpr int kPiecesPerRow = D / 8, kPieces = 64 * kPiecesPerRow / 128;   // 16-byte pieces per thread and sub-chunk
         for (int u = u_first; u < NU && !sums_only; ++u) {
+            // the gate of the sub-chunk, requested before the wait (requested where it is used, a chain of round trips
+            // to memory: the layer's 1003-token prompt spent 20 us of its scan on it)
+            uint4 gate[kPieces];
+            if (G != nullptr) {
+#pragma unroll
+                for (int it = 0; it < kPieces; ++it) {
+                    const int id = it * 128 + tid, t = min(u * 64 + id / kPiecesPerRow, N - 1);
+                    gate[it] = *reinterpret_cast<const uint4 *>(G + ((long long)bh * N + t) * D + (id % kPiecesPerRow) * 8);
+                }
+            }
             if (ok) ok = mbar_wait(r_done + (nq & 1), (nq >> 1) & 1, abort_flag, status, 68);
             ok = __all_sync(0xffffffffu, ok);
             if (ok) {
@@ -746,15 +838,12 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             asm volatile("bar.sync 2, 128;" ::: "memory");   // the four worker warps (always, whatever `ok`)
             if (ok) {
                 const int base = u * 64;
-                constexpr int kPiecesPerRow = D / 8;
-#pragma unroll 2
-                for (int it = 0; it < 64 * kPiecesPerRow / 128; ++it) {
+                auto piece = [&](int it, auto gated) {
                     const int id = it * 128 + tid, t = id / kPiecesPerRow, c = id % kPiecesPerRow;
                     if (base + t < N) {
                         uint4 v = *reinterpret_cast<const uint4 *>(smem + P::oStage + (t * D + c * 8) * 2);
-                        const long long off = ((long long)bh * N + base + t) * D + c * 8;
-                        if (G != nullptr) {
-                            const uint4 gg = *reinterpret_cast<const uint4 *>(G + off);
+                        if constexpr (decltype(gated)::value) {
+                            const uint4 gg = gate[it];
                             const uint32_t vw[4] = {v.x, v.y, v.z, v.w}, gw[4] = {gg.x, gg.y, gg.z, gg.w};
                             uint32_t rw[4];
 #pragma unroll
@@ -763,8 +852,16 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                                                   __uint_as_float(vw[q] & 0xffff0000u) * __uint_as_float(gw[q] & 0xffff0000u));
                             v = make_uint4(rw[0], rw[1], rw[2], rw[3]);
                         }
-                        *reinterpret_cast<uint4 *>(y_out + off) = v;
+                        *reinterpret_cast<uint4 *>(y_out + ((long long)bh * N + base + t) * D + c * 8) = v;
                     }
+                };
+                // (without a gate the loop stays short: the kernel is sensitive to its instruction footprint)
+                if (G != nullptr) {
+#pragma unroll
+                    for (int it = 0; it < kPieces; ++it) piece(it, std::true_type{});
+                } else {
+#pragma unroll 2
+                    for (int it = 0; it < kPieces; ++it) piece(it, std::false_type{});
                 }
             }
             asm volatile("bar.sync 2, 128;" ::: "memory");   // the staging tile has been read before the next one is written
@@ -953,32 +1050,6 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     }
 }
 
-// Rows of phi(K) [2 d_f] and V [d] of the selected tokens, per query head, in selection order (row j of a head is
-// token sel_idx[j]; -1 entries and the padding up to sel_rows are zero): with a salient-cache budget the tokens
-// that leave the cache enter the state from these copies, lam rows per chunk.  One warp per row.
-template <int D, int DF>
-__global__ void __launch_bounds__(256)
-gather_selected_kernel(const __nv_bfloat16 *__restrict__ phiK, const __nv_bfloat16 *__restrict__ V,
-                       const int32_t *__restrict__ sel_idx, __nv_bfloat16 *__restrict__ phiKsel,
-                       __nv_bfloat16 *__restrict__ Vsel, int H, int Hkv, long long N, long long n_idx, long long sel_rows) {
-    const int bh = blockIdx.y, b = bh / H, h = bh % H, kvh = h / (H / Hkv);
-    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    const long long j = (long long)blockIdx.x * 8 + warp;
-    if (j >= sel_rows) return;
-    long long pos = -1;
-    if (j < n_idx) pos = sel_idx[(long long)bh * n_idx + j];
-    constexpr int kPhiVec = 2 * DF / 8, kVVec = D / 8;   // uint4 per row
-    uint4 pp = make_uint4(0, 0, 0, 0), vv = pp;
-    const long long src = ((long long)b * Hkv + kvh) * N + pos;
-    if (pos >= 0) {
-        if (lane < kPhiVec) pp = reinterpret_cast<const uint4 *>(phiK + src * (2 * DF))[lane];
-        if (lane < kVVec) vv = reinterpret_cast<const uint4 *>(V + src * D)[lane];
-    }
-    const long long dst = (long long)bh * sel_rows + j;
-    if (lane < kPhiVec) reinterpret_cast<uint4 *>(phiKsel + dst * (2 * DF))[lane] = pp;
-    if (lane < kVVec) reinterpret_cast<uint4 *>(Vsel + dst * D)[lane] = vv;
-}
-
 // ------------------------------------------------------------------------------------------ host side
 
 template <int D, int DF, typename TOut>
@@ -993,6 +1064,19 @@ int launch_npmap(const void *X, const void *W, const void *bias, void *phi, floa
     dim3 grid((unsigned)((N + 127) / 128), (unsigned)heads, (unsigned)B);
     npmap_tc_kernel<D, DF, TOut><<<grid, 192, kSmem, st>>>(tx, tw, (const __nv_bfloat16 *)bias, (TOut *)phi, csum, status, heads,
                                                           (int)N, C);
+    ++*launches;
+    return cudaGetLastError() == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
+}
+
+template <int D, int DF>
+int launch_gather(const still_params_t *p, long long N, const void *K, const void *V, const void *phiK, const int32_t *sel_idx,
+                  void *k_sel, void *v_sel, void *phiK_sel, float *selsum, long long sel_rows, int n_routed, cudaStream_t st,
+                  int *launches) {
+    using bf = __nv_bfloat16;
+    const long long Tn = (N + p->chunk - 1) / p->chunk;
+    gather_kernel<D, DF><<<dim3((unsigned)(Tn + 1), (unsigned)(p->B * p->H)), 256, 0, st>>>(
+        (const bf *)K, (const bf *)V, (const bf *)phiK, sel_idx, (bf *)k_sel, (bf *)v_sel, (bf *)phiK_sel, selsum, p->H, p->Hkv, N,
+        p->topk, sel_rows, n_routed);
     ++*launches;
     return cudaGetLastError() == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
 }
@@ -1016,12 +1100,6 @@ int launch_fused(const still_params_t *p, long long N, const void *Q, const void
     tvs = tv;
     if (gathered) {
         if (BH * (unsigned long long)sel_rows >= (1ull << 31)) return STILL_ERR_UNSUPPORTED;   // TMA row coordinate
-        const long long Tn = (N + p->chunk - 1) / p->chunk;
-        dim3 ggrid((unsigned)((sel_rows + 7) / 8), (unsigned)BH);
-        gather_selected_kernel<D, DF><<<ggrid, 256, 0, st>>>((const bf *)phiK, (const bf *)V, sel_idx, (bf *)phiK_sel, (bf *)v_sel,
-                                                           p->H, p->Hkv, N, Tn * p->topk, sel_rows);
-        ++*launches;
-        if (cudaGetLastError() != cudaSuccess) return STILL_ERR_CUDA;
         if (!make_map_2d(&tks, phiK_sel, BH * (unsigned long long)sel_rows, 2 * DF, FusedPlan<D, DF>::kUTok, false) ||
             !make_map_2d(&tvs, v_sel, BH * (unsigned long long)sel_rows, D, FusedPlan<D, DF>::kUTok, false))
             return STILL_ERR_CUDA;
@@ -1071,7 +1149,7 @@ int tc_la_sum_parts(int seg_chunks) {
 int tc_la_branch(const still_params_t *p, long long N, const void *Q, const void *K, const void *V, const void *G,
                  const void *Wq, const void *bq, const void *Wk, const void *bk, const int32_t *sel_idx, void *phiK,
                  float *csum, float *zpre, void *y_part, float *d_part, float *seg_sums, float *S_out, float *z_out,
-                 void *phiK_sel, void *v_sel, long long sel_rows, int *status_words, cudaStream_t st, int *launches) {
+                 void *phiK_sel, void *k_sel, void *v_sel, long long sel_rows, int *status_words, cudaStream_t st, int *launches) {
     using bf = __nv_bfloat16;
     if ((long long)p->B * p->H * N >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;  // TMA row coordinate
     const int NF = 2 * p->d_f, C = p->chunk;
@@ -1086,16 +1164,24 @@ int tc_la_branch(const still_params_t *p, long long N, const void *Q, const void
     else
         rc = launch_npmap<128, 128, bf>(K, Wk, bk, phiK, csum, p->B, p->Hkv, N, C, status_words, st, launches);
     if (rc != STILL_OK) return rc;
-    // z after every routed chunk (per query head: the selection is per query head)
-    if (n_routed > 0) {
-        z_delta_kernel<<<dim3((unsigned)n_routed, (unsigned)BH), NF, 0, st>>>(csum, (const bf *)phiK, sel_idx, zpre, p->H, p->Hkv,
-                                                                                N, (int)Tn, n_routed, p->topk, C,
-                                                                                p->topk > 0 ? (int)(p->max_salient / p->topk) : 0, NF);
-        ++*launches;
-        if (cudaGetLastError() != cudaSuccess) return STILL_ERR_CUDA;
+    // selected rows of K, V (and phi(K)), then z after every routed chunk (per query head: the selection is per query
+    // head).  The sums of the selected rows lie where the branch's output will: the scan has taken them by then.
+    float *selsum = reinterpret_cast<float *>(y_part);
+    const int window = p->topk > 0 ? (int)(p->max_salient / p->topk) : 0;
+    if (p->topk < C) {
+        if (p->d == 64 && p->d_f == 64)
+            rc = launch_gather<64, 64>(p, N, K, V, phiK, sel_idx, k_sel, v_sel, phiK_sel, selsum, sel_rows, n_routed, st, launches);
+        else if (p->d == 128 && p->d_f == 64)
+            rc = launch_gather<128, 64>(p, N, K, V, phiK, sel_idx, k_sel, v_sel, phiK_sel, selsum, sel_rows, n_routed, st, launches);
+        else
+            rc = launch_gather<128, 128>(p, N, K, V, phiK, sel_idx, k_sel, v_sel, phiK_sel, selsum, sel_rows, n_routed, st, launches);
+        if (rc != STILL_OK) return rc;
     }
     if (n_routed > 0 || z_out != nullptr) {
-        z_scan_kernel<<<(unsigned)BH, NF, 0, st>>>(zpre, z_out, n_routed, NF);
+        // a warp per eight chunks, whose loads are in flight together; at most 32
+        const int warps = std::max(1, std::min(32, (n_routed + 7) / 8));
+        z_scan_kernel<<<dim3((unsigned)BH, NF / 32), 32 * warps, 0, st>>>(csum, selsum, zpre, z_out, p->H, p->Hkv, (int)Tn, n_routed,
+                                                                    p->topk >= C ? 1 : 0, window, NF);
         ++*launches;
         if (cudaGetLastError() != cudaSuccess) return STILL_ERR_CUDA;
     }

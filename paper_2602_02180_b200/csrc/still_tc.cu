@@ -1241,12 +1241,12 @@ bool make_map(CUtensorMap *m, const void *base, unsigned long long rows, int d) 
 template <int D>
 int launch_tc(const still_params_t *p, long long N, const void *Q, const void *K, const void *V,
               const int32_t *sel_idx, const void *y_part, const float *d_part, int n_parts, void *Y, void *k_sel, void *v_sel,
-              long long sel_rows, int *status, cudaStream_t st, int *launches) {
+              long long sel_rows, bool compact, int *status, cudaStream_t st, int *launches) {
     using bf = __nv_bfloat16;
     const long long T = (N + p->chunk - 1) / p->chunk, BH = (long long)p->B * p->H;
     const long long n_idx = T * p->topk;
     const bool identity = p->topk == p->chunk;  // the selection of every chunk is the chunk itself
-    if (!identity) {
+    if (!identity && compact) {
         dim3 grid((unsigned)((sel_rows + 7) / 8), (unsigned)BH);
         compact_kernel<D><<<grid, 256, 0, st>>>((const bf *)K, (const bf *)V, sel_idx, (bf *)k_sel, (bf *)v_sel, p->H,
                                                p->Hkv, N, n_idx, sel_rows);
@@ -1359,11 +1359,11 @@ long long tc_sel_rows(const still_params_t *p, long long N) {
 
 int tc_sa_merge(const still_params_t *p, long long N, const void *Q, const void *K, const void *V,
                 const int32_t *sel_idx, const void *y_part, const float *d_part, int n_parts, void *Y, void *k_sel, void *v_sel,
-                long long sel_rows, int *status_words, cudaStream_t st, int *launches) {
+                long long sel_rows, bool compact, int *status_words, cudaStream_t st, int *launches) {
     if ((long long)p->B * p->H * std::max(N, sel_rows) >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;  // TMA row coordinate
     if (p->d == 64)
-        return launch_tc<64>(p, N, Q, K, V, sel_idx, y_part, d_part, n_parts, Y, k_sel, v_sel, sel_rows, status_words, st, launches);
-    return launch_tc<128>(p, N, Q, K, V, sel_idx, y_part, d_part, n_parts, Y, k_sel, v_sel, sel_rows, status_words, st, launches);
+        return launch_tc<64>(p, N, Q, K, V, sel_idx, y_part, d_part, n_parts, Y, k_sel, v_sel, sel_rows, compact, status_words, st, launches);
+    return launch_tc<128>(p, N, Q, K, V, sel_idx, y_part, d_part, n_parts, Y, k_sel, v_sel, sel_rows, compact, status_words, st, launches);
 }
 
 }  // namespace still

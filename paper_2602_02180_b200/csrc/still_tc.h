@@ -40,12 +40,12 @@ long long tc_sel_rows(const still_params_t *p, long long N);
 // Self-Saliency Score + per-chunk top-k on tensor cores (scores may be NULL).
 int tc_score_select(const still_params_t *p, long long N, const void *Q, const void *K, float *scores,
                     int32_t *sel_idx, int *status_words, cudaStream_t st, int *launches);
-// Compacts the selected K/V rows and runs the softmax-attention + merge kernel.
+// Runs the softmax-attention + merge kernel, with `compact` after compacting the selected K/V rows.
 // The linear branch arrives as n_parts (0, 1 or 2) partial results: y_part [n_parts][B,H,N,d] bf16 = N_part /
 // D_part and d_part [n_parts][B,H,N] fp32; N_LA = sum y_part d_part, D_LA = sum d_part.
 int tc_sa_merge(const still_params_t *p, long long N, const void *Q, const void *K, const void *V,
                 const int32_t *sel_idx, const void *y_part, const float *d_part, int n_parts, void *Y, void *k_sel,
-                void *v_sel, long long sel_rows, int *status_words, cudaStream_t st, int *launches);
+                void *v_sel, long long sel_rows, bool compact, int *status_words, cudaStream_t st, int *launches);
 // fp32 N_LA / D_LA of the FMA kernels as one such part (y = N_LA / D_LA, d = D_LA).
 int tc_la_to_part(const float *N_LA, const float *D_LA, void *y_part, float *d_part, long long rows, int d,
                   cudaStream_t st, int *launches);
@@ -62,10 +62,12 @@ bool tc_la_supported(const still_params_t *p);
 // normaliser z after every routed chunk (zpre [B,H,T-2,2 d_f]), then the state scan with the query-side NP-Map
 // fused in: y_part [2][B,H,N,d] bf16 = N_part / D_part (gated), d_part [2][B,H,N] fp32, one part per feature
 // half; S_out / z_out (optional) receive the state after the chunks that have left the local region.
+// With topk < chunk it also compacts the selected rows: K_sel / V_sel (each optional) and, when phiK_sel is given (it is
+// needed with a budget), their phi(K) rows.
 int tc_la_branch(const still_params_t *p, long long N, const void *Q, const void *K, const void *V, const void *G,
                  const void *Wq, const void *bq, const void *Wk, const void *bk, const int32_t *sel_idx, void *phiK,
                  float *csum, float *zpre, void *y_part, float *d_part, float *seg_sums, float *S_out, float *z_out,
-                 void *phiK_sel, void *v_sel, long long sel_rows, int *status_words, cudaStream_t st, int *launches);
+                 void *phiK_sel, void *k_sel, void *v_sel, long long sel_rows, int *status_words, cudaStream_t st, int *launches);
 // Segments of the two-level state scan for these parameters (1 = plain scan); *seg_chunks = chunks per segment.
 // seg_sums holds (segments - 1) partial states [2 d_f, d] fp32 per (batch, head).
 int tc_la_segments(const still_params_t *p, long long N, int *seg_chunks);
