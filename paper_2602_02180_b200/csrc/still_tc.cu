@@ -38,6 +38,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <climits>
 
 #include "still_common.cuh"
 #include "still_tc_ptx.cuh"
@@ -921,7 +922,7 @@ struct ScoreSmem {
     static constexpr int kStage = kQBytes + kKBytes;
     static constexpr int kBar = 2 * kStage;          // full[2], mma_done[2], smem_free[2], tmem_free[2]
     static constexpr int kMisc = kBar + 8 * 8;       // tmem base, abort flag
-    static constexpr int kSc = kMisc + 16;           // [2][128] scores of the group's tile (16-byte aligned)
+    static constexpr int kSc = kMisc + 16;           // [2][128] ranking keys of the group's tile (16-byte aligned)
     static constexpr int kBallot = kSc + 2 * kBlockM * 4;   // [2][4]
     static constexpr int kTotal = kBallot + 2 * 4 * 4;
     static constexpr int kAlloc = kTotal + 1024;     // slack to align the base to 1024
@@ -930,7 +931,17 @@ struct ScoreSmem {
 static_assert(ScoreSmem<64>::kAlloc <= kMaxDynamicSmem && ScoreSmem<128>::kAlloc <= kMaxDynamicSmem,
               "score kernel: two stages must fit one CTA's shared memory");
 
-template <int D, int C>
+// log2 of a positive number.  The general form costs four instructions more to scale subnormal arguments; they cannot
+// occur when eps, which every argument contains, is a normal number.
+template <bool kTiny>
+__device__ __forceinline__ float log2_of(float x) {
+    if constexpr (kTiny) return __log2f(x);
+    float y;
+    asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+    return y;
+}
+
+template <int D, int C, bool kTinyEps>
 __global__ void __launch_bounds__(320, 1)
 score_select_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        float *__restrict__ scores, int32_t *__restrict__ sel_idx, int *status, int H, int Hkv,
@@ -1016,7 +1027,7 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
         const int g = (warp - 2) >> 2;                 // score group = stage = TMEM accumulator
         const int wq = warp & 3;                       // TMEM lane quarter this warp may read
         const int r = wq * 32 + lane;                  // row of the tile owned by this thread
-        float *sc = reinterpret_cast<float *>(smem + P::kSc) + g * kBlockM;
+        int *keys = reinterpret_cast<int *>(smem + P::kSc) + g * kBlockM;
         uint32_t *ballots = reinterpret_cast<uint32_t *>(smem + P::kBallot) + g * 4;
         const uint32_t taddr = tmem_base + g * 256 + ((uint32_t)(wq * 32) << 16) + (uint32_t)(wq * 32 + kBlockN - C);
         const int group_bar = 1 + g;
@@ -1069,99 +1080,86 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                     __syncwarp();
                     if (lane == 0) mbar_arrive(tmem_free + g);
                 };
-                if constexpr (kBlocks == 2) {
-                    // the row fits the register file: one read of tensor memory, exponentials kept in place
-                    uint32_t v0[32], v1[32];
-                    load_block(0, v0);
-                    load_block(1, v1);
-                    tmem_read_done();
-                    float mx0 = -INFINITY, mx1 = -INFINITY;
+                // The row fits the register file (C values): one read of tensor memory, exponentials kept in place.
+                uint32_t v[kBlocks][32];
+#pragma unroll
+                for (int q = 0; q < kBlocks; ++q) load_block(q, v[q]);
+                tmem_read_done();
+                float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
+#pragma unroll
+                for (int q = 0; q < kBlocks; ++q)
+#pragma unroll
+                    for (int jj = 0; jj < 32; jj += 2)
+                        mx[(jj >> 1) & 3] = max3(mx[(jj >> 1) & 3], __uint_as_float(v[q][jj]), __uint_as_float(v[q][jj + 1]));
+                const float neg_m = -fmaxf(fmaxf(mx[0], mx[1]), fmaxf(mx[2], mx[3])) * scale_log2;
+                const float2 scale2 = make_float2(scale_log2, scale_log2), negm2 = make_float2(neg_m, neg_m);
+                // e_j; the token's own (jj = lane of block 0) is taken out of the row, so that the sum without it is formed
+                // directly and the terms below need no case for it
+                float2 z2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
+                float e_self = 0.f;
+#pragma unroll
+                for (int q = 0; q < kBlocks; ++q)
 #pragma unroll
                     for (int jj = 0; jj < 32; jj += 2) {
-                        mx0 = max3(mx0, __uint_as_float(v0[jj]), __uint_as_float(v0[jj + 1]));
-                        mx1 = max3(mx1, __uint_as_float(v1[jj]), __uint_as_float(v1[jj + 1]));
-                    }
-                    const float neg_m = -fmaxf(mx0, mx1) * scale_log2;
-                    float z0 = 0.f, z1 = 0.f, e_self = 0.f;
-#pragma unroll
-                    for (int jj = 0; jj < 32; ++jj) {
-                        const float e0 = ex2(fmaf(__uint_as_float(v0[jj]), scale_log2, neg_m));
-                        const float e1 = ex2(fmaf(__uint_as_float(v1[jj]), scale_log2, neg_m));
-                        v1[jj] = __float_as_uint(e1);
-                        z1 += e1;
-                        if (jj == lane) e_self = e0;
-                        else z0 += e0;                    // the sum without the token itself is formed directly
-                        v0[jj] = __float_as_uint(e0);
-                    }
-                    const float z_nd = z0 + z1, z_all = z_nd + e_self;
-                    const float inv_all = 1.f / z_all, inv_nd = z_nd > 0.f ? 1.f / z_nd : 0.f;
-                    float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-                    for (int jj = 0; jj < 32; ++jj) {
-                        // a * ln((a + eps) / (b + eps)); a masked key has a = b = 0 and adds nothing
-                        const float e0 = __uint_as_float(v0[jj]), e1 = __uint_as_float(v1[jj]);
-                        const float a0 = e0 * inv_all, a1 = e1 * inv_all;
-                        const float b0 = (jj == lane) ? 0.f : e0 * inv_nd, b1 = e1 * inv_nd;
-                        s0 += a0 * (__log2f(a0 + eps) - __log2f(b0 + eps));
-                        s1 += a1 * (__log2f(a1 + eps) - __log2f(b1 + eps));
-                    }
-                    score = s0 + s1;
-                } else {
-                    float mx = -INFINITY;
-#pragma unroll 1
-                    for (int q = 0; q < kBlocks; ++q) {
-                        uint32_t v[32];
-                        load_block(q, v);
-#pragma unroll
-                        for (int jj = 0; jj < 32; jj += 2) mx = max3(mx, __uint_as_float(v[jj]), __uint_as_float(v[jj + 1]));
-                    }
-                    const float neg_m = -mx * scale_log2;
-                    float z_nd = 0.f, e_self = 0.f;
-#pragma unroll 1
-                    for (int q = 0; q < kBlocks; ++q) {
-                        uint32_t v[32];
-                        load_block(q, v);
-#pragma unroll
-                        for (int jj = 0; jj < 32; ++jj) {
-                            const float e = ex2(fmaf(__uint_as_float(v[jj]), scale_log2, neg_m));
-                            if (q == 0 && jj == lane) e_self = e;
-                            else z_nd += e;
+                        const float2 x = __ffma2_rn(make_float2(__uint_as_float(v[q][jj]), __uint_as_float(v[q][jj + 1])), scale2, negm2);
+                        float2 e = make_float2(ex2(x.x), ex2(x.y));
+                        if (q == 0) {
+                            if (jj == lane) { e_self = e.x; e.x = 0.f; }
+                            if (jj + 1 == lane) { e_self = e.y; e.y = 0.f; }
                         }
+                        z2[(jj >> 1) & 1] = __fadd2_rn(z2[(jj >> 1) & 1], e);
+                        v[q][jj] = __float_as_uint(e.x);
+                        v[q][jj + 1] = __float_as_uint(e.y);
                     }
-                    const float z_all = z_nd + e_self;
-                    const float inv_all = 1.f / z_all, inv_nd = z_nd > 0.f ? 1.f / z_nd : 0.f;
-#pragma unroll 1
-                    for (int q = 0; q < kBlocks; ++q) {
-                        uint32_t v[32];
-                        load_block(q, v);
+                const float z_nd = (z2[0].x + z2[0].y) + (z2[1].x + z2[1].y), z_all = z_nd + e_self;
+                const float inv_all = 1.f / z_all, inv_nd = z_nd > 0.f ? 1.f / z_nd : 0.f;
+                const float2 ia2 = make_float2(inv_all, inv_all), in2 = make_float2(inv_nd, inv_nd), eps2 = make_float2(eps, eps);
+                const float2 minus2 = make_float2(-1.f, -1.f);
+                float2 s2[2] = {make_float2(0.f, 0.f), make_float2(0.f, 0.f)};
 #pragma unroll
-                        for (int jj = 0; jj < 32; ++jj) {
-                            const float e = ex2(fmaf(__uint_as_float(v[jj]), scale_log2, neg_m));
-                            const float a = e * inv_all;
-                            const float bb = (q == 0 && jj == lane) ? 0.f : e * inv_nd;
-                            score += a * (__log2f(a + eps) - __log2f(bb + eps));
-                        }
+                for (int q = 0; q < kBlocks; ++q)
+#pragma unroll
+                    for (int jj = 0; jj < 32; jj += 2) {
+                        // a log2((a + eps) / (b + eps)) without the factor 1 / Z; a masked key has e = 0 and adds nothing
+                        const float2 e = make_float2(__uint_as_float(v[q][jj]), __uint_as_float(v[q][jj + 1]));
+                        const float2 a = __ffma2_rn(e, ia2, eps2), bb = __ffma2_rn(e, in2, eps2);
+                        const float2 la = make_float2(log2_of<kTinyEps>(a.x), log2_of<kTinyEps>(a.y));
+                        const float2 lb = make_float2(log2_of<kTinyEps>(bb.x), log2_of<kTinyEps>(bb.y));
+                        s2[(jj >> 1) & 1] = __ffma2_rn(e, __ffma2_rn(lb, minus2, la), s2[(jj >> 1) & 1]);
                     }
-                    tmem_read_done();
-                }
+                const float a_self = e_self * inv_all;
+                score = ((s2[0].x + s2[0].y) + (s2[1].x + s2[1].y)) * inv_all +
+                        a_self * (log2_of<kTinyEps>(a_self + eps) - log2_of<kTinyEps>(eps));
                 score *= 0.6931471805599453f;
             }
-            sc[r] = score;
+            // the score as an integer of the same order (NaN as -inf, -0 as 0): one comparison ranks two tokens
+            const int bits = __float_as_int(isnan(score) ? -INFINITY : score + 0.f);
+            const int key = bits ^ ((bits >> 31) & 0x7fffffff);
+            keys[r] = t < N ? key : INT_MIN;   // (below the key of -inf)
             if (t < N && scores != nullptr) scores[(long long)bh * N + t] = score;
             asm volatile("bar.sync %0, 128;" ::"r"(group_bar) : "memory");
             if (lam > 0) {
-                // top-k of each chunk of the tile: rank under (score descending, position ascending), NaN as -inf
+                // top-k of each chunk of the tile: rank under (score descending, position ascending)
                 const int cc = r / C, rr = r - cc * C;
                 const int n_c = min(C, N - (R0 + cc * C));   // tokens of this row's chunk (<= 0: past the end)
                 bool selected = false;
                 if (rr < n_c) {
-                    float mine = sc[r];
-                    if (isnan(mine)) mine = -INFINITY;
+                    // tokens before this one outrank it with an equal key: they are compared with key - 1.  Blocks of 32
+                    // tokens are before, after or (the warp's own) around it; a ragged chunk's missing tokens rank below all.
                     int rank = 0;
-                    for (int jx = 0; jx < n_c; ++jx) {
-                        float o = sc[cc * C + jx];
-                        if (isnan(o)) o = -INFINITY;
-                        rank += (o > mine) || (o == mine && jx < rr);
+#pragma unroll
+                    for (int q = 0; q < C / 32; ++q) {
+                        const int own = rr >> 5, base_key = q < own ? key - 1 : key;
+#pragma unroll
+                        for (int j4 = 0; j4 < 8; ++j4) {
+                            const int4 o = *reinterpret_cast<const int4 *>(keys + cc * C + q * 32 + j4 * 4);
+                            const int ov[4] = {o.x, o.y, o.z, o.w};
+#pragma unroll
+                            for (int e = 0; e < 4; ++e) {
+                                const int thr = q == own && j4 * 4 + e < lane ? key - 1 : base_key;
+                                rank += ov[e] > thr ? 1 : 0;
+                            }
+                        }
                     }
                     selected = rank < lam;
                 }
@@ -1178,7 +1176,7 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                     if (rr >= n_sel && rr < lam) out[rr] = -1;
                 }
             }
-            // sc / ballots are written again in the group's next tile
+            // keys / ballots are written again in the group's next tile
             asm volatile("bar.sync %0, 128;" ::"r"(group_bar) : "memory");
         }
     }
@@ -1296,9 +1294,8 @@ int launch_score_tc(const still_params_t *p, long long N, const void *Q, const v
         !make_map(&tk, K, (unsigned long long)p->B * p->Hkv * N, D))
         return STILL_ERR_CUDA;
     constexpr int kSmem = ScoreSmem<D>::kAlloc;
-    if (ensure_dynamic_smem((const void *)score_select_tc_kernel<D, C>, kSmem) !=
-        cudaSuccess)
-        return STILL_ERR_CUDA;
+    const auto kernel = p->eps < 1.17549435e-38f ? score_select_tc_kernel<D, C, true> : score_select_tc_kernel<D, C, false>;
+    if (ensure_dynamic_smem((const void *)kernel, kSmem) != cudaSuccess) return STILL_ERR_CUDA;
     int dev = 0, n_sm = 0;
     if (cudaGetDevice(&dev) != cudaSuccess ||
         cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n_sm <= 0)
@@ -1306,8 +1303,7 @@ int launch_score_tc(const still_params_t *p, long long N, const void *Q, const v
     const long long n_row_blocks = (N + kBlockM - 1) / kBlockM, n_tiles = n_row_blocks * BH;
     if (n_tiles >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;
     const unsigned grid = (unsigned)std::min<long long>(n_tiles, n_sm);   // one persistent CTA per SM
-    score_select_tc_kernel<D, C><<<grid, 320, kSmem, st>>>(tq, tk, scores, sel_idx, status, p->H, p->Hkv, (int)N,
-                                                           p->topk, p->sm_scale * 1.4426950408889634f, p->eps,
+    kernel<<<grid, 320, kSmem, st>>>(tq, tk, scores, sel_idx, status, p->H, p->Hkv, (int)N, p->topk, p->sm_scale * 1.4426950408889634f, p->eps,
                                                            (int)n_row_blocks, (int)n_tiles);
     ++*launches;
     return cudaGetLastError() == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
