@@ -55,12 +55,19 @@ class StillParams:
     eps: float = 1e-6
     max_salient: int = 0  # salient-cache budget per query head (a multiple of topk); 0 = unbounded
 
+    def __setattr__(self, name, value):
+        self.__dict__.pop("_c", None)   # the C struct is rebuilt after any change of a field
+        object.__setattr__(self, name, value)
+
     def c(self) -> _CParams:
-        return _CParams(
-            self.B, self.H, self.Hkv, self.d, self.d if self.d_f is None else self.d_f, self.chunk, self.topk,
-            DTYPE_FP32 if self.dtype == torch.float32 else DTYPE_BF16,
-            float(self.d) ** -0.5 if self.sm_scale is None else self.sm_scale, self.eps, self.max_salient,
-        )
+        c = self.__dict__.get("_c")
+        if c is None:
+            c = self.__dict__["_c"] = _CParams(
+                self.B, self.H, self.Hkv, self.d, self.d if self.d_f is None else self.d_f, self.chunk, self.topk,
+                DTYPE_FP32 if self.dtype == torch.float32 else DTYPE_BF16,
+                float(self.d) ** -0.5 if self.sm_scale is None else self.sm_scale, self.eps, self.max_salient,
+            )
+        return c
 
 
 _lib = None
@@ -117,11 +124,17 @@ def _ptr(t):
     if t is None:
         return None
     assert t.is_contiguous(), "tensors must be contiguous"
-    return ctypes.c_void_p(t.data_ptr())
+    return t.data_ptr()
+
+
+# (the raw handle of the current stream; torch.cuda.current_stream() builds a Stream object around it on every call)
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream():
-    return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def workspace_bytes(p: StillParams, N: int) -> int:
