@@ -50,7 +50,10 @@ struct StateKey {
 // Header words 0-13 against the call: 0 if they agree, else a detail code (1: token count, 2: not a
 // state / other layout version, 3: built with other parameters or another capacity, 4: an earlier step
 // has already failed).  Nothing writes these words while the first kernel of a step runs.
-__device__ __forceinline__ int state_mismatch(const int32_t *hdr, const StateKey &k) {
+__device__ __forceinline__ int state_mismatch(const int32_t *words, const StateKey &k) {
+    const int4 *w4 = reinterpret_cast<const int4 *>(words);   // (four loads in flight, not a chain of comparisons)
+    const int4 w0 = w4[0], w1 = w4[1], w2 = w4[2], w3 = w4[3];
+    const int32_t hdr[16] = {w0.x, w0.y, w0.z, w0.w, w1.x, w1.y, w1.z, w1.w, w2.x, w2.y, w2.z, w2.w, w3.x, w3.y, w3.z, w3.w};
     if (hdr[0] != 0x5354494c || hdr[1] != 1) return 2;
     if (hdr[2] != k.B || hdr[3] != k.H || hdr[4] != k.Hkv || hdr[5] != k.d || hdr[6] != k.d_f || hdr[7] != k.chunk ||
         hdr[8] != k.topk || hdr[9] != k.dtype)
@@ -407,18 +410,18 @@ struct StepArgs {
     int B, H, Hkv, df, la;
     float eps;
     // Plan.  A unit is what shares its K / V rows: the query heads of one (batch, KV head) (fp32: up to four of them).
-    // The units' tiles form one line of units * tiles, of which block i takes [i * per, (i + 1) * per): blocks that
-    // divide the line evenly, whatever the number of groups.  Items: the linear read-outs, one per (batch, query head).
-    int heads_per_unit, units_per_group, tiles;
-    long long per, total;
+    // The units' tiles form one line of units * unit_len, of which block i takes [i * per, (i + 1) * per): blocks that
+    // divide the line evenly, whatever the number of groups.  unit_len is the number of tiles of a unit, or that
+    // rounded up so that no block has tiles of two units.  Items: the linear read-outs, one per (batch, query head).
+    int heads_per_unit, units_per_group, tiles, unit_len, per, total;
     int first_item_block, n_items;   // blocks from first_item_block on share the items evenly
     int item_warps;                  // warps that work on an item together
 };
 
 // First block that works on unit u, and how many do.
-__device__ __forceinline__ long long unit_first_block(long long per, int tiles, long long u) { return u * tiles / per; }
-__device__ __forceinline__ int unit_blocks(long long per, int tiles, long long u) {
-    return (int)(((u + 1) * tiles - 1) / per - u * tiles / per) + 1;
+__device__ __forceinline__ int unit_first_block(int per, int unit_len, int u) { return u * unit_len / per; }
+__device__ __forceinline__ int unit_blocks(int per, int unit_len, int tiles, int u) {
+    return (u * unit_len + tiles - 1) / per - u * unit_len / per + 1;
 }
 
 // Eight (bf16) or four (fp32) consecutive values as fp32.
@@ -652,18 +655,19 @@ step_main_kernel(const __grid_constant__ StepArgs<T> a) {
             return;
         }
     }
-    const long long lo = blockIdx.x * a.per, hi = min(lo + a.per, a.total);
-    const int rep = a.H / a.Hkv;
-    for (long long x = lo; x < hi;) {
-        const long long u = x / a.tiles;
-        const int tile_lo = (int)(x - u * a.tiles), tile_hi = (int)min((long long)a.tiles, hi - u * a.tiles);
-        const long long row = u / a.units_per_group;               // batch * Hkv + KV head
-        const int h0 = (int)(u % a.units_per_group) * a.heads_per_unit;
-        const long long bh = row / a.Hkv * a.H + row % a.Hkv * rep + h0;
-        const long long slot = blockIdx.x - unit_first_block(a.per, a.tiles, u);
+    const int lo = min((int)blockIdx.x * a.per, a.total), hi = min(lo + a.per, a.total), rep = a.H / a.Hkv;
+    for (int x = lo; x < hi;) {
+        const int u = x / a.unit_len;
+        const int tile_lo = x - u * a.unit_len, tile_hi = min(a.tiles, hi - u * a.unit_len);
+        x = min((u + 1) * a.unit_len, hi);
+        if (tile_lo >= tile_hi) continue;
+        const int row = u / a.units_per_group;               // batch * Hkv + KV head
+        const int h0 = u % a.units_per_group * a.heads_per_unit;
+        const long long bh = (long long)(row / a.Hkv) * a.H + row % a.Hkv * rep + h0;
+        const int slot = (int)blockIdx.x - unit_first_block(a.per, a.unit_len, u);
         AttendView v = a.view;
         v.rep = min(a.heads_per_unit, rep - h0);
-        const T *kh = a.kc + row * a.kvr * D, *vh = a.vc + row * a.kvr * D;
+        const T *kh = a.kc + row * a.kvr * D, *vh = a.vc + row * a.kvr * D;   // (kvr is 64-bit)
         const uint32_t *mask = a.sel_mask + bh * v.n_chunk_cap * (v.C / 32);
         float *part = a.part + (bh * kRecords + slot) * (D + 2), *logits = a.part + (bh * kRecords + kLogitRecord) * (D + 2);
         if constexpr (sizeof(T) == 2)
@@ -672,7 +676,6 @@ step_main_kernel(const __grid_constant__ StepArgs<T> a) {
         else
             attend_segment_f32<D>(v, kh, vh, a.k + row * D, a.v + row * D, a.q + bh * D, mask, tile_lo, tile_hi,
                                   step_smem, part, logits, kRecords * (D + 2));
-        x = u * a.tiles + tile_hi;
     }
     if ((int)blockIdx.x < a.first_item_block) return;
     using Ring = StepRing<T, D>;
@@ -681,51 +684,31 @@ step_main_kernel(const __grid_constant__ StepArgs<T> a) {
     else work_on_items<T, D, kStepWarps, Ring>(a, step_smem);
 }
 
-// grid (H, B), D threads: one output column each.
+// grid (H, B), D + 64 threads: an output column each, then a warp that scores the new token and one that appends its K / V
+// row.  For a few sequences its latency counts: everything it reads is requested before the first use (13 partials read
+// four at a time, then the score, took 4 to 7 us).
 template <typename T, int D>
-__global__ void __launch_bounds__(D)
+__global__ void __launch_bounds__(D + 64)
 step_merge_kernel(const __grid_constant__ StepArgs<T> a) {
-    __shared__ float wts[32];
     grid_dep_wait();
     grid_dep_launch();
     if (a.hdr[14] != 0) return;   // mismatch recorded by the step's first kernel: no output, token count unchanged
     const int h = blockIdx.x, b = blockIdx.y, tid = threadIdx.x, lane = tid & 31, rep = a.H / a.Hkv;
     const long long bh = (long long)b * a.H + h;
-    const long long u = ((long long)b * a.Hkv + h / rep) * a.units_per_group + h % rep / a.heads_per_unit;
-    const int n = unit_blocks(a.per, a.tiles, u);    // at most kMaxSplits
     const float *pr = a.part + bh * kRecords * (D + 2);
-    if (h % rep == 0) {   // the new row of the K / V history (position p lives in ring row p % kvr)
-        const long long row = (long long)b * a.Hkv + h / rep, dst = (row * a.kvr + (uint32_t)a.t % (uint32_t)a.kvr) * D + tid;
-        a.kc[dst] = a.k[row * D + tid];
-        a.vc[dst] = a.v[row * D + tid];
+    if (tid >= D + 32) {   // the new row of the K / V history (position p lives in ring row p % kvr)
+        if (h % rep == 0) {
+            const long long row = (long long)b * a.Hkv + h / rep, dst = (row * a.kvr + (uint32_t)a.t % (uint32_t)a.kvr) * D;
+            constexpr int kVec = D * (int)sizeof(T) / 16;
+            if (lane < kVec) {
+                const uint4 kk = reinterpret_cast<const uint4 *>(a.k + row * D)[lane], vv = reinterpret_cast<const uint4 *>(a.v + row * D)[lane];
+                reinterpret_cast<uint4 *>(a.kc + dst)[lane] = kk;
+                reinterpret_cast<uint4 *>(a.vc + dst)[lane] = vv;
+            }
+        }
+        return;
     }
-    float nla = 0.f, dla = 0.f;
-    if (a.la) {
-        nla = pr[kLinRecord * (D + 2) + 2 + tid];
-        dla = pr[kLinRecord * (D + 2) + 1];
-        if (a.g) nla *= ld_f(a.g + bh * D + tid);
-    }
-    // every warp forms the weights of the partials (at most 30)
-    const float ms = lane < n ? pr[lane * (D + 2)] : -INFINITY, ls = lane < n ? pr[lane * (D + 2) + 1] : 0.f;
-    const float M = warp_max(ms);
-    const float w = ms == -INFINITY ? 0.f : expf(ms - M);
-    const float L = warp_sum(ms == -INFINITY ? 0.f : w * ls);
-    if (tid < 32) wts[lane] = w;
-    __syncthreads();
-    float O = 0.f;
-#pragma unroll 4
-    for (int s = 0; s < n; ++s) {
-        const float ws = wts[s], x = pr[s * (D + 2) + 2 + tid];
-        if (ws != 0.f) O = fmaf(ws, x, O);
-    }
-    float fs = 1.f, fl = 0.f;
-    if (dla > 0.f) {
-        const float mm = fmaxf(M, 0.f);
-        fs = expf(M - mm);
-        fl = expf(-mm);
-    }
-    st_f(a.y + bh * D + tid, (O * fs + fl * nla) / (L * fs + fl * dla));
-    if (tid >= D - 32) {   // Self-Saliency Score of the new token: its window's logits lie in the head's last records
+    if (tid >= D) {        // Self-Saliency Score of the new token: its window's logits lie in the head's last records
         const int C = a.view.C;
         float l[4];
 #pragma unroll
@@ -735,12 +718,52 @@ step_merge_kernel(const __grid_constant__ StepArgs<T> a) {
         }
         const float sc = window_score(l, lane, C >> 5, C, a.eps);
         if (lane == 0) a.score[bh * a.cap + a.t] = sc;
+        if (h == 0 && b == 0 && lane == 0) {
+            const long long nt = a.t + 1;
+            a.hdr[12] = (int32_t)(nt & 0xffffffffll);
+            a.hdr[13] = (int32_t)(nt >> 32);
+        }
+        return;
     }
-    if (h == 0 && b == 0 && tid == 0) {
-        const long long nt = a.t + 1;
-        a.hdr[12] = (int32_t)(nt & 0xffffffffll);
-        a.hdr[13] = (int32_t)(nt >> 32);
+    const int u = (b * a.Hkv + h / rep) * a.units_per_group + h % rep / a.heads_per_unit;
+    const int n = unit_blocks(a.per, a.unit_len, a.tiles, u);    // at most kMaxSplits
+    float nla = 0.f, dla = 0.f, gate = 1.f;
+    if (a.la) {
+        nla = pr[kLinRecord * (D + 2) + 2 + tid];
+        dla = pr[kLinRecord * (D + 2) + 1];
+        if (a.g) gate = ld_f(a.g + bh * D + tid);
     }
+    const float ms = lane < n ? pr[lane * (D + 2)] : -INFINITY, ls = lane < n ? pr[lane * (D + 2) + 1] : 0.f;
+    float x[16];
+#pragma unroll
+    for (int s = 0; s < 16; ++s) x[s] = s < n ? pr[s * (D + 2) + 2 + tid] : 0.f;
+    // every warp forms the weights of the partials
+    const float M = warp_max(ms);
+    const float w = ms == -INFINITY ? 0.f : expf(ms - M);
+    const float L = warp_sum(ms == -INFINITY ? 0.f : w * ls);
+    float O = 0.f;
+#pragma unroll
+    for (int s = 0; s < 16; ++s) {
+        const float ws = __shfl_sync(0xffffffffu, w, s);
+        if (ws != 0.f) O = fmaf(ws, x[s], O);
+    }
+    if (n > 16) {
+#pragma unroll
+        for (int s = 0; s < 16; ++s) x[s] = s + 16 < n ? pr[(s + 16) * (D + 2) + 2 + tid] : 0.f;
+#pragma unroll
+        for (int s = 0; s < 16; ++s) {
+            const float ws = __shfl_sync(0xffffffffu, w, s + 16);
+            if (ws != 0.f) O = fmaf(ws, x[s], O);
+        }
+    }
+    nla *= gate;
+    float fs = 1.f, fl = 0.f;
+    if (dla > 0.f) {
+        const float mm = fmaxf(M, 0.f);
+        fs = expf(M - mm);
+        fl = expf(-mm);
+    }
+    st_f(a.y + bh * D + tid, (O * fs + fl * nla) / (L * fs + fl * dla));
 }
 
 #define STILL_CUDA(expr)                               \
@@ -799,7 +822,7 @@ static int launch_main(const StepArgs<T> &a, unsigned grid, cudaStream_t st, int
     profile_mark_begin(st);
     STILL_CUDA(launch_dependent(step_main_kernel<T, D, NT>, dim3(grid), dim3(kStepThreads), kSmem, st, a));
     profile_mark_end(st);
-    STILL_CUDA(launch_dependent(step_merge_kernel<T, D>, dim3(a.H, a.B), dim3(D), 0, st, a));
+    STILL_CUDA(launch_dependent(step_merge_kernel<T, D>, dim3(a.H, a.B), dim3(D + 64), 0, st, a));
     *launches += 2;
     return STILL_OK;
 }
@@ -855,13 +878,24 @@ static int step_typed(const still_params_t *p, char *state, const still_state_la
     a.heads_per_unit = kBf16 ? rep : kUnitHeadsF32;
     a.units_per_group = (rep + a.heads_per_unit - 1) / a.heads_per_unit;
     a.tiles = (int)((t - w.first_pos) / kKeys) + 1;
-    a.total = (long long)p->B * p->Hkv * a.units_per_group * a.tiles;
+    const long long units = (long long)p->B * p->Hkv * a.units_per_group;
     a.n_items = a.la ? p->B * p->H : 0;
     // Few read-outs (a sequence or two): a block each, beside the blocks of the cache pass.  More: every block takes its
     // share of the tiles and then of the read-outs.
     const bool apart = a.n_items <= n_sm / 2;
     const long long blocks = apart ? n_sm - a.n_items : n_sm;
-    a.per = std::max<long long>({(a.total + blocks - 1) / blocks, (a.tiles + kMaxSplits - 2) / (kMaxSplits - 1), 1});
+    const long long least = (a.tiles + kMaxSplits - 2) / (kMaxSplits - 1);
+    a.unit_len = a.tiles;
+    a.per = (int)std::max<long long>({(units * a.tiles + blocks - 1) / blocks, least, 1});
+    // Whole blocks per unit where a block's share is short: one with tiles of two units does two passes, one after the
+    // other, and a pass of up to eight rounds of the warps is mostly latency.
+    const long long per_unit = blocks / units;
+    if (per_unit >= 4 && a.tiles <= per_unit * 8 * kStepWarps) {
+        a.per = (int)std::max<long long>((a.tiles + per_unit - 1) / per_unit, least);
+        a.unit_len = (a.tiles + a.per - 1) / a.per * a.per;
+    }
+    a.total = (int)(units * a.unit_len);   // (a state of 2^31 tiles would be 8 TB)
+    w.early_k = per_unit >= 4;
     const long long used = (a.total + a.per - 1) / a.per;           // blocks with tiles
     a.first_item_block = apart ? (int)used : 0;
     // The fewer warps share a read-out, the more run side by side and the longer one takes.

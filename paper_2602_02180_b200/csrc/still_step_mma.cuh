@@ -72,6 +72,7 @@ struct AttendView {
     int loc0;            // first position of the local region
     int C, lam, rep, n_chunk_cap;
     float scale, scale_log2;
+    int early_k;         // request K rows before it is known which of them are needed (see load_tile)
 };
 
 constexpr int kStepWarps = 8;
@@ -137,7 +138,9 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
     };
     const int c_piece = lane % P::kPieces, c_row = lane / P::kPieces;   // this lane's piece and first row of a copy
     constexpr int kRowsPerIt = 32 / P::kPieces;
-    auto load_tile = [&](int j, int stage, uint32_t rows) {
+    // With few sequences a step is a chain of latencies: K is then read without waiting for the membership words (all rows
+    // up to the new token; a masked logit is never used), V as soon as they are there.
+    auto load_tile = [&](int j, int stage, uint32_t rows, bool with_k, bool with_v) {
         uint8_t *ks = my + stage * P::kStage, *vs = ks + P::kTile;
         const int p0 = v.first_pos + j * kTileKeys;
         // position p lives in ring row p % kvr; kvr is a multiple of the chunk size, so a tile never straddles the end
@@ -150,9 +153,13 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
             const int dst = row * P::kRow + ((c_piece ^ (row & 7)) << 4);
             const bool valid = (rows >> row) & 1u;
             const bool is_new = row == t_row;
-            cp_async16(ks + dst, is_new ? k_new + c_piece * 8 : kp + it * kRowsPerIt * D, valid);
-            cp_async16(vs + dst, is_new ? v_new + c_piece * 8 : vp + it * kRowsPerIt * D, valid);
+            if (with_k) cp_async16(ks + dst, is_new ? k_new + c_piece * 8 : kp + it * kRowsPerIt * D, valid);
+            if (with_v) cp_async16(vs + dst, is_new ? v_new + c_piece * 8 : vp + it * kRowsPerIt * D, valid);
         }
+    };
+    auto rows_so_far = [&](int j) -> uint32_t {   // rows of tile j up to the new token
+        const int last = v.t - (v.first_pos + j * kTileKeys);
+        return last >= 15 ? 0xffffu : ((1u << (last + 1)) - 1u);
     };
 
     // ring: kStages - 1 tiles in flight; membership words run one tile ahead of the copies they steer
@@ -161,9 +168,15 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
     const int first = tile_lo + warp;
 #pragma unroll
     for (int i = 0; i <= kAhead; ++i) words[i] = member_word(first + kStepWarps * i);
+    if (v.early_k) {
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i)
+            if (first + kStepWarps * i < tile_hi) load_tile(first + kStepWarps * i, i, rows_so_far(first + kStepWarps * i), true, false);
+    }
 #pragma unroll
     for (int i = 0; i < kAhead; ++i) {
-        if (first + kStepWarps * i < tile_hi) load_tile(first + kStepWarps * i, i, __reduce_or_sync(0xffffffffu, words[i]));
+        if (first + kStepWarps * i < tile_hi)
+            load_tile(first + kStepWarps * i, i, __reduce_or_sync(0xffffffffu, words[i]), !v.early_k, true);
         cp_async_commit();
     }
     int stage = 0;
@@ -173,7 +186,7 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
             int ps = stage + kAhead;
             if (ps >= P::kStages) ps -= P::kStages;
             const int jn = j + kStepWarps * kAhead;
-            if (jn < tile_hi) load_tile(jn, ps, __reduce_or_sync(0xffffffffu, words[kAhead]));
+            if (jn < tile_hi) load_tile(jn, ps, __reduce_or_sync(0xffffffffu, words[kAhead]), true, true);
             cp_async_commit();
         }
         const uint32_t word = words[0];
