@@ -162,60 +162,123 @@ static cudaError_t set_smem(K kernel, size_t bytes) {
         if (e__ != cudaSuccess) return STILL_ERR_CUDA;     \
     } while (0)
 
+__device__ __forceinline__ void write_header(int32_t *hdr, const still_params_t &p, long long cap, long long t) {
+    hdr[0] = 0x5354494c;  // "STIL"
+    hdr[1] = 1;
+    hdr[2] = p.B; hdr[3] = p.H; hdr[4] = p.Hkv; hdr[5] = p.d; hdr[6] = p.d_f;
+    hdr[7] = p.chunk; hdr[8] = p.topk; hdr[9] = p.dtype;
+    hdr[10] = (int32_t)(cap & 0xffffffffll); hdr[11] = (int32_t)(cap >> 32);
+    hdr[12] = (int32_t)(t & 0xffffffffll); hdr[13] = (int32_t)(t >> 32);
+    hdr[14] = 0; hdr[15] = 0;
+}
 __global__ void write_header_kernel(int32_t *hdr, still_params_t p, long long cap, long long t) {
-    if (threadIdx.x == 0) {
-        hdr[0] = 0x5354494c;  // "STIL"
-        hdr[1] = 1;
-        hdr[2] = p.B; hdr[3] = p.H; hdr[4] = p.Hkv; hdr[5] = p.d; hdr[6] = p.d_f;
-        hdr[7] = p.chunk; hdr[8] = p.topk; hdr[9] = p.dtype;
-        hdr[10] = (int32_t)(cap & 0xffffffffll); hdr[11] = (int32_t)(cap >> 32);
-        hdr[12] = (int32_t)(t & 0xffffffffll); hdr[13] = (int32_t)(t >> 32);
-        hdr[14] = 0; hdr[15] = 0;
-    }
+    grid_dep_wait();
+    grid_dep_launch();
+    if (threadIdx.x == 0) write_header(hdr, p, cap, t);
 }
 
-// Selection of every chunk as bit masks for the decode state: one warp per (head, chunk); bit j of
-// word w is set when position chunk * C + 32 w + j is among the chunk's selected positions.
-__global__ void sel_mask_kernel(const int32_t *__restrict__ sel_idx, uint32_t *__restrict__ sel_mask, long long BH,
-                                long long T, long long capT, int C, int lam) {
-    const long long wid = (long long)blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5);
-    if (wid >= BH * T) return;
-    const int lane = threadIdx.x & 31;
-    const long long bh = wid / T, c = wid % T;
-    const int32_t *si = sel_idx + (bh * T + c) * lam;
-    for (int w = 0; w < C / 32; ++w) {
-        const long long p0 = c * C + 32ll * w;
-        uint32_t bits = 0u;
-        for (int i = lane; i < lam; i += 32) {
-            const long long p = si[i];
-            if (p >= p0 && p < p0 + 32) bits |= 1u << (int)(p - p0);
+// Everything of the decode state that a prefill only has to put in its place, in one launch of 256-thread blocks (as four
+// strided copies and two kernels it was 27 us of a 1003-token prompt, nearly all of it launches):
+//   kv_blocks per (K or V, batch, KV head): the rows [first, N) of the sequence into their ring rows (position q in row
+//     q % kvr; first > 0 only with a salient-cache budget), 16 bytes a thread and step;
+//   score_blocks per (batch, query head): the scores;
+//   then a warp per (batch, query head, chunk): the selected positions, also as bit masks -- bit j of word w is set when
+//     position chunk * C + 32 w + j is among them;
+//   the last block: the header.
+struct StateParts {
+    const char *K, *V;
+    char *k_cache, *v_cache;
+    const float *scores;
+    float *score_out;
+    const int32_t *sel;
+    int32_t *sel_out, *hdr;
+    uint32_t *mask_out;
+    long long N, first, kvr, cap, T, capT;
+    int BH, BHkv, row_bytes, C, lam, kv_blocks, score_blocks, sel_blocks;
+};
+constexpr int kStateSteps = 4;   // pieces (K / V) or scores per thread
+__global__ void __launch_bounds__(256)
+write_state_kernel(const __grid_constant__ StateParts s, const __grid_constant__ still_params_t p) {
+    grid_dep_wait();
+    grid_dep_launch();
+    long long blk = blockIdx.x;
+    const long long n_kv = 2ll * s.BHkv * s.kv_blocks, n_sc = (long long)s.BH * s.score_blocks;
+    if (blk < n_kv) {
+        const long long unit = blk / s.kv_blocks, head = unit >> 1;
+        const int ppr = s.row_bytes / 16;
+        const long long n = (s.N - s.first) * ppr, i0 = (blk - unit * s.kv_blocks) * (256 * kStateSteps) + threadIdx.x;
+        const uint4 *src = reinterpret_cast<const uint4 *>((unit & 1 ? s.V : s.K) + (head * s.N + s.first) * s.row_bytes);
+        uint4 *dst = reinterpret_cast<uint4 *>((unit & 1 ? s.v_cache : s.k_cache) + head * s.kvr * s.row_bytes);
+        uint4 v[kStateSteps];
+#pragma unroll
+        for (int k = 0; k < kStateSteps; ++k)
+            if (i0 + 256 * k < n) v[k] = src[i0 + 256 * k];
+#pragma unroll
+        for (int k = 0; k < kStateSteps; ++k) {
+            const long long i = i0 + 256 * k;
+            if (i < n) {
+                const uint32_t q = (uint32_t)(i / ppr + s.first), r = q < s.kvr ? q : q % (uint32_t)s.kvr;
+                dst[(long long)r * ppr + i % ppr] = v[k];
+            }
         }
-        bits = __reduce_or_sync(0xffffffffu, bits);
-        if (lane == 0) sel_mask[(bh * capT + c) * (C / 32) + w] = bits;
+        return;
     }
+    blk -= n_kv;
+    if (blk < n_sc) {
+        const long long bh = blk / s.score_blocks, i0 = (blk - bh * s.score_blocks) * (256 * kStateSteps) + threadIdx.x;
+#pragma unroll
+        for (int k = 0; k < kStateSteps; ++k)
+            if (i0 + 256 * k < s.N) s.score_out[bh * s.cap + i0 + 256 * k] = s.scores[bh * s.N + i0 + 256 * k];
+        return;
+    }
+    blk -= n_sc;
+    if (blk < s.sel_blocks) {
+        const long long wid = blk * 8 + (threadIdx.x >> 5);
+        if (wid >= (long long)s.BH * s.T) return;
+        const int lane = threadIdx.x & 31;
+        const long long bh = wid / s.T, c = wid % s.T;
+        const int32_t *si = s.sel + (bh * s.T + c) * s.lam;
+        int32_t *so = s.sel_out + (bh * s.capT + c) * s.lam;
+        int pos[4];
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            pos[i] = lane + 32 * i < s.lam ? si[lane + 32 * i] : -1;
+            if (lane + 32 * i < s.lam) so[lane + 32 * i] = pos[i];
+        }
+        for (int w = 0; w < s.C / 32; ++w) {
+            const long long p0 = c * s.C + 32ll * w;
+            uint32_t bits = 0u;
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+                if (pos[i] >= p0 && pos[i] < p0 + 32) bits |= 1u << (int)(pos[i] - p0);
+            bits = __reduce_or_sync(0xffffffffu, bits);
+            if (lane == 0) s.mask_out[(bh * s.capT + c) * (s.C / 32) + w] = bits;
+        }
+        return;
+    }
+    if (threadIdx.x == 0) write_header(s.hdr, p, s.cap, s.N);
 }
 
 // ------------------------------------------------------------------ FMA path launches
 
 template <typename T, int NJ>
 static int launch_score_select_t(const still_params_t *p, long long N, long long Tn, const T *Q, const T *K, float *scores,
-                                 int32_t *sel, cudaStream_t st) {
+                                 int32_t *sel, int *status, cudaStream_t st) {
     const size_t smem = score_select_smem(p->chunk, p->d);
     STILL_CUDA(set_smem(score_select_kernel<T, NJ>, smem));
-    score_select_kernel<T, NJ><<<dim3((unsigned)Tn, p->H, p->B), 256, smem, st>>>(Q, K, scores, sel, p->H, p->Hkv, N, p->d,
-                                                                                  p->topk, p->sm_scale, p->eps);
+    STILL_CUDA(launch_dependent(score_select_kernel<T, NJ>, dim3((unsigned)Tn, p->H, p->B), dim3(256), smem, st, Q, K, scores, sel, status, p->H,
+                                p->Hkv, N, p->d, p->topk, p->sm_scale, p->eps));
     ++g_launches;
-    STILL_CUDA(cudaGetLastError());
     return STILL_OK;
 }
 
 template <typename T>
 static int launch_score_select(const still_params_t *p, long long N, long long Tn, const T *Q, const T *K, float *scores,
-                               int32_t *sel, cudaStream_t st) {
+                               int32_t *sel, int *status, cudaStream_t st) {
     switch (p->chunk) {
-        case 32: return launch_score_select_t<T, 2>(p, N, Tn, Q, K, scores, sel, st);
-        case 64: return launch_score_select_t<T, 3>(p, N, Tn, Q, K, scores, sel, st);
-        default: return launch_score_select_t<T, 5>(p, N, Tn, Q, K, scores, sel, st);
+        case 32: return launch_score_select_t<T, 2>(p, N, Tn, Q, K, scores, sel, status, st);
+        case 64: return launch_score_select_t<T, 3>(p, N, Tn, Q, K, scores, sel, status, st);
+        default: return launch_score_select_t<T, 5>(p, N, Tn, Q, K, scores, sel, status, st);
     }
 }
 
@@ -226,9 +289,8 @@ static int launch_npmap(const still_params_t *p, long long N, int heads, const T
     const dim3 grid((unsigned)((N + 63) / 64), heads, p->B);
     auto launch = [&](auto kernel) -> int {
         STILL_CUDA(set_smem(kernel, smem));
-        kernel<<<grid, 256, smem, st>>>(X, W, bias, phi, heads, N, p->d);
+        STILL_CUDA(launch_dependent(kernel, grid, dim3(256), smem, st, X, W, bias, phi, heads, N, p->d));
         ++g_launches;
-        STILL_CUDA(cudaGetLastError());
         return STILL_OK;
     };
     switch (p->d_f) {
@@ -247,19 +309,17 @@ static int launch_la_scan_t(const still_params_t *p, long long N, long long Tn, 
     const int seg_chunks = (int)((Tn + n_seg - 1) / n_seg);
     n_seg = (int)((Tn + seg_chunks - 1) / seg_chunks);
     auto pass = [&](int segments, int sum_only) -> int {
-        la_seg_kernel<T, DP><<<dim3(p->B * p->H, segments, p->d / 64), 256, smem, st>>>(
-            phiQ, phiK, V, G, sel, nla, dla, sums, S_out, z_out, p->H, p->Hkv, N, p->d, p->chunk, p->topk, seg_chunks, n_seg, sum_only);
+        STILL_CUDA(launch_dependent(la_seg_kernel<T, DP>, dim3(p->B * p->H, segments, p->d / 64), dim3(256), smem, st, phiQ, phiK, V, G, sel,
+                                    nla, dla, sums, S_out, z_out, p->H, p->Hkv, N, p->d, p->chunk, p->topk, seg_chunks, n_seg, sum_only));
         ++g_launches;
-        STILL_CUDA(cudaGetLastError());
         return STILL_OK;
     };
     if (n_seg > 1) {
         int rc = pass(n_seg - 1, 1);
         if (rc != STILL_OK) return rc;
         const long long n4 = (long long)p->B * p->H * DP * (p->d + 1) / 4;
-        la_prefix_kernel<<<(unsigned)((n4 + 255) / 256), 256, 0, st>>>(sums, n4, n_seg);
+        STILL_CUDA(launch_dependent(la_prefix_kernel, dim3((unsigned)((n4 + 255) / 256)), dim3(256), 0, st, sums, n4, n_seg));
         ++g_launches;
-        STILL_CUDA(cudaGetLastError());
     }
     return pass(n_seg, 0);
 }
@@ -282,9 +342,9 @@ static int launch_sa_merge(const still_params_t *p, long long N, const T *Q, con
     auto launch = [&](auto kernel, int rows, int threads, int smem) -> int {
         STILL_CUDA(set_smem(kernel, smem));
         const dim3 grid((unsigned)((N + rows - 1) / rows), p->H, p->B);
-        kernel<<<grid, threads, smem, st>>>(Q, K, V, sel, nla, dla, Y, p->H, p->Hkv, N, p->chunk, p->topk, p->sm_scale);
+        STILL_CUDA(launch_dependent(kernel, grid, dim3(threads), smem, st, Q, K, V, sel, nla, dla, Y, p->H, p->Hkv, N, p->chunk, p->topk,
+                                    p->sm_scale));
         ++g_launches;
-        STILL_CUDA(cudaGetLastError());
         return STILL_OK;
     };
     // 64 rows a block halve the shared-memory reads per product; 32 where the chunk is that short or 64 would leave SMs idle
@@ -304,8 +364,7 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
     int rc;
     float *sc = scores ? scores : reinterpret_cast<float *>(ws + w.scores);
     int32_t *sel = sel_idx ? sel_idx : reinterpret_cast<int32_t *>(ws + w.sel_idx);
-    STILL_CUDA(cudaMemsetAsync(ws + w.status, 0, 256, st));
-
+    int *status = reinterpret_cast<int *>(ws + w.status);   // cleared by the first kernel
     still_state_layout_t L{};
     if (state) {
         if ((rc = plan_state(p, state_max_tokens, &L)) != STILL_OK) return rc;
@@ -314,9 +373,9 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
 
     // (1)+(2) Self-Saliency Score and per-chunk top-k.
     if (w.tc)
-        rc = tc_score_select(p, N, Q, K, sc, sel, reinterpret_cast<int *>(ws + w.status), st, &g_launches);
+        rc = tc_score_select(p, N, Q, K, sc, sel, status, st, &g_launches);
     else
-        rc = launch_score_select<T>(p, N, w.T, Q, K, sc, sel, st);
+        rc = launch_score_select<T>(p, N, w.T, Q, K, sc, sel, status, st);
     if (rc != STILL_OK) return rc;
 
     // (3) NP-Map + linear-attention scan (skipped when no token can be in M^LA).
@@ -335,7 +394,7 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
                               reinterpret_cast<float *>(ws + w.zpre), ypart, dpart, reinterpret_cast<float *>(ws + w.segs), S_out,
                               z_out, w.phiKsel ? ws + w.phiKsel : nullptr, Y && w.ksel ? ws + w.ksel : nullptr,
                               (Y || w.phiKsel) && w.vsel ? ws + w.vsel : nullptr, w.sel_rows,
-                              reinterpret_cast<int *>(ws + w.status), st, &g_launches);
+                              status, st, &g_launches);
             if (rc != STILL_OK) return rc;
         } else {
             T *phiQ = reinterpret_cast<T *>(ws + w.phiQ);
@@ -362,7 +421,7 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
     if (Y) {
         if (w.tc) {
             rc = tc_sa_merge(p, N, Q, K, V, sel, ypart, dpart, n_parts, Y, ws + w.ksel, ws + w.vsel, w.sel_rows, !w.tc_la,
-                             reinterpret_cast<int *>(ws + w.status), st, &g_launches);
+                             status, st, &g_launches);
         } else {
             profile_mark_begin(st);
             rc = launch_sa_merge<T>(p, N, Q, K, V, sel, nla, dla, Y, st);
@@ -373,38 +432,30 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
 
     // Decode state: K/V history, scores, selection; S and z were written above.
     if (state) {
-        const size_t es = sizeof(T);
-        const size_t BH = (size_t)p->B * p->H, BHkv = (size_t)p->B * p->Hkv;
-        // K / V history: the whole sequence, or with a budget the last kvr positions into their ring rows
-        // (position q in row q % kvr: at most two contiguous runs)
-        const long long kvr = state_kv_rows(p, L.capacity), first = std::max<long long>(0, N - kvr);
-        const size_t row = (size_t)p->d * es;
-        for (long long q0 = first; q0 < N;) {
-            const long long r0 = q0 % kvr, run = std::min<long long>(N - q0, kvr - r0);
-            STILL_CUDA(cudaMemcpy2DAsync(state + L.k_cache + r0 * row, kvr * row, reinterpret_cast<const char *>(K) + q0 * row,
-                                         (size_t)N * row, run * row, BHkv, cudaMemcpyDeviceToDevice, st));
-            STILL_CUDA(cudaMemcpy2DAsync(state + L.v_cache + r0 * row, kvr * row, reinterpret_cast<const char *>(V) + q0 * row,
-                                         (size_t)N * row, run * row, BHkv, cudaMemcpyDeviceToDevice, st));
-            q0 += run;
-        }
-        STILL_CUDA(cudaMemcpy2DAsync(state + L.score, (size_t)L.capacity * 4, sc, (size_t)N * 4,
-                                     (size_t)N * 4, BH, cudaMemcpyDeviceToDevice, st));
-        if (p->topk > 0)
-            STILL_CUDA(cudaMemcpy2DAsync(state + L.sel_idx, (size_t)(L.capacity / p->chunk) * p->topk * 4,
-                                         sel, (size_t)w.T * p->topk * 4, (size_t)w.T * p->topk * 4, BH,
-                                         cudaMemcpyDeviceToDevice, st));
-        if (p->topk > 0) {
-            const long long units = (long long)BH * w.T;
-            sel_mask_kernel<<<(unsigned)((units + 7) / 8), 256, 0, st>>>(
-                sel, reinterpret_cast<uint32_t *>(state + L.sel_mask), (long long)BH, w.T, L.capacity / p->chunk,
-                p->chunk, p->topk);
-            ++g_launches;
-            STILL_CUDA(cudaGetLastError());
-        }
-        write_header_kernel<<<1, 32, 0, st>>>(reinterpret_cast<int32_t *>(state + L.header), *p,
-                                              L.capacity, N);
+        const long long kvr = state_kv_rows(p, L.capacity);
+        StateParts sp{};
+        sp.K = reinterpret_cast<const char *>(K);
+        sp.V = reinterpret_cast<const char *>(V);
+        sp.k_cache = state + L.k_cache;
+        sp.v_cache = state + L.v_cache;
+        sp.scores = sc;
+        sp.score_out = reinterpret_cast<float *>(state + L.score);
+        sp.sel = sel;
+        sp.sel_out = reinterpret_cast<int32_t *>(state + L.sel_idx);
+        sp.mask_out = reinterpret_cast<uint32_t *>(state + L.sel_mask);
+        sp.hdr = reinterpret_cast<int32_t *>(state + L.header);
+        sp.N = N; sp.first = std::max<long long>(0, N - kvr); sp.kvr = kvr; sp.cap = L.capacity;
+        sp.T = w.T; sp.capT = L.capacity / p->chunk;
+        sp.BH = p->B * p->H; sp.BHkv = p->B * p->Hkv; sp.row_bytes = p->d * (int)sizeof(T);
+        sp.C = p->chunk; sp.lam = p->topk;
+        constexpr int kPer = 256 * kStateSteps;
+        sp.kv_blocks = (int)(((N - sp.first) * (sp.row_bytes / 16) + kPer - 1) / kPer);
+        sp.score_blocks = (int)((N + kPer - 1) / kPer);
+        sp.sel_blocks = p->topk > 0 ? (int)(((long long)sp.BH * w.T + 7) / 8) : 0;
+        const long long blocks = 2ll * sp.BHkv * sp.kv_blocks + (long long)sp.BH * sp.score_blocks + sp.sel_blocks + 1;
+        if (blocks >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;   // (a state of 32 TB)
+        STILL_CUDA(launch_dependent(write_state_kernel, dim3((unsigned)blocks), dim3(256), 0, st, sp, *p));
         ++g_launches;
-        STILL_CUDA(cudaGetLastError());
     }
     return STILL_OK;
 }

@@ -9,6 +9,13 @@ namespace still {
 // Words of the 256-byte status block at the start of a workspace / decode state.
 enum StatusWord { kStatusCode = 0, kStatusDetail = 1 };
 
+// Kernels of one call are launched with programmatic stream serialization (launch_dependent): a kernel's blocks are made
+// resident as soon as all blocks of its predecessor run, and wait here until the predecessor has ended and its writes are
+// visible.  Every kernel starts with the wait, in every block, so that the end of a kernel implies the end of all before
+// it, and reads nothing ahead of it.
+__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 __device__ __forceinline__ float ld_f(const float *p) { return *p; }
 __device__ __forceinline__ float ld_f(const __nv_bfloat16 *p) { return __bfloat162float(*p); }
 __device__ __forceinline__ void st_f(float *p, float v) { *p = v; }
@@ -28,6 +35,12 @@ __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
     return v;
+}
+
+// The first kernel of a call clears the workspace's status block.  Its first block does, at its start: a failure that
+// another block could record by then would be the end of a wait that takes seconds.
+__device__ __forceinline__ void clear_status(int *status) {
+    if (blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0 && threadIdx.x < 64) status[threadIdx.x] = 0;
 }
 
 // Records the first device-side failure (bounded wait expired, state mismatch).

@@ -38,6 +38,7 @@
 #include <algorithm>
 #include <type_traits>
 
+#include "still_common.cuh"
 #include "still_tc_ptx.cuh"
 
 namespace still {
@@ -80,6 +81,8 @@ __global__ void __launch_bounds__(192, 3)
 npmap_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
                 const __nv_bfloat16 *__restrict__ bias, TOut *__restrict__ phi, float *__restrict__ csum, int *status,
                 int heads, int N, int C) {
+    grid_dep_wait();
+    grid_dep_launch();
     constexpr int kXBytes = 128 * D * 2, kWBytes = D * DF * 2;
     using Lay = NpmapSmem<D, DF, TOut>;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -300,6 +303,8 @@ gather_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restri
               const int32_t *__restrict__ sel_idx, __nv_bfloat16 *__restrict__ Ksel, __nv_bfloat16 *__restrict__ Vsel,
               __nv_bfloat16 *__restrict__ phi_sel, float *__restrict__ selsum, int H, int Hkv, long long N, int lam,
               long long sel_rows, int n_routed) {
+    grid_dep_wait();
+    grid_dep_launch();
     constexpr int kVec = D / 8, kPhiVec = 2 * DF / 8;       // 16-byte pieces of a row
     constexpr int kPer = 32 / kVec, kPhiPer = 32 / kPhiVec;  // rows that a warp moves at a time
     __shared__ int pos[128];
@@ -374,6 +379,8 @@ gather_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restri
 __global__ void __launch_bounds__(1024)
 z_scan_kernel(const float *__restrict__ csum, const float *__restrict__ selsum, float *__restrict__ zpre, float *__restrict__ z_out,
               int H, int Hkv, int Tn, int n_routed, int all_selected, int window, int NF) {
+    grid_dep_wait();
+    grid_dep_launch();
     __shared__ float part[32][33];
     const int bh = blockIdx.x, b = bh / H, h = bh % H, warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int f = blockIdx.y * 32 + lane;
@@ -443,6 +450,8 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 float *__restrict__ d_part, float *__restrict__ S_out, float *__restrict__ seg_sums, int *status, int H, int Hkv,
                 int N, int C, int lam, int window, long long part_stride_y, long long part_stride_d, int seg_chunks, int n_seg,
                 int sum_parts, int sums_only, int sel_rows) {
+    grid_dep_wait();
+    grid_dep_launch();
     using P = FusedPlan<D, DF>;
     constexpr int NF = 2 * DF;
     extern __shared__ __align__(1024) uint8_t smem[];
@@ -1062,10 +1071,9 @@ int launch_npmap(const void *X, const void *W, const void *bias, void *phi, floa
     constexpr int kSmem = NpmapSmem<D, DF, TOut>::kTotal;
     if (ensure_dynamic_smem((const void *)npmap_tc_kernel<D, DF, TOut>, kSmem) != cudaSuccess) return STILL_ERR_CUDA;
     dim3 grid((unsigned)((N + 127) / 128), (unsigned)heads, (unsigned)B);
-    npmap_tc_kernel<D, DF, TOut><<<grid, 192, kSmem, st>>>(tx, tw, (const __nv_bfloat16 *)bias, (TOut *)phi, csum, status, heads,
-                                                          (int)N, C);
     ++*launches;
-    return cudaGetLastError() == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
+    return launch_dependent(npmap_tc_kernel<D, DF, TOut>, grid, dim3(192), kSmem, st, tx, tw, (const __nv_bfloat16 *)bias, (TOut *)phi,
+                            csum, status, heads, (int)N, C) == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
 }
 
 template <int D, int DF>
@@ -1074,11 +1082,10 @@ int launch_gather(const still_params_t *p, long long N, const void *K, const voi
                   int *launches) {
     using bf = __nv_bfloat16;
     const long long Tn = (N + p->chunk - 1) / p->chunk;
-    gather_kernel<D, DF><<<dim3((unsigned)(Tn + 1), (unsigned)(p->B * p->H)), 256, 0, st>>>(
-        (const bf *)K, (const bf *)V, (const bf *)phiK, sel_idx, (bf *)k_sel, (bf *)v_sel, (bf *)phiK_sel, selsum, p->H, p->Hkv, N,
-        p->topk, sel_rows, n_routed);
     ++*launches;
-    return cudaGetLastError() == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
+    return launch_dependent(gather_kernel<D, DF>, dim3((unsigned)(Tn + 1), (unsigned)(p->B * p->H)), dim3(256), 0, st, (const bf *)K,
+                            (const bf *)V, (const bf *)phiK, sel_idx, (bf *)k_sel, (bf *)v_sel, (bf *)phiK_sel, selsum, p->H, p->Hkv,
+                            N, p->topk, sel_rows, n_routed) == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
 }
 
 template <int D, int DF>
@@ -1111,13 +1118,13 @@ int launch_fused(const still_params_t *p, long long N, const void *Q, const void
     for (int pass = n_seg > 1 ? 0 : 1; pass < 2; ++pass) {
         // pass 0 (only with several segments): the sum of every segment's own updates; pass 1: the scan proper
         dim3 grid((unsigned)BH, 2, (unsigned)(pass == 0 ? (n_seg - 1) * parts : n_seg));   // head, feature half, segment (piece)
-        la_fused_kernel<D, DF><<<grid, 384, Plan::kTotal, st>>>(tq, tw, tk, tv, tks, tvs, (const bf *)bq, (const bf *)G, sel_idx, zpre,
+        const cudaError_t e = launch_dependent(la_fused_kernel<D, DF>, grid, dim3(384), Plan::kTotal, st, tq, tw, tk, tv, tks, tvs, (const bf *)bq, (const bf *)G, sel_idx, zpre,
                                                                (bf *)y_part, d_part, S_out, seg_sums, status, p->H, p->Hkv, (int)N,
                                                                p->chunk, p->topk, p->topk > 0 ? (int)(p->max_salient / p->topk) : 0,
                                                                (long long)BH * N * D, (long long)BH * N,
                                                                seg_chunks, n_seg, parts, pass == 0 ? 1 : 0, gathered ? (int)sel_rows : 0);
+        if (e != cudaSuccess) return STILL_ERR_CUDA;
         ++*launches;
-        if (cudaGetLastError() != cudaSuccess) return STILL_ERR_CUDA;
     }
     return STILL_OK;
 }
@@ -1180,10 +1187,10 @@ int tc_la_branch(const still_params_t *p, long long N, const void *Q, const void
     if (n_routed > 0 || z_out != nullptr) {
         // a warp per eight chunks, whose loads are in flight together; at most 32
         const int warps = std::max(1, std::min(32, (n_routed + 7) / 8));
-        z_scan_kernel<<<dim3((unsigned)BH, NF / 32), 32 * warps, 0, st>>>(csum, selsum, zpre, z_out, p->H, p->Hkv, (int)Tn, n_routed,
-                                                                    p->topk >= C ? 1 : 0, window, NF);
+        if (launch_dependent(z_scan_kernel, dim3((unsigned)BH, NF / 32), dim3(32 * warps), 0, st, csum, selsum, zpre, z_out, p->H, p->Hkv,
+                             (int)Tn, n_routed, p->topk >= C ? 1 : 0, window, NF) != cudaSuccess)
+            return STILL_ERR_CUDA;
         ++*launches;
-        if (cudaGetLastError() != cudaSuccess) return STILL_ERR_CUDA;
     }
     if (p->d == 64 && p->d_f == 64)
         return launch_fused<64, 64>(p, N, Q, V, G, Wq, bq, sel_idx, phiK, zpre, y_part, d_part, S_out, seg_sums, phiK_sel, v_sel, sel_rows,

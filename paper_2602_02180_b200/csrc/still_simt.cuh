@@ -56,7 +56,10 @@ inline size_t score_select_smem(int C, int d) {
 template <typename T, int NJ>
 __global__ void __launch_bounds__(256)
 score_select_kernel(const T *__restrict__ Q, const T *__restrict__ K, float *__restrict__ scores,
-                    int32_t *__restrict__ sel_idx, int H, int Hkv, long long N, int d, int lam, float scale, float eps) {
+                    int32_t *__restrict__ sel_idx, int *status, int H, int Hkv, long long N, int d, int lam, float scale, float eps) {
+    grid_dep_wait();
+    grid_dep_launch();
+    clear_status(status);
     constexpr int C = 32 * (NJ - 1);
     extern __shared__ __align__(16) float smem[];
     const int c = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
@@ -158,6 +161,8 @@ template <typename T, int DF>
 __global__ void __launch_bounds__(256)
 npmap_kernel(const T *__restrict__ X, const T *__restrict__ W, const T *__restrict__ bias,
              T *__restrict__ phi, int heads, long long N, int d) {
+    grid_dep_wait();
+    grid_dep_launch();
     constexpr int VC = DF >= 64 ? 4 : 2, NV = DF / (16 * VC);   // columns VC (tc + 16 j) .. + VC
     extern __shared__ __align__(16) float smem[];
     const int ds = d + 4, d4 = d >> 2;
@@ -299,6 +304,8 @@ la_seg_kernel(const T *__restrict__ phiQ, const T *__restrict__ phiK, const T *_
               float *__restrict__ D_LA, float *__restrict__ sums, float *__restrict__ S_out,
               float *__restrict__ z_out, int H, int Hkv, long long N, int d, int C, int lam, int seg_chunks,
               int n_seg, int sum_only) {
+    grid_dep_wait();
+    grid_dep_launch();
     constexpr int FPT = DP / 16;
     extern __shared__ __align__(16) float smem[];
     float *ph = smem;                 // [64][DP] feature rows of the current sub-tile
@@ -476,6 +483,8 @@ la_seg_kernel(const T *__restrict__ phiQ, const T *__restrict__ phiK, const T *_
 // sums [n_seg][n]: segment s receives the sum of the segments before it (the last segment's own sum is not needed).
 __global__ void __launch_bounds__(256)
 la_prefix_kernel(float *__restrict__ sums, long long n4, int n_seg) {
+    grid_dep_wait();
+    grid_dep_launch();
     const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
     if (i >= n4) return;
     float4 *p = reinterpret_cast<float4 *>(sums) + i;
@@ -520,6 +529,8 @@ sa_merge_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
                 const int32_t *__restrict__ sel_idx, const float *__restrict__ N_LA,
                 const float *__restrict__ D_LA, T *__restrict__ Y, int H, int Hkv, long long N, int C,
                 int lam, float scale) {
+    grid_dep_wait();
+    grid_dep_launch();
     using P = SaPlan<D, ROWS, RT>;
     constexpr int KT = P::KT, kThreads = P::kThreads, NK = KT / 16, NV = D / 64, DS = D + 4, PS = KT + 4;
     extern __shared__ __align__(16) float smem[];

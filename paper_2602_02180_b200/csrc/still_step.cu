@@ -37,10 +37,6 @@ size_t step_scratch_bytes(const still_params_t *p, long long) {
     return (size_t)p->B * p->H * kRecords * (p->d + 2) * sizeof(float);
 }
 
-// The kernel's predecessor in the stream has ended and its writes are visible; the successor may be made resident.
-__device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // What a step expects to find in the header of the decode state.
 struct StateKey {
     int32_t B, H, Hkv, d, d_f, chunk, topk, dtype;
@@ -771,21 +767,6 @@ step_merge_kernel(const __grid_constant__ StepArgs<T> a) {
         cudaError_t e__ = (expr);                      \
         if (e__ != cudaSuccess) return STILL_ERR_CUDA; \
     } while (0)
-
-template <typename... Params, typename... Args>
-static cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args... args) {
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = grid;
-    cfg.blockDim = block;
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
 
 template <typename T>
 static int launch_route(const still_params_t *p, const StepArgs<T> &a, int32_t *sel, const T *Wk, const T *bk, long long cr,

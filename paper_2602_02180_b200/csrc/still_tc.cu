@@ -345,6 +345,8 @@ sa_merge_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
                    const __grid_constant__ CUtensorMap tm_vsel, const __nv_bfloat16 *__restrict__ y_part,
                    const float *__restrict__ d_part, int n_parts, __nv_bfloat16 *__restrict__ Y, int *status, int H, int Hkv,
                    int N, int C, int lam, int budget, int sel_rows, int sel_identity, float scale_log2, int n_qblocks) {
+    grid_dep_wait();
+    grid_dep_launch();
     using P = SmemPlan<D>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -637,6 +639,8 @@ sa_merge_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
                      const __grid_constant__ CUtensorMap tm_vsel, const __nv_bfloat16 *__restrict__ y_part,
                      const float *__restrict__ d_part, int n_parts, __nv_bfloat16 *__restrict__ Y, int *status, int H, int Hkv, int N,
                      int C, int lam, int budget, int sel_rows, int sel_identity, float scale_log2, int n_pairs) {
+    grid_dep_wait();
+    grid_dep_launch();
     using P = PairPlan<D>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -946,6 +950,9 @@ __global__ void __launch_bounds__(320, 1)
 score_select_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        float *__restrict__ scores, int32_t *__restrict__ sel_idx, int *status, int H, int Hkv,
                        int N, int lam, float scale_log2, float eps, int n_row_blocks, int n_tiles) {
+    grid_dep_wait();
+    grid_dep_launch();
+    clear_status(status);
     using P = ScoreSmem<D>;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
@@ -1195,6 +1202,8 @@ __global__ void __launch_bounds__(256)
 compact_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restrict__ V,
                const int32_t *__restrict__ sel_idx, __nv_bfloat16 *__restrict__ Ksel,
                __nv_bfloat16 *__restrict__ Vsel, int H, int Hkv, long long N, long long n_idx, long long sel_rows) {
+    grid_dep_wait();
+    grid_dep_launch();
     const int bh = blockIdx.y, b = bh / H, h = bh % H, kvh = h / (H / Hkv);
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long j = (long long)blockIdx.x * 8 + warp;
@@ -1246,10 +1255,10 @@ int launch_tc(const still_params_t *p, long long N, const void *Q, const void *K
     const bool identity = p->topk == p->chunk;  // the selection of every chunk is the chunk itself
     if (!identity && compact) {
         dim3 grid((unsigned)((sel_rows + 7) / 8), (unsigned)BH);
-        compact_kernel<D><<<grid, 256, 0, st>>>((const bf *)K, (const bf *)V, sel_idx, (bf *)k_sel, (bf *)v_sel, p->H,
-                                               p->Hkv, N, n_idx, sel_rows);
+        if (launch_dependent(compact_kernel<D>, grid, dim3(256), 0, st, (const bf *)K, (const bf *)V, sel_idx, (bf *)k_sel, (bf *)v_sel,
+                             p->H, p->Hkv, N, n_idx, sel_rows) != cudaSuccess)
+            return STILL_ERR_CUDA;
         ++*launches;
-        if (cudaGetLastError() != cudaSuccess) return STILL_ERR_CUDA;
     }
     const unsigned long long kv_rows = (unsigned long long)p->B * p->Hkv * N;
     const unsigned long long sel_total = identity ? kv_rows : (unsigned long long)BH * sel_rows;
@@ -1266,19 +1275,21 @@ int launch_tc(const still_params_t *p, long long N, const void *Q, const void *K
         if (ensure_dynamic_smem((const void *)sa_merge_pair_kernel<D>, PairPlan<D>::kAlloc) != cudaSuccess) return STILL_ERR_CUDA;
         dim3 grid((unsigned)(2 * n_pairs), (unsigned)BH);   // clusters of two along x
         profile_mark_begin(st);
-        sa_merge_pair_kernel<D><<<grid, kThreads, PairPlan<D>::kAlloc, st>>>(
+        const cudaError_t e = launch_dependent(sa_merge_pair_kernel<D>, grid, dim3(kThreads), PairPlan<D>::kAlloc, st,
             tq, tk, tv, tks, tvs, (const bf *)y_part, d_part, n_parts, (bf *)Y, status, p->H, p->Hkv, (int)N, p->chunk, p->topk, (int)p->max_salient, (int)sel_rows,
             identity ? 1 : 0, scale_log2, n_pairs);
         profile_mark_end(st);
+        if (e != cudaSuccess) return STILL_ERR_CUDA;
     } else {
         const int n_qblocks = (int)((N + 2 * kBlockM - 1) / (2 * kBlockM));
         if (ensure_dynamic_smem((const void *)sa_merge_tc_kernel<D>, SmemPlan<D>::kAlloc) != cudaSuccess) return STILL_ERR_CUDA;
         dim3 grid((unsigned)n_qblocks, (unsigned)BH);
         profile_mark_begin(st);
-        sa_merge_tc_kernel<D><<<grid, kThreads, SmemPlan<D>::kAlloc, st>>>(
+        const cudaError_t e = launch_dependent(sa_merge_tc_kernel<D>, grid, dim3(kThreads), SmemPlan<D>::kAlloc, st,
             tq, tk, tv, tks, tvs, (const bf *)y_part, d_part, n_parts, (bf *)Y, status, p->H, p->Hkv, (int)N, p->chunk, p->topk, (int)p->max_salient, (int)sel_rows,
             identity ? 1 : 0, scale_log2, n_qblocks);
         profile_mark_end(st);
+        if (e != cudaSuccess) return STILL_ERR_CUDA;
     }
     ++*launches;
     if (cudaGetLastError() != cudaSuccess) return STILL_ERR_CUDA;
@@ -1303,10 +1314,11 @@ int launch_score_tc(const still_params_t *p, long long N, const void *Q, const v
     const long long n_row_blocks = (N + kBlockM - 1) / kBlockM, n_tiles = n_row_blocks * BH;
     if (n_tiles >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;
     const unsigned grid = (unsigned)std::min<long long>(n_tiles, n_sm);   // one persistent CTA per SM
-    kernel<<<grid, 320, kSmem, st>>>(tq, tk, scores, sel_idx, status, p->H, p->Hkv, (int)N, p->topk, p->sm_scale * 1.4426950408889634f, p->eps,
-                                                           (int)n_row_blocks, (int)n_tiles);
+    if (launch_dependent(kernel, dim3(grid), dim3(320), kSmem, st, tq, tk, scores, sel_idx, status, p->H, p->Hkv, (int)N, p->topk,
+                         p->sm_scale * 1.4426950408889634f, p->eps, (int)n_row_blocks, (int)n_tiles) != cudaSuccess)
+        return STILL_ERR_CUDA;
     ++*launches;
-    return cudaGetLastError() == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
+    return STILL_OK;
 }
 
 }  // namespace
@@ -1323,6 +1335,8 @@ int tc_score_select(const still_params_t *p, long long N, const void *Q, const v
 // N_LA / D_LA of the fp32-accumulating FMA kernels as one bf16 part: y = N_LA / D_LA, d = D_LA.
 __global__ void la_to_part_kernel(const float *__restrict__ N_LA, const float *__restrict__ D_LA, __nv_bfloat16 *__restrict__ y,
                                   float *__restrict__ dp, long long rows, int d) {
+    grid_dep_wait();
+    grid_dep_launch();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= rows * d) return;
     const long long r = i / d;
@@ -1334,9 +1348,9 @@ __global__ void la_to_part_kernel(const float *__restrict__ N_LA, const float *_
 int tc_la_to_part(const float *N_LA, const float *D_LA, void *y_part, float *d_part, long long rows, int d, cudaStream_t st,
                   int *launches) {
     const long long n = rows * d;
-    la_to_part_kernel<<<(unsigned)((n + 255) / 256), 256, 0, st>>>(N_LA, D_LA, (__nv_bfloat16 *)y_part, d_part, rows, d);
     ++*launches;
-    return cudaGetLastError() == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
+    return launch_dependent(la_to_part_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, N_LA, D_LA, (__nv_bfloat16 *)y_part,
+                            d_part, rows, d) == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
 }
 
 int tc_selftest_wait_timeout(int *status_words, long long limit_cycles, cudaStream_t st) {

@@ -28,6 +28,22 @@ inline cudaError_t ensure_dynamic_smem(const void *func, int bytes) {
     return e;
 }
 
+// Launch with programmatic stream serialization (see grid_dep_wait in still_common.cuh).
+template <typename... Params, typename... Args>
+inline cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 block, size_t smem, cudaStream_t st, Args &&...args) {
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = grid;
+    cfg.blockDim = block;
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+}
+
 // ---- timing of the dominant kernel (still_profile_enable / still_profile_collect) ----
 void profile_mark_begin(cudaStream_t st);
 void profile_mark_end(cudaStream_t st);
