@@ -185,6 +185,34 @@ def test_fma_kernels_feature_sizes_and_bias(dtype, d, df, C, k, N):
     U.check_outputs(w, Q, K, V, Wq, Wk, Y, scores, sel, heads, G=G, bq=bq, bk=bk)
 
 
+@pytest.mark.parametrize("d,C", [(64, 64), (128, 128)])
+def test_scores_with_a_subnormal_eps(d, C):
+    # every logarithm's argument contains eps; a subnormal one takes the form that scales its argument.  Scores reach
+    # log(1 / eps) = 90 here, seven times the range the score tolerance is stated for.
+    w = _small("t", "bf16", 1, 4, 2, d, C * 3 + 9, C, C // 4)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    Wq, Wk = synth.make_npmap_weights(w, "cuda")
+    p = still.StillParams(w.B, w.H, w.Hkv, d, C, w.k, torch.bfloat16, sm_scale=w.sm_scale, eps=1e-39)
+    Y, scores, sel = still.hybrid_attn_fwd(p, Q, K, V, Wq, Wk)
+    heads = [(0, h) for h in range(4)]
+    U.check_selection(scores, sel, C, w.k, heads)
+    U.check_outputs(w, Q, K, V, Wq, Wk, Y, scores, sel, heads, eps=float(np.float32(1e-39)), score_tol=7 * U.SCORE_TOL[torch.bfloat16])
+
+
+@pytest.mark.parametrize("d,B,H,Hkv,N", [(64, 3, 6, 2, 700), (128, 1, 8, 4, 1100), (64, 1, 8, 4, 128 * 1024 + 70), (128, 1, 4, 2, 64 * 1024 + 200)])
+def test_row_blocks_of_all_heads(d, B, H, Hkv, N):
+    # every row block of every head is worked on once, with the heads in one set and in several (65536 keys of a KV group
+    # at d = 128, 131072 at d = 64, fill a set): rows that were left out would keep the NaN they start with
+    w = _small("t", "bf16", B, H, Hkv, d, N, 64, 64)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    p = U.params_of(w)
+    Y, scores, sel = still.hybrid_attn_fwd(p, Q, K, V, Y=torch.full_like(Q, float("nan")))
+    heads = U.sample_heads(w, 3)
+    rows = U.sample_rows(N, 12, 64)
+    U.check_outputs(w, Q, K, V, *synth.make_npmap_weights(w, "cuda"), Y, scores, sel, heads, rows=rows)
+    assert bool(torch.isfinite(Y.float()).all())
+
+
 @pytest.mark.parametrize("k", [64, 16])
 def test_growing_logits_rescale_the_accumulator(k):
     # The tensor-core kernel keeps a row's softmax reference until a tile's maximum exceeds it by 2^8 and then
