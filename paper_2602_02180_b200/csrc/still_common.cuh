@@ -12,7 +12,11 @@ enum StatusWord { kStatusCode = 0, kStatusDetail = 1 };
 // Kernels of one call are launched with programmatic stream serialization (launch_dependent): a kernel's blocks are made
 // resident as soon as all blocks of its predecessor run, and wait here until the predecessor has ended and its writes are
 // visible.  Every kernel starts with the wait, in every block, so that the end of a kernel implies the end of all before
-// it, and reads nothing ahead of it.
+// it, and reads nothing ahead of it.  For the same reason no pointer parameter of such a kernel is restrict-qualified:
+// with const it would promise memory that nobody writes while the kernel is resident, which lets the compiler move a
+// load above the wait, and here the memory is written until the wait returns -- by the call's earlier kernels, and the
+// inputs by whatever kernel the caller launched before.  Where loads have to be in flight together ahead of stores the
+// code says so itself, by loading into registers first.
 __device__ __forceinline__ void grid_dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void grid_dep_launch() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 

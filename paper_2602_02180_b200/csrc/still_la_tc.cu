@@ -79,7 +79,7 @@ struct NpmapSmem {
 template <int D, int DF, typename TOut>
 __global__ void __launch_bounds__(192, 3)
 npmap_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant__ CUtensorMap tm_w,
-                const __nv_bfloat16 *__restrict__ bias, TOut *__restrict__ phi, float *__restrict__ csum, int *status,
+                const __nv_bfloat16 *bias, TOut *phi, float *csum, int *status,
                 int heads, int N, int C) {
     grid_dep_wait();
     grid_dep_launch();
@@ -299,9 +299,9 @@ npmap_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
 // gathered for themselves (and one that summed a row after the other) took 1023 us.
 template <int D, int DF>
 __global__ void __launch_bounds__(256)
-gather_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restrict__ V, const __nv_bfloat16 *__restrict__ phiK,
-              const int32_t *__restrict__ sel_idx, __nv_bfloat16 *__restrict__ Ksel, __nv_bfloat16 *__restrict__ Vsel,
-              __nv_bfloat16 *__restrict__ phi_sel, float *__restrict__ selsum, int H, int Hkv, long long N, int lam,
+gather_kernel(const __nv_bfloat16 *K, const __nv_bfloat16 *V, const __nv_bfloat16 *phiK,
+              const int32_t *sel_idx, __nv_bfloat16 *Ksel, __nv_bfloat16 *Vsel,
+              __nv_bfloat16 *phi_sel, float *selsum, int H, int Hkv, long long N, int lam,
               long long sel_rows, int n_routed) {
     grid_dep_wait();
     grid_dep_launch();
@@ -331,12 +331,18 @@ gather_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restri
         const __nv_bfloat16 *src = which ? V : K;
         __nv_bfloat16 *dst = which ? Vsel : Ksel;
         if (dst != nullptr) {
-#pragma unroll 4
-            for (int r = warp * (kPer / 2) + lane / (2 * kVec); r < lam; r += 8 * (kPer / 2)) {
-                const int p = pos[r];
-                uint4 v = make_uint4(0, 0, 0, 0);
-                if (p >= 0) v = reinterpret_cast<const uint4 *>(src + (src0 + p) * D)[piece];
-                reinterpret_cast<uint4 *>(dst + (dst0 + r) * D)[piece] = v;
+            constexpr int kStep = 8 * (kPer / 2);
+            for (int r0 = warp * (kPer / 2) + lane / (2 * kVec); r0 < lam; r0 += 4 * kStep) {
+                uint4 v[4];   // (four rows requested before the first is stored)
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const int r = r0 + i * kStep, p = r < lam ? pos[r] : -1;
+                    v[i] = make_uint4(0, 0, 0, 0);
+                    if (p >= 0) v[i] = reinterpret_cast<const uint4 *>(src + (src0 + p) * D)[piece];
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    if (r0 + i * kStep < lam) reinterpret_cast<uint4 *>(dst + (dst0 + r0 + i * kStep) * D)[piece] = v[i];
             }
         }
     }
@@ -346,17 +352,25 @@ gather_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restri
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-#pragma unroll 4
-    for (int r = warp * kPhiPer + lane / kPhiVec; r < lam; r += 8 * kPhiPer) {
-        const int p = pos[r];
-        uint4 v = make_uint4(0, 0, 0, 0);
-        if (p >= 0) v = reinterpret_cast<const uint4 *>(phiK + (src0 + p) * (2 * DF))[piece];
-        if (phi_sel) reinterpret_cast<uint4 *>(phi_sel + (dst0 + r) * (2 * DF))[piece] = v;
-        const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+    constexpr int kPhiStep = 8 * kPhiPer;
+    for (int r0 = warp * kPhiPer + lane / kPhiVec; r0 < lam; r0 += 4 * kPhiStep) {
+        uint4 v[4];
 #pragma unroll
-        for (int e = 0; e < 4; ++e) {
-            acc[2 * e] += __uint_as_float(w[e] << 16);
-            acc[2 * e + 1] += __uint_as_float(w[e] & 0xffff0000u);
+        for (int i = 0; i < 4; ++i) {
+            const int r = r0 + i * kPhiStep, p = r < lam ? pos[r] : -1;
+            v[i] = make_uint4(0, 0, 0, 0);
+            if (p >= 0) v[i] = reinterpret_cast<const uint4 *>(phiK + (src0 + p) * (2 * DF))[piece];
+        }
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const int r = r0 + i * kPhiStep;
+            if (phi_sel && r < lam) reinterpret_cast<uint4 *>(phi_sel + (dst0 + r) * (2 * DF))[piece] = v[i];
+            const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+#pragma unroll
+            for (int e = 0; e < 4; ++e) {
+                acc[2 * e] += __uint_as_float(w[e] << 16);
+                acc[2 * e + 1] += __uint_as_float(w[e] & 0xffff0000u);
+            }
         }
     }
     if (c >= n_routed) return;
@@ -377,7 +391,7 @@ gather_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restri
 // warps sums a part of the chunks, and adds them up again from the sum of the parts before.  (One thread per feature
 // over all chunks took 132 us for 1022 chunks of 32 heads, a chain of loads; this takes 53 us.)
 __global__ void __launch_bounds__(1024)
-z_scan_kernel(const float *__restrict__ csum, const float *__restrict__ selsum, float *__restrict__ zpre, float *__restrict__ z_out,
+z_scan_kernel(const float *csum, const float *selsum, float *zpre, float *z_out,
               int H, int Hkv, int Tn, int n_routed, int all_selected, int window, int NF) {
     grid_dep_wait();
     grid_dep_launch();
@@ -401,10 +415,15 @@ z_scan_kernel(const float *__restrict__ csum, const float *__restrict__ selsum, 
     __syncthreads();
     acc = 0.f;
     for (int w = 0; w < warp; ++w) acc += part[w][lane];
-#pragma unroll 8
-    for (int c = c0; c < c1; ++c) {
-        acc += delta(c);
-        z[(long long)c * NF] = acc;
+    for (int c = c0; c < c1; c += 8) {   // (eight chunks requested before the first is stored)
+        float d[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) d[i] = c + i < c1 ? delta(c + i) : 0.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+            acc += d[i];
+            if (c + i < c1) z[(long long)(c + i) * NF] = acc;
+        }
     }
     if (z_out != nullptr && warp == warps - 1) z_out[(long long)bh * NF + f] = acc;
 }
@@ -445,9 +464,9 @@ __global__ void __launch_bounds__(384, 1)
 la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_wq,
                 const __grid_constant__ CUtensorMap tm_phik, const __grid_constant__ CUtensorMap tm_v,
                 const __grid_constant__ CUtensorMap tm_phiks, const __grid_constant__ CUtensorMap tm_vs,
-                const __nv_bfloat16 *__restrict__ bq, const __nv_bfloat16 *__restrict__ G,
-                const int32_t *__restrict__ sel_idx, const float *__restrict__ zpre, __nv_bfloat16 *__restrict__ y_part,
-                float *__restrict__ d_part, float *__restrict__ S_out, float *__restrict__ seg_sums, int *status, int H, int Hkv,
+                const __nv_bfloat16 *bq, const __nv_bfloat16 *G,
+                const int32_t *sel_idx, const float *zpre, __nv_bfloat16 *y_part,
+                float *d_part, float *S_out, float *seg_sums, int *status, int H, int Hkv,
                 int N, int C, int lam, int window, long long part_stride_y, long long part_stride_d, int seg_chunks, int n_seg,
                 int sum_parts, int sums_only, int sel_rows) {
     grid_dep_wait();

@@ -55,8 +55,8 @@ inline size_t score_select_smem(int C, int d) {
 }
 template <typename T, int NJ>
 __global__ void __launch_bounds__(256)
-score_select_kernel(const T *__restrict__ Q, const T *__restrict__ K, float *__restrict__ scores,
-                    int32_t *__restrict__ sel_idx, int *status, int H, int Hkv, long long N, int d, int lam, float scale, float eps) {
+score_select_kernel(const T *Q, const T *K, float *scores,
+                    int32_t *sel_idx, int *status, int H, int Hkv, long long N, int d, int lam, float scale, float eps) {
     grid_dep_wait();
     grid_dep_launch();
     clear_status(status);
@@ -159,8 +159,8 @@ score_select_kernel(const T *__restrict__ Q, const T *__restrict__ K, float *__r
 inline size_t npmap_smem(int d, int df) { return ((size_t)d * df + (size_t)64 * (d + 4)) * 4; }
 template <typename T, int DF>
 __global__ void __launch_bounds__(256)
-npmap_kernel(const T *__restrict__ X, const T *__restrict__ W, const T *__restrict__ bias,
-             T *__restrict__ phi, int heads, long long N, int d) {
+npmap_kernel(const T *X, const T *W, const T *bias,
+             T *phi, int heads, long long N, int d) {
     grid_dep_wait();
     grid_dep_launch();
     constexpr int VC = DF >= 64 ? 4 : 2, NV = DF / (16 * VC);   // columns VC (tc + 16 j) .. + VC
@@ -299,10 +299,10 @@ npmap_kernel(const T *__restrict__ X, const T *__restrict__ W, const T *__restri
 inline size_t la_seg_smem(int dp) { return ((size_t)64 * dp + 64 * 64 + (size_t)dp * 64 + dp) * 4 + 64 * 4 + 16; }
 template <typename T, int DP>
 __global__ void __launch_bounds__(256)
-la_seg_kernel(const T *__restrict__ phiQ, const T *__restrict__ phiK, const T *__restrict__ V,
-              const T *__restrict__ G, const int32_t *__restrict__ sel_idx, float *__restrict__ N_LA,
-              float *__restrict__ D_LA, float *__restrict__ sums, float *__restrict__ S_out,
-              float *__restrict__ z_out, int H, int Hkv, long long N, int d, int C, int lam, int seg_chunks,
+la_seg_kernel(const T *phiQ, const T *phiK, const T *V,
+              const T *G, const int32_t *sel_idx, float *N_LA,
+              float *D_LA, float *sums, float *S_out,
+              float *z_out, int H, int Hkv, long long N, int d, int C, int lam, int seg_chunks,
               int n_seg, int sum_only) {
     grid_dep_wait();
     grid_dep_launch();
@@ -426,6 +426,10 @@ la_seg_kernel(const T *__restrict__ phiQ, const T *__restrict__ phiK, const T *_
             stage_wait();
             __syncthreads();
             if (4 * tf < rows) {   // rows 4 tf .. + 3 (rows past the end hold stale features and are not stored)
+                float4 gate[4];    // (requested ahead of the products and of the stores)
+#pragma unroll
+                for (int i = 0; i < 4; ++i)
+                    gate[i] = G && 4 * tf + i < rows ? ld4(G + ((long long)bh * N + base + 4 * tf + i) * d + e0 + 4 * te) : make_float4(1.f, 1.f, 1.f, 1.f);
                 float2 acc[4][2];
 #pragma unroll
                 for (int i = 0; i < 4; ++i) acc[i][0] = acc[i][1] = make_float2(0.f, 0.f);
@@ -450,10 +454,7 @@ la_seg_kernel(const T *__restrict__ phiQ, const T *__restrict__ phiK, const T *_
                     if (4 * tf + i < rows) {
                         const long long o = ((long long)bh * N + base + 4 * tf + i) * d + e0 + 4 * te;
                         float4 v = make_float4(acc[i][0].x, acc[i][0].y, acc[i][1].x, acc[i][1].y);
-                        if (G) {
-                            const float4 gg = ld4(G + o);
-                            v = make_float4(v.x * gg.x, v.y * gg.y, v.z * gg.z, v.w * gg.w);
-                        }
+                        if (G) v = make_float4(v.x * gate[i].x, v.y * gate[i].y, v.z * gate[i].z, v.w * gate[i].w);
                         st4(N_LA + o, v);
                     }
             }
@@ -482,7 +483,7 @@ la_seg_kernel(const T *__restrict__ phiQ, const T *__restrict__ phiK, const T *_
 }
 // sums [n_seg][n]: segment s receives the sum of the segments before it (the last segment's own sum is not needed).
 __global__ void __launch_bounds__(256)
-la_prefix_kernel(float *__restrict__ sums, long long n4, int n_seg) {
+la_prefix_kernel(float *sums, long long n4, int n_seg) {
     grid_dep_wait();
     grid_dep_launch();
     const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
@@ -525,9 +526,9 @@ struct SaPlan {
 };
 template <typename T, int D, int ROWS, int RT>
 __global__ void __launch_bounds__(SaPlan<D, ROWS, RT>::kThreads)
-sa_merge_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__restrict__ V,
-                const int32_t *__restrict__ sel_idx, const float *__restrict__ N_LA,
-                const float *__restrict__ D_LA, T *__restrict__ Y, int H, int Hkv, long long N, int C,
+sa_merge_kernel(const T *Q, const T *K, const T *V,
+                const int32_t *sel_idx, const float *N_LA,
+                const float *D_LA, T *Y, int H, int Hkv, long long N, int C,
                 int lam, float scale) {
     grid_dep_wait();
     grid_dep_launch();
@@ -650,13 +651,22 @@ sa_merge_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
         }
         __syncwarp();
     }
+    float dlas[RT];
+    float4 nla[RT][NV];   // the linear branch's rows, requested together
+#pragma unroll
+    for (int r = 0; r < RT; ++r) {
+        const long long t = row0 + ty * RT + r;
+        dlas[r] = D_LA && t < N ? D_LA[bh * N + t] : 0.f;
+#pragma unroll
+        for (int e = 0; e < NV; ++e) nla[r][e] = dlas[r] > 0.f ? ld4(N_LA + (bh * N + t) * D + 64 * e + 4 * tx) : make_float4(0.f, 0.f, 0.f, 0.f);
+    }
 #pragma unroll
     for (int r = 0; r < RT; ++r) {
         const long long t = row0 + ty * RT + r;
 #pragma unroll
         for (int w = 8; w > 0; w >>= 1) l[r] += __shfl_xor_sync(0xffffffffu, l[r], w);
         if (t >= N) continue;
-        const float dla = D_LA ? D_LA[bh * N + t] : 0.f;
+        const float dla = dlas[r];
         float fs = 1.f, fl = 0.f;
         if (dla > 0.f) {
             const float ms = fmaxf(m[r], 0.f);
@@ -669,7 +679,7 @@ sa_merge_kernel(const T *__restrict__ Q, const T *__restrict__ K, const T *__res
             const long long oidx = (bh * N + t) * D + 64 * e + 4 * tx;
             float4 num = make_float4(o[r][2 * e].x * fs, o[r][2 * e].y * fs, o[r][2 * e + 1].x * fs, o[r][2 * e + 1].y * fs);
             if (dla > 0.f) {
-                const float4 n = ld4(N_LA + oidx);
+                const float4 n = nla[r][e];
                 num = make_float4(num.x + fl * n.x, num.y + fl * n.y, num.z + fl * n.z, num.w + fl * n.w);
             }
             st4(Y + oidx, make_float4(num.x / den, num.y / den, num.z / den, num.w / den));

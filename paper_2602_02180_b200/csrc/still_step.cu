@@ -391,8 +391,8 @@ step_route_mma_kernel(__nv_bfloat16 *kc, __nv_bfloat16 *vc, float *score, int32_
     cp_async_wait<0>();
 }
 
-// Arguments of step_main_kernel / step_merge_kernel.  (Pointers are neither const nor restrict: their contents come
-// from kernels that may still run when a block becomes resident, and must not be loaded ahead of the wait.)
+// Arguments of step_main_kernel / step_merge_kernel.  (Their contents come from kernels that may still run when a block
+// becomes resident, and must not be loaded ahead of the wait: see grid_dep_wait.)
 template <typename T>
 struct StepArgs {
     T *kc, *vc;

@@ -138,9 +138,9 @@ template <int D, int kKStages, int kVStages, bool kPair, int kPolyOf4, class Str
 __device__ __forceinline__ void softmax_role(const StreamT &st, const int x, const int tile_row0, const uint32_t tmem_base,
                                              uint64_t *s_full, uint64_t *k_empty, uint64_t *v_empty, uint64_t *p_half,
                                              const uint32_t p_half_cluster, uint64_t *o_final, volatile int *abort_flag,
-                                             int *status, uint8_t *stage_tile, const __nv_bfloat16 *__restrict__ y_part,
-                                             const float *__restrict__ d_part, const int n_parts, const long long part_stride_y,
-                                             const long long part_stride_d, __nv_bfloat16 *__restrict__ Y, const int bh,
+                                             int *status, uint8_t *stage_tile, const __nv_bfloat16 *y_part,
+                                             const float *d_part, const int n_parts, const long long part_stride_y,
+                                             const long long part_stride_d, __nv_bfloat16 *Y, const int bh,
                                              const int N, const int C, const int lam, const int budget,
                                              const float scale_log2) {
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -360,8 +360,8 @@ template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 sa_merge_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                    const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ksel,
-                   const __grid_constant__ CUtensorMap tm_vsel, const __nv_bfloat16 *__restrict__ y_part,
-                   const float *__restrict__ d_part, int n_parts, __nv_bfloat16 *__restrict__ Y, int *status, int H, int Hkv,
+                   const __grid_constant__ CUtensorMap tm_vsel, const __nv_bfloat16 *y_part,
+                   const float *d_part, int n_parts, __nv_bfloat16 *Y, int *status, int H, int Hkv,
                    int N, int C, int lam, int budget, int sel_rows, int sel_identity, float scale_log2, int n_qblocks, int n_heads,
                    int set_heads) {
     grid_dep_wait();
@@ -656,8 +656,8 @@ template <int D>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
 sa_merge_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                      const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ksel,
-                     const __grid_constant__ CUtensorMap tm_vsel, const __nv_bfloat16 *__restrict__ y_part,
-                     const float *__restrict__ d_part, int n_parts, __nv_bfloat16 *__restrict__ Y, int *status, int H, int Hkv, int N,
+                     const __grid_constant__ CUtensorMap tm_vsel, const __nv_bfloat16 *y_part,
+                     const float *d_part, int n_parts, __nv_bfloat16 *Y, int *status, int H, int Hkv, int N,
                      int C, int lam, int budget, int sel_rows, int sel_identity, float scale_log2, int n_pairs, int n_heads,
                      int set_heads) {
     grid_dep_wait();
@@ -974,7 +974,7 @@ __device__ __forceinline__ float log2_of(float x) {
 template <int D, int C, bool kTinyEps>
 __global__ void __launch_bounds__(320, 1)
 score_select_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                       float *__restrict__ scores, int32_t *__restrict__ sel_idx, int *status, int H, int Hkv,
+                       float *scores, int32_t *sel_idx, int *status, int H, int Hkv,
                        int N, int lam, float scale_log2, float eps, int n_row_blocks, int n_tiles) {
     grid_dep_wait();
     grid_dep_launch();
@@ -1225,9 +1225,9 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
 // (a -1 entry, or a row of the padding, is zero).  One warp per row.
 template <int D>
 __global__ void __launch_bounds__(256)
-compact_kernel(const __nv_bfloat16 *__restrict__ K, const __nv_bfloat16 *__restrict__ V,
-               const int32_t *__restrict__ sel_idx, __nv_bfloat16 *__restrict__ Ksel,
-               __nv_bfloat16 *__restrict__ Vsel, int H, int Hkv, long long N, long long n_idx, long long sel_rows) {
+compact_kernel(const __nv_bfloat16 *K, const __nv_bfloat16 *V,
+               const int32_t *sel_idx, __nv_bfloat16 *Ksel,
+               __nv_bfloat16 *Vsel, int H, int Hkv, long long N, long long n_idx, long long sel_rows) {
     grid_dep_wait();
     grid_dep_launch();
     const int bh = blockIdx.y, b = bh / H, h = bh % H, kvh = h / (H / Hkv);
@@ -1366,8 +1366,8 @@ int tc_score_select(const still_params_t *p, long long N, const void *Q, const v
 }
 
 // N_LA / D_LA of the fp32-accumulating FMA kernels as one bf16 part: y = N_LA / D_LA, d = D_LA.
-__global__ void la_to_part_kernel(const float *__restrict__ N_LA, const float *__restrict__ D_LA, __nv_bfloat16 *__restrict__ y,
-                                  float *__restrict__ dp, long long rows, int d) {
+__global__ void la_to_part_kernel(const float *N_LA, const float *D_LA, __nv_bfloat16 *y,
+                                  float *dp, long long rows, int d) {
     grid_dep_wait();
     grid_dep_launch();
     const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;

@@ -76,3 +76,22 @@ def test_binding_refuses_cpu_tensors(lib):
         still.hybrid_attn_fwd(p, x, x, x, None, None)
     with pytest.raises(RuntimeError, match="no CPU path"):
         still.hybrid_attn_step(p, None, 0, 0, x[:, :, 0], x[:, :, 0], x[:, :, 0])
+
+
+def test_dependent_kernels_read_nothing_ahead_of_the_wait():
+    # Kernels are made resident while their predecessor runs (programmatic stream serialization): each has to wait before
+    # anything else, and no pointer parameter may promise (const restrict) that its memory does not change meanwhile.
+    csrc = still_build.CSRC
+    seen = 0
+    for name in sorted(os.listdir(csrc)):
+        text = re.sub(r"//[^\n]*", "", open(os.path.join(csrc, name)).read())
+        for m in re.finditer(r"__global__[^;{]*?\b(\w+_kernel)\(([^{]*)\)\s*\{", text):
+            if m.group(1) == "wait_timeout_selftest_kernel":   # launched by itself, in stream order
+                continue
+            seen += 1
+            assert "__restrict__" not in m.group(2), m.group(1)
+            ahead = text[m.end():].split("grid_dep_wait();")[0]
+            assert re.fullmatch(r"\s*(extern __shared__[^;]*;\s*)?", ahead), (m.group(1), ahead[:200])
+        # (device functions that kernels hand such pointers to are inlined into them)
+        assert "__restrict__" not in text, name
+    assert seen >= 19

@@ -341,3 +341,30 @@ def test_bounded_device_wait_runs_out_and_is_reported():
     ws = torch.empty(still.workspace_bytes(r["p"], w.N), dtype=torch.uint8, device="cuda")
     still.hybrid_attn_fwd(r["p"], r["Q"], r["K"], r["V"], r["Wq"], r["Wk"], workspace=ws)
     assert still.device_status(ws) == (0, 0)
+
+
+def test_prefills_back_to_back_on_one_workspace():
+    # Calls enqueued without waiting: the kernels of a call are resident while the call before, or the kernel that fills
+    # its inputs, still runs, and all use the same input, output and workspace buffers.  Every output has to be the one of
+    # the call made by itself.
+    for dtype, d, C, k, budget in [("bf16", 128, 64, 16, 0), ("bf16", 64, 128, 32, 64), ("fp32", 64, 32, 8, 0), ("bf16", 64, 32, 8, 0)]:
+        w = _small("t", dtype, 1, 4, 2, d, C * 9 + 5, C, k)
+        p = U.params_of(w, max_salient=budget)
+        ins = [(*synth.make_qkv(w.with_(seed=s), "cuda"), synth.make_gate(w.with_(seed=s), "cuda"), *synth.make_npmap_weights(w.with_(seed=s), "cuda"))
+               for s in range(4)]
+        call = lambda x, **kw: still.hybrid_attn_fwd(p, *x[:3], *x[4:], G=x[3], **kw)  # noqa: E731
+        alone = []
+        for x in ins:
+            alone.append(call(x))
+            torch.cuda.synchronize()
+        buf, out = [torch.empty_like(t) for t in ins[0]], [torch.empty_like(t) for t in alone[0]]
+        ws = torch.empty(still.workspace_bytes(p, w.N), dtype=torch.uint8, device="cuda")
+        got = []
+        torch.cuda.synchronize()
+        for x in ins * 2:
+            for dst, src in zip(buf, x):
+                dst.copy_(src)
+            got.append([t.clone() for t in call(buf, Y=out[0], scores=out[1], sel_idx=out[2], workspace=ws)])
+        torch.cuda.synchronize()
+        for want, have in zip(alone * 2, got):
+            assert all(torch.equal(a, b) for a, b in zip(want, have)), (dtype, d, C)
