@@ -308,7 +308,7 @@ gather_kernel(const __nv_bfloat16 *K, const __nv_bfloat16 *V, const __nv_bfloat1
     constexpr int kVec = D / 8, kPhiVec = 2 * DF / 8;       // 16-byte pieces of a row
     constexpr int kPer = 32 / kVec, kPhiPer = 32 / kPhiVec;  // rows that a warp moves at a time
     __shared__ int pos[128];
-    __shared__ float sums[8 * kPhiPer][2 * DF];
+    __shared__ __align__(16) float sums[8 * kPhiPer][2 * DF];   // (written 16 bytes at a time)
     const int bh = blockIdx.y, b = bh / H, h = bh % H, c = blockIdx.x, Tn = gridDim.x - 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long src0 = ((long long)b * Hkv + h / (H / Hkv)) * N, dst0 = (long long)bh * sel_rows + (long long)c * lam;

@@ -71,7 +71,7 @@ step_route_kernel(T *kc, T *vc, float *score,
                   float *z, T *Wk, T *bk, int32_t *hdr, StateKey key,
                   int H, int Hkv, long long cap, long long kvr, int d, int df, int C, int lam, long long cr, int window,
                   int w_in_smem) {
-    extern __shared__ float smem[];
+    extern __shared__ __align__(16) float smem[];
     grid_dep_wait();
     grid_dep_launch();
     {   // the step's first kernel when there is a chunk to route: the header against the call

@@ -95,3 +95,14 @@ def test_dependent_kernels_read_nothing_ahead_of_the_wait():
         # (device functions that kernels hand such pointers to are inlined into them)
         assert "__restrict__" not in text, name
     assert seen >= 19
+
+
+def test_shared_arrays_that_vectors_are_stored_to_are_aligned():
+    # A shared array is only as aligned as its element type unless it says more: those without an explicit alignment are
+    # the ones that are accessed element by element (or, smem_raw, aligned by hand).
+    plain = set()
+    for name in os.listdir(still_build.CSRC):
+        for m in re.finditer(r"__shared__ ([^;]*);", open(os.path.join(still_build.CSRC, name)).read()):
+            if "__align__" not in m.group(1):
+                plain.add(re.findall(r"(\w+)(?:\[[^\]]*\])*$", m.group(1))[0])
+    assert plain == {"pos", "part", "smem_raw", "bar", "abort_word"}
