@@ -298,7 +298,7 @@ npmap_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
 // and the rows read: 32 heads x 131072 tokens, d = 128, 32 of 128 selected, with phi_sel: three kernels that each
 // gathered for themselves (and one that summed a row after the other) took 1023 us.
 template <int D, int DF>
-__global__ void __launch_bounds__(256)
+__global__ void __launch_bounds__(256, D == 128 ? 4 : 5)
 gather_kernel(const __nv_bfloat16 *K, const __nv_bfloat16 *V, const __nv_bfloat16 *phiK,
               const int32_t *sel_idx, __nv_bfloat16 *Ksel, __nv_bfloat16 *Vsel,
               __nv_bfloat16 *phi_sel, float *selsum, int H, int Hkv, long long N, int lam,
@@ -307,7 +307,6 @@ gather_kernel(const __nv_bfloat16 *K, const __nv_bfloat16 *V, const __nv_bfloat1
     grid_dep_launch();
     constexpr int kVec = D / 8, kPhiVec = 2 * DF / 8;       // 16-byte pieces of a row
     constexpr int kPer = 32 / kVec, kPhiPer = 32 / kPhiVec;  // rows that a warp moves at a time
-    __shared__ int pos[128];
     __shared__ __align__(16) float sums[8 * kPhiPer][2 * DF];   // (written 16 bytes at a time)
     const int bh = blockIdx.y, b = bh / H, h = bh % H, c = blockIdx.x, Tn = gridDim.x - 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -323,49 +322,33 @@ gather_kernel(const __nv_bfloat16 *K, const __nv_bfloat16 *V, const __nv_bfloat1
             for (long long i = threadIdx.x; i < n_phi; i += 256) reinterpret_cast<uint4 *>(phi_sel + dst0 * (2 * DF))[i] = zero;
         return;
     }
-    for (int i = threadIdx.x; i < lam; i += 256) pos[i] = sel_idx[((long long)bh * Tn + c) * lam + i];
-    __syncthreads();
-    // K and V rows: K in even, V in odd groups of lanes
-    {
-        const int piece = lane % kVec, which = (lane / kVec) & 1;
-        const __nv_bfloat16 *src = which ? V : K;
-        __nv_bfloat16 *dst = which ? Vsel : Ksel;
-        if (dst != nullptr) {
-            constexpr int kStep = 8 * (kPer / 2);
-            for (int r0 = warp * (kPer / 2) + lane / (2 * kVec); r0 < lam; r0 += 4 * kStep) {
-                uint4 v[4];   // (four rows requested before the first is stored)
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const int r = r0 + i * kStep, p = r < lam ? pos[r] : -1;
-                    v[i] = make_uint4(0, 0, 0, 0);
-                    if (p >= 0) v[i] = reinterpret_cast<const uint4 *>(src + (src0 + p) * D)[piece];
-                }
-#pragma unroll
-                for (int i = 0; i < 4; ++i)
-                    if (r0 + i * kStep < lam) reinterpret_cast<uint4 *>(dst + (dst0 + r0 + i * kStep) * D)[piece] = v[i];
-            }
-        }
-    }
-    // phi(K) rows and their sum
-    if (phi_sel == nullptr && c >= n_routed) return;
-    const int piece = lane % kPhiVec;
+    const int32_t *pos = sel_idx + ((long long)bh * Tn + c) * lam;
+    // K and V rows: K in even, V in odd groups of lanes.  A thread requests kBatch of these and of the phi(K) pieces before it
+    // stores any: a store waits for its load, and the loads behind it would wait with it.
+    const int piece = lane % kVec, which = (lane / kVec) & 1, piece_phi = lane % kPhiVec;
+    const __nv_bfloat16 *src = which ? V : K;
+    __nv_bfloat16 *dst = which ? Vsel : Ksel;
+    const bool with_phi = phi_sel != nullptr || c < n_routed;
+    constexpr int kStep = 8 * (kPer / 2), kPhiStep = 8 * kPhiPer, kBatch = D == 128 ? 4 : 2;
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.f;
-    constexpr int kPhiStep = 8 * kPhiPer;
-    for (int r0 = warp * kPhiPer + lane / kPhiVec; r0 < lam; r0 += 4 * kPhiStep) {
-        uint4 v[4];
+    int r0 = dst ? warp * (kPer / 2) + lane / (2 * kVec) : lam, q0 = with_phi ? warp * kPhiPer + lane / kPhiVec : lam;
+    for (; r0 < lam || q0 < lam; r0 += kBatch * kStep, q0 += kBatch * kPhiStep) {
+        uint4 v[kBatch], f[kBatch];
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = r0 + i * kPhiStep, p = r < lam ? pos[r] : -1;
-            v[i] = make_uint4(0, 0, 0, 0);
-            if (p >= 0) v[i] = reinterpret_cast<const uint4 *>(phiK + (src0 + p) * (2 * DF))[piece];
+        for (int i = 0; i < kBatch; ++i) {
+            const int r = r0 + i * kStep, q = q0 + i * kPhiStep, p = r < lam ? pos[r] : -1, pq = q < lam ? pos[q] : -1;
+            v[i] = f[i] = make_uint4(0, 0, 0, 0);
+            if (p >= 0) v[i] = reinterpret_cast<const uint4 *>(src + (src0 + p) * D)[piece];
+            if (pq >= 0) f[i] = reinterpret_cast<const uint4 *>(phiK + (src0 + pq) * (2 * DF))[piece_phi];
         }
 #pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            const int r = r0 + i * kPhiStep;
-            if (phi_sel && r < lam) reinterpret_cast<uint4 *>(phi_sel + (dst0 + r) * (2 * DF))[piece] = v[i];
-            const uint32_t w[4] = {v[i].x, v[i].y, v[i].z, v[i].w};
+        for (int i = 0; i < kBatch; ++i) {
+            const int r = r0 + i * kStep, q = q0 + i * kPhiStep;
+            if (r < lam) reinterpret_cast<uint4 *>(dst + (dst0 + r) * D)[piece] = v[i];
+            if (phi_sel && q < lam) reinterpret_cast<uint4 *>(phi_sel + (dst0 + q) * (2 * DF))[piece_phi] = f[i];
+            const uint32_t w[4] = {f[i].x, f[i].y, f[i].z, f[i].w};
 #pragma unroll
             for (int e = 0; e < 4; ++e) {
                 acc[2 * e] += __uint_as_float(w[e] << 16);
@@ -374,7 +357,7 @@ gather_kernel(const __nv_bfloat16 *K, const __nv_bfloat16 *V, const __nv_bfloat1
         }
     }
     if (c >= n_routed) return;
-    float *mine = &sums[warp * kPhiPer + lane / kPhiVec][piece * 8];
+    float *mine = &sums[warp * kPhiPer + lane / kPhiVec][piece_phi * 8];
     *reinterpret_cast<float4 *>(mine) = make_float4(acc[0], acc[1], acc[2], acc[3]);
     *reinterpret_cast<float4 *>(mine + 4) = make_float4(acc[4], acc[5], acc[6], acc[7]);
     __syncthreads();
@@ -401,26 +384,38 @@ z_scan_kernel(const float *csum, const float *selsum, float *zpre, float *z_out,
     const float *cs = csum + ((long long)b * Hkv + h / (H / Hkv)) * Tn * NF + f;
     const float *ss = selsum + (long long)bh * n_routed * NF + f;
     float *z = zpre + (long long)bh * n_routed * NF + f;
-    auto delta = [&](int c) -> float {
-        float d = 0.f;
-        if (!all_selected) d = cs[(long long)c * NF] - ss[(long long)c * NF];
-        if (window > 0 && c >= window) d += all_selected ? cs[(long long)(c - window) * NF] : ss[(long long)(c - window) * NF];
-        return d;
+    const float *leaving = all_selected ? cs : ss;
+    constexpr int kAhead = 8;   // chunks whose sums are requested together
+    auto deltas = [&](int c, int c1, float (&d)[kAhead]) {   // of chunks c .. (zero from c1 on)
+        float a[kAhead], b[kAhead], w[kAhead];
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) {
+            a[i] = b[i] = w[i] = 0.f;
+            const bool in = c + i < c1;
+            if (in && !all_selected) {
+                a[i] = cs[(long long)(c + i) * NF];
+                b[i] = ss[(long long)(c + i) * NF];
+            }
+            if (in && window > 0 && c + i >= window) w[i] = leaving[(long long)(c + i - window) * NF];
+        }
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) d[i] = (a[i] - b[i]) + w[i];
     };
     const int warps = blockDim.x >> 5, per = (n_routed + warps - 1) / warps, c0 = warp * per, c1 = min(c0 + per, n_routed);
-    float acc = 0.f;
-#pragma unroll 8
-    for (int c = c0; c < c1; ++c) acc += delta(c);
+    float acc = 0.f, d[kAhead];
+    for (int c = c0; c < c1; c += kAhead) {
+        deltas(c, c1, d);
+#pragma unroll
+        for (int i = 0; i < kAhead; ++i) acc += d[i];
+    }
     part[warp][lane] = acc;
     __syncthreads();
     acc = 0.f;
     for (int w = 0; w < warp; ++w) acc += part[w][lane];
-    for (int c = c0; c < c1; c += 8) {   // (eight chunks requested before the first is stored)
-        float d[8];
+    for (int c = c0; c < c1; c += kAhead) {
+        deltas(c, c1, d);
 #pragma unroll
-        for (int i = 0; i < 8; ++i) d[i] = c + i < c1 ? delta(c + i) : 0.f;
-#pragma unroll
-        for (int i = 0; i < 8; ++i) {
+        for (int i = 0; i < kAhead; ++i) {
             acc += d[i];
             if (c + i < c1) z[(long long)(c + i) * NF] = acc;
         }

@@ -301,15 +301,20 @@ __device__ __forceinline__ void softmax_role(const StreamT &st, const int x, con
             for (int hh = 0; hh < 2; ++hh) {   // halves of D / 2 columns
                 if (with_la) {
                     __syncwarp();
+                    uint4 v[kPieces];   // (all requested before the first is stored: one round trip to memory, not kPieces)
 #pragma unroll
                     for (int it = 0; it < kPieces; ++it) {
                         const int id = it * 32 + lane, row = id / kPieces, c = id % kPieces;
                         const int part = c / kPartPieces, cc = c % kPartPieces;
-                        uint4 v = make_uint4(0, 0, 0, 0);
+                        v[it] = make_uint4(0, 0, 0, 0);
                         if (t0 + row < N && part < n_parts)
-                            v = *reinterpret_cast<const uint4 *>(y_part + part * part_stride_y + ((long long)bh * N + t0 + row) * D +
-                                                                 hh * (D / 2) + cc * 8);
-                        *reinterpret_cast<uint4 *>(stg + row * kRowBytes + ((c ^ (row & (kPieces - 1))) << 4)) = v;
+                            v[it] = *reinterpret_cast<const uint4 *>(y_part + part * part_stride_y + ((long long)bh * N + t0 + row) * D +
+                                                                     hh * (D / 2) + cc * 8);
+                    }
+#pragma unroll
+                    for (int it = 0; it < kPieces; ++it) {
+                        const int id = it * 32 + lane, row = id / kPieces, c = id % kPieces;
+                        *reinterpret_cast<uint4 *>(stg + row * kRowBytes + ((c ^ (row & (kPieces - 1))) << 4)) = v[it];
                     }
                     __syncwarp();
                 }

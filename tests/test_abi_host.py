@@ -105,4 +105,4 @@ def test_shared_arrays_that_vectors_are_stored_to_are_aligned():
         for m in re.finditer(r"__shared__ ([^;]*);", open(os.path.join(still_build.CSRC, name)).read()):
             if "__align__" not in m.group(1):
                 plain.add(re.findall(r"(\w+)(?:\[[^\]]*\])*$", m.group(1))[0])
-    assert plain == {"pos", "part", "smem_raw", "bar", "abort_word"}
+    assert plain == {"part", "smem_raw", "bar", "abort_word"}
