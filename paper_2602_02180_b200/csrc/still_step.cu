@@ -19,6 +19,7 @@
 #include "still_tc.h"
 
 #include <algorithm>
+#include <type_traits>
 
 namespace still {
 
@@ -639,7 +640,7 @@ static_assert(step_main_smem<__nv_bfloat16, 128>() <= 232448 && step_main_smem<f
 // 1.27 ms; with one launch each for the append and score, the cache pass in equal splits per group and the merge with
 // its read-out it was 1.65 ms; B = 16, 16K, a quarter kept: 143 us, before 305 us), at one sequence the latency of a
 // block's chain (one user, 2K prefix: 10.5 us a step with the merge, of which the host needs 10; before 71 us).
-template <typename T, int D, int NT>
+template <typename T, int D, int NH>
 __global__ void __launch_bounds__(kStepThreads, 1)
 step_main_kernel(const __grid_constant__ StepArgs<T> a) {
     extern __shared__ __align__(128) uint8_t step_smem[];
@@ -668,7 +669,7 @@ step_main_kernel(const __grid_constant__ StepArgs<T> a) {
         const uint32_t *mask = a.sel_mask + bh * v.n_chunk_cap * (v.C / 32);
         float *part = a.part + (bh * kRecords + slot) * (D + 2), *logits = a.part + (bh * kRecords + kLogitRecord) * (D + 2);
         if constexpr (sizeof(T) == 2)
-            attend_segment<D, NT>(v, kh, vh, a.k + row * D, a.v + row * D, a.q + bh * D, mask, tile_lo, tile_hi, step_smem, part,
+            attend_segment<D, NH>(v, kh, vh, a.k + row * D, a.v + row * D, a.q + bh * D, mask, tile_lo, tile_hi, step_smem, part,
                                   logits, kRecords * (D + 2));
         else
             attend_segment_f32<D>(v, kh, vh, a.k + row * D, a.v + row * D, a.q + bh * D, mask, tile_lo, tile_hi,
@@ -797,12 +798,12 @@ static int launch_route(const still_params_t *p, const StepArgs<T> &a, int32_t *
     return STILL_OK;
 }
 
-template <typename T, int D, int NT>
+template <typename T, int D, int NH>
 static int launch_main(const StepArgs<T> &a, unsigned grid, cudaStream_t st, int *launches) {
     constexpr int kSmem = step_main_smem<T, D>();
-    STILL_CUDA(ensure_dynamic_smem((const void *)step_main_kernel<T, D, NT>, kSmem));
+    STILL_CUDA(ensure_dynamic_smem((const void *)step_main_kernel<T, D, NH>, kSmem));
     profile_mark_begin(st);
-    STILL_CUDA(launch_dependent(step_main_kernel<T, D, NT>, dim3(grid), dim3(kStepThreads), kSmem, st, a));
+    STILL_CUDA(launch_dependent(step_main_kernel<T, D, NH>, dim3(grid), dim3(kStepThreads), kSmem, st, a));
     profile_mark_end(st);
     STILL_CUDA(launch_dependent(step_merge_kernel<T, D>, dim3(a.H, a.B), dim3(D + 64), 0, st, a));
     *launches += 2;
@@ -883,18 +884,16 @@ static int step_typed(const still_params_t *p, char *state, const still_state_la
     // The fewer warps share a read-out, the more run side by side and the longer one takes.
     a.item_warps = a.n_items <= n_sm ? kStepWarps : a.n_items <= n_sm * (kStepWarps / 2) ? 2 : 1;
     const unsigned grid = (unsigned)(apart ? used + a.n_items : n_sm);
-    if (d == 64) {
+    auto launch = [&](auto head_dim) -> int {
+        constexpr int D = decltype(head_dim)::value;
         if constexpr (kBf16) {
-            return rep <= 8 ? launch_main<T, 64, 1>(a, grid, st, launches) : launch_main<T, 64, 2>(a, grid, st, launches);
+            if (rep <= 4) return launch_main<T, D, 4>(a, grid, st, launches);
+            return rep <= 8 ? launch_main<T, D, 8>(a, grid, st, launches) : launch_main<T, D, 16>(a, grid, st, launches);
         } else {
-            return launch_main<T, 64, 1>(a, grid, st, launches);
+            return launch_main<T, D, kUnitHeadsF32>(a, grid, st, launches);
         }
-    }
-    if constexpr (kBf16) {
-        return rep <= 8 ? launch_main<T, 128, 1>(a, grid, st, launches) : launch_main<T, 128, 2>(a, grid, st, launches);
-    } else {
-        return launch_main<T, 128, 1>(a, grid, st, launches);
-    }
+    };
+    return d == 64 ? launch(std::integral_constant<int, 64>{}) : launch(std::integral_constant<int, 128>{});
 }
 
 int step_launch(const still_params_t *p, char *state, const still_state_layout_t *L, long long t_pos,

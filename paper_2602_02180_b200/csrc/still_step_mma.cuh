@@ -12,9 +12,12 @@
 // selection (the sel_mask words of the decode state) contains it; for the two-chunk local region, every position up
 // to the new token.  A row is read from memory only if some head of the group selected it; with topk = chunk that is
 // every row.  A tile without a new maximum (most of them, past the first few) costs one vote instead of a reduction and
-// a rescaling of O.  (Raising the maximum only when it is exceeded by 2^8, as the prefill does, gained nothing here and
-// cost precision: the largest weight is then no longer exactly one when it is rounded to bf16, and the output's error
-// against 64 bits grew from 2.0e-3 to 2.3e-3.)
+// a rescaling of O.
+//
+// The weights P enter the second product as two bf16 parts, the upper 8 bits of the significand and the rest: rounded
+// to bf16 once they would be the largest error of a step, and one that depends on how the history is cut (a weight is
+// exact where it is its partial's maximum).  A group of up to four heads costs nothing for it: the four columns that it
+// leaves idle carry the second part.
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -64,6 +67,13 @@ __device__ __forceinline__ uint32_t pack2_bf16(float lo, float hi) {
     asm("cvt.rn.bf16x2.f32 %0, %1, %2;" : "=r"(r) : "f"(hi), "f"(lo));
     return r;
 }
+// Two weights (>= 0) as bf16 parts: their upper halves, and what these leave off.  The rest of a weight that is not
+// zero is never zero, so that an infinite value stays infinite under both parts.
+__device__ __forceinline__ uint32_t weight_hi2(float a, float b) { return __byte_perm(__float_as_uint(a), __float_as_uint(b), 0x7632); }
+__device__ __forceinline__ uint32_t weight_lo2(float a, float b) {
+    const float ra = a - __uint_as_float(__float_as_uint(a) & 0xffff0000u), rb = b - __uint_as_float(__float_as_uint(b) & 0xffff0000u);
+    return pack2_bf16(fmaxf(ra, a * 0x1p-24f), fmaxf(rb, b * 0x1p-24f));
+}
 
 // Geometry of a decode step's cache pass (see step_main_kernel).
 struct AttendView {
@@ -93,16 +103,20 @@ struct AttendPlan {
 // token's (position t is read from the call's inputs, not from the row that another block is writing); qh: the
 // group's queries; mask: sel_mask of the group's first head.  Leaves one record per head (maximum in natural-log
 // units, sum, numerator [D]) at part + head * part_stride, and the new token's logits against the last C positions,
-// oldest first, at logits + head * part_stride.  NT: tiles of 8 heads.
-template <int D, int NT>
+// oldest first, at logits + head * part_stride.  NH: room for heads, 4, 8 or 16 (tiles of 8 columns; with 4 the second
+// half of the tile repeats the heads and takes the second part of their weights).
+template <int D, int NH>
 __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_bfloat16 *kh, const __nv_bfloat16 *vh,
                                                const __nv_bfloat16 *k_new, const __nv_bfloat16 *v_new,
                                                const __nv_bfloat16 *qh, const uint32_t *mask, int tile_lo, int tile_hi,
                                                uint8_t *smem, float *part, float *logits, long long part_stride) {
     using P = AttendPlan<D>;
+    constexpr int NT = NH == 16 ? 2 : 1;
+    constexpr bool kRepeat = NH == 4;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int g = lane >> 2, tig = lane & 3;
     uint8_t *my = smem + warp * P::kWarp;
+    auto head_of = [](int column) { return kRepeat ? column & 3 : column; };
 
     // Q^T as B fragments: columns are heads (head >= rep: zero)
     uint32_t qb[NT][D / 16][2];
@@ -110,7 +124,7 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
     for (int nt = 0; nt < NT; ++nt)
 #pragma unroll
         for (int ks = 0; ks < D / 16; ++ks) {
-            const int h = nt * 8 + g, col = ks * 16 + tig * 2;
+            const int h = head_of(nt * 8 + g), col = ks * 16 + tig * 2;
             qb[nt][ks][0] = h < v.rep ? *reinterpret_cast<const uint32_t *>(qh + h * D + col) : 0u;
             qb[nt][ks][1] = h < v.rep ? *reinterpret_cast<const uint32_t *>(qh + h * D + col + 8) : 0u;
         }
@@ -231,7 +245,7 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
         for (int nt = 0; nt < NT; ++nt) {
 #pragma unroll
             for (int hh = 0; hh < 2; ++hh) {
-                const uint32_t vis = __shfl_sync(0xffffffffu, word, nt * 8 + tig * 2 + hh);
+                const uint32_t vis = __shfl_sync(0xffffffffu, word, head_of(nt * 8 + tig * 2 + hh));
                 s[nt][hh] = (vis >> g) & 1u ? s[nt][hh] * v.scale_log2 : -INFINITY;
                 s[nt][2 + hh] = (vis >> (g + 8)) & 1u ? s[nt][2 + hh] * v.scale_log2 : -INFINITY;
                 grow |= fmaxf(s[nt][hh], s[nt][2 + hh]) > m_run[nt][hh];
@@ -261,7 +275,7 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
                 }
             }
         }
-        uint32_t pb[NT][2];   // P^T as B fragments
+        uint32_t pb[NT][2], pr[NT][2];   // P^T as B fragments: first part (repeated heads: the column's part), second part
 #pragma unroll
         for (int nt = 0; nt < NT; ++nt) {
             float pv[4];
@@ -272,8 +286,14 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
             }
             l_run[nt][0] += pv[0] + pv[2];
             l_run[nt][1] += pv[1] + pv[3];
-            pb[nt][0] = movmatrix_trans(pack2_bf16(pv[0], pv[1]));
-            pb[nt][1] = movmatrix_trans(pack2_bf16(pv[2], pv[3]));
+            const uint32_t h0 = weight_hi2(pv[0], pv[1]), h1 = weight_hi2(pv[2], pv[3]);
+            const uint32_t l0 = weight_lo2(pv[0], pv[1]), l1 = weight_lo2(pv[2], pv[3]);
+            pb[nt][0] = movmatrix_trans(kRepeat && tig >= 2 ? l0 : h0);
+            pb[nt][1] = movmatrix_trans(kRepeat && tig >= 2 ? l1 : h1);
+            if constexpr (!kRepeat) {
+                pr[nt][0] = movmatrix_trans(l0);
+                pr[nt][1] = movmatrix_trans(l1);
+            }
         }
         // O^T += V^T P^T: rows are value columns
 #pragma unroll
@@ -282,7 +302,10 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
             const int row = (lane >> 4) * 8 + (lane & 7), piece = dt * 2 + ((lane >> 3) & 1);
             ldmatrix_x4_trans(a, vs + row * P::kRow + ((piece ^ (row & 7)) << 4));
 #pragma unroll
-            for (int nt = 0; nt < NT; ++nt) mma_16816(o[nt][dt], a, pb[nt][0], pb[nt][1]);
+            for (int nt = 0; nt < NT; ++nt) {
+                mma_16816(o[nt][dt], a, pb[nt][0], pb[nt][1]);
+                if constexpr (!kRepeat) mma_16816(o[nt][dt], a, pr[nt][0], pr[nt][1]);
+            }
         }
         __syncwarp();   // the stage may be overwritten
         if (++stage == P::kStages) stage = 0;
@@ -294,6 +317,12 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
     float *mg = reinterpret_cast<float *>(smem);
     constexpr int kStride = D + 2;
     const int rep = v.rep;
+    if constexpr (kRepeat) {   // both parts of a head's sums
+#pragma unroll
+        for (int dt = 0; dt < D / 16; ++dt)
+#pragma unroll
+            for (int e = 0; e < 4; ++e) o[0][dt][e] += __shfl_xor_sync(0xffffffffu, o[0][dt][e], 2);
+    }
 #pragma unroll
     for (int nt = 0; nt < NT; ++nt) {
 #pragma unroll

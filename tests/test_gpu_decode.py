@@ -253,3 +253,47 @@ def test_state_full_and_mismatch():
     still.hybrid_attn_fwd(p, Q, K, V, Wq, Wk, state=state2, state_max_tokens=128)
     still.hybrid_attn_step(p, state2, 128, 64, q, k, v, Wq, Wk, y=y)
     assert still.device_status(state2) == (0, 0) and torch.isfinite(y.float()).all()
+
+
+def _dense_steps(B, Hkv, rep, d, n0, steps, edit=None):
+    """Decode with every token selected (softmax attention alone, bf16) beside float64: (y, exact), [B, H, steps, d]."""
+    H, C, N = Hkv * rep, 64, n0 + steps
+    w = synth.Workload("t", B, H, Hkv, d, N, C, C, "bf16", "iid", 55)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    if edit is not None:
+        edit(Q, K, V)
+    p = U.params_of(w)
+    state = torch.zeros(still.state_bytes(p, N), dtype=torch.uint8, device="cuda")
+    cut = lambda x: x[:, :, :n0].contiguous()  # noqa: E731
+    still.hybrid_attn_fwd(p, cut(Q), cut(K), cut(V), state=state, state_max_tokens=N, want_y=False)
+    y = torch.stack([still.hybrid_attn_step(p, state, N, t, *(x[:, :, t].contiguous() for x in (Q, K, V))) for t in range(n0, N)], 2)
+    K, V = (x.double().repeat_interleave(rep, 1) for x in (K, V))
+    seen = torch.arange(N, device="cuda") <= torch.arange(n0, N, device="cuda")[:, None]
+    e = (Q[:, :, n0:].double() @ K.transpose(2, 3) * w.sm_scale).masked_fill(~seen, -torch.inf).softmax(-1)
+    return y, e @ V, e
+
+
+@pytest.mark.parametrize("d,rep", [(64, 1), (128, 3), (128, 4), (64, 5), (128, 8), (128, 9), (64, 16), (128, 16)])
+def test_decode_outputs_are_float64_rounded_once(d, rep):
+    # Weights rounded to bf16 (2^-9) would change about a quarter of the outputs' last bits; kept to 2^-17 they change an
+    # output of the size of its terms in 2 x 2^-17 / 2^-8 = 0.4 % of the cases, the smaller ones (cancellation) in more.
+    y, exact, _ = _dense_steps(2, 2, rep, d, 700, 20)
+    differ = (y != exact.to(torch.bfloat16)).double().mean().item()
+    assert differ <= 0.02, differ
+
+
+@pytest.mark.parametrize("rep", [4, 8])
+def test_decode_with_an_infinite_value(rep):
+    # an infinite value under a weight that bf16 holds exactly (the maximum's, 1) and under others
+    def edit(Q, K, V):
+        V[:, :, 100, 3] = torch.inf
+        V[:, :, 650, 7] = -torch.inf
+        K[:, :, 650] = 0
+        K[:, :, 650, 0] = 60.0
+        Q[:, :, :, 0] = 4.0
+
+    y, exact, _ = _dense_steps(1, 2, rep, 64, 700, 5, edit)
+    assert torch.equal(y[..., 3], exact[..., 3].to(torch.bfloat16)) and bool((y[..., 3] == torch.inf).all())
+    assert bool((y[..., 7] == -torch.inf).all())
+    rest = [c for c in range(64) if c not in (3, 7)]
+    assert bool(torch.isfinite(y[..., rest]).all())
