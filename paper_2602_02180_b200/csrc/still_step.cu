@@ -184,8 +184,9 @@ step_route_kernel(T *kc, T *vc, float *score,
 
 // The same for bf16 states on the tensor cores; grid (H, B), 256 threads.  f = K W_k and S += phi(K)^T V are bf16
 // products with fp32 accumulation (the features are bf16 in the prefill as well); f is kept in fp32 and a row of f is
-// replaced in place by the row's features, zero for a token that stays out.  The state is read straight into the
-// accumulators and written back from them.  What bounds it is the read and write of S (128 KB a head each way) and, for
+// replaced in place by the row's features, zero for a token that stays out.  The chunk's sum is formed by itself and
+// then added to the state in fp32: carried through the accumulators, the state would take their rounding (not to
+// nearest) sixteen tokens at a time for a whole generation.  What bounds it is the read and write of S (128 KB a head each way) and, for
 // few heads, the chain of loads, two products and the row-wise softmax.  (A quarter kept, C = 64, d = 128: 512 heads 70 us,
 // 1024 heads with a chunk leaving the cache as well 235 us, 32 heads 25 us; on the FMA pipes 416, 1168 and 95 us.)
 template <int D>
@@ -356,12 +357,13 @@ step_route_mma_kernel(__nv_bfloat16 *kc, __nv_bfloat16 *vc, float *score, int32_
         // S += phi^T V: 16 features x 64 value columns at a time
         for (int u = warp; u < (dp / 16) * (D / 64); u += 8) {
             const int mt = u / (D / 64), e0 = u % (D / 64) * 64;
-            float acc[8][4];
+            float acc[8][4] = {};
+            float2 lo[8], hi[8];   // the state, requested ahead of the products
             float *Sr = S + (bh * dp + mt * 16 + g) * D + e0 + tig * 2;
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt) {
-                const float2 lo = *reinterpret_cast<const float2 *>(Sr + nt * 8), hi = *reinterpret_cast<const float2 *>(Sr + 8 * D + nt * 8);
-                acc[nt][0] = lo.x; acc[nt][1] = lo.y; acc[nt][2] = hi.x; acc[nt][3] = hi.y;
+                lo[nt] = *reinterpret_cast<const float2 *>(Sr + nt * 8);
+                hi[nt] = *reinterpret_cast<const float2 *>(Sr + 8 * D + nt * 8);
             }
             for (int k16 = 0; k16 < C / 16; ++k16) {
                 uint32_t af[4], bf[4];
@@ -378,8 +380,8 @@ step_route_mma_kernel(__nv_bfloat16 *kc, __nv_bfloat16 *vc, float *score, int32_
             }
 #pragma unroll
             for (int nt = 0; nt < 8; ++nt) {
-                *reinterpret_cast<float2 *>(Sr + nt * 8) = make_float2(acc[nt][0], acc[nt][1]);
-                *reinterpret_cast<float2 *>(Sr + 8 * D + nt * 8) = make_float2(acc[nt][2], acc[nt][3]);
+                *reinterpret_cast<float2 *>(Sr + nt * 8) = make_float2(lo[nt].x + acc[nt][0], lo[nt].y + acc[nt][1]);
+                *reinterpret_cast<float2 *>(Sr + 8 * D + nt * 8) = make_float2(hi[nt].x + acc[nt][2], hi[nt].y + acc[nt][3]);
             }
         }
         for (int f = tid; f < dp; f += 256) {

@@ -297,3 +297,34 @@ def test_decode_with_an_infinite_value(rep):
     assert bool((y[..., 7] == -torch.inf).all())
     rest = [c for c in range(64) if c not in (3, 7)]
     assert bool(torch.isfinite(y[..., rest]).all())
+
+
+@pytest.mark.parametrize("d", [64, 128])
+def test_state_after_many_routings_is_rounded_to_nearest(d):
+    # With zero maps every feature is 1 / d_f, exactly: S is then a sum of values that fp32 cannot hold exactly (large and
+    # small positive ones), and its error is what the additions leave.  A routing adds a chunk's sum (error below two units
+    # of the chunk's sum per product of sixteen tokens) to S, rounded to nearest: half a unit of S each.
+    C, n0, routings = 64, 130, 24
+    N = n0 + C * routings
+    p = still.StillParams(1, 2, 1, d, C, 0, torch.bfloat16)
+    g = torch.Generator(device="cuda").manual_seed(3)
+    V = 1 + torch.rand(1, 1, N, d, generator=g, device="cuda")
+    V[:, :, 1::2] *= 2.0 ** -12
+    V = V.to(torch.bfloat16)
+    Q, K = (torch.randn(1, h, N, d, generator=g, device="cuda").to(torch.bfloat16) for h in (2, 1))
+    W = torch.zeros(2, d, d, dtype=torch.bfloat16, device="cuda")
+    lay = still.state_layout(p, N)
+    state = torch.zeros(lay["total"], dtype=torch.uint8, device="cuda")
+    cut = lambda x: x[:, :, :n0].contiguous()  # noqa: E731
+    still.hybrid_attn_fwd(p, cut(Q), cut(K), cut(V), W, W[:1], state=state, state_max_tokens=N, want_y=False)
+    for t in range(n0, N):
+        still.hybrid_attn_step(p, state, N, t, *(x[:, :, t].contiguous() for x in (Q, K, V)), W, W[:1])
+    done = ((N - 1) // C - 1) * C                  # tokens that have left the local region
+    S = state[lay["S"]: lay["S"] + 2 * 2 * d * d * 4].view(torch.float32).view(2, 2 * d, d).double()
+    z = state[lay["z"]: lay["z"] + 2 * 2 * d * 4].view(torch.float32)
+    assert bool((z == done / d).all())
+    want = V[0, 0, :done].double().sum(0) / d      # every feature's row
+    ulp = 2.0 ** (torch.floor(torch.log2(want)) - 23)
+    chunk_ulp = 2.0 ** -23 * 2.0 ** torch.ceil(torch.log2(want / (done // C)))
+    bound = routings * (0.5 * ulp + 4 * 2 * chunk_ulp)
+    assert bool(((S - want).abs() <= bound).all()), ((S - want).abs() / ulp).max().item()
