@@ -25,6 +25,13 @@ __device__ __forceinline__ float ld_f(const __nv_bfloat16 *p) { return __bfloat1
 __device__ __forceinline__ void st_f(float *p, float v) { *p = v; }
 __device__ __forceinline__ void st_f(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
 
+// Maximum that is NaN when an argument is (fmaxf drops it).  A row's running maximum is formed with it, so that a NaN logit
+// makes the row NaN also where it is the only one seen so far: with the maximum still at -inf it would count for nothing.
+__device__ __forceinline__ float max_nan(float a, float b) {
+    float r;
+    asm("max.NaN.f32 %0, %1, %2;" : "=f"(r) : "f"(a), "f"(b));
+    return r;
+}
 __device__ __forceinline__ float warp_max(float v) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v = fmaxf(v, __shfl_xor_sync(0xffffffffu, v, o));

@@ -611,11 +611,11 @@ sa_merge_kernel(const T *Q, const T *K, const T *V,
 #pragma unroll
             for (int j = 0; j < NK; ++j) {
                 s[j] = kp[j] >= 0 && kp[j] <= t ? (acc[r][j].x + acc[r][j].y) * scale : -INFINITY;
-                mx = fmaxf(mx, s[j]);
+                mx = max_nan(mx, s[j]);
             }
 #pragma unroll
-            for (int w = 8; w > 0; w >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, w));
-            const float mnew = fmaxf(m[r], mx);
+            for (int w = 8; w > 0; w >>= 1) mx = max_nan(mx, __shfl_xor_sync(0xffffffffu, mx, w));
+            const float mnew = max_nan(m[r], mx);
             const float alpha = mnew == -INFINITY ? 1.f : expf(m[r] - mnew);
             m[r] = mnew;
             float sum = 0.f;

@@ -114,10 +114,10 @@ __device__ __forceinline__ void attend_segment_f32(const AttendView &v, const fl
         const int slot = v.first_pos + j * kKeys + key - (v.t - (v.C - 1));   // of this lane's key in the new token's window
         if (slot >= 0 && slot < v.C && hd < v.rep) logits[hd * part_stride + slot] = dot;
         float mx = s;
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
-        mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
-        const float mn = fmaxf(m_run, mx);
+        mx = max_nan(mx, __shfl_xor_sync(0xffffffffu, mx, 1));
+        mx = max_nan(mx, __shfl_xor_sync(0xffffffffu, mx, 2));
+        mx = max_nan(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
+        const float mn = max_nan(m_run, mx);
         const float alpha = (mn == -INFINITY) ? 1.f : expf(m_run - mn);
         const float p = (on && mn != -INFINITY) ? expf(s - mn) : 0.f;
         m_run = mn;
@@ -173,7 +173,7 @@ __device__ __forceinline__ void attend_segment_f32(const AttendView &v, const fl
 #pragma unroll
         for (int w = 0; w < kStepWarps; ++w) {
             mw[w] = mg[(w * NH + h) * kStride];
-            M = fmaxf(M, mw[w]);
+            M = max_nan(M, mw[w]);
         }
         float acc = 0.f;
         if (col == 0) {

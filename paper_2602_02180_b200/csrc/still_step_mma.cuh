@@ -248,7 +248,7 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
                 const uint32_t vis = __shfl_sync(0xffffffffu, word, head_of(nt * 8 + tig * 2 + hh));
                 s[nt][hh] = (vis >> g) & 1u ? s[nt][hh] * v.scale_log2 : -INFINITY;
                 s[nt][2 + hh] = (vis >> (g + 8)) & 1u ? s[nt][2 + hh] * v.scale_log2 : -INFINITY;
-                grow |= fmaxf(s[nt][hh], s[nt][2 + hh]) > m_run[nt][hh];
+                grow |= !(max_nan(s[nt][hh], s[nt][2 + hh]) <= m_run[nt][hh]);
             }
         }
         if (__any_sync(0xffffffffu, grow)) {
@@ -257,11 +257,11 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
                 float alpha[2];
 #pragma unroll
                 for (int hh = 0; hh < 2; ++hh) {
-                    float mx = fmaxf(s[nt][hh], s[nt][2 + hh]);
-                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
-                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
-                    mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
-                    const float mn = fmaxf(m_run[nt][hh], mx);
+                    float mx = max_nan(s[nt][hh], s[nt][2 + hh]);
+                    mx = max_nan(mx, __shfl_xor_sync(0xffffffffu, mx, 4));
+                    mx = max_nan(mx, __shfl_xor_sync(0xffffffffu, mx, 8));
+                    mx = max_nan(mx, __shfl_xor_sync(0xffffffffu, mx, 16));
+                    const float mn = max_nan(m_run[nt][hh], mx);
                     alpha[hh] = (mn == -INFINITY) ? 1.f : ex2_approx(m_run[nt][hh] - mn);
                     m_run[nt][hh] = mn;
                     l_run[nt][hh] *= alpha[hh];
@@ -353,7 +353,7 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
 #pragma unroll
         for (int w = 0; w < kStepWarps; ++w) {
             mw[w] = mg[(w * rep + h) * kStride];
-            M = fmaxf(M, mw[w]);
+            M = max_nan(M, mw[w]);
         }
         float acc = 0.f;
         if (col == 0) {

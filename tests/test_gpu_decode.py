@@ -328,3 +328,20 @@ def test_state_after_many_routings_is_rounded_to_nearest(d):
     chunk_ulp = 2.0 ** -23 * 2.0 ** torch.ceil(torch.log2(want / (done // C)))
     bound = routings * (0.5 * ulp + 4 * 2 * chunk_ulp)
     assert bool(((S - want).abs() <= bound).all()), ((S - want).abs() / ulp).max().item()
+
+
+@pytest.mark.parametrize("dtype,n_nan", [("bf16", 16), ("fp32", 8)])
+def test_decode_nan_logits_make_the_output_nan(dtype, n_nan):
+    # a run of NaN keys as long as a tile of the pass: the tile's maximum is then no number, and the first of a warp's
+    # tiles has no earlier one; the outputs of the group are NaN, those of the other group are not
+    B, Hkv, rep, d, n0, steps, C = 1, 2, 4, 64, 700, 3, 64
+    w = synth.Workload("t", B, Hkv * rep, Hkv, d, n0 + steps, C, C, dtype, "iid", 56)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    K[:, 0, :n_nan] = torch.nan
+    p = U.params_of(w)
+    state = torch.zeros(still.state_bytes(p, w.N), dtype=torch.uint8, device="cuda")
+    cut = lambda x: x[:, :, :n0].contiguous()  # noqa: E731
+    still.hybrid_attn_fwd(p, cut(Q), cut(K), cut(V), state=state, state_max_tokens=w.N, want_y=False)
+    for t in range(n0, w.N):
+        y = still.hybrid_attn_step(p, state, w.N, t, *(x[:, :, t].contiguous() for x in (Q, K, V)))
+        assert bool(torch.isnan(y[:, :rep]).all()) and bool(torch.isfinite(y[:, rep:]).all())

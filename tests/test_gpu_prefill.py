@@ -368,3 +368,12 @@ def test_prefills_back_to_back_on_one_workspace():
         torch.cuda.synchronize()
         for want, have in zip(alone * 2, got):
             assert all(torch.equal(a, b) for a, b in zip(want, have)), (dtype, d, C)
+
+
+def test_fp32_nan_logits_make_the_output_nan():
+    # the first tile of keys (64 at d = 64) NaN for one KV head: every row of its query heads sees a NaN
+    w = _small("t", "fp32", 1, 4, 2, 64, 300, 64, 64)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    K[:, 0, :64] = torch.nan
+    Y = still.hybrid_attn_fwd(U.params_of(w), Q, K, V)[0]
+    assert bool(torch.isnan(Y[:, :2]).all()) and bool(torch.isfinite(Y[:, 2:]).all())
