@@ -60,11 +60,17 @@ static inline bool la_active(const still_params_t *p) { return p->topk < p->chun
 struct FwdPlan {
     size_t status, scores, sel_idx, phiQ, phiK, csum, zpre, segs, nla, dla, ypart, dpart, ksel, vsel, phiKsel, total;
     long long T, sel_rows;  // chunks; rows of the compacted salient K/V per head
-    int n_seg;              // segments of the fp32 scan
+    int n_seg, seg_chunks;  // segments of the fp32 scan, chunks of each (the last one takes the rest)
+    bool own_sums;          // their sums have a place of their own (segs); else they lie in the segments' rows of nla, dla
     bool la, tc, tc_la;
 };
 
-static FwdPlan plan_fwd(const still_params_t *p, long long N) {
+// Segments of the fp32 scan: two waves of two blocks per SM.  (These sizes are planned without a device; the kernels run
+// on any count of SMs.)
+constexpr int kScanBlocks = 4 * 148;
+
+// The workspace never takes more than `limit` bytes for the sake of speed alone (the sums of the scan's segments).
+static FwdPlan plan_fwd(const still_params_t *p, long long N, size_t limit = SIZE_MAX) {
     FwdPlan w{};
     const long long T = (N + p->chunk - 1) / p->chunk;
     const size_t BH = (size_t)p->B * p->H, BHkv = (size_t)p->B * p->Hkv;
@@ -112,14 +118,30 @@ static FwdPlan plan_fwd(const still_params_t *p, long long N) {
         }
     }
     if (w.la && !w.tc_la) {
-        // Segments of the fp32 scan, enough for two waves of two blocks per SM.  Their sums are extra workspace: a call
-        // that fits the library's static workspace with fewer segments takes fewer.
+        // Wanted: enough segments to fill the GPU.  Their sums (S, z of every head and segment) get a place of their own
+        // where the call's room allows; a call that fits the static workspace without them is kept within it.  Otherwise
+        // a sum lies in the rows of N_LA and D_LA that its segment writes later, which takes segments of at least 2 d_f
+        // tokens, the last one included.  Of the two the one with the shorter segments is taken.  (At 16 heads, d = 64,
+        // C = 64 the sums lie in the rows between 1011 and 1160 tokens, where the static workspace is full.)
         const long long units = (long long)BH * (p->d / 64);
-        w.n_seg = (int)std::max<long long>(1, std::min<long long>((592 + units - 1) / units, T - 2));
+        const long long want = std::max<long long>(1, std::min<long long>((kScanBlocks + units - 1) / units, T - 2));
         const size_t per_seg = BH * dp * (size_t)(p->d + 1) * 4;
-        if (off <= STILL_STATIC_WORKSPACE_BYTES)
-            while (w.n_seg > 1 && off + align_up(w.n_seg * per_seg, 1024) > STILL_STATIC_WORKSPACE_BYTES) --w.n_seg;
-        if (w.n_seg > 1) w.segs = take(w.n_seg * per_seg);
+        if (off <= STILL_STATIC_WORKSPACE_BYTES) limit = std::min(limit, (size_t)STILL_STATIC_WORKSPACE_BYTES);
+        long long n = want;
+        while (n > 1 && off + align_up(n * per_seg, 1024) > limit) --n;
+        w.seg_chunks = (int)((T + n - 1) / n);
+        w.n_seg = (int)((T + w.seg_chunks - 1) / w.seg_chunks);
+        w.own_sums = w.n_seg > 1;
+        if (n < want) {
+            const long long chunks = std::max<long long>((T + want - 1) / want, ((long long)dp + p->chunk - 1) / p->chunk);
+            const long long segs = std::max<long long>(1, N / (chunks * p->chunk)), each = T / segs;   // (each >= chunks)
+            if (T - (segs - 1) * each < w.seg_chunks) {   // (the last segment is the longest)
+                w.seg_chunks = (int)each;
+                w.n_seg = (int)segs;
+                w.own_sums = false;
+            }
+        }
+        if (w.own_sums) w.segs = take(w.n_seg * per_seg);
     }
     w.total = off;
     return w;
@@ -301,37 +323,38 @@ static int launch_npmap(const still_params_t *p, long long N, int heads, const T
 }
 
 template <typename T, int DP>
-static int launch_la_scan_t(const still_params_t *p, long long N, long long Tn, const T *phiQ, const T *phiK, const T *V,
-                            const T *G, const int32_t *sel, float *nla, float *dla, float *sums, int n_seg, float *S_out,
-                            float *z_out, cudaStream_t st) {
+static int launch_la_scan_t(const still_params_t *p, long long N, const FwdPlan &w, char *ws, const T *phiQ, const T *phiK, const T *V,
+                            const T *G, const int32_t *sel, float *nla, float *dla, float *S_out, float *z_out, cudaStream_t st) {
     const size_t smem = la_seg_smem(DP);
     STILL_CUDA(set_smem(la_seg_kernel<T, DP>, smem));
-    const int seg_chunks = (int)((Tn + n_seg - 1) / n_seg);
-    n_seg = (int)((Tn + seg_chunks - 1) / seg_chunks);
+    const int BH = p->B * p->H, d = p->d, n_seg = w.n_seg;
+    const long long rows = (long long)w.seg_chunks * p->chunk;
+    float *own = reinterpret_cast<float *>(ws + w.segs);
+    const SegSums sums = w.own_sums ? SegSums{own, own + (long long)n_seg * BH * DP * d, DP * d, (long long)BH * DP * d, DP, (long long)BH * DP}
+                                    : SegSums{nla, dla, N * d, rows * d, N, rows};
     auto pass = [&](int segments, int sum_only) -> int {
-        STILL_CUDA(launch_dependent(la_seg_kernel<T, DP>, dim3(p->B * p->H, segments, p->d / 64), dim3(256), smem, st, phiQ, phiK, V, G, sel,
-                                    nla, dla, sums, S_out, z_out, p->H, p->Hkv, N, p->d, p->chunk, p->topk, seg_chunks, n_seg, sum_only));
+        STILL_CUDA(launch_dependent(la_seg_kernel<T, DP>, dim3(BH, segments, d / 64), dim3(256), smem, st, phiQ, phiK, V, G, sel,
+                                    nla, dla, sums, S_out, z_out, p->H, p->Hkv, N, d, p->chunk, p->topk, w.seg_chunks, n_seg, sum_only));
         ++g_launches;
         return STILL_OK;
     };
     if (n_seg > 1) {
         int rc = pass(n_seg - 1, 1);
         if (rc != STILL_OK) return rc;
-        const long long n4 = (long long)p->B * p->H * DP * (p->d + 1) / 4;
-        STILL_CUDA(launch_dependent(la_prefix_kernel, dim3((unsigned)((n4 + 255) / 256)), dim3(256), 0, st, sums, n4, n_seg));
+        const long long n = (long long)BH * (DP * d / 4 + DP);
+        STILL_CUDA(launch_dependent(la_prefix_kernel, dim3((unsigned)((n + 255) / 256)), dim3(256), 0, st, sums, DP * d / 4, DP, n, n_seg));
         ++g_launches;
     }
     return pass(n_seg, 0);
 }
 
 template <typename T>
-static int launch_la_scan(const still_params_t *p, long long N, long long Tn, const T *phiQ,
-                          const T *phiK, const T *V, const T *G, const int32_t *sel, float *nla,
-                          float *dla, float *sums, int n_seg, float *S_out, float *z_out, cudaStream_t st) {
+static int launch_la_scan(const still_params_t *p, long long N, const FwdPlan &w, char *ws, const T *phiQ, const T *phiK, const T *V,
+                          const T *G, const int32_t *sel, float *nla, float *dla, float *S_out, float *z_out, cudaStream_t st) {
     switch (p->d_f) {
-        case 32: return launch_la_scan_t<T, 64>(p, N, Tn, phiQ, phiK, V, G, sel, nla, dla, sums, n_seg, S_out, z_out, st);
-        case 64: return launch_la_scan_t<T, 128>(p, N, Tn, phiQ, phiK, V, G, sel, nla, dla, sums, n_seg, S_out, z_out, st);
-        default: return launch_la_scan_t<T, 256>(p, N, Tn, phiQ, phiK, V, G, sel, nla, dla, sums, n_seg, S_out, z_out, st);
+        case 32: return launch_la_scan_t<T, 64>(p, N, w, ws, phiQ, phiK, V, G, sel, nla, dla, S_out, z_out, st);
+        case 64: return launch_la_scan_t<T, 128>(p, N, w, ws, phiQ, phiK, V, G, sel, nla, dla, S_out, z_out, st);
+        default: return launch_la_scan_t<T, 256>(p, N, w, ws, phiQ, phiK, V, G, sel, nla, dla, S_out, z_out, st);
     }
 }
 
@@ -402,9 +425,7 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
             dla = reinterpret_cast<float *>(ws + w.dla);
             if ((rc = launch_npmap<T>(p, N, p->H, Q, Wq, bq, phiQ, st)) != STILL_OK) return rc;
             if ((rc = launch_npmap<T>(p, N, p->Hkv, K, Wk, bk, phiK, st)) != STILL_OK) return rc;
-            if ((rc = launch_la_scan<T>(p, N, w.T, phiQ, phiK, V, G, sel, nla, dla, reinterpret_cast<float *>(ws + w.segs), w.n_seg, S_out,
-                                        z_out, st)) != STILL_OK)
-                return rc;
+            if ((rc = launch_la_scan<T>(p, N, w, ws, phiQ, phiK, V, G, sel, nla, dla, S_out, z_out, st)) != STILL_OK) return rc;
             if (w.tc && Y) {   // the tensor-core attention kernel takes the linear branch as bf16 parts
                 ypart = ws + w.ypart;
                 dpart = reinterpret_cast<float *>(ws + w.dpart);
@@ -462,6 +483,56 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
 
 static bool misaligned(const void *ptr) { return (reinterpret_cast<uintptr_t>(ptr) & 15u) != 0; }
 
+// still_hybrid_attn_fwd with a plan that takes at most `limit` bytes of workspace, if the call can do with them.
+static int run_fwd(const still_params_t *p, int64_t N, const void *Q, const void *K, const void *V, const void *G, const void *Wq,
+                   const void *bq, const void *Wk, const void *bk, void *Y, float *scores, int32_t *sel_idx, void *state_out,
+                   int64_t state_max_tokens, void *workspace, size_t workspace_bytes, size_t limit, void *cuda_stream) {
+    g_launches = 0;
+    int rc = validate(p);
+    if (rc != STILL_OK) return rc;
+    if (N < 0) return STILL_ERR_INVALID_ARG;
+    if (N > (int64_t)1 << 30) return STILL_ERR_UNSUPPORTED;  // positions are int32
+    if (N == 0) {
+        // An empty prefill only initialises the decode state (no tokens, zero S and z).
+        if (!state_out) return STILL_OK;
+        if (misaligned(state_out)) return STILL_ERR_INVALID_ARG;
+        still_state_layout_t L{};
+        if ((rc = plan_state(p, state_max_tokens, &L)) != STILL_OK) return rc;
+        cudaStream_t st0 = reinterpret_cast<cudaStream_t>(cuda_stream);
+        char *s0 = reinterpret_cast<char *>(state_out);
+        STILL_CUDA(cudaMemsetAsync(s0 + L.S, 0, L.scratch - L.S, st0));
+        write_header_kernel<<<1, 32, 0, st0>>>(reinterpret_cast<int32_t *>(s0 + L.header), *p, L.capacity, 0);
+        ++g_launches;
+        STILL_CUDA(cudaGetLastError());
+        return STILL_OK;
+    }
+    if (!Q || !K || !V || !workspace) return STILL_ERR_INVALID_ARG;
+    if (!Y && !state_out && !scores && !sel_idx) return STILL_ERR_INVALID_ARG;
+    const void *ptrs[] = {Q, K, V, G, Wq, bq, Wk, bk, Y, scores, sel_idx, state_out, workspace};
+    for (const void *ptr : ptrs)
+        if (ptr && misaligned(ptr)) return STILL_ERR_INVALID_ARG;
+    FwdPlan w = plan_fwd(p, N, limit);
+    if (workspace_bytes < w.total) return STILL_ERR_WORKSPACE_TOO_SMALL;
+    if (w.la && (!Wq || !Wk)) return STILL_ERR_INVALID_ARG;   // the linear branch needs both maps
+    if (state_out) {
+        still_state_layout_t L{};
+        if ((rc = plan_state(p, state_max_tokens, &L)) != STILL_OK) return rc;
+        if (N > L.capacity) return STILL_ERR_STATE_FULL;
+    }
+    cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
+    char *ws = reinterpret_cast<char *>(workspace);
+    char *state = reinterpret_cast<char *>(state_out);
+    if (p->dtype == STILL_DTYPE_FP32)
+        return fwd_typed<float>(p, N, (const float *)Q, (const float *)K, (const float *)V,
+                                (const float *)G, (const float *)Wq, (const float *)bq,
+                                (const float *)Wk, (const float *)bk, (float *)Y, scores, sel_idx,
+                                state, state_max_tokens, ws, w, st);
+    using bf = __nv_bfloat16;
+    return fwd_typed<bf>(p, N, (const bf *)Q, (const bf *)K, (const bf *)V, (const bf *)G,
+                         (const bf *)Wq, (const bf *)bq, (const bf *)Wk, (const bf *)bk, (bf *)Y,
+                         scores, sel_idx, state, state_max_tokens, ws, w, st);
+}
+
 }  // namespace still
 
 using namespace still;
@@ -491,50 +562,8 @@ int still_hybrid_attn_fwd(const still_params_t *p, int64_t N, const void *Q, con
                           const void *Wk, const void *bk, void *Y, float *scores, int32_t *sel_idx,
                           void *state_out, int64_t state_max_tokens, void *workspace,
                           size_t workspace_bytes, void *cuda_stream) {
-    g_launches = 0;
-    int rc = validate(p);
-    if (rc != STILL_OK) return rc;
-    if (N < 0) return STILL_ERR_INVALID_ARG;
-    if (N > (int64_t)1 << 30) return STILL_ERR_UNSUPPORTED;  // positions are int32
-    if (N == 0) {
-        // An empty prefill only initialises the decode state (no tokens, zero S and z).
-        if (!state_out) return STILL_OK;
-        if (misaligned(state_out)) return STILL_ERR_INVALID_ARG;
-        still_state_layout_t L{};
-        if ((rc = plan_state(p, state_max_tokens, &L)) != STILL_OK) return rc;
-        cudaStream_t st0 = reinterpret_cast<cudaStream_t>(cuda_stream);
-        char *s0 = reinterpret_cast<char *>(state_out);
-        STILL_CUDA(cudaMemsetAsync(s0 + L.S, 0, L.scratch - L.S, st0));
-        write_header_kernel<<<1, 32, 0, st0>>>(reinterpret_cast<int32_t *>(s0 + L.header), *p, L.capacity, 0);
-        ++g_launches;
-        STILL_CUDA(cudaGetLastError());
-        return STILL_OK;
-    }
-    if (!Q || !K || !V || !workspace) return STILL_ERR_INVALID_ARG;
-    if (!Y && !state_out && !scores && !sel_idx) return STILL_ERR_INVALID_ARG;
-    const void *ptrs[] = {Q, K, V, G, Wq, bq, Wk, bk, Y, scores, sel_idx, state_out, workspace};
-    for (const void *ptr : ptrs)
-        if (ptr && misaligned(ptr)) return STILL_ERR_INVALID_ARG;
-    FwdPlan w = plan_fwd(p, N);
-    if (workspace_bytes < w.total) return STILL_ERR_WORKSPACE_TOO_SMALL;
-    if (w.la && (!Wq || !Wk)) return STILL_ERR_INVALID_ARG;   // the linear branch needs both maps
-    if (state_out) {
-        still_state_layout_t L{};
-        if ((rc = plan_state(p, state_max_tokens, &L)) != STILL_OK) return rc;
-        if (N > L.capacity) return STILL_ERR_STATE_FULL;
-    }
-    cudaStream_t st = reinterpret_cast<cudaStream_t>(cuda_stream);
-    char *ws = reinterpret_cast<char *>(workspace);
-    char *state = reinterpret_cast<char *>(state_out);
-    if (p->dtype == STILL_DTYPE_FP32)
-        return fwd_typed<float>(p, N, (const float *)Q, (const float *)K, (const float *)V,
-                                (const float *)G, (const float *)Wq, (const float *)bq,
-                                (const float *)Wk, (const float *)bk, (float *)Y, scores, sel_idx,
-                                state, state_max_tokens, ws, w, st);
-    using bf = __nv_bfloat16;
-    return fwd_typed<bf>(p, N, (const bf *)Q, (const bf *)K, (const bf *)V, (const bf *)G,
-                         (const bf *)Wq, (const bf *)bq, (const bf *)Wk, (const bf *)bk, (bf *)Y,
-                         scores, sel_idx, state, state_max_tokens, ws, w, st);
+    return run_fwd(p, N, Q, K, V, G, Wq, bq, Wk, bk, Y, scores, sel_idx, state_out, state_max_tokens, workspace, workspace_bytes,
+                   SIZE_MAX, cuda_stream);
 }
 
 int still_hybrid_attn_step(const still_params_t *p, void *state, int64_t state_max_tokens,
@@ -665,9 +694,11 @@ int still_hybrid_attn_fwd_host(const still_params_t *p, int64_t N, const void *h
     sub.B = 1;
     sub.Hkv = g;
     sub.H = g * rep;
-    // a second workspace for the alternate compute stream, if the arena's workspace holds two of a part's size
-    const size_t ws_part = align_up(plan_fwd(&sub, N).total, 1024);
-    const bool two_streams = n_parts > 1 && 2 * ws_part <= ws_bytes;
+    // a second workspace for the alternate compute stream, if the arena's workspace holds two of the least that a part needs;
+    // a part then has half of it (planned by itself, a part may want more than the whole call has: its scan has fewer heads
+    // to fill the GPU with and takes more segments)
+    const bool two_streams = n_parts > 1 && 2 * plan_fwd(&sub, N, 0).total <= ws_bytes;
+    const size_t ws_part = two_streams ? ws_bytes / 2 / 1024 * 1024 : ws_bytes;
     const size_t q_part = (size_t)g * rep * N * p->d * es, kv_part = (size_t)g * N * p->d * es;
     const size_t sc_part = (size_t)g * rep * N * 4, si_part = (size_t)g * rep * T * std::max(p->topk, 1) * 4;
     const char *cQ = static_cast<const char *>(hQ), *cK = static_cast<const char *>(hK), *cV = static_cast<const char *>(hV);
@@ -685,16 +716,12 @@ int still_hybrid_attn_fwd_host(const still_params_t *p, int64_t N, const void *h
         const bool alt = two_streams && (i & 1);
         cudaStream_t cs = alt ? s_alt : st;
         char *ws_i = alt ? ws + ws_part : ws;
-        const size_t ws_i_bytes = two_streams ? ws_part : ws_bytes;
         if (cudaStreamWaitEvent(cs, ev_in[i], 0) != cudaSuccess) { rc = STILL_ERR_CUDA; break; }
-        rc = still_hybrid_attn_fwd(&sub, N, dQ + i * q_part, dK + i * kv_part, dV + i * kv_part,
-                                   hG ? dG + i * q_part : nullptr,
-                                   hWq ? dWq + (size_t)kv0 * rep * p->d * p->d_f * es : nullptr,
-                                   hbq ? dbq + (size_t)kv0 * rep * p->d_f * es : nullptr,
-                                   hWk ? dWk + (size_t)kv0 * p->d * p->d_f * es : nullptr,
-                                   hbk ? dbk + (size_t)kv0 * p->d_f * es : nullptr, dY + i * q_part,
-                                   reinterpret_cast<float *>(dsc + i * sc_part), reinterpret_cast<int32_t *>(dsi + i * si_part),
-                                   nullptr, 0, ws_i, ws_i_bytes, cs);
+        rc = run_fwd(&sub, N, dQ + i * q_part, dK + i * kv_part, dV + i * kv_part, hG ? dG + i * q_part : nullptr,
+                     hWq ? dWq + (size_t)kv0 * rep * p->d * p->d_f * es : nullptr, hbq ? dbq + (size_t)kv0 * rep * p->d_f * es : nullptr,
+                     hWk ? dWk + (size_t)kv0 * p->d * p->d_f * es : nullptr, hbk ? dbk + (size_t)kv0 * p->d_f * es : nullptr,
+                     dY + i * q_part, reinterpret_cast<float *>(dsc + i * sc_part), reinterpret_cast<int32_t *>(dsi + i * si_part),
+                     nullptr, 0, ws_i, ws_part, ws_part, cs);
         if (rc != STILL_OK) break;
         cudaError_t e = cudaEventRecord(ev_done[i], cs);
         if (e == cudaSuccess) e = cudaStreamWaitEvent(s_out, ev_done[i], 0);

@@ -289,6 +289,8 @@ npmap_kernel(const T *X, const T *W, const T *bias,
 //   sum_only = 1: what segment blockIdx.y folds, into sums (blockIdx.y < n_seg - 1)
 //   sum_only = 0: the scan of a segment, from sums made exclusive prefixes by
 //                 la_prefix_kernel
+// The sums may lie in the segment's own rows of N_LA and D_LA (SegSums): a block takes
+// its columns of them into registers before it writes any of its rows.
 // grid (B*H, segments, d / 64), 256 threads: thread (tf, te) owns DP / 16 features x
 // four of the block's 64 value columns of S in registers; for the read-out S passes
 // through shared memory and a thread owns four rows x four columns of N_LA.  The same
@@ -296,12 +298,16 @@ npmap_kernel(const T *X, const T *W, const T *bias,
 // chunks by one block per 32 value columns.
 // Final S, z go to the decode state when asked.
 // ---------------------------------------------------------------------------
+struct SegSums {   // of segment seg of head bh: S [DP][d] at S + bh S_bh + seg S_seg, z [DP] at z + bh z_bh + seg z_seg
+    float *S, *z;
+    long long S_bh, S_seg, z_bh, z_seg;
+};
 inline size_t la_seg_smem(int dp) { return ((size_t)64 * dp + 64 * 64 + (size_t)dp * 64 + dp) * 4 + 64 * 4 + 16; }
 template <typename T, int DP>
 __global__ void __launch_bounds__(256)
 la_seg_kernel(const T *phiQ, const T *phiK, const T *V,
               const T *G, const int32_t *sel_idx, float *N_LA,
-              float *D_LA, float *sums, float *S_out,
+              float *D_LA, SegSums sums, float *S_out,
               float *z_out, int H, int Hkv, long long N, int d, int C, int lam, int seg_chunks,
               int n_seg, int sum_only) {
     grid_dep_wait();
@@ -320,7 +326,7 @@ la_seg_kernel(const T *phiQ, const T *phiK, const T *V,
     const T *pq = phiQ + (long long)bh * N * DP;
     const T *pk = phiK + ((long long)b * Hkv + kv) * N * DP;
     const T *vh = V + ((long long)b * Hkv + kv) * N * d;
-    float *mine = sums + ((long long)seg * gridDim.x + bh) * DP * (d + 1);   // [DP][d], then z [DP]
+    float *mine_S = sums.S + bh * sums.S_bh + seg * sums.S_seg, *mine_z = sums.z + bh * sums.z_bh + seg * sums.z_seg;
     float2 S[FPT / 2][4];   // features tf * FPT + 2 i, + 1; columns e0 + 4 te + e
 #pragma unroll
     for (int i = 0; i < FPT / 2; ++i)
@@ -330,17 +336,19 @@ la_seg_kernel(const T *phiQ, const T *phiK, const T *V,
     if (!sum_only && seg > 0) {
 #pragma unroll
         for (int i = 0; i < FPT / 2; ++i) {
-            const float4 a = ld4(mine + (long long)(tf * FPT + 2 * i) * d + e0 + 4 * te);
-            const float4 c = ld4(mine + (long long)(tf * FPT + 2 * i + 1) * d + e0 + 4 * te);
+            const float4 a = ld4(mine_S + (long long)(tf * FPT + 2 * i) * d + e0 + 4 * te);
+            const float4 c = ld4(mine_S + (long long)(tf * FPT + 2 * i + 1) * d + e0 + 4 * te);
             S[i][0] = make_float2(a.x, c.x);
             S[i][1] = make_float2(a.y, c.y);
             S[i][2] = make_float2(a.z, c.z);
             S[i][3] = make_float2(a.w, c.w);
         }
-        for (int i = tid; i < DP; i += 256) zs[i] = mine[(long long)DP * d + i];
+        if (blockIdx.z == 0)   // (z is used by these blocks alone, which also write the rows of D_LA that it may lie in)
+            for (int i = tid; i < DP; i += 256) zs[i] = mine_z[i];
+        __syncthreads();       // the sums are taken before any row is written
     }
     const int W = C < 64 ? C : 64;    // tokens of a sub-tile
-    const long long c1 = min((long long)(seg + 1) * seg_chunks, Tn);
+    const long long c1 = seg == n_seg - 1 ? Tn : (long long)(seg + 1) * seg_chunks;
     for (long long c = (long long)seg * seg_chunks; c < c1; ++c) {
         if (c >= 2) {
             const long long ub = (c - 2) * C;  // chunk c-2 is complete
@@ -471,7 +479,7 @@ la_seg_kernel(const T *phiQ, const T *phiK, const T *V,
     const bool last = !sum_only && seg == n_seg - 1;
     if (sum_only || (last && S_out)) {
         __syncthreads();
-        float *So = sum_only ? mine : S_out + (long long)bh * DP * d, *zo = sum_only ? mine + (long long)DP * d : z_out + (long long)bh * DP;
+        float *So = sum_only ? mine_S : S_out + (long long)bh * DP * d, *zo = sum_only ? mine_z : z_out + (long long)bh * DP;
 #pragma unroll
         for (int i = 0; i < FPT / 2; ++i) {
             st4(So + (long long)(tf * FPT + 2 * i) * d + e0 + 4 * te, make_float4(S[i][0].x, S[i][1].x, S[i][2].x, S[i][3].x));
@@ -481,25 +489,36 @@ la_seg_kernel(const T *phiQ, const T *phiK, const T *V,
             for (int i = tid; i < DP; i += 256) zo[i] = zs[i];
     }
 }
-// sums [n_seg][n]: segment s receives the sum of the segments before it (the last segment's own sum is not needed).
+// Segment s receives the sum of the segments before it (the last segment's own sum is not needed).  n_S = DP d / 4 and n_z =
+// DP threads per head.
+template <typename T>
+__device__ __forceinline__ void prefix_over_segments(T *p, long long stride, int n_seg) {
+    auto add = [](const T &a, const T &b) -> T {
+        if constexpr (sizeof(T) == 16) return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+        else return a + b;
+    };
+    T run{};
+    for (int s0 = 0; s0 < n_seg; s0 += 8) {   // eight independent loads in flight, then the running sum
+        T v[8];
+#pragma unroll
+        for (int s = 0; s < 8; ++s) v[s] = s0 + s < n_seg - 1 ? p[(s0 + s) * stride] : T{};
+#pragma unroll
+        for (int s = 0; s < 8; ++s) {
+            if (s0 + s < n_seg) p[(s0 + s) * stride] = run;
+            run = add(run, v[s]);
+        }
+    }
+}
 __global__ void __launch_bounds__(256)
-la_prefix_kernel(float *sums, long long n4, int n_seg) {
+la_prefix_kernel(SegSums sums, int n_S, int n_z, long long n_threads, int n_seg) {
     grid_dep_wait();
     grid_dep_launch();
     const long long i = (long long)blockIdx.x * 256 + threadIdx.x;
-    if (i >= n4) return;
-    float4 *p = reinterpret_cast<float4 *>(sums) + i;
-    float4 run = make_float4(0.f, 0.f, 0.f, 0.f);
-    for (int s0 = 0; s0 < n_seg; s0 += 8) {   // eight independent loads in flight, then the running sum
-        float4 v[8];
-#pragma unroll
-        for (int s = 0; s < 8; ++s) v[s] = s0 + s < n_seg - 1 ? p[(long long)(s0 + s) * n4] : make_float4(0.f, 0.f, 0.f, 0.f);
-#pragma unroll
-        for (int s = 0; s < 8; ++s) {
-            if (s0 + s < n_seg) p[(long long)(s0 + s) * n4] = run;
-            run = make_float4(run.x + v[s].x, run.y + v[s].y, run.z + v[s].z, run.w + v[s].w);
-        }
-    }
+    if (i >= n_threads) return;
+    const long long bh = i / (n_S + n_z);
+    const int r = (int)(i - bh * (n_S + n_z));
+    if (r < n_S) prefix_over_segments(reinterpret_cast<float4 *>(sums.S + bh * sums.S_bh) + r, sums.S_seg / 4, n_seg);
+    else prefix_over_segments(sums.z + bh * sums.z_bh + (r - n_S), sums.z_seg, n_seg);
 }
 
 // ---------------------------------------------------------------------------

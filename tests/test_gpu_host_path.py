@@ -32,3 +32,28 @@ def test_host_buffers_match_device_buffers(B, H, Hkv, d, N, k):
         assert torch.equal(hsel, want_sel.cpu())
         assert torch.equal(hsc, want_sc.cpu())
         assert torch.equal(hY, want_Y.cpu())
+
+
+@pytest.mark.parametrize("dtype,H,Hkv,d,C,k,N", [
+    ("fp32", 16, 2, 64, 32, 8, 1200),    # each of two parts would plan more workspace than the whole call has
+    ("fp32", 4, 2, 128, 32, 8, 1408),
+    ("fp32", 4, 2, 128, 32, 8, 2016),
+    ("bf16", 32, 8, 128, 32, 16, 416),   # eight parts on two streams
+    ("fp32", 2, 2, 64, 64, 16, 130),     # a short one: a single segment
+])
+def test_host_buffers_on_the_fma_kernels(dtype, H, Hkv, d, C, k, N):
+    # The parts of a call have fewer heads than the call and cut the linear scan into more segments for it; what a part
+    # needs still has to fit its share of the arena that host_arena_bytes gives.  The segments differ from the whole
+    # call's, and with them the order of the fp32 sums of N_LA: a few units in the last place of Y.
+    w = synth.Workload("h", 1, H, Hkv, d, N, C, k, dtype, "iid", 78)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    Wq, Wk = synth.make_npmap_weights(w, "cuda")
+    p = U.params_of(w)
+    want_Y, want_sc, want_sel = still.hybrid_attn_fwd(p, Q, K, V, Wq, Wk)
+    pin = lambda t: t.cpu().pin_memory()  # noqa: E731
+    hsc = torch.empty(1, H, N, dtype=torch.float32).pin_memory()
+    hsel = torch.empty(1, H, -(-N // C), k, dtype=torch.int32).pin_memory()
+    hY = still.hybrid_attn_fwd_host(p, pin(Q), pin(K), pin(V), pin(Wq), pin(Wk), hscores=hsc, hsel_idx=hsel)
+    assert torch.equal(hsel, want_sel.cpu()) and torch.equal(hsc, want_sc.cpu())
+    err = (hY.float() - want_Y.cpu().float()).norm() / want_Y.cpu().float().norm()
+    assert err <= (1e-6 if dtype == "fp32" else 2e-3), err   # (bf16: one value in a few hundred rounds the other way)

@@ -377,3 +377,44 @@ def test_fp32_nan_logits_make_the_output_nan():
     K[:, 0, :64] = torch.nan
     Y = still.hybrid_attn_fwd(U.params_of(w), Q, K, V)[0]
     assert bool(torch.isnan(Y[:, :2]).all()) and bool(torch.isfinite(Y[:, 2:]).all())
+
+
+@pytest.mark.parametrize("H,Hkv,d,df,C,k,N", [
+    (16, 4, 64, 64, 64, 16, 1024),     # 14 segments wanted, room for three beside the workspace: eight in N_LA
+    (16, 4, 64, 64, 64, 16, 1150),     # no room at all
+    (16, 4, 64, 64, 64, 16, 1200),     # past the static workspace: a place of their own again
+    (8, 4, 128, 128, 64, 16, 1000),    # segments of four chunks (2 d_f = 256 tokens) and a longer last one
+    (32, 4, 64, 32, 128, 32, 640 + 127),   # segments of one chunk: the second one's rows are answered with zeros
+    (16, 4, 128, 64, 32, 8, 515),
+])
+def test_fp32_scan_segments_without_room_for_their_sums(H, Hkv, d, df, C, k, N):
+    # Below the 16 MiB of the static workspace the sums of the scan's segments have no place of their own; they then lie in
+    # rows of N_LA and D_LA.  Parity on every head, with the state, and no fall back to one serial pass.
+    w = _small("t", "fp32", 1, H, Hkv, d, N, C, k)
+    p = still.StillParams(1, H, Hkv, d, C, k, torch.float32, d_f=df, sm_scale=w.sm_scale)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    g = torch.Generator(device="cuda").manual_seed(12)
+    Wq, Wk = (torch.randn(n, d, df, generator=g, device="cuda") * 0.05 for n in (H, Hkv))
+    G = synth.make_gate(w, "cuda")
+    lay = still.state_layout(p, N)
+    state = torch.zeros(lay["total"], dtype=torch.uint8, device="cuda")
+    ws = torch.full((still.workspace_bytes(p, N) + 4096,), 255, dtype=torch.uint8, device="cuda")   # (NaN wherever nothing is written)
+    Y, scores, sel = still.hybrid_attn_fwd(p, Q, K, V, Wq, Wk, G=G, state=state, state_max_tokens=N, workspace=ws[:-4096])
+    assert still.last_launch_count() == 8      # score, two maps, sums, prefix, scan, attention, state
+    assert bool((ws[-4096:] == 255).all())
+    heads = [(0, h) for h in range(0, H, 3)]
+    U.check_selection(scores, sel, C, k, heads)
+    U.check_outputs(w, Q, K, V, Wq, Wk, Y, scores, sel, heads, G=G, tol=1e-5)
+    # S and z: phi(K)^T [V, 1] over the unselected tokens of the routed chunks, in float64
+    n = (-(-N // C) - 2) * C
+    S = state[lay["S"]: lay["S"] + H * 2 * df * d * 4].view(torch.float32).view(H, 2 * df, d)
+    z = state[lay["z"]: lay["z"] + H * 2 * df * 4].view(torch.float32).view(H, 2 * df)
+    for _, h in heads:
+        x, W = K[0, h // (H // Hkv), :n].double(), Wk[h // (H // Hkv)].double()
+        f = x @ W
+        u = f * (x.norm(dim=1, keepdim=True) / f.norm(dim=1, keepdim=True))
+        phi = torch.cat([u.softmax(1), (-u).softmax(1)], 1)
+        idx = sel[0, h].flatten().long()
+        phi[idx[(idx >= 0) & (idx < n)]] = 0
+        for got, want in ((S[h], phi.T @ V[0, h // (H // Hkv), :n].double()), (z[h], phi.sum(0))):
+            assert float((got - want).norm() / want.norm()) <= 2e-6   # (fp32 features and sums of up to 1100 terms)
