@@ -41,7 +41,9 @@ inline cudaError_t launch_dependent(void (*kernel)(Params...), dim3 grid, dim3 b
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, static_cast<Params>(args)...);
+    if (e != cudaSuccess) (void)cudaGetLastError();   // (the call returns it; left pending it would fail the next call as well)
+    return e;
 }
 
 // ---- timing of the dominant kernel (still_profile_enable / still_profile_collect) ----

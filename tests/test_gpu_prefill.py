@@ -418,3 +418,16 @@ def test_fp32_scan_segments_without_room_for_their_sums(H, Hkv, d, df, C, k, N):
         phi[idx[(idx >= 0) & (idx < n)]] = 0
         for got, want in ((S[h], phi.T @ V[0, h // (H // Hkv), :n].double()), (z[h], phi.sum(0))):
             assert float((got - want).norm() / want.norm()) <= 2e-6   # (fp32 features and sums of up to 1100 terms)
+
+
+def test_a_refused_launch_does_not_fail_the_next_call():
+    # 65536 KV heads exceed a grid dimension: the launch is refused on the host and the call says so.  The next call, which
+    # checks for launch errors itself, must not find that one.
+    many = still.StillParams(1, 65536, 65536, 64, 64, 16)
+    x, w = torch.zeros(1, 65536, 4, 64, dtype=torch.bfloat16, device="cuda"), torch.zeros(65536, 64, 64, dtype=torch.bfloat16, device="cuda")
+    with pytest.raises(still.StillError) as e:
+        still.hybrid_attn_fwd(many, x, x, x, w, w)
+    assert e.value.code == -5
+    del x, w
+    r = U.run_prefill(_small("t", "bf16", 1, 2, 1, 64, 200, 64, 16))
+    assert bool(torch.isfinite(r["Y"].float()).all())
