@@ -106,3 +106,30 @@ def test_shared_arrays_that_vectors_are_stored_to_are_aligned():
             if "__align__" not in m.group(1):
                 plain.add(re.findall(r"(\w+)(?:\[[^\]]*\])*$", m.group(1))[0])
     assert plain == {"part", "smem_raw", "bar", "abort_word"}
+
+
+def test_parameters_stay_a_plain_dataclass(lib):
+    # A call leaves nothing among the fields, c() hands out a struct of the caller's own, and every call sees the fields as
+    # they are, however they were set.
+    import copy
+    import dataclasses
+    import pickle
+
+    p = still.StillParams(2, 8, 2, 64, 64, 16, sm_scale=0.5)
+    n = still.workspace_bytes(p, 1000)
+    assert set(vars(p)) == {f.name for f in dataclasses.fields(p)}
+    assert still.StillParams(**vars(p)) == p and dataclasses.replace(p, topk=8).topk == 8
+    for q in (copy.copy(p), copy.deepcopy(p), pickle.loads(pickle.dumps(p))):
+        assert q == p and still.workspace_bytes(q, 1000) == n
+        q.B = 4
+        assert still.workspace_bytes(q, 1000) > n and still.workspace_bytes(p, 1000) == n
+    p.c().B = 0
+    assert still.workspace_bytes(p, 1000) == n and p.c().B == 2
+    vars(p)["B"] = 4
+    assert still.workspace_bytes(p, 1000) > n
+    p.sm_scale = 0.0
+    assert still.workspace_bytes(p, 1000) == 0
+    p.sm_scale = torch.tensor(0.0)          # a value that can change in place
+    assert still.workspace_bytes(p, 1000) == 0
+    p.sm_scale.fill_(0.5)
+    assert still.workspace_bytes(p, 1000) > n
