@@ -65,11 +65,10 @@ __device__ __forceinline__ int state_mismatch(const int32_t *words, const StateK
 // fp32 states; grid (H, B), 256 threads.  Routes chunk cr (complete, C tokens): top-k into sel_idx / sel_mask, the other tokens
 // into (S, z).  With a salient-cache budget of `window` chunks the selected tokens of chunk cr - window leave the
 // cache at the same moment and are folded into (S, z) as well.
-template <typename T>
 __global__ void __launch_bounds__(256)
-step_route_kernel(T *kc, T *vc, float *score,
+step_route_kernel(float *kc, float *vc, float *score,
                   int32_t *sel_idx, uint32_t *sel_mask, float *S,
-                  float *z, T *Wk, T *bk, int32_t *hdr, StateKey key,
+                  float *z, float *Wk, float *bk, int32_t *hdr, StateKey key,
                   int H, int Hkv, long long cap, long long kvr, int d, int df, int C, int lam, long long cr, int window,
                   int w_in_smem) {
     extern __shared__ __align__(16) float smem[];
@@ -89,7 +88,7 @@ step_route_kernel(T *kc, T *vc, float *score,
     float *xs = vs + C * d;           // [8][d]
     float *sc = xs + 8 * d;           // [C]
     int *flag = reinterpret_cast<int *>(sc + C);  // [C]
-    T *Ws = reinterpret_cast<T *>(flag + C);      // [d][df] the head's W_k (read once per row of the chunk otherwise)
+    float *Ws = reinterpret_cast<float *>(flag + C);  // [d][df] the head's W_k (read once per row of the chunk otherwise)
     const int h = blockIdx.x, b = blockIdx.y, kv = h / (H / Hkv);
     const long long bh = (long long)b * H + h;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -105,10 +104,10 @@ step_route_kernel(T *kc, T *vc, float *score,
         for (int j = 0; j < 32; ++j) bits |= (flag[threadIdx.x * 32 + j] ? 1u : 0u) << j;
         sel_mask[(bh * (cap / C) + cr) * (C / 32) + threadIdx.x] = bits;
     }
-    const T *Wh = Wk + (long long)kv * d * df;
-    const T *bh_ = bk ? bk + (long long)kv * df : nullptr;
+    const float *Wh = Wk + (long long)kv * d * df;
+    const float *bh_ = bk ? bk + (long long)kv * df : nullptr;
     float *Sh = S + bh * dp * d;
-    const T *Wuse = Wh;   // W_k from shared memory when it fits beside the chunk's tiles, else from global memory
+    const float *Wuse = Wh;   // W_k from shared memory when it fits beside the chunk's tiles, else from global memory
     if (w_in_smem && (lam < C || window > 0)) {
         for (int i = threadIdx.x; i < d * df; i += blockDim.x) Ws[i] = Wh[i];
         Wuse = Ws;
@@ -124,14 +123,14 @@ step_route_kernel(T *kc, T *vc, float *score,
             __syncthreads();
         }
         const long long base = chunk * C;
-        const T *kh = kc + (((long long)b * Hkv + kv) * kvr + base % kvr) * d;   // (a chunk never straddles the ring's end)
-        const T *vh = vc + (((long long)b * Hkv + kv) * kvr + base % kvr) * d;
-        for (int i = threadIdx.x; i < C * d; i += blockDim.x) vs[i] = ld_f(vh + i);
+        const float *kh = kc + (((long long)b * Hkv + kv) * kvr + base % kvr) * d;   // (a chunk never straddles the ring's end)
+        const float *vh = vc + (((long long)b * Hkv + kv) * kvr + base % kvr) * d;
+        for (int i = threadIdx.x; i < C * d; i += blockDim.x) vs[i] = vh[i];
         float *xw = xs + warp * d;
         for (int r = warp; r < C; r += 8) {   // flag[r] != 0: the token stays out of this pass
             float ep[4], en[4];
             if (!flag[r]) {
-                for (int i = lane; i < d; i += 32) xw[i] = ld_f(kh + (long long)r * d + i);
+                for (int i = lane; i < d; i += 32) xw[i] = kh[(long long)r * d + i];
                 __syncwarp();
                 npmap_row(xw, Wuse, bh_, d, df, lane, ep, en);
             }
@@ -139,12 +138,8 @@ step_route_kernel(T *kc, T *vc, float *score,
             for (int jj = 0; jj < 4; ++jj)
                 if (jj < (df >> 5)) {
                     int j = lane + 32 * jj;
-                    // features are rounded to the storage type, as the prefill stores them
-                    T a, c2;
-                    st_f(&a, flag[r] ? 0.f : ep[jj]);
-                    st_f(&c2, flag[r] ? 0.f : en[jj]);
-                    ph[r * dp + j] = ld_f(&a);
-                    ph[r * dp + df + j] = ld_f(&c2);
+                    ph[r * dp + j] = flag[r] ? 0.f : ep[jj];
+                    ph[r * dp + df + j] = flag[r] ? 0.f : en[jj];
                 }
             __syncwarp();
         }
@@ -791,8 +786,8 @@ static int launch_route(const still_params_t *p, const StepArgs<T> &a, int32_t *
         size_t smem = ((size_t)C * 2 * df + (size_t)C * d + 8 * (size_t)d + C) * 4 + (size_t)C * 4;
         const int w_in_smem = smem + (size_t)d * df * sizeof(T) <= 200 * 1024 ? 1 : 0;
         if (w_in_smem) smem += (size_t)d * df * sizeof(T);
-        STILL_CUDA(cudaFuncSetAttribute(step_route_kernel<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
-        STILL_CUDA(launch_dependent(step_route_kernel<T>, dim3(p->H, p->B), dim3(256), smem, st, a.kc, a.vc, a.score, sel, a.sel_mask,
+        STILL_CUDA(cudaFuncSetAttribute(step_route_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+        STILL_CUDA(launch_dependent(step_route_kernel, dim3(p->H, p->B), dim3(256), smem, st, a.kc, a.vc, a.score, sel, a.sel_mask,
                                     a.S, a.z, wk, bkp, a.hdr, a.key, p->H, p->Hkv, a.cap, a.kvr, d, df, C, p->topk, cr, window,
                                     w_in_smem));
     }
