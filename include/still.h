@@ -286,7 +286,8 @@ int still_selftest_wait_timeout(void *status_block, int64_t limit_cycles, void *
 
 /*
  * Optional timing of the dominant kernel (the softmax-attention + merge kernel of the
- * prefill, the split-KV attend kernel of the decode step) for roofline reports.
+ * prefill; of the decode step the kernel that reads the K / V history and the linear
+ * state) for roofline reports.
  * still_profile_enable(n) creates n pairs of CUDA events owned by the library (host
  * objects, no device memory); from then on every call on this host thread records one
  * pair around that kernel on the caller's stream, until n pairs are used.

@@ -65,9 +65,9 @@ struct FwdPlan {
     bool la, tc, tc_la;
 };
 
-// Segments of the fp32 scan: two waves of two blocks per SM.  (These sizes are planned without a device; the kernels run
-// on any count of SMs.)
-constexpr int kScanBlocks = 4 * 148;
+// SMs that sizes are planned for (without a device; the kernels run on any count), and blocks of the fp32 scan: two waves
+// of two blocks per SM.
+constexpr int kSms = 148, kScanBlocks = 4 * kSms;
 
 // The workspace never takes more than `limit` bytes for the sake of speed alone (the sums of the scan's segments).
 static FwdPlan plan_fwd(const still_params_t *p, long long N, size_t limit = SIZE_MAX) {
@@ -122,7 +122,8 @@ static FwdPlan plan_fwd(const still_params_t *p, long long N, size_t limit = SIZ
         // where the call's room allows; a call that fits the static workspace without them is kept within it.  Otherwise
         // a sum lies in the rows of N_LA and D_LA that its segment writes later, which takes segments of at least 2 d_f
         // tokens, the last one included.  Of the two the one with the shorter segments is taken.  (At 16 heads, d = 64,
-        // C = 64 the sums lie in the rows between 1011 and 1160 tokens, where the static workspace is full.)
+        // C = 64 the sums lie in the rows between 1011 and 1160 tokens, where the static workspace is full: 175 us a call
+        // at 1100 tokens, 273 with one serial pass, 165 at 1200 with a place of their own.)
         const long long units = (long long)BH * (p->d / 64);
         const long long want = std::max<long long>(1, std::min<long long>((kScanBlocks + units - 1) / units, T - 2));
         const size_t per_seg = BH * dp * (size_t)(p->d + 1) * 4;
@@ -370,8 +371,11 @@ static int launch_sa_merge(const still_params_t *p, long long N, const T *Q, con
         ++g_launches;
         return STILL_OK;
     };
-    // 64 rows a block halve the shared-memory reads per product; 32 where the chunk is that short or 64 would leave SMs idle
-    const bool small = p->chunk == 32 || (N + 63) / 64 * p->H * p->B <= 148;
+    // 64 rows a block halve the shared-memory reads per product; 32 where the chunk is that short or 64 would leave SMs idle.
+    // (us a call of 4 heads, d = 64, 32 / 64 rows: 32 blocks of 64 rows 84.9 / 92.3, 128: 136 / 153, 148: 147 / 176, 160:
+    // 162 / 185, 256: 276 / 265; d = 128: 64 blocks 165 / 167, 144: 253 / 301, 160: 311 / 361.  Just past one block per SM
+    // the 32 rows are still ahead; where that ends between 160 and 256 blocks was not looked for.)
+    const bool small = p->chunk == 32 || (N + 63) / 64 * p->H * p->B <= kSms;
 #define STILL_SA(DD, ROWS, RT) \
     launch(sa_merge_kernel<T, DD, ROWS, RT>, ROWS, SaPlan<DD, ROWS, RT>::kThreads, SaPlan<DD, ROWS, RT>::kBytes)
     if (p->d == 64) return small ? STILL_SA(64, 32, 2) : STILL_SA(64, 64, 4);

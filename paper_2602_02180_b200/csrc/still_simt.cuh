@@ -529,7 +529,7 @@ la_prefix_kernel(SegSums sums, int n_S, int n_z, long long n_threads, int n_seg)
 // they pass through two buffers of KT keys.  Thread (ty, tx) owns RT rows: of the
 // logits the keys tx, tx + 16, ..., of the output the columns 4 tx .. + 3 (and + 64).
 // The rows' probabilities go from one product to the other through shared memory that
-// only the half warp of the row reads.  Bound by shared-memory reads (69 % of the rate):
+// only the half warp of the row reads.  Bound by shared-memory reads (57 % of the rate, issue slots 53 %):
 // 32 heads x 2000 tokens, d = 64, a quarter selected take 250 us with RT = 4 (16 warps an
 // SM), 264 us with RT = 8 (8 warps); with one read per operand and multiply 756 us.
 // Merge: with m the running max, ms = max(m, 0):

@@ -633,10 +633,11 @@ constexpr int step_main_smem() {
 }
 static_assert(step_main_smem<__nv_bfloat16, 128>() <= 232448 && step_main_smem<float, 128>() <= 232448, "shared memory of a step");
 
-// One block per SM.  At large batches the bytes of K, V and S bound it (B = 64, 32K prefix, every token: 6.6 TB/s a step,
-// 1.27 ms; with one launch each for the append and score, the cache pass in equal splits per group and the merge with
-// its read-out it was 1.65 ms; B = 16, 16K, a quarter kept: 143 us, before 305 us), at one sequence the latency of a
-// block's chain (one user, 2K prefix: 10.5 us a step with the merge, of which the host needs 10; before 71 us).
+// One block per SM.  At large batches the bytes of K, V and S bound it (us a step, the merge included; in brackets the form
+// with a launch each for append and score, routing, the cache pass in equal splits per group and the merge with its
+// read-out, timed in turn on one box: B = 64, 32K prefix, every token 1302 (1657), 6.6 TB/s; B = 16, 16K, a quarter kept
+// 148 (307); B = 32, 8K, capped at 448: 72 (203)), at one sequence the latency of a block's chain (one user, 2K prefix:
+// 10.5 (72), of which the host needs 10).
 template <typename T, int D, int NH>
 __global__ void __launch_bounds__(kStepThreads, 1)
 step_main_kernel(const __grid_constant__ StepArgs<T> a) {
@@ -861,14 +862,19 @@ static int step_typed(const still_params_t *p, char *state, const still_state_la
     const long long units = (long long)p->B * p->Hkv * a.units_per_group;
     a.n_items = a.la ? p->B * p->H : 0;
     // Few read-outs (a sequence or two): a block each, beside the blocks of the cache pass.  More: every block takes its
-    // share of the tiles and then of the read-outs.
+    // share of the tiles and then of the read-outs.  (us a step, d = 128, a quarter kept, apart / together: 32 read-outs
+    // 10.4 / 12.8 at 2000 tokens and 19.4 / 19.5 at 16000, 64: 11.4 / 13.9 and 35.0 / 29.9, 96: 17.2 / 15.1 and 73.9 / 39.5.)
     const bool apart = a.n_items <= n_sm / 2;
     const long long blocks = apart ? n_sm - a.n_items : n_sm;
     const long long least = (a.tiles + kMaxSplits - 2) / (kMaxSplits - 1);
     a.unit_len = a.tiles;
     a.per = (int)std::max<long long>({(units * a.tiles + blocks - 1) / blocks, least, 1});
     // Whole blocks per unit where a block's share is short: one with tiles of two units does two passes, one after the
-    // other, and a pass of up to eight rounds of the warps is mostly latency.
+    // other, and a pass of up to eight rounds of the warps is mostly latency.  (us a step, whole blocks / one line, every
+    // token kept: 8 units of 31, 125 and 500 tiles 7.3 / 9.0, 8.8 / 10.4, 11.4 / 13.8, of 2000 (past the second limit)
+    // 28.6 / 30.6; 32 units of 62 and 187 tiles 9.6 / 12.2, 13.2 / 14.7, of 1000 (past it) 46.1 / 48.9; 64 units (past the
+    // first limit) of 62 and 250 tiles 11.9 / 14.2, 28.5 / 28.7; 128 units 15.7 / 17.2, 47.0 / 49.5.  The limits are on the safe
+    // side: units just above half the SMs would leave nearly half of these without tiles, which was not timed.)
     const long long per_unit = blocks / units;
     if (per_unit >= 4 && a.tiles <= per_unit * 8 * kStepWarps) {
         a.per = (int)std::max<long long>((a.tiles + per_unit - 1) / per_unit, least);
@@ -878,7 +884,9 @@ static int step_typed(const still_params_t *p, char *state, const still_state_la
     w.early_k = per_unit >= 4;
     const long long used = (a.total + a.per - 1) / a.per;           // blocks with tiles
     a.first_item_block = apart ? (int)used : 0;
-    // The fewer warps share a read-out, the more run side by side and the longer one takes.
+    // The fewer warps share a read-out, the more run side by side and the longer one takes.  (us a step, d = 128, 2000 tokens,
+    // by eight / two / one warps: 128 read-outs 16.5 / 18.3 / 23.1, 160: 23.1 / 21.4 / 26.4, 576: 49.5 / 42.4 / 44.7,
+    // 640: 57.0 / 51.3 / 48.6, 2048: 147 / 120 / 120.)
     a.item_warps = a.n_items <= n_sm ? kStepWarps : a.n_items <= n_sm * (kStepWarps / 2) ? 2 : 1;
     const unsigned grid = (unsigned)(apart ? used + a.n_items : n_sm);
     auto launch = [&](auto head_dim) -> int {

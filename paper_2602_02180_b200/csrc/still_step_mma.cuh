@@ -16,8 +16,9 @@
 //
 // The weights P enter the second product as two bf16 parts, the upper 8 bits of the significand and the rest: rounded
 // to bf16 once they would be the largest error of a step, and one that depends on how the history is cut (a weight is
-// exact where it is its partial's maximum).  A group of up to four heads costs nothing for it: the four columns that it
-// leaves idle carry the second part.
+// exact where it is its partial's maximum): relative error of y against 64 bits 1.84e-3 to 2.25e-3, with both parts
+// 1.66e-3, which is y's own rounding.  A group of up to four heads takes no further product for it: the four columns
+// that it leaves idle carry the second part (16 x 16000 tokens, a quarter kept: 148 us a step, rounded once 145.5).
 #pragma once
 #include <cuda_bf16.h>
 #include <cuda_runtime.h>
@@ -153,7 +154,8 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
     const int c_piece = lane % P::kPieces, c_row = lane / P::kPieces;   // this lane's piece and first row of a copy
     constexpr int kRowsPerIt = 32 / P::kPieces;
     // With few sequences a step is a chain of latencies: K is then read without waiting for the membership words (all rows
-    // up to the new token; a masked logit is never used), V as soon as they are there.
+    // up to the new token; a masked logit is never used), V as soon as they are there.  (One user, 2000 tokens: 10.5 us a
+    // step, waiting 10.6; at 2 to 4 sequences waiting is 0.1 to 0.5 us faster, from 6 on 0.2 to 0.6.)
     auto load_tile = [&](int j, int stage, uint32_t rows, bool with_k, bool with_v) {
         uint8_t *ks = my + stage * P::kStage, *vs = ks + P::kTile;
         const int p0 = v.first_pos + j * kTileKeys;
