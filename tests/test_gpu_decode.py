@@ -345,3 +345,10 @@ def test_decode_nan_logits_make_the_output_nan(dtype, n_nan):
     for t in range(n0, w.N):
         y = still.hybrid_attn_step(p, state, w.N, t, *(x[:, :, t].contiguous() for x in (Q, K, V)))
         assert bool(torch.isnan(y[:, :rep]).all()) and bool(torch.isfinite(y[:, rep:]).all())
+
+
+def test_decode_with_the_most_partials_a_head_can_have():
+    # four KV heads of 2377 tiles as one line of blocks of 82: the second head's tiles lie in 30 blocks, the records that
+    # the scratch has room for
+    y, exact, _ = _dense_steps(1, 4, 1, 64, 38016, 4)
+    assert (y != exact.to(torch.bfloat16)).double().mean().item() <= 0.02
