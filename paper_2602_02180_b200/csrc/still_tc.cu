@@ -8,26 +8,20 @@
 // ascending position), so that "selected tokens of chunks 0..c-2" is the prefix
 // [0, (c-1)*lambda) of a contiguous array that TMA can tile.
 //
-// One CTA owns 256 consecutive query rows of one (batch, head): two query tiles
-// A and B of 128 rows, each with its own S accumulator (128 fp32 columns of TMEM)
-// and O accumulator (d columns).  The key stream of the CTA is a sequence of
-// 128-key tiles: SEL tiles j (rows [128j, 128j+128) of K_sel / V_sel) followed by
-// the three LOC tiles (rows of K / V at positions [128m, 128m+128), m = m0-1, m0,
-// m0+1 with m0 = first row / 128).  Which columns of a tile a query row sees is a
-// per-row column interval, applied as a mask in the softmax.
+// One CTA owns 256 consecutive query rows of one (batch, head), a pair of CTAs 512: two query tiles A and B of 128
+// (256) rows.  Their keys come as a stream of 128-key tiles: SEL tiles j (rows [128j, 128j+128) of K_sel / V_sel), and
+// the LOC tiles around the rows (rows of K / V at positions [128m, 128m+128)).  First the SEL tiles that both query
+// tiles see, then what only one of them sees, by turns.  Which columns of a tile a query row sees is a per-row column
+// interval, applied as a mask in the softmax.
 //
 // Warp roles (384 threads):
-//   warp 0     TMA producer: Q tiles once, then K and V tiles through mbarrier rings
-//   warp 1     MMA issuer (one elected thread): S_X = Q_X K^T (operands in shared
-//              memory, SWIZZLE_128B K-major), O_X += P_X V (P_X read from TMEM, V in
-//              shared memory MN-major); tcgen05.commit signals the softmax warps and
-//              frees the ring stages
-//   warps 4-7  softmax of tile A: one thread per query row (tcgen05.ld of the S row),
-//              online softmax in the log2 domain with lazy rescaling of O, P written
-//              back to TMEM as bf16 over S
-//   warps 8-11 the same for tile B
-//   The softmax warps also run the epilogue: O / l merged with the linear branch
-//   (N_LA, D_LA) under one denominator and stored as bf16.
+//   warps 0-7  softmax, four warps per query tile, one thread per query row (tcgen05.ld of the S row): online softmax in
+//              the log2 domain with lazy rescaling of O, P to TMEM as bf16; then the epilogue: O / l merged with the
+//              linear branch (N_LA, D_LA) under one denominator and stored as bf16
+//   warp 8     TMA producer: Q tiles once, then K and V tiles through mbarrier rings
+//   warp 9     MMA issuer (one elected thread): S = Q_X K^T (operands in shared memory, SWIZZLE_128B K-major),
+//              O_X += P_X V (P_X read from TMEM, V in shared memory MN-major)
+//   (warps 10, 11 only give up their registers)
 //
 // Every mbarrier wait is bounded: on expiry the kernel records
 // STILL_ERR_DEVICE_TIMEOUT in the status word, all roles leave their loops, and
@@ -43,61 +37,113 @@
 #include "still_common.cuh"
 #include "still_tc_ptx.cuh"
 
-// Column pairs out of every four whose exponential is computed on the FMA pipes (see softmax_role); measured
-// best at one: two and three were slower on both head dims.
-#ifndef STILL_POLY_OF4
-#define STILL_POLY_OF4 1
-#endif
-
 namespace still {
 
 namespace {
 
-constexpr int kBlockM = 128;   // query rows per tile
+constexpr int kBlockM = 128;   // query rows per tile and CTA
 constexpr int kBlockN = 128;   // keys per tile
-constexpr int kThreads = 384;
+constexpr int kThreads = 384, kProducerWarp = 8, kMmaWarp = 9;
+constexpr int kMaxDynamicSmem = 232448;   // 227 KiB: the most a CTA can be given on sm_100
 using namespace ptx;
 
 // ----------------------------------------------------------------- shared memory plan
 
-template <int D>
-struct SmemPlan {
-    static constexpr int kTileBytes = kBlockN * D * 2;        // one K or V or Q tile
-    static constexpr int kKStages = (D == 128) ? 3 : 4;
-    static constexpr int kVStages = (D == 128) ? 2 : 3;
-    static constexpr int kQ = 0;                               // two Q tiles
-    static constexpr int kK = kQ + 2 * kTileBytes;
-    static constexpr int kV = kK + kKStages * kTileBytes;
-    static constexpr int kBar = kV + kVStages * kTileBytes;    // mbarriers
-    static constexpr int kNumBars = 1 + 2 * kKStages + 2 * kVStages + 9;
-    static constexpr int kMisc = kBar + kNumBars * 8;          // tmem base, abort flag
+// In a CTA pair every CTA holds half of each key tile: 64 of the 128 keys of K, half of the value columns of V.
+template <int D, bool kPair>
+struct AttnPlan {
+    static constexpr int kQTile = kBlockM * D * 2;             // one Q tile of this CTA
+    static constexpr int kKRows = kPair ? kBlockN / 2 : kBlockN;
+    static constexpr int kVCols = kPair ? D / 2 : D;
+    static constexpr int kKTile = kKRows * D * 2;
+    static constexpr int kVTile = kBlockN * kVCols * 2;
+    static constexpr int kStages = 5;                          // of the ring: a K and a V tile each
+    static constexpr int kQ = 0;
+    static constexpr int kK = kQ + 2 * kQTile;
+    static constexpr int kV = kK + kStages * kKTile;
+    static constexpr int kBar = kV + kStages * kVTile;         // mbarriers
+    static constexpr int kNumBars = 1 + 2 * kStages + 2 + 2 + 2 + 2 + 1;
+    static constexpr int kMisc = kBar + kNumBars * 8;          // tmem base, abort flag, "a CTA has failed before"
     static constexpr int kTotal = kMisc + 16;
     static constexpr int kAlloc = kTotal + 1024;               // slack to align the base to 1024
+    static_assert(kAlloc <= kMaxDynamicSmem, "attention kernel: the shared-memory plan exceeds what a CTA can have");
+    static_assert(kMisc % 8 == 0 && kKTile % 1024 == 0 && kVTile % 1024 == 0, "attention kernel: operand tiles are swizzle-aligned");
 };
 
-constexpr int kMaxDynamicSmem = 232448;   // 227 KiB: the most a CTA can be given on sm_100
-static_assert(SmemPlan<64>::kAlloc <= kMaxDynamicSmem && SmemPlan<128>::kAlloc <= kMaxDynamicSmem,
-              "attention kernel: the shared-memory plan exceeds what a CTA can have");
-// every operand descriptor of the attention kernel addresses a whole tile inside its ring
-static_assert(SmemPlan<128>::kK == SmemPlan<128>::kQ + 2 * SmemPlan<128>::kTileBytes &&
-              SmemPlan<128>::kBar == SmemPlan<128>::kV + SmemPlan<128>::kVStages * SmemPlan<128>::kTileBytes,
-              "attention kernel: rings must follow each other without gaps");
+struct AttnBars {
+    uint64_t *q_full;
+    uint64_t *kv_full, *kv_empty;   // [kStages]
+    uint64_t *s_full;    // [2] S of query tile x is in tensor memory
+    uint64_t *s_free;    // [2] ... and has been read
+    uint64_t *p_full;    // [2] P_x is in tensor memory
+    uint64_t *pv_done;   // [2] O_x includes the tile's product (and P_x may be overwritten)
+    uint64_t *drain;     // MMA warp: everything issued has completed (failure path)
+    template <class P>
+    __device__ __forceinline__ static AttnBars at(uint8_t *smem, P) {
+        AttnBars b;
+        b.q_full = reinterpret_cast<uint64_t *>(smem + P::kBar);
+        b.kv_full = b.q_full + 1;
+        b.kv_empty = b.kv_full + P::kStages;
+        b.s_full = b.kv_empty + P::kStages;
+        b.s_free = b.s_full + 2;
+        b.p_full = b.s_free + 2;
+        b.pv_done = b.p_full + 2;
+        b.drain = b.pv_done + 2;
+        return b;
+    }
+};
 
-// Per-CTA description of the key stream.
+// A stage of the ring and the parity of its round.
+struct RingPos {
+    int stage, parity;
+    __device__ __forceinline__ void next(int n_stages) {
+        if (++stage == n_stages) {
+            stage = 0;
+            parity ^= 1;
+        }
+    }
+};
+
+// Tensor memory (512 columns): S_A, S_B, O_A, O_B and, beside them, P_A and P_B (64 columns each: 128 bf16).  P has a place
+// of its own so that S_x of the next tile can be formed while the softmax warps still work on this one, which they hold
+// in registers.  At D = 128 that leaves 128 columns for S: S_A and S_B share them, one after the other.
+template <int D>
+struct TmemPlan {
+    static constexpr bool kOneS = D == 128;
+    __device__ __forceinline__ static uint32_t s(int x) { return kOneS ? 0u : (uint32_t)x * 128u; }
+    __device__ __forceinline__ static uint32_t p(int x) { return (kOneS ? 128u : 384u) + (uint32_t)x * 64u; }
+    __device__ __forceinline__ static uint32_t o(int x) { return 256u + (uint32_t)x * (uint32_t)D; }
+};
+
+// The key stream of a CTA (or CTA pair).  Entries 0 .. n_shared - 1 are SEL tiles that both query tiles use; then come
+// the entries of one query tile each, A and B by turns until one has no more: its other SEL tiles, then its LOC tiles.
+// (With an entry's query tiles one after the other at the end, A waited for B there and B for A.)
 struct Stream {
-    int sel_first;          // first SEL tile of the stream (0 unless the salient cache has a budget)
-    int n_sel_a, n_sel_b;   // SEL tiles used by tile A / tile B, counted from sel_first
-    int m0;                 // first LOC tile index of interest is m0 - 1
-    int has_prev;           // m0 > 0
-    int has_b;              // tile B has rows below N
-    int n_tiles;            // stream length
-    // stream index i: [0, n_sel_b) SEL(i); then LOC(m0-1) (if has_prev), LOC(m0), LOC(m0+1) (if has_b)
-    __device__ __forceinline__ bool is_sel(int i) const { return i < n_sel_b; }
-    __device__ __forceinline__ int loc_m(int i) const { return m0 - has_prev + (i - n_sel_b); }
-    __device__ __forceinline__ bool used_by(int x, int i) const {
-        if (i < n_sel_b) return x == 0 ? (i < n_sel_a) : true;
-        int m = loc_m(i);
-        return x == 0 ? (m <= m0) : (m >= m0);
+    int sel0, n_shared;              // first shared SEL tile, number of shared entries
+    int sel_a, n_sel_a, loc_a, n_a;  // A's own: first SEL tile, SEL tiles, first LOC tile, entries
+    int sel_b, n_sel_b, loc_b, n_b;
+    __device__ __forceinline__ int entries() const { return n_shared + n_a + n_b; }
+    __device__ __forceinline__ int entries_of(int x) const { return n_shared + (x ? n_b : n_a); }
+    // entry of the k-th tile of query tile x
+    __device__ __forceinline__ int entry(int x, int k) const {
+        const int i = k - n_shared, turns = min(n_a, n_b);
+        return i < 0 ? k : n_shared + (i < turns ? 2 * i + x : i + turns);
+    }
+    // query tile and its running number of own entry s
+    __device__ __forceinline__ void own(int s, int &x, int &i) const {
+        const int turns = min(n_a, n_b);
+        x = s < 2 * turns ? s & 1 : (n_a > n_b ? 0 : 1);
+        i = s < 2 * turns ? s >> 1 : s - turns;
+    }
+    // entry e: a SEL tile, or a LOC tile?  Returns its number.
+    __device__ __forceinline__ int tile(int e, bool &sel) const {
+        sel = true;
+        if (e < n_shared) return sel0 + e;
+        int x, i;
+        own(e - n_shared, x, i);
+        const int n = x ? n_sel_b : n_sel_a;
+        sel = i < n;
+        return sel ? (x ? sel_b : sel_a) + i : (x ? loc_b : loc_a) + i - n;
     }
 };
 
@@ -127,78 +173,120 @@ __device__ __forceinline__ int sel_limit(long long pos, int C, int lam) {  // en
 // the oldest cached tokens have left for the linear state) the last `budget` entries before the end.
 __device__ __forceinline__ int sel_start(int limit, int budget) { return budget > 0 ? max(limit - budget, 0) : 0; }
 
+// The key stream of the query tiles that start at rows R0 and R0 + rows, of `rows` (a multiple of 128) rows each.
+__device__ __forceinline__ Stream make_stream(int R0, int rows, int N, int C, int lam, int budget) {
+    Stream st;
+    const int last_m = (N - 1) / kBlockN, m_a = R0 / kBlockN, m_b = m_a + rows / kBlockN;
+    const int last_a = min(R0 + rows, N) - 1, last_b = min(R0 + 2 * rows, N) - 1;
+    // SEL tiles [a0, a1) and [b0, b1): a tile's first row sees the oldest entries, its last row the newest
+    const int a0 = sel_start(sel_limit(R0, C, lam), budget) / kBlockN, a1 = (sel_limit(last_a, C, lam) + kBlockN - 1) / kBlockN;
+    st.loc_a = max(m_a - 1, 0);
+    st.sel_a = st.sel0 = a0;
+    st.n_shared = st.n_b = st.n_sel_b = st.sel_b = st.loc_b = 0;
+    st.n_sel_a = max(a1 - a0, 0);
+    if (R0 + rows < N) {
+        const int b0 = sel_start(sel_limit(R0 + rows, C, lam), budget) / kBlockN, b1 = (sel_limit(last_b, C, lam) + kBlockN - 1) / kBlockN;
+        st.sel0 = b0;                        // (a0 <= b0 and a1 <= b1)
+        st.n_shared = max(a1 - b0, 0);
+        st.n_sel_a = max(min(a1, b0) - a0, 0);
+        st.sel_b = max(b0, a1);
+        st.n_sel_b = max(b1 - st.sel_b, 0);
+        st.loc_b = m_b - 1;
+        st.n_b = st.n_sel_b + min(m_b + rows / kBlockN - 1, last_m) - st.loc_b + 1;
+    }
+    st.n_a = st.n_sel_a + min(m_b - 1, last_m) - st.loc_a + 1;
+    return st;
+}
+
 // ---------------------------------------------------------------------------
-// Softmax warps of the attention kernels (one warpgroup per query tile, a thread per query row) and the
-// merge epilogue.  `st` describes the CTA's (or the CTA pair's) key stream, x is the query tile (0: A, 1: B),
-// tile_row0 the position of the tile's first row, stage_tile the tile's Q region in shared memory (the
-// epilogue's staging space).  The barriers are this CTA's, except that in a CTA pair the two halves of P
-// are announced on the first CTA's p_half barriers (p_half_cluster: their address in the cluster window).
+// Softmax warps of the attention kernels (one warpgroup per query tile, a thread per query row) and the merge epilogue.
+// x is the query tile (0: A, 1: B), tile_row0 the position of the tile's first row, stage_tile the tile's Q region in
+// shared memory (the epilogue's staging space).  The barriers are this CTA's, except that in a CTA pair what the issuing
+// warp waits for is announced on the first CTA's.
 // ---------------------------------------------------------------------------
-template <int D, int kKStages, int kVStages, bool kPair, int kPolyOf4, class StreamT>
-__device__ __forceinline__ void softmax_role(const StreamT &st, const int x, const int tile_row0, const uint32_t tmem_base,
-                                             uint64_t *s_full, uint64_t *k_empty, uint64_t *v_empty, uint64_t *p_half,
-                                             const uint32_t p_half_cluster, uint64_t *o_final, volatile int *abort_flag,
-                                             int *status, uint8_t *stage_tile, const __nv_bfloat16 *y_part,
+template <int D, bool kPair>
+__device__ __forceinline__ void softmax_role(const Stream &st, const AttnBars &bar, const int x, const int tile_row0,
+                                             const uint32_t tmem_base, volatile int *abort_flag, int *status,
+                                             uint8_t *stage_tile, const __nv_bfloat16 *y_part,
                                              const float *d_part, const int n_parts, const long long part_stride_y,
                                              const long long part_stride_d, __nv_bfloat16 *Y, const int bh,
                                              const int N, const int C, const int lam, const int budget,
                                              const float scale_log2) {
+    constexpr int kStages = AttnPlan<D, kPair>::kStages;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-    auto col_s = [](int xx) -> uint32_t { return (uint32_t)xx * 128u; };
-    auto col_o = [](int xx) -> uint32_t { return 256u + (uint32_t)xx * (uint32_t)D; };
-    auto arrive_p = [&](int half) {
-        if constexpr (kPair) mbar_arrive_cluster(p_half_cluster + (uint32_t)(2 * x + half) * 8u);
-        else mbar_arrive(p_half + 2 * x + half);
+    auto arrive_first = [&](uint64_t *b) {   // on the barrier of the CTA whose warp issues the products
+        if constexpr (kPair) mbar_arrive_cluster(mapa(smem_u32(b), 0));
+        else mbar_arrive(b);
     };
-        const int row_in_tile = ((warp & 3) << 5) | lane;
+    const int row_in_tile = ((warp & 3) << 5) | lane;
     const int t = tile_row0 + row_in_tile;         // this thread's query position
-    const bool tile_present = (x == 0) || st.has_b;   // (a tile without rows below N still runs in a pair)
-    if (tile_present) {
+    const int n_mine = st.entries_of(x);
+    if (n_mine > 0) {                              // (in a pair also where none of this CTA's rows are below N)
         const uint32_t lane_addr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+        const uint32_t s_addr = lane_addr + TmemPlan<D>::s(x), p_addr = lane_addr + TmemPlan<D>::p(x), o_addr = lane_addr + TmemPlan<D>::o(x);
         const int tq = min(t, N - 1);              // rows past N mimic the last row (never stored)
         const int c = tq / C;
         const int lim_sel = c >= 2 ? (c - 1) * lam : 0, lo_sel = sel_start(lim_sel, budget);
         const int loc_lo = c >= 1 ? (c - 1) * C : 0;
         float m_used = -INFINITY, l_sum = 0.f;     // log2 domain
-        int n_seen = 0, prev_i = -1;
         bool ok = true;
-        for (int i = 0; i < st.n_tiles && ok; ++i) {
-            if (!st.used_by(x, i)) continue;
-            // visible column interval [lo, hi] of this row in stream tile i
-            int lo, hi;
-            if (st.is_sel(i)) {
-                lo = lo_sel - (st.sel_first + i) * kBlockN;
-                hi = lim_sel - (st.sel_first + i) * kBlockN - 1;
-            } else {
-                const int p0 = st.loc_m(i) * kBlockN;
-                lo = loc_lo - p0;
-                hi = tq - p0;
-            }
-            lo = max(lo, 0);
-            hi = min(hi, kBlockN - 1);
+        // one thread of a query tile releases the stage of its last product: its share of two, or both where the entry is
+        // the tile's alone
+        auto release = [&](int e) {
+            if (row_in_tile != 0) return;
+            mbar_arrive(bar.kv_empty + e % kStages);
+            if (e >= st.n_shared) mbar_arrive(bar.kv_empty + e % kStages);
+        };
+        for (int k = 0; k < n_mine && ok; ++k) {
+            // visible column interval [lo, hi] of this row in the stream tile
+            bool sel;
+            const int p0 = st.tile(st.entry(x, k), sel) * kBlockN;
+            const int lo = max((sel ? lo_sel : loc_lo) - p0, 0), hi = min((sel ? lim_sel - 1 : tq) - p0, kBlockN - 1);
             const bool need_mask = __any_sync(0xffffffffu, lo > 0 || hi < kBlockN - 1);
-            ok = mbar_wait(s_full + x, n_seen & 1, abort_flag, status, 8);
+            const bool none = need_mask && !__any_sync(0xffffffffu, lo <= hi);   // (a warp whose rows see none of it writes zeros)
+            ok = mbar_wait(bar.s_full + x, k & 1, abort_flag, status, 8);
             if (!ok) break;
             tc_fence_after();
-            if (row_in_tile == 0) {
-                // S_x of tile i is complete, and so is everything the MMA warp issued before it (each
-                // tcgen05.commit costs the tensor pipe a bubble, so the ring stages are released here
-                // instead): tile x is done with this K stage and with the V stage of its previous tile.
-                mbar_arrive(k_empty + i % kKStages);
-                if (prev_i >= 0) mbar_arrive(v_empty + prev_i % kVStages);
+            if (none) {
+                if (lane == 0) arrive_first(bar.s_free + x);
+                uint32_t zero[32];
+#pragma unroll
+                for (int j = 0; j < 32; ++j) zero[j] = 0u;
+                if (k > 0) {
+                    ok = mbar_wait(bar.pv_done + x, (k - 1) & 1, abort_flag, status, 11);
+                    if (!ok) break;
+                    release(st.entry(x, k - 1));
+                    tc_fence_after();
+                }
+                __syncwarp();
+                tmem_st32(p_addr, zero);
+                tmem_st32(p_addr + 32, zero);
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) arrive_first(bar.p_full + x);
+                continue;
             }
-            prev_i = i;
             uint32_t sr[128];
-            tmem_ld32(lane_addr + col_s(x) + 0, sr + 0);
-            tmem_ld32(lane_addr + col_s(x) + 32, sr + 32);
-            tmem_ld32(lane_addr + col_s(x) + 64, sr + 64);
-            tmem_ld32(lane_addr + col_s(x) + 96, sr + 96);
+            tmem_ld32(s_addr, sr);
+            tmem_ld32(s_addr + 32, sr + 32);
+            tmem_ld32(s_addr + 64, sr + 64);
+            tmem_ld32(s_addr + 96, sr + 96);
             tmem_wait_ld();
+            tc_fence_before();
+            __syncwarp();
+            if (lane == 0) arrive_first(bar.s_free + x);
             float *s = reinterpret_cast<float *>(sr);
             if (need_mask) {
 #pragma unroll
-                for (int j = 0; j < 128; ++j)
-                    if (j < lo || j > hi) s[j] = -INFINITY;
+                for (int q = 0; q < 4; ++q) {
+                    // columns of this block of 32 that the row sees, as a bit set
+                    const int l = min(max(lo - 32 * q, 0), 32), n = min(max(hi - 32 * q + 1, 0), 32);
+                    const uint32_t seen = n > l ? (0xffffffffu >> (32 - n)) & (0xffffffffu << l) : 0u;
+#pragma unroll
+                    for (int j = 0; j < 32; ++j)
+                        if (!((seen >> j) & 1u)) s[q * 32 + j] = -INFINITY;
+                }
             }
             float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
 #pragma unroll
@@ -216,53 +304,61 @@ __device__ __forceinline__ void softmax_role(const StreamT &st, const int x, con
                 alpha = (m_used == -INFINITY) ? 0.f : ex2(m_used - mt);
                 m_used = mt;
             }
-            if (n_seen > 0 && __any_sync(0xffffffffu, grow)) {
-                // S of this tile was committed after the previous P V product: O is quiescent
+            // the previous product is in O, has read P and is done with its stage (asked for as late as P is written: the
+            // issuing warp takes it up behind a product of the other query tile)
+            auto previous_done = [&]() { return mbar_wait(bar.pv_done + x, (k - 1) & 1, abort_flag, status, 11); };
+            if (k > 0 && __any_sync(0xffffffffu, grow)) {
+                ok = previous_done();
+                if (!ok) break;
+                tc_fence_after();
+                {
 #pragma unroll
-                for (int q = 0; q < D / 32; ++q) {
-                    uint32_t orow[32];
-                    tmem_ld32(lane_addr + col_o(x) + q * 32, orow);
-                    tmem_wait_ld();
+                    for (int q = 0; q < D / 32; ++q) {
+                        uint32_t orow[32];
+                        tmem_ld32(o_addr + q * 32, orow);
+                        tmem_wait_ld();
 #pragma unroll
-                    for (int j = 0; j < 32; ++j) orow[j] = __float_as_uint(__uint_as_float(orow[j]) * alpha);
-                    tmem_st32(lane_addr + col_o(x) + q * 32, orow);
+                        for (int j = 0; j < 32; ++j) orow[j] = __float_as_uint(__uint_as_float(orow[j]) * alpha);
+                        tmem_st32(o_addr + q * 32, orow);
+                    }
                 }
             }
             l_sum *= alpha;
             const float neg_m = (m_used == -INFINITY) ? 0.f : -m_used;
             const float2 scale2 = make_float2(scale_log2, scale_log2), negm2 = make_float2(neg_m, neg_m);
             float2 acc = make_float2(0.f, 0.f);
-            // P = 2^(s * scale - m) as bf16 over S, in two halves of 64 columns; the MMA warp starts on the first
-            // half while the second is computed.  The MUFU unit (one warp instruction per eight cycles) would need
-            // 1024 cycles for a warp's 128 exponentials of a tile, which is as long as the tensor pipe needs for the
-            // tile's two products; so kPolyOf4 of every four column pairs take 2^x from the FMA pipes instead (see
-            // exp2_fma2), interleaved with the others so that both units work at the same time.
+            // P = 2^(s * scale - m) as bf16.  The MUFU unit (one warp instruction per eight cycles) would need 1024 cycles
+            // for a query tile's exponentials, which is as long as the tensor pipe needs for the tile's two products; so
+            // one of kPolyEvery column pairs takes 2^x from the FMA pipes instead (see exp2_fma2), interleaved with the
+            // others so that both units work at the same time.  (32768 tokens, d = 128, every token kept: none 14.5 ms, one
+            // of 8 14.3, of 4 14.45, 5 of 16 14.7; 4096 tokens, d = 64: 536, 515, 512 and 517 us.)
+            constexpr int kPolyEvery = D == 64 ? 4 : 8;
+            uint32_t pk[2][32];
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
-                uint32_t pk[32];
 #pragma unroll
                 for (int j = 0; j < 32; ++j) {
                     const float2 sv = make_float2(s[q * 64 + 2 * j], s[q * 64 + 2 * j + 1]);
                     const float2 xv = __ffma2_rn(sv, scale2, negm2);
-                    const float2 pr = (j % 4) < kPolyOf4 ? exp2_fma2(xv) : make_float2(ex2(xv.x), ex2(xv.y));
+                    const float2 pr = j % kPolyEvery == 0 ? exp2_fma2(xv) : make_float2(ex2(xv.x), ex2(xv.y));
                     acc = __fadd2_rn(acc, pr);
-                    pk[j] = pack_bf16(pr.x, pr.y);
-                    if (q == 1 && j == 12) {
-                        // the first half of P has had time to land: hand it to the MMA warp
-                        tmem_wait_st();
-                        tc_fence_before();
-                        __syncwarp();
-                        if (lane == 0) arrive_p(0);
-                    }
+                    pk[q][j] = pack_bf16(pr.x, pr.y);
                 }
-                tmem_st32(lane_addr + col_s(x) + q * 32, pk);
             }
+            if (k > 0) {
+                if (ok) ok = previous_done();
+                if (!ok) break;
+                tc_fence_after();
+                release(st.entry(x, k - 1));
+                __syncwarp();
+            }
+            tmem_st32(p_addr, pk[0]);
+            tmem_st32(p_addr + 32, pk[1]);
             l_sum += acc.x + acc.y;
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
-            if (lane == 0) arrive_p(1);
-            ++n_seen;
+            if (lane == 0) arrive_first(bar.p_full + x);
         }
         // ---- epilogue: y = (O e^{m-ms} + e^{-ms} N_LA) / (l e^{m-ms} + e^{-ms} D_LA), ms = max(m, 0)
         // The linear branch arrives as up to two partial results (one per feature half): y_p = N_p / D_p as bf16
@@ -272,10 +368,11 @@ __device__ __forceinline__ void softmax_role(const StreamT &st, const int x, con
         // warp's 32 rows of the tile's Q region (one row = D bf16 = 2 D bytes: D / 2 columns of both parts), free
         // once the tile's last Q K^T has completed; 16-byte pieces are swizzled by the row so that row-wise and
         // piece-wise accesses avoid bank conflicts.
-        if (ok) ok = mbar_wait(o_final + x, 0, abort_flag, status, 9);
+        if (ok) ok = mbar_wait(bar.pv_done + x, (n_mine - 1) & 1, abort_flag, status, 9);   // (every query tile has a LOC tile)
         ok = __all_sync(0xffffffffu, ok);
         if (ok) {
             tc_fence_after();
+            release(st.entry(x, n_mine - 1));   // (the other query tile may have entries left)
             constexpr int kRowBytes = D * 2, kPieces = kRowBytes / 16;   // pieces of 16 bytes per staged row
             constexpr int kPartPieces = kPieces / 2;                     // pieces of one part (D / 2 columns)
             uint8_t *stg = stage_tile + (warp & 3) * 32 * kRowBytes;
@@ -321,7 +418,7 @@ __device__ __forceinline__ void softmax_role(const StreamT &st, const int x, con
 #pragma unroll
                 for (int q = 0; q < D / 64; ++q) {
                     uint32_t orow[32];
-                    tmem_ld32(lane_addr + col_o(x) + hh * (D / 2) + q * 32, orow);
+                    tmem_ld32(o_addr + hh * (D / 2) + q * 32, orow);
                     tmem_wait_ld();
 #pragma unroll
                     for (int j8 = 0; j8 < 4; ++j8) {
@@ -361,323 +458,192 @@ __device__ __forceinline__ void softmax_role(const StreamT &st, const int x, con
     }
 }
 
-template <int D>
-__global__ void __launch_bounds__(kThreads, 1)
-sa_merge_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                   const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ksel,
-                   const __grid_constant__ CUtensorMap tm_vsel, const __nv_bfloat16 *y_part,
-                   const float *d_part, int n_parts, __nv_bfloat16 *Y, int *status, int H, int Hkv,
-                   int N, int C, int lam, int budget, int sel_rows, int sel_identity, float scale_log2, int n_qblocks, int n_heads,
-                   int set_heads) {
-    grid_dep_wait();
-    grid_dep_launch();
-    using P = SmemPlan<D>;
-    extern __shared__ uint8_t smem_raw[];
-    uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + P::kBar);
-    uint64_t *q_full = bars;
-    uint64_t *k_full = bars + 1, *k_empty = k_full + P::kKStages;
-    uint64_t *v_full = k_empty + P::kKStages, *v_empty = v_full + P::kVStages;
-    uint64_t *s_full = v_empty + P::kVStages;  // [2]
-    uint64_t *p_half = s_full + 2;             // [2][2]: columns [0,64) / [64,128) of P_X are in TMEM
-    uint64_t *o_final = p_half + 4;            // [2]
-    uint64_t *drain = o_final + 2;             // MMA warp: everything issued has completed (failure path)
-    uint32_t *tmem_base_slot = reinterpret_cast<uint32_t *>(smem + P::kMisc);
-    volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + P::kMisc + 8);
-
-    const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;   // (known to be the same in all lanes)
-    int qb, bh;
-    row_block(blockIdx.x, n_qblocks, n_heads, set_heads, qb, bh);
-    const int b = bh / H, h = bh % H, kvh = h / (H / Hkv);
-    const int R0 = qb * 2 * kBlockM;
-
-    Stream st;
-    st.m0 = R0 / kBlockN;
-    st.has_prev = st.m0 > 0;
-    st.has_b = (R0 + kBlockM) < N;
-    {
-        int last_a = min(R0 + kBlockM - 1, N - 1), last_b = min(R0 + 2 * kBlockM - 1, N - 1);
-        st.sel_first = sel_start(sel_limit(R0, C, lam), budget) / kBlockN;   // the CTA's first row sees the oldest entries
-        st.n_sel_a = max((sel_limit(last_a, C, lam) + kBlockN - 1) / kBlockN - st.sel_first, 0);
-        st.n_sel_b = st.has_b ? max((sel_limit(last_b, C, lam) + kBlockN - 1) / kBlockN - st.sel_first, 0) : st.n_sel_a;
+// TMA producer (one thread): the Q tiles, then the K and V tiles of the stream, as far ahead as the ring has free stages.  In a
+// pair every CTA loads its halves; their byte counts complete on the first CTA's barriers.
+template <int D, bool kPair, class TellPeer>
+__device__ __forceinline__ void producer_role(const Stream &st, const AttnBars &bar, uint8_t *smem, const uint32_t rank,
+                                              const CUtensorMap &tm_q, const CUtensorMap &tm_k, const CUtensorMap &tm_v,
+                                              const CUtensorMap &tm_ksel, const CUtensorMap &tm_vsel, const int q_row,
+                                              const int kv_row0, const int sel_row0, volatile int *abort_flag, int *status,
+                                              TellPeer tell_peer) {
+    using P = AttnPlan<D, kPair>;
+    constexpr int kCtas = kPair ? 2 : 1, kStages = P::kStages;
+    const uint32_t q_full0 = mapa(smem_u32(bar.q_full), 0), kv_full0 = mapa(smem_u32(bar.kv_full), 0);
+    auto load = [&](uint8_t *dst, const CUtensorMap &map, uint64_t *b, uint32_t b0, int col, int row) {
+        if constexpr (kPair) tma_load_2d_pair(dst, &map, b0, col, row);
+        else tma_load_2d(dst, &map, b, col, row);
+    };
+    const int n_q = st.n_b > 0 ? 2 : 1, n = st.entries();   // (every query tile has a LOC tile)
+    if (rank == 0) mbar_expect_tx(bar.q_full, kCtas * n_q * P::kQTile);
+    for (int x = 0; x < n_q; ++x)
+        for (int half = 0; half < D / 64; ++half)
+            load(smem + P::kQ + x * P::kQTile + half * (kBlockM * 128), tm_q, bar.q_full, q_full0, half * 64,
+                 q_row + ((int)rank + x * kCtas) * kBlockM);
+    bool ok = true;
+    int armed = 0;
+    RingPos pos{0, 0}, last{0, 0};
+    for (; armed < n; ++armed) {
+        ok = mbar_wait(bar.kv_empty + pos.stage, pos.parity ^ 1, abort_flag, status, 1);
+        if (!ok) break;
+        bool sel;
+        const int tile = st.tile(armed, sel), row = (sel ? sel_row0 : kv_row0) + tile * kBlockN;
+        if (rank == 0) mbar_expect_tx(bar.kv_full + pos.stage, kCtas * (P::kKTile + P::kVTile));
+        for (int half = 0; half < D / 64; ++half)   // (of a pair: this CTA's 64 keys)
+            load(smem + P::kK + pos.stage * P::kKTile + half * (P::kKRows * 128), sel ? tm_ksel : tm_k, bar.kv_full + pos.stage,
+                 kv_full0 + pos.stage * 8, half * 64, row + (int)rank * P::kKRows);
+        for (int q = 0; q < P::kVCols / 64; ++q)    // this CTA's value columns, 64 at a time
+            load(smem + P::kV + pos.stage * P::kVTile + q * (kBlockN * 128), sel ? tm_vsel : tm_v, bar.kv_full + pos.stage,
+                 kv_full0 + pos.stage * 8, (int)rank * P::kVCols + q * 64, row);
+        last = pos;
+        pos.next(kStages);
     }
-    st.n_tiles = st.n_sel_b + st.has_prev + 1 + st.has_b;
-
-    // A CTA that starts after another one has reported a failure does nothing.
-    if (threadIdx.x == 0) *abort_flag = *reinterpret_cast<volatile int *>(status) != 0;
-    __syncthreads();
-    if (*abort_flag) return;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        mbar_init(q_full, 1);
-        for (int i = 0; i < P::kKStages; ++i) { mbar_init(k_full + i, 1); mbar_init(k_empty + i, 2); }
-        for (int i = 0; i < P::kVStages; ++i) { mbar_init(v_full + i, 1); mbar_init(v_empty + i, 2); }
-        for (int i = 0; i < 2; ++i) { mbar_init(s_full + i, 1); mbar_init(o_final + i, 1); }
-        for (int i = 0; i < 4; ++i) mbar_init(p_half + i, 4);  // one arrival per softmax warp
-        mbar_init(drain, 1);
-        *abort_flag = 0;
-        fence_barrier_init();
-    }
-    if (warp == 1) {
-        tmem_alloc(tmem_base_slot, 512);
-        tmem_relinquish();
-    }
-    tc_fence_before();
-    __syncthreads();
-    tc_fence_after();
-    const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_base_slot, 0);
-    // TMEM columns: S_A [0,128), S_B [128,256), O_A [256,256+D), O_B [256+D, 256+2D); P_X overlays S_X.
-    auto col_s = [](int x) -> uint32_t { return (uint32_t)x * 128u; };
-    auto col_o = [](int x) -> uint32_t { return 256u + (uint32_t)x * (uint32_t)D; };
-
-    // The softmax threads keep a whole 128-column row in registers: move registers from the
-    // load / MMA warpgroup to the two softmax warpgroups (128 * 64 + 256 * 216 <= 384 * 168).
-    if (warp < 4) {
-    reg_dec<64>();
-    if (warp == 0) {
-        // ------------------------------------------------------------ TMA producer
-        if (lane == 0) {
-            const int q_row = bh * N + R0;
-            mbar_expect_tx(q_full, (st.has_b ? 2 : 1) * P::kTileBytes);
-            for (int x = 0; x < (st.has_b ? 2 : 1); ++x)
-                for (int half = 0; half < D / 64; ++half)
-                    tma_load_2d(smem + P::kQ + x * P::kTileBytes + half * (kBlockM * 128), &tm_q, q_full, half * 64,
-                                q_row + x * kBlockM);
-            // With topk = chunk every token is selected and the compacted arrays would be copies of K / V:
-            // the salient prefix is then read from K / V themselves (tm_ksel / tm_vsel alias tm_k / tm_v).
-            const int sel_base = sel_identity ? (b * Hkv + kvh) * N : bh * sel_rows;
-            // K and V rings advance independently, each as far ahead as its free stages allow.
-            bool ok = true;
-            int armed_k = 0, armed_v = 0, spins = 0;
-            long long t0 = clock64();
-            while (armed_k < st.n_tiles || armed_v < st.n_tiles) {
-                bool progressed = false;
-                if (armed_k < st.n_tiles) {
-                    const int i = armed_k, ks = i % P::kKStages;
-                    if (mbar_try_wait(k_empty + ks, ((i / P::kKStages) & 1) ^ 1)) {
-                        const bool sel = st.is_sel(i);
-                        const int row = sel ? sel_base + (st.sel_first + i) * kBlockN : (b * Hkv + kvh) * N + st.loc_m(i) * kBlockN;
-                        mbar_expect_tx(k_full + ks, P::kTileBytes);
-                        for (int half = 0; half < D / 64; ++half)
-                            tma_load_2d(smem + P::kK + ks * P::kTileBytes + half * (kBlockN * 128), sel ? &tm_ksel : &tm_k,
-                                        k_full + ks, half * 64, row);
-                        ++armed_k;
-                        progressed = true;
-                    }
-                }
-                if (armed_v < st.n_tiles) {
-                    const int i = armed_v, vs = i % P::kVStages;
-                    if (mbar_try_wait(v_empty + vs, ((i / P::kVStages) & 1) ^ 1)) {
-                        const bool sel = st.is_sel(i);
-                        const int row = sel ? sel_base + (st.sel_first + i) * kBlockN : (b * Hkv + kvh) * N + st.loc_m(i) * kBlockN;
-                        mbar_expect_tx(v_full + vs, P::kTileBytes);
-                        for (int half = 0; half < D / 64; ++half)
-                            tma_load_2d(smem + P::kV + vs * P::kTileBytes + half * (kBlockN * 128), sel ? &tm_vsel : &tm_v,
-                                        v_full + vs, half * 64, row);
-                        ++armed_v;
-                        progressed = true;
-                    }
-                }
-                if (progressed) {
-                    spins = 0;
-                } else if ((++spins & 1023) == 0) {
-                    if (spins == 1024) t0 = clock64();
-                    if (*abort_flag) { ok = false; break; }
-                    if (clock64() - t0 > kWaitLimitCycles) {
-                        *abort_flag = 1;
-                        report_status(status, STILL_ERR_DEVICE_TIMEOUT, 1);
-                        ok = false;
-                        break;
-                    }
-                }
-            }
-            if (!ok) {
-                // leave no copy in flight behind: wait (bounded) for the loads already issued
-                if (armed_k > 0) {
-                    int i = armed_k - 1;
-                    mbar_wait_drain(k_full + i % P::kKStages, (i / P::kKStages) & 1);
-                }
-                if (armed_v > 0) {
-                    int i = armed_v - 1;
-                    mbar_wait_drain(v_full + i % P::kVStages, (i / P::kVStages) & 1);
-                }
-            }
+    if (!ok) {
+        if constexpr (kPair) tell_peer();
+        // leave no copy in flight behind: wait (bounded) for the last stage armed, which in a pair counts both CTAs'
+        // bytes; the second CTA of a pair, whose copies complete on the first's barriers, waits out a fixed stretch
+        // that is long against a tile load
+        if (rank == 0) {
+            if (armed > 0) mbar_wait_drain(bar.kv_full + last.stage, last.parity);
+        } else {
+            const long long t1 = clock64();
+            while (clock64() - t1 < 200000) {}
         }
-    } else if (warp == 1) {
-        // ------------------------------------------------------------ MMA issuer
-        // The whole warp walks the stream and waits on the barriers; one elected lane issues (control flow and
-        // descriptors stay the same in all lanes and can live in uniform registers, where the tensor-core
-        // instructions take their operands from).  A failed wait does not leave the loop: it switches off the
-        // remaining waits and instructions, and the loop runs out.
-        {
-            const bool leader = elect_one();
-            constexpr uint32_t idesc_qk = make_idesc(kBlockM, kBlockN, false);
-            constexpr uint32_t idesc_pv = make_idesc(kBlockM, D, true);
-            bool ok = mbar_wait(q_full, 0, abort_flag, status, 4);
-            tc_fence_after();
-            // descriptors as low words: a k-step adds a constant
-            const uint32_t q_lo0 = desc_lo(smem_u32(smem + P::kQ), 0);
-            const uint32_t k_lo0 = desc_lo(smem_u32(smem + P::kK), 0);
-            const uint32_t v_lo0 = desc_lo(smem_u32(smem + P::kV), kBlockN * 128);
-            int pending[2] = {-1, -1};   // stream tile whose P V product is still to be issued
-            int n_done[2] = {0, 0};      // tiles processed per query tile (phase of p_full)
-            auto wait = [&](uint64_t *bar, int parity, int where) {
-                if (ok) ok = mbar_wait(bar, (uint32_t)parity, abort_flag, status, where);
-            };
-            auto issue_pv = [&](int x, int ip) {
-                const int vs = ip % P::kVStages;
-                // (V has normally arrived long ago: checking it first hides the check behind the wait for P)
-                wait(v_full + vs, (ip / P::kVStages) & 1, 6);
-                wait(p_half + 2 * x, n_done[x] & 1, 5);
-                tc_fence_after();
-                const uint32_t v_lo = v_lo0 + vs * (P::kTileBytes >> 4);
-                const uint32_t d_o = tmem_base + col_o(x), a_p = tmem_base + col_s(x);
-                const uint32_t acc0 = n_done[x] > 0 ? 1u : 0u;
-                if (leader && ok) {
-                    mma_ts_lo<idesc_pv>(d_o, a_p, v_lo, acc0);
-#pragma unroll
-                    for (int k = 1; k < kBlockN / 32; ++k)
-                        mma_ts_lo<idesc_pv>(d_o, a_p + k * 8, v_lo + k * (16 * 128 >> 4), 1u);
-                }
-                wait(p_half + 2 * x + 1, n_done[x] & 1, 5);
-                tc_fence_after();
-                if (leader && ok) {
-#pragma unroll
-                    for (int k = kBlockN / 32; k < kBlockN / 16; ++k)
-                        mma_ts_lo<idesc_pv>(d_o, a_p + k * 8, v_lo + k * (16 * 128 >> 4), 1u);
-                }
-                ++n_done[x];
-            };
-            for (int i = 0; i < st.n_tiles; ++i) {
-                const int ks = i % P::kKStages;
-                wait(k_full + ks, (i / P::kKStages) & 1, 7);
-                tc_fence_after();
-                const uint32_t k_lo = k_lo0 + ks * (P::kTileBytes >> 4);
-#pragma unroll
-                for (int x = 0; x < 2; ++x) {
-                    const bool present = (x == 0) || st.has_b;
-                    if (present && st.used_by(x, i)) {
-                        if (pending[x] >= 0) {
-                            const int ip = pending[x];
-                            issue_pv(x, ip);
-                            // a V stage is released by two arrivals: pay the other tile's share if it skipped ip
-                            if (leader && ok && !(((1 - x) == 0 || st.has_b) && st.used_by(1 - x, ip)))
-                                mbar_arrive(v_empty + ip % P::kVStages);
-                        }
-                        const uint32_t q_lo = q_lo0 + x * (P::kTileBytes >> 4), d_s = tmem_base + col_s(x);
-                        if (leader && ok) {
-                            mma_ss_lo<idesc_qk, 0>(d_s, q_lo, k_lo);
-#pragma unroll
-                            for (int k = 1; k < D / 16; ++k) {
-                                // k-step of 16 elements: 32 bytes within a 64-element swizzle atom, atoms 128 rows apart
-                                const uint32_t off = ((k / 4) * (kBlockM * 128) + (k % 4) * 32) >> 4;
-                                mma_ss_lo<idesc_qk, 1>(d_s, q_lo + off, k_lo + off);
-                            }
-                            tc_commit(s_full + x);
-                        }
-                        pending[x] = i;
-                    } else if (leader && ok) {
-                        mbar_arrive(k_empty + ks);  // the share of a tile that skips this stream tile
-                    }
-                }
-            }
-#pragma unroll
-            for (int x = 0; x < 2; ++x) {
-                if (pending[x] >= 0) {
-                    issue_pv(x, pending[x]);
-                    if (leader && ok) tc_commit(o_final + x);
-                }
-            }
-            if (!__all_sync(0xffffffffu, ok) && leader) {  // no MMA may still be running when tensor memory is freed
-                tc_commit(drain);
-                mbar_wait_drain(drain, 0);
-            }
-        }
-    }
-    } else {
-        reg_inc<216>();
-        // ------------------------------------------------------------ softmax + epilogue
-        const int x = (warp - 4) >> 2;                 // 0: tile A, 1: tile B
-        softmax_role<D, P::kKStages, P::kVStages, false, STILL_POLY_OF4>(st, x, R0 + x * kBlockM, tmem_base, s_full, k_empty, v_empty, p_half, 0u,
-                                                         o_final, abort_flag, status, smem + P::kQ + x * P::kTileBytes, y_part,
-                                                         d_part, n_parts, (long long)n_heads * N * D, (long long)n_heads * N,
-                                                         Y, bh, N, C, lam, budget, scale_log2);
-    }
-    tc_fence_before();
-    __syncthreads();
-    if (warp == 1) {
-        tc_fence_after();
-        tmem_dealloc(tmem_base, 512);
     }
 }
 
-// ---------------------------------------------------------------------------
-// The same branch on CTA pairs (head dim 128): two CTAs of a cluster work on 512 consecutive query rows of
-// one (batch, head) with UMMAs of the cta_group::2 form.  Query tile X of the pair is 256 rows -- rows
-// [R0 + 256 X + 128 r, + 128) belong to the CTA of cluster rank r -- and one instruction, issued by a thread
-// of rank 0, computes S_X = Q_X K^T (or O_X += P_X V) for both CTAs.  Each CTA keeps only its half of every
-// key tile in shared memory: 64 of the 128 keys of K (the B operand of Q K^T is split along N) and 64 of the
-// 128 value columns of V (likewise for P V); the tensor cores of both SMs read both halves.  Per FLOP a CTA
-// therefore pulls half the K / V bytes from L2 and reads a quarter less shared memory than a CTA working
-// alone, and the rings hold five stages each.
+// MMA issuer (in a pair: of the first CTA).  The whole warp walks the items and waits on the barriers; one elected lane
+// issues.  Kept this way, control flow and every descriptor are the same in all lanes, which lets them live in the
+// warp's uniform registers, where the tensor-core instructions take their operands from.  (With a single lane in a
+// divergent branch each instruction cost that lane 55 - 80 cycles of operand marshalling, whatever the instruction's
+// size, and the tensor pipe starved behind it.)  A failed wait does not leave the loop: it switches off the remaining
+// waits and instructions, and the loop runs out.
 //
-// Who signals whom.  K / V / Q tiles: every CTA loads its halves into its own shared memory with plain TMA
-// loads (no multicast) whose byte counts complete on the full-barriers of rank 0, where the issuing thread
-// waits.  S_X ready, O_X final: one tcgen05.commit arrives on the barrier of both CTAs.  P_X written: the
-// softmax warps of both CTAs arrive on rank 0's p_half barriers (eight arrivals).  Ring stages are released
-// locally: when a CTA's softmax warps see S_X of stream tile i, the pair's instruction has completed in both
-// CTAs.  Everything else -- stream, masks, online softmax, merge epilogue -- is as in the kernel above.
-// ---------------------------------------------------------------------------
-template <int D>
-struct PairPlan {
-    static constexpr int kQTile = kBlockM * D * 2;             // one Q tile of this CTA (128 rows)
-    static constexpr int kKHalf = (kBlockN / 2) * D * 2;       // 64 keys of a K tile
-    static constexpr int kVHalf = kBlockN * (D / 2) * 2;       // 128 keys x D / 2 value columns
-    static constexpr int kKStages = 5, kVStages = 5;
-    static constexpr int kQ = 0;
-    static constexpr int kK = kQ + 2 * kQTile;
-    static constexpr int kV = kK + kKStages * kKHalf;
-    static constexpr int kBar = kV + kVStages * kVHalf;
-    static constexpr int kNumBars = 1 + 2 * kKStages + 2 * kVStages + 9;
-    static constexpr int kMisc = kBar + kNumBars * 8;          // tmem base, abort flag, "a CTA has failed before"
-    static constexpr int kTotal = kMisc + 16;
-    static constexpr int kAlloc = kTotal + 1024;
-};
-static_assert(PairPlan<128>::kAlloc <= kMaxDynamicSmem, "pair attention kernel: the shared-memory plan exceeds what a CTA can have");
-
-// Key stream of a CTA pair (same in both CTAs): SEL tiles, then the LOC tiles m_first .. m_last.
-struct PairStream {
-    int sel_first, n_sel_a, n_sel_b, m0, m_first, has_b, n_tiles;   // SEL tiles are counted from sel_first
-    __device__ __forceinline__ bool is_sel(int i) const { return i < n_sel_b; }
-    __device__ __forceinline__ int loc_m(int i) const { return m_first + (i - n_sel_b); }
-    __device__ __forceinline__ bool used_by(int x, int i) const {
-        if (i < n_sel_b) return x == 0 ? (i < n_sel_a) : true;
-        const int m = loc_m(i);
-        return x == 0 ? (m <= m0 + 1) : (m >= m0 + 1);
+// Q K^T runs three items ahead of P V: P_A V, Q_B K^T of B's next tile, P_B V, Q_A K^T of A's next but one, and so on.
+// S of A's next tile is then complete when its softmax warps come back for it, and where S_A and S_B share their place
+// the warps of A have read theirs by the time B's is to be formed.  What bounds the kernel is then the softmax warps'
+// arithmetic, two of them per scheduler (issue slots 49 %, special-function unit 45 %, tensor pipe 62 %), and for short
+// streams the start and the end of a CTA.  With P over S, S of a tile waited for the softmax warps of the tile before
+// and these for it: 32768 tokens x 64 heads, d = 128, every token kept 15.07 ms a call (now 14.3), a quarter 5.99 (5.6),
+// 131072 x 32, capped at 896, 8.53 (7.65); 4096 x 128, d = 64, every token 554 us (512), a quarter 588 (560).  Two
+// threads per row instead of one (16 softmax warps) were slower by 10 %: the stream's bookkeeping doubles.
+template <int D, bool kPair, class TellPeer>
+__device__ __forceinline__ void mma_role(const Stream &st, const AttnBars &bar, uint8_t *smem, const uint32_t tmem_base,
+                                         volatile int *abort_flag, int *status, TellPeer tell_peer) {
+    using P = AttnPlan<D, kPair>;
+    using TM = TmemPlan<D>;
+    constexpr int kM = kPair ? 2 * kBlockM : kBlockM, kStages = P::kStages, kAhead = 3;
+    constexpr uint32_t idesc_qk = make_idesc(kM, kBlockN, false);
+    constexpr uint32_t idesc_pv = make_idesc(kM, D, true);
+    const bool leader = elect_one();
+    bool ok = mbar_wait(bar.q_full, 0, abort_flag, status, 4);
+    tc_fence_after();
+    // descriptors as low words: a k-step adds a constant
+    const uint32_t q_lo0 = desc_lo(smem_u32(smem + P::kQ), 0);
+    const uint32_t k_lo0 = desc_lo(smem_u32(smem + P::kK), 0);
+    const uint32_t v_lo0 = desc_lo(smem_u32(smem + P::kV), kBlockN * 128);
+    auto wait = [&](uint64_t *b, int parity, int where) {
+        if (ok) ok = mbar_wait(b, (uint32_t)parity, abort_flag, status, where);
+    };
+    auto commit = [&](uint64_t *b) {
+        if constexpr (kPair) tc_commit_pair(b, 3);
+        else tc_commit(b);
+    };
+    // A place in the order of the products: query tile x, its k-th tile, and the ring stage of that.
+    const int n_items = 2 * st.n_shared + st.n_a + st.n_b, turns = min(st.n_a, st.n_b), x_last = st.n_a > st.n_b ? 0 : 1;
+    struct Item {
+        int m, x, k;
+        RingPos pos;
+    };
+    auto advance = [&](Item &it) {
+        ++it.m;
+        if (it.m < 2 * st.n_shared) {
+            it.x ^= 1;
+            if (it.x == 1) return;   // (both query tiles use the entry)
+            ++it.k;
+        } else {
+            const int s = it.m - 2 * st.n_shared;
+            it.x = s < 2 * turns ? s & 1 : x_last;
+            it.k = st.n_shared + (s < 2 * turns ? s >> 1 : s - turns);
+        }
+        it.pos.next(kStages);
+    };
+    Item qk{0, 0, 0, {0, 0}}, pv{0, 0, 0, {0, 0}};
+    int x_prev = 0, k_prev = 0;   // of the item whose S was formed last
+    auto issue_qk = [&]() {
+        // K and V of the entry have arrived (B follows A on the entries that they share)
+        if (qk.m >= 2 * st.n_shared || qk.x == 0) wait(bar.kv_full + qk.pos.stage, qk.pos.parity, 7);
+        // the place of S is free: its last tile has been read
+        if constexpr (TM::kOneS) {
+            if (qk.m > 0) wait(bar.s_free + x_prev, k_prev & 1, 3);
+        } else {
+            if (qk.k > 0) wait(bar.s_free + qk.x, (qk.k - 1) & 1, 3);
+        }
+        tc_fence_after();
+        const uint32_t q_lo = q_lo0 + qk.x * (P::kQTile >> 4), k_lo = k_lo0 + qk.pos.stage * (P::kKTile >> 4), d_s = tmem_base + TM::s(qk.x);
+        if (leader && ok) {
+#pragma unroll
+            for (int j = 0; j < D / 16; ++j) {
+                // k-step of 16 elements: 32 bytes within a 64-element swizzle atom; atoms are 128 rows apart in a Q
+                // tile, and in a K tile as many as the CTA holds
+                const uint32_t off_q = ((j / 4) * (kBlockM * 128) + (j % 4) * 32) >> 4;
+                const uint32_t off_k = ((j / 4) * (P::kKRows * 128) + (j % 4) * 32) >> 4;
+                if constexpr (kPair) {
+                    if (j == 0) mma_ss_lo_pair<idesc_qk, 0>(d_s, q_lo, k_lo);
+                    else mma_ss_lo_pair<idesc_qk, 1>(d_s, q_lo + off_q, k_lo + off_k);
+                } else {
+                    if (j == 0) mma_ss_lo<idesc_qk, 0>(d_s, q_lo, k_lo);
+                    else mma_ss_lo<idesc_qk, 1>(d_s, q_lo + off_q, k_lo + off_k);
+                }
+            }
+            commit(bar.s_full + qk.x);
+        }
+        x_prev = qk.x;
+        k_prev = qk.k;
+        advance(qk);
+    };
+    auto issue_pv = [&]() {
+        const uint32_t v_lo = v_lo0 + pv.pos.stage * (P::kVTile >> 4), d_o = tmem_base + TM::o(pv.x), a_p = tmem_base + TM::p(pv.x);
+        const uint32_t acc0 = pv.k > 0 ? 1u : 0u;
+        wait(bar.p_full + pv.x, pv.k & 1, 5);
+        tc_fence_after();
+        if (leader && ok) {
+#pragma unroll
+            for (int j = 0; j < 8; ++j) {   // 16 keys a step
+                if constexpr (kPair) mma_ts_lo_pair<idesc_pv>(d_o, a_p + j * 8, v_lo + j * (16 * 128 >> 4), j == 0 ? acc0 : 1u);
+                else mma_ts_lo<idesc_pv>(d_o, a_p + j * 8, v_lo + j * (16 * 128 >> 4), j == 0 ? acc0 : 1u);
+            }
+            commit(bar.pv_done + pv.x);
+        }
+        advance(pv);
+    };
+    for (int m = 0; m < min(kAhead, n_items); ++m) issue_qk();
+    while (pv.m < n_items) {
+        issue_pv();
+        if (qk.m < n_items) issue_qk();
     }
-};
+    if (!__all_sync(0xffffffffu, ok) && leader) {  // no MMA may still be running when tensor memory is freed
+        if constexpr (kPair) {
+            tell_peer();
+            tc_commit_pair_local(bar.drain);
+        } else {
+            tc_commit(bar.drain);
+        }
+        mbar_wait_drain(bar.drain, 0);
+    }
+}
 
-template <int D>
-__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-sa_merge_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ksel,
-                     const __grid_constant__ CUtensorMap tm_vsel, const __nv_bfloat16 *y_part,
-                     const float *d_part, int n_parts, __nv_bfloat16 *Y, int *status, int H, int Hkv, int N,
-                     int C, int lam, int budget, int sel_rows, int sel_identity, float scale_log2, int n_pairs, int n_heads,
-                     int set_heads) {
-    grid_dep_wait();
-    grid_dep_launch();
-    using P = PairPlan<D>;
+// Softmax-attention branch and merge for rows [R0, R0 + 256) (a pair: 512) of one (batch, head).
+template <int D, bool kPair>
+__device__ __forceinline__ void attention_body(const CUtensorMap &tm_q, const CUtensorMap &tm_k, const CUtensorMap &tm_v,
+                                               const CUtensorMap &tm_ksel, const CUtensorMap &tm_vsel, const __nv_bfloat16 *y_part,
+                                               const float *d_part, int n_parts, __nv_bfloat16 *Y, int *status, int H, int Hkv, int N,
+                                               int C, int lam, int budget, int sel_rows, int sel_identity, float scale_log2,
+                                               int n_blocks, int n_heads, int set_heads) {
+    using P = AttnPlan<D, kPair>;
+    constexpr int kCtas = kPair ? 2 : 1, kRows = kCtas * kBlockM;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-    uint64_t *bars = reinterpret_cast<uint64_t *>(smem + P::kBar);
-    uint64_t *q_full = bars;
-    uint64_t *k_full = bars + 1, *k_empty = k_full + P::kKStages;
-    uint64_t *v_full = k_empty + P::kKStages, *v_empty = v_full + P::kVStages;
-    uint64_t *s_full = v_empty + P::kVStages;  // [2]
-    uint64_t *p_half = s_full + 2;             // [2][2]
-    uint64_t *o_final = p_half + 4;            // [2]
-    uint64_t *drain = o_final + 2;
+    const AttnBars bar = AttnBars::at(smem, P{});
     uint32_t *tmem_base_slot = reinterpret_cast<uint32_t *>(smem + P::kMisc);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + P::kMisc + 4);
     volatile int *failed_before = reinterpret_cast<volatile int *>(smem + P::kMisc + 8);
@@ -685,249 +651,131 @@ sa_merge_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
     // (warp index and cluster rank through a shuffle / from the block index: values the compiler knows to be
     // the same in all lanes)
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
-    const uint32_t rank = blockIdx.x & 1u, peer = rank ^ 1u;
-    int pb, bh;
-    row_block(blockIdx.x >> 1, n_pairs, n_heads, set_heads, pb, bh);
+    const uint32_t rank = kPair ? blockIdx.x & 1u : 0u, peer = rank ^ 1u;
+    int rb, bh;
+    row_block(kPair ? blockIdx.x >> 1 : blockIdx.x, n_blocks, n_heads, set_heads, rb, bh);
     const int b = bh / H, h = bh % H, kvh = h / (H / Hkv);
-    const int R0 = pb * 4 * kBlockM;
-
-    PairStream st;
-    st.m0 = R0 / kBlockN;
-    st.m_first = st.m0 - (st.m0 > 0 ? 1 : 0);
-    st.has_b = (R0 + 2 * kBlockM) < N;
-    {
-        const int last_a = min(R0 + 2 * kBlockM - 1, N - 1), last_b = min(R0 + 4 * kBlockM - 1, N - 1);
-        st.sel_first = sel_start(sel_limit(R0, C, lam), budget) / kBlockN;   // the pair's first row sees the oldest entries
-        st.n_sel_a = max((sel_limit(last_a, C, lam) + kBlockN - 1) / kBlockN - st.sel_first, 0);
-        st.n_sel_b = st.has_b ? max((sel_limit(last_b, C, lam) + kBlockN - 1) / kBlockN - st.sel_first, 0) : st.n_sel_a;
-        const int m_last = min(st.m0 + (st.has_b ? 3 : 1), (N - 1) / kBlockN);
-        st.n_tiles = st.n_sel_b + (m_last - st.m_first + 1);
-    }
+    const int R0 = rb * 2 * kRows;
+    const Stream st = make_stream(R0, kRows, N, C, lam, budget);
+    auto sync_all = [&]() {
+        if constexpr (kPair) cluster_sync_all();
+        else __syncthreads();
+    };
 
     if (threadIdx.x == 0) {
-        mbar_init(q_full, 1);
-        for (int i = 0; i < P::kKStages; ++i) { mbar_init(k_full + i, 1); mbar_init(k_empty + i, 2); }
-        for (int i = 0; i < P::kVStages; ++i) { mbar_init(v_full + i, 1); mbar_init(v_empty + i, 2); }
-        for (int i = 0; i < 2; ++i) { mbar_init(s_full + i, 1); mbar_init(o_final + i, 1); }
-        for (int i = 0; i < 4; ++i) mbar_init(p_half + i, 8);  // one arrival per softmax warp of either CTA
-        mbar_init(drain, 1);
+        mbar_init(bar.q_full, 1);
+        for (int i = 0; i < P::kStages; ++i) {
+            mbar_init(bar.kv_full + i, 1);
+            mbar_init(bar.kv_empty + i, 2);   // one share per query tile
+        }
+        for (int i = 0; i < 2; ++i) {
+            mbar_init(bar.s_full + i, 1);
+            mbar_init(bar.s_free + i, kCtas * 4);   // one arrival per softmax warp of the query tile
+            mbar_init(bar.p_full + i, kCtas * 4);
+            mbar_init(bar.pv_done + i, 1);
+        }
+        mbar_init(bar.drain, 1);
         *abort_flag = 0;
-        *failed_before = 0;
+        // A CTA that starts after another one has reported a failure does nothing; in a pair the first decides for both.
+        if (!kPair || rank == 0) *failed_before = *reinterpret_cast<volatile int *>(status) != 0;
         fence_barrier_init();
     }
     // The peer's barriers exist and its shared memory may be written from here on.
-    cluster_sync_all();
-    // A pair that starts after some CTA has reported a failure does nothing; rank 0 decides for both.
-    if (threadIdx.x == 0 && rank == 0) {
-        const int seen = *reinterpret_cast<volatile int *>(status) != 0;
-        *failed_before = seen;
-        st_cluster_u32(mapa(smem_u32(const_cast<int *>(failed_before)), 1), (uint32_t)seen);
+    sync_all();
+    if constexpr (kPair) {
+        if (threadIdx.x == 0 && rank == 0)
+            st_cluster_u32(mapa(smem_u32(const_cast<int *>(failed_before)), 1), (uint32_t)*failed_before);
+        cluster_sync_all();
     }
-    cluster_sync_all();
     if (*failed_before) return;
-    if (warp == 1) {
-        tmem_alloc_pair(tmem_base_slot, 512);
-        tmem_relinquish_pair();
+    if (warp == kMmaWarp) {
+        if constexpr (kPair) {
+            tmem_alloc_pair(tmem_base_slot, 512);
+            tmem_relinquish_pair();
+        } else {
+            tmem_alloc(tmem_base_slot, 512);
+            tmem_relinquish();
+        }
     }
     tc_fence_before();
-    cluster_sync_all();   // both CTAs hold their tensor memory before the first instruction of the pair
+    sync_all();   // (both CTAs of a pair hold their tensor memory before its first instruction)
     tc_fence_after();
     const uint32_t tmem_base = __shfl_sync(0xffffffffu, *tmem_base_slot, 0);
-    auto col_s = [](int x) -> uint32_t { return (uint32_t)x * 128u; };
-    auto col_o = [](int x) -> uint32_t { return 256u + (uint32_t)x * (uint32_t)D; };
     // a role that gives up tells the other CTA, whose waits would otherwise run to their own limit
     auto tell_peer = [&]() { st_cluster_u32(mapa(smem_u32(const_cast<int *>(abort_flag)), peer), 1u); };
 
-    if (warp < 4) {
-    reg_dec<72>();
-    if (warp == 0) {
-        // ------------------------------------------------------------ TMA producer (both CTAs)
-        if (lane == 0) {
-            const uint32_t q_full0 = mapa(smem_u32(q_full), 0), k_full0 = mapa(smem_u32(k_full), 0),
-                           v_full0 = mapa(smem_u32(v_full), 0);
-            const int n_q = st.has_b ? 2 : 1;
-            const int q_row = bh * N + R0 + (int)rank * kBlockM;
-            if (rank == 0) mbar_expect_tx(q_full, 2 * n_q * P::kQTile);   // both CTAs' tiles
-            for (int x = 0; x < n_q; ++x)
-                for (int half = 0; half < D / 64; ++half)
-                    tma_load_2d_pair(smem + P::kQ + x * P::kQTile + half * (kBlockM * 128), &tm_q, q_full0, half * 64,
-                                     q_row + x * 2 * kBlockM);
-            const int sel_base = sel_identity ? (b * Hkv + kvh) * N : bh * sel_rows;
-            bool ok = true;
-            int armed_k = 0, armed_v = 0, spins = 0;
-            long long t0 = clock64();
-            while (armed_k < st.n_tiles || armed_v < st.n_tiles) {
-                bool progressed = false;
-                if (armed_k < st.n_tiles) {
-                    const int i = armed_k, ks = i % P::kKStages;
-                    if (mbar_try_wait(k_empty + ks, ((i / P::kKStages) & 1) ^ 1)) {
-                        const bool sel = st.is_sel(i);
-                        const int row = (sel ? sel_base + (st.sel_first + i) * kBlockN : (b * Hkv + kvh) * N + st.loc_m(i) * kBlockN) +
-                                        (int)rank * (kBlockN / 2);   // this CTA's 64 keys
-                        if (rank == 0) mbar_expect_tx(k_full + ks, 2 * P::kKHalf);
-                        for (int half = 0; half < D / 64; ++half)
-                            tma_load_2d_pair(smem + P::kK + ks * P::kKHalf + half * ((kBlockN / 2) * 128), sel ? &tm_ksel : &tm_k,
-                                             k_full0 + ks * 8, half * 64, row);
-                        ++armed_k;
-                        progressed = true;
-                    }
-                }
-                if (armed_v < st.n_tiles) {
-                    const int i = armed_v, vs = i % P::kVStages;
-                    if (mbar_try_wait(v_empty + vs, ((i / P::kVStages) & 1) ^ 1)) {
-                        const bool sel = st.is_sel(i);
-                        const int row = sel ? sel_base + (st.sel_first + i) * kBlockN : (b * Hkv + kvh) * N + st.loc_m(i) * kBlockN;
-                        if (rank == 0) mbar_expect_tx(v_full + vs, 2 * P::kVHalf);
-                        for (int q = 0; q < D / 128; ++q)           // this CTA's D / 2 value columns, 64 at a time
-                            tma_load_2d_pair(smem + P::kV + vs * P::kVHalf + q * (kBlockN * 128), sel ? &tm_vsel : &tm_v,
-                                             v_full0 + vs * 8, (int)rank * (D / 2) + q * 64, row);
-                        ++armed_v;
-                        progressed = true;
-                    }
-                }
-                if (progressed) {
-                    spins = 0;
-                } else if ((++spins & 1023) == 0) {
-                    if (spins == 1024) t0 = clock64();
-                    if (*abort_flag) { ok = false; break; }
-                    if (clock64() - t0 > kWaitLimitCycles) {
-                        *abort_flag = 1;
-                        report_status(status, STILL_ERR_DEVICE_TIMEOUT, 51);
-                        ok = false;
-                        break;
-                    }
-                }
-            }
-            if (!ok) {
-                tell_peer();
-                // leave no copy in flight behind: rank 0 waits (bounded) for the last stages armed, which count
-                // both CTAs' bytes; rank 1, whose copies complete on rank 0's barriers, waits out a fixed
-                // stretch that is long against a tile load
-                if (rank == 0) {
-                    if (armed_k > 0) mbar_wait_drain(k_full + (armed_k - 1) % P::kKStages, ((armed_k - 1) / P::kKStages) & 1);
-                    if (armed_v > 0) mbar_wait_drain(v_full + (armed_v - 1) % P::kVStages, ((armed_v - 1) / P::kVStages) & 1);
-                } else {
-                    const long long t1 = clock64();
-                    while (clock64() - t1 < 200000) {}
-                }
-            }
+    // Registers move from the last four warps to the softmax warps, whose threads hold a row of S (per scheduler: 2 x 208 + 88
+    // registers for its three warps, of the 3 x 168 that the CTA was launched with).
+    if (warp >= kProducerWarp) {
+        reg_dec<88>();
+        if (warp == kProducerWarp) {
+            // With topk = chunk every token is selected and the compacted arrays would be copies of K / V: the salient
+            // prefix is then read from K / V themselves (tm_ksel / tm_vsel alias tm_k / tm_v).
+            const int kv_row0 = (b * Hkv + kvh) * N;
+            if (lane == 0)
+                producer_role<D, kPair>(st, bar, smem, rank, tm_q, tm_k, tm_v, tm_ksel, tm_vsel, bh * N + R0, kv_row0,
+                                        sel_identity ? kv_row0 : bh * sel_rows, abort_flag, status, tell_peer);
+        } else if (warp == kMmaWarp && rank == 0) {
+            mma_role<D, kPair>(st, bar, smem, tmem_base, abort_flag, status, tell_peer);
         }
-    } else if (warp == 1 && rank == 0) {
-        // ------------------------------------------------------------ MMA issuer (rank 0 only)
-        // The whole warp walks the stream and waits on the barriers; one elected lane issues.  Kept this way,
-        // control flow and every descriptor are the same in all lanes, which lets them live in the warp's
-        // uniform registers, where the tensor-core instructions take their operands from.  (With a single lane
-        // in a divergent branch each instruction cost that lane 55 - 80 cycles of operand marshalling, whatever
-        // the instruction's size, and the tensor pipe starved behind it.)  A failed wait does not leave the loop:
-        // it switches off the remaining waits and instructions, and the loop runs out.
-        {
-            const bool leader = elect_one();
-            constexpr uint32_t idesc_qk = make_idesc(2 * kBlockM, kBlockN, false);
-            constexpr uint32_t idesc_pv = make_idesc(2 * kBlockM, D, true);
-            bool ok = mbar_wait(q_full, 0, abort_flag, status, 54);
-            tc_fence_after();
-            const uint32_t q_lo0 = desc_lo(smem_u32(smem + P::kQ), 0);
-            const uint32_t k_lo0 = desc_lo(smem_u32(smem + P::kK), 0);
-            const uint32_t v_lo0 = desc_lo(smem_u32(smem + P::kV), kBlockN * 128);
-            const uint32_t k_empty1 = mapa(smem_u32(k_empty), 1), v_empty1 = mapa(smem_u32(v_empty), 1);
-            int pending[2] = {-1, -1};
-            int n_done[2] = {0, 0};
-            auto wait = [&](uint64_t *bar, int parity, int where) {
-                if (ok) ok = mbar_wait(bar, (uint32_t)parity, abort_flag, status, where);
-            };
-            auto issue_pv = [&](int x, int ip) {
-                const int vs = ip % P::kVStages;
-                wait(v_full + vs, (ip / P::kVStages) & 1, 56);
-                wait(p_half + 2 * x, n_done[x] & 1, 55);
-                tc_fence_after();
-                const uint32_t v_lo = v_lo0 + vs * (P::kVHalf >> 4);
-                const uint32_t d_o = tmem_base + col_o(x), a_p = tmem_base + col_s(x);
-                const uint32_t acc0 = n_done[x] > 0 ? 1u : 0u;
-                if (leader && ok) {
-                    mma_ts_lo_pair<idesc_pv>(d_o, a_p, v_lo, acc0);
-#pragma unroll
-                    for (int k = 1; k < kBlockN / 32; ++k)
-                        mma_ts_lo_pair<idesc_pv>(d_o, a_p + k * 8, v_lo + k * (16 * 128 >> 4), 1u);
-                }
-                wait(p_half + 2 * x + 1, n_done[x] & 1, 55);
-                tc_fence_after();
-                if (leader && ok) {
-#pragma unroll
-                    for (int k = kBlockN / 32; k < kBlockN / 16; ++k)
-                        mma_ts_lo_pair<idesc_pv>(d_o, a_p + k * 8, v_lo + k * (16 * 128 >> 4), 1u);
-                }
-                ++n_done[x];
-            };
-            for (int i = 0; i < st.n_tiles; ++i) {
-                const int ks = i % P::kKStages;
-                wait(k_full + ks, (i / P::kKStages) & 1, 57);
-                tc_fence_after();
-                const uint32_t k_lo = k_lo0 + ks * (P::kKHalf >> 4);
-#pragma unroll
-                for (int x = 0; x < 2; ++x) {
-                    const bool present = (x == 0) || st.has_b;
-                    if (present && st.used_by(x, i)) {
-                        if (pending[x] >= 0) {
-                            const int ip = pending[x];
-                            issue_pv(x, ip);
-                            // a V stage is released by two arrivals per CTA: pay the other tile's share if it skipped ip
-                            if (leader && ok && !(((1 - x) == 0 || st.has_b) && st.used_by(1 - x, ip))) {
-                                mbar_arrive(v_empty + ip % P::kVStages);
-                                mbar_arrive_cluster(v_empty1 + (ip % P::kVStages) * 8);
-                            }
-                        }
-                        const uint32_t q_lo = q_lo0 + x * (P::kQTile >> 4), d_s = tmem_base + col_s(x);
-                        if (leader && ok) {
-                            mma_ss_lo_pair<idesc_qk, 0>(d_s, q_lo, k_lo);
-#pragma unroll
-                            for (int k = 1; k < D / 16; ++k) {
-                                // k-step of 16 elements: 32 bytes within a 64-element swizzle atom; atoms are 128
-                                // rows apart in a Q tile, 64 rows apart in a CTA's half of a K tile
-                                const uint32_t off_q = ((k / 4) * (kBlockM * 128) + (k % 4) * 32) >> 4;
-                                const uint32_t off_k = ((k / 4) * ((kBlockN / 2) * 128) + (k % 4) * 32) >> 4;
-                                mma_ss_lo_pair<idesc_qk, 1>(d_s, q_lo + off_q, k_lo + off_k);
-                            }
-                            tc_commit_pair(s_full + x, 3);
-                        }
-                        pending[x] = i;
-                    } else if (leader && ok) {
-                        mbar_arrive(k_empty + ks);  // the share of a tile that skips this stream tile, in both CTAs
-                        mbar_arrive_cluster(k_empty1 + ks * 8);
-                    }
-                }
-            }
-#pragma unroll
-            for (int x = 0; x < 2; ++x) {
-                if (pending[x] >= 0) {
-                    issue_pv(x, pending[x]);
-                    if (leader && ok) tc_commit_pair(o_final + x, 3);
-                }
-            }
-            if (!__all_sync(0xffffffffu, ok) && leader) {  // no MMA may still be running when tensor memory is freed
-                tell_peer();
-                tc_commit_pair_local(drain);
-                mbar_wait_drain(drain, 0);
-            }
-        }
-    }
     } else {
-        reg_inc<216>();
-        // ------------------------------------------------------------ softmax + epilogue (both CTAs)
-        const int x = (warp - 4) >> 2;                 // 0: tile A, 1: tile B
-        softmax_role<D, P::kKStages, P::kVStages, true, STILL_POLY_OF4>(st, x, R0 + x * 2 * kBlockM + (int)rank * kBlockM, tmem_base, s_full,
-                                                        k_empty, v_empty, p_half, mapa(smem_u32(p_half), 0), o_final,
-                                                        abort_flag, status, smem + P::kQ + x * P::kQTile, y_part, d_part, n_parts,
-                                                        (long long)n_heads * N * D, (long long)n_heads * N, Y, bh, N, C, lam,
-                                                        budget, scale_log2);
-        if (*abort_flag) tell_peer();
+        reg_inc<208>();
+        const int x = warp >> 2;                       // 0: tile A, 1: tile B
+        softmax_role<D, kPair>(st, bar, x, R0 + (x * kCtas + (int)rank) * kBlockM, tmem_base, abort_flag, status,
+                                               smem + P::kQ + x * P::kQTile, y_part, d_part, n_parts, (long long)n_heads * N * D, (long long)n_heads * N, Y, bh, N,
+                                               C, lam, budget, scale_log2);
+        if constexpr (kPair) {
+            if (*abort_flag) tell_peer();
+        }
     }
-    // Nobody touches the peer's shared memory or tensor memory after this point.
+    // (Of a pair nobody touches the peer's shared memory or tensor memory after this point.)
     tc_fence_before();
-    cluster_sync_all();
-    if (warp == 1) {
+    sync_all();
+    if (warp == kMmaWarp) {
         tc_fence_after();
-        tmem_dealloc_pair(tmem_base, 512);
+        if constexpr (kPair) tmem_dealloc_pair(tmem_base, 512);
+        else tmem_dealloc(tmem_base, 512);
     }
+}
+
+template <int D>
+__global__ void __launch_bounds__(kThreads, 1)
+sa_merge_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+                   const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ksel,
+                   const __grid_constant__ CUtensorMap tm_vsel, const __nv_bfloat16 *y_part, const float *d_part, int n_parts,
+                   __nv_bfloat16 *Y, int *status, int H, int Hkv, int N, int C, int lam, int budget, int sel_rows, int sel_identity,
+                   float scale_log2, int n_blocks, int n_heads, int set_heads) {
+    grid_dep_wait();
+    grid_dep_launch();
+    attention_body<D, false>(tm_q, tm_k, tm_v, tm_ksel, tm_vsel, y_part, d_part, n_parts, Y, status, H, Hkv, N, C, lam, budget, sel_rows,
+                             sel_identity, scale_log2, n_blocks, n_heads, set_heads);
+}
+
+// The same branch on CTA pairs (head dim 128): two CTAs of a cluster work on 512 consecutive query rows of
+// one (batch, head) with UMMAs of the cta_group::2 form.  Query tile X of the pair is 256 rows -- rows
+// [R0 + 256 X + 128 r, + 128) belong to the CTA of cluster rank r -- and one instruction, issued by a thread
+// of rank 0, computes S_X = Q_X K^T (or O_X += P_X V) for both CTAs.  Each CTA keeps only its half of every
+// key tile in shared memory: 64 of the 128 keys of K (the B operand of Q K^T is split along N) and 64 of the
+// 128 value columns of V (likewise for P V); the tensor cores of both SMs read both halves.  Per FLOP a CTA
+// therefore pulls half the K / V bytes from L2 and reads a quarter less shared memory than a CTA working
+// alone.
+//
+// Who signals whom.  K / V / Q tiles: every CTA loads its halves into its own shared memory with plain TMA
+// loads (no multicast) whose byte counts complete on the full-barriers of rank 0, where the issuing thread
+// waits.  S_X ready, P_X V done: one tcgen05.commit arrives on the barrier of both CTAs.  S_X read, P_X written: the
+// softmax warps of both CTAs arrive on rank 0's barriers.  Ring stages are released locally: what a CTA's softmax
+// warps see completed has completed in both CTAs.
+template <int D>
+__global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
+sa_merge_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
+                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ksel,
+                     const __grid_constant__ CUtensorMap tm_vsel, const __nv_bfloat16 *y_part, const float *d_part, int n_parts,
+                     __nv_bfloat16 *Y, int *status, int H, int Hkv, int N, int C, int lam, int budget, int sel_rows, int sel_identity,
+                     float scale_log2, int n_blocks, int n_heads, int set_heads) {
+    grid_dep_wait();
+    grid_dep_launch();
+    attention_body<D, true>(tm_q, tm_k, tm_v, tm_ksel, tm_vsel, y_part, d_part, n_parts, Y, status, H, Hkv, N, C, lam, budget, sel_rows,
+                            sel_identity, scale_log2, n_blocks, n_heads, set_heads);
 }
 
 // ---------------------------------------------------------------------------
@@ -1312,20 +1160,20 @@ int launch_tc(const still_params_t *p, long long N, const void *Q, const void *K
     const int set_heads = set_of_heads(BH, rep, ((identity ? 0 : sel_rows) + N / rep + 1) * D * 4);
     if constexpr (kPair) {
         const int n_pairs = (int)((N + 4 * kBlockM - 1) / (4 * kBlockM));
-        if (ensure_dynamic_smem((const void *)sa_merge_pair_kernel<D>, PairPlan<D>::kAlloc) != cudaSuccess) return STILL_ERR_CUDA;
+        if (ensure_dynamic_smem((const void *)sa_merge_pair_kernel<D>, (AttnPlan<D, true>::kAlloc)) != cudaSuccess) return STILL_ERR_CUDA;
         dim3 grid((unsigned)(2 * n_pairs * BH));   // clusters of two
         profile_mark_begin(st);
-        const cudaError_t e = launch_dependent(sa_merge_pair_kernel<D>, grid, dim3(kThreads), PairPlan<D>::kAlloc, st,
+        const cudaError_t e = launch_dependent(sa_merge_pair_kernel<D>, grid, dim3(kThreads), (AttnPlan<D, true>::kAlloc), st,
             tq, tk, tv, tks, tvs, (const bf *)y_part, d_part, n_parts, (bf *)Y, status, p->H, p->Hkv, (int)N, p->chunk, p->topk, (int)p->max_salient, (int)sel_rows,
             identity ? 1 : 0, scale_log2, n_pairs, (int)BH, set_heads);
         profile_mark_end(st);
         if (e != cudaSuccess) return STILL_ERR_CUDA;
     } else {
         const int n_qblocks = (int)((N + 2 * kBlockM - 1) / (2 * kBlockM));
-        if (ensure_dynamic_smem((const void *)sa_merge_tc_kernel<D>, SmemPlan<D>::kAlloc) != cudaSuccess) return STILL_ERR_CUDA;
+        if (ensure_dynamic_smem((const void *)sa_merge_tc_kernel<D>, (AttnPlan<D, false>::kAlloc)) != cudaSuccess) return STILL_ERR_CUDA;
         dim3 grid((unsigned)(n_qblocks * BH));
         profile_mark_begin(st);
-        const cudaError_t e = launch_dependent(sa_merge_tc_kernel<D>, grid, dim3(kThreads), SmemPlan<D>::kAlloc, st,
+        const cudaError_t e = launch_dependent(sa_merge_tc_kernel<D>, grid, dim3(kThreads), (AttnPlan<D, false>::kAlloc), st,
             tq, tk, tv, tks, tvs, (const bf *)y_part, d_part, n_parts, (bf *)Y, status, p->H, p->Hkv, (int)N, p->chunk, p->topk, (int)p->max_salient, (int)sel_rows,
             identity ? 1 : 0, scale_log2, n_qblocks, (int)BH, set_heads);
         profile_mark_end(st);
