@@ -436,6 +436,9 @@ struct FusedPlan {
     static constexpr int kPhiQ = 64 * DF * 4;           // phi_q half of 64 tokens, fp32 (TF32 operand)
     static constexpr int kUTok = 32;                    // tokens per state-update tile
     static constexpr int kUStages = 4;                  // ring of update tiles (loads run this far ahead of the MMAs)
+    // ... of the pass that only sums, whose ring takes the room of W_q, Q and phi(Q) too: with four stages a tile cost it 920
+    // cycles, a quarter of a load's way from memory.  (131072 tokens x 32 heads, C = 128, capped at 896: 8.53 -> 8.20 ms a call.)
+    static constexpr int kMaxStages = 12;
     static constexpr int kPhiK = kUTok * DF * 2;        // phi_k half of an update tile, bf16
     static constexpr int kVt = kUTok * D * 2;           // V of an update tile
     static constexpr int kUStage = kPhiK + kVt;
@@ -447,12 +450,16 @@ struct FusedPlan {
     static constexpr int oZ = oDinv + 8 * 64 * 4;       // [4 map warps][d_f] z half of the chunk two back
     static constexpr int oStage = oZ + 4 * DF * 4;      // [64 tokens][d] bf16: the output of a sub-chunk on its way out
     static constexpr int oBar = oStage + 64 * D * 2;
-    static constexpr int kNumBars = 30;
+    static constexpr int kSumStages = (oDinv / kUStage) < kMaxStages ? oDinv / kUStage : kMaxStages;
+    static constexpr int kNumBars = 18 + 3 * kMaxStages;
     static constexpr int oMisc = oBar + kNumBars * 8;
     static constexpr int kTotal = oMisc + 16;
 };
 static_assert(FusedPlan<128, 128>::kTotal <= 232448 && FusedPlan<128, 64>::kTotal <= 232448 && FusedPlan<64, 64>::kTotal <= 232448,
               "fused scan: the shared-memory plan exceeds what a CTA can have");
+
+// What a launch of la_fused_kernel does (see there).
+enum LaMode { kFromSums = 0, kSumsOnly = 1, kFoldAll = 2 };
 
 template <int D, int DF>
 __global__ void __launch_bounds__(384, 1)
@@ -463,7 +470,7 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 const int32_t *sel_idx, const float *zpre, __nv_bfloat16 *y_part,
                 float *d_part, float *S_out, float *seg_sums, int *status, int H, int Hkv,
                 int N, int C, int lam, int window, long long part_stride_y, long long part_stride_d, int seg_chunks, int n_seg,
-                int sum_parts, int sums_only, int sel_rows) {
+                int sum_parts, int mode, int sel_rows) {
     grid_dep_wait();
     grid_dep_launch();
     using P = FusedPlan<D, DF>;
@@ -471,10 +478,36 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     extern __shared__ __align__(1024) uint8_t smem[];
     uint64_t *bars = reinterpret_cast<uint64_t *>(smem + P::oBar);
     uint64_t *w_full = bars, *x_full = bars + 1, *x_empty = bars + 2;
-    uint64_t *f_done = bars + 28, *f_free = bars + 3;   // [2] each: f of even / odd blocks
+    uint64_t *f_done = bars + 15, *f_free = bars + 3;   // [2] each: f of even / odd blocks
     uint64_t *pq_full = bars + 5, *pq_empty = bars + 7, *r_done = bars + 9, *out_free = bars + 11, *fin = bars + 13;
-    uint64_t *init_done = bars + 14, *u_full = bars + 15, *u_empty = u_full + P::kUStages, *u_masked = u_empty + P::kUStages;
-    constexpr int kUS = P::kUStages, kUTok = P::kUTok;
+    uint64_t *init_done = bars + 14, *u_full = bars + 18, *u_empty = u_full + P::kMaxStages, *u_masked = u_empty + P::kMaxStages;
+    constexpr int kUTok = P::kUTok;
+    const bool sums_only = mode == kSumsOnly;
+    const int n_stages = sums_only ? P::kSumStages : P::kUStages;
+    uint8_t *ring = smem + (sums_only ? 0 : P::oU);
+    // The ring stage of a tile, and the parity of its round; next: of the tile n further on (n <= n_stages).
+    struct Slot {
+        int stage, parity;
+        __device__ __forceinline__ void next(int n, int n_stages) {
+            stage += n;
+            if (stage >= n_stages) {
+                stage -= n_stages;
+                parity ^= 1;
+            }
+        }
+    };
+    // Chunk of a tile and its number among the chunk's (counted up from tile to tile: a division by the tiles of a chunk costs
+    // a single-thread role more than the tile's loads)
+    struct Tile {
+        int chunk, rt;
+        __device__ __forceinline__ void next(int n, int per_chunk) {
+            rt += n;
+            if (rt >= per_chunk) {
+                rt -= per_chunk;
+                ++chunk;
+            }
+        }
+    };
     uint32_t *tmem_base_slot = reinterpret_cast<uint32_t *>(smem + P::oMisc);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + P::oMisc + 8);
     float *dinv_ring = reinterpret_cast<float *>(smem + P::oDinv);
@@ -487,7 +520,8 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const int n_routed = Tn >= 3 ? Tn - 2 : 0;  // chunks whose tokens enter the state
     // The sequence is cut into n_seg segments of seg_chunks chunks (two-level scan): segment g answers the
     // sub-chunks [u_first, NU) and performs the updates that fall between them, starting from the sum of the
-    // earlier segments' updates (seg_sums, produced by a first pass of this kernel with sums_only set).
+    // earlier segments' updates (kFromSums: seg_sums, produced by a first pass of this kernel, kSumsOnly), or folding
+    // the chunks before it itself (kFoldAll, where they are few).
     // The first pass cuts every segment into sum_parts pieces, one CTA each (it has no scan to keep in order, and
     // the pieces fill the SMs that the n_seg - 1 summed segments alone would leave idle).
     const int seg = blockIdx.z;
@@ -505,9 +539,9 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const int su = C / kUTok;
     const int nl = sel_rows > 0 ? (lam + kUTok - 1) / kUTok : su;
     const int per_chunk = window > 0 ? su + nl : su;
-    const int nu0 = (u_first / sc - 2) * per_chunk;    // first update tile of the segment
-    const int n_upd = NU > u_first ? ((NU - 1) / sc - 1) * per_chunk - nu0 : 0;
-    const bool has_init = !sums_only && seg > 0;
+    const int chunk0 = mode == kFoldAll ? 0 : u_first / sc - 2;   // first chunk that the segment folds
+    const int n_upd = NU > u_first ? ((NU - 1) / sc - 1 - chunk0) * per_chunk : 0;
+    const bool has_init = mode == kFromSums && seg > 0;
     __nv_bfloat16 *y_out = y_part + (long long)half * part_stride_y;
     float *d_out = d_part + (long long)half * part_stride_d;
 
@@ -533,7 +567,7 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             mbar_init(r_done + i, 1);
             mbar_init(out_free + i, 4);
         }
-        for (int i = 0; i < kUS; ++i) {
+        for (int i = 0; i < P::kMaxStages; ++i) {
             mbar_init(u_full + i, 1);
             mbar_init(u_empty + i, 1);
             mbar_init(u_masked + i, 1);
@@ -569,6 +603,8 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 for (int a = 0; a < DF / 64; ++a) tma_load_2d(smem + P::oW + a * (D * 128), &tm_wq, w_full, a * 64, h * D);
             }
             int nu = 0, nx = 0, spins = 0;
+            Slot us{0, 0}, last{0, 0};
+            Tile ut{chunk0, 0};
             long long t0 = clock64();
             while (nu < n_upd || nx < n_blk) {
                 bool progressed = false;
@@ -579,21 +615,22 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     ++nx;
                     progressed = true;
                 }
-                if (nu < n_upd && mbar_try_wait(u_empty + nu % kUS, ((nu / kUS) & 1) ^ 1)) {
-                    uint8_t *stg = smem + P::oU + (nu % kUS) * P::kUStage;
-                    // tile a = nu0 + nu: chunk a / per_chunk, then which of its tiles; a leaving-tile reads the chunk
-                    // `window` back (before there is one, any valid tile: all its rows are zeroed)
-                    const int a_t = nu0 + nu, cc = a_t / per_chunk, rt = a_t % per_chunk;
-                    const int src = (rt >= su && cc >= window) ? cc - window : cc;
-                    const bool gathered = rt >= su && sel_rows > 0;
+                if (nu < n_upd && mbar_try_wait(u_empty + us.stage, us.parity ^ 1)) {
+                    uint8_t *stg = ring + us.stage * P::kUStage;
+                    // a leaving-tile reads the chunk `window` back (before there is one, any valid tile: all its rows are zeroed)
+                    const bool leaving = ut.rt >= su, gathered = leaving && sel_rows > 0;
+                    const int src = leaving && ut.chunk >= window ? ut.chunk - window : ut.chunk, tile = leaving ? ut.rt - su : ut.rt;
                     // first row of the tile: in phi(K) / V of the KV head, or in the head's gathered rows
-                    const int row = gathered ? bh * sel_rows + src * lam + (rt - su) * kUTok : kv_row0 + (src * su + rt % su) * kUTok;
+                    const int row = gathered ? bh * sel_rows + src * lam + tile * kUTok : kv_row0 + (src * su + tile) * kUTok;
                     const CUtensorMap *mp = gathered ? &tm_phiks : &tm_phik, *mv = gathered ? &tm_vs : &tm_v;
-                    mbar_expect_tx(u_full + nu % kUS, P::kUStage);
+                    mbar_expect_tx(u_full + us.stage, P::kUStage);
                     for (int a = 0; a < DF / 64; ++a)  // phi(K) half: MN-major, 64-feature atoms kUTok rows apart
-                        tma_load_2d(stg + a * (kUTok * 128), mp, u_full + nu % kUS, half * DF + a * 64, row);
+                        tma_load_2d(stg + a * (kUTok * 128), mp, u_full + us.stage, half * DF + a * 64, row);
                     for (int a = 0; a < D / 64; ++a)   // V: M-major A operand, 64-column atoms kUTok rows apart
-                        tma_load_2d(stg + P::kPhiK + a * (kUTok * 128), mv, u_full + nu % kUS, a * 64, row);
+                        tma_load_2d(stg + P::kPhiK + a * (kUTok * 128), mv, u_full + us.stage, a * 64, row);
+                    last = us;
+                    us.next(1, n_stages);
+                    ut.next(1, per_chunk);
                     ++nu;
                     progressed = true;
                 }
@@ -610,7 +647,7 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 }
             }
             if (*abort_flag) {  // leave no copy in flight behind
-                if (nu > 0) mbar_wait_drain(u_full + (nu - 1) % kUS, ((nu - 1) / kUS) & 1);
+                if (nu > 0) mbar_wait_drain(u_full + last.stage, last.parity);
                 if (nx > 0) mbar_wait_drain(x_full, (nx - 1) & 1);
                 if (n_blk > 0) mbar_wait_drain(w_full, 0);
             }
@@ -628,14 +665,15 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             constexpr uint32_t idesc_rd = make_idesc_tf32(128, 64);
             bool ok = true;
             int nu = 0, nq = 0, nx = 0;
+            Slot us{0, 0};
             auto wait = [&](uint64_t *bar, int parity, int where) {
                 if (ok) ok = mbar_wait(bar, (uint32_t)parity, abort_flag, status, where);
             };
             // descriptors as low words: a k-step adds a constant
             const uint32_t x_lo = desc_lo(smem_u32(smem + P::oX), 0), w_lo = desc_lo(smem_u32(smem + P::oW), D * 128);
             const uint32_t q_lo0 = desc_lo(smem_u32(smem + P::oQ), 0);
-            const uint32_t pk_lo0 = desc_lo(smem_u32(smem + P::oU), kUTok * 128);
-            const uint32_t v_lo0 = desc_lo(smem_u32(smem + P::oU + P::kPhiK), D == 128 ? kUTok * 128 : 0);
+            const uint32_t pk_lo0 = desc_lo(smem_u32(ring), kUTok * 128);
+            const uint32_t v_lo0 = desc_lo(smem_u32(ring + P::kPhiK), D == 128 ? kUTok * 128 : 0);
             // f = x W_q of block b_first + nx (the map warps have taken the previous f out of tensor memory)
             auto issue_f = [&]() {
                 if (nx == 0) wait(w_full, 0, 61);
@@ -659,22 +697,24 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 tc_fence_after();
             }
             auto issue_update = [&]() {
-                wait(u_masked + nu % kUS, (nu / kUS) & 1, 64);
+                wait(u_masked + us.stage, us.parity, 64);
                 tc_fence_after();
-                const uint32_t so = (uint32_t)(nu % kUS) * (P::kUStage >> 4);
+                const uint32_t so = (uint32_t)us.stage * (P::kUStage >> 4);
                 const uint32_t acc0 = (nu > 0 || has_init) ? 1u : 0u;
                 if (leader && ok) {
                     mma_ss_lo_acc<idesc_upd>(tmem_base + col_state, v_lo0 + so, pk_lo0 + so, acc0);
 #pragma unroll
                     for (int k = 1; k < kUTok / 16; ++k)   // 16 tokens per step: 16 rows of 128 bytes in both operands
                         mma_ss_lo_acc<idesc_upd>(tmem_base + col_state, v_lo0 + so + k * (2048 >> 4), pk_lo0 + so + k * (2048 >> 4), 1u);
-                    tc_commit(u_empty + nu % kUS);
+                    tc_commit(u_empty + us.stage);
                 }
+                us.next(1, n_stages);
                 ++nu;
             };
-            if (sums_only)
-                while (nu < n_upd) issue_update();
             if (NB > b_first) issue_f();
+            // what is folded ahead of the segment's first read-out: everything in a pass of sums
+            const int ahead = sums_only ? n_upd : min(n_upd, (u_first / sc - 2 - chunk0) * per_chunk);
+            while (nu < ahead) issue_update();
             for (int u = u_first; u < NU && !sums_only; ++u) {
                 if (u % sc == 0) {
                     // the chunk that has just left the local region: sub-chunks of chunk u / sc - 2
@@ -710,21 +750,20 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         // state.  The indices of a tile's chunk are requested one tile ahead (a round trip to L2 per tile would
         // otherwise pace the whole update path), and two warps take turns.
         bool ok = true;
-        // positions of the selected tokens of tile nu's chunk relative to the tile's first row (-1: none)
-        auto fetch = [&](int nu, int (&r)[4]) {
-            const int a_t = nu0 + nu, cc = a_t / per_chunk, rt = a_t % per_chunk, sub = rt % su;
-            const int chunk = rt >= su ? cc - window : cc;       // (chunk < 0: nothing leaves yet, every row is zeroed)
-            const bool need = !(rt >= su && sel_rows > 0);       // (a gathered tile needs no indices)
+        // positions of the selected tokens of a tile's chunk relative to the tile's first row (-1: none)
+        auto fetch = [&](bool live, const Tile &ut, int (&r)[4]) {
+            const bool leaving = ut.rt >= su;
+            const int chunk = leaving ? ut.chunk - window : ut.chunk;   // (chunk < 0: nothing leaves yet, every row is zeroed)
+            const int first = chunk * C + (leaving ? ut.rt - su : ut.rt) * kUTok;
+            const bool need = live && chunk >= 0 && !(leaving && sel_rows > 0);   // (a gathered tile needs no indices)
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
                 const int i = lane + 32 * q;
-                r[q] = (need && nu < n_upd && i < lam && chunk >= 0)
-                           ? sel_idx[((long long)bh * Tn + chunk) * lam + i] - (chunk * C + sub * kUTok) : -1;
+                r[q] = need && i < lam ? sel_idx[((long long)bh * Tn + chunk) * lam + i] - first : -1;
             }
         };
-        auto process = [&](int nu, const int (&sel)[4]) {
-            const int rt = (nu0 + nu) % per_chunk;
-            const bool leaving = rt >= su;                       // tile of the tokens that leave the salient cache
+        auto process = [&](const Slot &us, const Tile &ut, const int (&sel)[4]) {
+            const bool leaving = ut.rt >= su;                    // tile of the tokens that leave the salient cache
             // the selected rows of the tile as a 32-bit set
             uint32_t rows = 0u;
 #pragma unroll
@@ -734,16 +773,15 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             if (leaving) rows = ~rows;                           // rows to zero: the selected ones, or all the others
             if (leaving && sel_rows > 0) {
                 // gathered tile: its first `valid` rows are the chunk's leaving tokens, the rest belong to the next chunk
-                const int cw = (nu0 + nu) / per_chunk - window;
-                const int valid = cw < 0 ? 0 : min(kUTok, lam - (rt - su) * kUTok);
+                const int valid = ut.chunk < window ? 0 : min(kUTok, lam - (ut.rt - su) * kUTok);
                 rows = valid >= 32 ? 0u : ~((1u << valid) - 1u);
             }
-            if (ok) ok = mbar_wait(u_full + nu % kUS, (nu / kUS) & 1, abort_flag, status, 67);
+            if (ok) ok = mbar_wait(u_full + us.stage, us.parity, abort_flag, status, 67);
             ok = __all_sync(0xffffffffu, ok);
             if (ok) {
                 // A row is 128 bytes in each 64-feature atom.  Eight lanes clear one such line (all 32 banks, no
                 // conflict), so a store instruction clears the lines of four rows.
-                uint8_t *tile = smem + P::oU + (nu % kUS) * P::kUStage;
+                uint8_t *tile = ring + us.stage * P::kUStage;
 #pragma unroll
                 for (int it = 0; it < kUTok / 4; ++it) {
                     const int rz = it * 4 + (lane >> 3);
@@ -756,16 +794,30 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 fence_proxy_async();
             }
             __syncwarp();
-            if (lane == 0) mbar_arrive(u_masked + nu % kUS);
+            if (lane == 0) mbar_arrive(u_masked + us.stage);
         };
         // (two register sets that change roles: a copy from one to the other would wait for the loads)
         int sel_a[4], sel_b[4];
-        fetch(warp - 2, sel_a);
+        Slot us{0, 0};
+        Tile ut{chunk0, 0}, ft{chunk0, 0};   // of the next tile to process, and to fetch for
+        if (warp == 3) {
+            us.next(1, n_stages);
+            ut.next(1, per_chunk);
+            ft.next(1, per_chunk);
+        }
+        auto turn = [&](const int (&sel)[4]) {
+            process(us, ut, sel);
+            us.next(2, n_stages);
+            ut.next(2, per_chunk);
+        };
+        fetch(warp - 2 < n_upd, ft, sel_a);
         for (int nu = warp - 2; nu < n_upd; nu += 4) {
-            fetch(nu + 2, sel_b);
-            process(nu, sel_a);
-            fetch(nu + 4, sel_a);
-            if (nu + 2 < n_upd) process(nu + 2, sel_b);
+            ft.next(2, per_chunk);
+            fetch(nu + 2 < n_upd, ft, sel_b);
+            turn(sel_a);
+            ft.next(2, per_chunk);
+            fetch(nu + 4 < n_upd, ft, sel_a);
+            if (nu + 2 < n_upd) turn(sel_b);
         }
     }
     } else if (warp < 8) {
@@ -1102,6 +1154,12 @@ int launch_gather(const still_params_t *p, long long N, const void *K, const voi
                             N, p->topk, sel_rows, n_routed) == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
 }
 
+// Update tiles up to which every segment of the scan folds the chunks before it itself.  (us a call, folding again / a pass of
+// sums, a quarter kept: 32 heads, d = 128, 16 tiles 76.9 / 90.5, 32: 131.9 / 144.3, 48: 192.1 / 199.4, 64: 248.6 / 253.3, 96: 363.9 /
+// 360.9; d = 64, 64 tiles 168.5 / 170.3; C = 128, 64 tiles 258.4 / 261.5; 16 heads, 48 tiles 90.5 / 106.1, 96: 162.5 / 169.2,
+// 192: 315 / 290; 4 heads, d = 64, 96 tiles 93.9 / 78.7.)
+constexpr int kFoldAllTiles = 64;
+
 template <int D, int DF>
 int launch_fused(const still_params_t *p, long long N, const void *Q, const void *V, const void *G, const void *Wq,
                  const void *bq, const int32_t *sel_idx, const void *phiK, const float *zpre, void *y_part, float *d_part,
@@ -1129,14 +1187,17 @@ int launch_fused(const still_params_t *p, long long N, const void *Q, const void
     if (ensure_dynamic_smem((const void *)la_fused_kernel<D, DF>, Plan::kTotal) != cudaSuccess) return STILL_ERR_CUDA;
     int seg_chunks = 0;
     const int n_seg = tc_la_segments(p, N, &seg_chunks), parts = tc_la_sum_parts(seg_chunks);
-    for (int pass = n_seg > 1 ? 0 : 1; pass < 2; ++pass) {
+    // The chunks before the last segment are folded again by every segment where that is a short stretch of update tiles, and
+    // summed by a pass of its own where it is not.
+    const bool again = n_seg > 1 && (long long)(n_seg - 1) * seg_chunks * (p->chunk / Plan::kUTok) * (p->max_salient > 0 ? 2 : 1) <= kFoldAllTiles;
+    for (int pass = n_seg > 1 && !again ? 0 : 1; pass < 2; ++pass) {
         // pass 0 (only with several segments): the sum of every segment's own updates; pass 1: the scan proper
         dim3 grid((unsigned)BH, 2, (unsigned)(pass == 0 ? (n_seg - 1) * parts : n_seg));   // head, feature half, segment (piece)
         const cudaError_t e = launch_dependent(la_fused_kernel<D, DF>, grid, dim3(384), Plan::kTotal, st, tq, tw, tk, tv, tks, tvs, (const bf *)bq, (const bf *)G, sel_idx, zpre,
                                                                (bf *)y_part, d_part, S_out, seg_sums, status, p->H, p->Hkv, (int)N,
                                                                p->chunk, p->topk, p->topk > 0 ? (int)(p->max_salient / p->topk) : 0,
                                                                (long long)BH * N * D, (long long)BH * N,
-                                                               seg_chunks, n_seg, parts, pass == 0 ? 1 : 0, gathered ? (int)sel_rows : 0);
+                                                               seg_chunks, n_seg, parts, pass == 0 ? kSumsOnly : again ? kFoldAll : kFromSums, gathered ? (int)sel_rows : 0);
         if (e != cudaSuccess) return STILL_ERR_CUDA;
         ++*launches;
     }
