@@ -457,6 +457,8 @@ struct FusedPlan {
 };
 static_assert(FusedPlan<128, 128>::kTotal <= 232448 && FusedPlan<128, 64>::kTotal <= 232448 && FusedPlan<64, 64>::kTotal <= 232448,
               "fused scan: the shared-memory plan exceeds what a CTA can have");
+static_assert(FusedPlan<128, 128>::oStage % 1024 == 0 && FusedPlan<128, 64>::oStage % 1024 == 0 && FusedPlan<64, 64>::oStage % 1024 == 0,
+              "fused scan: the staging tile is swizzle-aligned");
 
 // What a launch of la_fused_kernel does (see there).
 enum LaMode { kFromSums = 0, kSumsOnly = 1, kFoldAll = 2 };
@@ -466,6 +468,7 @@ __global__ void __launch_bounds__(384, 1)
 la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_wq,
                 const __grid_constant__ CUtensorMap tm_phik, const __grid_constant__ CUtensorMap tm_v,
                 const __grid_constant__ CUtensorMap tm_phiks, const __grid_constant__ CUtensorMap tm_vs,
+                const __grid_constant__ CUtensorMap tm_y,
                 const __nv_bfloat16 *bq, const __nv_bfloat16 *G,
                 const int32_t *sel_idx, const float *zpre, __nv_bfloat16 *y_part,
                 float *d_part, float *S_out, float *seg_sums, int *status, int H, int Hkv,
@@ -878,31 +881,32 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             }
             if (ok) ok = mbar_wait(r_done + (nq & 1), (nq >> 1) & 1, abort_flag, status, 68);
             ok = __all_sync(0xffffffffu, ok);
+            // y_part[t][e] = N_part / D_part (times the gate): the read-out scaled by 1 / (e . z) of its token.  Tensor memory
+            // holds it by value column, y_part is token-major.  Read as fragments of 8 x 8 (value columns g and g + 8 of 16,
+            // tokens 8 i + 2 tig and + 1 in a thread), two tokens are a register of bf16, and stmatrix transposes on the way
+            // to shared memory: 8 stores a thread for a sub-chunk where a thread per value column needs 64 of two bytes.  Rows
+            // lie there as the tensor map has them (64 columns of 128 bytes, swizzled by the row), and one thread stores the
+            // tile.  The workers, which were as busy as the map warps (3300 cycles a sub-chunk), now wait for half of the
+            // time: 64 heads x 32768 tokens, a quarter kept, 6020 -> 5800 us a call.
+            uint32_t out[2][16];
+            uint8_t *stg = smem + P::oStage;
+            const bool has_rows = wq * 32 < D;   // (at d = 64 the upper lanes of the product repeat the lower)
             if (ok) {
                 tc_fence_after();
-                // y_part[t][e] = N_part / D_part (times the gate): the read-out scaled by 1 / (e . z) of its token.  A thread holds one value column of 64 tokens, but
-                // the rows of y_part are token-major and a store loop over tokens costs about a hundred clocks per
-                // instruction; so the tile is transposed through shared memory and leaves in 16-byte pieces.  Two
-                // rolled rounds of 32 tokens keep the instruction stream short; the scales of a round are loaded
-                // before its first store (shared-memory loads are kept behind earlier stores).
-                const float4 *dinv = reinterpret_cast<const float4 *>(dinv_ring + (u & 7) * 64);
-                __nv_bfloat16 *stg = reinterpret_cast<__nv_bfloat16 *>(smem + P::oStage);
-#pragma unroll 1
-                for (int hf = 0; hf < 2; ++hf) {
-                    uint32_t o[32];
-                    tmem_ld32(taddr + col_out + (nq & 1) * 64 + hf * 32, o);
-                    float4 sc4[8];
+                const float *dinv = dinv_ring + (u & 7) * 64 + 2 * (lane & 3);
+                if (has_rows) {
 #pragma unroll
-                    for (int t4 = 0; t4 < 8; ++t4) sc4[t4] = dinv[hf * 8 + t4];
-                    tmem_wait_ld();
-                    if (e < D) {
+                    for (int h16 = 0; h16 < 2; ++h16) {
+                        uint32_t o[32];
+                        tmem_ld_frag64(taddr + col_out + (nq & 1) * 64 + ((uint32_t)(h16 * 16) << 16), o);
+                        float2 sc2[8];
 #pragma unroll
-                        for (int t4 = 0; t4 < 8; ++t4) {
-                            __nv_bfloat16 *dst = stg + (hf * 32 + 4 * t4) * D + e;
-                            dst[0] = __float2bfloat16_rn(__uint_as_float(o[4 * t4]) * sc4[t4].x);
-                            dst[D] = __float2bfloat16_rn(__uint_as_float(o[4 * t4 + 1]) * sc4[t4].y);
-                            dst[2 * D] = __float2bfloat16_rn(__uint_as_float(o[4 * t4 + 2]) * sc4[t4].z);
-                            dst[3 * D] = __float2bfloat16_rn(__uint_as_float(o[4 * t4 + 3]) * sc4[t4].w);
+                        for (int i = 0; i < 8; ++i) sc2[i] = *reinterpret_cast<const float2 *>(dinv + 8 * i);
+                        tmem_wait_ld();
+#pragma unroll
+                        for (int i = 0; i < 8; ++i) {
+                            out[h16][2 * i] = pack_bf16(__uint_as_float(o[4 * i]) * sc2[i].x, __uint_as_float(o[4 * i + 1]) * sc2[i].y);
+                            out[h16][2 * i + 1] = pack_bf16(__uint_as_float(o[4 * i + 2]) * sc2[i].x, __uint_as_float(o[4 * i + 3]) * sc2[i].y);
                         }
                     }
                 }
@@ -910,38 +914,53 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 __syncwarp();
                 if (lane == 0) mbar_arrive(out_free + (nq & 1));
             }
+            if (tid == 0) bulk_store_wait_read();            // the store of the sub-chunk before has read the staging tile
             asm volatile("bar.sync 2, 128;" ::: "memory");   // the four worker warps (always, whatever `ok`)
+            if (ok && has_rows) {
+#pragma unroll
+                for (int h16 = 0; h16 < 2; ++h16)
+#pragma unroll
+                    for (int i = 0; i < 8; i += 2) {
+                        // this lane's row of the four matrices: tokens 8 i .. + 7 and + 8 .. + 15, columns 0-7 and 8-15 of the 16
+                        const int t = 8 * (i + (lane >> 4)) + (lane & 7), p = wq * 4 + h16 * 2 + ((lane >> 3) & 1);
+                        stmatrix_x4_trans(stg + (p >> 3) * (64 * 128) + t * 128 + (((p & 7) ^ (t & 7)) << 4), out[h16][2 * i],
+                                          out[h16][2 * i + 1], out[h16][2 * i + 2], out[h16][2 * i + 3]);
+                    }
+                fence_proxy_async();
+            }
+            asm volatile("bar.sync 2, 128;" ::: "memory");
             if (ok) {
                 const int base = u * 64;
-                auto piece = [&](int it, auto gated) {
-                    const int id = it * 128 + tid, t = id / kPiecesPerRow, c = id % kPiecesPerRow;
-                    if (base + t < N) {
-                        uint4 v = *reinterpret_cast<const uint4 *>(smem + P::oStage + (t * D + c * 8) * 2);
-                        if constexpr (decltype(gated)::value) {
-                            const uint4 gg = gate[it];
-                            const uint32_t vw[4] = {v.x, v.y, v.z, v.w}, gw[4] = {gg.x, gg.y, gg.z, gg.w};
-                            uint32_t rw[4];
+                if (G == nullptr && base + 64 <= N) {
+                    if (tid == 0) {
 #pragma unroll
-                            for (int q = 0; q < 4; ++q)
-                                rw[q] = pack_bf16(__uint_as_float(vw[q] << 16) * __uint_as_float(gw[q] << 16),
-                                                  __uint_as_float(vw[q] & 0xffff0000u) * __uint_as_float(gw[q] & 0xffff0000u));
-                            v = make_uint4(rw[0], rw[1], rw[2], rw[3]);
-                        }
-                        *reinterpret_cast<uint4 *>(y_out + ((long long)bh * N + base + t) * D + c * 8) = v;
+                        for (int a = 0; a < D / 64; ++a) tma_store_2d(&tm_y, stg + a * (64 * 128), a * 64, (int)((half * gridDim.x + bh) * N) + base);
+                        bulk_store_commit();
                     }
-                };
-                // (without a gate the loop stays short: the kernel is sensitive to its instruction footprint)
-                if (G != nullptr) {
+                } else {   // with a gate, and the last rows of a sequence
 #pragma unroll
-                    for (int it = 0; it < kPieces; ++it) piece(it, std::true_type{});
-                } else {
-#pragma unroll 2
-                    for (int it = 0; it < kPieces; ++it) piece(it, std::false_type{});
+                    for (int it = 0; it < kPieces; ++it) {
+                        const int id = it * 128 + tid, t = id / kPiecesPerRow, c = id % kPiecesPerRow;
+                        if (base + t < N) {
+                            uint4 v = *reinterpret_cast<const uint4 *>(stg + (c >> 3) * (64 * 128) + t * 128 + (((c & 7) ^ (t & 7)) << 4));
+                            if (G != nullptr) {
+                                const uint4 gg = gate[it];
+                                const uint32_t vw[4] = {v.x, v.y, v.z, v.w}, gw[4] = {gg.x, gg.y, gg.z, gg.w};
+                                uint32_t rw[4];
+#pragma unroll
+                                for (int q = 0; q < 4; ++q)
+                                    rw[q] = pack_bf16(__uint_as_float(vw[q] << 16) * __uint_as_float(gw[q] << 16),
+                                                      __uint_as_float(vw[q] & 0xffff0000u) * __uint_as_float(gw[q] & 0xffff0000u));
+                                v = make_uint4(rw[0], rw[1], rw[2], rw[3]);
+                            }
+                            *reinterpret_cast<uint4 *>(y_out + ((long long)bh * N + base + t) * D + c * 8) = v;
+                        }
+                    }
                 }
             }
-            asm volatile("bar.sync 2, 128;" ::: "memory");   // the staging tile has been read before the next one is written
             ++nq;
         }
+        if (tid == 0) bulk_store_wait();
         // the state after the segment's last update: the segment's own sum for the second pass (sums_only), or,
         // from the last segment, S [2 d_f, d] of the decode state (this CTA's features)
         float *S_dst = nullptr;
@@ -980,17 +999,18 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         float *zs = reinterpret_cast<float *>(smem + P::oZ) + (warp - 8) * DF;   // this warp's copy of the z row
         bool ok = true;
         int nx = 0;
+        // z half of the chunk two back (every row of the warp dots its features with it): requested a block ahead (a round
+        // trip to memory otherwise stood in every block), placed in shared memory when its block begins
+        auto request_z = [&](int blk) {
+            const int chunk = min(((2 * blk + (r >> 6)) * 64) / C, Tn - 1);   // (a sub-chunk past the end of a ragged last block has no chunk)
+            const float *zrow = zpre + ((long long)bh * n_routed + (chunk - 2)) * NF + half * DF;
+            return lane < DF / 4 ? reinterpret_cast<const float4 *>(zrow)[lane] : make_float4(0.f, 0.f, 0.f, 0.f);
+        };
+        float4 zreg = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (b_first < NB) zreg = request_z(b_first);
         for (int blk = b_first; blk < NB; ++blk, ++nx) {
             const int u = 2 * blk + (r >> 6);            // this row's sub-chunk; its slot is u & 1 = r >> 6
             const int slot = r >> 6, rr = r & 63;
-            // z half of the chunk two back (every row of the warp dots its features with it): requested now,
-            // placed in shared memory when it is needed
-            float4 zreg = make_float4(0.f, 0.f, 0.f, 0.f);
-            {
-                const int chunk = min((u * 64) / C, Tn - 1);   // (a sub-chunk past the end of a ragged last block has no chunk)
-                const float *zrow = zpre + ((long long)bh * n_routed + (chunk - 2)) * NF + half * DF;
-                if (lane < DF / 4) zreg = reinterpret_cast<const float4 *>(zrow)[lane];
-            }
             if (ok) ok = mbar_wait(x_full, nx & 1, abort_flag, status, 70);
             ok = __all_sync(0xffffffffu, ok);
             float nx2 = 0.f;
@@ -1014,6 +1034,7 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             __syncwarp();
             if (lane == 0) mbar_arrive(x_empty);
             if (lane < DF / 4) reinterpret_cast<float4 *>(zs)[lane] = zreg;
+            if (blk + 1 < NB) zreg = request_z(blk + 1);
             // f of this block is read from tensor memory twice, 32 columns at a time, in loops that stay rolled: the
             // warp's instruction stream per block is then a few kilobytes.  (With the row held in 128 registers and
             // everything unrolled, instruction fetch was the first stall reason of the kernel.)  f has a buffer per
@@ -1166,11 +1187,11 @@ int launch_fused(const still_params_t *p, long long N, const void *Q, const void
                  float *S_out, float *seg_sums, void *phiK_sel, void *v_sel, long long sel_rows, int *status, cudaStream_t st,
                  int *launches) {
     using bf = __nv_bfloat16;
-    CUtensorMap tq, tw, tk, tv, tks, tvs;
+    CUtensorMap tq, tw, tk, tv, tks, tvs, ty;
     const unsigned long long BH = (unsigned long long)p->B * p->H, BHkv = (unsigned long long)p->B * p->Hkv;
     if (!make_map_2d(&tq, Q, BH * N, D, 128, false) || !make_map_2d(&tw, Wq, (unsigned long long)p->H * D, DF, D, false) ||
         !make_map_2d(&tk, phiK, BHkv * N, 2 * DF, FusedPlan<D, DF>::kUTok, false) ||
-        !make_map_2d(&tv, V, BHkv * N, D, FusedPlan<D, DF>::kUTok, false))
+        !make_map_2d(&tv, V, BHkv * N, D, FusedPlan<D, DF>::kUTok, false) || !make_map_2d(&ty, y_part, 2 * BH * N, D, 64, false))
         return STILL_ERR_CUDA;
     // With a salient-cache budget and topk < chunk the leaving tokens are read from gathered copies of their rows
     // (otherwise every token of a chunk is selected and the chunk's own tiles are the leaving tiles).
@@ -1193,7 +1214,7 @@ int launch_fused(const still_params_t *p, long long N, const void *Q, const void
     for (int pass = n_seg > 1 && !again ? 0 : 1; pass < 2; ++pass) {
         // pass 0 (only with several segments): the sum of every segment's own updates; pass 1: the scan proper
         dim3 grid((unsigned)BH, 2, (unsigned)(pass == 0 ? (n_seg - 1) * parts : n_seg));   // head, feature half, segment (piece)
-        const cudaError_t e = launch_dependent(la_fused_kernel<D, DF>, grid, dim3(384), Plan::kTotal, st, tq, tw, tk, tv, tks, tvs, (const bf *)bq, (const bf *)G, sel_idx, zpre,
+        const cudaError_t e = launch_dependent(la_fused_kernel<D, DF>, grid, dim3(384), Plan::kTotal, st, tq, tw, tk, tv, tks, tvs, ty, (const bf *)bq, (const bf *)G, sel_idx, zpre,
                                                                (bf *)y_part, d_part, S_out, seg_sums, status, p->H, p->Hkv, (int)N,
                                                                p->chunk, p->topk, p->topk > 0 ? (int)(p->max_salient / p->topk) : 0,
                                                                (long long)BH * N * D, (long long)BH * N,
@@ -1233,7 +1254,7 @@ int tc_la_branch(const still_params_t *p, long long N, const void *Q, const void
                  float *csum, float *zpre, void *y_part, float *d_part, float *seg_sums, float *S_out, float *z_out,
                  void *phiK_sel, void *k_sel, void *v_sel, long long sel_rows, int *status_words, cudaStream_t st, int *launches) {
     using bf = __nv_bfloat16;
-    if ((long long)p->B * p->H * N >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;  // TMA row coordinate
+    if ((long long)p->B * p->H * N >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;  // TMA row coordinate (y_part's 2^32 rows would be 0.5 TB)
     const int NF = 2 * p->d_f, C = p->chunk;
     const long long Tn = (N + C - 1) / C, BH = (long long)p->B * p->H;
     const int n_routed = Tn >= 3 ? (int)(Tn - 2) : 0;
