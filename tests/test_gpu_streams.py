@@ -1,0 +1,68 @@
+"""Edges of the tensor-core prefill: the key streams of the attention kernels' query tiles, and the segments of the linear
+branch's scan."""
+import pytest
+import torch
+
+import paper_2602_02180_b200 as still
+from paper_2602_02180_b200 import synth
+
+from . import util_parity as U
+
+pytestmark = pytest.mark.gpu
+
+
+def _workload(H, Hkv, d, N, C, k):
+    return synth.Workload("t", 1, H, Hkv, d, N, C, k, "bf16", "head_scale", 31)
+
+
+@pytest.mark.parametrize("d,N,C,k,budget", [
+    # one query tile; a second one of a single row; a CTA (256 rows; a pair: 512) that is just full, and one row more
+    (64, 1, 64, 16, 0), (64, 128, 64, 16, 0), (64, 129, 64, 16, 0), (64, 256, 64, 64, 0), (64, 257, 128, 32, 0),
+    (128, 1, 64, 16, 0), (128, 256, 64, 64, 0), (128, 257, 128, 32, 0), (128, 512, 64, 16, 0), (128, 513, 64, 16, 0),
+    # shared tiles that run through the ring several times, and own tiles of both query tiles behind them
+    (64, 2111, 64, 64, 0), (128, 2303, 64, 64, 0), (128, 2200, 128, 1, 0),
+    # windows of the capped cache that two query tiles share in part, or not at all (then every tile is one's own)
+    (64, 1500, 64, 16, 64), (64, 1500, 64, 64, 64), (128, 2000, 64, 64, 64), (128, 2000, 128, 32, 32), (128, 2100, 64, 32, 896),
+])
+def test_key_streams(d, N, C, k, budget):
+    w = _workload(4, 2, d, N, C, k)
+    r = U.run_prefill(w, max_salient=budget)
+    heads = [(0, 0), (0, 3)]
+    U.check_selection(r["scores"], r["sel"], C, k, heads)
+    U.check_outputs(w, r["Q"], r["K"], r["V"], r["Wq"], r["Wk"], r["Y"], r["scores"], r["sel"], heads, max_salient=budget)
+
+
+@pytest.mark.parametrize("H,Hkv,d,N,C,k,budget,gate", [
+    (32, 8, 128, 1003, 64, 16, 0, True),      # two segments that fold again, gated
+    (32, 8, 64, 1090, 64, 16, 0, False),      # rows that are no whole sub-chunk, without a gate
+    (16, 4, 128, 2048, 64, 16, 0, False),     # four segments, 48 tiles before the last: folded again
+    (16, 4, 128, 2752, 64, 16, 0, False),     # 72 tiles: a pass of sums, pieces of three chunks
+    (4, 4, 64, 3000, 64, 32, 0, False),       # ... a ring of eleven stages
+    (16, 4, 128, 4200, 128, 32, 128, False),  # ... with tokens leaving a capped cache
+    (4, 2, 128, 4300, 128, 128, 256, False),  # ... every token selected: the state holds the leaving ones alone
+])
+def test_linear_scan_segments(H, Hkv, d, N, C, k, budget, gate):
+    w = _workload(H, Hkv, d, N, C, k)
+    p = U.params_of(w, max_salient=budget)
+    lay = still.state_layout(p, N)
+    state = torch.zeros(lay["total"], dtype=torch.uint8, device="cuda")
+    r = U.run_prefill(w, gate=gate, max_salient=budget, state=state, state_max_tokens=N)
+    heads = [(0, 0), (0, H - 1)]
+    U.check_outputs(w, r["Q"], r["K"], r["V"], r["Wq"], r["Wk"], r["Y"], r["scores"], r["sel"], heads, G=r["G"],
+                    rows=U.sample_rows(N, 200, C), max_salient=budget)
+    # S and z: phi(K)^T [V, 1] over the tokens that have left for the state, in float64.  The features are rounded to bf16, by at
+    # most 2^-9 each, independently of the signs of V: twice that for S, once for sums of positive terms.
+    T, window = -(-N // C), budget // k
+    n = (T - 2) * C
+    S = state[lay["S"]: lay["S"] + H * 2 * d * d * 4].view(torch.float32).view(H, 2 * d, d)
+    z = state[lay["z"]: lay["z"] + H * 2 * d * 4].view(torch.float32).view(H, 2 * d)
+    for _, h in heads:
+        kv = h // (H // Hkv)
+        x, W = r["K"][0, kv, :n].double(), r["Wk"][kv].double()
+        f = x @ W
+        u = f * (x.norm(dim=1, keepdim=True) / f.norm(dim=1, keepdim=True))
+        phi = torch.cat([u.softmax(1), (-u).softmax(1)], 1)
+        still_cached = r["sel"][0, h, max(T - 2 - window, 0) if window else 0: T - 2].flatten().long()
+        phi[still_cached] = 0
+        for got, want, tol in ((S[h], phi.T @ r["V"][0, kv, :n].double(), 2 ** -8), (z[h], phi.sum(0), 2 ** -9)):
+            assert float((got - want).norm() / want.norm()) <= tol
