@@ -794,7 +794,7 @@ sa_merge_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
 // TMEM accumulators, so that the loads of tile n+1 and its UMMA run under the row epilogue of tile n.
 // The row's epilogue bounds it: three special-function instructions per window element (one 2^x, two logarithms) against
 // six or seven others, by eight warps an SM, two tiles at a time (special-function unit 45 % busy, issue slots 40 %,
-// DRAM 34 % at d = 128, C = 64).  2 x 32 heads x 32768 tokens, d = 128, C = 64: 222 us, 4 x 32 x 4096, d = 64: 59 us, 32 x 131072,
+// DRAM 34 % at d = 128, C = 64).  With the ranking as it was before (see below), 2 x 32 heads x 32768 tokens, d = 128, C = 64: 222 us, 4 x 32 x 4096, d = 64: 59 us, 32 x 131072,
 // d = 128, C = 128: 807 us (with scalar arithmetic, logarithms for subnormal arguments, and for C = 128 a second set of
 // exponentials: 325 to 368, 83 and 1030 us).
 // Warps: 0 TMA producer, 1 MMA issuer, 2-5 score group 0 (even tiles of the CTA), 6-9 score group 1 (odd
