@@ -330,9 +330,10 @@ __device__ __forceinline__ void softmax_role(const Stream &st, const AttnBars &b
             // P = 2^(s * scale - m) as bf16.  The MUFU unit (one warp instruction per eight cycles) would need 1024 cycles
             // for a query tile's exponentials, which is as long as the tensor pipe needs for the tile's two products; so
             // one of kPolyEvery column pairs takes 2^x from the FMA pipes instead (see exp2_fma2), interleaved with the
-            // others so that both units work at the same time.  (32768 tokens, d = 128, every token kept: none 14.5 ms, one
-            // of 8 14.3, of 4 14.45, 5 of 16 14.7; 4096 tokens, d = 64: 536, 515, 512 and 517 us.)
-            constexpr int kPolyEvery = D == 64 ? 4 : 8;
+            // others so that both units work at the same time.  The same share on both head dims: equal logits then get
+            // equal weights, bit for bit.  (4096 tokens, d = 64: none 536 us, one of 8 515, of 4 512, 5 of 16 517; 32768
+            // tokens, d = 128, every token kept, in turn on one box: one of 8 15.17 ms, of 4 15.28.)
+            constexpr int kPolyEvery = 4;
             uint32_t pk[2][32];
 #pragma unroll
             for (int q = 0; q < 2; ++q) {

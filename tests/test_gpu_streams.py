@@ -66,3 +66,22 @@ def test_linear_scan_segments(H, Hkv, d, N, C, k, budget, gate):
         phi[still_cached] = 0
         for got, want, tol in ((S[h], phi.T @ r["V"][0, kv, :n].double(), 2 ** -8), (z[h], phi.sum(0), 2 ** -9)):
             assert float((got - want).norm() / want.norm()) <= tol
+
+
+@pytest.mark.parametrize("N,C,k,budget", [
+    (700, 64, 64, 0), (2303, 64, 64, 0), (1500, 128, 32, 0),
+])
+def test_both_head_dims_give_the_same_rows(N, C, k, budget):
+    # A head of 64 dims, and the same head with 64 more that add nothing to its logits and features and hold its values once
+    # more: the kernels of both head dims weigh and sum the same numbers in the same order, so the rows are equal, bit for bit.
+    w = _workload(4, 2, 64, N, C, k)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    Wq, Wk = synth.make_npmap_weights(w, "cuda")
+    call = lambda d, *x: still.hybrid_attn_fwd(still.StillParams(1, 4, 2, d, C, k, torch.bfloat16, d_f=64, sm_scale=w.sm_scale,  # noqa: E731
+                                                                 max_salient=budget), *x)
+    wide = lambda x: torch.cat([x, torch.zeros_like(x)], -1)  # noqa: E731
+    Y, scores, sel = call(64, Q, K, V, Wq, Wk)
+    Y2, scores2, sel2 = call(128, wide(Q), wide(K), torch.cat([V, V], -1), torch.cat([Wq, torch.zeros_like(Wq)], 1),
+                             torch.cat([Wk, torch.zeros_like(Wk)], 1))
+    assert torch.equal(scores, scores2) and torch.equal(sel, sel2)
+    assert torch.equal(torch.cat([Y, Y], -1), Y2)
