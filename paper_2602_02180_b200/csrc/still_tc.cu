@@ -11,8 +11,8 @@
 // One CTA owns 256 consecutive query rows of one (batch, head), a pair of CTAs 512: two query tiles A and B of 128
 // (256) rows.  Their keys come as a stream of 128-key tiles: SEL tiles j (rows [128j, 128j+128) of K_sel / V_sel), and
 // the LOC tiles around the rows (rows of K / V at positions [128m, 128m+128)).  First the SEL tiles that both query
-// tiles see, then what only one of them sees, by turns.  Which columns of a tile a query row sees is a per-row column
-// interval, applied as a mask in the softmax.
+// tiles see (before them what has already left the window of B), then what only one of them sees, by turns.  Which
+// columns of a tile a query row sees is a per-row column interval, applied as a mask in the softmax.
 //
 // Warp roles (384 threads):
 //   warps 0-7  softmax, four warps per query tile, one thread per query row (tcgen05.ld of the S row): online softmax in
@@ -115,35 +115,37 @@ struct TmemPlan {
     __device__ __forceinline__ static uint32_t o(int x) { return 256u + (uint32_t)x * (uint32_t)D; }
 };
 
-// The key stream of a CTA (or CTA pair).  Entries 0 .. n_shared - 1 are SEL tiles that both query tiles use; then come
-// the entries of one query tile each, A and B by turns until one has no more: its other SEL tiles, then its LOC tiles.
-// (With an entry's query tiles one after the other at the end, A waited for B there and B for A.)
+// The key stream of a CTA (or CTA pair).  Query tile x takes its SEL tiles in the order of their positions, then its LOC
+// tiles; that order is the one in which a row's weights are rounded and summed, and it does not depend on where the query
+// tiles lie.  Entries: n_lead SEL tiles that only A sees (the oldest of its window, with a salient-cache budget), n_shared
+// that both use, then what is left of either, A and B by turns until one has no more.  (With an entry's query tiles one
+// after the other at the end, A waited for B there and B for A.  The n_lead tiles, at most two, wait for nobody: taken
+// behind the shared ones and by turns with B's, 32 heads x 131072 tokens capped at 896 took 7908 us a call, like this 7992.)
 struct Stream {
-    int sel0, n_shared;              // first shared SEL tile, number of shared entries
-    int sel_a, n_sel_a, loc_a, n_a;  // A's own: first SEL tile, SEL tiles, first LOC tile, entries
+    int n_lead, n_shared;
+    int sel_a, n_sel_a, loc_a, n_a;  // A's first SEL tile, SEL tiles, first LOC tile, and its entries behind the shared ones
     int sel_b, n_sel_b, loc_b, n_b;
-    __device__ __forceinline__ int entries() const { return n_shared + n_a + n_b; }
-    __device__ __forceinline__ int entries_of(int x) const { return n_shared + (x ? n_b : n_a); }
-    // entry of the k-th tile of query tile x
-    __device__ __forceinline__ int entry(int x, int k) const {
-        const int i = k - n_shared, turns = min(n_a, n_b);
-        return i < 0 ? k : n_shared + (i < turns ? 2 * i + x : i + turns);
-    }
-    // query tile and its running number of own entry s
-    __device__ __forceinline__ void own(int s, int &x, int &i) const {
-        const int turns = min(n_a, n_b);
-        x = s < 2 * turns ? s & 1 : (n_a > n_b ? 0 : 1);
-        i = s < 2 * turns ? s >> 1 : s - turns;
-    }
-    // entry e: a SEL tile, or a LOC tile?  Returns its number.
-    __device__ __forceinline__ int tile(int e, bool &sel) const {
-        sel = true;
-        if (e < n_shared) return sel0 + e;
-        int x, i;
-        own(e - n_shared, x, i);
+    __device__ __forceinline__ int first_own(int x) const { return n_shared + (x ? 0 : n_lead); }   // (x's tiles before those)
+    __device__ __forceinline__ int entries() const { return n_lead + n_shared + n_a + n_b; }
+    __device__ __forceinline__ int entries_of(int x) const { return first_own(x) + (x ? n_b : n_a); }
+    __device__ __forceinline__ bool shared(int e) const { return e >= n_lead && e < n_lead + n_shared; }
+    // k-th tile of query tile x: a SEL tile, or a LOC tile?  Returns its number.
+    __device__ __forceinline__ int tile_of(int x, int k, bool &sel) const {
         const int n = x ? n_sel_b : n_sel_a;
-        sel = i < n;
-        return sel ? (x ? sel_b : sel_a) + i : (x ? loc_b : loc_a) + i - n;
+        sel = k < n;
+        return k + (sel ? (x ? sel_b : sel_a) : (x ? loc_b : loc_a) - n);
+    }
+    // ... and its entry
+    __device__ __forceinline__ int entry(int x, int k) const {
+        const int i = k - first_own(x), turns = min(n_a, n_b);
+        return i < 0 ? k + (x ? n_lead : 0) : n_lead + n_shared + (i < turns ? 2 * i + x : i + turns);
+    }
+    // the tile of entry e
+    __device__ __forceinline__ int tile(int e, bool &sel) const {
+        const int s = e - n_lead - n_shared, turns = min(n_a, n_b);
+        if (s < 0) return tile_of(0, e, sel);
+        const int x = s < 2 * turns ? s & 1 : (n_a > n_b ? 0 : 1);
+        return tile_of(x, first_own(x) + (s < 2 * turns ? s >> 1 : s - turns), sel);
     }
 };
 
@@ -180,21 +182,20 @@ __device__ __forceinline__ Stream make_stream(int R0, int rows, int N, int C, in
     const int last_a = min(R0 + rows, N) - 1, last_b = min(R0 + 2 * rows, N) - 1;
     // SEL tiles [a0, a1) and [b0, b1): a tile's first row sees the oldest entries, its last row the newest
     const int a0 = sel_start(sel_limit(R0, C, lam), budget) / kBlockN, a1 = (sel_limit(last_a, C, lam) + kBlockN - 1) / kBlockN;
-    st.loc_a = max(m_a - 1, 0);
-    st.sel_a = st.sel0 = a0;
-    st.n_shared = st.n_b = st.n_sel_b = st.sel_b = st.loc_b = 0;
+    st.sel_a = a0;
     st.n_sel_a = max(a1 - a0, 0);
+    st.loc_a = max(m_a - 1, 0);
+    st.n_lead = st.n_shared = st.sel_b = st.n_sel_b = st.loc_b = st.n_b = 0;
     if (R0 + rows < N) {
         const int b0 = sel_start(sel_limit(R0 + rows, C, lam), budget) / kBlockN, b1 = (sel_limit(last_b, C, lam) + kBlockN - 1) / kBlockN;
-        st.sel0 = b0;                        // (a0 <= b0 and a1 <= b1)
-        st.n_shared = max(a1 - b0, 0);
-        st.n_sel_a = max(min(a1, b0) - a0, 0);
-        st.sel_b = max(b0, a1);
-        st.n_sel_b = max(b1 - st.sel_b, 0);
+        st.n_shared = max(a1 - b0, 0);                    // (a0 <= b0 and a1 <= b1)
+        st.n_lead = st.n_shared > 0 ? b0 - a0 : 0;
+        st.sel_b = b0;
+        st.n_sel_b = max(b1 - b0, 0);
         st.loc_b = m_b - 1;
-        st.n_b = st.n_sel_b + min(m_b + rows / kBlockN - 1, last_m) - st.loc_b + 1;
+        st.n_b = st.n_sel_b - st.n_shared + min(m_b + rows / kBlockN - 1, last_m) - st.loc_b + 1;
     }
-    st.n_a = st.n_sel_a + min(m_b - 1, last_m) - st.loc_a + 1;
+    st.n_a = st.n_sel_a - st.n_lead - st.n_shared + min(m_b - 1, last_m) - st.loc_a + 1;
     return st;
 }
 
@@ -213,6 +214,12 @@ __device__ __forceinline__ void softmax_role(const Stream &st, const AttnBars &b
                                              const int N, const int C, const int lam, const int budget,
                                              const float scale_log2) {
     constexpr int kStages = AttnPlan<D, kPair>::kStages;
+    // The MUFU unit (one warp instruction per eight cycles) would need 1024 cycles for a query tile's exponentials, which is as
+    // long as the tensor pipe needs for the tile's two products; so one of kPolyEvery column pairs takes 2^x from the FMA
+    // pipes instead (see exp2_fma2), interleaved with the others so that both units work at the same time.  The same share
+    // on both head dims: equal logits then get equal weights, bit for bit.  (4096 tokens, d = 64: none 536 us, one of 8 515,
+    // of 4 512, 5 of 16 517; 32768 tokens, d = 128, every token kept, in turn on one box: one of 8 15.17 ms, of 4 15.28.)
+    constexpr int kPolyEvery = 4;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     auto arrive_first = [&](uint64_t *b) {   // on the barrier of the CTA whose warp issues the products
         if constexpr (kPair) mbar_arrive_cluster(mapa(smem_u32(b), 0));
@@ -235,23 +242,23 @@ __device__ __forceinline__ void softmax_role(const Stream &st, const AttnBars &b
         auto release = [&](int e) {
             if (row_in_tile != 0) return;
             mbar_arrive(bar.kv_empty + e % kStages);
-            if (e >= st.n_shared) mbar_arrive(bar.kv_empty + e % kStages);
+            if (!st.shared(e)) mbar_arrive(bar.kv_empty + e % kStages);
         };
         for (int k = 0; k < n_mine && ok; ++k) {
             // visible column interval [lo, hi] of this row in the stream tile
             bool sel;
-            const int p0 = st.tile(st.entry(x, k), sel) * kBlockN;
+            const int p0 = st.tile_of(x, k, sel) * kBlockN;
             const int lo = max((sel ? lo_sel : loc_lo) - p0, 0), hi = min((sel ? lim_sel - 1 : tq) - p0, kBlockN - 1);
             const bool need_mask = __any_sync(0xffffffffu, lo > 0 || hi < kBlockN - 1);
-            const bool none = need_mask && !__any_sync(0xffffffffu, lo <= hi);   // (a warp whose rows see none of it writes zeros)
+            const bool none = need_mask && !__any_sync(0xffffffffu, lo <= hi);   // (a warp whose rows see none of it skips the arithmetic)
             ok = mbar_wait(bar.s_full + x, k & 1, abort_flag, status, 8);
             if (!ok) break;
             tc_fence_after();
             if (none) {
                 if (lane == 0) arrive_first(bar.s_free + x);
-                uint32_t zero[32];
+                uint32_t masked[32];   // the weights of masked columns: 0, and 2^-126 from the cubic
 #pragma unroll
-                for (int j = 0; j < 32; ++j) zero[j] = 0u;
+                for (int j = 0; j < 32; ++j) masked[j] = j % kPolyEvery == 0 ? 0x00800080u : 0u;
                 if (k > 0) {
                     ok = mbar_wait(bar.pv_done + x, (k - 1) & 1, abort_flag, status, 11);
                     if (!ok) break;
@@ -259,8 +266,8 @@ __device__ __forceinline__ void softmax_role(const Stream &st, const AttnBars &b
                     tc_fence_after();
                 }
                 __syncwarp();
-                tmem_st32(p_addr, zero);
-                tmem_st32(p_addr + 32, zero);
+                tmem_st32(p_addr, masked);
+                tmem_st32(p_addr + 32, masked);
                 tmem_wait_st();
                 tc_fence_before();
                 __syncwarp();
@@ -327,13 +334,7 @@ __device__ __forceinline__ void softmax_role(const Stream &st, const AttnBars &b
             const float neg_m = (m_used == -INFINITY) ? 0.f : -m_used;
             const float2 scale2 = make_float2(scale_log2, scale_log2), negm2 = make_float2(neg_m, neg_m);
             float2 acc = make_float2(0.f, 0.f);
-            // P = 2^(s * scale - m) as bf16.  The MUFU unit (one warp instruction per eight cycles) would need 1024 cycles
-            // for a query tile's exponentials, which is as long as the tensor pipe needs for the tile's two products; so
-            // one of kPolyEvery column pairs takes 2^x from the FMA pipes instead (see exp2_fma2), interleaved with the
-            // others so that both units work at the same time.  The same share on both head dims: equal logits then get
-            // equal weights, bit for bit.  (4096 tokens, d = 64: none 536 us, one of 8 515, of 4 512, 5 of 16 517; 32768
-            // tokens, d = 128, every token kept, in turn on one box: one of 8 15.17 ms, of 4 15.28.)
-            constexpr int kPolyEvery = 4;
+            // P = 2^(s * scale - m) as bf16
             uint32_t pk[2][32];
 #pragma unroll
             for (int q = 0; q < 2; ++q) {
@@ -550,21 +551,27 @@ __device__ __forceinline__ void mma_role(const Stream &st, const AttnBars &bar, 
         else tc_commit(b);
     };
     // A place in the order of the products: query tile x, its k-th tile, and the ring stage of that.
-    const int n_items = 2 * st.n_shared + st.n_a + st.n_b, turns = min(st.n_a, st.n_b), x_last = st.n_a > st.n_b ? 0 : 1;
+    const int n_own0 = st.n_lead + 2 * st.n_shared, n_items = n_own0 + st.n_a + st.n_b;
+    const int turns = min(st.n_a, st.n_b), x_last = st.n_a > st.n_b ? 0 : 1;
     struct Item {
         int m, x, k;
         RingPos pos;
     };
     auto advance = [&](Item &it) {
         ++it.m;
-        if (it.m < 2 * st.n_shared) {
-            it.x ^= 1;
-            if (it.x == 1) return;   // (both query tiles use the entry)
+        if (it.m <= st.n_lead && it.m < n_own0) {
             ++it.k;
+        } else if (it.m < n_own0) {
+            it.x ^= 1;
+            if (it.x == 1) {   // (both query tiles use the entry)
+                it.k -= st.n_lead;
+                return;
+            }
+            it.k += st.n_lead + 1;
         } else {
-            const int s = it.m - 2 * st.n_shared;
+            const int s = it.m - n_own0;
             it.x = s < 2 * turns ? s & 1 : x_last;
-            it.k = st.n_shared + (s < 2 * turns ? s >> 1 : s - turns);
+            it.k = st.first_own(it.x) + (s < 2 * turns ? s >> 1 : s - turns);
         }
         it.pos.next(kStages);
     };
@@ -572,7 +579,7 @@ __device__ __forceinline__ void mma_role(const Stream &st, const AttnBars &bar, 
     int x_prev = 0, k_prev = 0;   // of the item whose S was formed last
     auto issue_qk = [&]() {
         // K and V of the entry have arrived (B follows A on the entries that they share)
-        if (qk.m >= 2 * st.n_shared || qk.x == 0) wait(bar.kv_full + qk.pos.stage, qk.pos.parity, 7);
+        if (qk.m >= n_own0 || qk.x == 0) wait(bar.kv_full + qk.pos.stage, qk.pos.parity, 7);
         // the place of S is free: its last tile has been read
         if constexpr (TM::kOneS) {
             if (qk.m > 0) wait(bar.s_free + x_prev, k_prev & 1, 3);

@@ -70,6 +70,8 @@ def test_linear_scan_segments(H, Hkv, d, N, C, k, budget, gate):
 
 @pytest.mark.parametrize("N,C,k,budget", [
     (700, 64, 64, 0), (2303, 64, 64, 0), (1500, 128, 32, 0),
+    # windows of the capped cache: none, one or two tiles that the first query tile alone sees ahead of the shared ones
+    (1100, 64, 64, 256), (1500, 64, 64, 640), (2000, 128, 32, 64), (3000, 128, 32, 896), (1836, 64, 16, 64), (2100, 64, 32, 896),
 ])
 def test_both_head_dims_give_the_same_rows(N, C, k, budget):
     # A head of 64 dims, and the same head with 64 more that add nothing to its logits and features and hold its values once
