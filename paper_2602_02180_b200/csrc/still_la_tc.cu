@@ -526,9 +526,13 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     // earlier segments' updates (kFromSums: seg_sums, produced by a first pass of this kernel, kSumsOnly), or folding
     // the chunks before it itself (kFoldAll, where they are few).
     // The first pass cuts every segment into sum_parts pieces, one CTA each (it has no scan to keep in order, and
-    // the pieces fill the SMs that the n_seg - 1 summed segments alone would leave idle).
+    // the pieces fill the SMs that the n_seg - 1 summed segments alone would leave idle).  A segment that folds itself
+    // forms the same pieces, one after the other, each from zero, and adds them up in fp32 as the other does: carried
+    // through the accumulators, the state would take their rounding (with all-positive values a third to a half more
+    // error of S than the sum of the pieces), and how a call is launched would show in its results.
     const int seg = blockIdx.z;
-    if (sums_only) seg_chunks /= sum_parts;
+    const int piece_chunks = seg_chunks / sum_parts;
+    if (sums_only) seg_chunks = piece_chunks;
     const int NU_all = (N + 63) / 64;           // sub-chunks with query rows
     const int u_first = seg == 0 ? 2 * sc : seg * seg_chunks * sc;   // the first two chunks see an empty state
     const int NU = (!sums_only && seg == n_seg - 1) ? NU_all : min(NU_all, (seg + 1) * seg_chunks * sc);
@@ -545,6 +549,9 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const int chunk0 = mode == kFoldAll ? 0 : u_first / sc - 2;   // first chunk that the segment folds
     const int n_upd = NU > u_first ? ((NU - 1) / sc - 1 - chunk0) * per_chunk : 0;
     const bool has_init = mode == kFromSums && seg > 0;
+    // Pieces of what a segment folds before its own updates.  The sequence's first two chunks answer nothing, so the first
+    // piece is two chunks shorter than the others: with pieces of two chunks it is empty and there is one less.
+    const int n_pieces = mode == kFoldAll && n_upd > 0 ? seg * sum_parts - (seg > 0 && piece_chunks == 2 ? 1 : 0) : 0;
     __nv_bfloat16 *y_out = y_part + (long long)half * part_stride_y;
     float *d_out = d_part + (long long)half * part_stride_d;
 
@@ -591,6 +598,10 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     // TMEM columns: S^T half [value lanes x d_f features] fp32; f = x W_q of a block [128 rows x d_f]; two read-out
     // results [value lanes x 64 tokens]
     constexpr uint32_t col_state = 0, col_f = DF, col_out = 3 * DF;   // f: two buffers of DF columns
+    // Pieces behind the first are formed where the second f and the read-outs will lie, by turns, and are handed to the
+    // workers over the barriers of the read-outs: hand-over n (a piece or a read-out) uses r_done / out_free [n & 1].
+    static_assert(DF <= 128, "fused scan: a piece's sum takes the columns of both read-outs");
+    auto col_piece = [&](int n) -> uint32_t { return (n & 1) ? col_out : col_f + DF; };
 
     // Registers move from the first warpgroup (single-thread roles) to the map warps, whose threads hold a row of f
     // (per scheduler: 72 + 152 + 224 registers for its three warps, of the 3 x 168 the CTA was launched with).
@@ -699,35 +710,44 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 wait(init_done, 0, 73);
                 tc_fence_after();
             }
-            auto issue_update = [&]() {
+            auto issue_update = [&](uint32_t col, bool add) {   // into, or over, the sum at these columns
                 wait(u_masked + us.stage, us.parity, 64);
                 tc_fence_after();
                 const uint32_t so = (uint32_t)us.stage * (P::kUStage >> 4);
-                const uint32_t acc0 = (nu > 0 || has_init) ? 1u : 0u;
                 if (leader && ok) {
-                    mma_ss_lo_acc<idesc_upd>(tmem_base + col_state, v_lo0 + so, pk_lo0 + so, acc0);
+                    mma_ss_lo_acc<idesc_upd>(tmem_base + col, v_lo0 + so, pk_lo0 + so, add ? 1u : 0u);
 #pragma unroll
                     for (int k = 1; k < kUTok / 16; ++k)   // 16 tokens per step: 16 rows of 128 bytes in both operands
-                        mma_ss_lo_acc<idesc_upd>(tmem_base + col_state, v_lo0 + so + k * (2048 >> 4), pk_lo0 + so + k * (2048 >> 4), 1u);
+                        mma_ss_lo_acc<idesc_upd>(tmem_base + col, v_lo0 + so + k * (2048 >> 4), pk_lo0 + so + k * (2048 >> 4), 1u);
                     tc_commit(u_empty + us.stage);
                 }
                 us.next(1, n_stages);
                 ++nu;
             };
             if (NB > b_first) issue_f();
-            // what is folded ahead of the segment's first read-out: everything in a pass of sums
-            const int ahead = sums_only ? n_upd : min(n_upd, (u_first / sc - 2 - chunk0) * per_chunk);
-            while (nu < ahead) issue_update();
+            if (sums_only)
+                while (nu < n_upd) issue_update(col_state, nu > 0);
+            for (int g = 0; g < n_pieces; ++g) {
+                const int tiles = (g == 0 && piece_chunks > 2 ? piece_chunks - 2 : piece_chunks) * per_chunk;
+                const uint32_t col = g == 0 ? col_state : col_piece(nq);
+                if (g > 0) wait(out_free + (nq & 1), ((nq >> 1) & 1) ^ 1, 74);
+                for (int i = 0; i < tiles; ++i) issue_update(col, i > 0);
+                if (g > 0) {
+                    if (leader && ok) tc_commit(r_done + (nq & 1));
+                    ++nq;
+                }
+            }
+            if (n_pieces > 1) wait(out_free + ((nq - 1) & 1), ((nq - 1) >> 1) & 1, 75);   // the last has been added
             for (int u = u_first; u < NU && !sums_only; ++u) {
                 if (u % sc == 0) {
                     // the chunk that has just left the local region: sub-chunks of chunk u / sc - 2
-                    for (int j = 0; j < per_chunk; ++j) issue_update();
+                    for (int j = 0; j < per_chunk; ++j) issue_update(col_state, nu > 0 || has_init);
                 }
                 // The next block's f = x W_q goes out as soon as its rows have arrived and the map warps have taken the
                 // current f out of tensor memory: it is then ready when they finish the current block.  (Issued after
                 // this block's read-out, it made the map warps wait for a round trip through this warp per block.)
                 if ((u & 1) == 0 && b_first + nx < NB) issue_f();
-                wait(pq_full + (u & 1), (nq >> 1) & 1, 65);
+                wait(pq_full + (u & 1), ((u - u_first) >> 1) & 1, 65);   // (u_first is even)
                 wait(out_free + (nq & 1), ((nq >> 1) & 1) ^ 1, 66);
                 tc_fence_after();
                 const uint32_t q_lo = q_lo0 + (uint32_t)(u & 1) * (P::kPhiQ >> 4), d_out_t = tmem_base + col_out + (nq & 1) * 64;
@@ -866,6 +886,27 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(init_done);
+        }
+        for (int g = 1; g < n_pieces; ++g, ++nq) {
+            if (ok) ok = mbar_wait(r_done + (nq & 1), (nq >> 1) & 1, abort_flag, status, 76);
+            ok = __all_sync(0xffffffffu, ok);
+            if (ok) {   // (the commit behind a piece's updates covers those of the pieces before it)
+                tc_fence_after();
+#pragma unroll 1
+                for (int q = 0; q < DF / 32; ++q) {
+                    uint32_t sum[32], add[32];
+                    tmem_ld32(taddr + col_state + q * 32, sum);
+                    tmem_ld32(taddr + col_piece(nq) + q * 32, add);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) sum[j] = __float_as_uint(__uint_as_float(sum[j]) + __uint_as_float(add[j]));
+                    tmem_st32(taddr + col_state + q * 32, sum);
+                }
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(out_free + (nq & 1));
+            }
         }
         constexpr int kPiecesPerRow = D / 8, kPieces = 64 * kPiecesPerRow / 128;   // 16-byte pieces per thread and sub-chunk
         for (int u = u_first; u < NU && !sums_only; ++u) {

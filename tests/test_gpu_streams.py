@@ -87,3 +87,42 @@ def test_both_head_dims_give_the_same_rows(N, C, k, budget):
                              torch.cat([Wk, torch.zeros_like(Wk)], 1))
     assert torch.equal(scores, scores2) and torch.equal(sel, sel2)
     assert torch.equal(torch.cat([Y, Y], -1), Y2)
+
+
+@pytest.mark.parametrize("H,d,df,N", [
+    (32, 64, 64, 1003), (32, 128, 128, 1003),   # two segments; pieces of two chunks, the first of them empty
+    (37, 128, 64, 2100),                        # the most heads that are cut
+    (16, 128, 128, 2048),                       # four segments: eleven pieces
+    (16, 64, 64, 2500),                         # pieces of five chunks
+    (32, 128, 128, 3000),                       # pieces of six chunks
+    (4, 64, 64, 3000),                          # a pass of sums
+])
+def test_linear_state_is_the_fp32_sum_of_its_pieces(H, d, df, N):
+    # W_k = 0 makes every feature 1 / d_f exactly.  Chunk 0 brings 2^24 into the state of every head, whose neighbours in fp32
+    # are 2 apart; the chunks of a later piece bring 1 each, 1/4 at most in one step of the tensor cores.  A piece of 2 n
+    # chunks then adds 2 n exactly, if it is summed by itself and added in fp32; step by step it would be rounded away.
+    # (With an odd number of chunks a piece's sum is odd, and 1 is lost to rounding.)
+    C = 64
+    T = -(-N // C)
+    n_seg = 4 if H <= 18 and T >= 32 else 2
+    per = -(-T // n_seg)
+    per += per & 1                                                   # chunks of a segment
+    parts = 4 if per % 4 == 0 and per >= 8 else 2 if per >= 4 else 1
+    own = (n_seg - 1) * per - 2                                      # first chunk of the last segment's own updates
+    p = still.StillParams(1, H, 1, d, C, C // 2, torch.bfloat16, d_f=df)
+    g = torch.Generator(device="cuda").manual_seed(7)
+    Q, K = (torch.randn(1, n, N, d, generator=g, device="cuda").bfloat16() for n in (H, 1))
+    Wq = (torch.randn(H, d, df, generator=g, device="cuda") * 0.02).bfloat16()
+    V = torch.zeros(1, 1, N, d, device="cuda", dtype=torch.bfloat16)
+    first = per // parts - 2 if per // parts > 2 else per // parts   # chunks of the first piece
+    V[:, :, :C] = 2.0 ** 19 * df                                     # (32 unselected tokens of a chunk)
+    V[:, :, first * C: own * C] = df / 32
+    lay = still.state_layout(p, N)
+    state = torch.zeros(lay["total"], dtype=torch.uint8, device="cuda")
+    still.hybrid_attn_fwd(p, Q, K, V, Wq, torch.zeros(1, d, df, device="cuda", dtype=torch.bfloat16), state=state, state_max_tokens=N)
+    S = state[lay["S"]: lay["S"] + H * 2 * df * d * 4].view(torch.float32)
+    pieces, chunks = (own - first) // (per // parts), per // parts
+    want = torch.tensor(2.0 ** 24, dtype=torch.float32)
+    for _ in range(pieces):
+        want = want + chunks
+    assert S.unique().tolist() == [float(want)]
