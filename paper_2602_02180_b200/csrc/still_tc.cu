@@ -237,31 +237,37 @@ __device__ __forceinline__ void softmax_role(const Stream &st, const AttnBars &b
         const int loc_lo = c >= 1 ? (c - 1) * C : 0;
         float m_used = -INFINITY, l_sum = 0.f;     // log2 domain
         bool ok = true;
+        // A wait can end in one lane and run out in another, and the warp has to stay together for the instructions that take
+        // it whole.  So no wait is left by a branch: the loop runs out with whatever has been read (a wait gives up at once
+        // where a role has given up before), and the warp votes behind it.  (A vote behind every wait took 0.6 % longer at
+        // 64 heads x 32768 tokens, d = 128, one a tile 0.5 % at 128 x 4096, d = 64; skipping the waits after a failure 2 %.)
+        auto wait = [&](uint64_t *b, int parity, int where) {
+            ok = mbar_wait(b, (uint32_t)parity, abort_flag, status, where) && ok;
+        };
         // one thread of a query tile releases the stage of its last product: its share of two, or both where the entry is
         // the tile's alone
         auto release = [&](int e) {
-            if (row_in_tile != 0) return;
+            if (row_in_tile != 0 || !ok) return;
             mbar_arrive(bar.kv_empty + e % kStages);
             if (!st.shared(e)) mbar_arrive(bar.kv_empty + e % kStages);
         };
-        for (int k = 0; k < n_mine && ok; ++k) {
+        for (int k = 0; k < n_mine; ++k) {
             // visible column interval [lo, hi] of this row in the stream tile
             bool sel;
             const int p0 = st.tile_of(x, k, sel) * kBlockN;
             const int lo = max((sel ? lo_sel : loc_lo) - p0, 0), hi = min((sel ? lim_sel - 1 : tq) - p0, kBlockN - 1);
             const bool need_mask = __any_sync(0xffffffffu, lo > 0 || hi < kBlockN - 1);
             const bool none = need_mask && !__any_sync(0xffffffffu, lo <= hi);   // (a warp whose rows see none of it skips the arithmetic)
-            ok = mbar_wait(bar.s_full + x, k & 1, abort_flag, status, 8);
-            if (!ok) break;
+            wait(bar.s_full + x, k & 1, 8);
             tc_fence_after();
             if (none) {
+                __syncwarp();   // (no lane still looks for this phase)
                 if (lane == 0) arrive_first(bar.s_free + x);
                 uint32_t masked[32];   // the weights of masked columns: 0, and 2^-126 from the cubic
 #pragma unroll
                 for (int j = 0; j < 32; ++j) masked[j] = j % kPolyEvery == 0 ? 0x00800080u : 0u;
                 if (k > 0) {
-                    ok = mbar_wait(bar.pv_done + x, (k - 1) & 1, abort_flag, status, 11);
-                    if (!ok) break;
+                    wait(bar.pv_done + x, (k - 1) & 1, 11);
                     release(st.entry(x, k - 1));
                     tc_fence_after();
                 }
@@ -313,10 +319,9 @@ __device__ __forceinline__ void softmax_role(const Stream &st, const AttnBars &b
             }
             // the previous product is in O, has read P and is done with its stage (asked for as late as P is written: the
             // issuing warp takes it up behind a product of the other query tile)
-            auto previous_done = [&]() { return mbar_wait(bar.pv_done + x, (k - 1) & 1, abort_flag, status, 11); };
+            auto previous_done = [&]() { wait(bar.pv_done + x, (k - 1) & 1, 11); };
             if (k > 0 && __any_sync(0xffffffffu, grow)) {
-                ok = previous_done();
-                if (!ok) break;
+                previous_done();
                 tc_fence_after();
                 {
 #pragma unroll
@@ -348,8 +353,7 @@ __device__ __forceinline__ void softmax_role(const Stream &st, const AttnBars &b
                 }
             }
             if (k > 0) {
-                if (ok) ok = previous_done();
-                if (!ok) break;
+                previous_done();
                 tc_fence_after();
                 release(st.entry(x, k - 1));
                 __syncwarp();
@@ -370,9 +374,8 @@ __device__ __forceinline__ void softmax_role(const Stream &st, const AttnBars &b
         // warp's 32 rows of the tile's Q region (one row = D bf16 = 2 D bytes: D / 2 columns of both parts), free
         // once the tile's last Q K^T has completed; 16-byte pieces are swizzled by the row so that row-wise and
         // piece-wise accesses avoid bank conflicts.
-        if (ok) ok = mbar_wait(bar.pv_done + x, (n_mine - 1) & 1, abort_flag, status, 9);   // (every query tile has a LOC tile)
-        ok = __all_sync(0xffffffffu, ok);
-        if (ok) {
+        wait(bar.pv_done + x, (n_mine - 1) & 1, 9);   // (every query tile has a LOC tile)
+        if (__all_sync(0xffffffffu, ok)) {
             tc_fence_after();
             release(st.entry(x, n_mine - 1));   // (the other query tile may have entries left)
             constexpr int kRowBytes = D * 2, kPieces = kRowBytes / 16;   // pieces of 16 bytes per staged row

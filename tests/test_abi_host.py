@@ -97,6 +97,24 @@ def test_dependent_kernels_read_nothing_ahead_of_the_wait():
     assert seen >= 19
 
 
+def _csrc(name):
+    return re.sub(r"//[^\n]*", "", open(os.path.join(still_build.CSRC, name)).read())
+
+
+def test_a_warp_leaves_a_wait_as_a_whole():
+    # A bounded wait can succeed in one lane and run out in another.  Roles of whole warps go on to instructions that take the
+    # whole warp (tensor-memory loads, votes, __syncwarp): the softmax warps never leave their loop for one and vote behind it,
+    # the scan's vote on every wait.
+    softmax = _csrc("still_tc.cu").split("softmax_role(", 1)[1].split("producer_role(", 1)[0]
+    head = "for (int k = 0; k < n_mine; ++k) {"
+    loop, behind = softmax.split(head)[1].split("wait(bar.pv_done + x, (n_mine - 1) & 1, 9);")
+    assert not re.search(r"\b(break|return)\b", loop) and loop.count("wait(bar.") == 3
+    assert softmax.count("mbar_wait(") == 1 and re.match(r"\s*if \(__all_sync\(0xffffffffu, ok\)\) \{", behind)
+    scan = _csrc("still_la_tc.cu").split("la_fused_kernel(", 1)[1].split("MMA issuer", 1)[-1]
+    waits = re.findall(r"if \(ok\) ok = mbar_wait\((?!bar,)[^\n]*\n([^\n]*)", scan)   # (bar: of the issuing warp, see there)
+    assert len(waits) == 7 and all("ok = __all_sync(0xffffffffu, ok);" in after for after in waits)
+
+
 def test_shared_arrays_that_vectors_are_stored_to_are_aligned():
     # A shared array is only as aligned as its element type unless it says more: those without an explicit alignment are
     # the ones that are accessed element by element (or, smem_raw, aligned by hand).
