@@ -617,7 +617,7 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 for (int a = 0; a < DF / 64; ++a) tma_load_2d(smem + P::oW + a * (D * 128), &tm_wq, w_full, a * 64, h * D);
             }
             int nu = 0, nx = 0, spins = 0;
-            Slot us{0, 0}, last{0, 0};
+            Slot us{0, 0};
             Tile ut{chunk0, 0};
             long long t0 = clock64();
             while (nu < n_upd || nx < n_blk) {
@@ -642,7 +642,6 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                         tma_load_2d(stg + a * (kUTok * 128), mp, u_full + us.stage, half * DF + a * 64, row);
                     for (int a = 0; a < D / 64; ++a)   // V: M-major A operand, 64-column atoms kUTok rows apart
                         tma_load_2d(stg + P::kPhiK + a * (kUTok * 128), mv, u_full + us.stage, a * 64, row);
-                    last = us;
                     us.next(1, n_stages);
                     ut.next(1, per_chunk);
                     ++nu;
@@ -660,11 +659,10 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                     }
                 }
             }
-            if (*abort_flag) {  // leave no copy in flight behind
-                if (nu > 0) mbar_wait_drain(u_full + last.stage, last.parity);
-                if (nx > 0) mbar_wait_drain(x_full, (nx - 1) & 1);
-                if (n_blk > 0) mbar_wait_drain(w_full, 0);
-            }
+            const long long t1 = clock64();
+            if (n_blk > 0) mbar_wait_drain(w_full, 0, t1);
+            mbar_drain_ring(x_full, 1, nx, t1);
+            mbar_drain_ring(u_full, n_stages, nu, t1);
         }
     } else if (warp == 1) {
         // ------------------------------------------------------------ MMA issuer

@@ -486,7 +486,7 @@ __device__ __forceinline__ void producer_role(const Stream &st, const AttnBars &
                  q_row + ((int)rank + x * kCtas) * kBlockM);
     bool ok = true;
     int armed = 0;
-    RingPos pos{0, 0}, last{0, 0};
+    RingPos pos{0, 0};
     for (; armed < n; ++armed) {
         ok = mbar_wait(bar.kv_empty + pos.stage, pos.parity ^ 1, abort_flag, status, 1);
         if (!ok) break;
@@ -499,20 +499,19 @@ __device__ __forceinline__ void producer_role(const Stream &st, const AttnBars &
         for (int q = 0; q < P::kVCols / 64; ++q)    // this CTA's value columns, 64 at a time
             load(smem + P::kV + pos.stage * P::kVTile + q * (kBlockN * 128), sel ? tm_vsel : tm_v, bar.kv_full + pos.stage,
                  kv_full0 + pos.stage * 8, (int)rank * P::kVCols + q * 64, row);
-        last = pos;
         pos.next(kStages);
     }
-    if (!ok) {
-        if constexpr (kPair) tell_peer();
-        // leave no copy in flight behind: wait (bounded) for the last stage armed, which in a pair counts both CTAs'
-        // bytes; the second CTA of a pair, whose copies complete on the first's barriers, waits out a fixed stretch
-        // that is long against a tile load
-        if (rank == 0) {
-            if (armed > 0) mbar_wait_drain(bar.kv_full + last.stage, last.parity);
-        } else {
-            const long long t1 = clock64();
-            while (clock64() - t1 < 200000) {}
-        }
+    // leave no copy in flight behind.  In a pair the first CTA's barriers count both CTAs' bytes; the second, where it has
+    // given up and the first may not know of its last copies, waits out a fixed stretch that is long against a tile load.
+    const long long t0 = clock64();
+    if constexpr (kPair) {
+        if (!ok) tell_peer();
+    }
+    if (rank == 0) {
+        mbar_wait_drain(bar.q_full, 0, t0);
+        mbar_drain_ring(bar.kv_full, kStages, armed, t0);
+    } else if (!ok) {
+        while (clock64() - t0 < 200000) {}
     }
 }
 
@@ -893,9 +892,7 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                     tma_load_2d(k_s + half * (2 * kBlockN * 128) + kBlockN * 128, &tm_k, full + s, half * 64, k_row + kBlockN);
                 }
             }
-            // leave no copy in flight behind: every armed stage is waited for by the MMA warp in the normal
-            // course; after a failure wait (bounded) for the last one armed
-            if (*abort_flag && it > 0) mbar_wait_drain(full + ((it - 1) & 1), ((it - 1) >> 1) & 1);
+            mbar_drain_ring(full, 2, it, clock64());
         }
     } else if (warp == 1) {
         if (lane == 0) {

@@ -73,12 +73,18 @@ __device__ __forceinline__ bool mbar_wait(uint64_t *bar, uint32_t parity, volati
                                           int *status, int where) {
     return mbar_wait_limit(bar, parity, abort_flag, status, where, kWaitLimitCycles);
 }
-// Bounded wait of the failure path: waits for work already in flight even though the CTA has
-// been flagged as aborted.
-__device__ __forceinline__ void mbar_wait_drain(uint64_t *bar, uint32_t parity) {
-    const long long t0 = clock64();
+// Wait for work already in flight even though the CTA may have been flagged as aborted, bounded from t0 on.
+__device__ __forceinline__ void mbar_wait_drain(uint64_t *bar, uint32_t parity, long long t0) {
     while (!mbar_try_wait(bar, parity))
         if (clock64() - t0 > kWaitLimitCycles) return;
+}
+__device__ __forceinline__ void mbar_wait_drain(uint64_t *bar, uint32_t parity) { mbar_wait_drain(bar, parity, clock64()); }
+// The last thing a producer does, whoever may give up later: no load may still be in flight when the CTA's shared memory is
+// handed on, and loads of different stages need not land in order.  Waits for the loads numbered up to `armed` of a ring of
+// n_stages stages (load i: stage i % n_stages); those before the last n_stages have been waited for to arm these.
+__device__ __forceinline__ void mbar_drain_ring(uint64_t *full, int n_stages, int armed, long long t0) {
+    for (int i = armed > n_stages ? armed - n_stages : 0; i < armed; ++i)
+        mbar_wait_drain(full + i % n_stages, (uint32_t)(i / n_stages) & 1u, t0);
 }
 __device__ __forceinline__ void fence_barrier_init() {
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");

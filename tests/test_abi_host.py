@@ -115,6 +115,30 @@ def test_a_warp_leaves_a_wait_as_a_whole():
     assert len(waits) == 7 and all("ok = __all_sync(0xffffffffu, ok);" in after for after in waits)
 
 
+def test_producers_leave_no_load_in_flight():
+    # Loads of different ring stages need not land in order, and another role can give up after the producer has armed its last
+    # stage: every producer with a ring ends with a wait for all stages that may still be filled, not for the last one, and
+    # whether or not it has failed itself.
+    drain = _csrc("still_tc_ptx.cuh").split("mbar_drain_ring(", 1)[1].split("}", 1)[0]
+    parts = [m.strip() for m in re.search(r"for \(int i = ([^;]*); (i < armed); \+\+i\)\s*mbar_wait_drain\(full \+ ([^,]*), ([^;]*), t0\);", drain).groups()]
+    first, more, slot, parity = (m.replace("(uint32_t)", "").replace("/", "//").replace("1u", "1") for m in parts)
+    first = re.sub(r"(.*) \? (.*) : (.*)", r"(\2) if (\1) else (\3)", first)
+    for n_stages in (1, 2, 4, 5, 11, 12):
+        for armed in range(40):
+            waited, i = {}, eval(first, {"armed": armed, "n_stages": n_stages})
+            while eval(more, {"i": i, "armed": armed}):
+                at = {"i": i, "n_stages": n_stages}
+                waited[eval(slot, at)] = eval(parity, at)
+                i += 1
+            last = {k % n_stages: k // n_stages % 2 for k in range(armed)}   # the round in which a stage was armed last
+            assert waited == last
+    tc, la = _csrc("still_tc.cu"), _csrc("still_la_tc.cu")
+    assert "mbar_drain_ring(bar.kv_full, kStages, armed, t0);" in tc.split("producer_role(", 1)[1].split("mma_role(", 1)[0]
+    assert "mbar_drain_ring(full, 2, it, clock64());" in tc.split("score_select_tc_kernel(", 1)[1]
+    scan = la.split("la_fused_kernel(", 1)[1]
+    assert re.search(r"mbar_drain_ring\(x_full, 1, nx, t1\);\s*mbar_drain_ring\(u_full, n_stages, nu, t1\);", scan)
+
+
 def test_shared_arrays_that_vectors_are_stored_to_are_aligned():
     # A shared array is only as aligned as its element type unless it says more: those without an explicit alignment are
     # the ones that are accessed element by element (or, smem_raw, aligned by hand).
