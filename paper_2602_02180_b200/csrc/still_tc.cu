@@ -304,18 +304,20 @@ __device__ __forceinline__ void softmax_role(const Stream &st, const AttnBars &b
             float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
 #pragma unroll
             for (int j = 0; j < 128; j += 8) {
-                mx0 = max3(mx0, s[j], s[j + 1]);
-                mx1 = max3(mx1, s[j + 2], s[j + 3]);
-                mx2 = max3(mx2, s[j + 4], s[j + 5]);
-                mx3 = max3(mx3, s[j + 6], s[j + 7]);
+                mx0 = max3_nan(mx0, s[j], s[j + 1]);
+                mx1 = max3_nan(mx1, s[j + 2], s[j + 3]);
+                mx2 = max3_nan(mx2, s[j + 4], s[j + 5]);
+                mx3 = max3_nan(mx3, s[j + 6], s[j + 7]);
             }
-            const float mt = fmaxf(fmaxf(mx0, mx1), fmaxf(mx2, mx3)) * scale_log2;
-            // lazy rescale: keep the old reference unless the new maximum exceeds it by 2^8
-            const bool grow = mt > m_used + 8.f;
+            const float mt = max_nan(max_nan(mx0, mx1), max_nan(mx2, mx3)) * scale_log2;
+            // lazy rescale: keep the old reference unless the new maximum exceeds it by 2^8.  A NaN or +inf logit makes the
+            // reference NaN, and with it every weight that is not a cubic's: those would lose it in the clamp.
+            const bool grow = !(mt <= m_used + 8.f);
             float alpha = 1.f;
             if (grow) {
-                alpha = (m_used == -INFINITY) ? 0.f : ex2(m_used - mt);
-                m_used = mt;
+                const float m_new = mt < INFINITY ? mt : NAN;
+                alpha = (m_used == -INFINITY) ? 0.f : ex2(m_used - m_new);
+                m_used = m_new;
             }
             // the previous product is in O, has read P and is done with its stage (asked for as late as P is written: the
             // issuing warp takes it up behind a product of the other query tile)

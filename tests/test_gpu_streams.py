@@ -126,3 +126,18 @@ def test_linear_state_is_the_fp32_sum_of_its_pieces(H, d, df, N):
     for _ in range(pieces):
         want = want + chunks
     assert S.unique().tolist() == [float(want)]
+
+
+@pytest.mark.parametrize("bad", [float("nan"), float("inf")])
+@pytest.mark.parametrize("d,N,key", [
+    (64, 400, 0), (64, 400, 8), (64, 400, 131), (128, 700, 0), (128, 700, 17), (128, 700, 250), (128, 1300, 70),
+])
+def test_nan_and_infinite_logits_make_the_output_nan(d, N, key, bad):
+    # One key of one KV head, also in columns whose exponential is the cubic: every row that sees it is NaN in every column, as
+    # inf - inf and NaN are, and no other row.  (Q > 0, so that the logit is +inf and not -inf.)
+    w = _workload(4, 2, d, N, 64, 64)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    K[:, 0, key] = bad
+    Y = still.hybrid_attn_fwd(U.params_of(w), Q.abs() + 1, K, V)[0]
+    assert bool(torch.isnan(Y[:, :2, key:]).all())
+    assert bool(torch.isfinite(Y[:, :2, :key]).all()) and bool(torch.isfinite(Y[:, 2:]).all())
