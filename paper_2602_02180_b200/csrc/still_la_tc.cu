@@ -468,7 +468,7 @@ __global__ void __launch_bounds__(384, 1)
 la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_wq,
                 const __grid_constant__ CUtensorMap tm_phik, const __grid_constant__ CUtensorMap tm_v,
                 const __grid_constant__ CUtensorMap tm_phiks, const __grid_constant__ CUtensorMap tm_vs,
-                const __grid_constant__ CUtensorMap tm_y,
+                const __grid_constant__ CUtensorMap tm_y0, const __grid_constant__ CUtensorMap tm_y1,   // (a map per part: rows in 31 bits)
                 const __nv_bfloat16 *bq, const __nv_bfloat16 *G,
                 const int32_t *sel_idx, const float *zpre, __nv_bfloat16 *y_part,
                 float *d_part, float *S_out, float *seg_sums, int *status, int H, int Hkv,
@@ -973,7 +973,7 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 if (G == nullptr && base + 64 <= N) {
                     if (tid == 0) {
 #pragma unroll
-                        for (int a = 0; a < D / 64; ++a) tma_store_2d(&tm_y, stg + a * (64 * 128), a * 64, (int)((half * gridDim.x + bh) * N) + base);
+                        for (int a = 0; a < D / 64; ++a) tma_store_2d(half ? &tm_y1 : &tm_y0, stg + a * (64 * 128), a * 64, bh * N + base);
                         bulk_store_commit();
                     }
                 } else {   // with a gate, and the last rows of a sequence
@@ -1226,11 +1226,12 @@ int launch_fused(const still_params_t *p, long long N, const void *Q, const void
                  float *S_out, float *seg_sums, void *phiK_sel, void *v_sel, long long sel_rows, int *status, cudaStream_t st,
                  int *launches) {
     using bf = __nv_bfloat16;
-    CUtensorMap tq, tw, tk, tv, tks, tvs, ty;
+    CUtensorMap tq, tw, tk, tv, tks, tvs, ty0, ty1;
     const unsigned long long BH = (unsigned long long)p->B * p->H, BHkv = (unsigned long long)p->B * p->Hkv;
     if (!make_map_2d(&tq, Q, BH * N, D, 128, false) || !make_map_2d(&tw, Wq, (unsigned long long)p->H * D, DF, D, false) ||
         !make_map_2d(&tk, phiK, BHkv * N, 2 * DF, FusedPlan<D, DF>::kUTok, false) ||
-        !make_map_2d(&tv, V, BHkv * N, D, FusedPlan<D, DF>::kUTok, false) || !make_map_2d(&ty, y_part, 2 * BH * N, D, 64, false))
+        !make_map_2d(&tv, V, BHkv * N, D, FusedPlan<D, DF>::kUTok, false) || !make_map_2d(&ty0, y_part, BH * N, D, 64, false) ||
+        !make_map_2d(&ty1, (bf *)y_part + BH * N * D, BH * N, D, 64, false))
         return STILL_ERR_CUDA;
     // With a salient-cache budget and topk < chunk the leaving tokens are read from gathered copies of their rows
     // (otherwise every token of a chunk is selected and the chunk's own tiles are the leaving tiles).
@@ -1253,7 +1254,7 @@ int launch_fused(const still_params_t *p, long long N, const void *Q, const void
     for (int pass = n_seg > 1 && !again ? 0 : 1; pass < 2; ++pass) {
         // pass 0 (only with several segments): the sum of every segment's own updates; pass 1: the scan proper
         dim3 grid((unsigned)BH, 2, (unsigned)(pass == 0 ? (n_seg - 1) * parts : n_seg));   // head, feature half, segment (piece)
-        const cudaError_t e = launch_dependent(la_fused_kernel<D, DF>, grid, dim3(384), Plan::kTotal, st, tq, tw, tk, tv, tks, tvs, ty, (const bf *)bq, (const bf *)G, sel_idx, zpre,
+        const cudaError_t e = launch_dependent(la_fused_kernel<D, DF>, grid, dim3(384), Plan::kTotal, st, tq, tw, tk, tv, tks, tvs, ty0, ty1, (const bf *)bq, (const bf *)G, sel_idx, zpre,
                                                                (bf *)y_part, d_part, S_out, seg_sums, status, p->H, p->Hkv, (int)N,
                                                                p->chunk, p->topk, p->topk > 0 ? (int)(p->max_salient / p->topk) : 0,
                                                                (long long)BH * N * D, (long long)BH * N,
@@ -1293,7 +1294,7 @@ int tc_la_branch(const still_params_t *p, long long N, const void *Q, const void
                  float *csum, float *zpre, void *y_part, float *d_part, float *seg_sums, float *S_out, float *z_out,
                  void *phiK_sel, void *k_sel, void *v_sel, long long sel_rows, int *status_words, cudaStream_t st, int *launches) {
     using bf = __nv_bfloat16;
-    if ((long long)p->B * p->H * N >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;  // TMA row coordinate (y_part's 2^32 rows would be 0.5 TB)
+    if ((long long)p->B * p->H * N >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;  // TMA row coordinate
     const int NF = 2 * p->d_f, C = p->chunk;
     const long long Tn = (N + C - 1) / C, BH = (long long)p->B * p->H;
     const int n_routed = Tn >= 3 ? (int)(Tn - 2) : 0;

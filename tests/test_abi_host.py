@@ -139,6 +139,16 @@ def test_producers_leave_no_load_in_flight():
     assert re.search(r"mbar_drain_ring\(x_full, 1, nx, t1\);\s*mbar_drain_ring\(u_full, n_stages, nu, t1\);", scan)
 
 
+def test_tensor_map_rows_stay_below_the_guard():
+    # Calls are taken up to B H N < 2^31 rows of a tensor, and a TMA row is a signed 32-bit coordinate.  So no map of the scan
+    # spans more than one tensor of that many rows, and the row of its stores counts rows of one part.
+    la = _csrc("still_la_tc.cu")
+    assert "if ((long long)p->B * p->H * N >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;" in la
+    rows = re.findall(r"make_map_2d\(&t\w+, [^,]*(?:\([^)]*\))?[^,]*, ([^,]*),", la.split("int launch_fused(", 1)[1])
+    assert len(rows) >= 8 and set(rows) <= {"BH * N", "BHkv * N", "(unsigned long long)p->H * D", "BH * (unsigned long long)sel_rows"}
+    assert re.search(r"tma_store_2d\([^;]*, bh \* N \+ base\);", la)
+
+
 def test_shared_arrays_that_vectors_are_stored_to_are_aligned():
     # A shared array is only as aligned as its element type unless it says more: those without an explicit alignment are
     # the ones that are accessed element by element (or, smem_raw, aligned by hand).
