@@ -47,6 +47,8 @@ namespace {
 
 using namespace ptx;
 
+constexpr int kSms = 148;   // SMs that grids are planned for
+
 // Instruction descriptor of kind::tf32 (fp32 accumulation, both operands TF32, B K-major).
 __host__ __device__ constexpr uint32_t make_idesc_tf32(int M, int N) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
@@ -1214,11 +1216,17 @@ int launch_gather(const still_params_t *p, long long N, const void *K, const voi
                             N, p->topk, sel_rows, n_routed) == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
 }
 
-// Update tiles up to which every segment of the scan folds the chunks before it itself.  (us a call, folding again / a pass of
-// sums, a quarter kept: 32 heads, d = 128, 16 tiles 76.9 / 90.5, 32: 131.9 / 144.3, 48: 192.1 / 199.4, 64: 248.6 / 253.3, 96: 363.9 /
-// 360.9; d = 64, 64 tiles 168.5 / 170.3; C = 128, 64 tiles 258.4 / 261.5; 16 heads, 48 tiles 90.5 / 106.1, 96: 162.5 / 169.2,
-// 192: 315 / 290; 4 heads, d = 64, 96 tiles 93.9 / 78.7.)
-constexpr int kFoldAllTiles = 64;
+// Whether every segment of the scan folds the chunks before it itself, rather than starting from a pass of sums: up to a
+// number of update tiles before the last segment, 64 where the pass has more CTAs than SMs; fewer where they run at once,
+// its time then being that of one piece.  (Gain of folding in % of a call, C = 64, a quarter kept.  One wave, d = 64: 1 to 4
+// heads 16 tiles 4 to 8, 24 2 to 4, 48 -5 to -6, 72 -11 to -13, 96 -18; d = 128: 16 10 to 11, 24 5 to 6, 48 1 to 3, 72 -5 to -8,
+// 96 -12 to -15; C = 128: 32 tiles 1 to 5, 48 -4 to 2.  Two waves, 8 heads: 48 tiles 1 at d = 64, 7 at 128, 72 -6 and -1, 96 -12
+// and -6; 32 heads: 16 tiles 15 and 17, 32 9 and 11, 64 2 and 3, 96 -1 and 0, 128 -3 and -2.  Three, 16 heads: 48 tiles 8 and 17,
+// 72 1 and 9, 96 -3 and 3, 144 -8 and -5.)
+bool fold_again(const still_params_t *p, int n_seg, int seg_chunks, int parts, int tiles_per_chunk) {
+    const long long pass_ctas = 2ll * p->B * p->H * (n_seg - 1) * parts, tiles = (long long)(n_seg - 1) * seg_chunks * tiles_per_chunk;
+    return n_seg > 1 && tiles <= (pass_ctas > kSms ? 64 : p->d == 64 ? 40 : 48);
+}
 
 template <int D, int DF>
 int launch_fused(const still_params_t *p, long long N, const void *Q, const void *V, const void *G, const void *Wq,
@@ -1248,9 +1256,9 @@ int launch_fused(const still_params_t *p, long long N, const void *Q, const void
     if (ensure_dynamic_smem((const void *)la_fused_kernel<D, DF>, Plan::kTotal) != cudaSuccess) return STILL_ERR_CUDA;
     int seg_chunks = 0;
     const int n_seg = tc_la_segments(p, N, &seg_chunks), parts = tc_la_sum_parts(seg_chunks);
-    // The chunks before the last segment are folded again by every segment where that is a short stretch of update tiles, and
-    // summed by a pass of its own where it is not.
-    const bool again = n_seg > 1 && (long long)(n_seg - 1) * seg_chunks * (p->chunk / Plan::kUTok) * (p->max_salient > 0 ? 2 : 1) <= kFoldAllTiles;
+    // (tiles of a chunk, and of the tokens that leave a capped cache with it: see the kernel)
+    const int su = p->chunk / Plan::kUTok, nl = gathered ? (p->topk + Plan::kUTok - 1) / Plan::kUTok : su;
+    const bool again = fold_again(p, n_seg, seg_chunks, parts, p->max_salient > 0 ? su + nl : su);
     for (int pass = n_seg > 1 && !again ? 0 : 1; pass < 2; ++pass) {
         // pass 0 (only with several segments): the sum of every segment's own updates; pass 1: the scan proper
         dim3 grid((unsigned)BH, 2, (unsigned)(pass == 0 ? (n_seg - 1) * parts : n_seg));   // head, feature half, segment (piece)
@@ -1277,7 +1285,7 @@ bool tc_la_supported(const still_params_t *p) {
 int tc_la_segments(const still_params_t *p, long long N, int *seg_chunks) {
     const long long Tn = (N + p->chunk - 1) / p->chunk, ctas = 2ll * p->B * p->H;
     int n_seg = 1;
-    while (n_seg < 4 && ctas * (n_seg * 2) <= 148 && Tn / (n_seg * 2) >= 8) n_seg *= 2;
+    while (n_seg < 4 && ctas * (n_seg * 2) <= kSms && Tn / (n_seg * 2) >= 8) n_seg *= 2;
     long long sc = (Tn + n_seg - 1) / n_seg;
     sc += sc & 1;
     if (seg_chunks) *seg_chunks = (int)sc;

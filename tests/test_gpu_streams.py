@@ -95,7 +95,8 @@ def test_both_head_dims_give_the_same_rows(N, C, k, budget):
     (16, 128, 128, 2048),                       # four segments: eleven pieces
     (16, 64, 64, 2500),                         # pieces of five chunks
     (32, 128, 128, 3000),                       # pieces of six chunks
-    (4, 64, 64, 3000),                          # a pass of sums
+    (4, 128, 128, 2048), (8, 64, 64, 2048),     # 48 tiles, folded again in one wave at d = 128 and in two
+    (4, 64, 64, 2048), (4, 64, 64, 3000),       # ... a pass of sums at d = 64; 72 tiles
 ])
 def test_linear_state_is_the_fp32_sum_of_its_pieces(H, d, df, N):
     # W_k = 0 makes every feature 1 / d_f exactly.  Chunk 0 brings 2^24 into the state of every head, whose neighbours in fp32
