@@ -29,14 +29,13 @@
 //   The lag of two chunks between update and read-out is the delayed selection of Sec. 3.3.  Work is
 //   tiled in 64-token sub-chunks, so C = 128 is two sub-chunks per chunk.
 //
-// Roles of la_fused_kernel (384 threads): warp 0 TMA producer, warp 1 MMA issuer, warp 2 zeroes the
+// Roles of la_fused_kernel (384 threads): warp 0 TMA producer, warp 1 MMA issuer, warps 2 and 3 take turns at zeroing the
 // selected rows of the phi(K) tiles, warps 4-7 write the output, warps 8-11 the query-side map.  Every mbarrier
 // wait is bounded; on expiry the kernel records STILL_ERR_DEVICE_TIMEOUT in the status word, all roles
 // leave their loops and tensor memory is freed before the CTA exits.
 #include "still_tc.h"
 
 #include <algorithm>
-#include <type_traits>
 
 #include "still_common.cuh"
 #include "still_tc_ptx.cuh"
@@ -52,15 +51,6 @@ constexpr int kSms = 148;   // SMs that grids are planned for
 // Instruction descriptor of kind::tf32 (fp32 accumulation, both operands TF32, B K-major).
 __host__ __device__ constexpr uint32_t make_idesc_tf32(int M, int N) {
     return (1u << 4) | (2u << 7) | (2u << 10) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(M >> 4) << 24);
-}
-// D[tmem] (+)= A[tmem, fp32 read as TF32] * B[smem desc]
-__device__ __forceinline__ void mma_ts_tf32(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                            uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::tf32 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
 }
 
 // ------------------------------------------------------------------------------------------

@@ -128,16 +128,6 @@ __device__ __forceinline__ void mma_ss(uint32_t d_tmem, uint64_t a_desc, uint64_
         ::"r"(d_tmem), "l"(a_desc), "l"(b_desc), "r"(idesc), "r"(accumulate)
         : "memory");
 }
-// D[tmem] (+)= A[tmem] * B[smem desc]
-__device__ __forceinline__ void mma_ts(uint32_t d_tmem, uint32_t a_tmem, uint64_t b_desc, uint32_t idesc,
-                                       uint32_t accumulate) {
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.b32 p, %4, 0;\n\t"
-        "tcgen05.mma.cta_group::1.kind::f16 [%0], [%1], %2, %3, p;\n\t}"
-        ::"r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate)
-        : "memory");
-}
-
 // Shared-memory descriptor split in two words so that a k-step only adds a constant to the low
 // word: low = start address / 16 (bits 0-13) | leading-dimension byte offset / 16 (bits 16-29);
 // high = 1024 / 16 (stride between 8-row groups) | descriptor version 1 (bit 46) | SWIZZLE_128B (bits 61-63).
@@ -195,11 +185,6 @@ __device__ __forceinline__ void mma_ts_lo(uint32_t d_tmem, uint32_t a_tmem, uint
 // and half of the B operand (N / 2), and receives its 128 rows of D in its own tensor memory.  One thread
 // of the pair's first CTA (cluster rank 0) issues for both.
 
-__device__ __forceinline__ uint32_t cluster_ctarank() {
-    uint32_t r;
-    asm volatile("mov.u32 %0, %%cluster_ctarank;" : "=r"(r));
-    return r;
-}
 // Address, in the cluster's shared-memory window, of the CTA `rank`'s copy of a shared-memory location.
 __device__ __forceinline__ uint32_t mapa(uint32_t saddr, uint32_t rank) {
     uint32_t r;
