@@ -21,6 +21,8 @@ def _workload(H, Hkv, d, N, C, k):
     (128, 1, 64, 16, 0), (128, 256, 64, 64, 0), (128, 257, 128, 32, 0), (128, 512, 64, 16, 0), (128, 513, 64, 16, 0),
     # shared tiles that run through the ring several times, and own tiles of both query tiles behind them
     (64, 2111, 64, 64, 0), (128, 2303, 64, 64, 0), (128, 2200, 128, 1, 0),
+    # a CTA pair whose last rows are few: the first query tile goes on after the second has no more
+    (128, 820, 64, 16, 0), (128, 1836, 64, 16, 64), (128, 1836, 64, 32, 64),
     # windows of the capped cache that two query tiles share in part, or not at all (then every tile is one's own)
     (64, 1500, 64, 16, 64), (64, 1500, 64, 64, 64), (128, 2000, 64, 64, 64), (128, 2000, 128, 32, 32), (128, 2100, 64, 32, 896),
 ])
