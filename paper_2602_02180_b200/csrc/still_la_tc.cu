@@ -452,10 +452,11 @@ static_assert(FusedPlan<128, 128>::kTotal <= 232448 && FusedPlan<128, 64>::kTota
 static_assert(FusedPlan<128, 128>::oStage % 1024 == 0 && FusedPlan<128, 64>::oStage % 1024 == 0 && FusedPlan<64, 64>::oStage % 1024 == 0,
               "fused scan: the staging tile is swizzle-aligned");
 
-// What a launch of la_fused_kernel does (see there).
-enum LaMode { kFromSums = 0, kSumsOnly = 1, kFoldAll = 2 };
+// What a launch of la_fused_kernel does (see there).  Folding again is a kernel of its own: beside the code for it the others
+// took 1 to 2 % longer (128 heads x 4096 tokens, d = 64, a quarter kept: 512 -> 518 us a call).
+enum LaMode { kFromSums, kSumsOnly, kFoldAll };
 
-template <int D, int DF>
+template <int D, int DF, bool kFoldAgain>
 __global__ void __launch_bounds__(384, 1)
 la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_wq,
                 const __grid_constant__ CUtensorMap tm_phik, const __grid_constant__ CUtensorMap tm_v,
@@ -465,7 +466,7 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 const int32_t *sel_idx, const float *zpre, __nv_bfloat16 *y_part,
                 float *d_part, float *S_out, float *seg_sums, int *status, int H, int Hkv,
                 int N, int C, int lam, int window, long long part_stride_y, long long part_stride_d, int seg_chunks, int n_seg,
-                int sum_parts, int mode, int sel_rows) {
+                int sum_parts, int sums_pass, int sel_rows) {
     grid_dep_wait();
     grid_dep_launch();
     using P = FusedPlan<D, DF>;
@@ -477,6 +478,7 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     uint64_t *pq_full = bars + 5, *pq_empty = bars + 7, *r_done = bars + 9, *out_free = bars + 11, *fin = bars + 13;
     uint64_t *init_done = bars + 14, *u_full = bars + 18, *u_empty = u_full + P::kMaxStages, *u_masked = u_empty + P::kMaxStages;
     constexpr int kUTok = P::kUTok;
+    const LaMode mode = kFoldAgain ? kFoldAll : sums_pass ? kSumsOnly : kFromSums;
     const bool sums_only = mode == kSumsOnly;
     const int n_stages = sums_only ? P::kSumStages : P::kUStages;
     uint8_t *ring = smem + (sums_only ? 0 : P::oU);
@@ -541,9 +543,9 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     const int chunk0 = mode == kFoldAll ? 0 : u_first / sc - 2;   // first chunk that the segment folds
     const int n_upd = NU > u_first ? ((NU - 1) / sc - 1 - chunk0) * per_chunk : 0;
     const bool has_init = mode == kFromSums && seg > 0;
-    // Pieces of what a segment folds before its own updates.  The sequence's first two chunks answer nothing, so the first
+    // Pieces of what a segment folds before its own updates, one after the other (a pass of sums has one).  The sequence's first two chunks answer nothing, so the first
     // piece is two chunks shorter than the others: with pieces of two chunks it is empty and there is one less.
-    const int n_pieces = mode == kFoldAll && n_upd > 0 ? seg * sum_parts - (seg > 0 && piece_chunks == 2 ? 1 : 0) : 0;
+    const int n_pieces = sums_only ? 1 : mode == kFoldAll && n_upd > 0 ? seg * sum_parts - (seg > 0 && piece_chunks == 2 ? 1 : 0) : 0;
     __nv_bfloat16 *y_out = y_part + (long long)half * part_stride_y;
     float *d_out = d_part + (long long)half * part_stride_d;
 
@@ -596,7 +598,7 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     auto col_piece = [&](int n) -> uint32_t { return (n & 1) ? col_out : col_f + DF; };
 
     // Registers move from the first warpgroup (single-thread roles) to the map warps, whose threads hold a row of f
-    // (per scheduler: 72 + 152 + 224 registers for its three warps, of the 3 x 168 the CTA was launched with).
+    // (per scheduler: 72 + 160 + 224 registers for its three warps, of the 3 x 168 the CTA was launched with).
     if (warp < 4) {
     reg_dec<72>();
     if (warp == 0) {
@@ -715,10 +717,8 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
                 ++nu;
             };
             if (NB > b_first) issue_f();
-            if (sums_only)
-                while (nu < n_upd) issue_update(col_state, nu > 0);
             for (int g = 0; g < n_pieces; ++g) {
-                const int tiles = (g == 0 && piece_chunks > 2 ? piece_chunks - 2 : piece_chunks) * per_chunk;
+                const int tiles = sums_only ? n_upd : (g == 0 && piece_chunks > 2 ? piece_chunks - 2 : piece_chunks) * per_chunk;
                 const uint32_t col = g == 0 ? col_state : col_piece(nq);
                 if (g > 0) wait(out_free + (nq & 1), ((nq >> 1) & 1) ^ 1, 74);
                 for (int i = 0; i < tiles; ++i) issue_update(col, i > 0);
@@ -834,7 +834,7 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         }
     }
     } else if (warp < 8) {
-        reg_dec<152>();
+        reg_dec<160>();
         // ------------------------------------------------------------ workers: output
         const int wq = warp & 3;                     // TMEM lane quarter this warp may read
         const int e = wq * 32 + lane;                // value column (lane of S^T and of the read-out result)
@@ -842,6 +842,27 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
         const int tid = threadIdx.x - 128;           // 0..127
         bool ok = true;
         int nq = 0;
+        for (int g = 1; g < n_pieces; ++g, ++nq) {
+            if (ok) ok = mbar_wait(r_done + (nq & 1), (nq >> 1) & 1, abort_flag, status, 76);
+            ok = __all_sync(0xffffffffu, ok);
+            if (ok) {   // (the commit behind a piece's updates covers those of the pieces before it)
+                tc_fence_after();
+#pragma unroll 1
+                for (int q = 0; q < DF / 32; ++q) {
+                    uint32_t sum[32], add[32];
+                    tmem_ld32(taddr + col_state + q * 32, sum);
+                    tmem_ld32(taddr + col_piece(nq) + q * 32, add);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) sum[j] = __float_as_uint(__uint_as_float(sum[j]) + __uint_as_float(add[j]));
+                    tmem_st32(taddr + col_state + q * 32, sum);
+                }
+                tmem_wait_st();
+                tc_fence_before();
+                __syncwarp();
+                if (lane == 0) mbar_arrive(out_free + (nq & 1));
+            }
+        }
         // rows of the first two chunks see an empty state
         if (seg == 0 && !sums_only) {
             const int n0 = min(N, 2 * C);
@@ -876,27 +897,6 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
             tc_fence_before();
             __syncwarp();
             if (lane == 0) mbar_arrive(init_done);
-        }
-        for (int g = 1; g < n_pieces; ++g, ++nq) {
-            if (ok) ok = mbar_wait(r_done + (nq & 1), (nq >> 1) & 1, abort_flag, status, 76);
-            ok = __all_sync(0xffffffffu, ok);
-            if (ok) {   // (the commit behind a piece's updates covers those of the pieces before it)
-                tc_fence_after();
-#pragma unroll 1
-                for (int q = 0; q < DF / 32; ++q) {
-                    uint32_t sum[32], add[32];
-                    tmem_ld32(taddr + col_state + q * 32, sum);
-                    tmem_ld32(taddr + col_piece(nq) + q * 32, add);
-                    tmem_wait_ld();
-#pragma unroll
-                    for (int j = 0; j < 32; ++j) sum[j] = __float_as_uint(__uint_as_float(sum[j]) + __uint_as_float(add[j]));
-                    tmem_st32(taddr + col_state + q * 32, sum);
-                }
-                tmem_wait_st();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) mbar_arrive(out_free + (nq & 1));
-            }
         }
         constexpr int kPiecesPerRow = D / 8, kPieces = 64 * kPiecesPerRow / 128;   // 16-byte pieces per thread and sub-chunk
         for (int u = u_first; u < NU && !sums_only; ++u) {
@@ -1243,20 +1243,21 @@ int launch_fused(const still_params_t *p, long long N, const void *Q, const void
             return STILL_ERR_CUDA;
     }
     using Plan = FusedPlan<D, DF>;
-    if (ensure_dynamic_smem((const void *)la_fused_kernel<D, DF>, Plan::kTotal) != cudaSuccess) return STILL_ERR_CUDA;
     int seg_chunks = 0;
     const int n_seg = tc_la_segments(p, N, &seg_chunks), parts = tc_la_sum_parts(seg_chunks);
     // (tiles of a chunk, and of the tokens that leave a capped cache with it: see the kernel)
     const int su = p->chunk / Plan::kUTok, nl = gathered ? (p->topk + Plan::kUTok - 1) / Plan::kUTok : su;
     const bool again = fold_again(p, n_seg, seg_chunks, parts, p->max_salient > 0 ? su + nl : su);
+    const auto kernel = again ? la_fused_kernel<D, DF, true> : la_fused_kernel<D, DF, false>;
+    if (ensure_dynamic_smem((const void *)kernel, Plan::kTotal) != cudaSuccess) return STILL_ERR_CUDA;
     for (int pass = n_seg > 1 && !again ? 0 : 1; pass < 2; ++pass) {
         // pass 0 (only with several segments): the sum of every segment's own updates; pass 1: the scan proper
         dim3 grid((unsigned)BH, 2, (unsigned)(pass == 0 ? (n_seg - 1) * parts : n_seg));   // head, feature half, segment (piece)
-        const cudaError_t e = launch_dependent(la_fused_kernel<D, DF>, grid, dim3(384), Plan::kTotal, st, tq, tw, tk, tv, tks, tvs, ty0, ty1, (const bf *)bq, (const bf *)G, sel_idx, zpre,
+        const cudaError_t e = launch_dependent(kernel, grid, dim3(384), Plan::kTotal, st, tq, tw, tk, tv, tks, tvs, ty0, ty1, (const bf *)bq, (const bf *)G, sel_idx, zpre,
                                                                (bf *)y_part, d_part, S_out, seg_sums, status, p->H, p->Hkv, (int)N,
                                                                p->chunk, p->topk, p->topk > 0 ? (int)(p->max_salient / p->topk) : 0,
                                                                (long long)BH * N * D, (long long)BH * N,
-                                                               seg_chunks, n_seg, parts, pass == 0 ? kSumsOnly : again ? kFoldAll : kFromSums, gathered ? (int)sel_rows : 0);
+                                                               seg_chunks, n_seg, parts, pass == 0 ? 1 : 0, gathered ? (int)sel_rows : 0);
         if (e != cudaSuccess) return STILL_ERR_CUDA;
         ++*launches;
     }
