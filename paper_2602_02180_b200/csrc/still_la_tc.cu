@@ -428,8 +428,8 @@ struct FusedPlan {
     static constexpr int kPhiQ = 64 * DF * 4;           // phi_q half of 64 tokens, fp32 (TF32 operand)
     static constexpr int kUTok = 32;                    // tokens per state-update tile
     static constexpr int kUStages = 4;                  // ring of update tiles (loads run this far ahead of the MMAs)
-    // ... of the pass that only sums, whose ring takes the room of W_q, Q and phi(Q) too: with four stages a tile cost it 920
-    // cycles, a quarter of a load's way from memory.  (131072 tokens x 32 heads, C = 128, capped at 896: 8.53 -> 8.20 ms a call.)
+    // ... of the pass that only sums, whose ring takes the room of W_q, Q and phi(Q) too: it does nothing but wait for its loads
+    // (with four stages 920 cycles a tile; 32768 tokens x 32 heads, d = 128: 136 us, with twelve 101).
     static constexpr int kMaxStages = 12;
     static constexpr int kPhiK = kUTok * DF * 2;        // phi_k half of an update tile, bf16
     static constexpr int kVt = kUTok * D * 2;           // V of an update tile
@@ -522,8 +522,9 @@ la_fused_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant_
     // The first pass cuts every segment into sum_parts pieces, one CTA each (it has no scan to keep in order, and
     // the pieces fill the SMs that the n_seg - 1 summed segments alone would leave idle).  A segment that folds itself
     // forms the same pieces, one after the other, each from zero, and adds them up in fp32 as the other does: carried
-    // through the accumulators, the state would take their rounding (with all-positive values a third to a half more
-    // error of S than the sum of the pieces), and how a call is launched would show in its results.
+    // through the accumulators, the state would take their rounding (with exact features and positive values S was 5 to 47 %
+    // further from float64 than as the sum of the pieces: 2.05e-7 and 1.39e-7 for 16 heads x 2048 tokens, d = 128), and how a
+    // call is launched would show in its results.
     const int seg = blockIdx.z;
     const int piece_chunks = seg_chunks / sum_parts;
     if (sums_only) seg_chunks = piece_chunks;

@@ -527,11 +527,12 @@ __device__ __forceinline__ void producer_role(const Stream &st, const AttnBars &
 // Q K^T runs three items ahead of P V: P_A V, Q_B K^T of B's next tile, P_B V, Q_A K^T of A's next but one, and so on.
 // S of A's next tile is then complete when its softmax warps come back for it, and where S_A and S_B share their place
 // the warps of A have read theirs by the time B's is to be formed.  What bounds the kernel is then the softmax warps'
-// arithmetic, two of them per scheduler (issue slots 49 %, special-function unit 45 %, tensor pipe 62 %), and for short
-// streams the start and the end of a CTA.  With P over S, S of a tile waited for the softmax warps of the tile before
-// and these for it: 32768 tokens x 64 heads, d = 128, every token kept 15.07 ms a call (now 14.3), a quarter 5.99 (5.6),
-// 131072 x 32, capped at 896, 8.53 (7.65); 4096 x 128, d = 64, every token 554 us (512), a quarter 588 (560).  Two
-// threads per row instead of one (16 softmax warps) were slower by 10 %: the stream's bookkeeping doubles.
+// arithmetic, two of them per scheduler (32768 tokens, d = 128: issue slots 52 %, special-function unit 51 %, tensor pipe 69 %;
+// 4096 tokens, d = 64: 50, 45 and 30 %), and for short streams the start and the end of a CTA.  With P over S, S of a tile
+// waited for the softmax warps of the tile before and these for it (us a call, then and now, in turn on one box: 64 heads x 32768
+// tokens, d = 128, every token kept 15887 and 15154, a quarter 6665 and 6208; 32 x 131072, capped at 896, 8697 and 7809; 128 x
+// 4096, d = 64, every token 551 and 502, a quarter 585 and 515; the scan and the score kernel have a part in the quarters and in
+// the capped call).  Two threads per row instead of one (16 softmax warps) were slower by 10 %: the stream's bookkeeping doubles.
 template <int D, bool kPair, class TellPeer>
 __device__ __forceinline__ void mma_role(const Stream &st, const AttnBars &bar, uint8_t *smem, const uint32_t tmem_base,
                                          volatile int *abort_flag, int *status, TellPeer tell_peer) {
@@ -805,10 +806,10 @@ sa_merge_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_cons
 // (tile n = head n / n_row_blocks, rows 128 (n % n_row_blocks) ...) with two stages of shared memory and two
 // TMEM accumulators, so that the loads of tile n+1 and its UMMA run under the row epilogue of tile n.
 // The row's epilogue bounds it: three special-function instructions per window element (one 2^x, two logarithms) against
-// six or seven others, by eight warps an SM, two tiles at a time (special-function unit 45 % busy, issue slots 40 %,
-// DRAM 34 % at d = 128, C = 64).  With the ranking as it was before (see below), 2 x 32 heads x 32768 tokens, d = 128, C = 64: 222 us, 4 x 32 x 4096, d = 64: 59 us, 32 x 131072,
-// d = 128, C = 128: 807 us (with scalar arithmetic, logarithms for subnormal arguments, and for C = 128 a second set of
-// exponentials: 325 to 368, 83 and 1030 us).
+// six or seven others, by eight warps an SM, two tiles at a time (d = 128, C = 64: special-function unit 53 % busy, issue slots
+// 38 %, DRAM 38 %; C = 128: 61, 37 and 24 %).  2 x 32 heads x 32768 tokens, d = 128, C = 64: 199 us, 4 x 32 x 4096, d = 64: 51 us,
+// 32 x 131072, d = 128, C = 128: 650 us (with a threshold per token in the ranking, see below: 223, 58 and 825; with scalar
+// arithmetic, logarithms for subnormal arguments, and for C = 128 a second set of exponentials as well: 325 to 368, 83 and 1030).
 // Warps: 0 TMA producer, 1 MMA issuer, 2-5 score group 0 (even tiles of the CTA), 6-9 score group 1 (odd
 // tiles); TMEM lane quarter = warp % 4.
 // ---------------------------------------------------------------------------
