@@ -7,7 +7,8 @@
 namespace still {
 
 // Words of the 256-byte status block at the start of a workspace / decode state.
-enum StatusWord { kStatusCode = 0, kStatusDetail = 1 };
+// kNextItem (of a workspace): items of the attention kernel handed out beyond the first of every CTA.
+enum StatusWord { kStatusCode = 0, kStatusDetail = 1, kNextItem = 32 };
 
 // Kernels of one call are launched with programmatic stream serialization (launch_dependent): a kernel's blocks are made
 // resident as soon as all blocks of its predecessor run, and wait here until the predecessor has ended and its writes are

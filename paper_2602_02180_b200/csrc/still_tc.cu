@@ -8,8 +8,8 @@
 // ascending position), so that "selected tokens of chunks 0..c-2" is the prefix
 // [0, (c-1)*lambda) of a contiguous array that TMA can tile.
 //
-// One CTA owns 256 consecutive query rows of one (batch, head), a pair of CTAs 512: two query tiles A and B of 128
-// (256) rows.  Their keys come as a stream of 128-key tiles: SEL tiles j (rows [128j, 128j+128) of K_sel / V_sel), and
+// An item is 256 consecutive query rows of one (batch, head), for a pair of CTAs 512: two query tiles A and B of 128
+// (256) rows.  CTAs stay and take one item after the other (Work).  The keys of an item come as a stream of 128-key tiles: SEL tiles j (rows [128j, 128j+128) of K_sel / V_sel), and
 // the LOC tiles around the rows (rows of K / V at positions [128m, 128m+128)).  First the SEL tiles that both query
 // tiles see (before them what has already left the window of B), then what only one of them sees, by turns.  Which
 // columns of a tile a query row sees is a per-row column interval, applied as a mask in the softmax.
@@ -17,11 +17,11 @@
 // Warp roles (384 threads):
 //   warps 0-7  softmax, four warps per query tile, one thread per query row (tcgen05.ld of the S row): online softmax in
 //              the log2 domain with lazy rescaling of O, P to TMEM as bf16; then the epilogue: O / l merged with the
-//              linear branch (N_LA, D_LA) under one denominator and stored as bf16
-//   warp 8     TMA producer: Q tiles once, then K and V tiles through mbarrier rings
+//              linear branch (N_LA, D_LA) under one denominator and left in shared memory as bf16
+//   warp 8     TMA producer: Q tiles of an item, then K and V tiles and the linear branch's results through one ring
 //   warp 9     MMA issuer (one elected thread): S = Q_X K^T (operands in shared memory, SWIZZLE_128B K-major),
 //              O_X += P_X V (P_X read from TMEM, V in shared memory MN-major)
-//   (warps 10, 11 only give up their registers)
+//   warps 10, 11  output: the rows of query tile A, of B, to memory by TMA
 //
 // Every mbarrier wait is bounded: on expiry the kernel records
 // STILL_ERR_DEVICE_TIMEOUT in the status word, all roles leave their loops, and
@@ -58,37 +58,54 @@ struct AttnPlan {
     static constexpr int kKTile = kKRows * D * 2;
     static constexpr int kVTile = kBlockN * kVCols * 2;
     static constexpr int kStages = 5;                          // of the ring: a K and a V tile each
+    static constexpr int kStage = kKTile + kVTile;
+    // The output of a query tile leaves through stages of the ring (entries behind the item's keys), which the linear
+    // branch's partial results come in by: at D = 128 a stage a part, at D = 64 both parts in one.
+    static constexpr int kPartTile = kBlockM * D * 2, kPartsPerStage = kStage / kPartTile;
     static constexpr int kQ = 0;
-    static constexpr int kK = kQ + 2 * kQTile;
-    static constexpr int kV = kK + kStages * kKTile;
-    static constexpr int kBar = kV + kStages * kVTile;         // mbarriers
-    static constexpr int kNumBars = 1 + 2 * kStages + 2 + 2 + 2 + 2 + 1;
-    static constexpr int kMisc = kBar + kNumBars * 8;          // tmem base, abort flag, "a CTA has failed before"
-    static constexpr int kTotal = kMisc + 16;
+    static constexpr int kK = kQ + 2 * kQTile;                 // stage s at kK + s kStage: its K tile, then its V tile
+    static constexpr int kV = kK + kKTile;
+    static constexpr int kBar = kK + kStages * kStage;         // mbarriers
+    static constexpr int kNumBars = 2 + 2 * kStages + 2 + 2 + 2 + 2 + 4 + 4 + 2;
+    static constexpr int kMisc = kBar + kNumBars * 8;          // tmem base, abort flag, "a CTA has failed before", -, item[2][2]
+    static constexpr int kTotal = kMisc + 32;
     static constexpr int kAlloc = kTotal + 1024;               // slack to align the base to 1024
+    // entries of the ring that the output of a query tile takes
+    __host__ __device__ static constexpr int y_entries(int n_parts) { return n_parts > kPartsPerStage ? 2 : 1; }
+    static_assert(kPartsPerStage == (D == 64 ? 2 : 1) && kKTile == kVTile, "attention kernel: a stage holds both parts at D = 64, one at D = 128");
     static_assert(kAlloc <= kMaxDynamicSmem, "attention kernel: the shared-memory plan exceeds what a CTA can have");
     static_assert(kMisc % 8 == 0 && kKTile % 1024 == 0 && kVTile % 1024 == 0, "attention kernel: operand tiles are swizzle-aligned");
 };
 
 struct AttnBars {
-    uint64_t *q_full;
+    uint64_t *q_full, *q_empty;     // ... and the item's last Q K^T has completed
     uint64_t *kv_full, *kv_empty;   // [kStages]
     uint64_t *s_full;    // [2] S of query tile x is in tensor memory
     uint64_t *s_free;    // [2] ... and has been read
     uint64_t *p_full;    // [2] P_x is in tensor memory
     uint64_t *pv_done;   // [2] O_x includes the tile's product (and P_x may be overwritten)
+    uint64_t *y_full;    // [2] the linear branch's results for query tile x are in their stages
+    uint64_t *y_ready;   // [2] ... and the output is where the first of them were
+    uint64_t *item_full, *item_empty;   // [2] an item to come is there; ... and has been read
+    uint64_t *first_done;   // (of a pair's second CTA) the first CTA's producer is done with an item
     uint64_t *drain;     // MMA warp: everything issued has completed (failure path)
     template <class P>
     __device__ __forceinline__ static AttnBars at(uint8_t *smem, P) {
         AttnBars b;
         b.q_full = reinterpret_cast<uint64_t *>(smem + P::kBar);
-        b.kv_full = b.q_full + 1;
+        b.q_empty = b.q_full + 1;
+        b.kv_full = b.q_empty + 1;
         b.kv_empty = b.kv_full + P::kStages;
         b.s_full = b.kv_empty + P::kStages;
         b.s_free = b.s_full + 2;
         b.p_full = b.s_free + 2;
         b.pv_done = b.p_full + 2;
-        b.drain = b.pv_done + 2;
+        b.y_full = b.pv_done + 2;
+        b.y_ready = b.y_full + 2;
+        b.item_full = b.y_ready + 2;
+        b.item_empty = b.item_full + 2;
+        b.first_done = b.item_empty + 2;
+        b.drain = b.first_done + 1;
         return b;
     }
 };
@@ -101,6 +118,9 @@ struct RingPos {
             stage = 0;
             parity ^= 1;
         }
+    }
+    __device__ __forceinline__ void skip(int n, int n_stages) {
+        for (int i = 0; i < n; ++i) next(n_stages);
     }
 };
 
@@ -128,17 +148,18 @@ struct Stream {
     __device__ __forceinline__ int first_own(int x) const { return n_shared + (x ? 0 : n_lead); }   // (x's tiles before those)
     __device__ __forceinline__ int entries() const { return n_lead + n_shared + n_a + n_b; }
     __device__ __forceinline__ int entries_of(int x) const { return first_own(x) + (x ? n_b : n_a); }
-    __device__ __forceinline__ bool shared(int e) const { return e >= n_lead && e < n_lead + n_shared; }
     // k-th tile of query tile x: a SEL tile, or a LOC tile?  Returns its number.
     __device__ __forceinline__ int tile_of(int x, int k, bool &sel) const {
         const int n = x ? n_sel_b : n_sel_a;
         sel = k < n;
         return k + (sel ? (x ? sel_b : sel_a) : (x ? loc_b : loc_a) - n);
     }
-    // ... and its entry
-    __device__ __forceinline__ int entry(int x, int k) const {
-        const int i = k - first_own(x), turns = min(n_a, n_b);
-        return i < 0 ? k + (x ? n_lead : 0) : n_lead + n_shared + (i < turns ? 2 * i + x : i + turns);
+    // ... as its softmax warps need it
+    struct Mine {
+        int n, n_sel, sel0, loc0;   // tiles, SEL tiles; the first SEL tile, the first LOC tile
+    };
+    __device__ __forceinline__ Mine mine(int x) const {
+        return x ? Mine{entries_of(1), n_sel_b, sel_b, loc_b} : Mine{entries_of(0), n_sel_a, sel_a, loc_a};
     }
     // the tile of entry e
     __device__ __forceinline__ int tile(int e, bool &sel) const {
@@ -167,27 +188,27 @@ __device__ __forceinline__ void row_block(int i, int n_blocks, int n_heads, int 
     bh = bh0 + (i - q * heads);
 }
 
-__device__ __forceinline__ int sel_limit(long long pos, int C, int lam) {  // end of the visible range of K_sel
-    long long c = pos / C;
-    return c >= 2 ? (int)((c - 1) * lam) : 0;
+__device__ __forceinline__ int sel_limit(int pos, int log2_c, int lam) {  // end of the visible range of K_sel
+    const int c = pos >> log2_c;
+    return c >= 2 ? (c - 1) * lam : 0;
 }
 // Start of the visible range: 0, or with a salient-cache budget of `budget` tokens per head (a multiple of lam;
 // the oldest cached tokens have left for the linear state) the last `budget` entries before the end.
 __device__ __forceinline__ int sel_start(int limit, int budget) { return budget > 0 ? max(limit - budget, 0) : 0; }
 
 // The key stream of the query tiles that start at rows R0 and R0 + rows, of `rows` (a multiple of 128) rows each.
-__device__ __forceinline__ Stream make_stream(int R0, int rows, int N, int C, int lam, int budget) {
+__device__ __forceinline__ Stream make_stream(int R0, int rows, int N, int log2_c, int lam, int budget) {
     Stream st;
     const int last_m = (N - 1) / kBlockN, m_a = R0 / kBlockN, m_b = m_a + rows / kBlockN;
     const int last_a = min(R0 + rows, N) - 1, last_b = min(R0 + 2 * rows, N) - 1;
     // SEL tiles [a0, a1) and [b0, b1): a tile's first row sees the oldest entries, its last row the newest
-    const int a0 = sel_start(sel_limit(R0, C, lam), budget) / kBlockN, a1 = (sel_limit(last_a, C, lam) + kBlockN - 1) / kBlockN;
+    const int a0 = sel_start(sel_limit(R0, log2_c, lam), budget) / kBlockN, a1 = (sel_limit(last_a, log2_c, lam) + kBlockN - 1) / kBlockN;
     st.sel_a = a0;
     st.n_sel_a = max(a1 - a0, 0);
     st.loc_a = max(m_a - 1, 0);
     st.n_lead = st.n_shared = st.sel_b = st.n_sel_b = st.loc_b = st.n_b = 0;
     if (R0 + rows < N) {
-        const int b0 = sel_start(sel_limit(R0 + rows, C, lam), budget) / kBlockN, b1 = (sel_limit(last_b, C, lam) + kBlockN - 1) / kBlockN;
+        const int b0 = sel_start(sel_limit(R0 + rows, log2_c, lam), budget) / kBlockN, b1 = (sel_limit(last_b, log2_c, lam) + kBlockN - 1) / kBlockN;
         st.n_shared = max(a1 - b0, 0);                    // (a0 <= b0 and a1 <= b1)
         st.n_lead = st.n_shared > 0 ? b0 - a0 : 0;
         st.sel_b = b0;
@@ -199,21 +220,85 @@ __device__ __forceinline__ Stream make_stream(int R0, int rows, int N, int C, in
     return st;
 }
 
+// What an attention kernel works on, and how its roles come to it.  A CTA (or pair) stays for the whole kernel and takes one
+// item (the rows of two query tiles of a head) after the other: the first by its own number, the others from a counter (of the
+// workspace's status block, which the call's first kernel clears), so that whoever is done first takes the next.  The producer
+// of the first CTA asks for an item while it loads the one before, and hands it to the other roles (of both CTAs) in one of two
+// places.
+struct Work {
+    int n_blocks, n_heads, set_heads, H, Hkv, N, log2_c, lam, budget, sel_rows, sel_identity, n_parts;
+    int rows;          // of a query tile: 128 a CTA
+    int first, total;
+    volatile int *item;   // [2][2]: head (-1: there are no more) and first row
+    int bh, R0;           // the current item
+    __device__ __forceinline__ void set(int i) {
+        int rb;
+        row_block(i, n_blocks, n_heads, set_heads, rb, bh);
+        R0 = rb * 2 * rows;
+    }
+    __device__ __forceinline__ Stream stream() const { return make_stream(R0, rows, N, log2_c, lam, budget); }
+    __device__ __forceinline__ int n_query_tiles() const { return R0 + rows < N ? 2 : 1; }
+};
+// One thread's wait for the n-th of the items that were handed out (n from 0).  Returns whether there is one; `taken` tells that
+// the warp has read it.
+template <bool kPair>
+__device__ __forceinline__ bool next_item(Work &w, const AttnBars &bar, int n, volatile int *abort_flag, int *status, bool &ok) {
+    ok = mbar_wait(bar.item_full + (n & 1), (uint32_t)(n >> 1) & 1u, abort_flag, status, 13);
+    if constexpr (kPair) mbar_acquire_cluster(bar.item_full + (n & 1), (uint32_t)(n >> 1) & 1u);
+    w.bh = w.item[2 * (n & 1)];
+    w.R0 = w.item[2 * (n & 1) + 1];
+    return ok && w.bh >= 0;
+}
+template <bool kPair>
+__device__ __forceinline__ void item_taken(const AttnBars &bar, int n) {
+    if constexpr (kPair) mbar_arrive_cluster(mapa(smem_u32(bar.item_empty + (n & 1)), 0));
+    else mbar_arrive(bar.item_empty + (n & 1));
+}
+// ... by a whole warp
+template <bool kPair>
+__device__ __forceinline__ bool next_item_of_warp(Work &w, const AttnBars &bar, int n, volatile int *abort_flag, int *status, bool &ok) {
+    (void)next_item<kPair>(w, bar, n, abort_flag, status, ok);
+    ok = __all_sync(0xffffffffu, ok);
+    w.bh = __shfl_sync(0xffffffffu, w.bh, 0);   // (known to be the same in all lanes, and so is what follows from it)
+    w.R0 = __shfl_sync(0xffffffffu, w.R0, 0);
+    if (ok && (threadIdx.x & 31) == 0) item_taken<kPair>(bar, n);
+    return ok && w.bh >= 0;
+}
+
+// The tensor maps of an attention kernel (p0, p1: the linear branch's partial results).
+struct AttnMaps {
+    CUtensorMap q, k, v, ksel, vsel, p0, p1, y;
+};
+
+// Rows t0 .. t0 + rows - 1 of a head, whose rows start at head0, from their place in an output's stage, by a warp.
+template <int D>
+__device__ __forceinline__ void store_rows(const uint8_t *tile, __nv_bfloat16 *Y, long long head0, int t0, int rows) {
+    constexpr int kPieces = D / 8;
+#pragma unroll 4
+    for (int id = threadIdx.x & 31; id < rows * kPieces; id += 32) {
+        const int row = id / kPieces, c = id % kPieces;
+        *reinterpret_cast<uint4 *>(Y + (head0 + t0 + row) * D + c * 8) =
+            *reinterpret_cast<const uint4 *>(tile + (c >> 3) * (kBlockM * 128) + row * 128 + (((c & 7) ^ (row & 7)) << 4));
+    }
+}
+
 // ---------------------------------------------------------------------------
 // Softmax warps of the attention kernels (one warpgroup per query tile, a thread per query row) and the merge epilogue.
-// x is the query tile (0: A, 1: B), tile_row0 the position of the tile's first row, stage_tile the tile's Q region in
-// shared memory (the epilogue's staging space).  The barriers are this CTA's, except that in a CTA pair what the issuing
-// warp waits for is announced on the first CTA's.
+// x is the query tile (0: A, 1: B), tile_row0 the position of the tile's first row, ring the key ring in shared memory.  The
+// barriers are this CTA's, except that in a CTA pair what the issuing warp waits for is announced on the first CTA's.  One item:
+// my is query tile x's view of the stream, y_stage the ring stage of its output, flip the parity of the tiles that query tile x
+// has had in the items before, y_flip that of these items; ahead(last)
+// is called while the last product runs and says whether the item is the CTA's last.  Returns whether all
+// waits ended.
 // ---------------------------------------------------------------------------
-template <int D, bool kPair>
-__device__ __forceinline__ void softmax_role(const Stream &st, const AttnBars &bar, const int x, const int tile_row0,
+template <int D, bool kPair, class Ahead>
+__device__ __forceinline__ bool softmax_role(const Stream::Mine my, const AttnBars &bar, const int x, const int tile_row0,
                                              const uint32_t tmem_base, volatile int *abort_flag, int *status,
-                                             uint8_t *stage_tile, const __nv_bfloat16 *y_part,
-                                             const float *d_part, const int n_parts, const long long part_stride_y,
-                                             const long long part_stride_d, __nv_bfloat16 *Y, const int bh,
-                                             const int N, const int C, const int lam, const int budget,
-                                             const float scale_log2) {
-    constexpr int kStages = AttnPlan<D, kPair>::kStages;
+                                             uint8_t *ring, const int y_stage, const int flip, const int y_flip,
+                                             const float *d_part, const int n_parts, const long long part_stride_d, __nv_bfloat16 *Y,
+                                             const int bh, const int N, const int log2_c, const int lam, const int budget,
+                                             const float scale_log2, Ahead ahead) {
+    using P = AttnPlan<D, kPair>;
     // The MUFU unit (one warp instruction per eight cycles) would need 1024 cycles for a query tile's exponentials, which is as
     // long as the tensor pipe needs for the tile's two products; so one of kPolyEvery column pairs takes 2^x from the FMA
     // pipes instead (see exp2_fma2), interleaved with the others so that both units work at the same time.  The same share
@@ -227,168 +312,166 @@ __device__ __forceinline__ void softmax_role(const Stream &st, const AttnBars &b
     };
     const int row_in_tile = ((warp & 3) << 5) | lane;
     const int t = tile_row0 + row_in_tile;         // this thread's query position
-    const int n_mine = st.entries_of(x);
-    if (n_mine > 0) {                              // (in a pair also where none of this CTA's rows are below N)
-        const uint32_t lane_addr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
-        const uint32_t s_addr = lane_addr + TmemPlan<D>::s(x), p_addr = lane_addr + TmemPlan<D>::p(x), o_addr = lane_addr + TmemPlan<D>::o(x);
-        const int tq = min(t, N - 1);              // rows past N mimic the last row (never stored)
-        const int c = tq / C;
-        const int lim_sel = c >= 2 ? (c - 1) * lam : 0, lo_sel = sel_start(lim_sel, budget);
-        const int loc_lo = c >= 1 ? (c - 1) * C : 0;
-        float m_used = -INFINITY, l_sum = 0.f;     // log2 domain
-        bool ok = true;
-        // A wait can end in one lane and run out in another, and the warp has to stay together for the instructions that take
-        // it whole.  So no wait is left by a branch: the loop runs out with whatever has been read (a wait gives up at once
-        // where a role has given up before), and the warp votes behind it.  (A vote behind every wait took 0.6 % longer at
-        // 64 heads x 32768 tokens, d = 128, one a tile 0.5 % at 128 x 4096, d = 64; skipping the waits after a failure 2 %.)
-        auto wait = [&](uint64_t *b, int parity, int where) {
-            ok = mbar_wait(b, (uint32_t)parity, abort_flag, status, where) && ok;
-        };
-        // one thread of a query tile releases the stage of its last product: its share of two, or both where the entry is
-        // the tile's alone
-        auto release = [&](int e) {
-            if (row_in_tile != 0 || !ok) return;
-            mbar_arrive(bar.kv_empty + e % kStages);
-            if (!st.shared(e)) mbar_arrive(bar.kv_empty + e % kStages);
-        };
-        for (int k = 0; k < n_mine; ++k) {
-            // visible column interval [lo, hi] of this row in the stream tile
-            bool sel;
-            const int p0 = st.tile_of(x, k, sel) * kBlockN;
-            const int lo = max((sel ? lo_sel : loc_lo) - p0, 0), hi = min((sel ? lim_sel - 1 : tq) - p0, kBlockN - 1);
-            const bool need_mask = __any_sync(0xffffffffu, lo > 0 || hi < kBlockN - 1);
-            const bool none = need_mask && !__any_sync(0xffffffffu, lo <= hi);   // (a warp whose rows see none of it skips the arithmetic)
-            wait(bar.s_full + x, k & 1, 8);
-            tc_fence_after();
-            if (none) {
-                __syncwarp();   // (no lane still looks for this phase)
-                if (lane == 0) arrive_first(bar.s_free + x);
-                uint32_t masked[32];   // the weights of masked columns: 0, and 2^-126 from the cubic
-#pragma unroll
-                for (int j = 0; j < 32; ++j) masked[j] = j % kPolyEvery == 0 ? 0x00800080u : 0u;
-                if (k > 0) {
-                    wait(bar.pv_done + x, (k - 1) & 1, 11);
-                    release(st.entry(x, k - 1));
-                    tc_fence_after();
-                }
-                __syncwarp();
-                tmem_st32(p_addr, masked);
-                tmem_st32(p_addr + 32, masked);
-                tmem_wait_st();
-                tc_fence_before();
-                __syncwarp();
-                if (lane == 0) arrive_first(bar.p_full + x);
-                continue;
-            }
-            uint32_t sr[128];
-            tmem_ld32(s_addr, sr);
-            tmem_ld32(s_addr + 32, sr + 32);
-            tmem_ld32(s_addr + 64, sr + 64);
-            tmem_ld32(s_addr + 96, sr + 96);
-            tmem_wait_ld();
-            tc_fence_before();
-            __syncwarp();
+    const int n_mine = my.n;
+    bool ok = true;
+    const uint32_t lane_addr = tmem_base + ((uint32_t)((warp & 3) * 32) << 16);
+    const uint32_t s_addr = lane_addr + TmemPlan<D>::s(x), p_addr = lane_addr + TmemPlan<D>::p(x), o_addr = lane_addr + TmemPlan<D>::o(x);
+    const int tq = min(t, N - 1);              // rows past N mimic the last row (never stored)
+    const int lim_sel = sel_limit(tq, log2_c, lam), lo_sel = sel_start(lim_sel, budget);
+    const int loc_lo = max((tq >> log2_c) - 1, 0) << log2_c;
+    float m_used = -INFINITY, l_sum = 0.f;     // log2 domain
+    // A wait can end in one lane and run out in another, and the warp has to stay together for the instructions that take
+    // it whole.  So no wait is left by a branch: the loop runs out with whatever has been read (a wait gives up at once
+    // where a role has given up before), and the warp votes behind it.  (A vote behind every wait took 0.6 % longer at
+    // 64 heads x 32768 tokens, d = 128, one a tile 0.5 % at 128 x 4096, d = 64; skipping the waits after a failure 2 %.)
+    auto wait = [&](uint64_t *b, int parity, int where) {
+        ok = mbar_wait(b, (uint32_t)(parity ^ flip), abort_flag, status, where) && ok;
+    };
+    int lo = lo_sel - my.sel0 * kBlockN, hi = lim_sel - 1 - my.sel0 * kBlockN;
+    for (int k = 0; k < n_mine; ++k) {
+        // visible column interval [lo, hi] of this row in the stream tile
+        if (k == my.n_sel) {
+            lo = loc_lo - my.loc0 * kBlockN;
+            hi = tq - my.loc0 * kBlockN;
+        }
+        const bool need_mask = __any_sync(0xffffffffu, lo > 0 || hi < kBlockN - 1);
+        const bool none = need_mask && !__any_sync(0xffffffffu, max(lo, 0) <= min(hi, kBlockN - 1));   // (a warp whose rows see none of it skips the arithmetic)
+        wait(bar.s_full + x, k & 1, 8);
+        tc_fence_after();
+        if (none) {
+            __syncwarp();   // (no lane still looks for this phase)
             if (lane == 0) arrive_first(bar.s_free + x);
-            float *s = reinterpret_cast<float *>(sr);
-            if (need_mask) {
+            uint32_t masked[32];   // the weights of masked columns: 0, and 2^-126 from the cubic
 #pragma unroll
-                for (int q = 0; q < 4; ++q) {
-                    // columns of this block of 32 that the row sees, as a bit set
-                    const int l = min(max(lo - 32 * q, 0), 32), n = min(max(hi - 32 * q + 1, 0), 32);
-                    const uint32_t seen = n > l ? (0xffffffffu >> (32 - n)) & (0xffffffffu << l) : 0u;
-#pragma unroll
-                    for (int j = 0; j < 32; ++j)
-                        if (!((seen >> j) & 1u)) s[q * 32 + j] = -INFINITY;
-                }
-            }
-            float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
-#pragma unroll
-            for (int j = 0; j < 128; j += 8) {
-                mx0 = max3_nan(mx0, s[j], s[j + 1]);
-                mx1 = max3_nan(mx1, s[j + 2], s[j + 3]);
-                mx2 = max3_nan(mx2, s[j + 4], s[j + 5]);
-                mx3 = max3_nan(mx3, s[j + 6], s[j + 7]);
-            }
-            const float mt = max_nan(max_nan(mx0, mx1), max_nan(mx2, mx3)) * scale_log2;
-            // lazy rescale: keep the old reference unless the new maximum exceeds it by 2^8.  A NaN or +inf logit makes the
-            // reference NaN, and with it every weight that is not a cubic's: those would lose it in the clamp.
-            const bool grow = !(mt <= m_used + 8.f);
-            float alpha = 1.f;
-            if (grow) {
-                const float m_new = mt < INFINITY ? mt : NAN;
-                alpha = (m_used == -INFINITY) ? 0.f : ex2(m_used - m_new);
-                m_used = m_new;
-            }
-            // the previous product is in O, has read P and is done with its stage (asked for as late as P is written: the
-            // issuing warp takes it up behind a product of the other query tile)
-            auto previous_done = [&]() { wait(bar.pv_done + x, (k - 1) & 1, 11); };
-            if (k > 0 && __any_sync(0xffffffffu, grow)) {
-                previous_done();
-                tc_fence_after();
-                {
-#pragma unroll
-                    for (int q = 0; q < D / 32; ++q) {
-                        uint32_t orow[32];
-                        tmem_ld32(o_addr + q * 32, orow);
-                        tmem_wait_ld();
-#pragma unroll
-                        for (int j = 0; j < 32; ++j) orow[j] = __float_as_uint(__uint_as_float(orow[j]) * alpha);
-                        tmem_st32(o_addr + q * 32, orow);
-                    }
-                }
-            }
-            l_sum *= alpha;
-            const float neg_m = (m_used == -INFINITY) ? 0.f : -m_used;
-            const float2 scale2 = make_float2(scale_log2, scale_log2), negm2 = make_float2(neg_m, neg_m);
-            float2 acc = make_float2(0.f, 0.f);
-            // P = 2^(s * scale - m) as bf16
-            uint32_t pk[2][32];
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-#pragma unroll
-                for (int j = 0; j < 32; ++j) {
-                    const float2 sv = make_float2(s[q * 64 + 2 * j], s[q * 64 + 2 * j + 1]);
-                    const float2 xv = __ffma2_rn(sv, scale2, negm2);
-                    const float2 pr = j % kPolyEvery == 0 ? exp2_fma2(xv) : make_float2(ex2(xv.x), ex2(xv.y));
-                    acc = __fadd2_rn(acc, pr);
-                    pk[q][j] = pack_bf16(pr.x, pr.y);
-                }
-            }
+            for (int j = 0; j < 32; ++j) masked[j] = j % kPolyEvery == 0 ? 0x00800080u : 0u;
             if (k > 0) {
-                previous_done();
+                wait(bar.pv_done + x, (k - 1) & 1, 11);
                 tc_fence_after();
-                release(st.entry(x, k - 1));
-                __syncwarp();
             }
-            tmem_st32(p_addr, pk[0]);
-            tmem_st32(p_addr + 32, pk[1]);
-            l_sum += acc.x + acc.y;
+            __syncwarp();
+            tmem_st32(p_addr, masked);
+            tmem_st32(p_addr + 32, masked);
             tmem_wait_st();
             tc_fence_before();
             __syncwarp();
             if (lane == 0) arrive_first(bar.p_full + x);
+            lo -= kBlockN;
+            hi -= kBlockN;
+            continue;
         }
-        // ---- epilogue: y = (O e^{m-ms} + e^{-ms} N_LA) / (l e^{m-ms} + e^{-ms} D_LA), ms = max(m, 0)
-        // The linear branch arrives as up to two partial results (one per feature half): y_p = N_p / D_p as bf16
-        // and D_p, so N_LA = sum y_p D_p and D_LA = sum D_p.  A thread owns a row, but loads / stores in which
-        // every lane touches a different row cost a memory instruction per 16 bytes and row; so the y_p come in
-        // and Y goes out through shared memory with 16 consecutive lanes per row.  The staging space is this
-        // warp's 32 rows of the tile's Q region (one row = D bf16 = 2 D bytes: D / 2 columns of both parts), free
-        // once the tile's last Q K^T has completed; 16-byte pieces are swizzled by the row so that row-wise and
-        // piece-wise accesses avoid bank conflicts.
+        uint32_t sr[128];
+        tmem_ld32(s_addr, sr);
+        tmem_ld32(s_addr + 32, sr + 32);
+        tmem_ld32(s_addr + 64, sr + 64);
+        tmem_ld32(s_addr + 96, sr + 96);
+        tmem_wait_ld();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) arrive_first(bar.s_free + x);
+        float *s = reinterpret_cast<float *>(sr);
+        if (need_mask) {
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                // columns of this block of 32 that the row sees, as a bit set
+                const int l = min(max(lo - 32 * q, 0), 32), n = min(max(hi - 32 * q + 1, 0), 32);
+                const uint32_t seen = n > l ? (0xffffffffu >> (32 - n)) & (0xffffffffu << l) : 0u;
+#pragma unroll
+                for (int j = 0; j < 32; ++j)
+                    if (!((seen >> j) & 1u)) s[q * 32 + j] = -INFINITY;
+            }
+        }
+        float mx0 = -INFINITY, mx1 = -INFINITY, mx2 = -INFINITY, mx3 = -INFINITY;
+#pragma unroll
+        for (int j = 0; j < 128; j += 8) {
+            mx0 = max3_nan(mx0, s[j], s[j + 1]);
+            mx1 = max3_nan(mx1, s[j + 2], s[j + 3]);
+            mx2 = max3_nan(mx2, s[j + 4], s[j + 5]);
+            mx3 = max3_nan(mx3, s[j + 6], s[j + 7]);
+        }
+        const float mt = max_nan(max_nan(mx0, mx1), max_nan(mx2, mx3)) * scale_log2;
+        // lazy rescale: keep the old reference unless the new maximum exceeds it by 2^8.  A NaN or +inf logit makes the
+        // reference NaN, and with it every weight that is not a cubic's: those would lose it in the clamp.
+        const bool grow = !(mt <= m_used + 8.f);
+        float alpha = 1.f;
+        if (grow) {
+            const float m_new = mt < INFINITY ? mt : NAN;
+            alpha = (m_used == -INFINITY) ? 0.f : ex2(m_used - m_new);
+            m_used = m_new;
+        }
+        // the previous product is in O, has read P and is done with its stage (asked for as late as P is written: the
+        // issuing warp takes it up behind a product of the other query tile)
+        auto previous_done = [&]() { wait(bar.pv_done + x, (k - 1) & 1, 11); };
+        if (k > 0 && __any_sync(0xffffffffu, grow)) {
+            previous_done();
+            tc_fence_after();
+            {
+#pragma unroll
+                for (int q = 0; q < D / 32; ++q) {
+                    uint32_t orow[32];
+                    tmem_ld32(o_addr + q * 32, orow);
+                    tmem_wait_ld();
+#pragma unroll
+                    for (int j = 0; j < 32; ++j) orow[j] = __float_as_uint(__uint_as_float(orow[j]) * alpha);
+                    tmem_st32(o_addr + q * 32, orow);
+                }
+            }
+        }
+        l_sum *= alpha;
+        const float neg_m = (m_used == -INFINITY) ? 0.f : -m_used;
+        const float2 scale2 = make_float2(scale_log2, scale_log2), negm2 = make_float2(neg_m, neg_m);
+        float2 acc = make_float2(0.f, 0.f);
+        // P = 2^(s * scale - m) as bf16
+        uint32_t pk[2][32];
+#pragma unroll
+        for (int q = 0; q < 2; ++q) {
+#pragma unroll
+            for (int j = 0; j < 32; ++j) {
+                const float2 sv = make_float2(s[q * 64 + 2 * j], s[q * 64 + 2 * j + 1]);
+                const float2 xv = __ffma2_rn(sv, scale2, negm2);
+                const float2 pr = j % kPolyEvery == 0 ? exp2_fma2(xv) : make_float2(ex2(xv.x), ex2(xv.y));
+                acc = __fadd2_rn(acc, pr);
+                pk[q][j] = pack_bf16(pr.x, pr.y);
+            }
+        }
+        if (k > 0) {
+            previous_done();
+            tc_fence_after();
+            __syncwarp();
+        }
+        tmem_st32(p_addr, pk[0]);
+        tmem_st32(p_addr + 32, pk[1]);
+        l_sum += acc.x + acc.y;
+        tmem_wait_st();
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) arrive_first(bar.p_full + x);
+        lo -= kBlockN;
+        hi -= kBlockN;
+    }
+    // ---- epilogue: y = (O e^{m-ms} + e^{-ms} N_LA) / (l e^{m-ms} + e^{-ms} D_LA), ms = max(m, 0)
+    // The linear branch arrives as up to two partial results (one per feature half): y_p = N_p / D_p as bf16
+    // and D_p, so N_LA = sum y_p D_p and D_LA = sum D_p.  A thread owns a row, but loads / stores in which
+    // every lane touches a different row cost a memory instruction per 16 bytes and row; so the y_p come in by TMA, into
+    // stages of the ring behind the item's keys (they are there by the time the last product is), and Y goes out the same
+    // way (output_role), from where the first part lay.
+    float da = 0.f, db = 0.f;
+    if (n_parts > 0 && t < N) {
+        da = d_part[(long long)bh * N + t];
+        if (n_parts > 1) db = d_part[part_stride_d + (long long)bh * N + t];
+    }
+    bool last;
+    const bool there = ahead(last);
+    if (n_mine > 0) {                              // (in a pair also where none of this CTA's rows are below N)
         wait(bar.pv_done + x, (n_mine - 1) & 1, 9);   // (every query tile has a LOC tile)
         if (__all_sync(0xffffffffu, ok)) {
             tc_fence_after();
-            release(st.entry(x, n_mine - 1));   // (the other query tile may have entries left)
-            constexpr int kRowBytes = D * 2, kPieces = kRowBytes / 16;   // pieces of 16 bytes per staged row
-            constexpr int kPartPieces = kPieces / 2;                     // pieces of one part (D / 2 columns)
-            uint8_t *stg = stage_tile + (warp & 3) * 32 * kRowBytes;
-            const int t0 = tile_row0 + (warp & 3) * 32;                    // first row of this warp
-            float fs = 1.f, fa = 0.f, fb = 0.f, dla = 0.f;
-            if (n_parts > 0 && t < N) {
-                const float da = d_part[(long long)bh * N + t];
-                const float db = n_parts > 1 ? d_part[part_stride_d + (long long)bh * N + t] : 0.f;
-                dla = da + db;
+            wait(bar.y_full + x, y_flip ^ flip, 12);
+            if (__all_sync(0xffffffffu, ok)) {
+                // this warp's 32 rows of a part: 64 columns of 128 bytes a row, 16-byte pieces swizzled by the row
+                uint8_t *part0 = ring + y_stage * P::kStage + (warp & 3) * 32 * 128;
+                uint8_t *part1 = P::kPartsPerStage > 1 ? part0 + P::kPartTile : ring + (y_stage + 1) % P::kStages * P::kStage + (warp & 3) * 32 * 128;
+                float fs = 1.f, fa = 0.f, fb = 0.f;
+                const float dla = da + db;
                 if (dla > 0.f) {
                     const float m_nat = m_used * 0.6931471805599453f;
                     const float ms = fmaxf(m_nat, 0.f);
@@ -397,82 +480,64 @@ __device__ __forceinline__ void softmax_role(const Stream &st, const AttnBars &b
                     fa = fl * da;
                     fb = fl * db;
                 }
-            }
-            const float inv = 1.f / (l_sum * fs + fa + fb);
-            const bool with_la = (n_parts > 0) && __any_sync(0xffffffffu, dla > 0.f);
-            uint32_t out[D / 2];   // the row as packed bf16
-#pragma unroll
-            for (int hh = 0; hh < 2; ++hh) {   // halves of D / 2 columns
-                if (with_la) {
-                    __syncwarp();
-                    uint4 v[kPieces];   // (all requested before the first is stored: one round trip to memory, not kPieces)
-#pragma unroll
-                    for (int it = 0; it < kPieces; ++it) {
-                        const int id = it * 32 + lane, row = id / kPieces, c = id % kPieces;
-                        const int part = c / kPartPieces, cc = c % kPartPieces;
-                        v[it] = make_uint4(0, 0, 0, 0);
-                        if (t0 + row < N && part < n_parts)
-                            v[it] = *reinterpret_cast<const uint4 *>(y_part + part * part_stride_y + ((long long)bh * N + t0 + row) * D +
-                                                                     hh * (D / 2) + cc * 8);
-                    }
-#pragma unroll
-                    for (int it = 0; it < kPieces; ++it) {
-                        const int id = it * 32 + lane, row = id / kPieces, c = id % kPieces;
-                        *reinterpret_cast<uint4 *>(stg + row * kRowBytes + ((c ^ (row & (kPieces - 1))) << 4)) = v[it];
-                    }
-                    __syncwarp();
-                }
-#pragma unroll
-                for (int q = 0; q < D / 64; ++q) {
+                const float inv = 1.f / (l_sum * fs + fa + fb);
+                const bool with_la = (n_parts > 0) && __any_sync(0xffffffffu, dla > 0.f);
+                const float2 fs2 = make_float2(fs, fs), fa2 = make_float2(fa, fa), fb2 = make_float2(fb, fb), inv2 = make_float2(inv, inv);
+#pragma unroll 1
+                for (int q = 0; q < D / 32; ++q) {
                     uint32_t orow[32];
-                    tmem_ld32(o_addr + hh * (D / 2) + q * 32, orow);
+                    tmem_ld32(o_addr + q * 32, orow);
+                    auto offset = [&](int j8) { return (q >> 1) * (kBlockM * 128) + lane * 128 + ((((q & 1) * 4 + j8) ^ (lane & 7)) << 4); };
+                    uint4 pa[4], pb[4];   // (read before the first is written over)
+#pragma unroll
+                    for (int j8 = 0; j8 < 4; ++j8) {
+                        pa[j8] = pb[j8] = make_uint4(0, 0, 0, 0);
+                        if (with_la) {
+                            pa[j8] = *reinterpret_cast<const uint4 *>(part0 + offset(j8));
+                            if (n_parts > 1) pb[j8] = *reinterpret_cast<const uint4 *>(part1 + offset(j8));
+                        }
+                    }
                     tmem_wait_ld();
 #pragma unroll
                     for (int j8 = 0; j8 < 4; ++j8) {
-                        uint4 pa = make_uint4(0, 0, 0, 0), pb = pa;
-                        if (with_la) {
-                            const int ca = q * 4 + j8, cb = kPartPieces + ca;
-                            pa = *reinterpret_cast<const uint4 *>(stg + lane * kRowBytes + ((ca ^ (lane & (kPieces - 1))) << 4));
-                            pb = *reinterpret_cast<const uint4 *>(stg + lane * kRowBytes + ((cb ^ (lane & (kPieces - 1))) << 4));
-                        }
-                        const uint32_t wa[4] = {pa.x, pa.y, pa.z, pa.w}, wb[4] = {pb.x, pb.y, pb.z, pb.w};
+                        const uint32_t wa[4] = {pa[j8].x, pa[j8].y, pa[j8].z, pa[j8].w}, wb[4] = {pb[j8].x, pb[j8].y, pb[j8].z, pb[j8].w};
+                        uint32_t out[4];
 #pragma unroll
                         for (int e = 0; e < 4; ++e) {   // two columns per 32-bit word
-                            const float la0 = fmaf(fa, __uint_as_float(wa[e] << 16), fb * __uint_as_float(wb[e] << 16));
-                            const float la1 = fmaf(fa, __uint_as_float(wa[e] & 0xffff0000u), fb * __uint_as_float(wb[e] & 0xffff0000u));
-                            const float a0 = fmaf(__uint_as_float(orow[8 * j8 + 2 * e]), fs, la0);
-                            const float a1 = fmaf(__uint_as_float(orow[8 * j8 + 2 * e + 1]), fs, la1);
-                            out[hh * (D / 4) + q * 16 + 4 * j8 + e] = pack_bf16(a0 * inv, a1 * inv);
+                            const float2 a = make_float2(__uint_as_float(wa[e] << 16), __uint_as_float(wa[e] & 0xffff0000u));
+                            const float2 b = make_float2(__uint_as_float(wb[e] << 16), __uint_as_float(wb[e] & 0xffff0000u));
+                            const float2 la = __ffma2_rn(fa2, a, __fmul2_rn(fb2, b));
+                            const float2 o2 = make_float2(__uint_as_float(orow[8 * j8 + 2 * e]), __uint_as_float(orow[8 * j8 + 2 * e + 1]));
+                            const float2 y2 = __fmul2_rn(__ffma2_rn(o2, fs2, la), inv2);
+                            out[e] = pack_bf16(y2.x, y2.y);
                         }
+                        *reinterpret_cast<uint4 *>(part0 + offset(j8)) = make_uint4(out[0], out[1], out[2], out[3]);
                     }
                 }
-            }
-            // Y: own row into the staging space, then the warp writes its 32 rows piece-wise
-            __syncwarp();
-#pragma unroll
-            for (int c = 0; c < kPieces; ++c)
-                *reinterpret_cast<uint4 *>(stg + lane * kRowBytes + ((c ^ (lane & (kPieces - 1))) << 4)) =
-                    make_uint4(out[4 * c], out[4 * c + 1], out[4 * c + 2], out[4 * c + 3]);
-            __syncwarp();
-#pragma unroll
-            for (int it = 0; it < kPieces; ++it) {
-                const int id = it * 32 + lane, row = id / kPieces, c = id % kPieces;
-                if (t0 + row < N)
-                    *reinterpret_cast<uint4 *>(Y + ((long long)bh * N + t0 + row) * D + c * 8) =
-                        *reinterpret_cast<const uint4 *>(stg + row * kRowBytes + ((c ^ (row & (kPieces - 1))) << 4));
+                tc_fence_before();
+                if (last) {   // (nothing is left to hand the stores to an output warp for)
+                    __syncwarp();
+                    store_rows<D>(part0, Y, (long long)bh * N, tile_row0 + (warp & 3) * 32, min(N - tile_row0 - (warp & 3) * 32, 32));
+                } else {
+                    fence_proxy_async();
+                    __syncwarp();
+                    if (lane == 0) mbar_arrive(bar.y_ready + x);
+                }
             }
         }
     }
+    ok = ok && there;
+    return __all_sync(0xffffffffu, ok);
 }
 
-// TMA producer (one thread): the Q tiles, then the K and V tiles of the stream, as far ahead as the ring has free stages.  In a
-// pair every CTA loads its halves; their byte counts complete on the first CTA's barriers.
+// TMA producer (one thread): the Q tiles of an item, then the K and V tiles of its stream, as far ahead as the ring has free
+// stages, then what the epilogue merges.  In a pair every CTA loads its halves; the byte counts of Q, K and V complete on the
+// first CTA's barriers.
 template <int D, bool kPair, class TellPeer>
-__device__ __forceinline__ void producer_role(const Stream &st, const AttnBars &bar, uint8_t *smem, const uint32_t rank,
+__device__ __forceinline__ void producer_role(Work w, const AttnBars &bar, uint8_t *smem, const uint32_t rank,
                                               const CUtensorMap &tm_q, const CUtensorMap &tm_k, const CUtensorMap &tm_v,
-                                              const CUtensorMap &tm_ksel, const CUtensorMap &tm_vsel, const int q_row,
-                                              const int kv_row0, const int sel_row0, volatile int *abort_flag, int *status,
-                                              TellPeer tell_peer) {
+                                              const CUtensorMap &tm_ksel, const CUtensorMap &tm_vsel, const CUtensorMap &tm_p0,
+                                              const CUtensorMap &tm_p1, volatile int *abort_flag, int *status, TellPeer tell_peer) {
     using P = AttnPlan<D, kPair>;
     constexpr int kCtas = kPair ? 2 : 1, kStages = P::kStages;
     const uint32_t q_full0 = mapa(smem_u32(bar.q_full), 0), kv_full0 = mapa(smem_u32(bar.kv_full), 0);
@@ -480,28 +545,102 @@ __device__ __forceinline__ void producer_role(const Stream &st, const AttnBars &
         if constexpr (kPair) tma_load_2d_pair(dst, &map, b0, col, row);
         else tma_load_2d(dst, &map, b, col, row);
     };
-    const int n_q = st.n_b > 0 ? 2 : 1, n = st.entries();   // (every query tile has a LOC tile)
-    if (rank == 0) mbar_expect_tx(bar.q_full, kCtas * n_q * P::kQTile);
-    for (int x = 0; x < n_q; ++x)
-        for (int half = 0; half < D / 64; ++half)
-            load(smem + P::kQ + x * P::kQTile + half * (kBlockM * 128), tm_q, bar.q_full, q_full0, half * 64,
-                 q_row + ((int)rank + x * kCtas) * kBlockM);
+    const int n_y = P::y_entries(w.n_parts);
     bool ok = true;
-    int armed = 0;
+    int armed = 0, n = 0, q_armed = 0, a_armed = 0, b_armed = 0;
     RingPos pos{0, 0};
-    for (; armed < n; ++armed) {
-        ok = mbar_wait(bar.kv_empty + pos.stage, pos.parity ^ 1, abort_flag, status, 1);
+    w.set(w.first);
+    prefetch_map(&tm_k);
+    prefetch_map(&tm_v);
+    if (w.n_parts > 0) prefetch_map(&tm_p0);
+    if (w.n_parts > 1) prefetch_map(&tm_p1);
+    for (bool more = true; more && ok; ++n) {
+        const Stream st = w.stream();
+        const int kv_row0 = (w.bh / w.H * w.Hkv + w.bh % w.H / (w.H / w.Hkv)) * w.N, q_row = w.bh * w.N + w.R0;
+        // (with topk = chunk every token is selected and the compacted arrays would be copies of K / V: the salient prefix is
+        // then read from K / V themselves, and tm_ksel / tm_vsel alias tm_k / tm_v)
+        const int sel_row0 = w.sel_identity ? kv_row0 : w.bh * w.sel_rows;
+        const int n_q = w.n_query_tiles(), entries = st.entries();   // (every query tile has a LOC tile)
+        ok = mbar_wait(bar.q_empty, (n & 1) ^ 1, abort_flag, status, 2);
         if (!ok) break;
-        bool sel;
-        const int tile = st.tile(armed, sel), row = (sel ? sel_row0 : kv_row0) + tile * kBlockN;
-        if (rank == 0) mbar_expect_tx(bar.kv_full + pos.stage, kCtas * (P::kKTile + P::kVTile));
-        for (int half = 0; half < D / 64; ++half)   // (of a pair: this CTA's 64 keys)
-            load(smem + P::kK + pos.stage * P::kKTile + half * (P::kKRows * 128), sel ? tm_ksel : tm_k, bar.kv_full + pos.stage,
-                 kv_full0 + pos.stage * 8, half * 64, row + (int)rank * P::kKRows);
-        for (int q = 0; q < P::kVCols / 64; ++q)    // this CTA's value columns, 64 at a time
-            load(smem + P::kV + pos.stage * P::kVTile + q * (kBlockN * 128), sel ? tm_vsel : tm_v, bar.kv_full + pos.stage,
-                 kv_full0 + pos.stage * 8, (int)rank * P::kVCols + q * 64, row);
-        pos.next(kStages);
+        if (rank == 0) mbar_expect_tx(bar.q_full, kCtas * n_q * P::kQTile);
+        ++q_armed;
+        for (int x = 0; x < n_q; ++x)
+            for (int half = 0; half < D / 64; ++half)
+                load(smem + P::kQ + x * P::kQTile + half * (kBlockM * 128), tm_q, bar.q_full, q_full0, half * 64,
+                     q_row + ((int)rank + x * kCtas) * kBlockM);
+        // the item after this one, unless a CTA has failed (asked for here, needed behind the loop)
+        int next = 0, failed = 0;
+        if (rank == 0) {
+            next = atomicAdd(status + kNextItem, 1);
+            failed = *reinterpret_cast<volatile int *>(status);
+        }
+        for (int e = 0; e < entries; ++e, ++armed) {
+            ok = mbar_wait(bar.kv_empty + pos.stage, pos.parity ^ 1, abort_flag, status, 1);
+            if (!ok) break;
+            bool sel;
+            const int tile = st.tile(e, sel), row = (sel ? sel_row0 : kv_row0) + tile * kBlockN;
+            if (rank == 0) mbar_expect_tx(bar.kv_full + pos.stage, kCtas * P::kStage);
+            for (int half = 0; half < D / 64; ++half)   // (of a pair: this CTA's 64 keys)
+                load(smem + P::kK + pos.stage * P::kStage + half * (P::kKRows * 128), sel ? tm_ksel : tm_k, bar.kv_full + pos.stage,
+                     kv_full0 + pos.stage * 8, half * 64, row + (int)rank * P::kKRows);
+            for (int q = 0; q < P::kVCols / 64; ++q)    // this CTA's value columns, 64 at a time
+                load(smem + P::kV + pos.stage * P::kStage + q * (kBlockN * 128), sel ? tm_vsel : tm_v, bar.kv_full + pos.stage,
+                     kv_full0 + pos.stage * 8, (int)rank * P::kVCols + q * 64, row);
+            pos.next(kStages);
+        }
+        if (!ok) break;
+        if (rank == 0) {   // (ahead of the outputs, which come only with the last products)
+            ok = mbar_wait(bar.item_empty + (n & 1), (uint32_t)((n >> 1) & 1) ^ 1u, abort_flag, status, 14);
+            if (!ok) break;
+            next += (int)(gridDim.x / kCtas);
+            more = failed == 0 && next < w.total;
+            if (more) w.set(next);
+            else w.bh = -1;
+            volatile int *slot = w.item + 2 * (n & 1);
+            slot[0] = w.bh;
+            slot[1] = w.R0;
+            mbar_arrive(bar.item_full + (n & 1));
+            if constexpr (kPair) {
+                const uint32_t peer_slot = mapa(smem_u32(const_cast<int *>(slot)), 1);
+                st_cluster_u32(peer_slot, (uint32_t)w.bh);
+                st_cluster_u32(peer_slot + 4, (uint32_t)w.R0);
+                mbar_arrive_release_cluster(mapa(smem_u32(bar.item_full + (n & 1)), 1));
+            }
+        }
+        // Entries of the outputs: the parts' rows of this CTA's query tiles (rows behind the last of a head are never used).
+        // They pass the ring's full-barrier at once: nobody waits for it, but its phases count the rounds.
+        for (int x = 0; x < n_q && ok; ++x) {
+            for (int y = 0; y < n_y; ++y, ++armed) {
+                ok = mbar_wait(bar.kv_empty + pos.stage, pos.parity ^ 1, abort_flag, status, 10);
+                if (!ok) {
+                    if (y > 0) mbar_arrive(bar.y_full + x);   // (for the wait below)
+                    break;
+                }
+                if (rank == 0) mbar_arrive(bar.kv_full + pos.stage);
+                const int parts = min(w.n_parts - y * P::kPartsPerStage, P::kPartsPerStage);   // of this entry
+                if (parts > 0) mbar_expect_tx(bar.y_full + x, parts * P::kPartTile);
+                else mbar_arrive(bar.y_full + x);
+                if (y == 0) ++(x ? b_armed : a_armed);
+                for (int part = y * P::kPartsPerStage; part < y * P::kPartsPerStage + parts; ++part)
+                    for (int half = 0; half < D / 64; ++half)
+                        tma_load_2d(smem + P::kK + pos.stage * P::kStage + (part - y * P::kPartsPerStage) * P::kPartTile + half * (kBlockM * 128),
+                                    part ? &tm_p1 : &tm_p0, bar.y_full + x, half * 64, q_row + ((int)rank + x * kCtas) * kBlockM);
+                pos.next(kStages);
+            }
+        }
+        if (!ok) break;
+        if constexpr (kPair) {
+            // The second CTA's loads count on the first's full-barriers, whose phases the first's own output entries move on as
+            // well: it begins with an item when the first has passed those of the item before.
+            if (rank == 0) {
+                mbar_arrive_cluster(mapa(smem_u32(bar.first_done), 1));
+            } else {
+                more = next_item<kPair>(w, bar, n, abort_flag, status, ok);
+                item_taken<kPair>(bar, n);
+                ok = ok && mbar_wait(bar.first_done, (uint32_t)n & 1u, abort_flag, status, 16);
+            }
+        }
     }
     // leave no copy in flight behind.  In a pair the first CTA's barriers count both CTAs' bytes; the second, where it has
     // given up and the first may not know of its last copies, waits out a fixed stretch that is long against a tile load.
@@ -509,11 +648,59 @@ __device__ __forceinline__ void producer_role(const Stream &st, const AttnBars &
     if constexpr (kPair) {
         if (!ok) tell_peer();
     }
+    if (a_armed > 0) mbar_wait_drain(bar.y_full, (uint32_t)(a_armed - 1) & 1u, t0);
+    if (b_armed > 0) mbar_wait_drain(bar.y_full + 1, (uint32_t)(b_armed - 1) & 1u, t0);
     if (rank == 0) {
-        mbar_wait_drain(bar.q_full, 0, t0);
+        if (q_armed > 0) mbar_wait_drain(bar.q_full, (uint32_t)(q_armed - 1) & 1u, t0);
         mbar_drain_ring(bar.kv_full, kStages, armed, t0);
     } else if (!ok) {
         while (clock64() - t0 < 200000) {}
+    }
+}
+
+// Stores of query tile x (a warp): the tile's rows as the softmax warps have left them in the output's first stage.  While an
+// item runs, what its epilogue reads of D_p comes into L2.
+template <int D, bool kPair>
+__device__ __forceinline__ void output_role(Work w, const AttnBars &bar, const uint8_t *ring, const int x, const uint32_t rank,
+                                            const CUtensorMap &tm_y, const float *d_part, __nv_bfloat16 *Y, volatile int *abort_flag,
+                                            int *status) {
+    using P = AttnPlan<D, kPair>;
+    constexpr int kCtas = kPair ? 2 : 1, kStages = P::kStages;
+    const int lane = threadIdx.x & 31, n_y = P::y_entries(w.n_parts);
+    int ring0 = 0, y_odd = 0;
+    bool ok = true;
+    if (lane == 0) prefetch_map(&tm_y);
+    bool more = true;
+    w.set(w.first);
+    for (int n = 0; more; ++n) {
+        const Stream st = w.stream();
+        const int y_entry = ring0 + st.entries() + x * n_y, t0 = w.R0 + (x * kCtas + (int)rank) * kBlockM, rows = min(w.N - t0, kBlockM);
+        const int bh = w.bh;
+        const bool live = x < w.n_query_tiles();   // (below, w is at the next item)
+        ring0 = (ring0 + st.entries() + n_y * w.n_query_tiles()) % kStages;
+        if (rows > 0 && lane < 8 && (lane >> 2) < w.n_parts)   // 128 bytes a lane
+            prefetch_l2(d_part + ((long long)(lane >> 2) * w.n_heads + bh) * w.N + t0 + min((lane & 3) * 32, rows - 1));
+        more = next_item_of_warp<kPair>(w, bar, n, abort_flag, status, ok);
+        if (!ok || !more) break;   // (the last item's rows are stored by the softmax warps)
+        if (!live) continue;
+        ok = mbar_wait(bar.y_ready + x, y_odd, abort_flag, status, 15);
+        if (!__all_sync(0xffffffffu, ok)) break;
+        y_odd ^= 1;
+        const uint8_t *tile = ring + y_entry % kStages * P::kStage;
+        if (rows == kBlockM) {
+            if (lane == 0) {
+#pragma unroll
+                for (int a = 0; a < D / 64; ++a) tma_store_2d(&tm_y, tile + a * (kBlockM * 128), a * 64, bh * w.N + t0);
+                bulk_store_commit();
+                bulk_store_wait_read();
+            }
+        } else {   // the last rows of a sequence (the map does not know where a head ends)
+            store_rows<D>(tile, Y, (long long)bh * w.N, t0, rows);
+            fence_proxy_async();   // (the stage is next written by TMA)
+        }
+        __syncwarp();
+        if (lane == 0)
+            for (int y = 0; y < n_y; ++y) mbar_arrive(bar.kv_empty + (y_entry + y) % kStages);
     }
 }
 
@@ -534,7 +721,7 @@ __device__ __forceinline__ void producer_role(const Stream &st, const AttnBars &
 // 4096, d = 64, every token 551 and 502, a quarter 585 and 515; the scan and the score kernel have a part in the quarters and in
 // the capped call).  Two threads per row instead of one (16 softmax warps) were slower by 10 %: the stream's bookkeeping doubles.
 template <int D, bool kPair, class TellPeer>
-__device__ __forceinline__ void mma_role(const Stream &st, const AttnBars &bar, uint8_t *smem, const uint32_t tmem_base,
+__device__ __forceinline__ void mma_role(Work w, const AttnBars &bar, uint8_t *smem, const uint32_t tmem_base,
                                          volatile int *abort_flag, int *status, TellPeer tell_peer) {
     using P = AttnPlan<D, kPair>;
     using TM = TmemPlan<D>;
@@ -542,8 +729,7 @@ __device__ __forceinline__ void mma_role(const Stream &st, const AttnBars &bar, 
     constexpr uint32_t idesc_qk = make_idesc(kM, kBlockN, false);
     constexpr uint32_t idesc_pv = make_idesc(kM, D, true);
     const bool leader = elect_one();
-    bool ok = mbar_wait(bar.q_full, 0, abort_flag, status, 4);
-    tc_fence_after();
+    bool ok = true;
     // descriptors as low words: a k-step adds a constant
     const uint32_t q_lo0 = desc_lo(smem_u32(smem + P::kQ), 0);
     const uint32_t k_lo0 = desc_lo(smem_u32(smem + P::kK), 0);
@@ -556,83 +742,101 @@ __device__ __forceinline__ void mma_role(const Stream &st, const AttnBars &bar, 
         else tc_commit(b);
     };
     // A place in the order of the products: query tile x, its k-th tile, and the ring stage of that.
-    const int n_own0 = st.n_lead + 2 * st.n_shared, n_items = n_own0 + st.n_a + st.n_b;
-    const int turns = min(st.n_a, st.n_b), x_last = st.n_a > st.n_b ? 0 : 1;
     struct Item {
         int m, x, k;
         RingPos pos;
     };
-    auto advance = [&](Item &it) {
-        ++it.m;
-        if (it.m <= st.n_lead && it.m < n_own0) {
-            ++it.k;
-        } else if (it.m < n_own0) {
-            it.x ^= 1;
-            if (it.x == 1) {   // (both query tiles use the entry)
-                it.k -= st.n_lead;
-                return;
-            }
-            it.k += st.n_lead + 1;
-        } else {
-            const int s = it.m - n_own0;
-            it.x = s < 2 * turns ? s & 1 : x_last;
-            it.k = st.first_own(it.x) + (s < 2 * turns ? s >> 1 : s - turns);
-        }
-        it.pos.next(kStages);
-    };
     Item qk{0, 0, 0, {0, 0}}, pv{0, 0, 0, {0, 0}};
-    int x_prev = 0, k_prev = 0;   // of the item whose S was formed last
-    auto issue_qk = [&]() {
-        // K and V of the entry have arrived (B follows A on the entries that they share)
-        if (qk.m >= n_own0 || qk.x == 0) wait(bar.kv_full + qk.pos.stage, qk.pos.parity, 7);
-        // the place of S is free: its last tile has been read
-        if constexpr (TM::kOneS) {
-            if (qk.m > 0) wait(bar.s_free + x_prev, k_prev & 1, 3);
-        } else {
-            if (qk.k > 0) wait(bar.s_free + qk.x, (qk.k - 1) & 1, 3);
-        }
-        tc_fence_after();
-        const uint32_t q_lo = q_lo0 + qk.x * (P::kQTile >> 4), k_lo = k_lo0 + qk.pos.stage * (P::kKTile >> 4), d_s = tmem_base + TM::s(qk.x);
-        if (leader && ok) {
-#pragma unroll
-            for (int j = 0; j < D / 16; ++j) {
-                // k-step of 16 elements: 32 bytes within a 64-element swizzle atom; atoms are 128 rows apart in a Q
-                // tile, and in a K tile as many as the CTA holds
-                const uint32_t off_q = ((j / 4) * (kBlockM * 128) + (j % 4) * 32) >> 4;
-                const uint32_t off_k = ((j / 4) * (P::kKRows * 128) + (j % 4) * 32) >> 4;
-                if constexpr (kPair) {
-                    if (j == 0) mma_ss_lo_pair<idesc_qk, 0>(d_s, q_lo, k_lo);
-                    else mma_ss_lo_pair<idesc_qk, 1>(d_s, q_lo + off_q, k_lo + off_k);
-                } else {
-                    if (j == 0) mma_ss_lo<idesc_qk, 0>(d_s, q_lo, k_lo);
-                    else mma_ss_lo<idesc_qk, 1>(d_s, q_lo + off_q, k_lo + off_k);
+    const int n_y = P::y_entries(w.n_parts);
+    uint32_t qk_odd = 0, pv_odd = 0;   // bit x: parity of the S (of the P V) of query tile x that there have been
+    int x_prev = -1;                   // of the item whose S was formed last
+    bool more = true;
+    w.set(w.first);
+    for (int n = 0; more; ++n) {
+        const Stream st = w.stream();
+        const int n_own0 = st.n_lead + 2 * st.n_shared, n_items = n_own0 + st.n_a + st.n_b;
+        const int turns = min(st.n_a, st.n_b), x_last = st.n_a > st.n_b ? 0 : 1;
+        auto advance = [&](Item &it) {
+            ++it.m;
+            if (it.m <= st.n_lead && it.m < n_own0) {
+                ++it.k;
+            } else if (it.m < n_own0) {
+                it.x ^= 1;
+                if (it.x == 1) {   // (both query tiles use the entry)
+                    it.k -= st.n_lead;
+                    return;
                 }
+                it.k += st.n_lead + 1;
+            } else {
+                const int s = it.m - n_own0;
+                it.x = s < 2 * turns ? s & 1 : x_last;
+                it.k = st.first_own(it.x) + (s < 2 * turns ? s >> 1 : s - turns);
             }
-            commit(bar.s_full + qk.x);
-        }
-        x_prev = qk.x;
-        k_prev = qk.k;
-        advance(qk);
-    };
-    auto issue_pv = [&]() {
-        const uint32_t v_lo = v_lo0 + pv.pos.stage * (P::kVTile >> 4), d_o = tmem_base + TM::o(pv.x), a_p = tmem_base + TM::p(pv.x);
-        const uint32_t acc0 = pv.k > 0 ? 1u : 0u;
-        wait(bar.p_full + pv.x, pv.k & 1, 5);
-        tc_fence_after();
-        if (leader && ok) {
+            it.pos.next(kStages);
+        };
+        auto issue_qk = [&]() {
+            // K and V of the entry have arrived (B follows A on the entries that they share)
+            if (qk.m >= n_own0 || qk.x == 0) wait(bar.kv_full + qk.pos.stage, qk.pos.parity, 7);
+            // the place of S is free: its last tile has been read (before the first there is none)
+            if constexpr (TM::kOneS) {
+                if (x_prev >= 0) wait(bar.s_free + x_prev, ((qk_odd >> x_prev) & 1) ^ 1, 3);
+            } else {
+                wait(bar.s_free + qk.x, ((qk_odd >> qk.x) & 1) ^ 1, 3);
+            }
+            tc_fence_after();
+            const uint32_t q_lo = q_lo0 + qk.x * (P::kQTile >> 4), k_lo = k_lo0 + qk.pos.stage * (P::kStage >> 4), d_s = tmem_base + TM::s(qk.x);
+            if (leader && ok) {
 #pragma unroll
-            for (int j = 0; j < 8; ++j) {   // 16 keys a step
-                if constexpr (kPair) mma_ts_lo_pair<idesc_pv>(d_o, a_p + j * 8, v_lo + j * (16 * 128 >> 4), j == 0 ? acc0 : 1u);
-                else mma_ts_lo<idesc_pv>(d_o, a_p + j * 8, v_lo + j * (16 * 128 >> 4), j == 0 ? acc0 : 1u);
+                for (int j = 0; j < D / 16; ++j) {
+                    // k-step of 16 elements: 32 bytes within a 64-element swizzle atom; atoms are 128 rows apart in a Q
+                    // tile, and in a K tile as many as the CTA holds
+                    const uint32_t off_q = ((j / 4) * (kBlockM * 128) + (j % 4) * 32) >> 4;
+                    const uint32_t off_k = ((j / 4) * (P::kKRows * 128) + (j % 4) * 32) >> 4;
+                    if constexpr (kPair) {
+                        if (j == 0) mma_ss_lo_pair<idesc_qk, 0>(d_s, q_lo, k_lo);
+                        else mma_ss_lo_pair<idesc_qk, 1>(d_s, q_lo + off_q, k_lo + off_k);
+                    } else {
+                        if (j == 0) mma_ss_lo<idesc_qk, 0>(d_s, q_lo, k_lo);
+                        else mma_ss_lo<idesc_qk, 1>(d_s, q_lo + off_q, k_lo + off_k);
+                    }
+                }
+                commit(bar.s_full + qk.x);
+                if (qk.m + 1 == n_items) commit(bar.q_empty);
             }
-            commit(bar.pv_done + pv.x);
+            x_prev = qk.x;
+            qk_odd ^= 1u << qk.x;
+            advance(qk);
+        };
+        auto issue_pv = [&]() {
+            const uint32_t v_lo = v_lo0 + pv.pos.stage * (P::kStage >> 4), d_o = tmem_base + TM::o(pv.x), a_p = tmem_base + TM::p(pv.x);
+            const uint32_t acc0 = pv.k > 0 ? 1u : 0u;
+            wait(bar.p_full + pv.x, (pv_odd >> pv.x) & 1, 5);
+            tc_fence_after();
+            if (leader && ok) {
+#pragma unroll
+                for (int j = 0; j < 8; ++j) {   // 16 keys a step
+                    if constexpr (kPair) mma_ts_lo_pair<idesc_pv>(d_o, a_p + j * 8, v_lo + j * (16 * 128 >> 4), j == 0 ? acc0 : 1u);
+                    else mma_ts_lo<idesc_pv>(d_o, a_p + j * 8, v_lo + j * (16 * 128 >> 4), j == 0 ? acc0 : 1u);
+                }
+                commit(bar.pv_done + pv.x);
+                // (an entry that both query tiles use is done with B's product)
+                if (pv.x == 1 || pv.m < st.n_lead || pv.m >= n_own0) commit(bar.kv_empty + pv.pos.stage);
+            }
+            pv_odd ^= 1u << pv.x;
+            advance(pv);
+        };
+        wait(bar.q_full, n & 1, 4);
+        tc_fence_after();
+        for (int m = 0; m < min(kAhead, n_items); ++m) issue_qk();
+        while (pv.m < n_items) {
+            issue_pv();
+            if (qk.m < n_items) issue_qk();
         }
-        advance(pv);
-    };
-    for (int m = 0; m < min(kAhead, n_items); ++m) issue_qk();
-    while (pv.m < n_items) {
-        issue_pv();
-        if (qk.m < n_items) issue_qk();
+        // past the entries of the outputs
+        qk.pos.skip(n_y * w.n_query_tiles(), kStages);
+        pv = qk = Item{0, 0, 0, qk.pos};
+        if (!__all_sync(0xffffffffu, ok)) break;
+        more = next_item_of_warp<kPair>(w, bar, n, abort_flag, status, ok);
     }
     if (!__all_sync(0xffffffffu, ok) && leader) {  // no MMA may still be running when tensor memory is freed
         if constexpr (kPair) {
@@ -645,15 +849,19 @@ __device__ __forceinline__ void mma_role(const Stream &st, const AttnBars &bar, 
     }
 }
 
-// Softmax-attention branch and merge for rows [R0, R0 + 256) (a pair: 512) of one (batch, head).
+// Softmax-attention branch and merge: items of 256 (a pair: 512) rows of one (batch, head), see Work.  Between two items little
+// comes: the next Q comes in while the last products run, its first S is formed while the softmax warps merge, and the linear
+// branch's results and the output pass through the key ring, so that neither waits for memory.  (With a CTA per item an item
+// had, beside 2900 to 3300 cycles for a tile of both query tiles, a start of some 3000 cycles and an end of 3000 to 5000 without
+// a linear branch, 8000 with it, and 15000 to 38000 where its results had left L2; now 3000 to 6500 in all.  us of the
+// kernel, then and now, in turn on one box: 128 heads x 4096 tokens, d = 64, a quarter kept 270 and 227; 64 x 32768, d = 128, a
+// quarter kept 4229 and 3745; 32 x 131072, capped at 896, 3960 and 2865.)
 template <int D, bool kPair>
-__device__ __forceinline__ void attention_body(const CUtensorMap &tm_q, const CUtensorMap &tm_k, const CUtensorMap &tm_v,
-                                               const CUtensorMap &tm_ksel, const CUtensorMap &tm_vsel, const __nv_bfloat16 *y_part,
-                                               const float *d_part, int n_parts, __nv_bfloat16 *Y, int *status, int H, int Hkv, int N,
-                                               int C, int lam, int budget, int sel_rows, int sel_identity, float scale_log2,
-                                               int n_blocks, int n_heads, int set_heads) {
+__device__ __forceinline__ void attention_body(const AttnMaps &tm, const float *d_part, __nv_bfloat16 *Y, int *status, int H, int Hkv,
+                                               int N, int C, int lam, int budget, int sel_rows, int sel_identity, int n_parts,
+                                               float scale_log2, int n_blocks, int n_heads, int set_heads) {
     using P = AttnPlan<D, kPair>;
-    constexpr int kCtas = kPair ? 2 : 1, kRows = kCtas * kBlockM;
+    constexpr int kCtas = kPair ? 2 : 1, kRows = kCtas * kBlockM, kStages = P::kStages;
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     const AttnBars bar = AttnBars::at(smem, P{});
@@ -665,11 +873,8 @@ __device__ __forceinline__ void attention_body(const CUtensorMap &tm_q, const CU
     // the same in all lanes)
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const uint32_t rank = kPair ? blockIdx.x & 1u : 0u, peer = rank ^ 1u;
-    int rb, bh;
-    row_block(kPair ? blockIdx.x >> 1 : blockIdx.x, n_blocks, n_heads, set_heads, rb, bh);
-    const int b = bh / H, h = bh % H, kvh = h / (H / Hkv);
-    const int R0 = rb * 2 * kRows;
-    const Stream st = make_stream(R0, kRows, N, C, lam, budget);
+    Work w{n_blocks, n_heads, set_heads, H, Hkv, N, C == 128 ? 7 : 6, lam, budget, sel_rows, sel_identity, n_parts, kRows,
+           (int)(kPair ? blockIdx.x >> 1 : blockIdx.x), n_blocks * n_heads, reinterpret_cast<volatile int *>(smem + P::kMisc + 16), 0, 0};
     auto sync_all = [&]() {
         if constexpr (kPair) cluster_sync_all();
         else __syncthreads();
@@ -677,16 +882,22 @@ __device__ __forceinline__ void attention_body(const CUtensorMap &tm_q, const CU
 
     if (threadIdx.x == 0) {
         mbar_init(bar.q_full, 1);
-        for (int i = 0; i < P::kStages; ++i) {
+        mbar_init(bar.q_empty, 1);
+        for (int i = 0; i < kStages; ++i) {
             mbar_init(bar.kv_full + i, 1);
-            mbar_init(bar.kv_empty + i, 2);   // one share per query tile
+            mbar_init(bar.kv_empty + i, 1);   // the last product that reads the stage has, or the output has left it
         }
         for (int i = 0; i < 2; ++i) {
             mbar_init(bar.s_full + i, 1);
             mbar_init(bar.s_free + i, kCtas * 4);   // one arrival per softmax warp of the query tile
             mbar_init(bar.p_full + i, kCtas * 4);
             mbar_init(bar.pv_done + i, 1);
+            mbar_init(bar.y_full + i, P::y_entries(n_parts));
+            mbar_init(bar.item_full + i, 1);
+            mbar_init(bar.y_ready + i, 4);
+            mbar_init(bar.item_empty + i, kCtas * 10 + 1 + (kCtas - 1));   // softmax and output warps, the issuing warp, the other producer
         }
+        mbar_init(bar.first_done, 1);
         mbar_init(bar.drain, 1);
         *abort_flag = 0;
         // A CTA that starts after another one has reported a failure does nothing; in a pair the first decides for both.
@@ -717,26 +928,43 @@ __device__ __forceinline__ void attention_body(const CUtensorMap &tm_q, const CU
     // a role that gives up tells the other CTA, whose waits would otherwise run to their own limit
     auto tell_peer = [&]() { st_cluster_u32(mapa(smem_u32(const_cast<int *>(abort_flag)), peer), 1u); };
 
-    // Registers move from the last four warps to the softmax warps, whose threads hold a row of S (per scheduler: 2 x 208 + 88
-    // registers for its three warps, of the 3 x 168 that the CTA was launched with).
+    // Registers move from the last four warps to the softmax warps, whose threads hold a row of S (per scheduler, of the 3 x 168
+    // registers that the CTA was launched with).
+    constexpr int kSoftmaxRegs = 224, kOtherRegs = 3 * 168 - 2 * kSoftmaxRegs;
     if (warp >= kProducerWarp) {
-        reg_dec<88>();
+        reg_dec<kOtherRegs>();
         if (warp == kProducerWarp) {
-            // With topk = chunk every token is selected and the compacted arrays would be copies of K / V: the salient
-            // prefix is then read from K / V themselves (tm_ksel / tm_vsel alias tm_k / tm_v).
-            const int kv_row0 = (b * Hkv + kvh) * N;
             if (lane == 0)
-                producer_role<D, kPair>(st, bar, smem, rank, tm_q, tm_k, tm_v, tm_ksel, tm_vsel, bh * N + R0, kv_row0,
-                                        sel_identity ? kv_row0 : bh * sel_rows, abort_flag, status, tell_peer);
+                producer_role<D, kPair>(w, bar, smem, rank, tm.q, tm.k, tm.v, tm.ksel, tm.vsel, tm.p0, tm.p1, abort_flag, status, tell_peer);
         } else if (warp == kMmaWarp && rank == 0) {
-            mma_role<D, kPair>(st, bar, smem, tmem_base, abort_flag, status, tell_peer);
+            mma_role<D, kPair>(w, bar, smem, tmem_base, abort_flag, status, tell_peer);
+        } else if (warp > kMmaWarp) {
+            output_role<D, kPair>(w, bar, smem + P::kK, warp - kMmaWarp - 1, rank, tm.y, d_part, Y, abort_flag, status);
         }
     } else {
-        reg_inc<208>();
+        reg_inc<kSoftmaxRegs>();
         const int x = warp >> 2;                       // 0: tile A, 1: tile B
-        softmax_role<D, kPair>(st, bar, x, R0 + (x * kCtas + (int)rank) * kBlockM, tmem_base, abort_flag, status,
-                                               smem + P::kQ + x * P::kQTile, y_part, d_part, n_parts, (long long)n_heads * N * D, (long long)n_heads * N, Y, bh, N,
-                                               C, lam, budget, scale_log2);
+        const int n_y = P::y_entries(n_parts);
+        int ring0 = 0, flip = 0, y_flip = 0;           // ring stage of the item's first entry; see softmax_role
+        w.set(w.first);
+        bool ok = true, more = true;
+        for (int n = 0; more && ok; ++n) {
+            const Stream st = w.stream();
+            const Stream::Mine my = st.mine(x);
+            const int y_stage = (ring0 + st.entries() + x * n_y) % kStages;
+            ring0 = (ring0 + st.entries() + n_y * w.n_query_tiles()) % kStages;
+            const int row0 = w.R0 + (x * kCtas + (int)rank) * kBlockM, bh = w.bh;
+            auto ahead = [&](bool &last) {   // (while the item's last product runs)
+                bool waited;
+                more = next_item_of_warp<kPair>(w, bar, n, abort_flag, status, waited);
+                last = !more;
+                return waited;
+            };
+            ok = softmax_role<D, kPair>(my, bar, x, row0, tmem_base, abort_flag, status, smem + P::kK, y_stage, flip, y_flip, d_part,
+                                        n_parts, (long long)n_heads * N, Y, bh, N, w.log2_c, lam, budget, scale_log2, ahead);
+            flip ^= my.n & 1;
+            y_flip ^= my.n > 0 ? 1 : 0;
+        }
         if constexpr (kPair) {
             if (*abort_flag) tell_peer();
         }
@@ -753,15 +981,13 @@ __device__ __forceinline__ void attention_body(const CUtensorMap &tm_q, const CU
 
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
-sa_merge_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                   const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ksel,
-                   const __grid_constant__ CUtensorMap tm_vsel, const __nv_bfloat16 *y_part, const float *d_part, int n_parts,
-                   __nv_bfloat16 *Y, int *status, int H, int Hkv, int N, int C, int lam, int budget, int sel_rows, int sel_identity,
-                   float scale_log2, int n_blocks, int n_heads, int set_heads) {
+sa_merge_tc_kernel(const __grid_constant__ AttnMaps tm, const float *d_part, __nv_bfloat16 *Y, int *status, int H, int Hkv, int N, int C,
+                   int lam, int budget, int sel_rows, int sel_identity, int n_parts, float scale_log2, int n_blocks, int n_heads,
+                   int set_heads) {
     grid_dep_wait();
     grid_dep_launch();
-    attention_body<D, false>(tm_q, tm_k, tm_v, tm_ksel, tm_vsel, y_part, d_part, n_parts, Y, status, H, Hkv, N, C, lam, budget, sel_rows,
-                             sel_identity, scale_log2, n_blocks, n_heads, set_heads);
+    attention_body<D, false>(tm, d_part, Y, status, H, Hkv, N, C, lam, budget, sel_rows, sel_identity, n_parts, scale_log2, n_blocks,
+                             n_heads, set_heads);
 }
 
 // The same branch on CTA pairs (head dim 128): two CTAs of a cluster work on 512 consecutive query rows of
@@ -776,19 +1002,17 @@ sa_merge_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_consta
 // Who signals whom.  K / V / Q tiles: every CTA loads its halves into its own shared memory with plain TMA
 // loads (no multicast) whose byte counts complete on the full-barriers of rank 0, where the issuing thread
 // waits.  S_X ready, P_X V done: one tcgen05.commit arrives on the barrier of both CTAs.  S_X read, P_X written: the
-// softmax warps of both CTAs arrive on rank 0's barriers.  Ring stages are released locally: what a CTA's softmax
-// warps see completed has completed in both CTAs.
+// softmax warps of both CTAs arrive on rank 0's barriers.  Ring stages of keys are free in both CTAs with the commit of the last
+// product that reads them, an output's stage when the CTA's own output warp is done with it.
 template <int D>
 __global__ void __cluster_dims__(2, 1, 1) __launch_bounds__(kThreads, 1)
-sa_merge_pair_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
-                     const __grid_constant__ CUtensorMap tm_v, const __grid_constant__ CUtensorMap tm_ksel,
-                     const __grid_constant__ CUtensorMap tm_vsel, const __nv_bfloat16 *y_part, const float *d_part, int n_parts,
-                     __nv_bfloat16 *Y, int *status, int H, int Hkv, int N, int C, int lam, int budget, int sel_rows, int sel_identity,
-                     float scale_log2, int n_blocks, int n_heads, int set_heads) {
+sa_merge_pair_kernel(const __grid_constant__ AttnMaps tm, const float *d_part, __nv_bfloat16 *Y, int *status, int H, int Hkv, int N, int C,
+                     int lam, int budget, int sel_rows, int sel_identity, int n_parts, float scale_log2, int n_blocks, int n_heads,
+                     int set_heads) {
     grid_dep_wait();
     grid_dep_launch();
-    attention_body<D, true>(tm_q, tm_k, tm_v, tm_ksel, tm_vsel, y_part, d_part, n_parts, Y, status, H, Hkv, N, C, lam, budget, sel_rows,
-                            sel_identity, scale_log2, n_blocks, n_heads, set_heads);
+    attention_body<D, true>(tm, d_part, Y, status, H, Hkv, N, C, lam, budget, sel_rows, sel_identity, n_parts, scale_log2, n_blocks,
+                            n_heads, set_heads);
 }
 
 // ---------------------------------------------------------------------------
@@ -1158,36 +1382,36 @@ int launch_tc(const still_params_t *p, long long N, const void *Q, const void *K
     const unsigned long long kv_rows = (unsigned long long)p->B * p->Hkv * N;
     const unsigned long long sel_total = identity ? kv_rows : (unsigned long long)BH * sel_rows;
     constexpr bool kPair = D == 128;   // head dim 128 runs on CTA pairs, each CTA holding 64 keys of a K tile
-    CUtensorMap tq, tk, tv, tks, tvs;
-    if (!make_map(&tq, Q, (unsigned long long)BH * N, D) ||
-        !make_map_2d(&tk, K, kv_rows, D, kPair ? kBlockN / 2 : kBlockN, false) || !make_map(&tv, V, kv_rows, D) ||
-        !make_map_2d(&tks, identity ? K : k_sel, sel_total, D, kPair ? kBlockN / 2 : kBlockN, false) ||
-        !make_map(&tvs, identity ? V : v_sel, sel_total, D))
+    const unsigned long long q_rows = (unsigned long long)BH * N;
+    const bf *part = (const bf *)(n_parts > 0 ? y_part : Y);   // (the maps of absent parts are not used)
+    AttnMaps tm;
+    if (!make_map(&tm.q, Q, q_rows, D) || !make_map_2d(&tm.k, K, kv_rows, D, kPair ? kBlockN / 2 : kBlockN, false) ||
+        !make_map(&tm.v, V, kv_rows, D) ||
+        !make_map_2d(&tm.ksel, identity ? K : k_sel, sel_total, D, kPair ? kBlockN / 2 : kBlockN, false) ||
+        !make_map(&tm.vsel, identity ? V : v_sel, sel_total, D) || !make_map(&tm.p0, part, q_rows, D) ||
+        !make_map(&tm.p1, n_parts > 1 ? part + q_rows * D : part, q_rows, D) || !make_map(&tm.y, Y, q_rows, D))
         return STILL_ERR_CUDA;
     const float scale_log2 = p->sm_scale * 1.4426950408889634f;
     const int rep = p->H / p->Hkv;
     const int set_heads = set_of_heads(BH, rep, ((identity ? 0 : sel_rows) + N / rep + 1) * D * 4);
-    if constexpr (kPair) {
-        const int n_pairs = (int)((N + 4 * kBlockM - 1) / (4 * kBlockM));
-        if (ensure_dynamic_smem((const void *)sa_merge_pair_kernel<D>, (AttnPlan<D, true>::kAlloc)) != cudaSuccess) return STILL_ERR_CUDA;
-        dim3 grid((unsigned)(2 * n_pairs * BH));   // clusters of two
-        profile_mark_begin(st);
-        const cudaError_t e = launch_dependent(sa_merge_pair_kernel<D>, grid, dim3(kThreads), (AttnPlan<D, true>::kAlloc), st,
-            tq, tk, tv, tks, tvs, (const bf *)y_part, d_part, n_parts, (bf *)Y, status, p->H, p->Hkv, (int)N, p->chunk, p->topk, (int)p->max_salient, (int)sel_rows,
-            identity ? 1 : 0, scale_log2, n_pairs, (int)BH, set_heads);
-        profile_mark_end(st);
-        if (e != cudaSuccess) return STILL_ERR_CUDA;
-    } else {
-        const int n_qblocks = (int)((N + 2 * kBlockM - 1) / (2 * kBlockM));
-        if (ensure_dynamic_smem((const void *)sa_merge_tc_kernel<D>, (AttnPlan<D, false>::kAlloc)) != cudaSuccess) return STILL_ERR_CUDA;
-        dim3 grid((unsigned)(n_qblocks * BH));
-        profile_mark_begin(st);
-        const cudaError_t e = launch_dependent(sa_merge_tc_kernel<D>, grid, dim3(kThreads), (AttnPlan<D, false>::kAlloc), st,
-            tq, tk, tv, tks, tvs, (const bf *)y_part, d_part, n_parts, (bf *)Y, status, p->H, p->Hkv, (int)N, p->chunk, p->topk, (int)p->max_salient, (int)sel_rows,
-            identity ? 1 : 0, scale_log2, n_qblocks, (int)BH, set_heads);
-        profile_mark_end(st);
-        if (e != cudaSuccess) return STILL_ERR_CUDA;
-    }
+    int dev = 0, n_sm = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess ||
+        cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess || n_sm <= 0)
+        return STILL_ERR_CUDA;
+    constexpr int kCtas = kPair ? 2 : 1, kSmem = AttnPlan<D, kPair>::kAlloc;
+    const auto kernel = [] {
+        if constexpr (kPair) return sa_merge_pair_kernel<D>;
+        else return sa_merge_tc_kernel<D>;
+    }();
+    if (ensure_dynamic_smem((const void *)kernel, kSmem) != cudaSuccess) return STILL_ERR_CUDA;
+    const long long n_blocks = (N + kCtas * 2 * kBlockM - 1) / (kCtas * 2 * kBlockM), items = n_blocks * BH;
+    const dim3 grid((unsigned)(kCtas * std::min<long long>(items, std::max(1, n_sm / kCtas))));   // they stay (see Work)
+    profile_mark_begin(st);
+    const cudaError_t e = launch_dependent(kernel, grid, dim3(kThreads), kSmem, st, tm, d_part, (bf *)Y, status, p->H, p->Hkv, (int)N, p->chunk,
+                                           p->topk, (int)p->max_salient, (int)sel_rows, identity ? 1 : 0, n_parts, scale_log2, (int)n_blocks,
+                                           (int)BH, set_heads);
+    profile_mark_end(st);
+    if (e != cudaSuccess) return STILL_ERR_CUDA;
     ++*launches;
     if (cudaGetLastError() != cudaSuccess) return STILL_ERR_CUDA;
     return STILL_OK;

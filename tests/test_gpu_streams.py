@@ -144,3 +144,21 @@ def test_nan_and_infinite_logits_make_the_output_nan(d, N, key, bad):
     Y = still.hybrid_attn_fwd(U.params_of(w), Q.abs() + 1, K, V)[0]
     assert bool(torch.isnan(Y[:, :2, key:]).all())
     assert bool(torch.isfinite(Y[:, :2, :key]).all()) and bool(torch.isfinite(Y[:, 2:]).all())
+
+
+@pytest.mark.parametrize("d,B,N,k,budget", [
+    # more items than CTAs: of 256 rows (d = 64) or 512; the last one of a head without a second query tile, with whole rows
+    # only, with one row
+    (64, 5, 300, 16, 0), (64, 5, 512, 64, 0), (64, 3, 641, 16, 64), (128, 5, 700, 16, 0), (128, 3, 700, 32, 64), (128, 3, 1024, 64, 0),
+    (128, 3, 1025, 64, 0),
+])
+def test_items_of_a_cta_do_not_mix(d, B, N, k, budget):
+    # A head's rows are those of the call with this head alone, bit for bit, whatever its CTAs worked on before.
+    w = synth.Workload("t", B, 32, 32, d, N, 64, k, "bf16", "head_scale", 33)
+    r = U.run_prefill(w, gate=k < 64, max_salient=budget)
+    one = synth.Workload("t", 1, 1, 1, d, N, 64, k, "bf16", "head_scale", 33)
+    p = U.params_of(one, max_salient=budget)
+    for b, h in ((0, 0), (0, 31), (B // 2, 7), (B - 1, 30), (B - 1, 31)):
+        x = [None if t is None else t[b: b + 1, h: h + 1].contiguous() for t in (r["Q"], r["K"], r["V"], r["G"])]
+        Y, _, _ = still.hybrid_attn_fwd(p, x[0], x[1], x[2], r["Wq"][h: h + 1].contiguous(), r["Wk"][h: h + 1].contiguous(), G=x[3])
+        assert torch.equal(Y[0, 0], r["Y"][b, h])
