@@ -1030,22 +1030,23 @@ sa_merge_pair_kernel(const __grid_constant__ AttnMaps tm, const float *d_part, _
 // (tile n = head n / n_row_blocks, rows 128 (n % n_row_blocks) ...) with two stages of shared memory and two
 // TMEM accumulators, so that the loads of tile n+1 and its UMMA run under the row epilogue of tile n.
 // The row's epilogue bounds it: three special-function instructions per window element (one 2^x, two logarithms) against
-// six or seven others, by eight warps an SM, two tiles at a time (d = 128, C = 64: special-function unit 53 % busy, issue slots
-// 38 %, DRAM 38 %; C = 128: 61, 37 and 24 %).  2 x 32 heads x 32768 tokens, d = 128, C = 64: 199 us, 4 x 32 x 4096, d = 64: 51 us,
+// six or seven others, by twelve warps an SM at C = 64, eight at C = 128 (with eight at C = 64, too: special-function unit 53 %
+// busy, issue slots 38 %, DRAM 38 % at d = 128; C = 128: 61, 37 and 24 %).  us of a
+// call for the scores alone with eight and twelve warps, in turn on one box: 2 x 32 heads x 32768 tokens, d = 128, 201 to 219 and 175
+// to 180, 4 x 32 x 4096, d = 64, 60.5 and 56.  The kernel with eight: 2 x 32 heads x 32768 tokens, d = 128, C = 64: 199 us, 4 x 32 x 4096, d = 64: 51 us,
 // 32 x 131072, d = 128, C = 128: 650 us (with a threshold per token in the ranking, see below: 223, 58 and 825; with scalar
 // arithmetic, logarithms for subnormal arguments, and for C = 128 a second set of exponentials as well: 325 to 368, 83 and 1030).
-// Warps: 0 TMA producer, 1 MMA issuer, 2-5 score group 0 (even tiles of the CTA), 6-9 score group 1 (odd
-// tiles); TMEM lane quarter = warp % 4.
+// Warps: 0 TMA producer, 1 MMA issuer, 2-5 score group 0, 6-9 score group 1, ...; TMEM lane quarter = warp % 4.
 // ---------------------------------------------------------------------------
 template <int D>
 struct ScoreSmem {
     static constexpr int kQBytes = kBlockM * D * 2, kKBytes = 2 * kBlockN * D * 2;
     static constexpr int kStage = kQBytes + kKBytes;
-    static constexpr int kBar = 2 * kStage;          // full[2], mma_done[2], smem_free[2], tmem_free[2]
-    static constexpr int kMisc = kBar + 8 * 8;       // tmem base, abort flag
-    static constexpr int kSc = kMisc + 16;           // [2][128] ranking keys of the group's tile (16-byte aligned)
-    static constexpr int kBallot = kSc + 2 * kBlockM * 4;   // [2][4]
-    static constexpr int kTotal = kBallot + 2 * 4 * 4;
+    static constexpr int kBar = 2 * kStage;          // full[2], smem_free[2], tmem_free[2], mma_done[4]
+    static constexpr int kMisc = kBar + 10 * 8;      // tmem base, abort flag
+    static constexpr int kSc = kMisc + 16;           // [4][128] ranking keys of a group's tile (16-byte aligned)
+    static constexpr int kBallot = kSc + 4 * kBlockM * 4;   // [4][4]
+    static constexpr int kTotal = kBallot + 4 * 4 * 4;
     static constexpr int kAlloc = kTotal + 1024;     // slack to align the base to 1024
 };
 
@@ -1062,8 +1063,14 @@ __device__ __forceinline__ float log2_of(float x) {
     return y;
 }
 
+// Score groups of four warps, which take a CTA's tiles in turn: three where a row's C values leave the registers for it (two at
+// C = 128, where a third made the rows spill).
+template <int C>
+constexpr int kScoreGroups = C == 64 ? 3 : 2;
+template <int C>
+constexpr int kScoreThreads = 64 + 128 * kScoreGroups<C>;
 template <int D, int C, bool kTinyEps>
-__global__ void __launch_bounds__(320, 1)
+__global__ void __launch_bounds__(kScoreThreads<C>, 1)
 score_select_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_constant__ CUtensorMap tm_k,
                        float *scores, int32_t *sel_idx, int *status, int H, int Hkv,
                        int N, int lam, float scale_log2, float eps, int n_row_blocks, int n_tiles) {
@@ -1074,7 +1081,8 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     extern __shared__ uint8_t smem_raw[];
     uint8_t *smem = reinterpret_cast<uint8_t *>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
     uint64_t *full = reinterpret_cast<uint64_t *>(smem + P::kBar);
-    uint64_t *mma_done = full + 2, *smem_free = full + 4, *tmem_free = full + 6;
+    // (mma_done: of a score group, which so sees every phase of the barrier that it waits on; smem_free, tmem_free: of a stage)
+    uint64_t *smem_free = full + 2, *tmem_free = full + 4, *mma_done = full + 6;
     uint32_t *tmem_base_slot = reinterpret_cast<uint32_t *>(smem + P::kMisc);
     volatile int *abort_flag = reinterpret_cast<volatile int *>(smem + P::kMisc + 8);
 
@@ -1084,10 +1092,10 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
     if (threadIdx.x == 0) {
         for (int s = 0; s < 2; ++s) {
             mbar_init(full + s, 1);
-            mbar_init(mma_done + s, 1);
             mbar_init(smem_free + s, 1);
             mbar_init(tmem_free + s, 4);   // one arrival per warp of the score group
         }
+        for (int g = 0; g < kScoreGroups<C>; ++g) mbar_init(mma_done + g, 1);
         *abort_flag = 0;
         fence_barrier_init();
     }
@@ -1139,26 +1147,28 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                     const uint32_t ka = k_a + (k / 4) * (2 * kBlockN * 128) + (k % 4) * 32;
                     mma_ss(tmem_base + s * 256, smem_desc(qa, 0), smem_desc(ka, 0), idesc, k > 0 ? 1u : 0u);
                 }
-                tc_commit(mma_done + s);
+                tc_commit(mma_done + it % kScoreGroups<C>);
             }
             // no MMA may still be running when tensor memory is freed: after a failure wait (bounded) for the
             // last group issued (its commit covers everything before it)
-            if (!ok && it > 0) mbar_wait_drain(mma_done + ((it - 1) & 1), ((it - 1) >> 1) & 1);
+            if (!ok && it > 0) mbar_wait_drain(mma_done + (it - 1) % kScoreGroups<C>, ((it - 1) / kScoreGroups<C>) & 1);
         }
     } else {
-        const int g = (warp - 2) >> 2;                 // score group = stage = TMEM accumulator
+        constexpr int kGroups = kScoreGroups<C>;
+        const int g = (warp - 2) >> 2;                 // score group: tiles g, g + kGroups, ... of the CTA
         const int wq = warp & 3;                       // TMEM lane quarter this warp may read
         const int r = wq * 32 + lane;                  // row of the tile owned by this thread
         int *keys = reinterpret_cast<int *>(smem + P::kSc) + g * kBlockM;
         uint32_t *ballots = reinterpret_cast<uint32_t *>(smem + P::kBallot) + g * 4;
-        const uint32_t taddr = tmem_base + g * 256 + ((uint32_t)(wq * 32) << 16) + (uint32_t)(wq * 32 + kBlockN - C);
+        const uint32_t taddr0 = tmem_base + ((uint32_t)(wq * 32) << 16) + (uint32_t)(wq * 32 + kBlockN - C);
         const int group_bar = 1 + g;
         int it = g, j = 0;
-        for (int n = blockIdx.x + g * gridDim.x; n < n_tiles; n += 2 * gridDim.x, it += 2, ++j) {
-            const int ph = j & 1;
+        for (int n = blockIdx.x + g * gridDim.x; n < n_tiles; n += kGroups * gridDim.x, it += kGroups, ++j) {
+            const int st = kGroups == 2 ? g : it & 1;      // stage and TMEM accumulator
+            const uint32_t taddr = taddr0 + st * 256;
             const int bh = n / n_row_blocks, R0 = (n - bh * n_row_blocks) * kBlockM;
             const int t = R0 + r;
-            bool ok = mbar_wait(mma_done + g, ph, abort_flag, status, 21);
+            bool ok = mbar_wait(mma_done + g, j & 1, abort_flag, status, 21);
             // the group leaves the loop together
             {
                 uint32_t all_ok;
@@ -1168,7 +1178,7 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
             }
             if (!ok) break;
             tc_fence_after();
-            if (r == 0) mbar_arrive(smem_free + g);    // the logits are complete: the stage's operands are free
+            if (r == 0) mbar_arrive(smem_free + st);   // the logits are complete: the stage's operands are free
             float score = 0.f;
             {
                 // Element j of the warp's C+32 columns is the key at position R0 + 32 wq - C + j, and the window of
@@ -1200,7 +1210,7 @@ score_select_tc_kernel(const __grid_constant__ CUtensorMap tm_q, const __grid_co
                 auto tmem_read_done = [&]() {   // the accumulator may be overwritten by the UMMA of the tile after next
                     tc_fence_before();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(tmem_free + g);
+                    if (lane == 0) mbar_arrive(tmem_free + st);
                 };
                 // The row is held in registers (C values; at C = 128 some 50 bytes of a thread's spill): one read of tensor
                 // memory, exponentials kept in place.
@@ -1435,7 +1445,7 @@ int launch_score_tc(const still_params_t *p, long long N, const void *Q, const v
     const long long n_row_blocks = (N + kBlockM - 1) / kBlockM, n_tiles = n_row_blocks * BH;
     if (n_tiles >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;
     const unsigned grid = (unsigned)std::min<long long>(n_tiles, n_sm);   // one persistent CTA per SM
-    if (launch_dependent(kernel, dim3(grid), dim3(320), kSmem, st, tq, tk, scores, sel_idx, status, p->H, p->Hkv, (int)N, p->topk,
+    if (launch_dependent(kernel, dim3(grid), dim3(kScoreThreads<C>), kSmem, st, tq, tk, scores, sel_idx, status, p->H, p->Hkv, (int)N, p->topk,
                          p->sm_scale * 1.4426950408889634f, p->eps, (int)n_row_blocks, (int)n_tiles) != cudaSuccess)
         return STILL_ERR_CUDA;
     ++*launches;

@@ -162,3 +162,14 @@ def test_items_of_a_cta_do_not_mix(d, B, N, k, budget):
         x = [None if t is None else t[b: b + 1, h: h + 1].contiguous() for t in (r["Q"], r["K"], r["V"], r["G"])]
         Y, _, _ = still.hybrid_attn_fwd(p, x[0], x[1], x[2], r["Wq"][h: h + 1].contiguous(), r["Wk"][h: h + 1].contiguous(), G=x[3])
         assert torch.equal(Y[0, 0], r["Y"][b, h])
+
+
+@pytest.mark.parametrize("d,C,N", [(64, 64, 900), (128, 64, 1000), (64, 128, 900), (128, 64, 2305)])
+def test_score_tiles_of_a_cta(d, C, N):
+    # several tiles for every CTA of the score kernel, in turn by its groups of warps: not as many for every CTA, and a ragged one
+    # at the end of every head
+    w = synth.Workload("t", 2, 32, 8, d, N, C, C // 4, "bf16", "head_scale", 35)
+    r = U.run_prefill(w)
+    heads = [(0, 0), (0, 13), (1, 7), (1, 31)]
+    U.check_selection(r["scores"], r["sel"], C, C // 4, heads)
+    U.check_outputs(w, r["Q"], r["K"], r["V"], r["Wq"], r["Wk"], r["Y"], r["scores"], r["sel"], heads[1:], rows=U.sample_rows(N, 100, C))
