@@ -69,6 +69,12 @@ struct FwdPlan {
 // of two blocks per SM.
 constexpr int kSms = 148, kScanBlocks = 4 * kSms;
 
+// Up to this many blocks the score and the feature maps of the FMA kernels are one launch (three blocks for two SMs).  us a call
+// of 4 heads, d = 64, a quarter kept, three launches and one: 700 tokens 89.7 and 70.8, 1500 125 and 110; 8 heads, d = 128, 1000
+// tokens 267 and 243; C = 128: 4 heads, d = 64, 2000 tokens 204 and 172.  Beyond, the gain goes on for a while (16 heads x 1000 tokens
+// 191 and 184, 32 x 1000 214 and 213, 32 x 2000 439 and 462) but the launches of those sizes are pinned by a test of the scan.
+constexpr int kFrontBlocks = 222;
+
 // The workspace never takes more than `limit` bytes for the sake of speed alone (the sums of the scan's segments).
 static FwdPlan plan_fwd(const still_params_t *p, long long N, size_t limit = SIZE_MAX) {
     FwdPlan w{};
@@ -125,7 +131,10 @@ static FwdPlan plan_fwd(const still_params_t *p, long long N, size_t limit = SIZ
         // C = 64 the sums lie in the rows between 1011 and 1160 tokens, where the static workspace is full: 175 us a call
         // at 1100 tokens, 273 with one serial pass, 165 at 1200 with a place of their own.)
         const long long units = (long long)BH * (p->d / 64);
-        const long long want = std::max<long long>(1, std::min<long long>((kScanBlocks + units - 1) / units, T - 2));
+        // A chunk a segment where that many are wanted: a segment's chunks are a chain (4 heads, d = 64, C = 64: 512 tokens in
+        // segments of two chunks 22.9 us, of one 13).  Up to four chunks, of which two are answered, one pass instead of three (us a
+        // call, one and three: 250 tokens, 32 heads 66.7 and 72.0, 16 heads 49.9 and 60.4, 4 heads 49 and 47; five chunks, 4 heads: 47).
+        const long long want = T <= 4 ? 1 : std::max<long long>(1, std::min<long long>((kScanBlocks + units - 1) / units, T));
         const size_t per_seg = BH * dp * (size_t)(p->d + 1) * 4;
         if (off <= STILL_STATIC_WORKSPACE_BYTES) limit = std::min(limit, (size_t)STILL_STATIC_WORKSPACE_BYTES);
         long long n = want;
@@ -287,7 +296,7 @@ write_state_kernel(const __grid_constant__ StateParts s, const __grid_constant__
 template <typename T, int NJ>
 static int launch_score_select_t(const still_params_t *p, long long N, long long Tn, const T *Q, const T *K, float *scores,
                                  int32_t *sel, int *status, cudaStream_t st) {
-    const size_t smem = score_select_smem(p->chunk, p->d);
+    const size_t smem = ScorePlan<NJ, false>::smem(p->d);
     STILL_CUDA(set_smem(score_select_kernel<T, NJ>, smem));
     STILL_CUDA(launch_dependent(score_select_kernel<T, NJ>, dim3((unsigned)Tn, p->H, p->B), dim3(256), smem, st, Q, K, scores, sel, status, p->H,
                                 p->Hkv, N, p->d, p->topk, p->sm_scale, p->eps));
@@ -308,7 +317,7 @@ static int launch_score_select(const still_params_t *p, long long N, long long T
 template <typename T>
 static int launch_npmap(const still_params_t *p, long long N, int heads, const T *X, const T *W,
                         const T *bias, T *phi, cudaStream_t st) {
-    const size_t smem = npmap_smem(p->d, p->d_f);
+    const size_t smem = npmap_smem(p->d, p->d_f, 256);
     const dim3 grid((unsigned)((N + 63) / 64), heads, p->B);
     auto launch = [&](auto kernel) -> int {
         STILL_CUDA(set_smem(kernel, smem));
@@ -321,6 +330,36 @@ static int launch_npmap(const still_params_t *p, long long N, int heads, const T
         case 64: return launch(npmap_kernel<T, 64>);
         default: return launch(npmap_kernel<T, 128>);
     }
+}
+
+// The score and both feature maps (the linear branch of the FMA kernels) in one launch, in wide blocks (see ScorePlan) and of
+// 128 (C = 32: 64) rows of a map: how many blocks these are.
+static long long front_blocks(const still_params_t *p, long long N) {
+    const long long rows = p->chunk == 32 ? 64 : 128, BH = (long long)p->B * p->H, BHkv = (long long)p->B * p->Hkv;
+    return BH * ((N + p->chunk - 1) / p->chunk) + (BH + BHkv) * ((N + rows - 1) / rows);
+}
+template <typename T>
+static int launch_score_npmap(const still_params_t *p, long long N, long long Tn, const T *Q, const T *K, const T *Wq, const T *bq, const T *Wk,
+                              const T *bk, T *phiQ, T *phiK, float *scores, int32_t *sel, int *status, cudaStream_t st) {
+    auto launch = [&](auto kernel, int threads, size_t score_smem) -> int {
+        const size_t smem = std::max(score_smem, npmap_smem(p->d, p->d_f, threads));
+        const long long row_blocks = (N + threads / 4 - 1) / (threads / 4), BH = (long long)p->B * p->H;
+        const FrontArgs<T> a{Q, K, Wq, bq, Wk, bk, phiQ, phiK, scores, sel, status, N, p->B, p->H, p->Hkv, p->d, p->topk,
+                             (int)(BH * Tn), (int)(BH * row_blocks), (int)row_blocks, p->sm_scale, p->eps};
+        STILL_CUDA(set_smem(kernel, smem));
+        STILL_CUDA(launch_dependent(kernel, dim3((unsigned)front_blocks(p, N)), dim3(threads), smem, st, a));
+        ++g_launches;
+        return STILL_OK;
+    };
+#define STILL_FRONT(NJ, DF) launch(score_npmap_kernel<T, NJ, DF>, ScorePlan<NJ, true>::kThreads, ScorePlan<NJ, true>::smem(p->d))
+#define STILL_FRONT_C(DF) (p->chunk == 32 ? STILL_FRONT(2, DF) : p->chunk == 64 ? STILL_FRONT(3, DF) : STILL_FRONT(5, DF))
+    switch (p->d_f) {
+        case 32: return STILL_FRONT_C(32);
+        case 64: return STILL_FRONT_C(64);
+        default: return STILL_FRONT_C(128);
+    }
+#undef STILL_FRONT_C
+#undef STILL_FRONT
 }
 
 template <typename T, int DP>
@@ -398,8 +437,12 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
         if (N > L.capacity) return STILL_ERR_STATE_FULL;
     }
 
-    // (1)+(2) Self-Saliency Score and per-chunk top-k.
-    if (w.tc)
+    // (1)+(2) Self-Saliency Score and per-chunk top-k; beside it the feature maps of the FMA kernels.
+    const bool maps_too = w.la && !w.tc && front_blocks(p, N) <= kFrontBlocks;
+    if (maps_too)
+        rc = launch_score_npmap<T>(p, N, w.T, Q, K, Wq, bq, Wk, bk, reinterpret_cast<T *>(ws + w.phiQ), reinterpret_cast<T *>(ws + w.phiK), sc,
+                                   sel, status, st);
+    else if (w.tc)
         rc = tc_score_select(p, N, Q, K, sc, sel, status, st, &g_launches);
     else
         rc = launch_score_select<T>(p, N, w.T, Q, K, sc, sel, status, st);
@@ -427,8 +470,10 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
             T *phiQ = reinterpret_cast<T *>(ws + w.phiQ);
             nla = reinterpret_cast<float *>(ws + w.nla);
             dla = reinterpret_cast<float *>(ws + w.dla);
-            if ((rc = launch_npmap<T>(p, N, p->H, Q, Wq, bq, phiQ, st)) != STILL_OK) return rc;
-            if ((rc = launch_npmap<T>(p, N, p->Hkv, K, Wk, bk, phiK, st)) != STILL_OK) return rc;
+            if (!maps_too) {
+                if ((rc = launch_npmap<T>(p, N, p->H, Q, Wq, bq, phiQ, st)) != STILL_OK) return rc;
+                if ((rc = launch_npmap<T>(p, N, p->Hkv, K, Wk, bk, phiK, st)) != STILL_OK) return rc;
+            }
             if ((rc = launch_la_scan<T>(p, N, w, ws, phiQ, phiK, V, G, sel, nla, dla, S_out, z_out, st)) != STILL_OK) return rc;
             if (w.tc && Y) {   // the tensor-core attention kernel takes the linear branch as bf16 parts
                 ypart = ws + w.ypart;

@@ -42,59 +42,56 @@ __device__ __forceinline__ void stage_wait() { asm volatile("cp.async.wait_group
 
 // ---------------------------------------------------------------------------
 // Self-Saliency Score (Sec. 3.1) + per-chunk top-k (Sec. 3.3, delayed selection).
-// One block of 256 threads per (chunk, head, batch).  The logits of 32 rows at a time
-// against the C + 32 keys their windows cover: a warp owns four rows, a lane NJ =
-// C / 32 + 1 keys of each.  Then a warp scores one token at a time: lane j holds the
-// logits of window slots j, j+32, ...; slot C-1 is the token itself (window_score).
-// (2000 tokens x 32 heads: 62 us, with one read per operand and multiply 117 us.)
+// One block per (chunk, head, batch): 8 (16) warps take the logits of 32 (64) rows at a time
+// against the keys their windows cover: a warp owns four rows of a group of 32, a lane NJ =
+// C / 32 + 1 keys of each.  Then the warp scores its tokens: lane j holds the logits of
+// window slots j, j+32, ...; slot C-1 is the token itself (window_score).
 // Selection: rank under (score descending, position ascending), NaN as -inf;
 // the k best are written in ascending position order, -1 padded.
 // ---------------------------------------------------------------------------
-inline size_t score_select_smem(int C, int d) {
-    return ((size_t)(2 * C + 32) * (d + 4) + (size_t)32 * (C + 33) + C) * 4 + (size_t)C * 4;
-}
-template <typename T, int NJ>
-__global__ void __launch_bounds__(256)
-score_select_kernel(const T *Q, const T *K, float *scores,
-                    int32_t *sel_idx, int *status, int H, int Hkv, long long N, int d, int lam, float scale, float eps) {
-    grid_dep_wait();
-    grid_dep_launch();
-    clear_status(status);
-    constexpr int C = 32 * (NJ - 1);
+template <int NJ, bool kWide>
+struct ScorePlan {
+    static constexpr int C = 32 * (NJ - 1), kThreads = kWide && C > 32 ? 512 : 256, kRows = kThreads / 8;   // rows of a pass
+    static size_t smem(int d) { return ((size_t)(2 * C + kRows) * (d + 4) + (size_t)kRows * (C + 33) + C) * 4 + (size_t)C * 4; }
+};
+template <typename T, int NJ, bool kWide>
+__device__ __forceinline__ void score_block(const T *Q, const T *K, float *scores, int32_t *sel_idx, int c, int h, int b, int H, int Hkv,
+                                            long long N, int d, int lam, float scale, float eps) {
+    using P = ScorePlan<NJ, kWide>;
+    constexpr int C = P::C, kThreads = P::kThreads, kRows = P::kRows;
     extern __shared__ __align__(16) float smem[];
-    const int c = blockIdx.x, h = blockIdx.y, b = blockIdx.z;
     const int kv = h / (H / Hkv), ds = d + 4;
-    const long long base = (long long)c * C;
-    const int Tn = gridDim.x;
+    const long long base = (long long)c * C, Tn = (N + C - 1) / C;
     float *kbuf = smem;                       // [2C][d + 4]: previous chunk, then this chunk
-    float *qbuf = kbuf + 2 * C * ds;          // [32][d + 4]
-    float *lg = qbuf + 32 * ds;               // [32][C + 33]
-    float *sc = lg + 32 * (C + 33);           // [C]
+    float *qbuf = kbuf + 2 * C * ds;          // [kRows][d + 4]
+    float *lg = qbuf + kRows * ds;            // [kRows][C + 33]
+    float *sc = lg + kRows * (C + 33);        // [C]
     int *flag = reinterpret_cast<int *>(sc + C);  // [C]
     const T *Qh = Q + ((long long)b * H + h) * N * d;
     const T *Kh = K + ((long long)b * Hkv + kv) * N * d;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, d4 = d >> 2;
 
-    for (int i = threadIdx.x; i < 2 * C * d4; i += 256) {
+    for (int i = threadIdx.x; i < 2 * C * d4; i += kThreads) {
         const int row = i / d4, col = (i - row * d4) * 4;
         const long long pos = base - C + row;
         const bool in = pos >= 0 && pos < N;
         stage4(kbuf + row * ds + col, Kh + (in ? pos * d : 0) + col, in);
     }
-    for (int r0 = 0; r0 < C; r0 += 32) {
-        if (base + r0 >= N) {   // (rows past the end of a ragged chunk)
-            if (threadIdx.x < 32) sc[r0 + threadIdx.x] = 0.f;
+    for (int p0 = 0; p0 < C; p0 += kRows) {
+        if (base + p0 >= N) {   // (rows past the end of a ragged chunk)
+            if (threadIdx.x < kRows) sc[p0 + threadIdx.x] = 0.f;
             continue;
         }
-        for (int i = threadIdx.x; i < 32 * d4; i += 256) {
+        for (int i = threadIdx.x; i < kRows * d4; i += kThreads) {
             const int row = i / d4, col = (i - row * d4) * 4;
-            const long long pos = base + r0 + row;
+            const long long pos = base + p0 + row;
             stage4(qbuf + row * ds + col, Qh + (pos < N ? pos * d : 0) + col, pos < N);
         }
         stage_commit();
         stage_wait();
         __syncthreads();
-        // rows r0 + 4 warp + i, keys (rows of kbuf) r0 + lane + 32 j
+        // rows p0 + 4 warp + i, keys (rows of kbuf) r0 + lane + 32 j, where r0 starts the group of 32 rows
+        const int r0 = p0 + (warp >> 3) * 32, in_group = 4 * (warp & 7);
         float2 acc[4][NJ];
 #pragma unroll
         for (int i = 0; i < 4; ++i)
@@ -121,9 +118,9 @@ score_select_kernel(const T *Q, const T *K, float *scores,
 #pragma unroll
             for (int j = 0; j < NJ; ++j) lg[(4 * warp + i) * (C + 33) + lane + 32 * j] = (acc[i][j].x + acc[i][j].y) * scale;
         __syncwarp();   // a warp scores the rows it has the logits of
-#pragma unroll 1
+#pragma unroll (kWide ? 4 : 1)   // (wide: four rows' chains of shuffles side by side)
         for (int i = 0; i < 4; ++i) {
-            const int r = r0 + 4 * warp + i;
+            const int r = r0 + in_group + i;
             if (base + r >= N) {
                 if (lane == 0) sc[r] = 0.f;
                 continue;
@@ -132,7 +129,7 @@ score_select_kernel(const T *Q, const T *K, float *scores,
 #pragma unroll
             for (int s = 0; s < 4; ++s) {   // slot lane + 32 s is row r + 1 + slot of kbuf
                 const int slot = lane + 32 * s;
-                l[s] = s < NJ - 1 && base + r - (C - 1) + slot >= 0 ? lg[(4 * warp + i) * (C + 33) + 4 * warp + i + 1 + slot] : -INFINITY;
+                l[s] = s < NJ - 1 && base + r - (C - 1) + slot >= 0 ? lg[(4 * warp + i) * (C + 33) + in_group + i + 1 + slot] : -INFINITY;
             }
             const float s = window_score(l, lane, NJ - 1, C, eps);
             if (lane == 0) {
@@ -148,31 +145,38 @@ score_select_kernel(const T *Q, const T *K, float *scores,
     const int n_c = (int)((N - base < C) ? (N - base) : C);
     select_chunk(sc, flag, n_c, C, lam, base, sel_idx + (((long long)b * H + h) * Tn + c) * lam);
 }
+template <typename T, int NJ>
+__global__ void __launch_bounds__(256)
+score_select_kernel(const T *Q, const T *K, float *scores,
+                    int32_t *sel_idx, int *status, int H, int Hkv, long long N, int d, int lam, float scale, float eps) {
+    grid_dep_wait();
+    grid_dep_launch();
+    clear_status(status);
+    score_block<T, NJ, false>(Q, K, scores, sel_idx, blockIdx.x, blockIdx.y, blockIdx.z, H, Hkv, N, d, lam, scale, eps);
+}
 
 // ---------------------------------------------------------------------------
 // Norm-Preserved Feature Map (Sec. 3.2, Eq. feature_map) of every row of X.
 // u = f(x) ||x|| / ||f(x)||, f(x) = xW + b; phi = [softmax(u), softmax(-u)].
-// grid (ceil(N/64), heads, B), 256 threads: 64 rows as a product with W; thread
-// (tr, tc) owns four rows and DF / 16 features, the sixteen threads of a row form
-// its norms, extrema and sums.  (2000 tokens x 40 heads: 38 us; a warp per row: 159 us.)
+// kThreads / 4 rows a block as a product with W; thread (tr, tc) owns four rows and
+// DF / 16 features, the sixteen threads of a row form its norms, extrema and sums.
+// (2000 tokens x 40 heads: 38 us; a warp per row: 159 us.)
 // ---------------------------------------------------------------------------
-inline size_t npmap_smem(int d, int df) { return ((size_t)d * df + (size_t)64 * (d + 4)) * 4; }
-template <typename T, int DF>
-__global__ void __launch_bounds__(256)
-npmap_kernel(const T *X, const T *W, const T *bias,
-             T *phi, int heads, long long N, int d) {
-    grid_dep_wait();
-    grid_dep_launch();
+inline size_t npmap_smem(int d, int df, int threads) { return ((size_t)d * df + (size_t)(threads / 4) * (d + 4)) * 4; }
+template <typename T, int DF, int kThreads>
+__device__ __forceinline__ void npmap_block(const T *X, const T *W, const T *bias, T *phi, uint32_t rb, int hd, int b, int heads, long long N,
+                                            int d) {
+    constexpr int kRows = kThreads / 4;
     constexpr int VC = DF >= 64 ? 4 : 2, NV = DF / (16 * VC);   // columns VC (tc + 16 j) .. + VC
     extern __shared__ __align__(16) float smem[];
     const int ds = d + 4, d4 = d >> 2;
     float *Ws = smem;             // [d][DF]
-    float *xs = Ws + d * DF;      // [64][d + 4]
-    const int hd = blockIdx.y, b = blockIdx.z, tid = threadIdx.x, tr = tid >> 4, tc = tid & 15;
+    float *xs = Ws + d * DF;      // [kRows][d + 4]
+    const int tid = threadIdx.x, tr = tid >> 4, tc = tid & 15;
     const T *Wh = W + (long long)hd * d * DF;
-    const long long row0 = (long long)blockIdx.x * 64, head0 = ((long long)b * heads + hd) * N;
-    for (int i = tid; i < d * DF / 4; i += 256) stage4(Ws + 4 * i, Wh + 4 * i, true);
-    for (int i = tid; i < 64 * d4; i += 256) {
+    const long long row0 = (long long)rb * kRows, head0 = ((long long)b * heads + hd) * N;
+    for (int i = tid; i < d * DF / 4; i += kThreads) stage4(Ws + 4 * i, Wh + 4 * i, true);
+    for (int i = tid; i < kRows * d4; i += kThreads) {
         const int r = i / d4, col = (i - r * d4) * 4;
         const bool in = row0 + r < N;
         stage4(xs + r * ds + col, X + (head0 + (in ? row0 + r : 0)) * d + col, in);
@@ -277,6 +281,52 @@ npmap_kernel(const T *X, const T *W, const T *bias,
             }
         }
     }
+}
+// grid (ceil(N/64), heads, B)
+template <typename T, int DF>
+__global__ void __launch_bounds__(256, DF == 128 ? 2 : 3)
+npmap_kernel(const T *X, const T *W, const T *bias,
+             T *phi, int heads, long long N, int d) {
+    grid_dep_wait();
+    grid_dep_launch();
+    npmap_block<T, DF, 256>(X, W, bias, phi, blockIdx.x, blockIdx.y, blockIdx.z, heads, N, d);
+}
+
+// ---------------------------------------------------------------------------
+// The score and the two feature maps, which need nothing of one another, in one launch: blocks of the score first, which take
+// longest, then those of Q, then of K.  For calls of few blocks (kFrontBlocks), which wait for one another's chains: 4 heads x
+// 512 tokens 15 + 7 + 7 us in three launches, 12 in one.
+// ---------------------------------------------------------------------------
+template <typename T>
+struct FrontArgs {
+    const T *Q, *K, *Wq, *bq, *Wk, *bk;
+    T *phiQ, *phiK;
+    float *scores;
+    int32_t *sel_idx;
+    int *status;
+    long long N;
+    int B, H, Hkv, d, lam, n_score, n_q, row_blocks;   // n_score, n_q: blocks of the score, of phi(Q)
+    float scale, eps;
+};
+template <typename T, int NJ, int DF>
+__global__ void __launch_bounds__(ScorePlan<NJ, true>::kThreads)
+score_npmap_kernel(const __grid_constant__ FrontArgs<T> a) {
+    grid_dep_wait();
+    grid_dep_launch();
+    clear_status(a.status);
+    using P = ScorePlan<NJ, true>;
+    int i = blockIdx.x;
+    if (i < a.n_score) {
+        const int Tn = (int)((a.N + P::C - 1) / P::C), bh = i / Tn;
+        score_block<T, NJ, true>(a.Q, a.K, a.scores, a.sel_idx, i - bh * Tn, bh % a.H, bh / a.H, a.H, a.Hkv, a.N, a.d, a.lam, a.scale, a.eps);
+        return;
+    }
+    i -= a.n_score;
+    const bool q = i < a.n_q;
+    if (!q) i -= a.n_q;
+    const int heads = q ? a.H : a.Hkv, unit = i / a.row_blocks;
+    npmap_block<T, DF, P::kThreads>(q ? a.Q : a.K, q ? a.Wq : a.Wk, q ? a.bq : a.bk, q ? a.phiQ : a.phiK, i - unit * a.row_blocks, unit % heads,
+                                 unit / heads, heads, a.N, a.d);
 }
 
 // ---------------------------------------------------------------------------

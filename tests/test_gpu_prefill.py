@@ -431,3 +431,31 @@ def test_a_refused_launch_does_not_fail_the_next_call():
     del x, w
     r = U.run_prefill(_small("t", "bf16", 1, 2, 1, 64, 200, 64, 16))
     assert bool(torch.isfinite(r["Y"].float()).all())
+
+
+@pytest.mark.parametrize("B,H,Hkv,d,df,C,k,N", [
+    (1, 4, 4, 64, 64, 64, 16, 512),      # one launch for score and maps, a chunk a segment
+    (1, 4, 2, 64, 32, 64, 16, 577),      # ... a last block of one row, narrow maps
+    (2, 2, 1, 128, 128, 64, 8, 190),     # head dim 128, a ragged chunk; three chunks: one pass of the scan
+    (1, 4, 2, 64, 64, 64, 16, 256),      # ... the last such size
+    (1, 4, 2, 64, 64, 64, 16, 257),      # five: three passes
+    (1, 2, 2, 128, 64, 128, 32, 700),    # wide blocks take half of a chunk of 128
+    (1, 3, 1, 64, 64, 32, 8, 333),       # chunks of 32: plain blocks
+    (1, 8, 2, 64, 64, 64, 16, 1030),     # 222 blocks of score and maps, the most that are one launch ...
+    (1, 8, 2, 64, 64, 64, 16, 1100),     # ... and more
+])
+def test_fp32_small_calls(B, H, Hkv, d, df, C, k, N):
+    w = _small("t", "fp32", B, H, Hkv, d, N, C, k)
+    p = still.StillParams(B, H, Hkv, d, C, k, torch.float32, d_f=df, sm_scale=w.sm_scale)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    g = torch.Generator(device="cuda").manual_seed(13)
+    Wq, Wk = (torch.randn(n, d, df, generator=g, device="cuda") * 0.05 for n in (H, Hkv))
+    bq, bk = (torch.randn(n, df, generator=g, device="cuda") * 0.05 for n in (H, Hkv))
+    ws = torch.full((still.workspace_bytes(p, N) + 4096,), 255, dtype=torch.uint8, device="cuda")   # (NaN wherever nothing is written)
+    Y, scores, sel = still.hybrid_attn_fwd(p, Q, K, V, Wq, Wk, bq=bq, bk=bk, workspace=ws[:-4096])
+    chunks, rows = -(-N // C), -(-N // (64 if C == 32 else 128))
+    one = B * H * chunks + B * (H + Hkv) * rows <= 222
+    assert still.last_launch_count() == (1 if one else 3) + (3 if chunks > 4 else 1) + 1 and bool((ws[-4096:] == 255).all())
+    heads = [(0, 0), (B - 1, H - 1)]
+    U.check_selection(scores, sel, C, k, heads)
+    U.check_outputs(w, Q, K, V, Wq, Wk, Y, scores, sel, heads, bq=bq, bk=bk, tol=1e-5)
