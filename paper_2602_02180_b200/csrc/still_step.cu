@@ -389,6 +389,11 @@ step_route_mma_kernel(__nv_bfloat16 *kc, __nv_bfloat16 *vc, float *score, int32_
     cp_async_wait<0>();
 }
 
+template <uint32_t kRegs>
+__device__ __forceinline__ void reg_inc_step() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(kRegs)); }
+template <uint32_t kRegs>
+__device__ __forceinline__ void reg_dec_step() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(kRegs)); }
+
 // Arguments of step_main_kernel / step_merge_kernel.  (Their contents come from kernels that may still run when a block
 // becomes resident, and must not be loaded ahead of the wait: see grid_dep_wait.)
 template <typename T>
@@ -435,15 +440,59 @@ __device__ __forceinline__ void load16(const float *p, float (&o)[4]) {
 }
 
 // Read-outs are worked on by groups of NW warps (1, 2 or all 8 of a block).
-template <int NW>
+template <int NW, bool kOthers = false>
 __device__ __forceinline__ void group_sync() {
     if constexpr (NW == 1) __syncwarp();
-    else if constexpr (NW == kStepWarps) __syncthreads();
+    else if constexpr (NW == kStepWarps) step_sync<kOthers>();
     else asm volatile("bar.sync %0, %1;" ::"r"(1 + (int)(threadIdx.x >> 5) / NW), "n"(NW * 32) : "memory");
 }
 // Shared memory of a group beside the rings, in floats: q [D], phi [2 d_f], sums of z [8], partial sums [NW][D].
 constexpr int kItemFloats = 128 + 256 + 8;
 constexpr int kItemSmem = kStepWarps * (kItemFloats + 128) * 4;
+
+// phi(q) [softmax(u), softmax(-u)] of a row by a warp, from its f + b: lane j holds features j, j + 32, ...  nx2: ||q||^2.  The
+// features are rounded to the storage type, as the prefill stores them.
+template <typename T>
+__device__ __forceinline__ void features_of_row(float (&f)[4], float nx2, int df, float *ph) {
+    const int lane = threadIdx.x & 31, jpl = df >> 5;
+    float nf2 = 0.f, umax = -INFINITY, umin = INFINITY;
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj) nf2 += f[jj] * f[jj];
+    nf2 = warp_sum(nf2);
+    const float ratio = sqrtf(nx2) / fmaxf(sqrtf(nf2), 1e-12f);
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj)
+        if (jj < jpl) {
+            f[jj] *= ratio;
+            umax = fmaxf(umax, f[jj]);
+            umin = fminf(umin, f[jj]);
+        }
+    umax = warp_max(umax);
+    umin = warp_min(umin);
+    float zp = 0.f, zn = 0.f, ep[4], en[4];
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj) {
+        ep[jj] = en[jj] = 0.f;
+        if (jj < jpl) {
+            ep[jj] = expf(f[jj] - umax);
+            en[jj] = expf(umin - f[jj]);
+            zp += ep[jj];
+            zn += en[jj];
+        }
+    }
+    zp = warp_sum(zp);
+    zn = warp_sum(zn);
+    if (ph == nullptr) return;
+#pragma unroll
+    for (int jj = 0; jj < 4; ++jj)
+        if (jj < jpl) {
+            T p0, p1;
+            st_f(&p0, ep[jj] / zp);
+            st_f(&p1, en[jj] / zn);
+            ph[lane + 32 * jj] = ld_f(&p0);
+            ph[df + lane + 32 * jj] = ld_f(&p1);
+        }
+}
 
 // Linear read-out of one (batch, query head): N_LA = phi(q) S, D_LA = phi(q) z into the head's last record.  S [2 d_f, D]
 // fp32 (128 KB at d = d_f = 128) and W_q are what it costs.  A warp takes a contiguous slice of either through its
@@ -511,8 +560,8 @@ __device__ __forceinline__ void linear_item(const StepArgs<T> &a, long long bh, 
         }
         group_sync<NW>();
     }
-    {   // every warp forms the norms and sums; features are rounded to the storage type, as the prefill stores them
-        float nx2 = 0.f, nf2 = 0.f, f[4], umax = -INFINITY, umin = INFINITY;
+    {   // every warp forms the norms and sums
+        float nx2 = 0.f, f[4];
         for (int i = lane; i < D; i += 32) nx2 += qs[i] * qs[i];
         nx2 = warp_sum(nx2);
 #pragma unroll
@@ -523,43 +572,8 @@ __device__ __forceinline__ void linear_item(const StepArgs<T> &a, long long bh, 
 #pragma unroll
                 for (int w = 0; w < NW; ++w) f[jj] += red[w * df + lane + 32 * jj];
             }
-            nf2 += f[jj] * f[jj];
         }
-        nf2 = warp_sum(nf2);
-        const float ratio = sqrtf(nx2) / fmaxf(sqrtf(nf2), 1e-12f);
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj)
-            if (jj < jpl) {
-                f[jj] *= ratio;
-                umax = fmaxf(umax, f[jj]);
-                umin = fminf(umin, f[jj]);
-            }
-        umax = warp_max(umax);
-        umin = warp_min(umin);
-        float zp = 0.f, zn = 0.f, ep[4], en[4];
-#pragma unroll
-        for (int jj = 0; jj < 4; ++jj) {
-            ep[jj] = en[jj] = 0.f;
-            if (jj < jpl) {
-                ep[jj] = expf(f[jj] - umax);
-                en[jj] = expf(umin - f[jj]);
-                zp += ep[jj];
-                zn += en[jj];
-            }
-        }
-        zp = warp_sum(zp);
-        zn = warp_sum(zn);
-        if (warp == 0) {
-#pragma unroll
-            for (int jj = 0; jj < 4; ++jj)
-                if (jj < jpl) {
-                    T p0, p1;
-                    st_f(&p0, ep[jj] / zp);
-                    st_f(&p1, en[jj] / zn);
-                    ph[lane + 32 * jj] = ld_f(&p0);
-                    ph[df + lane + 32 * jj] = ld_f(&p1);
-                }
-        }
+        features_of_row<T>(f, nx2, df, warp == 0 ? ph : nullptr);
         group_sync<NW>();
     }
     float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
@@ -611,35 +625,212 @@ __device__ __forceinline__ void linear_item(const StepArgs<T> &a, long long bh, 
     group_sync<NW>();
 }
 
-// This block's share of the read-outs, by groups of NW warps.
+// This block's share of the read-outs, by groups of NW warps, from the first-th of the block on: its j-th is item j * blocks +
+// (its place among the blocks), and belongs to group j % groups.
 template <typename T, int D, int NW, class Ring>
-__device__ __forceinline__ void work_on_items(const StepArgs<T> &a, uint8_t *smem) {
+__device__ __forceinline__ void work_on_items(const StepArgs<T> &a, uint8_t *smem, int first) {
     constexpr int kGroups = kStepWarps / NW;
     const int warp = threadIdx.x >> 5, group = warp / NW, blocks = (int)gridDim.x - a.first_item_block;
-    const long long worker = (int)blockIdx.x - a.first_item_block + (long long)group * blocks, workers = (long long)blocks * kGroups;
     float *mine = reinterpret_cast<float *>(smem + Ring::kTotal) + group * (kItemFloats + NW * 128);
-    for (long long i = worker; i < a.n_items; i += workers) linear_item<T, D, NW, Ring>(a, i, smem + warp * Ring::kWarp, mine);
+    for (int j = group; ; j += kGroups) {
+        const long long i = (int)blockIdx.x - a.first_item_block + (long long)j * blocks;
+        if (i >= a.n_items) break;
+        if (j >= first) linear_item<T, D, NW, Ring>(a, i, smem + warp * Ring::kWarp, mine);
+    }
 }
+
+// ---- bf16: the features of the block's first read-outs are formed by four warps of their own while the eight others work on the
+// cache, so that these have nothing left to do for a read-out but to stream S.  (As a chain of q, W_q, phi(q) and S behind the
+// cache pass a read-out took 7 of its 21 us before S came in at the rate of HBM.  us a step, then and now, d = 128, a quarter
+// kept: 4 sequences of 32 heads x 2000 tokens 18.2 and 17.1, 8 x 4000 35.5 and 33.5, 32 x 8192 capped at 448 71.9 and 69.1; 64 of 16
+// heads x 3000 82.7 and 81.4.)
+constexpr int kMapWarps = 4, kMaxPhi = 14;   // features kept per block (a KB each beside the rings); read-outs beyond: work_on_items
+// Shared memory behind the rings, in bytes: read-outs (kItemSmem), features, the map warps' q.
+constexpr int kPhiAt = kItemSmem, kMapAt = kPhiAt + kMaxPhi * 256 * 4, kBesideSmem = kMapAt + kMapWarps * 128 * 4;
+constexpr int kPhiBarrier = 15;   // (barriers 1 to 8: see group_sync)
+
+// Features of the block's first read-outs, and their D_LA, by the map warps: f is the sum over rows in the order of linear_item
+// by one warp.
+template <int D>
+__device__ __forceinline__ void map_items(const StepArgs<__nv_bfloat16> &a, uint8_t *beside) {
+    using bf = __nv_bfloat16;
+    const int mw = (threadIdx.x >> 5) - kStepWarps, lane = threadIdx.x & 31, df = a.df, dp = 2 * df, blocks = gridDim.x;
+    float *qs = reinterpret_cast<float *>(beside + kMapAt) + mw * 128;
+    const int lpr = df / 8, rpl = 32 / lpr, cg = lane % lpr;
+    for (int j = mw; j < kMaxPhi; j += kMapWarps) {
+        const long long bh = (int)blockIdx.x + (long long)j * blocks;
+        if (bh >= a.n_items) break;
+        const int h = (int)(bh % a.H);
+        float *ph = reinterpret_cast<float *>(beside + kPhiAt) + j * 256;
+        const bf *W = a.Wq + (long long)h * D * df + (lane / lpr) * df + cg * 8;
+        float nx2 = 0.f;
+        for (int i = lane; i < D; i += 32) {
+            const float x = ld_f(a.q + bh * D + i);
+            qs[i] = x;
+            nx2 += x * x;
+        }
+        nx2 = warp_sum(nx2);
+        float zv[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) zv[i] = lane + 32 * i < dp ? a.z[bh * dp + lane + 32 * i] : 0.f;
+        float acc[8];
+#pragma unroll
+        for (int e = 0; e < 8; ++e) acc[e] = 0.f;
+        constexpr int kBatch = 8;   // rows of W_q requested together
+        for (int r0 = 0; r0 < D; r0 += kBatch * rpl) {
+            uint4 raw[kBatch];
+#pragma unroll
+            for (int k = 0; k < kBatch; ++k) raw[k] = *reinterpret_cast<const uint4 *>(W + (long long)(r0 + k * rpl) * df);
+#pragma unroll
+            for (int k = 0; k < kBatch; ++k) {
+                const float x = qs[r0 + k * rpl + lane / lpr];
+                const uint32_t w4[4] = {raw[k].x, raw[k].y, raw[k].z, raw[k].w};
+#pragma unroll
+                for (int e = 0; e < 4; ++e) {
+                    acc[2 * e] = fmaf(x, __uint_as_float(w4[e] << 16), acc[2 * e]);
+                    acc[2 * e + 1] = fmaf(x, __uint_as_float(w4[e] & 0xffff0000u), acc[2 * e + 1]);
+                }
+            }
+        }
+        for (int o = lpr; o < 32; o <<= 1) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) acc[e] += __shfl_xor_sync(0xffffffffu, acc[e], o);
+        }
+        __syncwarp();   // (every lane has read q)
+        if (lane < lpr) {
+#pragma unroll
+            for (int e = 0; e < 8; ++e) qs[cg * 8 + e] = acc[e];
+        }
+        __syncwarp();
+        float f[4];
+#pragma unroll
+        for (int jj = 0; jj < 4; ++jj) f[jj] = 32 * jj < df ? (a.bq ? ld_f(a.bq + (long long)h * df + lane + 32 * jj) : 0.f) + qs[lane + 32 * jj] : 0.f;
+        features_of_row<bf>(f, nx2, df, ph);
+        __syncwarp();
+        float dz = 0.f;
+#pragma unroll
+        for (int i = 0; i < 8; ++i)
+            if (lane + 32 * i < dp) dz = fmaf(ph[lane + 32 * i], zv[i], dz);
+        dz = warp_sum(dz);
+        if (lane == 0) a.part[(bh * kRecords + kLinRecord) * (D + 2) + 1] = dz;
+    }
+}
+
+// The streams of S of the block's first read-outs, by groups of a.item_warps warps: request() is called when the warp's ring is
+// free, run() when the features are there.
+template <typename T, int D, class Ring>
+struct StateStream {
+    static constexpr int kStage = Ring::kStage, kStages = Ring::kStages, LPR = D / 4, RPW = 32 / LPR;
+    const StepArgs<T> &a;
+    uint8_t *ring;
+    int group, in_group, groups;   // this warp's group, its place there; groups
+    int s_bytes, n_s, total;       // this warp's slice of S, its stages; stages in all
+    int requested = 0;
+    __device__ __forceinline__ StateStream(const StepArgs<T> &args, uint8_t *smem)
+        : a(args), ring(smem + (threadIdx.x >> 5) * Ring::kWarp) {
+        group = (threadIdx.x >> 5) / a.item_warps;
+        in_group = (threadIdx.x >> 5) % a.item_warps;
+        groups = kStepWarps / a.item_warps;
+        s_bytes = 2 * a.df * D * 4 / a.item_warps;
+        n_s = (s_bytes + kStage - 1) / kStage;
+        const int mine = (int)min((long long)kMaxPhi, (a.n_items - (int)blockIdx.x + (long long)gridDim.x - 1) / gridDim.x);   // of the block
+        total = max(0, (mine - group + groups - 1) / groups) * n_s;
+    }
+    __device__ __forceinline__ long long item(int k) const {   // the group's k-th
+        return (int)blockIdx.x + (long long)(group + k * groups) * gridDim.x;
+    }
+    __device__ __forceinline__ void issue() {
+        if (requested < total) {
+            const int k = requested / n_s, off = (requested - k * n_s) * kStage, bytes = min(kStage, s_bytes - off);
+            const char *src = reinterpret_cast<const char *>(a.S + item(k) * 2 * a.df * D) + (long long)in_group * s_bytes + off;
+            uint8_t *dst = ring + requested % kStages * kStage;
+#pragma unroll 4
+            for (int i = (threadIdx.x & 31) * 16; i < bytes; i += 512) cp_async16(dst + i, src + i, true);
+        }
+        ++requested;
+        cp_async_commit();
+    }
+    __device__ __forceinline__ void request() {
+#pragma unroll
+        for (int c = 0; c < kStages; ++c) issue();
+    }
+    template <int NW>
+    __device__ __forceinline__ void run(uint8_t *beside) {
+        const int warp = in_group, lane = threadIdx.x & 31, tid = warp * 32 + lane;
+        float *red = reinterpret_cast<float *>(beside) + group * NW * 128;
+        for (int k = 0, c = 0; c < total; ++k) {
+            const float *ph = reinterpret_cast<const float *>(beside + kPhiAt) + (group + k * groups) * 256 + warp * s_bytes / (D * 4) + lane / LPR;
+            float4 acc = make_float4(0.f, 0.f, 0.f, 0.f);
+            for (int off = 0; off < s_bytes; off += kStage, ++c) {
+                cp_async_wait<kStages - 1>();
+                __syncwarp();
+                const int rows = min(kStage, s_bytes - off) / (D * 4);
+                const float *sr = reinterpret_cast<const float *>(ring + c % kStages * kStage) + lane * 4;
+                const float *pr = ph + off / (D * 4);
+#pragma unroll 4
+                for (int r = 0; r < rows; r += RPW) {
+                    const float4 x = *reinterpret_cast<const float4 *>(sr + r * D);
+                    const float p = pr[r];
+                    acc.x = fmaf(p, x.x, acc.x);
+                    acc.y = fmaf(p, x.y, acc.y);
+                    acc.z = fmaf(p, x.z, acc.z);
+                    acc.w = fmaf(p, x.w, acc.w);
+                }
+                __syncwarp();
+                issue();
+            }
+            if constexpr (RPW == 2) {
+                acc.x += __shfl_xor_sync(0xffffffffu, acc.x, 16);
+                acc.y += __shfl_xor_sync(0xffffffffu, acc.y, 16);
+                acc.z += __shfl_xor_sync(0xffffffffu, acc.z, 16);
+                acc.w += __shfl_xor_sync(0xffffffffu, acc.w, 16);
+            }
+            float *rec = a.part + (item(k) * kRecords + kLinRecord) * (D + 2) + 2;
+            if constexpr (NW == 1) {
+                if (lane < LPR) {
+                    rec[lane * 4] = acc.x;       // (records are not 16-byte aligned)
+                    rec[lane * 4 + 1] = acc.y;
+                    rec[lane * 4 + 2] = acc.z;
+                    rec[lane * 4 + 3] = acc.w;
+                }
+            } else {
+                if (lane < LPR) *reinterpret_cast<float4 *>(red + warp * D + lane * 4) = acc;
+                group_sync<NW, true>();
+                for (int i = tid; i < D; i += NW * 32) {
+                    float n = 0.f;
+#pragma unroll
+                    for (int w = 0; w < NW; ++w) n += red[w * D + i];
+                    rec[i] = n;
+                }
+                group_sync<NW, true>();
+            }
+        }
+        cp_async_wait<0>();
+    }
+};
 
 // Rings of the cache pass.
 template <typename T, int D>
 struct StepRing : AttendPlan<D> {};
 template <int D>
 struct StepRing<float, D> : AttendPlanF32<D> {};
-// Shared memory of step_main_kernel: the rings, and the read-outs' staging beside them.
-template <typename T, int D>
+// kMaps: with the map warps.
+template <bool kMaps>
+constexpr int kMainThreads = kStepThreads + (kMaps ? kMapWarps * 32 : 0);
+// Shared memory of step_main_kernel: the rings, and what lies beside them.
+template <typename T, int D, bool kMaps>
 constexpr int step_main_smem() {
-    return StepRing<T, D>::kTotal + kItemSmem;
+    return StepRing<T, D>::kTotal + (kMaps ? kBesideSmem : kItemSmem);
 }
-static_assert(step_main_smem<__nv_bfloat16, 128>() <= 232448 && step_main_smem<float, 128>() <= 232448, "shared memory of a step");
+static_assert(step_main_smem<__nv_bfloat16, 128, true>() <= 232448 && step_main_smem<float, 128, false>() <= 232448, "shared memory of a step");
 
 // One block per SM.  At large batches the bytes of K, V and S bound it (us a step, the merge included; in brackets the form
 // with a launch each for append and score, routing, the cache pass in equal splits per group and the merge with its
 // read-out, timed in turn on one box: B = 64, 32K prefix, every token 1302 (1657), 6.6 TB/s; B = 16, 16K, a quarter kept
 // 148 (307); B = 32, 8K, capped at 448: 72 (203)), at one sequence the latency of a block's chain (one user, 2K prefix:
 // 10.5 (72), of which the host needs 10).
-template <typename T, int D, int NH>
-__global__ void __launch_bounds__(kStepThreads, 1)
+template <typename T, int D, int NH, bool kMaps>
+__global__ void __launch_bounds__(kMaps ? 512 : kStepThreads, 1)   // (512: 128 registers a thread, see below)
 step_main_kernel(const __grid_constant__ StepArgs<T> a) {
     extern __shared__ __align__(128) uint8_t step_smem[];
     grid_dep_wait();
@@ -651,7 +842,23 @@ step_main_kernel(const __grid_constant__ StepArgs<T> a) {
             return;
         }
     }
+    using Ring = StepRing<T, D>;
+    uint8_t *beside = step_smem + Ring::kTotal;
+    if constexpr (kMaps) {
+        if (threadIdx.x >= kStepThreads) {
+            reg_dec_step<64>();
+            map_items<D>(a, beside);
+            asm volatile("bar.arrive %0, %1;" ::"n"(kPhiBarrier), "n"(kMainThreads<kMaps>) : "memory");
+            return;
+        }
+        // Per scheduler 2 x 160 + 64 registers, of the 3 x 128 that the block was launched with.  (The quarter of the register file
+        // that is left over is what lets the blocks of the next kernel come in beside this one: with all of it taken a step was 4
+        // us longer at 4 sequences, 12 at 32.)
+        reg_inc_step<160>();
+    }
     const int lo = min((int)blockIdx.x * a.per, a.total), hi = min(lo + a.per, a.total), rep = a.H / a.Hkv;
+    [[maybe_unused]] StateStream<T, D, Ring> states(a, step_smem);
+    constexpr bool kBeside = kMaps && NH == 4;   // (the sums of eight heads do not fit beside the rings)
     for (int x = lo; x < hi;) {
         const int u = x / a.unit_len;
         const int tile_lo = x - u * a.unit_len, tile_hi = min(a.tiles, hi - u * a.unit_len);
@@ -667,17 +874,29 @@ step_main_kernel(const __grid_constant__ StepArgs<T> a) {
         const uint32_t *mask = a.sel_mask + bh * v.n_chunk_cap * (v.C / 32);
         float *part = a.part + (bh * kRecords + slot) * (D + 2), *logits = a.part + (bh * kRecords + kLogitRecord) * (D + 2);
         if constexpr (sizeof(T) == 2)
-            attend_segment<D, NH>(v, kh, vh, a.k + row * D, a.v + row * D, a.q + bh * D, mask, tile_lo, tile_hi, step_smem, part,
-                                  logits, kRecords * (D + 2));
+            attend_segment<D, NH, kMaps, kBeside>(v, kh, vh, a.k + row * D, a.v + row * D, a.q + bh * D, mask, tile_lo, tile_hi, step_smem,
+                                           reinterpret_cast<float *>(kBeside ? beside : step_smem), part, logits, kRecords * (D + 2), [&] {
+                                               if constexpr (kBeside) {
+                                                   if (x >= hi) states.request();   // (the block's last segment)
+                                               }
+                                           });
         else
             attend_segment_f32<D>(v, kh, vh, a.k + row * D, a.v + row * D, a.q + bh * D, mask, tile_lo, tile_hi,
                                   step_smem, part, logits, kRecords * (D + 2));
     }
+    if constexpr (kMaps) {
+        if (states.requested == 0) states.request();
+        asm volatile("bar.sync %0, %1;" ::"n"(kPhiBarrier), "n"(kMainThreads<kMaps>) : "memory");
+        if (a.item_warps == 1) states.template run<1>(beside);
+        else if (a.item_warps == 2) states.template run<2>(beside);
+        else states.template run<kStepWarps>(beside);
+    }
     if ((int)blockIdx.x < a.first_item_block) return;
-    using Ring = StepRing<T, D>;
-    if (a.item_warps == 1) work_on_items<T, D, 1, Ring>(a, step_smem);
-    else if (a.item_warps == 2) work_on_items<T, D, 2, Ring>(a, step_smem);
-    else work_on_items<T, D, kStepWarps, Ring>(a, step_smem);
+    // (beyond kMaxPhi a block only has more where a read-out is one warp's: the groups' places beside the rings do not meet)
+    const int first = kMaps ? kMaxPhi : 0;
+    if (a.item_warps == 1) work_on_items<T, D, 1, Ring>(a, step_smem, first);
+    else if (a.item_warps == 2) work_on_items<T, D, 2, Ring>(a, step_smem, first);
+    else work_on_items<T, D, kStepWarps, Ring>(a, step_smem, first);
 }
 
 // grid (H, B), D + 64 threads: an output column each, then a warp that scores the new token and one that appends its K / V
@@ -796,13 +1015,28 @@ static int launch_route(const still_params_t *p, const StepArgs<T> &a, int32_t *
     return STILL_OK;
 }
 
+constexpr int kMapTiles = 512;   // tiles of a block
 template <typename T, int D, int NH>
 static int launch_main(const StepArgs<T> &a, unsigned grid, cudaStream_t st, int *launches) {
-    constexpr int kSmem = step_main_smem<T, D>();
-    STILL_CUDA(ensure_dynamic_smem((const void *)step_main_kernel<T, D, NH>, kSmem));
-    profile_mark_begin(st);
-    STILL_CUDA(launch_dependent(step_main_kernel<T, D, NH>, dim3(grid), dim3(kStepThreads), kSmem, st, a));
-    profile_mark_end(st);
+    auto launch = [&](auto maps) -> int {
+        constexpr bool kMaps = decltype(maps)::value;
+        constexpr int kSmem = step_main_smem<T, D, kMaps>();
+        STILL_CUDA(ensure_dynamic_smem((const void *)step_main_kernel<T, D, NH, kMaps>, kSmem));
+        profile_mark_begin(st);
+        STILL_CUDA(launch_dependent(step_main_kernel<T, D, NH, kMaps>, dim3(grid), dim3(kMainThreads<kMaps>), kSmem, st, a));
+        profile_mark_end(st);
+        return STILL_OK;
+    };
+    int rc;
+    // Map warps where the blocks have read-outs behind their tiles (bf16, up to eight heads a KV group: with 16 the cache pass
+    // needs the registers) and these are not many: what the read-outs gain is a few us whatever the tiles, and the cache pass, in
+    // fewer registers and beside the loads of W_q, takes up to 2 % longer.  (us a
+    // step without and with them: 325 tiles a block 82.7 and 81.4, 865 tiles, 16 sequences x 16000 tokens, 141.2 and 142.5.)
+    if constexpr (sizeof(T) == 2 && NH <= 8)
+        rc = a.n_items > 0 && a.first_item_block == 0 && a.per <= kMapTiles ? launch(std::true_type{}) : launch(std::false_type{});
+    else
+        rc = launch(std::false_type{});
+    if (rc != STILL_OK) return rc;
     STILL_CUDA(launch_dependent(step_merge_kernel<T, D>, dim3(a.H, a.B), dim3(D + 64), 0, st, a));
     *launches += 2;
     return STILL_OK;

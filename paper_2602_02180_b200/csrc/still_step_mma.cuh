@@ -100,17 +100,26 @@ struct AttendPlan {
     static constexpr int kTotal = kStepWarps * kWarp;
 };
 
-// Tiles [tile_lo, tile_hi) of one KV head by one block of 8 warps.  kh, vh: the head's rows; k_new, v_new: the new
+// The barrier of the eight warps of the cache pass; kOthers: the block has other warps too.
+template <bool kOthers>
+__device__ __forceinline__ void step_sync() {
+    if constexpr (kOthers) asm volatile("bar.sync 0, %0;" ::"n"(kStepWarps * 32) : "memory");
+    else __syncthreads();
+}
+
+// Tiles [tile_lo, tile_hi) of one KV head by 8 warps.  kh, vh: the head's rows; k_new, v_new: the new
 // token's (position t is read from the call's inputs, not from the row that another block is writing); qh: the
 // group's queries; mask: sel_mask of the group's first head.  Leaves one record per head (maximum in natural-log
 // units, sum, numerator [D]) at part + head * part_stride, and the new token's logits against the last C positions,
 // oldest first, at logits + head * part_stride.  NH: room for heads, 4, 8 or 16 (tiles of 8 columns; with 4 the second
-// half of the tile repeats the heads and takes the second part of their weights).
-template <int D, int NH>
+// half of the tile repeats the heads and takes the second part of their weights).  The warps' sums are merged through
+// `staging`: the rings, or (kBeside) a place of its own, so that what after() requests into the rings is on its way meanwhile.
+template <int D, int NH, bool kOthers, bool kBeside, class After>
 __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_bfloat16 *kh, const __nv_bfloat16 *vh,
                                                const __nv_bfloat16 *k_new, const __nv_bfloat16 *v_new,
                                                const __nv_bfloat16 *qh, const uint32_t *mask, int tile_lo, int tile_hi,
-                                               uint8_t *smem, float *part, float *logits, long long part_stride) {
+                                               uint8_t *smem, float *staging, float *part, float *logits, long long part_stride,
+                                               After after) {
     using P = AttendPlan<D>;
     constexpr int NT = NH == 16 ? 2 : 1;
     constexpr bool kRepeat = NH == 4;
@@ -312,11 +321,15 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
         __syncwarp();   // the stage may be overwritten
         if (++stage == P::kStages) stage = 0;
     }
-    cp_async_wait<0>();
-    __syncthreads();
+    if constexpr (kBeside) {
+        after();
+    } else {
+        cp_async_wait<0>();
+        step_sync<kOthers>();
+    }
 
     // merge the eight warps: [8 warps][rep][D + 2] in shared memory
-    float *mg = reinterpret_cast<float *>(smem);
+    float *mg = staging;
     constexpr int kStride = D + 2;
     const int rep = v.rep;
     if constexpr (kRepeat) {   // both parts of a head's sums
@@ -348,7 +361,7 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
             }
         }
     }
-    __syncthreads();
+    step_sync<kOthers>();
     for (int idx = threadIdx.x; idx < rep * kStride; idx += kStepWarps * 32) {
         const int h = idx / kStride, col = idx % kStride;
         float mw[kStepWarps], M = -INFINITY;
@@ -367,7 +380,7 @@ __device__ __forceinline__ void attend_segment(const AttendView &v, const __nv_b
         }
         part[h * part_stride + col] = acc;
     }
-    __syncthreads();   // the staging space is the next segment's ring
+    step_sync<kOthers>();   // the staging space is the next segment's
 }
 
 }  // namespace still

@@ -352,3 +352,37 @@ def test_decode_with_the_most_partials_a_head_can_have():
     # the scratch has room for
     y, exact, _ = _dense_steps(1, 4, 1, 64, 38016, 4)
     assert (y != exact.to(torch.bfloat16)).double().mean().item() <= 0.02
+
+
+@pytest.mark.parametrize("B,H,Hkv,d,df,C,k,budget", [
+    (5, 16, 4, 128, 128, 64, 16, 0),     # 80 read-outs beside the cache pass: one a block, by its eight warps
+    (9, 20, 4, 64, 32, 64, 32, 0),       # 180, two warps each, narrow maps; five heads a group
+    (9, 20, 4, 128, 64, 64, 32, 64),     # ... tokens that leave a capped cache
+    (7, 32, 4, 128, 64, 32, 8, 0),       # 224, eight heads a group
+    (20, 32, 8, 64, 64, 64, 16, 0),      # 640, a warp each
+    (66, 32, 8, 64, 64, 32, 8, 0),       # 2112: more for some blocks than they keep features for
+    (5, 32, 2, 64, 64, 64, 16, 0),       # sixteen heads a group: no warps for the features
+])
+def test_decode_batch_gives_each_sequence_its_own(B, H, Hkv, d, df, C, k, budget):
+    # The read-outs of a batch (features by warps of their own) against those of its sequences alone, and the rounding between:
+    # y differs by at most two of its roundings to bf16.
+    n0, steps = 2 * C + 9, 3
+    w = synth.Workload("t", B, H, Hkv, d, n0 + steps, C, k, "bf16", "iid", 21)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    g = torch.Generator(device="cuda").manual_seed(10)
+    mk = lambda *s: (torch.randn(*s, generator=g, device="cuda") * 0.05).bfloat16()  # noqa: E731
+    Wq, Wk, bq, bk, G = mk(H, d, df), mk(Hkv, d, df), mk(H, df), mk(Hkv, df), torch.rand(B, H, w.N, d, generator=g, device="cuda").bfloat16()
+
+    def run(bs):
+        p = still.StillParams(len(bs), H, Hkv, d, C, k, torch.bfloat16, d_f=df, sm_scale=w.sm_scale, max_salient=budget)
+        x = [t[bs] for t in (Q, K, V, G)]
+        state = torch.zeros(still.state_bytes(p, w.N), dtype=torch.uint8, device="cuda")
+        pre = [t[:, :, :n0].contiguous() for t in x]
+        still.hybrid_attn_fwd(p, *pre[:3], Wq, Wk, G=pre[3], bq=bq, bk=bk, state=state, state_max_tokens=w.N)
+        return torch.stack([still.hybrid_attn_step(p, state, w.N, t, *(y[:, :, t].contiguous() for y in x[:3]), Wq, Wk,
+                                                   g=x[3][:, :, t].contiguous(), bq=bq, bk=bk) for t in range(n0, w.N)], 2).float()
+
+    Y = run(list(range(B)))
+    for b in {0, B // 2, B - 1}:
+        alone = run([b])[0]
+        assert bool(((Y[b] - alone).abs() <= 2 ** -7 * alone.abs() + 1e-4).all())
