@@ -289,8 +289,10 @@ npmap_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
 // -1 entries and the rows of the padding (block T) are zero.  NULL outputs are not made.  Bound by the bytes written
 // and the rows read: 32 heads x 131072 tokens, d = 128, 32 of 128 selected, with phi_sel: three kernels that each
 // gathered for themselves (and one that summed a row after the other) took 1023 us, this one 305.
-template <int D, int DF>
-__global__ void __launch_bounds__(256, D == 128 ? 4 : 5)
+// kFew: at d = 64 up to 16 tokens of a chunk are one row a thread; eight blocks an SM instead of five keep as many rows in flight
+// (128 heads x 4096 tokens, 16 of 64: 29.7 us and 23.7; with 32 of 64 a thread's two rows one after the other 6 us more).
+template <int D, int DF, bool kFew>
+__global__ void __launch_bounds__(256, D == 128 ? 4 : kFew ? 8 : 5)
 gather_kernel(const __nv_bfloat16 *K, const __nv_bfloat16 *V, const __nv_bfloat16 *phiK,
               const int32_t *sel_idx, __nv_bfloat16 *Ksel, __nv_bfloat16 *Vsel,
               __nv_bfloat16 *phi_sel, float *selsum, int H, int Hkv, long long N, int lam,
@@ -321,7 +323,7 @@ gather_kernel(const __nv_bfloat16 *K, const __nv_bfloat16 *V, const __nv_bfloat1
     const __nv_bfloat16 *src = which ? V : K;
     __nv_bfloat16 *dst = which ? Vsel : Ksel;
     const bool with_phi = phi_sel != nullptr || c < n_routed;
-    constexpr int kStep = 8 * (kPer / 2), kPhiStep = 8 * kPhiPer, kBatch = D == 128 ? 4 : 2;
+    constexpr int kStep = 8 * (kPer / 2), kPhiStep = 8 * kPhiPer, kBatch = D == 128 ? 4 : kFew ? 1 : 2;
     float acc[8];
 #pragma unroll
     for (int e = 0; e < 8; ++e) acc[e] = 0.f;
@@ -1202,7 +1204,7 @@ int launch_gather(const still_params_t *p, long long N, const void *K, const voi
     using bf = __nv_bfloat16;
     const long long Tn = (N + p->chunk - 1) / p->chunk;
     ++*launches;
-    return launch_dependent(gather_kernel<D, DF>, dim3((unsigned)(Tn + 1), (unsigned)(p->B * p->H)), dim3(256), 0, st, (const bf *)K,
+    return launch_dependent(D == 64 && p->topk <= 16 ? gather_kernel<D, DF, D == 64> : gather_kernel<D, DF, false>, dim3((unsigned)(Tn + 1), (unsigned)(p->B * p->H)), dim3(256), 0, st, (const bf *)K,
                             (const bf *)V, (const bf *)phiK, sel_idx, (bf *)k_sel, (bf *)v_sel, (bf *)phiK_sel, selsum, p->H, p->Hkv,
                             N, p->topk, sel_rows, n_routed) == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
 }
