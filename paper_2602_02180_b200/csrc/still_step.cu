@@ -498,8 +498,10 @@ __device__ __forceinline__ void features_of_row(float (&f)[4], float nx2, int df
 // fp32 (128 KB at d = d_f = 128) and W_q are what it costs.  A warp takes a contiguous slice of either through its
 // cp.async ring, first W_q, then S, so that the whole ring is in flight also while phi(q) is formed.  (With the rows
 // requested into registers instead, a warp had too little in flight: 512 read-outs took 60 us, 1.1 TB/s.)
-template <typename T, int D, int NW, class Ring>
-__device__ __forceinline__ void linear_item(const StepArgs<T> &a, long long bh, uint8_t *ring, float *smem) {
+// Of a read-out apart (kApart), which a step of few sequences waits for, state_ok() is asked before anything of the state is read,
+// but behind the requests for q and W_q.  (One user, 2000 tokens: 10.5 us a step with the header first, 10.0 like this.)
+template <typename T, int D, int NW, bool kApart, class Ring, class StateOk>
+__device__ __forceinline__ void linear_item(const StepArgs<T> &a, long long bh, uint8_t *ring, float *smem, StateOk state_ok) {
     constexpr int V = 16 / (int)sizeof(T);
     constexpr int LPR = D / 4, RPW = 32 / LPR;        // lanes per row of S (16 bytes each), rows per warp and load
     constexpr int kStage = Ring::kStage, kStages = Ring::kStages;
@@ -521,13 +523,31 @@ __device__ __forceinline__ void linear_item(const StepArgs<T> &a, long long bh, 
         }
         cp_async_commit();
     };
+    if constexpr (kApart) {
+        const int early = min(n_w, kStages);
+        for (int c = 0; c < early; ++c) issue(c);
+        for (int i = tid; i < D; i += NW * 32) qs[i] = ld_f(a.q + bh * D + i);
+        if (!state_ok()) {
+            cp_async_wait<0>();
+            return;
+        }
+        for (int c = early; c < kStages; ++c) issue(c);
+    } else {
 #pragma unroll
-    for (int c = 0; c < kStages; ++c) issue(c);
-    for (int i = tid; i < D; i += NW * 32) qs[i] = ld_f(a.q + bh * D + i);
+        for (int c = 0; c < kStages; ++c) issue(c);
+        for (int i = tid; i < D; i += NW * 32) qs[i] = ld_f(a.q + bh * D + i);
+    }
     float dz = 0.f, zv[8];
 #pragma unroll
     for (int i = 0; i < 8 / NW + (8 % NW ? 1 : 0); ++i) zv[i] = tid + i * NW * 32 < dp ? a.z[bh * dp + tid + i * NW * 32] : 0.f;
     group_sync<NW>();
+    auto norm2_of_q = [&] {
+        float x2 = 0.f;
+        for (int i = lane; i < D; i += 32) x2 += qs[i] * qs[i];
+        return warp_sum(x2);
+    };
+    float nx2 = 0.f;
+    if constexpr (kApart) nx2 = norm2_of_q();   // (while W_q comes in)
     {   // f = q W_q: 16 bytes of a row per lane
         const int lpr = df / V, rpl = 32 / lpr, cg = lane % lpr;
         float acc[V];
@@ -561,9 +581,8 @@ __device__ __forceinline__ void linear_item(const StepArgs<T> &a, long long bh, 
         group_sync<NW>();
     }
     {   // every warp forms the norms and sums
-        float nx2 = 0.f, f[4];
-        for (int i = lane; i < D; i += 32) nx2 += qs[i] * qs[i];
-        nx2 = warp_sum(nx2);
+        float f[4];
+        if constexpr (!kApart) nx2 = norm2_of_q();
 #pragma unroll
         for (int jj = 0; jj < 4; ++jj) {
             f[jj] = 0.f;
@@ -627,15 +646,15 @@ __device__ __forceinline__ void linear_item(const StepArgs<T> &a, long long bh, 
 
 // This block's share of the read-outs, by groups of NW warps, from the first-th of the block on: its j-th is item j * blocks +
 // (its place among the blocks), and belongs to group j % groups.
-template <typename T, int D, int NW, class Ring>
-__device__ __forceinline__ void work_on_items(const StepArgs<T> &a, uint8_t *smem, int first) {
+template <typename T, int D, int NW, bool kApart, class Ring, class StateOk>
+__device__ __forceinline__ void work_on_items(const StepArgs<T> &a, uint8_t *smem, int first, StateOk state_ok) {
     constexpr int kGroups = kStepWarps / NW;
     const int warp = threadIdx.x >> 5, group = warp / NW, blocks = (int)gridDim.x - a.first_item_block;
     float *mine = reinterpret_cast<float *>(smem + Ring::kTotal) + group * (kItemFloats + NW * 128);
     for (int j = group; ; j += kGroups) {
         const long long i = (int)blockIdx.x - a.first_item_block + (long long)j * blocks;
         if (i >= a.n_items) break;
-        if (j >= first) linear_item<T, D, NW, Ring>(a, i, smem + warp * Ring::kWarp, mine);
+        if (j >= first) linear_item<T, D, NW, kApart, Ring>(a, i, smem + warp * Ring::kWarp, mine, state_ok);
     }
 }
 
@@ -814,7 +833,8 @@ template <typename T, int D>
 struct StepRing : AttendPlan<D> {};
 template <int D>
 struct StepRing<float, D> : AttendPlanF32<D> {};
-// kMaps: with the map warps.
+// What a block does beside its tiles: the read-outs apart have blocks of their own; or all share them, with map warps or without.
+enum StepMode { kItemsApart, kItemsShared, kItemsMapped };
 template <bool kMaps>
 constexpr int kMainThreads = kStepThreads + (kMaps ? kMapWarps * 32 : 0);
 // Shared memory of step_main_kernel: the rings, and what lies beside them.
@@ -829,12 +849,21 @@ static_assert(step_main_smem<__nv_bfloat16, 128, true>() <= 232448 && step_main_
 // read-out, timed in turn on one box: B = 64, 32K prefix, every token 1302 (1657), 6.6 TB/s; B = 16, 16K, a quarter kept
 // 148 (307); B = 32, 8K, capped at 448: 72 (203)), at one sequence the latency of a block's chain (one user, 2K prefix:
 // 10.5 (72), of which the host needs 10).
-template <typename T, int D, int NH, bool kMaps>
-__global__ void __launch_bounds__(kMaps ? 512 : kStepThreads, 1)   // (512: 128 registers a thread, see below)
+template <typename T, int D, int NH, StepMode kMode>
+__global__ void __launch_bounds__(kMode == kItemsMapped ? 512 : kStepThreads, 1)   // (512: 128 registers a thread, see below)
 step_main_kernel(const __grid_constant__ StepArgs<T> a) {
     extern __shared__ __align__(128) uint8_t step_smem[];
     grid_dep_wait();
     grid_dep_launch();
+    constexpr bool kMaps = kMode == kItemsMapped;
+    using Ring = StepRing<T, D>;
+    uint8_t *beside = step_smem + Ring::kTotal;
+    if constexpr (kMode == kItemsApart) {
+        if ((int)blockIdx.x >= a.first_item_block) {
+            work_on_items<T, D, kStepWarps, true, Ring>(a, step_smem, 0, [&] { return state_mismatch(a.hdr, a.key) == 0; });
+            return;
+        }
+    }
     {   // the header against the call; on a mismatch nothing is written but the status word
         const int bad = state_mismatch(a.hdr, a.key);
         if (bad != 0) {
@@ -842,8 +871,6 @@ step_main_kernel(const __grid_constant__ StepArgs<T> a) {
             return;
         }
     }
-    using Ring = StepRing<T, D>;
-    uint8_t *beside = step_smem + Ring::kTotal;
     if constexpr (kMaps) {
         if (threadIdx.x >= kStepThreads) {
             reg_dec_step<64>();
@@ -891,12 +918,12 @@ step_main_kernel(const __grid_constant__ StepArgs<T> a) {
         else if (a.item_warps == 2) states.template run<2>(beside);
         else states.template run<kStepWarps>(beside);
     }
-    if ((int)blockIdx.x < a.first_item_block) return;
+    if (kMode == kItemsApart || (int)blockIdx.x < a.first_item_block) return;   // (they have blocks of their own, or there are none)
     // (beyond kMaxPhi a block only has more where a read-out is one warp's: the groups' places beside the rings do not meet)
     const int first = kMaps ? kMaxPhi : 0;
-    if (a.item_warps == 1) work_on_items<T, D, 1, Ring>(a, step_smem, first);
-    else if (a.item_warps == 2) work_on_items<T, D, 2, Ring>(a, step_smem, first);
-    else work_on_items<T, D, kStepWarps, Ring>(a, step_smem, first);
+    if (a.item_warps == 1) work_on_items<T, D, 1, false, Ring>(a, step_smem, first, [] { return true; });
+    else if (a.item_warps == 2) work_on_items<T, D, 2, false, Ring>(a, step_smem, first, [] { return true; });
+    else work_on_items<T, D, kStepWarps, false, Ring>(a, step_smem, first, [] { return true; });
 }
 
 // grid (H, B), D + 64 threads: an output column each, then a warp that scores the new token and one that appends its K / V
@@ -1018,24 +1045,25 @@ static int launch_route(const still_params_t *p, const StepArgs<T> &a, int32_t *
 constexpr int kMapTiles = 512;   // tiles of a block
 template <typename T, int D, int NH>
 static int launch_main(const StepArgs<T> &a, unsigned grid, cudaStream_t st, int *launches) {
-    auto launch = [&](auto maps) -> int {
-        constexpr bool kMaps = decltype(maps)::value;
+    auto launch = [&](auto mode) -> int {
+        constexpr StepMode kMode = decltype(mode)::value;
+        constexpr bool kMaps = kMode == kItemsMapped;
         constexpr int kSmem = step_main_smem<T, D, kMaps>();
-        STILL_CUDA(ensure_dynamic_smem((const void *)step_main_kernel<T, D, NH, kMaps>, kSmem));
+        STILL_CUDA(ensure_dynamic_smem((const void *)step_main_kernel<T, D, NH, kMode>, kSmem));
         profile_mark_begin(st);
-        STILL_CUDA(launch_dependent(step_main_kernel<T, D, NH, kMaps>, dim3(grid), dim3(kMainThreads<kMaps>), kSmem, st, a));
+        STILL_CUDA(launch_dependent(step_main_kernel<T, D, NH, kMode>, dim3(grid), dim3(kMainThreads<kMaps>), kSmem, st, a));
         profile_mark_end(st);
         return STILL_OK;
     };
-    int rc;
     // Map warps where the blocks have read-outs behind their tiles (bf16, up to eight heads a KV group: with 16 the cache pass
     // needs the registers) and these are not many: what the read-outs gain is a few us whatever the tiles, and the cache pass, in
-    // fewer registers and beside the loads of W_q, takes up to 2 % longer.  (us a
-    // step without and with them: 325 tiles a block 82.7 and 81.4, 865 tiles, 16 sequences x 16000 tokens, 141.2 and 142.5.)
-    if constexpr (sizeof(T) == 2 && NH <= 8)
-        rc = a.n_items > 0 && a.first_item_block == 0 && a.per <= kMapTiles ? launch(std::true_type{}) : launch(std::false_type{});
-    else
-        rc = launch(std::false_type{});
+    // fewer registers and beside the loads of W_q, takes up to 2 % longer.  (us a step without and with them: 325 tiles a block
+    // 82.7 and 81.4, 865 tiles, 16 sequences x 16000 tokens, 141.2 and 142.5.)
+    constexpr bool kCanMap = sizeof(T) == 2 && NH <= 8;
+    int rc;
+    if (a.n_items > 0 && a.first_item_block > 0) rc = launch(std::integral_constant<StepMode, kItemsApart>{});
+    else if (kCanMap && a.n_items > 0 && a.per <= kMapTiles) rc = launch(std::integral_constant<StepMode, kCanMap ? kItemsMapped : kItemsShared>{});
+    else rc = launch(std::integral_constant<StepMode, kItemsShared>{});
     if (rc != STILL_OK) return rc;
     STILL_CUDA(launch_dependent(step_merge_kernel<T, D>, dim3(a.H, a.B), dim3(D + 64), 0, st, a));
     *launches += 2;
