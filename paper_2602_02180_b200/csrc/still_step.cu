@@ -858,13 +858,8 @@ step_main_kernel(const __grid_constant__ StepArgs<T> a) {
     constexpr bool kMaps = kMode == kItemsMapped;
     using Ring = StepRing<T, D>;
     uint8_t *beside = step_smem + Ring::kTotal;
-    if constexpr (kMode == kItemsApart) {
-        if ((int)blockIdx.x >= a.first_item_block) {
-            work_on_items<T, D, kStepWarps, true, Ring>(a, step_smem, 0, [&] { return state_mismatch(a.hdr, a.key) == 0; });
-            return;
-        }
-    }
-    {   // the header against the call; on a mismatch nothing is written but the status word
+    // (a block with a read-out apart has no tiles, and compares the header itself)
+    if (kMode != kItemsApart || (int)blockIdx.x < a.first_item_block) {   // the header against the call; on a mismatch nothing is written but the status word
         const int bad = state_mismatch(a.hdr, a.key);
         if (bad != 0) {
             if (blockIdx.x == 0 && threadIdx.x == 0 && bad != 4) report_status(a.hdr + 14, STILL_ERR_STATE_MISMATCH, bad);
@@ -918,7 +913,11 @@ step_main_kernel(const __grid_constant__ StepArgs<T> a) {
         else if (a.item_warps == 2) states.template run<2>(beside);
         else states.template run<kStepWarps>(beside);
     }
-    if (kMode == kItemsApart || (int)blockIdx.x < a.first_item_block) return;   // (they have blocks of their own, or there are none)
+    if ((int)blockIdx.x < a.first_item_block) return;
+    if constexpr (kMode == kItemsApart) {
+        work_on_items<T, D, kStepWarps, true, Ring>(a, step_smem, 0, [&] { return state_mismatch(a.hdr, a.key) == 0; });
+        return;
+    }
     // (beyond kMaxPhi a block only has more where a read-out is one warp's: the groups' places beside the rings do not meet)
     const int first = kMaps ? kMaxPhi : 0;
     if (a.item_warps == 1) work_on_items<T, D, 1, false, Ring>(a, step_smem, first, [] { return true; });
