@@ -11,6 +11,7 @@
 #include <cstring>
 
 #include "still_simt.cuh"
+#include "still_state.cuh"
 #include "still_tc.h"
 
 namespace still {
@@ -194,101 +195,18 @@ static cudaError_t set_smem(K kernel, size_t bytes) {
         if (e__ != cudaSuccess) return STILL_ERR_CUDA;     \
     } while (0)
 
-__device__ __forceinline__ void write_header(int32_t *hdr, const still_params_t &p, long long cap, long long t) {
-    hdr[0] = 0x5354494c;  // "STIL"
-    hdr[1] = 1;
-    hdr[2] = p.B; hdr[3] = p.H; hdr[4] = p.Hkv; hdr[5] = p.d; hdr[6] = p.d_f;
-    hdr[7] = p.chunk; hdr[8] = p.topk; hdr[9] = p.dtype;
-    hdr[10] = (int32_t)(cap & 0xffffffffll); hdr[11] = (int32_t)(cap >> 32);
-    hdr[12] = (int32_t)(t & 0xffffffffll); hdr[13] = (int32_t)(t >> 32);
-    hdr[14] = 0; hdr[15] = 0;
-}
 __global__ void write_header_kernel(int32_t *hdr, still_params_t p, long long cap, long long t) {
     grid_dep_wait();
     grid_dep_launch();
     if (threadIdx.x == 0) write_header(hdr, p, cap, t);
 }
 
-// Everything of the decode state that a prefill only has to put in its place, in one launch of 256-thread blocks (as four
-// strided copies and two kernels it was 27 us of a 1003-token prompt, nearly all of it launches):
-//   kv_blocks per (K or V, batch, KV head): the rows [first, N) of the sequence into their ring rows (position q in row
-//     q % kvr; first > 0 only with a salient-cache budget), 16 bytes a thread and step;
-//   score_blocks per (batch, query head): the scores;
-//   then a warp per (batch, query head, chunk): the selected positions, also as bit masks -- bit j of word w is set when
-//     position chunk * C + 32 w + j is among them;
-//   the last block: the header.
-struct StateParts {
-    const char *K, *V;
-    char *k_cache, *v_cache;
-    const float *scores;
-    float *score_out;
-    const int32_t *sel;
-    int32_t *sel_out, *hdr;
-    uint32_t *mask_out;
-    long long N, first, kvr, cap, T, capT;
-    int BH, BHkv, row_bytes, C, lam, kv_blocks, score_blocks, sel_blocks;
-};
-constexpr int kStateSteps = 4;   // pieces (K / V) or scores per thread
+// The decode state's part of a prefill (write_state_block) as a launch of its own.
 __global__ void __launch_bounds__(256)
 write_state_kernel(const __grid_constant__ StateParts s, const __grid_constant__ still_params_t p) {
     grid_dep_wait();
     grid_dep_launch();
-    long long blk = blockIdx.x;
-    const long long n_kv = 2ll * s.BHkv * s.kv_blocks, n_sc = (long long)s.BH * s.score_blocks;
-    if (blk < n_kv) {
-        const long long unit = blk / s.kv_blocks, head = unit >> 1;
-        const int ppr = s.row_bytes / 16;
-        const long long n = (s.N - s.first) * ppr, i0 = (blk - unit * s.kv_blocks) * (256 * kStateSteps) + threadIdx.x;
-        const uint4 *src = reinterpret_cast<const uint4 *>((unit & 1 ? s.V : s.K) + (head * s.N + s.first) * s.row_bytes);
-        uint4 *dst = reinterpret_cast<uint4 *>((unit & 1 ? s.v_cache : s.k_cache) + head * s.kvr * s.row_bytes);
-        uint4 v[kStateSteps];
-#pragma unroll
-        for (int k = 0; k < kStateSteps; ++k)
-            if (i0 + 256 * k < n) v[k] = src[i0 + 256 * k];
-#pragma unroll
-        for (int k = 0; k < kStateSteps; ++k) {
-            const long long i = i0 + 256 * k;
-            if (i < n) {
-                const uint32_t q = (uint32_t)(i / ppr + s.first), r = q < s.kvr ? q : q % (uint32_t)s.kvr;
-                dst[(long long)r * ppr + i % ppr] = v[k];
-            }
-        }
-        return;
-    }
-    blk -= n_kv;
-    if (blk < n_sc) {
-        const long long bh = blk / s.score_blocks, i0 = (blk - bh * s.score_blocks) * (256 * kStateSteps) + threadIdx.x;
-#pragma unroll
-        for (int k = 0; k < kStateSteps; ++k)
-            if (i0 + 256 * k < s.N) s.score_out[bh * s.cap + i0 + 256 * k] = s.scores[bh * s.N + i0 + 256 * k];
-        return;
-    }
-    blk -= n_sc;
-    if (blk < s.sel_blocks) {
-        const long long wid = blk * 8 + (threadIdx.x >> 5);
-        if (wid >= (long long)s.BH * s.T) return;
-        const int lane = threadIdx.x & 31;
-        const long long bh = wid / s.T, c = wid % s.T;
-        const int32_t *si = s.sel + (bh * s.T + c) * s.lam;
-        int32_t *so = s.sel_out + (bh * s.capT + c) * s.lam;
-        int pos[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            pos[i] = lane + 32 * i < s.lam ? si[lane + 32 * i] : -1;
-            if (lane + 32 * i < s.lam) so[lane + 32 * i] = pos[i];
-        }
-        for (int w = 0; w < s.C / 32; ++w) {
-            const long long p0 = c * s.C + 32ll * w;
-            uint32_t bits = 0u;
-#pragma unroll
-            for (int i = 0; i < 4; ++i)
-                if (pos[i] >= p0 && pos[i] < p0 + 32) bits |= 1u << (int)(pos[i] - p0);
-            bits = __reduce_or_sync(0xffffffffu, bits);
-            if (lane == 0) s.mask_out[(bh * s.capT + c) * (s.C / 32) + w] = bits;
-        }
-        return;
-    }
-    if (threadIdx.x == 0) write_header(s.hdr, p, s.cap, s.N);
+    write_state_block(s, p, blockIdx.x);
 }
 
 // ------------------------------------------------------------------ FMA path launches
@@ -437,6 +355,33 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
         if (N > L.capacity) return STILL_ERR_STATE_FULL;
     }
 
+    // What of the decode state only has to be put in its place (see write_state_block).
+    StateParts sp{};
+    bool state_written = false;
+    if (state) {
+        const long long kvr = state_kv_rows(p, L.capacity);
+        sp.K = reinterpret_cast<const char *>(K);
+        sp.V = reinterpret_cast<const char *>(V);
+        sp.k_cache = state + L.k_cache;
+        sp.v_cache = state + L.v_cache;
+        sp.scores = sc;
+        sp.score_out = reinterpret_cast<float *>(state + L.score);
+        sp.sel = sel;
+        sp.sel_out = reinterpret_cast<int32_t *>(state + L.sel_idx);
+        sp.mask_out = reinterpret_cast<uint32_t *>(state + L.sel_mask);
+        sp.hdr = reinterpret_cast<int32_t *>(state + L.header);
+        sp.N = N; sp.first = std::max<long long>(0, N - kvr); sp.kvr = kvr; sp.cap = L.capacity;
+        sp.T = w.T; sp.capT = L.capacity / p->chunk;
+        sp.BH = p->B * p->H; sp.BHkv = p->B * p->Hkv; sp.row_bytes = p->d * (int)sizeof(T);
+        sp.C = p->chunk; sp.lam = p->topk;
+        constexpr int kPer = 256 * kStateSteps;
+        sp.kv_blocks = (int)(((N - sp.first) * (sp.row_bytes / 16) + kPer - 1) / kPer);
+        sp.score_blocks = (int)((N + kPer - 1) / kPer);
+        sp.sel_blocks = p->topk > 0 ? (int)(((long long)sp.BH * w.T + 7) / 8) : 0;
+        sp.blocks = 2ll * sp.BHkv * sp.kv_blocks + (long long)sp.BH * sp.score_blocks + sp.sel_blocks + 1;
+        if (sp.blocks >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;   // (a state of 32 TB)
+    }
+
     // (1)+(2) Self-Saliency Score and per-chunk top-k; beside it the feature maps of the FMA kernels.
     const bool maps_too = w.la && !w.tc && front_blocks(p, N) <= kFrontBlocks;
     if (maps_too)
@@ -464,7 +409,7 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
                               reinterpret_cast<float *>(ws + w.zpre), ypart, dpart, reinterpret_cast<float *>(ws + w.segs), S_out,
                               z_out, w.phiKsel ? ws + w.phiKsel : nullptr, Y && w.ksel ? ws + w.ksel : nullptr,
                               (Y || w.phiKsel) && w.vsel ? ws + w.vsel : nullptr, w.sel_rows,
-                              status, st, &g_launches);
+                              state ? &sp : nullptr, &state_written, status, st, &g_launches);
             if (rc != STILL_OK) return rc;
         } else {
             T *phiQ = reinterpret_cast<T *>(ws + w.phiQ);
@@ -500,31 +445,10 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
         if (rc != STILL_OK) return rc;
     }
 
-    // Decode state: K/V history, scores, selection; S and z were written above.
-    if (state) {
-        const long long kvr = state_kv_rows(p, L.capacity);
-        StateParts sp{};
-        sp.K = reinterpret_cast<const char *>(K);
-        sp.V = reinterpret_cast<const char *>(V);
-        sp.k_cache = state + L.k_cache;
-        sp.v_cache = state + L.v_cache;
-        sp.scores = sc;
-        sp.score_out = reinterpret_cast<float *>(state + L.score);
-        sp.sel = sel;
-        sp.sel_out = reinterpret_cast<int32_t *>(state + L.sel_idx);
-        sp.mask_out = reinterpret_cast<uint32_t *>(state + L.sel_mask);
-        sp.hdr = reinterpret_cast<int32_t *>(state + L.header);
-        sp.N = N; sp.first = std::max<long long>(0, N - kvr); sp.kvr = kvr; sp.cap = L.capacity;
-        sp.T = w.T; sp.capT = L.capacity / p->chunk;
-        sp.BH = p->B * p->H; sp.BHkv = p->B * p->Hkv; sp.row_bytes = p->d * (int)sizeof(T);
-        sp.C = p->chunk; sp.lam = p->topk;
-        constexpr int kPer = 256 * kStateSteps;
-        sp.kv_blocks = (int)(((N - sp.first) * (sp.row_bytes / 16) + kPer - 1) / kPer);
-        sp.score_blocks = (int)((N + kPer - 1) / kPer);
-        sp.sel_blocks = p->topk > 0 ? (int)(((long long)sp.BH * w.T + 7) / 8) : 0;
-        const long long blocks = 2ll * sp.BHkv * sp.kv_blocks + (long long)sp.BH * sp.score_blocks + sp.sel_blocks + 1;
-        if (blocks >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;   // (a state of 32 TB)
-        STILL_CUDA(launch_dependent(write_state_kernel, dim3((unsigned)blocks), dim3(256), 0, st, sp, *p));
+    // Decode state: K/V history, scores, selection, where they have not been written with the gathered rows; S and z were written
+    // above.
+    if (state && !state_written) {
+        STILL_CUDA(launch_dependent(write_state_kernel, dim3((unsigned)sp.blocks), dim3(256), 0, st, sp, *p));
         ++g_launches;
     }
     return STILL_OK;

@@ -38,6 +38,7 @@
 #include <algorithm>
 
 #include "still_common.cuh"
+#include "still_state.cuh"
 #include "still_tc_ptx.cuh"
 
 namespace still {
@@ -282,7 +283,7 @@ npmap_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
 // Selected rows, and the normaliser z (Eq. cache_routing_sum): z after chunk c = sum over the chunks 0..c of the
 // features of their unselected tokens = (column sums of phi(K) over the chunk) - (rows of its selected tokens).
 // ------------------------------------------------------------------------------------------
-// grid (T + 1, B*H), 256 threads: the lam selected tokens of chunk blockIdx.x of a query head, read once for everything
+// grid (T + 1, B*H; with the decode state: and as many rows as its blocks take), 256 threads: the lam selected tokens of chunk blockIdx.x of a query head, read once for everything
 // that is made of them: their K and V rows in selection order (row j of a head is token sel_idx[j]; K_sel / V_sel, what
 // the attention kernel tiles), with a salient-cache budget also their phi(K) rows (phi_sel, from which the tokens that
 // leave the cache enter the state), and the sum of the phi(K) rows (selsum [B*H, n_routed, 2 DF], of the routed chunks).
@@ -291,14 +292,19 @@ npmap_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
 // gathered for themselves (and one that summed a row after the other) took 1023 us, this one 305.
 // kFew: at d = 64 up to 16 tokens of a chunk are one row a thread; eight blocks an SM instead of five keep as many rows in flight
 // (128 heads x 4096 tokens, 16 of 64: 29.7 us and 23.7; with 32 of 64 a thread's two rows one after the other 6 us more).
-template <int D, int DF, bool kFew>
+template <int D, int DF, bool kFew, bool kState>
 __global__ void __launch_bounds__(256, D == 128 ? 4 : kFew ? 8 : 5)
 gather_kernel(const __nv_bfloat16 *K, const __nv_bfloat16 *V, const __nv_bfloat16 *phiK,
               const int32_t *sel_idx, __nv_bfloat16 *Ksel, __nv_bfloat16 *Vsel,
               __nv_bfloat16 *phi_sel, float *selsum, int H, int Hkv, long long N, int lam,
-              long long sel_rows, int n_routed) {
+              long long sel_rows, int n_routed, int BH, const __grid_constant__ StateParts state, const __grid_constant__ still_params_t p) {
     grid_dep_wait();
     grid_dep_launch();
+    if (kState && (int)blockIdx.y >= BH) {   // the decode state (its blocks behind the others)
+        const long long blk = (long long)((int)blockIdx.y - BH) * gridDim.x + blockIdx.x;
+        if (blk < state.blocks) write_state_block(state, p, blk);
+        return;
+    }
     constexpr int kVec = D / 8, kPhiVec = 2 * DF / 8;       // 16-byte pieces of a row
     constexpr int kPer = 32 / kVec, kPhiPer = 32 / kPhiVec;  // rows that a warp moves at a time
     __shared__ __align__(16) float sums[8 * kPhiPer][2 * DF];   // (written 16 bytes at a time)
@@ -1199,14 +1205,18 @@ int launch_npmap(const void *X, const void *W, const void *bias, void *phi, floa
 
 template <int D, int DF>
 int launch_gather(const still_params_t *p, long long N, const void *K, const void *V, const void *phiK, const int32_t *sel_idx,
-                  void *k_sel, void *v_sel, void *phiK_sel, float *selsum, long long sel_rows, int n_routed, cudaStream_t st,
-                  int *launches) {
+                  void *k_sel, void *v_sel, void *phiK_sel, float *selsum, long long sel_rows, int n_routed, const StateParts *state,
+                  cudaStream_t st, int *launches) {
     using bf = __nv_bfloat16;
     const long long Tn = (N + p->chunk - 1) / p->chunk;
     ++*launches;
-    return launch_dependent(D == 64 && p->topk <= 16 ? gather_kernel<D, DF, D == 64> : gather_kernel<D, DF, false>, dim3((unsigned)(Tn + 1), (unsigned)(p->B * p->H)), dim3(256), 0, st, (const bf *)K,
-                            (const bf *)V, (const bf *)phiK, sel_idx, (bf *)k_sel, (bf *)v_sel, (bf *)phiK_sel, selsum, p->H, p->Hkv,
-                            N, p->topk, sel_rows, n_routed) == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
+    const long long BH = (long long)p->B * p->H, rows = state != nullptr ? (state->blocks + Tn) / (Tn + 1) : 0;
+    const bool few = D == 64 && p->topk <= 16;
+    return launch_dependent(state == nullptr ? (few ? gather_kernel<D, DF, D == 64, false> : gather_kernel<D, DF, false, false>)
+                                             : (few ? gather_kernel<D, DF, D == 64, true> : gather_kernel<D, DF, false, true>),
+                            dim3((unsigned)(Tn + 1), (unsigned)(BH + rows)), dim3(256), 0, st, (const bf *)K, (const bf *)V,
+                            (const bf *)phiK, sel_idx, (bf *)k_sel, (bf *)v_sel, (bf *)phiK_sel, selsum, p->H, p->Hkv, N, p->topk, sel_rows,
+                            n_routed, (int)BH, state != nullptr ? *state : StateParts{}, *p) == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
 }
 
 // Whether every segment of the scan folds the chunks before it itself, rather than starting from a pass of sums: up to a
@@ -1294,7 +1304,8 @@ int tc_la_sum_parts(int seg_chunks) {
 int tc_la_branch(const still_params_t *p, long long N, const void *Q, const void *K, const void *V, const void *G,
                  const void *Wq, const void *bq, const void *Wk, const void *bk, const int32_t *sel_idx, void *phiK,
                  float *csum, float *zpre, void *y_part, float *d_part, float *seg_sums, float *S_out, float *z_out,
-                 void *phiK_sel, void *k_sel, void *v_sel, long long sel_rows, int *status_words, cudaStream_t st, int *launches) {
+                 void *phiK_sel, void *k_sel, void *v_sel, long long sel_rows, const StateParts *state_parts, bool *state_written,
+                 int *status_words, cudaStream_t st, int *launches) {
     using bf = __nv_bfloat16;
     if ((long long)p->B * p->H * N >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;  // TMA row coordinate
     const int NF = 2 * p->d_f, C = p->chunk;
@@ -1314,13 +1325,18 @@ int tc_la_branch(const still_params_t *p, long long N, const void *Q, const void
     float *selsum = reinterpret_cast<float *>(y_part);
     const int window = p->topk > 0 ? (int)(p->max_salient / p->topk) : 0;
     if (p->topk < C) {
+        // The decode state rides along up to 512 blocks, where a launch is longer than what it does.  (32 heads, d = 128, gated, 1003
+        // tokens, 350 blocks: 82.9 us a call with a launch of its own, 80.7 like this; 4000 tokens, 1250 blocks: 215 and 224, the rows'
+        // copies stand in the gather's way.)
+        if (state_parts != nullptr && (state_parts->blocks > 512 || BH > 32768)) state_parts = nullptr;   // (BH: rows of a grid)
         if (p->d == 64 && p->d_f == 64)
-            rc = launch_gather<64, 64>(p, N, K, V, phiK, sel_idx, k_sel, v_sel, phiK_sel, selsum, sel_rows, n_routed, st, launches);
+            rc = launch_gather<64, 64>(p, N, K, V, phiK, sel_idx, k_sel, v_sel, phiK_sel, selsum, sel_rows, n_routed, state_parts, st, launches);
         else if (p->d == 128 && p->d_f == 64)
-            rc = launch_gather<128, 64>(p, N, K, V, phiK, sel_idx, k_sel, v_sel, phiK_sel, selsum, sel_rows, n_routed, st, launches);
+            rc = launch_gather<128, 64>(p, N, K, V, phiK, sel_idx, k_sel, v_sel, phiK_sel, selsum, sel_rows, n_routed, state_parts, st, launches);
         else
-            rc = launch_gather<128, 128>(p, N, K, V, phiK, sel_idx, k_sel, v_sel, phiK_sel, selsum, sel_rows, n_routed, st, launches);
+            rc = launch_gather<128, 128>(p, N, K, V, phiK, sel_idx, k_sel, v_sel, phiK_sel, selsum, sel_rows, n_routed, state_parts, st, launches);
         if (rc != STILL_OK) return rc;
+        *state_written = state_parts != nullptr;
     }
     if (n_routed > 0 || z_out != nullptr) {
         // a warp per eight chunks, whose loads are in flight together; at most 32

@@ -74,6 +74,7 @@ int tc_la_to_part(const float *N_LA, const float *D_LA, void *y_part, float *d_p
 int tc_selftest_wait_timeout(int *status_words, long long limit_cycles, cudaStream_t st);
 
 // ---- tensor-core linear-attention branch of the prefill, bf16 only --------------------
+struct StateParts;   // still_state.cuh
 // True when NP-Map and the chunk-wise state scan of these parameters run on the tcgen05 kernels.
 bool tc_la_supported(const still_params_t *p);
 // NP-Map of K (bf16 features into phiK [B,Hkv,N,2 d_f], chunk column sums into csum [B,Hkv,T,2 d_f]), the
@@ -81,11 +82,12 @@ bool tc_la_supported(const still_params_t *p);
 // fused in: y_part [2][B,H,N,d] bf16 = N_part / D_part (gated), d_part [2][B,H,N] fp32, one part per feature
 // half; S_out / z_out (optional) receive the state after the chunks that have left the local region.
 // With topk < chunk it also compacts the selected rows: K_sel / V_sel (each optional) and, when phiK_sel is given (it is
-// needed with a budget), their phi(K) rows.
+// needed with a budget), their phi(K) rows; and then, where state_parts is given, what that describes (*state_written).
 int tc_la_branch(const still_params_t *p, long long N, const void *Q, const void *K, const void *V, const void *G,
                  const void *Wq, const void *bq, const void *Wk, const void *bk, const int32_t *sel_idx, void *phiK,
                  float *csum, float *zpre, void *y_part, float *d_part, float *seg_sums, float *S_out, float *z_out,
-                 void *phiK_sel, void *k_sel, void *v_sel, long long sel_rows, int *status_words, cudaStream_t st, int *launches);
+                 void *phiK_sel, void *k_sel, void *v_sel, long long sel_rows, const StateParts *state_parts, bool *state_written,
+                 int *status_words, cudaStream_t st, int *launches);
 // Segments of the two-level state scan for these parameters (1 = plain scan); *seg_chunks = chunks per segment.
 // seg_sums holds (segments - 1) partial states [2 d_f, d] fp32 per (batch, head).
 int tc_la_segments(const still_params_t *p, long long N, int *seg_chunks);
