@@ -714,9 +714,9 @@ __device__ __forceinline__ void output_role(Work w, const AttnBars &bar, const u
 // Q K^T runs three items ahead of P V: P_A V, Q_B K^T of B's next tile, P_B V, Q_A K^T of A's next but one, and so on.
 // S of A's next tile is then complete when its softmax warps come back for it, and where S_A and S_B share their place
 // the warps of A have read theirs by the time B's is to be formed.  What bounds the kernel is then the softmax warps'
-// arithmetic, two of them per scheduler (32768 tokens, d = 128: issue slots 52 %, special-function unit 51 %, tensor pipe 69 %;
-// 4096 tokens, d = 64: 50, 45 and 30 %), and for short streams the start and the end of a CTA.  With P over S, S of a tile
-// waited for the softmax warps of the tile before and these for it (us a call, then and now, in turn on one box: 64 heads x 32768
+// arithmetic, two of them per scheduler (32768 tokens, d = 128: issue slots 52 %, special-function unit 52 %, tensor pipe 71 %;
+// 4096 tokens, d = 64: 50, 47 and 32 %).  With P over S, S of a tile waited for the softmax warps of the tile before and these for
+// it (us a call, then and with P in its own place, when a CTA ended with its item, in turn on one box: 64 heads x 32768
 // tokens, d = 128, every token kept 15887 and 15154, a quarter 6665 and 6208; 32 x 131072, capped at 896, 8697 and 7809; 128 x
 // 4096, d = 64, every token 551 and 502, a quarter 585 and 515; the scan and the score kernel have a part in the quarters and in
 // the capped call).  Two threads per row instead of one (16 softmax warps) were slower by 10 %: the stream's bookkeeping doubles.
