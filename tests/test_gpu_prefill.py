@@ -459,3 +459,30 @@ def test_fp32_small_calls(B, H, Hkv, d, df, C, k, N):
     heads = [(0, 0), (B - 1, H - 1)]
     U.check_selection(scores, sel, C, k, heads)
     U.check_outputs(w, Q, K, V, Wq, Wk, Y, scores, sel, heads, bq=bq, bk=bk, tol=1e-5)
+
+
+@pytest.mark.parametrize("N,rides", [(200, True), (1400, True), (1500, False)])
+def test_state_written_among_the_gathered_rows(N, rides):
+    # 505 and 545 blocks of copies: the last size that rides along with the gather, and one with a launch of its own
+    B, H, Hkv, d, C, k = 1, 32, 8, 128, 64, 16
+    w = _small("t", "bf16", B, H, Hkv, d, N, C, k)
+    p, cap = U.params_of(w), N + 70
+    lay = still.state_layout(p, cap)
+    state = torch.full((lay["total"],), 255, dtype=torch.uint8, device="cuda")
+    r = U.run_prefill(w, state=state, state_max_tokens=cap)
+    with_state = still.last_launch_count()
+    U.run_prefill(w)
+    assert with_state - still.last_launch_count() == (0 if rides else 1)
+    n_cap, part = lay["capacity"], lambda at, n, dt: state[lay[at]: lay[at] + n * dt.itemsize].view(dt)
+    for at, x in (("k_cache", r["K"]), ("v_cache", r["V"])):
+        assert torch.equal(part(at, B * Hkv * n_cap * d, torch.bfloat16).view(B, Hkv, n_cap, d)[:, :, :N], x)
+    assert torch.equal(part("score", B * H * n_cap, torch.float32).view(B, H, n_cap)[:, :, :N], r["scores"])
+    T = -(-N // C)
+    assert torch.equal(part("sel_idx", B * H * (n_cap // C) * k, torch.int32).view(B, H, -1, k)[:, :, :T], r["sel"])
+    words = part("sel_mask", B * H * (n_cap // C) * (C // 32), torch.int32).view(B, H, -1)[:, :, : T * (C // 32)].cpu()
+    bits = ((words[..., None] >> torch.arange(32)) & 1).flatten(2)
+    want = torch.zeros(B, H, T * C, dtype=torch.int32)
+    sel = r["sel"].cpu().flatten(2).long()
+    want.scatter_add_(2, sel.clamp_min(0), (sel >= 0).int())
+    assert torch.equal(bits, want)
+    assert part("header", 14, torch.int32)[12].item() == N
