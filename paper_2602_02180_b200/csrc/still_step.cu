@@ -1058,10 +1058,15 @@ static int launch_main(const StepArgs<T> &a, unsigned grid, cudaStream_t st, int
     // needs the registers) and these are not many: what the read-outs gain is a few us whatever the tiles, and the cache pass, in
     // fewer registers and beside the loads of W_q, takes up to 2 % longer.  (us a step without and with them: 325 tiles a block
     // 82.7 and 81.4, 865 tiles, 16 sequences x 16000 tokens, 141.2 and 142.5.)
+    // Nor where the map warps, four read-outs at a time, would be what the block waits for (70 tiles are as long as a round of theirs:
+    // 32 sequences x 8192 tokens capped at 448, 204 tiles and two rounds, 71.9 without and 69.1 with them; 64 x 1000, 215 and four, 104.9 and
+    // 109.9; 64 x 3000 capped at 128, 160 and four, 100.7 and 106.5); with one round they always gain.
+    const long long items = (a.n_items + (long long)grid - 1) / grid, rounds = (items + kMapWarps - 1) / kMapWarps;
+    const bool map = a.n_items > 0 && a.per <= kMapTiles && (rounds == 1 || a.per >= 70 * rounds);
     constexpr bool kCanMap = sizeof(T) == 2 && NH <= 8;
     int rc;
     if (a.n_items > 0 && a.first_item_block > 0) rc = launch(std::integral_constant<StepMode, kItemsApart>{});
-    else if (kCanMap && a.n_items > 0 && a.per <= kMapTiles) rc = launch(std::integral_constant<StepMode, kCanMap ? kItemsMapped : kItemsShared>{});
+    else if (kCanMap && map) rc = launch(std::integral_constant<StepMode, kCanMap ? kItemsMapped : kItemsShared>{});
     else rc = launch(std::integral_constant<StepMode, kItemsShared>{});
     if (rc != STILL_OK) return rc;
     STILL_CUDA(launch_dependent(step_merge_kernel<T, D>, dim3(a.H, a.B), dim3(D + 64), 0, st, a));

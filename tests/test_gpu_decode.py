@@ -360,13 +360,14 @@ def test_decode_with_the_most_partials_a_head_can_have():
     (9, 20, 4, 128, 64, 64, 32, 64),     # ... tokens that leave a capped cache
     (7, 32, 4, 128, 64, 32, 8, 0),       # 224, eight heads a group
     (20, 32, 8, 64, 64, 64, 16, 0),      # 640, a warp each
-    (66, 32, 8, 64, 64, 32, 8, 0),       # 2112: more for some blocks than they keep features for
+    (66, 32, 8, 64, 64, 32, 8, 0),       # 2112, and few tiles: no warps for the features
+    (66, 32, 8, 64, 64, 64, 16, -1),     # ... long prefixes (-1): more for some blocks than they keep features for
     (5, 32, 2, 64, 64, 64, 16, 0),       # sixteen heads a group: no warps for the features
 ])
 def test_decode_batch_gives_each_sequence_its_own(B, H, Hkv, d, df, C, k, budget):
     # The read-outs of a batch (features by warps of their own) against those of its sequences alone, and the rounding between:
     # y differs by at most two of its roundings to bf16.
-    n0, steps = 2 * C + 9, 3
+    n0, steps, budget = (1290 if budget < 0 else 2 * C + 9), 3, max(budget, 0)
     w = synth.Workload("t", B, H, Hkv, d, n0 + steps, C, k, "bf16", "iid", 21)
     Q, K, V = synth.make_qkv(w, "cuda")
     g = torch.Generator(device="cuda").manual_seed(10)
