@@ -66,7 +66,7 @@ struct AttnPlan {
     static constexpr int kK = kQ + 2 * kQTile;                 // stage s at kK + s kStage: its K tile, then its V tile
     static constexpr int kV = kK + kKTile;
     static constexpr int kBar = kK + kStages * kStage;         // mbarriers
-    static constexpr int kNumBars = 2 + 2 * kStages + 2 + 2 + 2 + 2 + 4 + 4 + 2;
+    static constexpr int kNumBars = 2 + 2 * kStages + 2 + 2 + 2 + 2 + 4 + 4 + 3;
     static constexpr int kMisc = kBar + kNumBars * 8;          // tmem base, abort flag, "a CTA has failed before", -, item[2][2]
     static constexpr int kTotal = kMisc + 32;
     static constexpr int kAlloc = kTotal + 1024;               // slack to align the base to 1024
@@ -87,7 +87,7 @@ struct AttnBars {
     uint64_t *y_full;    // [2] the linear branch's results for query tile x are in their stages
     uint64_t *y_ready;   // [2] ... and the output is where the first of them were
     uint64_t *item_full, *item_empty;   // [2] an item to come is there; ... and has been read
-    uint64_t *first_done;   // (of a pair's second CTA) the first CTA's producer is done with an item
+    uint64_t *first_done;   // [2] (of a pair's second CTA) the first CTA's producer is done with an item
     uint64_t *drain;     // MMA warp: everything issued has completed (failure path)
     template <class P>
     __device__ __forceinline__ static AttnBars at(uint8_t *smem, P) {
@@ -105,7 +105,7 @@ struct AttnBars {
         b.item_full = b.y_ready + 2;
         b.item_empty = b.item_full + 2;
         b.first_done = b.item_empty + 2;
-        b.drain = b.first_done + 1;
+        b.drain = b.first_done + 2;
         return b;
     }
 };
@@ -632,13 +632,15 @@ __device__ __forceinline__ void producer_role(Work w, const AttnBars &bar, uint8
         if (!ok) break;
         if constexpr (kPair) {
             // The second CTA's loads count on the first's full-barriers, whose phases the first's own output entries move on as
-            // well: it begins with an item when the first has passed those of the item before.
+            // well: it begins with an item when the first has passed those of the item before.  It gives the item's place back
+            // behind that wait, and the first has waited for the place of the item before last, so that of the two
+            // barriers, taken by turns, none is two phases ahead.
             if (rank == 0) {
-                mbar_arrive_cluster(mapa(smem_u32(bar.first_done), 1));
+                mbar_arrive_cluster(mapa(smem_u32(bar.first_done + (n & 1)), 1));
             } else {
                 more = next_item<kPair>(w, bar, n, abort_flag, status, ok);
-                item_taken<kPair>(bar, n);
-                ok = ok && mbar_wait(bar.first_done, (uint32_t)n & 1u, abort_flag, status, 16);
+                ok = ok && mbar_wait(bar.first_done + (n & 1), (uint32_t)(n >> 1) & 1u, abort_flag, status, 16);
+                if (ok) item_taken<kPair>(bar, n);
             }
         }
     }
@@ -895,9 +897,9 @@ __device__ __forceinline__ void attention_body(const AttnMaps &tm, const float *
             mbar_init(bar.y_full + i, P::y_entries(n_parts));
             mbar_init(bar.item_full + i, 1);
             mbar_init(bar.y_ready + i, 4);
+            mbar_init(bar.first_done + i, 1);
             mbar_init(bar.item_empty + i, kCtas * 10 + 1 + (kCtas - 1));   // softmax and output warps, the issuing warp, the other producer
         }
-        mbar_init(bar.first_done, 1);
         mbar_init(bar.drain, 1);
         *abort_flag = 0;
         // A CTA that starts after another one has reported a failure does nothing; in a pair the first decides for both.

@@ -173,3 +173,31 @@ def test_score_tiles_of_a_cta(d, C, N):
     heads = [(0, 0), (0, 13), (1, 7), (1, 31)]
     U.check_selection(r["scores"], r["sel"], C, C // 4, heads)
     U.check_outputs(w, r["Q"], r["K"], r["V"], r["Wq"], r["Wk"], r["Y"], r["scores"], r["sel"], heads[1:], rows=U.sample_rows(N, 100, C))
+
+
+def _items_as_alone(d, B, N, C, k, df):
+    # More items than CTAs (pairs), of few tiles each: the rows of every sequence are those of the call with this sequence alone, where
+    # a CTA has one item, bit for bit, and every wait ended.
+    w = synth.Workload("t", B, 32, 32, d, N, C, k, "bf16", "head_scale", 37)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    G = synth.make_gate(w, "cuda")
+    g = torch.Generator(device="cuda").manual_seed(8)
+    Wq, Wk = ((torch.randn(32, d, df, generator=g, device="cuda") * 0.05).bfloat16() for _ in range(2))
+
+    def run(b0, b1):
+        p = still.StillParams(b1 - b0, 32, 32, d, C, k, torch.bfloat16, d_f=df, sm_scale=w.sm_scale)
+        ws = torch.empty(still.workspace_bytes(p, N), dtype=torch.uint8, device="cuda")
+        x = [t[b0:b1].contiguous() for t in (Q, K, V, G)]
+        Y = still.hybrid_attn_fwd(p, *x[:3], Wq, Wk, G=x[3] if k < C else None, workspace=ws)[0]
+        assert still.device_status(ws) == (0, 0)
+        return Y
+
+    Y = run(0, B)
+    for b in range(B):
+        assert torch.equal(Y[b], run(b, b + 1)[0])
+
+
+@pytest.mark.parametrize("N", [200, 600])
+def test_short_items_of_a_pair(N):
+    # five ring entries: the first CTA's producer can be through with an item while the second has not seen that it may begin with it
+    _items_as_alone(128, 5, N, 64, 16, 128)
