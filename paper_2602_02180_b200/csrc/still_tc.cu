@@ -66,7 +66,7 @@ struct AttnPlan {
     static constexpr int kK = kQ + 2 * kQTile;                 // stage s at kK + s kStage: its K tile, then its V tile
     static constexpr int kV = kK + kKTile;
     static constexpr int kBar = kK + kStages * kStage;         // mbarriers
-    static constexpr int kNumBars = 2 + 2 * kStages + 2 + 2 + 2 + 2 + 4 + 4 + 3;
+    static constexpr int kNumBars = 2 + 2 * kStages + 2 + 2 + 2 + 2 + 6 + 4 + 3;
     static constexpr int kMisc = kBar + kNumBars * 8;          // tmem base, abort flag, "a CTA has failed before", -, item[2][2]
     static constexpr int kTotal = kMisc + 32;
     static constexpr int kAlloc = kTotal + 1024;               // slack to align the base to 1024
@@ -86,6 +86,7 @@ struct AttnBars {
     uint64_t *pv_done;   // [2] O_x includes the tile's product (and P_x may be overwritten)
     uint64_t *y_full;    // [2] the linear branch's results for query tile x are in their stages
     uint64_t *y_ready;   // [2] ... and the output is where the first of them were
+    uint64_t *y_taken;   // [2] ... and the output warp has passed y_ready, as the softmax warps have y_full: the next may be announced
     uint64_t *item_full, *item_empty;   // [2] an item to come is there; ... and has been read
     uint64_t *first_done;   // [2] (of a pair's second CTA) the first CTA's producer is done with an item
     uint64_t *drain;     // MMA warp: everything issued has completed (failure path)
@@ -102,7 +103,8 @@ struct AttnBars {
         b.pv_done = b.p_full + 2;
         b.y_full = b.pv_done + 2;
         b.y_ready = b.y_full + 2;
-        b.item_full = b.y_ready + 2;
+        b.y_taken = b.y_ready + 2;
+        b.item_full = b.y_taken + 2;
         b.item_empty = b.item_full + 2;
         b.first_done = b.item_empty + 2;
         b.drain = b.first_done + 2;
@@ -610,7 +612,12 @@ __device__ __forceinline__ void producer_role(Work w, const AttnBars &bar, uint8
         }
         // Entries of the outputs: the parts' rows of this CTA's query tiles (rows behind the last of a head are never used).
         // They pass the ring's full-barrier at once: nobody waits for it, but its phases count the rounds.
+        // (An item of few tiles leaves the ring free for the outputs of the next one before the warps that wait for its own have
+        // looked; they would look for a parity that has come round again.  So the next outputs wait for these to be taken up.  us a call,
+        // without that and with it: 128 heads x 4096 tokens, d = 64, 478.4 and 481.0, a quarter kept 442.7 and 443.9; d = 128 the same.)
         for (int x = 0; x < n_q && ok; ++x) {
+            ok = mbar_wait(bar.y_taken + x, (uint32_t)((x ? b_armed : a_armed) & 1) ^ 1u, abort_flag, status, 17);
+            if (!ok) break;
             for (int y = 0; y < n_y; ++y, ++armed) {
                 ok = mbar_wait(bar.kv_empty + pos.stage, pos.parity ^ 1, abort_flag, status, 10);
                 if (!ok) {
@@ -688,6 +695,7 @@ __device__ __forceinline__ void output_role(Work w, const AttnBars &bar, const u
         ok = mbar_wait(bar.y_ready + x, y_odd, abort_flag, status, 15);
         if (!__all_sync(0xffffffffu, ok)) break;
         y_odd ^= 1;
+        if (lane == 0) mbar_arrive(bar.y_taken + x);
         const uint8_t *tile = ring + y_entry % kStages * P::kStage;
         if (rows == kBlockM) {
             if (lane == 0) {
@@ -897,6 +905,7 @@ __device__ __forceinline__ void attention_body(const AttnMaps &tm, const float *
             mbar_init(bar.y_full + i, P::y_entries(n_parts));
             mbar_init(bar.item_full + i, 1);
             mbar_init(bar.y_ready + i, 4);
+            mbar_init(bar.y_taken + i, 1);
             mbar_init(bar.first_done + i, 1);
             mbar_init(bar.item_empty + i, kCtas * 10 + 1 + (kCtas - 1));   // softmax and output warps, the issuing warp, the other producer
         }

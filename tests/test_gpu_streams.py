@@ -201,3 +201,17 @@ def _items_as_alone(d, B, N, C, k, df):
 def test_short_items_of_a_pair(N):
     # five ring entries: the first CTA's producer can be through with an item while the second has not seen that it may begin with it
     _items_as_alone(128, 5, N, 64, 16, 128)
+
+
+@pytest.mark.parametrize("d,B,N,C,k,df", [
+    # without a linear branch, with one part, with two; no token kept; CTAs that get two items, and three
+    (64, 10, 1, 64, 64, 64), (64, 5, 100, 64, 64, 64), (64, 10, 100, 64, 16, 32), (64, 10, 128, 64, 16, 64), (64, 10, 129, 64, 64, 64),
+    (64, 10, 200, 64, 0, 64), (64, 5, 200, 64, 16, 32), (64, 10, 300, 64, 0, 64), (64, 10, 300, 128, 128, 64), (64, 10, 384, 64, 64, 64),
+    (64, 10, 384, 128, 32, 64),
+    (128, 5, 1, 64, 16, 128), (128, 5, 100, 64, 64, 128), (128, 5, 100, 64, 16, 32), (128, 10, 128, 64, 16, 128), (128, 5, 129, 128, 128, 128),
+    (128, 10, 200, 64, 64, 128), (128, 5, 200, 64, 16, 32), (128, 10, 250, 128, 128, 128), (128, 5, 256, 64, 0, 128), (128, 5, 600, 64, 0, 64),
+    (128, 5, 600, 64, 64, 128),
+])
+def test_short_items_of_a_cta(d, B, N, C, k, df):
+    # one to three key tiles: the producers can be ahead of the softmax and the output warps by more than an item
+    _items_as_alone(d, B, N, C, k, df)
