@@ -689,6 +689,7 @@ __device__ __forceinline__ void map_items(const StepArgs<__nv_bfloat16> &a, uint
             nx2 += x * x;
         }
         nx2 = warp_sum(nx2);
+        __syncwarp();   // (q is read by other lanes than wrote it)
         float zv[8];
 #pragma unroll
         for (int i = 0; i < 8; ++i) zv[i] = lane + 32 * i < dp ? a.z[bh * dp + lane + 32 * i] : 0.f;
