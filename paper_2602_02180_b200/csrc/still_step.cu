@@ -1042,7 +1042,32 @@ static int launch_route(const still_params_t *p, const StepArgs<T> &a, int32_t *
     return STILL_OK;
 }
 
+// Map warps where the blocks have read-outs behind their tiles (bf16, up to eight heads a KV group: with 16 the cache pass
+// needs the registers) and the tiles are not many: what the read-outs gain is a few us whatever the tiles, and the cache pass, in
+// fewer registers and beside the loads of W_q, takes up to 2 % longer.  (us a step without and with them: 325 tiles a block
+// 82.7 and 81.4, 865 tiles, 16 sequences x 16000 tokens, 141.2 and 142.5.)
 constexpr int kMapTiles = 512;   // tiles of a block
+// Nor where the map warps, four read-outs at a time, would be what the block waits for.  The fewest tiles of a block with which they
+// are worth it, by read-outs a block (us a step without and with them; a quarter kept, 32 heads unless said):
+//   two rounds and more: 70 tiles are as long as a round.  32 sequences x 8192 tokens capped at 448, 204 tiles and two rounds, 71.9
+//     and 69.1; 64 x 1000, 215 and four, 104.9 and 109.9; 64 x 3000 capped at 128, 160 and four, 100.7 and 106.5.  Up to 4.5 a block the
+//     second round is a few blocks' alone, and the others' eight warps have little to do: 20 sequences at 155 tiles 55.2 and
+//     56.3, at 170 57.1 and 56.0; 22 (4.8 a block) at 127 52.2 and 53.0, at 141 54.8 and 54.0;
+//   one round, d = d_f = 128: a map warp reads the 32 KB of W_q in eight batches.  One a block, which eight warps share otherwise:
+//     4 sequences at 16 tiles 16.1 and 16.5, 3 at 11 15.2 and 16.2, at 21 16.54 and 16.65, at 24 16.98 and 16.87, 4 at 32 18.2 and 17.0.
+//     Two or three: 6 at 7 tiles 19.3 and 18.9, 12 at 13 23.5 and 21.9.  Nearly four, whose loads stand in each other's way: 15
+//     (3.2 a block) at 16 tiles 25.2 and 24.8, 16 (3.5) at 17 25.8 and 26.7, 18 (3.9) at 20 24.9 and 28.6, at 49 36.1 and 37.5, at 62 36.9
+//     and 35.0;
+//   ... with narrower maps always: 3 sequences, d_f = 64, at 4 tiles 12.5 and 12.2, 18 at 20 20.0 and 17.5;
+//   ... d = 64: three a block, four groups of two warps otherwise: 10 sequences at 10 tiles 15.2 and 15.8, at 34 (d_f = 32) 16.4 and
+//     16.7, 12 at 44 18.25 and 18.18, at 82 22.2 and 22.1.  Else always: one 11.4 and 10.4, two 13.4 to 14.9 and 13.2 to 15.0, four 15.1 and 14.4.
+static int least_map_tiles(long long n_items, long long blocks, int d, int df) {
+    const long long rounds = (n_items + kMapWarps * blocks - 1) / (kMapWarps * blocks);
+    if (rounds > 1) return 2 * n_items <= 9 * blocks ? 168 : (int)(70 * rounds);
+    if (d == 64) return n_items > 2 * blocks && n_items <= 3 * blocks ? 48 : 0;
+    if (df < 128) return 0;
+    return n_items <= blocks ? 24 : 4 * n_items > 13 * blocks ? 60 : 0;
+}
 template <typename T, int D, int NH>
 static int launch_main(const StepArgs<T> &a, unsigned grid, cudaStream_t st, int *launches) {
     auto launch = [&](auto mode) -> int {
@@ -1055,15 +1080,7 @@ static int launch_main(const StepArgs<T> &a, unsigned grid, cudaStream_t st, int
         profile_mark_end(st);
         return STILL_OK;
     };
-    // Map warps where the blocks have read-outs behind their tiles (bf16, up to eight heads a KV group: with 16 the cache pass
-    // needs the registers) and these are not many: what the read-outs gain is a few us whatever the tiles, and the cache pass, in
-    // fewer registers and beside the loads of W_q, takes up to 2 % longer.  (us a step without and with them: 325 tiles a block
-    // 82.7 and 81.4, 865 tiles, 16 sequences x 16000 tokens, 141.2 and 142.5.)
-    // Nor where the map warps, four read-outs at a time, would be what the block waits for (70 tiles are as long as a round of theirs:
-    // 32 sequences x 8192 tokens capped at 448, 204 tiles and two rounds, 71.9 without and 69.1 with them; 64 x 1000, 215 and four, 104.9 and
-    // 109.9; 64 x 3000 capped at 128, 160 and four, 100.7 and 106.5); with one round they always gain.
-    const long long items = (a.n_items + (long long)grid - 1) / grid, rounds = (items + kMapWarps - 1) / kMapWarps;
-    const bool map = a.n_items > 0 && a.per <= kMapTiles && (rounds == 1 || a.per >= 70 * rounds);
+    const bool map = a.n_items > 0 && a.per <= kMapTiles && a.per >= least_map_tiles(a.n_items, grid, D, a.df);
     constexpr bool kCanMap = sizeof(T) == 2 && NH <= 8;
     int rc;
     if (a.n_items > 0 && a.first_item_block > 0) rc = launch(std::integral_constant<StepMode, kItemsApart>{});

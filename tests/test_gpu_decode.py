@@ -387,3 +387,32 @@ def test_decode_batch_gives_each_sequence_its_own(B, H, Hkv, d, df, C, k, budget
     for b in {0, B // 2, B - 1}:
         alone = run([b])[0]
         assert bool(((Y[b] - alone).abs() <= 2 ** -7 * alone.abs() + 1e-4).all())
+
+
+@pytest.mark.parametrize("B,H,Hkv,d,n0", [
+    # with few tiles a block the features of the read-outs are formed by the warps of the cache pass, with more by warps of their own
+    (5, 16, 4, 128, 2500), (5, 16, 4, 128, 2800),      # one a block: 23 and 26 tiles
+    (18, 32, 8, 128, 900), (18, 32, 8, 128, 1100),     # four: 56 and 68
+    (10, 32, 8, 64, 1300), (10, 32, 8, 64, 1600),      # three, d = 64: 45 and 55
+    (20, 32, 8, 128, 2350), (20, 32, 8, 128, 2700),    # five: 160 and 183
+])
+def test_decode_batch_on_both_sides_of_the_limits(B, H, Hkv, d, n0):
+    # Sequences of a batch against the same sequences alone, and the rounding between.
+    C, k, steps = 64, 16, 2
+    w = synth.Workload("t", B, H, Hkv, d, n0 + steps, C, k, "bf16", "iid", 27)
+    Q, K, V = synth.make_qkv(w, "cuda")
+    Wq, Wk = synth.make_npmap_weights(w, "cuda")
+
+    def run(bs):
+        p = still.StillParams(len(bs), H, Hkv, d, C, k, torch.bfloat16, sm_scale=w.sm_scale)
+        x = [t[bs] for t in (Q, K, V)]
+        state = torch.zeros(still.state_bytes(p, w.N), dtype=torch.uint8, device="cuda")
+        still.hybrid_attn_fwd(p, *(t[:, :, :n0].contiguous() for t in x), Wq, Wk, state=state, state_max_tokens=w.N)
+        y = torch.stack([still.hybrid_attn_step(p, state, w.N, t, *(z[:, :, t].contiguous() for z in x), Wq, Wk) for t in range(n0, w.N)], 2)
+        assert still.device_status(state) == (0, 0)
+        return y.float()
+
+    Y = run(list(range(B)))
+    for b in (0, B - 1):
+        alone = run([b])[0]
+        assert bool(((Y[b] - alone).abs() <= 2 ** -7 * alone.abs() + 1e-4).all())   # two roundings of y to bf16 apart
