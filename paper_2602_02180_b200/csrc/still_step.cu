@@ -1055,7 +1055,7 @@ constexpr int kMapTiles = 512;   // tiles of a block
 //     56.3, at 170 57.1 and 56.0; 22 (4.8 a block) at 127 52.2 and 53.0, at 141 54.8 and 54.0;
 //   one round, d = d_f = 128: a map warp reads the 32 KB of W_q in eight batches.  One a block, which eight warps share otherwise:
 //     4 sequences at 16 tiles 16.1 and 16.5, 3 at 11 15.2 and 16.2, at 21 16.54 and 16.65, at 24 16.98 and 16.87, 4 at 32 18.2 and 17.0.
-//     Two or three: 6 at 7 tiles 19.3 and 18.9, 12 at 13 23.5 and 21.9.  Nearly four, whose loads stand in each other's way: 15
+//     Two or three: 9 of 20 heads at 5 tiles 18.5 and 18.8, 6 at 7 tiles 19.3 and 18.9, 12 at 13 23.5 and 21.9.  Nearly four, whose loads stand in each other's way: 15
 //     (3.2 a block) at 16 tiles 25.2 and 24.8, 16 (3.5) at 17 25.8 and 26.7, 18 (3.9) at 20 24.9 and 28.6, at 49 36.1 and 37.5, at 62 36.9
 //     and 35.0;
 //   ... with narrower maps always: 3 sequences, d_f = 64, at 4 tiles 12.5 and 12.2, 18 at 20 20.0 and 17.5;
@@ -1066,7 +1066,7 @@ static int least_map_tiles(long long n_items, long long blocks, int d, int df) {
     if (rounds > 1) return 2 * n_items <= 9 * blocks ? 168 : (int)(70 * rounds);
     if (d == 64) return n_items > 2 * blocks && n_items <= 3 * blocks ? 48 : 0;
     if (df < 128) return 0;
-    return n_items <= blocks ? 24 : 4 * n_items > 13 * blocks ? 60 : 0;
+    return n_items <= blocks ? 24 : 4 * n_items > 13 * blocks ? 60 : 6;
 }
 template <typename T, int D, int NH>
 static int launch_main(const StepArgs<T> &a, unsigned grid, cudaStream_t st, int *launches) {
