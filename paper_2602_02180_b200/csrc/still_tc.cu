@@ -225,8 +225,10 @@ __device__ __forceinline__ Stream make_stream(int R0, int rows, int N, int log2_
 // What an attention kernel works on, and how its roles come to it.  A CTA (or pair) stays for the whole kernel and takes one
 // item (the rows of two query tiles of a head) after the other: the first by its own number, the others from a counter (of the
 // workspace's status block, which the call's first kernel clears), so that whoever is done first takes the next.  The producer
-// of the first CTA asks for an item while it loads the one before, and hands it to the other roles (of both CTAs) in one of two
-// places.
+// of the first CTA asks for an item with the last keys of the one before, and hands it to the other roles (of both CTAs) in one of
+// two places.  (Asked for with the first keys, items were dealt out in the order in which their predecessors began, not ended: us a
+// call, like that and like this, with a CTA per item 92, 62, 155: 8 heads x 5700 tokens, d = 128, C = 128, 96 items for 74 pairs, 111 and
+// 94; 16 x 3000, d = 128, 96 items, 77 and 60; 4 x 12000, d = 64, 188 items for 148 CTAs, 186 and 156; every token kept.)
 struct Work {
     int n_blocks, n_heads, set_heads, H, Hkv, N, log2_c, lam, budget, sel_rows, sel_identity, n_parts;
     int rows;          // of a query tile: 128 a CTA
@@ -571,13 +573,13 @@ __device__ __forceinline__ void producer_role(Work w, const AttnBars &bar, uint8
             for (int half = 0; half < D / 64; ++half)
                 load(smem + P::kQ + x * P::kQTile + half * (kBlockM * 128), tm_q, bar.q_full, q_full0, half * 64,
                      q_row + ((int)rank + x * kCtas) * kBlockM);
-        // the item after this one, unless a CTA has failed (asked for here, needed behind the loop)
         int next = 0, failed = 0;
-        if (rank == 0) {
-            next = atomicAdd(status + kNextItem, 1);
-            failed = *reinterpret_cast<volatile int *>(status);
-        }
         for (int e = 0; e < entries; ++e, ++armed) {
+            if (rank == 0 && e == entries - 1) {
+                // the item after this one, unless a CTA has failed: asked for ahead of the wait for the last stage, needed behind the loop
+                next = atomicAdd(status + kNextItem, 1);
+                failed = *reinterpret_cast<volatile int *>(status);
+            }
             ok = mbar_wait(bar.kv_empty + pos.stage, pos.parity ^ 1, abort_flag, status, 1);
             if (!ok) break;
             bool sel;
