@@ -381,6 +381,12 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
         sp.blocks = 2ll * sp.BHkv * sp.kv_blocks + (long long)sp.BH * sp.score_blocks + sp.sel_blocks + 1;
         if (sp.blocks >= (1ll << 31)) return STILL_ERR_UNSUPPORTED;   // (a state of 32 TB)
     }
+    // Written among the gathered rows, the header comes ahead of S, z and Y: a call that fails behind it takes it back, so that no
+    // decode step accepts the state.
+    auto failed = [&](int code) {
+        if (state_written) (void)cudaMemsetAsync(state + L.header, 0, 256, st);
+        return code;
+    };
 
     // (1)+(2) Self-Saliency Score and per-chunk top-k; beside it the feature maps of the FMA kernels.
     const bool maps_too = w.la && !w.tc && front_blocks(p, N) <= kFrontBlocks;
@@ -410,7 +416,7 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
                               z_out, w.phiKsel ? ws + w.phiKsel : nullptr, Y && w.ksel ? ws + w.ksel : nullptr,
                               (Y || w.phiKsel) && w.vsel ? ws + w.vsel : nullptr, w.sel_rows,
                               state ? &sp : nullptr, &state_written, status, st, &g_launches);
-            if (rc != STILL_OK) return rc;
+            if (rc != STILL_OK) return failed(rc);
         } else {
             T *phiQ = reinterpret_cast<T *>(ws + w.phiQ);
             nla = reinterpret_cast<float *>(ws + w.nla);
@@ -442,7 +448,7 @@ static int fwd_typed(const still_params_t *p, long long N, const T *Q, const T *
             rc = launch_sa_merge<T>(p, N, Q, K, V, sel, nla, dla, Y, st);
             profile_mark_end(st);
         }
-        if (rc != STILL_OK) return rc;
+        if (rc != STILL_OK) return failed(rc);
     }
 
     // Decode state: K/V history, scores, selection, where they have not been written with the gathered rows; S and z were written
