@@ -291,9 +291,11 @@ npmap_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
 // and the rows read: 32 heads x 131072 tokens, d = 128, 32 of 128 selected, with phi_sel: three kernels that each
 // gathered for themselves (and one that summed a row after the other) took 1023 us, this one 305.
 // kFew: at d = 64 up to 16 tokens of a chunk are one row a thread; eight blocks an SM instead of five keep as many rows in flight
-// (128 heads x 4096 tokens, 16 of 64: 29.7 us and 23.7; with 32 of 64 a thread's two rows one after the other 6 us more).
+// (128 heads x 4096 tokens, 16 of 64: 29.7 us and 23.7; with 32 of 64 a thread's two rows one after the other 6 us more).  Not with
+// the decode state, whose copies do not fit 32 registers, nor 48 (92 and 16 bytes of a thread spilled; with 64 none: us a call of 128 heads x
+// 300 tokens 69.4 and 66.9, 64 x 700 67.6 and 65.4, 32 x 1003 56.4 and 56.2).
 template <int D, int DF, bool kFew, bool kState>
-__global__ void __launch_bounds__(256, D == 128 ? 4 : kFew ? 8 : 5)
+__global__ void __launch_bounds__(256, D == 128 || kState ? 4 : kFew ? 8 : 5)
 gather_kernel(const __nv_bfloat16 *K, const __nv_bfloat16 *V, const __nv_bfloat16 *phiK,
               const int32_t *sel_idx, __nv_bfloat16 *Ksel, __nv_bfloat16 *Vsel,
               __nv_bfloat16 *phi_sel, float *selsum, int H, int Hkv, long long N, int lam,
@@ -1212,8 +1214,7 @@ int launch_gather(const still_params_t *p, long long N, const void *K, const voi
     ++*launches;
     const long long BH = (long long)p->B * p->H, rows = state != nullptr ? (state->blocks + Tn) / (Tn + 1) : 0;
     const bool few = D == 64 && p->topk <= 16;
-    return launch_dependent(state == nullptr ? (few ? gather_kernel<D, DF, D == 64, false> : gather_kernel<D, DF, false, false>)
-                                             : (few ? gather_kernel<D, DF, D == 64, true> : gather_kernel<D, DF, false, true>),
+    return launch_dependent(state != nullptr ? gather_kernel<D, DF, false, true> : few ? gather_kernel<D, DF, D == 64, false> : gather_kernel<D, DF, false, false>,
                             dim3((unsigned)(Tn + 1), (unsigned)(BH + rows)), dim3(256), 0, st, (const bf *)K, (const bf *)V,
                             (const bf *)phiK, sel_idx, (bf *)k_sel, (bf *)v_sel, (bf *)phiK_sel, selsum, p->H, p->Hkv, N, p->topk, sel_rows,
                             n_routed, (int)BH, state != nullptr ? *state : StateParts{}, *p) == cudaSuccess ? STILL_OK : STILL_ERR_CUDA;
