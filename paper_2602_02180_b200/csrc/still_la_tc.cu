@@ -283,13 +283,15 @@ npmap_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
 // Selected rows, and the normaliser z (Eq. cache_routing_sum): z after chunk c = sum over the chunks 0..c of the
 // features of their unselected tokens = (column sums of phi(K) over the chunk) - (rows of its selected tokens).
 // ------------------------------------------------------------------------------------------
-// grid (T + 1, B*H; with the decode state: and as many rows as its blocks take), 256 threads: the lam selected tokens of chunk blockIdx.x of a query head, read once for everything
+// grid (T + 1, B*H; with the decode state: and as many rows as its blocks take), 256 threads: the lam selected tokens of a chunk of a query head, read once for everything
 // that is made of them: their K and V rows in selection order (row j of a head is token sel_idx[j]; K_sel / V_sel, what
 // the attention kernel tiles), with a salient-cache budget also their phi(K) rows (phi_sel, from which the tokens that
 // leave the cache enter the state), and the sum of the phi(K) rows (selsum [B*H, n_routed, 2 DF], of the routed chunks).
-// -1 entries and the rows of the padding (block T) are zero.  NULL outputs are not made.  Bound by the bytes written
+// -1 entries and the rows of the padding (chunk T) are zero.  NULL outputs are not made.  Bound by the bytes written
 // and the rows read: 32 heads x 131072 tokens, d = 128, 32 of 128 selected, with phi_sel: three kernels that each
 // gathered for themselves (and one that summed a row after the other) took 1023 us, this one 305.
+// A head begins with another chunk than the one before: else, where T + 1 is a multiple of 37, all paddings, which are the longest,
+// lay on four SMs (32 heads x 2244 tokens, d = 64, with phi_sel: 15.2 us and 7.9; with five blocks an SM 10.8).
 // kFew: at d = 64 up to 16 tokens of a chunk are one row a thread; eight blocks an SM instead of five keep as many rows in flight
 // (128 heads x 4096 tokens, 16 of 64: 29.7 us and 23.7; with 32 of 64 a thread's two rows one after the other 6 us more).  Not with
 // the decode state, whose copies do not fit 32 registers, nor 48 (92 and 16 bytes of a thread spilled; with 64 none: us a call of 128 heads x
@@ -310,7 +312,7 @@ gather_kernel(const __nv_bfloat16 *K, const __nv_bfloat16 *V, const __nv_bfloat1
     constexpr int kVec = D / 8, kPhiVec = 2 * DF / 8;       // 16-byte pieces of a row
     constexpr int kPer = 32 / kVec, kPhiPer = 32 / kPhiVec;  // rows that a warp moves at a time
     __shared__ __align__(16) float sums[8 * kPhiPer][2 * DF];   // (written 16 bytes at a time)
-    const int bh = blockIdx.y, b = bh / H, h = bh % H, c = blockIdx.x, Tn = gridDim.x - 1;
+    const int bh = blockIdx.y, b = bh / H, h = bh % H, c = (int)((blockIdx.x + blockIdx.y) % gridDim.x), Tn = gridDim.x - 1;
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const long long src0 = ((long long)b * Hkv + h / (H / Hkv)) * N, dst0 = (long long)bh * sel_rows + (long long)c * lam;
     if (c == Tn) {   // padding up to sel_rows
