@@ -135,7 +135,11 @@ static FwdPlan plan_fwd(const still_params_t *p, long long N, size_t limit = SIZ
         // A chunk a segment where that many are wanted: a segment's chunks are a chain (4 heads, d = 64, C = 64: 512 tokens in
         // segments of two chunks 22.9 us, of one 13).  Up to four chunks, of which two are answered, one pass instead of three (us a
         // call, one and three: 250 tokens, 32 heads 66.7 and 72.0, 16 heads 49.9 and 60.4, 4 heads 49 and 47; five chunks, 4 heads: 47).
-        const long long want = T <= 4 ? 1 : std::max<long long>(1, std::min<long long>((kScanBlocks + units - 1) / units, T));
+        // With many blocks T - 2 segments at most, that is two chunks a segment: the sums' traffic then costs more than the chain.  (us a
+        // call of two chunks a segment and of one, by T x units: d = 64, 352 160 and 144, 448 164 and 151, 512 214.1 and 215.9; d = 128, 192
+        // 241 and 202, 320 168.7 and 165.5, 352 204.5 and 206.3, 448 193 and 200.)
+        const long long most = T * units <= (p->d == 64 ? 448 : 320) ? T : T - 2;
+        const long long want = T <= 4 ? 1 : std::max<long long>(1, std::min<long long>((kScanBlocks + units - 1) / units, most));
         const size_t per_seg = BH * dp * (size_t)(p->d + 1) * 4;
         if (off <= STILL_STATIC_WORKSPACE_BYTES) limit = std::min(limit, (size_t)STILL_STATIC_WORKSPACE_BYTES);
         long long n = want;

@@ -486,3 +486,23 @@ def test_state_written_among_the_gathered_rows(N, rides):
     want.scatter_add_(2, sel.clamp_min(0), (sel >= 0).int())
     assert torch.equal(bits, want)
     assert part("header", 14, torch.int32)[12].item() == N
+
+
+@pytest.mark.parametrize("H,Hkv,d,N", [
+    (32, 8, 128, 320), (32, 8, 128, 330),   # a chunk a segment, and two from 321 (chunks x heads x d / 64) on
+    (28, 4, 64, 1024), (28, 4, 64, 1030),   # ... from 449 on: 16 and 17 chunks
+])
+def test_fp32_segments_of_one_chunk_and_of_two(H, Hkv, d, N):
+    C, k = 64, 16
+    w = _small("t", "fp32", 1, H, Hkv, d, N, C, k)
+    lay = still.state_layout(U.params_of(w), N)
+    state = torch.zeros(lay["total"], dtype=torch.uint8, device="cuda")
+    r = U.run_prefill(w, state=state, state_max_tokens=N)
+    heads = [(0, 0), (0, H - 1)]
+    U.check_selection(r["scores"], r["sel"], C, k, heads)
+    U.check_outputs(w, r["Q"], r["K"], r["V"], r["Wq"], r["Wk"], r["Y"], r["scores"], r["sel"], heads, tol=1e-5)
+    # z: the features of the unselected tokens of the routed chunks, which sum to 2 each
+    z = state[lay["z"]: lay["z"] + H * 2 * d * 4].view(torch.float32).view(H, 2 * d)
+    n = -(-N // C) - 2
+    want = 2.0 * n * (C - k)
+    assert float((z.double().sum(1) - want).abs().max()) <= want * n * C * 2 ** -24   # (fp32 sums of up to n C terms)
