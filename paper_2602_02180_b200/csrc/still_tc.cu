@@ -230,7 +230,7 @@ __device__ __forceinline__ Stream make_stream(int R0, int rows, int N, int log2_
 // call, like that and like this, with a CTA per item 92, 62, 155: 8 heads x 5700 tokens, d = 128, C = 128, 96 items for 74 pairs, 111 and
 // 94; 16 x 3000, d = 128, 96 items, 77 and 60; 4 x 12000, d = 64, 188 items for 148 CTAs, 186 and 156; every token kept.)
 struct Work {
-    int n_blocks, n_heads, set_heads, H, Hkv, N, log2_c, lam, budget, sel_rows, sel_identity, n_parts;
+    int n_blocks, n_heads, set_heads, rep, N, log2_c, lam, budget, sel_rows, sel_identity, n_parts;
     int rows;          // of a query tile: 128 a CTA
     int first, total;
     volatile int *item;   // [2][2]: head (-1: there are no more) and first row
@@ -553,14 +553,13 @@ __device__ __forceinline__ void producer_role(Work w, const AttnBars &bar, uint8
     bool ok = true;
     int armed = 0, n = 0, q_armed = 0, a_armed = 0, b_armed = 0;
     RingPos pos{0, 0};
-    w.set(w.first);
     prefetch_map(&tm_k);
     prefetch_map(&tm_v);
     if (w.n_parts > 0) prefetch_map(&tm_p0);
     if (w.n_parts > 1) prefetch_map(&tm_p1);
     for (bool more = true; more && ok; ++n) {
         const Stream st = w.stream();
-        const int kv_row0 = (w.bh / w.H * w.Hkv + w.bh % w.H / (w.H / w.Hkv)) * w.N, q_row = w.bh * w.N + w.R0;
+        const int kv_row0 = w.bh / w.rep * w.N, q_row = w.bh * w.N + w.R0;
         // (with topk = chunk every token is selected and the compacted arrays would be copies of K / V: the salient prefix is
         // then read from K / V themselves, and tm_ksel / tm_vsel alias tm_k / tm_v)
         const int sel_row0 = w.sel_identity ? kv_row0 : w.bh * w.sel_rows;
@@ -682,7 +681,6 @@ __device__ __forceinline__ void output_role(Work w, const AttnBars &bar, const u
     bool ok = true;
     if (lane == 0) prefetch_map(&tm_y);
     bool more = true;
-    w.set(w.first);
     for (int n = 0; more; ++n) {
         const Stream st = w.stream();
         const int y_entry = ring0 + st.entries() + x * n_y, t0 = w.R0 + (x * kCtas + (int)rank) * kBlockM, rows = min(w.N - t0, kBlockM);
@@ -763,7 +761,6 @@ __device__ __forceinline__ void mma_role(Work w, const AttnBars &bar, uint8_t *s
     uint32_t qk_odd = 0, pv_odd = 0;   // bit x: parity of the S (of the P V) of query tile x that there have been
     int x_prev = -1;                   // of the item whose S was formed last
     bool more = true;
-    w.set(w.first);
     for (int n = 0; more; ++n) {
         const Stream st = w.stream();
         const int n_own0 = st.n_lead + 2 * st.n_shared, n_items = n_own0 + st.n_a + st.n_b;
@@ -885,8 +882,12 @@ __device__ __forceinline__ void attention_body(const AttnMaps &tm, const float *
     // the same in all lanes)
     const int warp = __shfl_sync(0xffffffffu, (int)(threadIdx.x >> 5), 0), lane = threadIdx.x & 31;
     const uint32_t rank = kPair ? blockIdx.x & 1u : 0u, peer = rank ^ 1u;
-    Work w{n_blocks, n_heads, set_heads, H, Hkv, N, C == 128 ? 7 : 6, lam, budget, sel_rows, sel_identity, n_parts, kRows,
+    Work w{n_blocks, n_heads, set_heads, H / Hkv, N, C == 128 ? 7 : 6, lam, budget, sel_rows, sel_identity, n_parts, kRows,
            (int)(kPair ? blockIdx.x >> 1 : blockIdx.x), n_blocks * n_heads, reinterpret_cast<volatile int *>(smem + P::kMisc + 16), 0, 0};
+    // Here, where all warps do it together, and the KV head by one division (rep): with the first in every role's own code and four
+    // divisions an item took some 500 cycles more, the first S of a call came 600 later (us a call: 128 heads x 4096 tokens, d = 64, 477.3
+    // and 474.1, a quarter kept 442.4 and 440.7, 128 x 1500 114.8 and 113.3, 64 x 214 18.55 and 18.09; d = 128, 16 x 1000 33.6 and 32.6).
+    w.set(w.first);
     auto sync_all = [&]() {
         if constexpr (kPair) cluster_sync_all();
         else __syncthreads();
@@ -959,7 +960,6 @@ __device__ __forceinline__ void attention_body(const AttnMaps &tm, const float *
         const int x = warp >> 2;                       // 0: tile A, 1: tile B
         const int n_y = P::y_entries(n_parts);
         int ring0 = 0, flip = 0, y_flip = 0;           // ring stage of the item's first entry; see softmax_role
-        w.set(w.first);
         bool ok = true, more = true;
         for (int n = 0; more && ok; ++n) {
             const Stream st = w.stream();
