@@ -283,7 +283,8 @@ npmap_tc_kernel(const __grid_constant__ CUtensorMap tm_x, const __grid_constant_
 // Selected rows, and the normaliser z (Eq. cache_routing_sum): z after chunk c = sum over the chunks 0..c of the
 // features of their unselected tokens = (column sums of phi(K) over the chunk) - (rows of its selected tokens).
 // ------------------------------------------------------------------------------------------
-// grid (T + 1, B*H; with the decode state: and as many rows as its blocks take), 256 threads: the lam selected tokens of a chunk of a query head, read once for everything
+// grid (T + 1, B*H; with the decode state: and as many rows as its blocks take), 256 threads: the lam selected tokens of a
+// chunk of a query head, read once for everything
 // that is made of them: their K and V rows in selection order (row j of a head is token sel_idx[j]; K_sel / V_sel, what
 // the attention kernel tiles), with a salient-cache budget also their phi(K) rows (phi_sel, from which the tokens that
 // leave the cache enter the state), and the sum of the phi(K) rows (selsum [B*H, n_routed, 2 DF], of the routed chunks).

@@ -9,9 +9,9 @@
 // [0, (c-1)*lambda) of a contiguous array that TMA can tile.
 //
 // An item is 256 consecutive query rows of one (batch, head), for a pair of CTAs 512: two query tiles A and B of 128
-// (256) rows.  CTAs stay and take one item after the other (Work).  The keys of an item come as a stream of 128-key tiles: SEL tiles j (rows [128j, 128j+128) of K_sel / V_sel), and
-// the LOC tiles around the rows (rows of K / V at positions [128m, 128m+128)).  First the SEL tiles that both query
-// tiles see (before them what has already left the window of B), then what only one of them sees, by turns.  Which
+// (256) rows.  CTAs stay and take one item after the other (Work).  The keys of an item come as a stream of 128-key
+// tiles: SEL tiles j (rows [128j, 128j+128) of K_sel / V_sel), and the LOC tiles around the rows (rows of K / V at
+// positions [128m, 128m+128)).  First the SEL tiles that both query tiles see (before them what has already left the window of B), then what only one of them sees, by turns.  Which
 // columns of a tile a query row sees is a per-row column interval, applied as a mask in the softmax.
 //
 // Warp roles (384 threads):
@@ -1043,12 +1043,10 @@ sa_merge_pair_kernel(const __grid_constant__ AttnMaps tm, const float *d_part, _
 // (tile n = head n / n_row_blocks, rows 128 (n % n_row_blocks) ...) with two stages of shared memory and two
 // TMEM accumulators, so that the loads of tile n+1 and its UMMA run under the row epilogue of tile n.
 // The row's epilogue bounds it: three special-function instructions per window element (one 2^x, two logarithms) against
-// six or seven others, by twelve warps an SM at C = 64, eight at C = 128 (with eight at C = 64, too: special-function unit 53 %
-// busy, issue slots 38 %, DRAM 38 % at d = 128; C = 128: 61, 37 and 24 %).  us of a
-// call for the scores alone with eight and twelve warps, in turn on one box: 2 x 32 heads x 32768 tokens, d = 128, 201 to 219 and 175
-// to 180, 4 x 32 x 4096, d = 64, 60.5 and 56.  The kernel with eight: 2 x 32 heads x 32768 tokens, d = 128, C = 64: 199 us, 4 x 32 x 4096, d = 64: 51 us,
-// 32 x 131072, d = 128, C = 128: 650 us (with a threshold per token in the ranking, see below: 223, 58 and 825; with scalar
-// arithmetic, logarithms for subnormal arguments, and for C = 128 a second set of exponentials as well: 325 to 368, 83 and 1030).
+// six or seven others, by twelve warps an SM at C = 64, eight at C = 128, where a third group's rows spill (special-function unit
+// 66 to 69 % busy and 61 %, issue slots 50 and 37 %).  us of the kernel: 32 heads x 32768 tokens, d = 128, 85.6, 128 x 4096, d = 64, 44.7;
+// C = 128, 32 x 32768, 179.8.  us of a call for the scores alone with eight warps and with twelve, in turn on one box: 64 x 32768,
+// d = 128, 201 to 219 and 175 to 180, 128 x 4096, d = 64, 60.5 and 56.
 // Warps: 0 TMA producer, 1 MMA issuer, 2-5 score group 0, 6-9 score group 1, ...; TMEM lane quarter = warp % 4.
 // ---------------------------------------------------------------------------
 template <int D>
